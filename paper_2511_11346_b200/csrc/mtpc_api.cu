@@ -58,6 +58,7 @@ struct Layout {
   // workspace offsets (bytes)
   size_t off_status, off_wemit, off_wsum, off_hidden, off_logA, off_G, off_logw, off_sel, off_logits, off_unit_lse;
   size_t off_prefix, off_partial, off_sum_bias;   // training loss: prefix log-marginals [max_positions, n], per-sequence terms
+  size_t off_msg;       // slot messages of the drafted windows [max_windows, n, r], kept for the acceptance stage
   int decode_max_p;     // positions the few-position draft path can take (0: path not available)
   bool can_draft;       // v <= 512: the sampling kernels hold a whole input unit on chip
   bool can_draft_many;  // the sampling epilogue of the projection kernel can tile a unit (draft of more than 128 positions)
@@ -168,6 +169,7 @@ int plan(const mtpc_config& c, Layout* L) {
   L->off_G = take(L->max_windows * c.n * c.r * 4);
   L->off_logw = take(static_cast<size_t>(c.max_positions) * L->sum_rows * 4);
   L->off_sel = take(L->max_windows * c.n * 4);
+  L->off_msg = take(L->max_windows * c.n * c.r * 4);
   // (latents of more than 32 values are handled for the mixture only; HMM and BTree are limited to r <= 32 anyway)
   L->decode_max_p = L->can_draft ? (c.max_positions < kDecodeMaxP ? c.max_positions : kDecodeMaxP) : 0;
   L->off_logits = take(static_cast<size_t>(L->decode_max_p) * emit_units * c.v * 4);
@@ -290,6 +292,7 @@ struct mtpc_head {
   int copy_event_count;
   int draft_P;              // positions whose draft state (logits, or after a many-position draft G and log omega) is in the workspace (0: none)
   int draft_wpp;            // windows per position of that draft
+  bool draft_msg;           // its slot messages are in the workspace too (a draft that asked for prefix marginals leaves them)
   const void* draft_hidden; // many-position draft: the bf16 hidden states it read (the acceptance stage stages rows of them)
   int ring;                 // calls whose per-kernel events are retained (0 = timing off)
   cudaEvent_t* ev;          // [ring][kMaxPhases][2]
@@ -502,17 +505,13 @@ int launch_gemm(mtpc_head* h, int mode, const void* hidden_bf16, int rows, int w
   return check_launch();
 }
 
-// Shared memory of one CTA of the binary-tree circuit kernel (see circuit_btree_kernel).
-size_t hmm_stream_smem_bytes(int r) { return static_cast<size_t>(kCircuitWarps) * (kHmmDepth * r * r + 32) * sizeof(float); }
-size_t btree_smem_bytes(int n, int r, bool with_prefix) {
-  return static_cast<size_t>(kCircuitWarps) * btree_warp_floats(n, r, with_prefix) * sizeof(float);
-}
+size_t btree_smem_bytes(int n, int r) { return static_cast<size_t>(kCircuitWarps) * btree_warp_floats(n, r) * sizeof(float); }
 
-// Circuit evaluation of W windows: out[w] = joint log-prob (may be NULL when prefix is given); prefix (may be NULL)
-// [W, n] = log-marginals of the prefixes x_0..x_i.
+// Circuit evaluation of W windows: out[w] = joint log-prob, prefix [W, n] = log-marginals of the prefixes x_0..x_i, msg
+// [W, n, r] = slot messages (each may be NULL, not all).
 // dependent: the launch directly follows draft_slot_kernel, which has zeroed the work counter, and may overlap its tail.
 int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cudaStream_t st, bool dependent = false,
-                   bool raw_mixture = false) {
+                   bool raw_mixture = false, float* msg = nullptr) {
   if (W <= 0) return MTPC_OK;
   const mtpc_config& c = h->cfg;
   const Layout& L = h->L;
@@ -520,24 +519,40 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
   const float* logw = at<float>(h, L.off_logw);
   const int blocks = (W + kCircuitWarps - 1) / kCircuitWarps;
   const int threads = kCircuitWarps * 32;
-  // kernels that stream per-position tables hand out windows through a counter next to the status word
-  unsigned* counter = at<unsigned>(h, L.off_status) + kWorkCounterWord;
-  const int resident = blocks < 8 * h->num_sms ? blocks : 8 * h->num_sms;   // more CTAs than an SM can hold do no harm
-  if (!dependent && (c.family == MTPC_BTREE || c.family == MTPC_HMM)) {
-    if (cudaMemsetAsync(counter, 0, sizeof(unsigned), st) != cudaSuccess) return MTPC_ERR_CUDA;
-  }
-  if (c.family == MTPC_CP) {
-    launch_kernel(circuit_cp_kernel, blocks, threads, 0, st, dependent, G, logw, out, prefix, W, wpp, c.n, c.r, L.sum_rows,
+  const bool sweep = prefix != nullptr || msg != nullptr;
+  if (c.family == MTPC_CP && sweep) {
+    const size_t per_warp = cp_prefix_warp_floats(c.n, c.r) * sizeof(float);
+    const int warps = W <= h->num_sms || per_warp > 8192 ? 1 : 4;       // few windows: one per SM
+    launch_kernel(circuit_cp_prefix_kernel, (W + warps - 1) / warps, warps * 32, warps * per_warp, st, dependent, G, logw, out,
+                  prefix, msg, W, wpp, c.n, c.r, L.sum_rows, raw_mixture ? 1 : 0);
+  } else if (c.family == MTPC_CP) {
+    launch_kernel(circuit_cp_kernel, blocks, threads, 0, st, dependent, G, logw, out, W, wpp, c.n, c.r, L.sum_rows,
                   raw_mixture ? 1 : 0);
   } else if (c.family == MTPC_HMM) {
-    launch_kernel(circuit_hmm_stream_kernel, resident, threads, hmm_stream_smem_bytes(c.r), st, dependent, G, logw,
-                  hmm_tables(h), hmm_table_stride(h), out, prefix, counter, W, wpp, c.n, c.r, L.sum_rows);
-  } else if (prefix != nullptr) {
-    launch_kernel(circuit_btree_kernel<true>, resident, threads, btree_smem_bytes(c.n, c.r, true), st, dependent, G, logw,
-                  out, prefix, counter, W, wpp, c.n, c.r, L.sum_rows);
+    // as many tables as fit beside the warps' vectors (all of them but for very long windows)
+    int chunk = c.n > 1 ? c.n - 1 : 1;
+    while (chunk > 1 && hmm_circuit_smem_floats(c.n, c.r, prefix != nullptr, chunk) * sizeof(float) > static_cast<size_t>(kSmemLimit)) --chunk;
+    const size_t smem = hmm_circuit_smem_floats(c.n, c.r, prefix != nullptr, chunk) * sizeof(float);
+    const int stride = hmm_table_stride(h);
+    const int items = stride == 0 ? (W + kHmmWarps - 1) / kHmmWarps : W / wpp * ((wpp + kHmmWarps - 1) / kHmmWarps);
+    const int resident = h->num_sms * (static_cast<int>(kSmemLimit / (smem + 1024)) > 8 ? 8 : static_cast<int>(kSmemLimit / (smem + 1024)) < 1 ? 1 : static_cast<int>(kSmemLimit / (smem + 1024)));
+    launch_kernel(circuit_hmm_kernel, items < resident ? items : resident, kHmmWarps * 32, smem, st, dependent, G, logw,
+                  hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r, L.sum_rows, chunk);
+  } else if (sweep) {
+    const int warps = c.n / 2 < 8 ? c.n / 2 : 8;                         // a warp per node of the owners' level
+    const bool fits = btree_prefix_smem_floats(c.n, c.r, warps, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
+    const size_t smem = btree_prefix_smem_floats(c.n, c.r, warps, fits) * sizeof(float);
+    const int per_sm = static_cast<int>(kSmemLimit / (smem + 1024));
+    const int resident = h->num_sms * (per_sm < 1 ? 1 : per_sm > 8 ? 8 : per_sm);
+    launch_kernel(circuit_btree_prefix_kernel, W < resident ? W : resident, warps * 32, smem, st, dependent, G, logw, out, prefix,
+                  msg, W, wpp, c.n, c.r, L.sum_rows, fits ? 1 : 0);
   } else {
-    launch_kernel(circuit_btree_kernel<false>, resident, threads, btree_smem_bytes(c.n, c.r, false), st, dependent, G,
-                  logw, out, static_cast<float*>(nullptr), counter, W, wpp, c.n, c.r, L.sum_rows);
+    // windows are handed out through a counter next to the status word
+    unsigned* counter = at<unsigned>(h, L.off_status) + kWorkCounterWord;
+    const int resident = blocks < 8 * h->num_sms ? blocks : 8 * h->num_sms;   // more CTAs than an SM can hold do no harm
+    if (!dependent && cudaMemsetAsync(counter, 0, sizeof(unsigned), st) != cudaSuccess) return MTPC_ERR_CUDA;
+    launch_kernel(circuit_btree_kernel, resident, threads, btree_smem_bytes(c.n, c.r), st, dependent, G, logw, out, counter, W,
+                  wpp, c.n, c.r, L.sum_rows);
   }
   h->launches++;
   return check_launch();
@@ -551,9 +566,10 @@ bool allow_full_smem(K kernel) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) == cudaSuccess;
 }
 bool set_circuit_attributes() {
-  bool ok = allow_full_smem(circuit_hmm_stream_kernel);
-  ok &= allow_full_smem(circuit_btree_kernel<false>);
-  ok &= allow_full_smem(circuit_btree_kernel<true>);
+  bool ok = allow_full_smem(circuit_hmm_kernel);
+  ok &= allow_full_smem(circuit_btree_kernel);
+  ok &= allow_full_smem(circuit_btree_prefix_kernel);
+  ok &= allow_full_smem(circuit_cp_prefix_kernel);
   return ok;
 }
 
@@ -716,6 +732,8 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
   const mtpc_config& c = h->cfg;
   const Layout& L = h->L;
   const int W = P * wpp;
+  // a draft that returns prefix marginals runs the sweep that also yields the slot messages of the acceptance stage
+  float* const msg = at<float>(h, L.off_msg);
   if (!L.can_draft) return MTPC_ERR_UNSUPPORTED;
   if (h->lr_k > 0 && P > L.decode_max_p && wpp == 1 && c.v <= kMaxDraftVocab && h->lr_off_base != 0) {
     // A long draft on a factored head, one window per position: log omega, the latent draws, then every (window, slot)
@@ -759,11 +777,12 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     pt.end();
     if (rc != MTPC_OK) return rc;
     pt.begin();
-    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st);
+    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, false, false, out_prefix ? msg : nullptr);
     pt.end();
-    if (rc == MTPC_OK) {               // G, log omega, W_base h and B h stay in place for an acceptance call
+    if (rc == MTPC_OK) {               // G, log omega, the messages, W_base h and B h stay in place for an acceptance call
       h->draft_P = P;
       h->draft_wpp = wpp;
+      h->draft_msg = out_prefix != nullptr;
       h->draft_hidden = nullptr;
     }
     return rc;
@@ -818,10 +837,12 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     h->launches++;
     h->draft_P = P;
     h->draft_wpp = wpp;
+    h->draft_msg = out_prefix != nullptr;
     pt.end();
     if ((rc = check_launch()) != MTPC_OK) return rc;
     pt.begin();
-    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*dependent=*/h->ring == 0, /*raw_mixture=*/c.r > 32);
+    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*dependent=*/h->ring == 0, /*raw_mixture=*/c.r > 32,
+                        out_prefix ? msg : nullptr);
     pt.end();
     return rc;
   }
@@ -895,11 +916,12 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
   pt.end();
   if (rc != MTPC_OK) return rc;
   pt.begin();
-  rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st);
+  rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, false, false, out_prefix ? msg : nullptr);
   pt.end();
-  if (rc == MTPC_OK) {                 // G, log omega and the hidden states stay in place for an acceptance call
+  if (rc == MTPC_OK) {                 // G, log omega, the messages and the hidden states stay in place for an acceptance call
     h->draft_P = P;
     h->draft_wpp = wpp;
+    h->draft_msg = out_prefix != nullptr;
     h->draft_hidden = hb;
   }
   return rc;
@@ -1603,17 +1625,25 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
   const Layout& L = head->L;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int W = P * wpp;
-  const size_t smem = accept_warp_floats(c.family, c.n, c.r, c.v) * sizeof(float);
+  const size_t smem = accept_smem_floats(c.r, c.v) * sizeof(float);
   if (smem > static_cast<size_t>(kSmemLimit)) return MTPC_ERR_UNSUPPORTED;      // a residual row of more than ~56k symbols
+  const int threads = accept_threads(c.v);
   PhaseTimer pt(head, st);
+  float* const msg = at<float>(head, L.off_msg);
+  if (!head->draft_msg) {
+    // the draft returned the joint alone: the slot messages are formed now, from the evidence and log omega it left
+    rc = launch_circuit(head, W, wpp, nullptr, nullptr, st, /*dependent=*/false,
+                        /*raw_mixture=*/P <= L.decode_max_p && c.r > 32, msg);
+    if (rc != MTPC_OK) return rc;
+    head->draft_msg = true;
+  }
   if (P <= L.decode_max_p) {
     // after a few-position draft: every logit of the drafted positions is still in the workspace
     pt.begin();
-    spec_accept_kernel<<<W, kAcceptThreads, smem, st>>>(
-        c.family, at<float>(head, L.off_logits), at<float>(head, L.off_unit_lse), at<float>(head, L.off_logw),
-        hmm_tables(head), draft_bytes, prefix_logprob, target_probs, accept_uniforms, out_accepted,
-        out_next_byte, at<unsigned>(head, L.off_status), W, wpp, c.n, c.r, c.v, valid_symbols(c), L.sum_rows,
-        hmm_table_stride(head), static_cast<const float*>(nullptr), static_cast<const int*>(nullptr));
+    launch_kernel(spec_accept_kernel, W, threads, smem, st, /*dependent=*/head->ring == 0, at<float>(head, L.off_logits),
+                  at<float>(head, L.off_unit_lse), msg, draft_bytes, prefix_logprob, target_probs, accept_uniforms, out_accepted,
+                  out_next_byte, at<unsigned>(head, L.off_status), W, wpp, c.n, c.r, c.v, valid_symbols(c),
+                  static_cast<const int*>(nullptr));
     head->launches++;
     pt.end();
     return check_launch();
@@ -1635,8 +1665,6 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
   float* lg = at<float>(head, L.off_acc_logits);
   float* lse = at<float>(head, L.off_acc_lse);
   const int chunk_pos = static_cast<int>(L.accept_rows / wpp);                  // >= 1 by construction
-  const float* tables = hmm_tables(head);
-  const int tstride = hmm_table_stride(head);
   for (int p0 = 0; p0 < P; p0 += chunk_pos) {
     const int pc = P - p0 < chunk_pos ? P - p0 : chunk_pos;
     const int wc = pc * wpp;
@@ -1661,11 +1689,9 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
       int rcf = check_launch();
       if (rcf != MTPC_OK) return rcf;
       pt.begin();
-      spec_accept_kernel<<<wc, kAcceptThreads, smem, st>>>(
-          c.family, lg, lse, at<float>(head, L.off_logw) + static_cast<size_t>(p0) * L.sum_rows,
-          tables + static_cast<size_t>(p0) * tstride, xb, pre, tp, ua, out_accepted + w0, out_next_byte + w0,
-          at<unsigned>(head, L.off_status), wc, wpp, c.n, c.r, c.v, valid_symbols(c), L.sum_rows, tstride,
-          at<float>(head, L.off_G) + w0 * c.n * c.r, row_of);
+      launch_kernel(spec_accept_kernel, wc, threads, smem, st, /*dependent=*/head->ring == 0, lg, lse, msg + w0 * c.n * c.r, xb,
+                    pre, tp, ua, out_accepted + w0, out_next_byte + w0, at<unsigned>(head, L.off_status), wc, wpp, c.n, c.r, c.v,
+                    valid_symbols(c), row_of);
       head->launches++;
       pt.end();
       if ((rcf = check_launch()) != MTPC_OK) return rcf;
@@ -1701,11 +1727,9 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
     pt.end();
     if (rc2 != MTPC_OK) return rc2;
     pt.begin();
-    spec_accept_kernel<<<wc, kAcceptThreads, smem, st>>>(
-        c.family, lg, lse, at<float>(head, L.off_logw) + static_cast<size_t>(p0) * L.sum_rows,
-        tables + static_cast<size_t>(p0) * tstride, xb, pre, tp, ua, out_accepted + w0, out_next_byte + w0,
-        at<unsigned>(head, L.off_status), wc, wpp, c.n, c.r, c.v, valid_symbols(c), L.sum_rows, tstride,
-        at<float>(head, L.off_G) + w0 * c.n * c.r, row_of);
+    launch_kernel(spec_accept_kernel, wc, threads, smem, st, /*dependent=*/head->ring == 0, lg, lse, msg + w0 * c.n * c.r, xb,
+                  pre, tp, ua, out_accepted + w0, out_next_byte + w0, at<unsigned>(head, L.off_status), wc, wpp, c.n, c.r, c.v,
+                  valid_symbols(c), row_of);
     head->launches++;
     pt.end();
     if ((rc2 = check_launch()) != MTPC_OK) return rc2;
@@ -2303,7 +2327,7 @@ extern "C" int mtpc_window_logprob_static(const mtpc_config* cfg, const void* W_
   L.off_G = take(static_cast<size_t>(c.max_positions) * c.n * c.r * 4);
   L.off_logw = take(static_cast<size_t>(c.max_positions) * L.sum_rows * 4);
   L.off_sel = L.off_wemit = L.off_wsum = L.off_hidden = L.off_logits = L.off_unit_lse = 0;   // unused by this call
-  L.off_prefix = L.off_partial = L.off_sum_bias = 0;
+  L.off_prefix = L.off_partial = L.off_sum_bias = L.off_msg = 0;
   L.off_h_hidden = L.off_h_targets = L.off_h_uniforms = L.off_h_bytes = L.off_h_out = 0;
   L.total = off;
   if (L.total > static_cast<size_t>(MTPC_STATIC_SCRATCH_BYTES)) return MTPC_ERR_STATIC_SCRATCH;

@@ -163,7 +163,7 @@ __device__ __forceinline__ void row_grad(const float* row, const float* pc, floa
 // beta_{i-1}[a] = LSE_b(logA_i[a][b] + G[i][b] + beta_i[b]). Posterior of the state: gamma_i = exp(alpha_i + beta_i - log q)
 // = d log q / d G[i, .]; pairwise posterior xi_i[a][b] = exp(alpha_{i-1}[a] + logA_i[a][b] + G[i][b] + beta_i[b] - log q)
 // = d log q / d logA_i[a][b]; through the row softmax of the transition logits: xi_i[a][b] - A_i[a][b] gamma_{i-1}[a].
-// Tables as in circuit_hmm_stream_kernel (static: stride 0; contextual: one set per position inside log omega).
+// Tables as in circuit_hmm_kernel (static: stride 0; contextual: one set per position inside log omega).
 // Contextual: the transition-logit gradients go to dsum (bf16, one row per position). Static: they are summed over
 // the windows into dT [n-1, r, r] (fp32): per CTA in shared memory first, then one atomicAdd per entry and CTA.
 // Shared memory: per warp n*r (alpha) + 2*r*r (tables) + 64 floats; static: + (n-1)*r*r floats per CTA.  r <= 32.
@@ -188,6 +188,7 @@ __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const 
   float* tabs = alphas + n * r;
   float* cvec = tabs + 2 * rr;
   const bool has = lane < r;
+  const HmmLanes l = hmm_lanes(r, lane);
   if (is_static) {
     for (int e = threadIdx.x; e < (n - 1) * rr; e += blockDim.x) acc[e] = 0.f;
     __syncthreads();
@@ -202,7 +203,7 @@ __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const 
     const size_t drow = static_cast<size_t>(w) * a_.dsum_pitch;
     // ---- forward, keeping every alpha_i
     if (len > 1) warp_table_load_async(tabs, tb, rr, lane);
-    float alpha = has ? lw[lane] + g[lane] : -CUDART_INF_F;
+    float alpha = l.active ? lw[l.k] + g[l.k] : -CUDART_INF_F;
     if (has) alphas[lane] = alpha;
     for (int i = 1; i < len; ++i) {
       if (i + 1 < len) {
@@ -212,20 +213,13 @@ __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const 
         cp_async_wait<0>();
       }
       __syncwarp();
-      const float* A = tabs + ((i - 1) & 1) * rr;
-      float m = alpha;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, off));
-      cvec[lane] = has ? __expf(alpha - m) : 0.f;
-      __syncwarp();
-      if (has) {
-        const float s = hmm_matvec(cvec, A, lane, r);
-        alpha = (m == -CUDART_INF_F) ? -CUDART_INF_F : g[i * r + lane] + m + __logf(s);
-        alphas[i * r + lane] = alpha;
-      }
+      const float c = hmm_forward_step<true>(alpha, cvec, tabs + ((i - 1) & 1) * rr, l, r);
+      alpha = l.active ? c + g[i * r + l.k] : -CUDART_INF_F;
+      if (has) alphas[i * r + lane] = alpha;
       __syncwarp();
     }
-    const float logq = warp_lse(alpha, has);
+    if (!has) alpha = -CUDART_INF_F;                                     // (the other parts' copies)
+    const float logq = warp_lse_nan(alpha);
     if (lane == 0 && a_.out != nullptr) a_.out[w] = logq;
     // ---- backward: tables in reverse order; the table of step len - 1 is still in its buffer
     float beta = 0.f;                                                    // beta_{len-1}
@@ -357,6 +351,7 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
   float* cvec = tabs + 2 * rr;                                           // G[i] - alpha_i (log domain)
   float* dvec = cvec + 32;                                               // abar_i (plain)
   const bool has = lane < r;
+  const HmmLanes l = hmm_lanes(r, lane);
   if (is_static) {
     for (int e = threadIdx.x; e < (n - 1) * rr; e += blockDim.x) acc[e] = 0.f;
     __syncthreads();
@@ -371,7 +366,7 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
     const size_t drow = static_cast<size_t>(w) * a_.dsum_pitch;
     // ---- forward, keeping every alpha_i
     if (n > 1) warp_table_load_async(tabs, tb, rr, lane);
-    float alpha = has ? lw[lane] + g[lane] : -CUDART_INF_F;
+    float alpha = l.active ? lw[l.k] + g[l.k] : -CUDART_INF_F;
     if (has) alphas[lane] = alpha;
     for (int i = 1; i < n; ++i) {
       if (i + 1 < n) {
@@ -381,20 +376,13 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
         cp_async_wait<0>();
       }
       __syncwarp();
-      const float* A = tabs + ((i - 1) & 1) * rr;
-      float m = alpha;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, off));
-      cvec[lane] = has ? __expf(alpha - m) : 0.f;
-      __syncwarp();
-      if (has) {
-        const float s = hmm_matvec(cvec, A, lane, r);
-        alpha = (m == -CUDART_INF_F) ? -CUDART_INF_F : g[i * r + lane] + m + __logf(s);
-        alphas[i * r + lane] = alpha;
-      }
+      const float c = hmm_forward_step<true>(alpha, cvec, tabs + ((i - 1) & 1) * rr, l, r);
+      alpha = l.active ? c + g[i * r + l.k] : -CUDART_INF_F;
+      if (has) alphas[i * r + lane] = alpha;
       __syncwarp();
     }
-    float lp = warp_lse(alpha, has);                                     // log p_{n-1}: the joint
+    if (!has) alpha = -CUDART_INF_F;                                     // (the other parts' copies)
+    const float lp = warp_lse_nan(alpha);                                // log p_{n-1}: the joint
     if (lane == 0 && a_.out != nullptr) a_.out[w] = lp;
     // ---- reverse sweep: tables in reverse order; the table of step n - 1 is still in its buffer
     float abar = has ? cw[n - 1] * __expf(alpha - lp) : 0.f;

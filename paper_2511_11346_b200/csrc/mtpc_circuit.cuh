@@ -32,12 +32,25 @@ __device__ __forceinline__ float warp_lse(float val, bool has) {
   return m + __logf(s);
 }
 
+// Warp-wide maximum; NaN if any lane holds one (so that refused evidence is not lost to the maximum).
+__device__ __forceinline__ float warp_max_nan(float x) {
+  float m;
+  asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+  return m;
+}
+// log-sum-exp of the `count` floats x[0], x[1], ... by one thread. All -inf: -inf; any NaN: NaN.
+__device__ __forceinline__ float thread_lse(const float* x, int count) {
+  float m = -CUDART_INF_F;
+  for (int k = 0; k < count; ++k) m = fmaxf(m, x[k]);
+  if (m == -CUDART_INF_F) m = 0.f;
+  float s = 0.f;
+  for (int k = 0; k < count; ++k) s += __expf(x[k] - m);
+  return m + __logf(s);
+}
+
 // Eq. (CP): out[w] = LSE_k( log omega[p, k] + sum_i G[w, i, k] ),  p = w / wpp.
-// With `prefix` (may be NULL) the kernel also writes prefix[w, i] = log q(x_0..x_i), the joint with the later bytes
-// summed out (Algorithm 3's marginals): for a mixture that is the same log-sum-exp over the first i+1 slots only.
 __global__ void circuit_cp_kernel(const float* __restrict__ G, const float* __restrict__ logw,
-                                  float* __restrict__ out, float* __restrict__ prefix, int W, int wpp, int n, int r,
-                                  int sum_rows, int raw_mixture) {
+                                  float* __restrict__ out, int W, int wpp, int n, int r, int sum_rows, int raw_mixture) {
   grid_dependency_wait();   // G and log omega come from the kernel before this one
   const int w = blockIdx.x * kCircuitWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -58,34 +71,6 @@ __global__ void circuit_cp_kernel(const float* __restrict__ G, const float* __re
     }
     norm = m + __logf(s);
   }
-  if (prefix != nullptr) {
-    // running sums of up to 4 units per lane (r <= 128); one warp log-sum-exp per slot
-    float a[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) a[q] = (lane + 32 * q < r) ? lw[lane + 32 * q] : 0.f;
-    float last = 0.f;
-    for (int i = 0; i < n; ++i) {
-      float m = -CUDART_INF_F, s = 0.f;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int k = lane + 32 * q;
-        if (k < r) {
-          a[q] += g[i * r + k];
-          if (a[q] != a[q]) { m = 0.f; s = a[q]; } else lse_merge(m, s, a[q], 1.f);
-        }
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float m2 = __shfl_xor_sync(kFull, m, off);
-        const float s2 = __shfl_xor_sync(kFull, s, off);
-        lse_merge(m, s, m2, s2);
-      }
-      last = m + __logf(s) - norm;
-      if (lane == 0) prefix[static_cast<size_t>(w) * n + i] = last;
-    }
-    if (lane == 0 && out != nullptr) out[w] = last;
-    return;
-  }
   float m = -CUDART_INF_F, s = 0.f;
   for (int k = lane; k < r; k += 32) {
     float a = lw[k];
@@ -102,54 +87,63 @@ __global__ void circuit_cp_kernel(const float* __restrict__ G, const float* __re
   if (lane == 0) out[w] = m + __logf(s) - norm;
 }
 
+// ---------------------------------------------------------------- prefix marginals and slot messages
+// The three kernels below write, for every window,
+//   prefix[w, i] = log q(x_0..x_i), the joint with the later bytes summed out (Algorithm 3's marginals; may be NULL),
+//   msg[w, i, k] = the log-weight of input unit k of slot i given the bytes before it, up to a constant per (w, i) (may
+//                  be NULL): log of p(the latent that owns slot i is k, x_0..x_{i-1}). q(x_i | x_<i) is the mixture of the
+//                  slot's input units under softmax(msg[w, i, :]), which is all the acceptance stage needs to know of the
+
+// Mixture: msg_i[k] = log omega_k + sum_{j<i} G[j, k], prefix_i = LSE_k msg_{i+1}[k]. One warp per window: lane = component
+// for the running sums (all loads of eight slots in flight), then lane = slot for the log-sum-exps, through a padded
+// shared tile, so that no slot waits for another one's reduction. Shared memory: cp_prefix_smem_floats per warp.
+constexpr int kCpTileSlots = 32;
+__host__ __device__ inline int cp_prefix_warp_floats(int n, int r) { return (n < kCpTileSlots ? n : kCpTileSlots) * (r + 1); }
+__global__ void circuit_cp_prefix_kernel(const float* __restrict__ G, const float* __restrict__ logw,
+                                         float* __restrict__ out, float* __restrict__ prefix, float* __restrict__ msg, int W,
+                                         int wpp, int n, int r, int sum_rows, int raw_mixture) {
+  extern __shared__ __align__(16) float sm[];
+  grid_launch_dependents();
+  grid_dependency_wait();   // G and log omega come from the kernel before this one
+  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (w >= W) return;
+  float* tile = sm + static_cast<size_t>(threadIdx.x >> 5) * cp_prefix_warp_floats(n, r);
+  const float* g = G + static_cast<size_t>(w) * n * r;
+  const float* lw = logw + static_cast<size_t>(w / wpp) * sum_rows;
+  float* mw = msg != nullptr ? msg + static_cast<size_t>(w) * n * r : nullptr;
+  float norm = 0.f;                                 // see circuit_cp_kernel
+  if (raw_mixture) norm = thread_lse(lw, r);
+  for (int i0 = 0; i0 < n; i0 += kCpTileSlots) {
+    const int nc = min(kCpTileSlots, n - i0);
+    for (int k = lane; k < r; k += 32) {
+      float a = i0 == 0 ? lw[k] : tile[(kCpTileSlots - 1) * (r + 1) + k];
+      for (int c0 = 0; c0 < nc; c0 += 8) {
+        float gv[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) gv[q] = c0 + q < nc ? g[(i0 + c0 + q) * r + k] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (c0 + q < nc) {
+            if (mw != nullptr) mw[(i0 + c0 + q) * r + k] = a;
+            a += gv[q];
+            tile[(c0 + q) * (r + 1) + k] = a;
+          }
+      }
+    }
+    __syncwarp();
+    if (lane < nc) {
+      const float res = thread_lse(tile + lane * (r + 1), r) - norm;
+      if (prefix != nullptr) prefix[static_cast<size_t>(w) * n + i0 + lane] = res;
+      if (out != nullptr && i0 + lane == n - 1) out[w] = res;
+    }
+    __syncwarp();
+  }
+}
+
 // Eq. (BTree), bottom-up over the heap-ordered latent tree. Node j >= 1 has the table
 // logOmega_j[a][b] = logw[p, r + (j-1) r^2 + a r + b] (parent's value a, own value b); the deepest internal node
 // n/2-1+m multiplies the input units of tokens 2m and 2m+1. prod[j][z] is the product unit under z_j = z.
-
-// One sum layer seen from the parent: returns, for lane = parent value z, LSE_b(logOmega_c[z][b] + pc[b]).
-// tab: the child's r x r table in global memory; pc: r floats in shared memory (written before the call; the
-// function synchronises the warp); table: r * (r+1) floats of per-warp shared scratch.
-// An r x r table from global memory into a padded shared tile (row pitch r + 1), by one warp. ROWS > 1: that many rows'
-// loads are in flight before the first store - for a kernel where one warp walks many tables on its own (a load-store pair
-// per row costs one memory round trip per row); a kernel with many such warps per SM hides that latency and is better
-// off with the plain loop's few registers.
-template <int ROWS>
-__device__ __forceinline__ void btree_stage_table(const float* __restrict__ tab, float* table, int lane, int r) {
-  const bool has = lane < r;
-  if (ROWS == 1) {
-    for (int a = 0; a < r; ++a)
-      if (has) table[a * (r + 1) + lane] = tab[a * r + lane];
-    return;
-  }
-  for (int a0 = 0; a0 < r; a0 += ROWS) {
-    float t[ROWS];
-#pragma unroll
-    for (int q = 0; q < ROWS; ++q) t[q] = (has && a0 + q < r) ? tab[(a0 + q) * r + lane] : 0.f;
-#pragma unroll
-    for (int q = 0; q < ROWS; ++q)
-      if (has && a0 + q < r) table[(a0 + q) * (r + 1) + lane] = t[q];
-  }
-}
-
-template <int ROWS = 1>
-__device__ __forceinline__ float btree_sum_layer(const float* __restrict__ tab, const float* pc, float* table,
-                                                 int lane, int r) {
-  const bool has = lane < r;
-  btree_stage_table<ROWS>(tab, table, lane, r);    // coalesced rows -> padded shared tile
-  __syncwarp();
-  float res = 0.f;
-  if (has) {
-    const float* row = table + lane * (r + 1);     // row z = lane, over the child's values b
-    float m = -CUDART_INF_F;
-    for (int b = 0; b < r; ++b) m = fmaxf(m, row[b] + pc[b]);
-    float s = 0.f;
-    for (int b = 0; b < r; ++b) s += __expf(row[b] + pc[b] - m);
-    res = (m == -CUDART_INF_F) ? -CUDART_INF_F : m + __logf(s);
-    if (s != s) res = s;                           // NaN evidence must survive the max
-  }
-  __syncwarp();
-  return res;
-}
 
 // Dynamic work distribution for the kernels whose cost per window is large: every warp takes the next window index
 // from a counter the host zeroes before the launch, so that all SMs stay busy until the last window.
@@ -184,8 +178,8 @@ __device__ __forceinline__ void warp_table_load_async(float* dst, const float* _
   }
   cp_async_commit();
 }
-// The same sum layer as btree_sum_layer on a table already in shared memory, unpadded [z][b]; lane z walks its row
-// starting at column z, so that the 32 lanes hit 32 different banks. R a multiple of 4 (both arrays 16-byte aligned):
+// One sum layer seen from the parent: lane z returns LSE_b(tab[z][b] + pc[b]); the child's table, unpadded [z][b], and its
+// vector pc are in shared memory. Lane z walks its row starting at column z, so that the 32 lanes hit 32 different banks. R a multiple of 4 (both arrays 16-byte aligned):
 // the row and the child's vector are read as float4, rotated by the lane so that a quarter-warp's requests fall in
 // different bank groups, and reduced in registers (max, then sum of exponentials).
 template <int R>
@@ -234,180 +228,367 @@ __device__ __forceinline__ float sum_layer_staged(const float* tab, const float*
   return res;
 }
 
-// Shared memory per warp: (n-1) * r floats of prod + 2 * r * r floats (two staged tables); with PREFIX another
-// (n-1) * r floats (the sum-layer outputs S[c][z], kept for the prefix passes) + r floats.  r <= 32.
+// Joint log-probability alone. Shared memory per warp: (n-1) * r floats of prod + 2 * r * r floats (two staged tables). r <= 32.
 // The n-2 tables of a position (57 KB at n = 16, r = 32) are read exactly once, in the order the bottom-up pass
 // needs them, through a two-deep cp.async pipeline: this kernel is bound by that stream from HBM.
-// PREFIX: also writes prefix[w, i] = log q(x_0..x_i). Summing the later bytes out sets their input units to one,
-// so every subtree right of token i evaluates to one, every subtree left of it keeps its value, and only the
-// nodes on the path from token i's owner to the root have to be re-evaluated.
-__host__ __device__ inline int btree_warp_floats(int n, int r, bool with_prefix) {
-  return (n - 1) * r + 2 * r * r + (with_prefix ? (n - 1) * r + r : 0);
-}
+__host__ __device__ inline int btree_warp_floats(int n, int r) { return (n - 1) * r + 2 * r * r; }
 
-template <bool PREFIX>
-__global__ void circuit_btree_kernel(const float* __restrict__ G, const float* __restrict__ logw,
-                                     float* __restrict__ out, float* __restrict__ prefix, unsigned* work_counter,
-                                     int W, int wpp, int n, int r, int sum_rows) {
+__global__ void circuit_btree_kernel(const float* __restrict__ G, const float* __restrict__ logw, float* __restrict__ out,
+                                     unsigned* work_counter, int W, int wpp, int n, int r, int sum_rows) {
   extern __shared__ __align__(16) float sm[];
   grid_dependency_wait();   // G, log omega and the zeroed work counter come from the kernels before this one
   const int wib = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  float* prod = sm + static_cast<size_t>(wib) * btree_warp_floats(n, r, PREFIX);
-  float* tabs = prod + (n - 1) * r;                // two tables; the prefix passes reuse the space as one padded table
-  float* table = tabs;
-  float* S = tabs + 2 * r * r;                     // PREFIX only
-  float* cur = S + (n - 1) * r;                    // PREFIX only
+  float* prod = sm + static_cast<size_t>(wib) * btree_warp_floats(n, r);
+  float* tabs = prod + (n - 1) * r;
   const bool has = lane < r;
   const int first_leaf_node = n / 2 - 1;
   const int rr = r * r;
   const int ntab = n - 2;                          // table t belongs to child c(t) of node j(t), deepest parents first
   auto child_of = [&](int t) { return 2 * (first_leaf_node - 1 - (t >> 1)) + 1 + (t & 1); };
   for (int w = next_window(work_counter, lane); w < W; w = next_window(work_counter, lane)) {
-  const float* g = G + static_cast<size_t>(w) * n * r;
-  const float* lw = logw + static_cast<size_t>(w / wpp) * sum_rows;
-  if (ntab > 0) warp_table_load_async(tabs, lw + r + static_cast<size_t>(child_of(0) - 1) * rr, rr, lane);
-  for (int j = n - 2; j >= first_leaf_node; --j) {
-    const int m = j - first_leaf_node;
-    if (has) prod[j * r + lane] = g[(2 * m) * r + lane] + g[(2 * m + 1) * r + lane];
-  }
-  __syncwarp();
-  float acc = 0.f;
-  for (int t = 0; t < ntab; ++t) {
-    const int c = child_of(t);
-    if (t + 1 < ntab) {
-      warp_table_load_async(tabs + ((t + 1) & 1) * rr, lw + r + static_cast<size_t>(child_of(t + 1) - 1) * rr, rr, lane);
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncwarp();                                  // table t is in shared memory for every lane
-    const float sc = sum_layer_staged(tabs + (t & 1) * rr, prod + c * r, lane, r);
-    if (PREFIX && has) S[c * r + lane] = sc;
-    acc += sc;
-    if (t & 1) {                                   // both children of node j done
-      if (has) prod[((c - 2) >> 1) * r + lane] = acc;
-      acc = 0.f;
-    }
-    __syncwarp();                                  // the buffer may be overwritten, prod[j] may be read
-  }
-  const float res = warp_lse(has ? lw[lane] + prod[lane] : 0.f, has);
-  if (lane == 0 && out != nullptr) out[w] = res;
-  if (PREFIX) {
-    if (lane == 0) prefix[static_cast<size_t>(w) * n + n - 1] = res;
-    for (int i = 0; i < n - 1; ++i) {
-      int c = first_leaf_node + (i >> 1);
-      bool full = (i & 1) != 0;                    // both tokens of the owner are inside the prefix
-      float val = has ? (full ? prod[c * r + lane] : g[i * r + lane]) : 0.f;
-      while (c > 0) {
-        const bool is_right = (c & 1) == 0;
-        float sc;
-        if (full) {
-          sc = has ? S[c * r + lane] : 0.f;
-        } else {
-          if (has) cur[lane] = val;
-          __syncwarp();
-          sc = btree_sum_layer(lw + r + static_cast<size_t>(c - 1) * r * r, cur, table, lane, r);
-        }
-        val = sc + ((is_right && has) ? S[(c - 1) * r + lane] : 0.f);   // left sibling: inside; right sibling: one
-        full = full && is_right;
-        c = (c - 1) >> 1;
-      }
-      const float pre = warp_lse(has ? lw[lane] + val : 0.f, has);
-      if (lane == 0) prefix[static_cast<size_t>(w) * n + i] = pre;
-    }
-  }
-  __syncwarp();                                    // the next window reuses the warp's shared memory
-  }
-}
-
-// sum_a e[a] * exp(A[a][lane]) for lane < r: e (r floats) and the table A [r, r] are in shared memory. Every lane reads
-// four e's per request (a broadcast) and keeps four independent accumulation chains.
-__device__ __forceinline__ float hmm_matvec(const float* evec, const float* A, int lane, int r) {
-  float s = 0.f;
-  if ((r & 3) == 0) {
-    const float4* e4 = reinterpret_cast<const float4*>(evec);
-    float s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll 4
-    for (int a = 0; a < r; a += 4) {
-      const float4 ev = e4[a >> 2];
-      s = fmaf(ev.x, __expf(A[a * r + lane]), s);
-      s1 = fmaf(ev.y, __expf(A[(a + 1) * r + lane]), s1);
-      s2 = fmaf(ev.z, __expf(A[(a + 2) * r + lane]), s2);
-      s3 = fmaf(ev.w, __expf(A[(a + 3) * r + lane]), s3);
-    }
-    s = (s + s1) + (s2 + s3);
-  } else {
-    for (int a = 0; a < r; ++a) s = fmaf(evec[a], __expf(A[a * r + lane]), s);
-  }
-  return s;
-}
-
-// Eq. (HMM), forward recursion over the window: alpha_0[k] = log pi[k] + G[0,k];
-// alpha_i[k] = G[i,k] + LSE_a(alpha_{i-1}[a] + logA_i[a][k]); out = LSE_k alpha_{n-1}[k].  r <= 32.
-// The inner log-sum-exp is taken as one scaled matrix-vector product per step: with m = max_a alpha_{i-1}[a],
-// alpha_i[k] = G[i,k] + m + log sum_a exp(alpha_{i-1}[a] - m) exp(logA_i[a][k]).
-// The transition tables are streamed per window: position p = w / wpp reads logA_i[a][k] at
-// tables[p * table_stride + (i-1) r^2 + a r + k]. Contextual transitions (App. H): tables = log omega + r and
-// table_stride = sum_rows, 28 KB per position at n = 8, r = 32, read exactly once from HBM, which bounds the kernel.
-// Static transitions: table_stride = 0, the one set of tables stays in L2. One warp per window, lane = state; table
-// i+1 is copied into shared memory by cp.async while table i is reduced (kHmmDepth buffers per warp).
-// Shared memory per warp: kHmmDepth * r * r + 32 floats. With `prefix` (may be NULL) also writes prefix[w, i] = LSE_k alpha_i[k].
-constexpr int kHmmDepth = 2;   // table buffers per warp (deeper pipelines were measured and bought nothing)
-__global__ void circuit_hmm_stream_kernel(const float* __restrict__ G, const float* __restrict__ logw,
-                                          const float* __restrict__ tables, int table_stride,
-                                          float* __restrict__ out, float* __restrict__ prefix, unsigned* work_counter,
-                                          int W, int wpp, int n, int r, int sum_rows) {
-  extern __shared__ __align__(16) float sm[];
-  grid_dependency_wait();   // G, log omega and the zeroed work counter come from the kernels before this one
-  const int lane = threadIdx.x & 31;
-  const int rr = r * r;
-  float* tabs = sm + static_cast<size_t>(threadIdx.x >> 5) * (kHmmDepth * rr + 32);
-  float* evec = tabs + kHmmDepth * rr;
-  const bool has = lane < r;
-  for (int w = next_window(work_counter, lane); w < W; w = next_window(work_counter, lane)) {
     const float* g = G + static_cast<size_t>(w) * n * r;
     const float* lw = logw + static_cast<size_t>(w / wpp) * sum_rows;
-    const float* tb = tables + static_cast<size_t>(w / wpp) * table_stride;   // logA_1 .. logA_{n-1} of this position
-    // kHmmDepth - 1 tables are in flight ahead of the one being reduced; every step commits exactly one copy group (an
-    // empty one once the tables run out), so "all but the newest kHmmDepth - 1 groups" always means "table i has landed"
-#pragma unroll
-    for (int s = 0; s < kHmmDepth - 1; ++s) {
-      if (s < n - 1) warp_table_load_async(tabs + s * rr, tb + static_cast<size_t>(s) * rr, rr, lane);
-      else cp_async_commit();
+    if (ntab > 0) warp_table_load_async(tabs, lw + r + static_cast<size_t>(child_of(0) - 1) * rr, rr, lane);
+    for (int j = n - 2; j >= first_leaf_node; --j) {
+      const int m = j - first_leaf_node;
+      if (has) prod[j * r + lane] = g[(2 * m) * r + lane] + g[(2 * m + 1) * r + lane];
     }
-    float alpha = has ? lw[lane] + g[lane] : -CUDART_INF_F;
-    for (int i = 1; i < n; ++i) {
-      const int nxt = i - 1 + kHmmDepth - 1;                 // index of the table to fetch now
-      if (nxt < n - 1) warp_table_load_async(tabs + (nxt % kHmmDepth) * rr, tb + static_cast<size_t>(nxt) * rr, rr, lane);
-      else cp_async_commit();
-      cp_async_wait<kHmmDepth - 1>();
-      __syncwarp();                                      // table i is in shared memory for every lane
-      if (prefix != nullptr) {
-        const float pre = warp_lse(alpha, has);
-        if (lane == 0) prefix[static_cast<size_t>(w) * n + i - 1] = pre;
+    __syncwarp();
+    float acc = 0.f;
+    for (int t = 0; t < ntab; ++t) {
+      const int c = child_of(t);
+      if (t + 1 < ntab) {
+        warp_table_load_async(tabs + ((t + 1) & 1) * rr, lw + r + static_cast<size_t>(child_of(t + 1) - 1) * rr, rr, lane);
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
       }
-      const float* A = tabs + ((i - 1) % kHmmDepth) * rr;
-      const float gi = has ? g[i * r + lane] : 0.f;
-      float m = alpha;
-      const bool poisoned = __any_sync(kFull, alpha != alpha);   // NaN evidence (a target or a draw that was refused)
+      __syncwarp();                                  // table t is in shared memory for every lane
+      acc += sum_layer_staged(tabs + (t & 1) * rr, prod + c * r, lane, r);
+      if (t & 1) {                                   // both children of node j done
+        if (has) prod[((c - 2) >> 1) * r + lane] = acc;
+        acc = 0.f;
+      }
+      __syncwarp();                                  // the buffer may be overwritten, prod[j] may be read
+    }
+    const float res = warp_lse(has ? lw[lane] + prod[lane] : 0.f, has);
+    if (lane == 0) out[w] = res;
+    __syncwarp();                                    // the next window reuses the warp's shared memory
+  }
+}
+
+// LSE_z(in[z] + tab[z][lane]): the message down to a child with value `lane`; tab [r, r] and in [r] in shared memory.
+template <int R>
+__device__ __forceinline__ float down_layer_vec(const float* tab, const float* in, int lane) {
+  if (lane >= R) return 0.f;
+  const float4* in4 = reinterpret_cast<const float4*>(in);
+  float v[R];
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, off));
-      // e[a] = exp(alpha[a] - m) goes through shared memory: every lane then reads four of them per request
-      // (a broadcast) instead of one shuffle each
-      evec[lane] = has ? __expf(alpha - m) : 0.f;
+  for (int q = 0; q < R / 4; ++q) {
+    const float4 a = in4[q];
+    v[4 * q] = a.x + tab[(4 * q) * R + lane];
+    v[4 * q + 1] = a.y + tab[(4 * q + 1) * R + lane];
+    v[4 * q + 2] = a.z + tab[(4 * q + 2) * R + lane];
+    v[4 * q + 3] = a.w + tab[(4 * q + 3) * R + lane];
+  }
+  float m = v[0];
+#pragma unroll
+  for (int q = 1; q < R; ++q) m = fmaxf(m, v[q]);
+  if (m == -CUDART_INF_F) m = 0.f;
+  float s = 0.f;
+#pragma unroll
+  for (int q = 0; q < R; ++q) s += __expf(v[q] - m);
+  return m + __logf(s);                            // NaN evidence survives through the sum
+}
+__device__ __forceinline__ float down_layer(const float* tab, const float* in, int lane, int r) {
+  switch (r) {
+    case 32: return down_layer_vec<32>(tab, in, lane);
+    case 16: return down_layer_vec<16>(tab, in, lane);
+    case 8: return down_layer_vec<8>(tab, in, lane);
+    case 4: return down_layer_vec<4>(tab, in, lane);
+    default: break;
+  }
+  if (lane >= r) return 0.f;
+  float m = -CUDART_INF_F;
+  for (int z = 0; z < r; ++z) m = fmaxf(m, in[z] + tab[z * r + lane]);
+  if (m == -CUDART_INF_F) m = 0.f;
+  float s = 0.f;
+  for (int z = 0; z < r; ++z) s += __expf(in[z] + tab[z * r + lane] - m);
+  return m + __logf(s);
+}
+// log-sum-exp of one value per lane (lanes without one pass -inf). All lanes return it.
+__device__ __forceinline__ float warp_lse_nan(float x) {
+  float m = warp_max_nan(x);
+  if (m == -CUDART_INF_F) m = 0.f;
+  float s = __expf(x - m);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
+  return m + __logf(s);
+}
+
+// Binary tree: every prefix marginal and slot message from one upward and one downward sweep. With
+//   S[c][z] = LSE_b(logOmega_c[z][b] + prod[c][b])  the subtree of node c under its parent's value z (all its tokens seen), and
+//   D[c][b] = log p(z_c = b, every token left of c's subtree),
+// D[root] = log omega_root, D[left child][b] = LSE_z(D[j][z] + logOmega[z][b]), D[right child][b] = LSE_z(D[j][z] + S[left
+// sibling][z] + logOmega[z][b]); at the node that owns the tokens 2m and 2m+1: msg_{2m} = D, msg_{2m+1} = D + G[2m], and the
+// prefix marginals are their log-sum-exps with the token's own evidence added. S is only needed inside left subtrees.
+// That is 2 (n - 2) table passes at most for all n prefixes; re-evaluating each prefix's path to the root took n log n.
+// One CTA per window, a warp per node of a level (2 log2 n - 2 levels one after the other instead of 2 (n - 2) tables): the
+// position's tables are fetched into shared memory in one go, so a decode-sized call (fewer windows than SMs) waits for one
+// memory round trip, and a batch has several windows' tables in flight per SM. tables_in_smem == 0 (they do not fit: n = 64 at
+// r = 32): each warp stages the table it needs. A CTA takes a contiguous run of windows and keeps the tables while the
+// position stays the same. Measured against one warp per window and a path per prefix: 4096 windows at n = 16, r = 32:
+// 256 -> 148 us; 108 windows at n = 8: 36 -> 6 us. Shared memory: btree_prefix_smem_floats.
+__host__ __device__ inline size_t btree_prefix_smem_floats(int n, int r, int warps, bool tables_in_smem) {
+  const size_t rr = static_cast<size_t>(r) * r, vec = (static_cast<size_t>(r) + 3) / 4 * 4;
+  return ((tables_in_smem ? (n - 2) * rr : warps * rr) + 3) / 4 * 4 + (2 * static_cast<size_t>(n - 1) + n + warps) * vec;
+}
+__global__ void __launch_bounds__(256) circuit_btree_prefix_kernel(const float* __restrict__ G, const float* __restrict__ logw,
+                                                                   float* __restrict__ out, float* __restrict__ prefix,
+                                                                   float* __restrict__ msg, int W, int wpp, int n, int r,
+                                                                   int sum_rows, int tables_in_smem) {
+  extern __shared__ __align__(16) float sm[];
+  grid_launch_dependents();
+  grid_dependency_wait();   // G and log omega come from the kernels before this one
+  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  const int rr = r * r, vr = (r + 3) / 4 * 4;
+  const bool has = lane < r;
+  float* tabs = sm;
+  float* S = sm + ((tables_in_smem ? (n - 2) * rr : warps * rr) + 3) / 4 * 4;
+  float* D = S + (n - 1) * vr;
+  float* gs = D + (n - 1) * vr;                    // evidence of the window [n][vr]
+  float* vec = gs + n * vr + wib * vr;             // one vector per warp
+  const int owners = n / 2, first_leaf_node = owners - 1;
+  const int depth = 31 - __clz(owners);            // the owners' level; level L holds the nodes 2^L - 1 .. 2^(L+1) - 2
+  const int w0 = static_cast<int>(static_cast<long long>(blockIdx.x) * W / gridDim.x);
+  const int w1 = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * W / gridDim.x);
+  int last_pos = -1;
+  for (int w = w0; w < w1; ++w) {
+    const int pos = w / wpp;
+    const float* lw = logw + static_cast<size_t>(pos) * sum_rows;
+    const float* g = G + static_cast<size_t>(w) * n * r;
+    if (tables_in_smem && pos != last_pos) {
+      const int count = (n - 2) * rr;
+      const bool vec16 = (count & 3) == 0 && ((reinterpret_cast<uintptr_t>(lw + r)) & 15u) == 0;
+      if (vec16) {
+        for (int e = threadIdx.x * 4; e < count; e += blockDim.x * 4) cp_async_16(tabs + e, lw + r + e);
+      } else {
+        for (int e = threadIdx.x; e < count; e += blockDim.x) cp_async_4(tabs + e, lw + r + e);
+      }
+      cp_async_commit();
+      last_pos = pos;
+    }
+    for (int e = threadIdx.x; e < n * r; e += blockDim.x) gs[(e / r) * vr + e % r] = g[e];
+    if (threadIdx.x < r) D[threadIdx.x] = lw[threadIdx.x];
+    cp_async_wait<0>();
+    __syncthreads();
+    auto table_of = [&](int c) -> const float* {   // node c's table; not resident: staged into the warp's own tile
+      if (tables_in_smem) return tabs + (c - 1) * rr;
+      warp_table_load_async(tabs + wib * rr, lw + r + static_cast<size_t>(c - 1) * rr, rr, lane);
+      cp_async_wait<0>();
       __syncwarp();
-      if (has) {
-        const float s = hmm_matvec(evec, A, lane, r);
-        alpha = (m == -CUDART_INF_F) ? -CUDART_INF_F : gi + m + __logf(s);
-        if (poisoned) alpha = CUDART_NAN_F;              // the max above skips NaN: it would be lost when every state is NaN
+      return tabs + wib * rr;
+    };
+    for (int L = depth; L >= 1; --L) {             // upward, without the nodes on the right edge
+      for (int c = (1 << L) - 1 + wib; c < (2 << L) - 2; c += warps) {
+        if (has) {
+          vec[lane] = L == depth ? gs[2 * (c - first_leaf_node) * vr + lane] + gs[(2 * (c - first_leaf_node) + 1) * vr + lane]
+                                 : S[(2 * c + 1) * vr + lane] + S[(2 * c + 2) * vr + lane];
+        }
+        __syncwarp();
+        const float sc = sum_layer_staged(table_of(c), vec, lane, r);
+        if (has) S[c * vr + lane] = sc;
+        __syncwarp();
       }
-      __syncwarp();                                      // the buffers may be overwritten
+      __syncthreads();
     }
-    const float res = warp_lse(alpha, has);
-    if (lane == 0) {
-      if (out != nullptr) out[w] = res;
-      if (prefix != nullptr) prefix[static_cast<size_t>(w) * n + n - 1] = res;
+    for (int L = 1; L <= depth; ++L) {             // downward
+      for (int c = (1 << L) - 1 + wib; c <= (2 << L) - 2; c += warps) {
+        if (has) vec[lane] = D[((c - 1) >> 1) * vr + lane] + ((c & 1) ? 0.f : S[(c - 1) * vr + lane]);
+        __syncwarp();
+        const float dc = down_layer(table_of(c), vec, lane, r);
+        if (has) D[c * vr + lane] = dc;
+        __syncwarp();
+      }
+      __syncthreads();
+    }
+    for (int m = wib; m < owners; m += warps) {    // the tokens 2m and 2m + 1
+      const float d = has ? D[(first_leaf_node + m) * vr + lane] : -CUDART_INF_F;
+      const float d1 = has ? d + gs[2 * m * vr + lane] : -CUDART_INF_F;
+      const float d2 = has ? d1 + gs[(2 * m + 1) * vr + lane] : -CUDART_INF_F;
+      if (msg != nullptr && has) {
+        float* mw = msg + (static_cast<size_t>(w) * n + 2 * m) * r + lane;
+        mw[0] = d;
+        mw[r] = d1;
+      }
+      const float p0 = warp_lse_nan(d1), p1 = warp_lse_nan(d2);
+      if (lane == 0) {
+        if (prefix != nullptr) {
+          prefix[static_cast<size_t>(w) * n + 2 * m] = p0;
+          prefix[static_cast<size_t>(w) * n + 2 * m + 1] = p1;
+        }
+        if (out != nullptr && m == owners - 1) out[w] = p1;
+      }
+    }
+    __syncthreads();                               // shared memory is reused by the next window
+  }
+}
+
+// Lanes of a warp that runs an HMM recursion over r <= 32 states (r a power of two): lane = (part, state); with r < 32 the
+// rows of a transition table are shared out over min(32 / r, r) parts.
+struct HmmLanes {
+  int k, part, parts, rows;
+  bool active;
+};
+__device__ __forceinline__ HmmLanes hmm_lanes(int r, int lane) {
+  HmmLanes l;
+  l.parts = min(32 / r, r);
+  l.rows = r / l.parts;
+  l.k = lane & (r - 1);
+  l.part = lane / r;
+  l.active = lane < r * l.parts;
+  return l;
+}
+// One step of the forward recursion: LSE_a(alpha[a] + logA[a][k]) = m + log sum_a exp(alpha[a] - m) A[a][k] for lane's state k
+// (every part returns it). alpha: per active lane, -inf elsewhere; NaN in any of them reaches every state. A [r, r] in shared
+// memory holds probabilities (LOG_TABLE: their logarithms); ev: 32 floats of the warp's shared memory, not reused before the
+// warp's next synchronisation. Every kernel that runs the recursion takes this step, so they return the same bits.
+template <bool LOG_TABLE>
+__device__ __forceinline__ float hmm_forward_step(float alpha, float* ev, const float* A, const HmmLanes& l, int r) {
+  float m = warp_max_nan(alpha);
+  if (m == -CUDART_INF_F) m = 0.f;
+  if (l.part == 0) ev[l.k] = __expf(alpha - m);
+  __syncwarp();
+  auto entry = [&](float a) { return LOG_TABLE ? __expf(a) : a; };
+  const float* col = A + l.part * l.rows * r + l.k;
+  const float* ep = ev + l.part * l.rows;
+  float s = 0.f;
+  if (l.rows == 32) {                                    // r = 32: four chains, the vector read four values at a time
+    const float4* e4 = reinterpret_cast<const float4*>(ep);
+    float s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const float4 e = e4[a];
+      s = fmaf(e.x, entry(col[(4 * a) * 32]), s);
+      s1 = fmaf(e.y, entry(col[(4 * a + 1) * 32]), s1);
+      s2 = fmaf(e.z, entry(col[(4 * a + 2) * 32]), s2);
+      s3 = fmaf(e.w, entry(col[(4 * a + 3) * 32]), s3);
+    }
+    s = (s + s1) + (s2 + s3);
+  } else if (l.active) {
+#pragma unroll 4
+    for (int a = 0; a < l.rows; ++a) s = fmaf(ep[a], entry(col[a * r]), s);
+  }
+  for (int off = r; off < r * l.parts; off <<= 1) s += __shfl_xor_sync(kFull, s, off);
+  return m + __logf(s);
+}
+
+// Eq. (HMM), forward recursion over the window: with msg_0 = log pi and alpha_i[k] = msg_i[k] + G[i,k],
+//   msg_i[k] = LSE_a(alpha_{i-1}[a] + logA_i[a][k]) = m + log sum_a exp(alpha_{i-1}[a] - m) A_i[a][k],  m = max_a alpha_{i-1}[a],
+//   prefix_i = LSE_k alpha_i[k], out = prefix_{n-1}.  r <= 32.
+// Position p = w / wpp reads logA_i[a][k] at tables[p * table_stride + (i-1) r^2 + a r + k]: contextual transitions (App. H)
+// have table_stride = sum_rows (28 KB per position at n = 8, r = 32, read once: the HBM stream that bounds the call then),
+// static ones table_stride = 0.
+// A CTA's warps work on windows that share tables. The tables are turned into probabilities on their way into shared
+// memory, by all threads: once per CTA for static transitions, once per position for contextual ones, so that a step of the
+// recursion is one warp maximum, 32 multiply-adds per lane and one logarithm, with no exponential of a table entry and no
+// memory round trip in it. Tables that do not fit (n = 64 at r = 32) go through in chunks of chunk_tables. The prefix log-sum-exps are taken at the
+// end, lane = slot. Measured against one warp per window streaming log tables: 8192 windows at n = 8, r = 32: 42 -> 22 us;
+// 128 windows at n = 16: 27 -> 13 us. Shared memory: hmm_circuit_smem_floats.
+constexpr int kHmmWarps = 8;
+__host__ __device__ inline int hmm_circuit_warp_floats(int n, int r, bool with_prefix) {
+  return 64 + (with_prefix ? (n * (r + 1) + 3) / 4 * 4 : 0);          // two vectors of 32, alphas [n][r + 1]
+}
+__host__ __device__ inline size_t hmm_circuit_smem_floats(int n, int r, bool with_prefix, int chunk_tables) {
+  return (static_cast<size_t>(chunk_tables) * r * r + 3) / 4 * 4 +
+         static_cast<size_t>(kHmmWarps) * hmm_circuit_warp_floats(n, r, with_prefix);
+}
+__global__ void __launch_bounds__(32 * kHmmWarps) circuit_hmm_kernel(
+    const float* __restrict__ G, const float* __restrict__ logw, const float* __restrict__ tables, int table_stride,
+    float* __restrict__ out, float* __restrict__ prefix, float* __restrict__ msg, int W, int wpp, int n, int r, int sum_rows,
+    int chunk_tables) {
+  extern __shared__ __align__(16) float sm[];
+  grid_launch_dependents();
+  grid_dependency_wait();   // G and log omega come from the kernel before this one
+  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rr = r * r;
+  float* E = sm;
+  float* mine = sm + (chunk_tables * rr + 3) / 4 * 4 + wib * hmm_circuit_warp_floats(n, r, prefix != nullptr);
+  float* evec = mine;                                      // [2][32], alternating
+  float* alphas = mine + 64;
+  const HmmLanes l = hmm_lanes(r, lane);
+  const int k = l.k, part = l.part;
+  const bool active = l.active;
+  // work items: kHmmWarps windows each; contextual tables: of one position
+  const int per_pos = table_stride == 0 ? 0 : (wpp + kHmmWarps - 1) / kHmmWarps;
+  const int items = table_stride == 0 ? (W + kHmmWarps - 1) / kHmmWarps : (W / wpp) * per_pos;
+  int loaded_pos = -1, loaded_first = -1;                  // which tables E holds
+  for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    int pos_tab = 0, w;
+    bool valid;
+    if (table_stride == 0) {
+      w = item * kHmmWarps + wib;
+      valid = w < W;
+    } else {
+      pos_tab = item / per_pos;
+      const int j = (item - pos_tab * per_pos) * kHmmWarps + wib;
+      w = pos_tab * wpp + j;
+      valid = j < wpp;
+    }
+    if (!valid) w = 0;
+    const float* g = G + static_cast<size_t>(w) * n * r;
+    const float* tb = tables + static_cast<size_t>(pos_tab) * table_stride;
+    float* mw = msg != nullptr && valid && part == 0 ? msg + static_cast<size_t>(w) * n * r : nullptr;
+    float alpha = -CUDART_INF_F, gi = 0.f;
+    if (active && valid) {
+      const float l0 = logw[static_cast<size_t>(w / wpp) * sum_rows + k];
+      if (mw != nullptr) mw[k] = l0;
+      alpha = l0 + g[k];
+      if (n > 1) gi = g[r + k];
+    }
+    if (prefix != nullptr && active && part == 0) alphas[k] = alpha;
+    for (int t0 = 0; t0 < n - 1; t0 += chunk_tables) {
+      const int nt = min(chunk_tables, n - 1 - t0);
+      if (loaded_pos != pos_tab || loaded_first != t0) {
+        __syncthreads();                                   // every warp is done with what E held
+        const float* src = tb + static_cast<size_t>(t0) * rr;
+        const int count = nt * rr;
+        if ((count & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+          for (int e = threadIdx.x * 4; e < count; e += 32 * kHmmWarps * 4) {
+            const float4 x = *reinterpret_cast<const float4*>(src + e);
+            *reinterpret_cast<float4*>(E + e) = make_float4(__expf(x.x), __expf(x.y), __expf(x.z), __expf(x.w));
+          }
+        } else {
+          for (int e = threadIdx.x; e < count; e += 32 * kHmmWarps) E[e] = __expf(src[e]);
+        }
+        __syncthreads();
+        loaded_pos = pos_tab;
+        loaded_first = t0;
+      }
+      if (!valid) continue;
+      for (int i = t0 + 1; i <= t0 + nt; ++i) {
+        const float g_next = (active && i + 1 < n) ? g[(i + 1) * r + k] : 0.f;
+        const float c = hmm_forward_step<false>(alpha, evec + (i & 1) * 32, E + (i - 1 - t0) * rr, l, r);
+        if (mw != nullptr && active) mw[i * r + k] = c;
+        alpha = active ? c + gi : -CUDART_INF_F;
+        gi = g_next;
+        if (prefix != nullptr && active && part == 0) alphas[i * (r + 1) + k] = alpha;
+      }
+    }
+    if (valid) {
+      if (prefix != nullptr) {
+        __syncwarp();
+        for (int i = lane; i < n; i += 32) {
+          const float res = thread_lse(alphas + i * (r + 1), r);
+          prefix[static_cast<size_t>(w) * n + i] = res;
+          if (out != nullptr && i == n - 1) out[w] = res;
+        }
+        __syncwarp();
+      } else if (out != nullptr) {
+        const float res = warp_lse_nan(part == 0 ? alpha : -CUDART_INF_F);
+        if (lane == 0) out[w] = res;
+      }
     }
   }
 }

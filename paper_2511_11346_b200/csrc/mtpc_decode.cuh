@@ -542,272 +542,173 @@ __global__ void __launch_bounds__(kSlotThreads, 2) draft_slot_kernel(
 }
 
 // ---------------------------------------------------------------- acceptance stage (Algorithm 3)
-constexpr int kAcceptThreads = 256;
+constexpr int kAcceptMaxThreads = 512;
 
-// Shared memory of one CTA (= one window) of spec_accept_kernel, in floats: the residual weights of the v bytes, the weight and the
-// log-sum-exp of every input unit of the slot (2 r), and for the binary tree the product and sum-layer vectors of every
-// node, one staged table and one vector.
-__host__ __device__ inline size_t accept_warp_floats(int family, int n, int r, int v) {
-  return 4 + static_cast<size_t>(v) + 2 * static_cast<size_t>(r) +                // 4: the accepted length, for all warps
-         (family == 2 ? 2 * static_cast<size_t>(n - 1) * r + static_cast<size_t>(r) * (r + 1) + r : 0);
-}
+// Shared memory of one CTA (= one window) of spec_accept_kernel, in floats: the residual weights of the v bytes; the log-weight
+// of every input unit of the slot (r), whose space then holds the warps' partial sums.
+__host__ __device__ inline size_t accept_smem_floats(int r, int v) { return static_cast<size_t>(v) + (r > 16 ? r : 16); }
+// One thread per byte up to 512 of them.
+inline int accept_threads(int v) { return v >= kAcceptMaxThreads ? kAcceptMaxThreads : (v + 31) / 32 * 32; }
 
-// One CTA per drafted window w (position p = w / wpp): warp 0 runs the tests and the short latent recursions, all
-// warps share the residual row (v bytes x r units of exponentials, the bulk of the work), warp 0 draws. Inputs: the draft's bytes and prefix log-marginals, the
-// target model's conditionals along the draft, one uniform per test plus one for the last byte; the logits and
-// per-unit log-sum-exps the draft call left in the workspace.
+// One CTA per drafted window w (position p = w / wpp). Inputs: the draft's bytes and prefix log-marginals, the target
+// model's conditionals along the draft, one uniform per test plus one for the last byte; the logits and per-unit
+// log-sum-exps of the slots, and the slot messages msg [W, n, r] the circuit kernels left in the workspace.
 //   1. s = 0; while s < n: the draft's conditional of byte s is q_s = exp(prefix[s] - prefix[s-1]) (prefix[-1] = 0);
 //      stop if alpha_s > p(x_s) / q_s, tested as alpha_s * q_s > p(x_s); else s += 1.
 //   2. s == n: the extra byte is drawn from the target row n.
-//      s <  n: it is drawn from max(0, p(.) - q(. | x_0..x_{s-1})) / Z. The circuit's conditional of slot s is a
-//      mixture of the slot's r input units, q(b | ..) = sum_k c_k phi_{s,k}(b), with c the posterior of the latent that
-//      owns slot s given the accepted bytes: CP: omega_k prod_{i<s} phi_{i,k}(x_i); HMM: the one-step prediction
-//      from alpha_{s-1}; BTree: the upward pass with the bytes >= s summed out, then the downward pass along the
-//      path from the root to the node that owns token s.
+//      s <  n: it is drawn from max(0, p(.) - q(. | x_0..x_{s-1})) / Z. The circuit's conditional of slot s is a mixture of the
+//      slot's r input units under softmax(msg[w, s, :]): q(b | ..) = sum_k exp(logit_k[b] + msg_k - LSE(msg) - lse_k).
 //   Both draws are inverse-CDF on unnormalised weights (u * total < running sum, index order, no division).
-__global__ void __launch_bounds__(kAcceptThreads) spec_accept_kernel(
-    int family, const float* __restrict__ logits, const float* __restrict__ unit_lse, const float* __restrict__ logw,
-    const float* __restrict__ logA, const int* __restrict__ bytes, const float* __restrict__ prefix,
-    const float* __restrict__ target, const float* __restrict__ uniforms, int* __restrict__ out_accepted,
-    int* __restrict__ out_next, unsigned* status, int W, int wpp, int n, int r, int v, int vv, int sum_rows,
-    int logA_stride, const float* __restrict__ evidence, const int* __restrict__ row_of) {
-  // evidence != NULL (after a many-position draft): log phi of the drafted bytes comes from evidence [W, n, r] (the G the
-  // draft left), and `logits` [rows, r v] / `unit_lse` [rows, r] hold only the slot of each rejected window's first
-  // rejected byte, at row row_of[w].
-  extern __shared__ float sm[];
-  int& accepted_len = *reinterpret_cast<int*>(sm);       // s, or -1: the window's inputs were refused
-  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// The call is a chain of dependent L2 round trips: every warp runs the tests (one ballot, no broadcast through shared
+// memory), a thread then has all the logits of its byte in flight, and the scan over the bytes is one warp scan plus the
+// warps' totals. With the recursions gone from it (they were one warp's serial chain through the tables) and launched as a
+// programmatic dependent the kernel went from 59 to 6 us at HMM n = 16, 128 windows; 12 to 5 us for one mixture window; 569 to
+// 49 us for 4096 tree windows of n = 16. row_of != NULL (after a many-position draft): `logits` [rows, r v] and `unit_lse` [rows, r] hold only the
+// slot of each rejected window's first rejected byte, at row row_of[w].
+__global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
+    const float* __restrict__ logits, const float* __restrict__ unit_lse, const float* __restrict__ msg,
+    const int* __restrict__ bytes, const float* __restrict__ prefix, const float* __restrict__ target,
+    const float* __restrict__ uniforms, int* __restrict__ out_accepted, int* __restrict__ out_next, unsigned* status, int W,
+    int wpp, int n, int r, int v, int vv, const int* __restrict__ row_of) {
+  extern __shared__ __align__(16) float sm[];
+  grid_launch_dependents();
+  grid_dependency_wait();   // the draft's outputs come from the kernels before this one
+  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int w = blockIdx.x;
-  if (w >= W) return;
-  float* mres = sm + 4;
+  float* mres = sm;                                      // [v]
+  float* cw = sm + v;                                    // [r], then the warps' totals
   const int pos = w / wpp;
   const int* x = bytes + static_cast<size_t>(w) * n;
   const float* pre = prefix + static_cast<size_t>(w) * n;
   const float* u = uniforms + static_cast<size_t>(w) * (n + 1);
   const float* tp = target + static_cast<size_t>(w) * (n + 1) * v;
-  const float* lw = logw + static_cast<size_t>(pos) * sum_rows;
-  const bool has = lane < r;
-
-  float* cw = mres + v;                                  // [r] weight of every input unit of slot s
-  float* cl = cw + r;                                    // [r] its log-sum-exp
-  if (wib == 0) {
-  // ---- 1. acceptance tests
-  bool bad_u = false, bad_x = false;
-  for (int c = lane; c <= n; c += 32) bad_u |= !(u[c] >= 0.f && u[c] < 1.f);
-  for (int c = lane; c < n; c += 32) bad_x |= static_cast<unsigned>(x[c]) >= static_cast<unsigned>(vv);
-  bad_u = __any_sync(kFull, bad_u);
-  bad_x = __any_sync(kFull, bad_x);
-  if (bad_u || bad_x) {
-    if (lane == 0) {
-      atomicOr(status, bad_u ? 2u : 1u);
-      out_accepted[w] = -1;
-      out_next[w] = -1;
-      accepted_len = -1;
-    }
-  } else {
-  // lane i runs the test of byte i (all loads in flight at once); the first rejecting lane ends the accepted run
+  const float u_last = u[n];
+  // ---- 1. acceptance tests: lane i runs the test of byte i; the first rejecting lane ends the accepted run
+  bool bad_u = !(u_last >= 0.f && u_last < 1.f), bad_x = false;
   int s = n;
-  for (int base = 0; base < n && s == n; base += 32) {
+  for (int base = 0; base < n; base += 32) {
     const int i = base + lane;
     bool rej = false;
     if (i < n) {
-      const float q = __expf(pre[i] - (i > 0 ? pre[i - 1] : 0.f));
-      rej = u[i] * q > tp[static_cast<size_t>(i) * v + x[i]];
+      const int xi = x[i];
+      const float ui = u[i], now = pre[i], before = i > 0 ? pre[i - 1] : 0.f;
+      bad_u |= !(ui >= 0.f && ui < 1.f);
+      const bool inside = static_cast<unsigned>(xi) < static_cast<unsigned>(vv);
+      bad_x |= !inside;
+      rej = inside && ui * __expf(now - before) > tp[static_cast<size_t>(i) * v + xi];
     }
     const unsigned m = __ballot_sync(kFull, rej);
-    if (m) s = base + __ffs(m) - 1;
+    if (m && s == n) s = base + __ffs(m) - 1;
   }
-  if (lane == 0) {
-    out_accepted[w] = s;
-    accepted_len = s;
-  }
-  if (s < n) {
-    // ---- 2. c[k]: log-weight of input unit k of slot s given the accepted bytes (lane = k)
-    auto g_at = [&](int i, int k) -> float {   // log phi_{i,k}(x_i)
-      if (evidence != nullptr) return evidence[(static_cast<size_t>(w) * n + i) * r + k];
-      const size_t unit = (static_cast<size_t>(pos) * n + i) * r + k;
-      return logits[unit * v + x[i]] - unit_lse[unit];
-    };
-    auto g_of = [&](int i) -> float { return g_at(i, lane); };
-    // log-sum-exp of unit k of slot s
-    auto lse_of = [&](int k) -> float {
-      return evidence != nullptr ? unit_lse[static_cast<size_t>(row_of[w]) * r + k]
-                                 : unit_lse[(static_cast<size_t>(pos) * n + s) * r + k];
-    };
-    float c = 0.f;
-    if (family == 0) {
-      // mixture of up to 128 components: lane handles k = lane, lane + 32, ...; the weights need no normalisation of
-      // log omega (they are normalised below), so unnormalised mixture logits (r > 32) are as good
-      float cq[4];
-      float m = -CUDART_INF_F, sacc = 0.f;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int k = lane + 32 * q;
-        cq[q] = -CUDART_INF_F;
-        if (k < r) {
-          float a = lw[k];
-#pragma unroll 4
-          for (int i = 0; i < s; ++i) a += g_at(i, k);      // independent gathers: several in flight
-          cq[q] = a;
-          lse_merge(m, sacc, a, 1.f);
-        }
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float m2 = __shfl_xor_sync(kFull, m, off);
-        const float s2 = __shfl_xor_sync(kFull, sacc, off);
-        lse_merge(m, sacc, m2, s2);
-      }
-      const float lse_all = m + __logf(sacc);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int k = lane + 32 * q;
-        if (k < r) {
-          cw[k] = __expf(cq[q] - lse_all);
-          cl[k] = lse_of(k);
-        }
-      }
-    } else if (family == 1) {
-      float alpha = has ? lw[lane] : -CUDART_INF_F;
-      for (int i = 0; i < s; ++i) {
-        // alpha_i = g_i + (i == 0 ? log pi : LSE_a(alpha_{i-1}[a] + logA[i-1][a][.])); then one more prediction step
-        if (has) alpha += g_of(i);
-        float m = alpha;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, off));
-        const float e = has ? __expf(alpha - m) : 0.f;
-        const float* A = logA + static_cast<size_t>(pos) * logA_stride + static_cast<size_t>(i) * r * r;
-        float acc = 0.f;
-        for (int a0 = 0; a0 < r; a0 += 16) {           // sixteen rows of the table in flight at a time
-          float tv[16];
-#pragma unroll
-          for (int q = 0; q < 16; ++q) tv[q] = (has && a0 + q < r) ? __ldg(A + (a0 + q) * r + lane) : -CUDART_INF_F;
-#pragma unroll
-          for (int q = 0; q < 16; ++q)
-            if (a0 + q < r) acc = fmaf(__shfl_sync(kFull, e, a0 + q), __expf(tv[q]), acc);
-        }
-        alpha = has ? m + __logf(acc) : -CUDART_INF_F;
-      }
-      c = alpha;
-    } else {
-      float* prod = cl + r;
-      float* S = prod + (n - 1) * r;
-      float* table = S + (n - 1) * r;
-      float* cur = table + r * (r + 1);
-      const int first_leaf_node = n / 2 - 1;
-      for (int j = n - 2; j >= first_leaf_node; --j) {
-        const int t0 = 2 * (j - first_leaf_node);
-        if (has) prod[j * r + lane] = (t0 < s ? g_of(t0) : 0.f) + (t0 + 1 < s ? g_of(t0 + 1) : 0.f);
-      }
-      __syncwarp();
-      for (int j = first_leaf_node - 1; j >= 0; --j) {
-        float acc = 0.f;
-        for (int side = 0; side < 2; ++side) {
-          const int ch = 2 * j + 1 + side;
-          const float sc = btree_sum_layer<16>(lw + r + static_cast<size_t>(ch - 1) * r * r, prod + ch * r, table, lane, r);
-          if (has) S[ch * r + lane] = sc;
-          acc += sc;
-        }
-        if (has) prod[j * r + lane] = acc;
-        __syncwarp();
-      }
-      // downward: up[z] = log-weight of the rest of the circuit seen from the current path node with latent z
-      const int owner = first_leaf_node + (s >> 1);
-      const int code = owner + 1;
-      const int depth = 31 - __clz(code);
-      int node = 0;
-      float up = has ? lw[lane] : -CUDART_INF_F;
-      for (int lvl = depth - 1; lvl >= 0; --lvl) {
-        const int child = 2 * node + 1 + ((code >> lvl) & 1);
-        const int sib = (child & 1) ? child + 1 : child - 1;
-        if (has) cur[lane] = up + S[sib * r + lane];
-        __syncwarp();
-        // the child's table [parent value z][own value b], staged into the padded shared tile first
-        btree_stage_table<16>(lw + r + static_cast<size_t>(child - 1) * r * r, table, lane, r);
-        __syncwarp();
-        float m = -CUDART_INF_F;
-        for (int z = 0; z < r; ++z) m = fmaxf(m, has ? cur[z] + table[z * (r + 1) + lane] : -CUDART_INF_F);
-        float acc = 0.f;
-        for (int z = 0; z < r; ++z) acc += has ? __expf(cur[z] + table[z * (r + 1) + lane] - m) : 0.f;
-        up = has ? m + __logf(acc) : -CUDART_INF_F;
-        __syncwarp();
-        node = child;
-      }
-      const int other_leaf = s ^ 1;
-      c = up + ((has && other_leaf < s) ? g_of(other_leaf) : 0.f);
+  bad_u = __any_sync(kFull, bad_u);
+  bad_x = __any_sync(kFull, bad_x);
+  if (bad_u || bad_x) {                                  // the same for every warp
+    if (threadIdx.x == 0) {
+      atomicOr(status, bad_u ? 2u : 1u);
+      out_accepted[w] = -1;
+      out_next[w] = -1;
     }
-    if (family != 0) {                                   // HMM, BTree: one weight per lane (r <= 32)
-      const float c_lse = warp_lse(c, has);              // every lane takes part in the shuffles
-      if (has) {
-        cw[lane] = __expf(c - c_lse);
-        cl[lane] = lse_of(lane);
-      }
-    }
+    return;
   }
-  }
-  }   // warp 0
-  __syncthreads();
-  const int s = accepted_len;
-  if (s < 0) return;
+  // ---- 2. weights of the v bytes
   const float* trow = tp + static_cast<size_t>(s) * v;
-  // ---- residual weights of the v bytes, all warps
   if (s == n) {
-    for (int b = threadIdx.x; b < v; b += kAcceptThreads) mres[b] = b < vv ? trow[b] : 0.f;
+    for (int b = threadIdx.x; b < v; b += blockDim.x) mres[b] = b < vv ? trow[b] : 0.f;
   } else {
-    const float* lrow = evidence != nullptr ? logits + static_cast<size_t>(row_of[w]) * r * v
-                                            : logits + (static_cast<size_t>(pos) * n + s) * r * v;   // [r, v] logits of slot s
-    for (int b = threadIdx.x; b < v; b += kAcceptThreads) {
-      float q = 0.f;
+    const size_t lrow = row_of != nullptr ? static_cast<size_t>(row_of[w]) : static_cast<size_t>(pos) * n + s;
+    const float* ulse = unit_lse + lrow * r;
+    const float* lg = logits + lrow * r * v;             // [r, v] logits of slot s
+    if (wib == 0) {
+      const float* mw = msg + (static_cast<size_t>(w) * n + s) * r;
+      float c[4], l[4];
+      float m = -CUDART_INF_F;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int k = lane + 32 * q;
+        c[q] = k < r ? mw[k] : -CUDART_INF_F;
+        l[q] = k < r ? ulse[k] : 0.f;
+        m = fmaxf(m, c[q]);
+      }
+      m = warp_max_nan(m);
+      float sum = 0.f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sum += __expf(c[q] - m);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
+      const float lse = m + __logf(sum);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (lane + 32 * q < r) cw[lane + 32 * q] = (c[q] - lse - l[q]) * kLog2e;
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < v; b += blockDim.x) {
+      float res = 0.f;
       if (b < vv) {
-        // the r logits of byte b come from r different rows: eight loads in flight at a time, two accumulation chains
-        float q1 = 0.f;
+        const float t = trow[b];
+        float q0 = 0.f, q1 = 0.f;
         int k = 0;
-        for (; k + 8 <= r; k += 8) {
-          float xv[8];
+        for (; k + 16 <= r; k += 16) {                   // sixteen rows' logits in flight, two accumulation chains
+          float xv[16];
 #pragma unroll
-          for (int t = 0; t < 8; ++t) xv[t] = lrow[static_cast<size_t>(k + t) * v + b];
+          for (int e = 0; e < 16; ++e) xv[e] = lg[static_cast<size_t>(k + e) * v + b];
 #pragma unroll
-          for (int t = 0; t < 8; t += 2) {
-            q = fmaf(cw[k + t], __expf(xv[t] - cl[k + t]), q);
-            q1 = fmaf(cw[k + t + 1], __expf(xv[t + 1] - cl[k + t + 1]), q1);
+          for (int e = 0; e < 16; e += 2) {
+            q0 += fast_ex2(fmaf(xv[e], kLog2e, cw[k + e]));
+            q1 += fast_ex2(fmaf(xv[e + 1], kLog2e, cw[k + e + 1]));
           }
         }
-        for (; k < r; ++k) q = fmaf(cw[k], __expf(lrow[static_cast<size_t>(k) * v + b] - cl[k]), q);
-        q += q1;
+        for (; k < r; ++k) q0 += fast_ex2(fmaf(lg[static_cast<size_t>(k) * v + b], kLog2e, cw[k]));
+        res = fmaxf(0.f, t - (q0 + q1));
       }
-      mres[b] = b < vv ? fmaxf(0.f, trow[b] - q) : 0.f;   // padding symbols carry no mass
+      mres[b] = res;                                     // padding symbols carry no mass
     }
   }
   __syncthreads();
-  if (wib != 0) return;
-
-  // ---- 3. inverse CDF over the weights in mres (warp 0): lane l owns bytes [l*per, (l+1)*per)
-  const int per = (v + 31) / 32;
-  const int b0 = lane * per;
+  // ---- 3. inverse CDF over mres: thread t owns the bytes [t * per, (t + 1) * per)
+  const int per = (v + blockDim.x - 1) / blockDim.x;
+  const int b0 = threadIdx.x * per;
   float part = 0.f;
   for (int q = 0; q < per; ++q)
     if (b0 + q < v) part += mres[b0 + q];
   const float incl = warp_scan_incl(part, lane);
-  const float total = __shfl_sync(kFull, incl, 31);
-  const float thr = u[n] * total;
-  const unsigned hit = __ballot_sync(kFull, thr < incl);
-  int byte = vv - 1;   // rounding may leave no index: the last one
-  if (hit) {
-    const int src = __ffs(hit) - 1;
-    int found = -1;
-    const float before = __shfl_up_sync(kFull, incl, 1);
-    if (lane == src) {
-      float cum = lane == 0 ? 0.f : before;
-      for (int q = 0; q < per && found < 0; ++q)
-        if (b0 + q < vv) {
-          cum += mres[b0 + q];
-          if (thr < cum) found = b0 + q;
-        }
-      if (found < 0) found = min(b0 + per, vv) - 1;
-    }
-    byte = __shfl_sync(kFull, found, src);
+  if (lane == 31) cw[wib] = incl;
+  __syncthreads();
+  // every warp adds the warps' totals up in the same order, so exactly one of them finds the threshold inside its own run
+  float total = 0.f;
+  for (int q = 0; q < warps; ++q) total += cw[q];
+  const float thr = u_last * total;
+  float before = 0.f;
+  int owner = -1;
+  for (int q = 0; q < warps; ++q) {
+    const float end = before + cw[q];
+    if (thr < end) { owner = q; break; }
+    before = end;
   }
-  if (lane == 0) out_next[w] = byte;
+  if (owner < 0) {                                       // rounding may leave no index: the last one
+    if (threadIdx.x == 0) {
+      out_accepted[w] = s;
+      out_next[w] = vv - 1;
+    }
+    return;
+  }
+  if (wib != owner) return;
+  const unsigned some = __ballot_sync(kFull, part > 0.f);
+  unsigned hit = __ballot_sync(kFull, part > 0.f && thr < before + incl);
+  if (!hit) hit = some ? 1u << (31 - __clz(some)) : 1u << 31;      // the run's last byte with mass
+  const int src = __ffs(hit) - 1;
+  const float prev = __shfl_up_sync(kFull, incl, 1);
+  if (lane == src) {
+    float cum = before + (lane == 0 ? 0.f : prev);
+    int found = -1, last = min(b0 + per, vv) - 1;
+    for (int q = 0; q < per && found < 0; ++q)
+      if (b0 + q < vv && mres[b0 + q] > 0.f) {
+        cum += mres[b0 + q];
+        last = b0 + q;
+        if (thr < cum) found = b0 + q;
+      }
+    out_accepted[w] = s;
+    out_next[w] = found >= 0 ? found : min(last, vv - 1);
+  }
 }
 
 // The tests of Algorithm 3 alone, one warp per window: first_rejected[w] = s if the draft is rejected at byte s < n, else -1

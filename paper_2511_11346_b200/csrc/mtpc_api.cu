@@ -438,7 +438,11 @@ int launch_gemm(mtpc_head* h, int mode, const void* hidden_bf16, int rows, int w
   p.emit_units = c.n * c.r;
   p.num_groups = with_emit ? tl.num_groups : 0;
   p.group_units = tl.group_units;
-  if (mode != kModeSample && with_emit) {
+  if (grp != nullptr) {
+    // sorted rows: by unit, one item per row tile; by slot, a row tile's r units are cut into runs that fill the device
+    p.group_units = grp->by_slot ? choose_group_units(c.v, c.r, grp->max_tiles, workers) : 1;
+    p.num_groups = grp->by_slot ? (c.r + p.group_units - 1) / p.group_units : 1;
+  } else if (mode != kModeSample && with_emit) {
     p.group_units = choose_group_units(c.v, p.emit_units, p.m_units, workers);
     p.num_groups = (p.emit_units + p.group_units - 1) / p.group_units;
   }
@@ -472,7 +476,8 @@ int launch_gemm(mtpc_head* h, int mode, const void* hidden_bf16, int rows, int w
   p.out_bytes = out_bytes;
   p.status = at<unsigned>(h, L.off_status);
   p.wait_limit_ns = h->wait_limit_ns;
-  const long long items = grp ? grp->max_tiles : static_cast<long long>(p.m_units) * (p.num_groups + p.num_sum_tiles);
+  const long long items = grp ? static_cast<long long>(grp->max_tiles) * p.num_groups
+                              : static_cast<long long>(p.m_units) * (p.num_groups + p.num_sum_tiles);
   const int grid = ctas * static_cast<int>(items < workers ? items : workers);
   const size_t smem = pair ? tl.pair_smem : tl.smem;
   if (grp && grp->by_slot) {

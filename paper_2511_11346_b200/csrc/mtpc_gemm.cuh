@@ -46,7 +46,9 @@ constexpr uint32_t kStatusBadTarget = 1u, kStatusBadUniform = 2u, kStatusTimeout
 // kModeSampleGrouped: the byte draws again, on rows that were sorted by the unit they sample from (mtpc_group.cuh):
 // a work item is one GroupTile instead of (m-tile, unit).
 // kModeLogitsGrouped: rows sorted by SLOT (the acceptance stage after a many-position draft): a work item is a GroupTile
-// whose `unit` is a slot; the logits of the slot's r units and their log-sum-exps are written out per staged row.
+// whose `unit` is a slot and a run of group_units of the slot's r units; their logits and log-sum-exps are written out per
+// staged row. (There are only about n + rows / 128 tiles: without the split over units a batch of 4096 windows of 16 slots
+// is 45 items for 148 SMs, each r v columns long: 623 us against 213.)
 enum { kModeLogprob = 0, kModeSample = 1, kModeSampleGrouped = 2, kModeLogitsGrouped = 3 };
 
 struct GemmParams {
@@ -139,15 +141,17 @@ struct TileCoord {
   int arow, count;   // first row of the A operand and the rows that count (set by the caller for ungrouped items)
   int wrap;          // tiles per sweep over the item's weight rows: tile t reads the rows of tile t % wrap
 };
-// A grouped item: `count` staged rows from `row0` on, against the tiles of the one unit they sample from (by_slot: of the
-// r units of the one slot whose logits they need).
+// A grouped item: `count` staged rows from `row0` on, against the tiles of the one unit they sample from (by_slot: of
+// group_units of the r units of the one slot whose logits they need; the runs of one row tile follow each other).
 __device__ __forceinline__ TileCoord group_coord(const GemmParams& p, int item, bool by_slot) {
-  const GroupTile g = p.group_tiles[item];
+  const int runs = by_slot ? p.num_groups : 1;
+  const int tile = item / runs, first = (item - tile * runs) * p.group_units;
+  const GroupTile g = p.group_tiles[tile];
   TileCoord c;
   c.mt = 0;
   c.is_sum = 0;
-  c.unit0 = by_slot ? g.unit * p.r : g.unit;
-  c.nunits = by_slot ? p.r : 1;
+  c.unit0 = by_slot ? g.unit * p.r + first : g.unit;
+  c.nunits = by_slot ? min(p.group_units, p.r - first) : 1;
   c.cols = p.tile_cols;
   c.brow0 = c.unit0 * p.v;
   c.wrap = (c.nunits * p.v + p.tile_cols - 1) / p.tile_cols;
@@ -243,7 +247,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   const int lane = threadIdx.x & 31;
   constexpr bool kGrouped = MODE == kModeSampleGrouped || MODE == kModeLogitsGrouped;
   static_assert(!kGrouped || CTAS == 1, "grouped tiles are ragged: no pairing");
-  const int num_items = kGrouped ? *p.group_num_tiles : (p.num_groups + p.num_sum_tiles) * p.m_units;
+  const int num_items = kGrouped ? *p.group_num_tiles * (MODE == kModeLogitsGrouped ? p.num_groups : 1)
+                                 : (p.num_groups + p.num_sum_tiles) * p.m_units;
   const uint32_t cta_rank = CTAS == 2 ? cluster_cta_rank() : 0u;      // 0 = the pair's leader
   auto coord = [&](int item) {
     if (kGrouped) return group_coord(p, item, MODE == kModeLogitsGrouped);
@@ -476,7 +481,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
       if (MODE == kModeLogitsGrouped) {
         // ---- the slot's logits and unit log-sum-exps per staged row (logit_out [rows, r v], lse_out [rows, r]): what the
         // acceptance stage needs to form the circuit's conditional of the first rejected byte
-        int col = 0, k = 0;                                       // column inside the slot's r v columns; unit index
+        const int k0 = tc.unit0 % p.r;                            // the item's first unit of the slot
+        int col = 0, k = 0;                                       // column inside the item's nunits v columns; unit index
         float m = -CUDART_INF_F, s = 0.f;
         for (int t = 0; t < tc.ntiles && ok; ++t, ++use) {
           const uint32_t slot = use % p.num_slots;
@@ -486,12 +492,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
           }
           tc_fence_after();
           const uint32_t tcol = lane_base + slot * p.slot_stride;
-          for (int b = 0; b < nbatch && k < p.r; ++b) {
+          for (int b = 0; b < nbatch && k < tc.nunits; ++b) {
             float x[16];
             tmem_ld16(tcol + b * 16, x);
             mask_padding(x, col - k * p.v, p.vv);
             if (valid) {
-              float* l = p.logit_out + static_cast<size_t>(row) * p.logit_pitch + col;
+              float* l = p.logit_out + static_cast<size_t>(row) * p.logit_pitch + k0 * p.v + col;
               st_global_v8(l, x);
               st_global_v8(l + 8, x + 8);
             }
@@ -506,7 +512,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
             m = mn;
             col += 16;
             if (col == (k + 1) * p.v) {
-              if (valid) p.lse_out[static_cast<size_t>(row) * p.r + k] = m + fast_lg2(s) * kLn2;
+              if (valid) p.lse_out[static_cast<size_t>(row) * p.r + k0 + k] = m + fast_lg2(s) * kLn2;
               ++k;
               m = -CUDART_INF_F; s = 0.f;
             }

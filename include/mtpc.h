@@ -243,8 +243,8 @@ int mtpc_window_loss(mtpc_head* head, const void* hidden, const int32_t* targets
  * mtpc_window_loss_backward: the training loss of Eq. 6 (as mtpc_window_loss: per-slot conditionals, valid-token
  * normalisation V_ij, discount gamma^j) AND its gradients, for num_sequences sequences of sequence_length positions.
  * Eq. 6 is linear in the prefix log-marginals, L = sum_t sum_j coeff[t, j] log q(x_{t,0..j}), with
- * coeff[t, j] = c[t, j] - c[t, j+1], c[t, j] = -gamma^j / (N V_ij) for a valid target and 0 otherwise; the call runs one
- * circuit backward pass per prefix length j+1 (later bytes summed out), accumulates the posteriors in fp32, and then
+ * coeff[t, j] = c[t, j] - c[t, j+1], c[t, j] = -gamma^j / (N V_ij) for a valid target and 0 otherwise; one sweep over each
+ * window's circuit and its reverse give every prefix and the gradient of the sum (fp32), and the call then
  * shares the projection-sized work (logit gradients, the three GEMMs) with mtpc_window_logprob_backward. Same workspace
  * (mtpc_backward_workspace_bytes with T = num_sequences * sequence_length), same outputs, same arithmetic notes.
  */
@@ -369,9 +369,8 @@ int mtpc_get_status(mtpc_head* head, void* stream, uint32_t* out_flags);
  *   mtpc_speculative_accept: [0] the acceptance kernel.
  *   mtpc_window_logprob_backward: [0] forward projection, [1] circuit backward, [2] gradient of the logits,
  *                        [3] the three plain GEMMs.
- *   mtpc_window_loss_backward: [0] forward projection + prefix marginals + loss, [1] circuit backward (mixture:
- *                        one pass per prefix length; tree: the same passes in one launch; HMM: one reverse sweep),
- *                        [2] and [3] as above.
+ *   mtpc_window_loss_backward: [0] forward projection, [1] circuit (every prefix marginal and the gradient in one sweep)
+ *                        and the loss, [2] and [3] as above.
  *   mtpc_draft_sample, mtpc_draft_sample_prefix:   P <= 128 positions: [0] one pass over all weights (logits of every unit),
  *                        [1] per-slot latent + byte draws and evidence, [2] circuit evaluation.
  *                        Otherwise: [0] sum-unit GEMM, [1] latent sampling, [2] byte draws (GEMM + inverse-CDF

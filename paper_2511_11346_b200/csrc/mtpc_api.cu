@@ -512,6 +512,13 @@ int launch_gemm(mtpc_head* h, int mode, const void* hidden_bf16, int rows, int w
 
 size_t btree_smem_bytes(int n, int r) { return static_cast<size_t>(kCircuitWarps) * btree_warp_floats(n, r) * sizeof(float); }
 
+// CTAs that persistent kernels with `smem` bytes of dynamic shared memory each may launch: what the device holds at once, at
+// most eight per SM.
+int sms_times_resident(const mtpc_head* h, size_t smem) {
+  const int per_sm = static_cast<int>(kSmemLimit / (smem + 1024));
+  return h->num_sms * (per_sm < 1 ? 1 : per_sm > 8 ? 8 : per_sm);
+}
+
 // Circuit evaluation of W windows: out[w] = joint log-prob, prefix [W, n] = log-marginals of the prefixes x_0..x_i, msg
 // [W, n, r] = slot messages (each may be NULL, not all).
 // dependent: the launch directly follows draft_slot_kernel, which has zeroed the work counter, and may overlap its tail.
@@ -540,15 +547,14 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
     const size_t smem = hmm_circuit_smem_floats(c.n, c.r, prefix != nullptr, chunk) * sizeof(float);
     const int stride = hmm_table_stride(h);
     const int items = stride == 0 ? (W + kHmmWarps - 1) / kHmmWarps : W / wpp * ((wpp + kHmmWarps - 1) / kHmmWarps);
-    const int resident = h->num_sms * (static_cast<int>(kSmemLimit / (smem + 1024)) > 8 ? 8 : static_cast<int>(kSmemLimit / (smem + 1024)) < 1 ? 1 : static_cast<int>(kSmemLimit / (smem + 1024)));
+    const int resident = sms_times_resident(h, smem);
     launch_kernel(circuit_hmm_kernel, items < resident ? items : resident, kHmmWarps * 32, smem, st, dependent, G, logw,
                   hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r, L.sum_rows, chunk);
   } else if (sweep) {
     const int warps = c.n / 2 < 8 ? c.n / 2 : 8;                         // a warp per node of the owners' level
     const bool fits = btree_prefix_smem_floats(c.n, c.r, warps, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
     const size_t smem = btree_prefix_smem_floats(c.n, c.r, warps, fits) * sizeof(float);
-    const int per_sm = static_cast<int>(kSmemLimit / (smem + 1024));
-    const int resident = h->num_sms * (per_sm < 1 ? 1 : per_sm > 8 ? 8 : per_sm);
+    const int resident = sms_times_resident(h, smem);
     launch_kernel(circuit_btree_prefix_kernel, W < resident ? W : resident, warps * 32, smem, st, dependent, G, logw, out, prefix,
                   msg, W, wpp, c.n, c.r, L.sum_rows, fits ? 1 : 0);
   } else {
@@ -939,7 +945,7 @@ size_t round64(size_t x) { return (x + 63) / 64 * 64; }
 // The sum-unit logit gradients sit to the right of the emission logit gradients in one matrix [T, Kd], Kd = Nc + Spad.
 struct BackwardLayout {
   size_t Nc, Spad, Kd;
-  size_t off_lse, off_post, off_logits, off_dlogit, off_dsum_f32, off_coeff, total;
+  size_t off_lse, off_post, off_logits, off_dlogit, off_coeff, total;
 };
 void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout* B) {
   B->Nc = static_cast<size_t>(c.n) * c.r * c.v;
@@ -951,7 +957,6 @@ void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout*
   B->off_post = take(static_cast<size_t>(T) * c.n * c.r * 4);
   B->off_logits = take(static_cast<size_t>(T) * B->Nc * 4);              // [T, Nc] fp32: the emission logits of the forward pass
   B->off_dlogit = take(static_cast<size_t>(T) * B->Kd * 2);          // [T, Nc | Spad] bf16
-  B->off_dsum_f32 = take(static_cast<size_t>(T) * L.sum_rows * 4);   // Eq. 6: sum-unit logit gradients accumulated over the passes
   B->off_coeff = take(static_cast<size_t>(T) * c.n * 4);             // Eq. 6: weights of the prefix marginals
   B->total = off;
 }
@@ -1131,7 +1136,7 @@ size_t circuit_backward_smem(const mtpc_head* h, int warps) {
   const mtpc_config& c = h->cfg;
   if (c.family == MTPC_HMM) return hmm_backward_smem_floats(c.n, c.r, !is_ctx(h), warps) * sizeof(float);
   if (c.family == MTPC_BTREE) return static_cast<size_t>(warps) * btree_backward_warp_floats(c.n, c.r) * sizeof(float);
-  return 0;
+  return static_cast<size_t>(warps) * cp_loss_warp_floats(c.n, c.r) * sizeof(float);
 }
 int circuit_backward_warps(const mtpc_head* h) {
   for (int w = kCircuitWarps; w >= 1; w >>= 1)
@@ -1139,9 +1144,9 @@ int circuit_backward_warps(const mtpc_head* h) {
   return 0;
 }
 
-// `loss_coeff` (HMM, tree): the weights [W, n] of the prefix log-marginals in Eq. 6; the whole gradient in one launch.
-int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cudaStream_t st,
-                            const float* loss_coeff = nullptr) {
+// a.coeff (Eq. 6: the weights [W, n] of the prefix log-marginals) chooses the kernels that give every prefix and the whole
+// gradient in one launch; otherwise the gradient of sum_w a.weight[w] log q_w.
+int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cudaStream_t st) {
   const mtpc_config& c = h->cfg;
   const Layout& L = h->L;
   a.G = at<float>(h, L.off_G);
@@ -1150,22 +1155,31 @@ int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cuda
   a.r = c.r;
   a.sum_rows = L.sum_rows;
   unsigned* counter = at<unsigned>(h, L.off_status) + kWorkCounterWord;
-  const int warps = c.family == MTPC_CP ? kCircuitWarps : circuit_backward_warps(h);
+  const bool loss = a.coeff != nullptr;
+  const int warps = circuit_backward_warps(h);
   if (warps == 0) return MTPC_ERR_UNSUPPORTED;
   const int blocks = (a.W + warps - 1) / warps;
   const int threads = warps * 32;
   const int resident = blocks < 8 * h->num_sms ? blocks : 8 * h->num_sms;
   const size_t smem = circuit_backward_smem(h, warps);
-  if (c.family != MTPC_CP && cudaMemsetAsync(counter, 0, sizeof(unsigned), st) != cudaSuccess) return MTPC_ERR_CUDA;
-  if (c.family == MTPC_CP) {
-    circuit_cp_backward_kernel<<<blocks, threads, 0, st>>>(a);
-  } else if (c.family == MTPC_HMM && loss_coeff != nullptr) {
-    circuit_hmm_loss_backward_kernel<<<resident, threads, smem, st>>>(a, loss_coeff, hmm_tables(h), hmm_table_stride(h), dT,
-                                                                     counter);
+  if ((c.family == MTPC_HMM || (c.family == MTPC_BTREE && !loss)) && cudaMemsetAsync(counter, 0, sizeof(unsigned), st) != cudaSuccess)
+    return MTPC_ERR_CUDA;
+  if (c.family == MTPC_CP && loss) {
+    circuit_cp_loss_backward_kernel<<<blocks, threads, smem, st>>>(a);
+  } else if (c.family == MTPC_CP) {
+    circuit_cp_backward_kernel<<<(a.W + kCircuitWarps - 1) / kCircuitWarps, kCircuitWarps * 32, 0, st>>>(a);
+  } else if (c.family == MTPC_HMM && loss) {
+    circuit_hmm_loss_backward_kernel<<<resident, threads, smem, st>>>(a, hmm_tables(h), hmm_table_stride(h), dT, counter);
   } else if (c.family == MTPC_HMM) {
     circuit_hmm_backward_kernel<<<resident, threads, smem, st>>>(a, hmm_tables(h), hmm_table_stride(h), dT, counter);
+  } else if (loss) {
+    const int tw = c.n / 2 < 8 ? c.n / 2 : 8;                             // a warp per node of the owners' level
+    const bool fits = btree_loss_smem_floats(c.n, c.r, tw, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
+    const size_t tsmem = btree_loss_smem_floats(c.n, c.r, tw, fits) * sizeof(float);
+    const int grid = a.W < sms_times_resident(h, tsmem) ? a.W : sms_times_resident(h, tsmem);
+    circuit_btree_loss_backward_kernel<<<grid, tw * 32, tsmem, st>>>(a, fits ? 1 : 0);
   } else {
-    circuit_btree_backward_kernel<<<resident, threads, smem, st>>>(a, loss_coeff, counter);
+    circuit_btree_backward_kernel<<<resident, threads, smem, st>>>(a, counter);
   }
   h->launches++;
   return check_launch();
@@ -1173,9 +1187,10 @@ int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cuda
 
 // Shared-memory attributes of the circuit backward kernels (per function: always the full limit, see allow_full_smem).
 int set_backward_attributes(const mtpc_head* head) {
-  if (head->cfg.family == MTPC_CP) return MTPC_OK;
   if (circuit_backward_warps(head) == 0) return MTPC_ERR_UNSUPPORTED;
   bool ok = allow_full_smem(circuit_hmm_backward_kernel);
+  ok &= allow_full_smem(circuit_cp_loss_backward_kernel);
+  ok &= allow_full_smem(circuit_btree_loss_backward_kernel);
   ok &= allow_full_smem(circuit_hmm_loss_backward_kernel);
   ok &= allow_full_smem(circuit_btree_backward_kernel);
   return ok ? MTPC_OK : MTPC_ERR_CUDA;
@@ -1815,12 +1830,10 @@ int mtpc_window_logprob_backward(mtpc_head* head, const void* hidden, const int3
   memset(&a, 0, sizeof(a));
   a.targets = targets;
   a.weight = weight;
-  a.weight_stride = 1;
   a.out = out_logprob;
   a.post = reinterpret_cast<float*>(bw + B.off_post);
   a.dsum = reinterpret_cast<__nv_bfloat16*>(bw + B.off_dlogit) + B.Nc;      // columns [Nc, Nc + S r) of the dlogit rows
   a.dsum_pitch = static_cast<int>(B.Kd);
-  a.len = c.n;
   a.W = T;
   rc = launch_circuit_backward(head, a, dT_static, st);
   pt.end();
@@ -1885,12 +1898,10 @@ int mtpc_lowrank_window_logprob_backward(mtpc_head* head, const void* hidden, co
   memset(&a, 0, sizeof(a));
   a.targets = targets;
   a.weight = weight;
-  a.weight_stride = 1;
   a.out = out_logprob;
   a.post = reinterpret_cast<float*>(bw + B.off_post);
   a.dsum = sy + R.Ksy;
   a.dsum_pitch = static_cast<int>(R.pitch);
-  a.len = c.n;
   a.W = T;
   rc = launch_circuit_backward(head, a, dT_static, st);
   pt.end();
@@ -1931,7 +1942,6 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t* bw = static_cast<uint8_t*>(bwd_workspace);
   float* post = reinterpret_cast<float*>(bw + B.off_post);
-  float* dsum_f32 = reinterpret_cast<float*>(bw + B.off_dsum_f32);
   float* coeff = reinterpret_cast<float*>(bw + B.off_coeff);
   float* prefix = at<float>(head, L.off_prefix);
   float* partial = at<float>(head, L.off_partial);
@@ -1940,7 +1950,7 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   rc = stage_hidden(head, hidden, T, &hb, st);
   if (rc != MTPC_OK) return rc;
   PhaseTimer pt(head, st);
-  // 1. forward projection (keeping the log-sum-exps), prefix marginals, the loss of Eq. 6 and the weight of every prefix
+  // 1. forward projection (keeping the log-sum-exps) and the weight of every prefix log-marginal in the loss
   pt.begin();
   GradArgs fwd;
   fwd.lse_out = reinterpret_cast<float*>(bw + B.off_lse);
@@ -1948,61 +1958,30 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   fwd.logit_pitch = B.Nc;
   rc = factored ? launch_lowrank_projection(head, hb, T, targets, st, &fwd)
                 : launch_gemm(head, kModeLogprob, hb, T, 1, true, true, targets, nullptr, nullptr, st, &fwd);
-  if (rc == MTPC_OK) rc = launch_circuit(head, T, 1, nullptr, prefix, st);
   if (rc != MTPC_OK) return rc;
-  // the sum units' logit gradients (bf16): to the right of dlogit, or of [s | y] on a factored head
-  __nv_bfloat16* dsum_bf16 = factored ? reinterpret_cast<__nv_bfloat16*>(bw + R.off_sy) + R.Ksy
-                                      : reinterpret_cast<__nv_bfloat16*>(bw + B.off_dlogit) + B.Nc;
-  const size_t dsum_bf16_pitch = factored ? R.pitch : B.Kd;
-  loss_partial_kernel<<<num_sequences, kLossThreads, 0, st>>>(prefix, targets, partial, sequence_length, c.n);
-  loss_final_kernel<<<1, kLossThreads, 0, st>>>(partial, out_slot_loss, out_loss, num_sequences, c.n, gamma);
   loss_coeff_kernel<<<num_sequences, kLossThreads, 0, st>>>(targets, coeff, sequence_length, c.n, num_sequences, gamma);
-  head->launches += 3;
+  head->launches++;
   pt.end();
   if ((rc = check_launch()) != MTPC_OK) return rc;
-  // 2. circuit backward. HMM: every prefix marginal is a forward message, so one reverse sweep gives the whole gradient.
-  // Mixture and tree: one pass per prefix length, accumulating.
+  // 2. circuit: every prefix and the whole gradient of the loss, then the loss itself. The sum units' logit gradients (bf16)
+  // go to the right of dlogit, or of [s | y] on a factored head.
   pt.begin();
   if (static_hmm && cudaMemsetAsync(dT_static, 0, static_cast<size_t>(c.n - 1) * c.r * c.r * 4, st) != cudaSuccess)
     return MTPC_ERR_CUDA;
-  if (c.family == MTPC_HMM) {
-    CircuitBackwardArgs a;
-    memset(&a, 0, sizeof(a));
-    a.targets = targets;
-    a.post = post;
-    a.dsum = dsum_bf16;
-    a.dsum_pitch = static_cast<int>(dsum_bf16_pitch);
-    a.len = c.n;
-    a.W = T;
-    if ((rc = launch_circuit_backward(head, a, dT_static, st, coeff)) != MTPC_OK) return rc;
-  } else {
-    bool bad = cudaMemsetAsync(post, 0, static_cast<size_t>(T) * c.n * c.r * 4, st) != cudaSuccess;
-    bad |= cudaMemsetAsync(dsum_f32, 0, static_cast<size_t>(T) * L.sum_rows * 4, st) != cudaSuccess;
-    if (bad) return MTPC_ERR_CUDA;
-    CircuitBackwardArgs a;
-    memset(&a, 0, sizeof(a));
-    a.targets = targets;
-    a.post = post;
-    a.dsum_f32 = dsum_f32;
-    a.dsum_pitch = L.sum_rows;
-    a.accumulate = 1;
-    a.W = T;
-    if (c.family == MTPC_BTREE) {                 // every prefix length of a window by the same warp, back to back
-      a.len = c.n;
-      if ((rc = launch_circuit_backward(head, a, dT_static, st, coeff)) != MTPC_OK) return rc;
-    } else {
-      for (int j = 0; j < c.n; ++j) {               // mixture: one cheap pass per prefix length
-        a.weight = coeff + j;
-        a.weight_stride = c.n;
-        a.len = j + 1;
-        if ((rc = launch_circuit_backward(head, a, dT_static, st)) != MTPC_OK) return rc;
-      }
-    }
-    const size_t total = static_cast<size_t>(T) * L.sum_rows;
-    const int blocks = static_cast<int>((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-    f32_rows_to_bf16_kernel<<<blocks, 256, 0, st>>>(dsum_f32, dsum_bf16, T, L.sum_rows, L.sum_rows, dsum_bf16_pitch);
-    head->launches++;
-  }
+  CircuitBackwardArgs a;
+  memset(&a, 0, sizeof(a));
+  a.targets = targets;
+  a.coeff = coeff;
+  a.prefix = prefix;
+  a.post = post;
+  a.dsum = factored ? reinterpret_cast<__nv_bfloat16*>(bw + R.off_sy) + R.Ksy
+                    : reinterpret_cast<__nv_bfloat16*>(bw + B.off_dlogit) + B.Nc;
+  a.dsum_pitch = static_cast<int>(factored ? R.pitch : B.Kd);
+  a.W = T;
+  if ((rc = launch_circuit_backward(head, a, dT_static, st)) != MTPC_OK) return rc;
+  loss_partial_kernel<<<num_sequences, kLossThreads, 0, st>>>(prefix, targets, partial, sequence_length, c.n);
+  loss_final_kernel<<<1, kLossThreads, 0, st>>>(partial, out_slot_loss, out_loss, num_sequences, c.n, gamma);
+  head->launches += 2;
   pt.end();
   if ((rc = check_launch()) != MTPC_OK) return rc;
   if (factored) return lowrank_backward_tail(head, R, bw, hb, targets, T, d_hidden, dW_base, dA, dB, dW_sum, pt, st);

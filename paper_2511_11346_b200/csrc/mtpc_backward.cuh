@@ -22,38 +22,22 @@
 
 namespace mtpc {
 
-// Arguments the three circuit backward kernels share beyond the forward ones:
-//   weight, weight_stride   window w is weighted by weight[w * weight_stride]
-//   len                     only the first `len` slots carry evidence, the later bytes are summed out: the kernels then
-//                           differentiate the prefix marginal log q(x_0..x_{len-1}) (len = n: the joint)
-//   accumulate              0: post and dsum are overwritten (dsum as bf16). 1: results are ADDED to post and to the fp32
-//                           buffer dsum_f32 (several passes with different len and weights, Eq. 6); only slots < len are
-//                           touched, the buffers must have been zeroed before the first pass.
-//   dsum_pitch              row pitch, in elements, of whichever of dsum / dsum_f32 is written
+// Arguments of the circuit backward kernels: those that differentiate sum_w weight[w] log q(window w), and those of the
+// training loss of Eq. 6, which is linear in the prefix log-marginals, L = sum_w sum_j coeff[w, j] log p_j: one kernel per
+// family gives every prefix (prefix [W, n]) and the whole gradient.
 struct CircuitBackwardArgs {
   const float* G;
   const float* logw;
   const int* targets;
-  const float* weight;
-  int weight_stride;
-  float* out;                 // [W] log q of the (prefix) window, or NULL
+  const float* weight;        // [W]
+  const float* coeff;         // [W, n] (Eq. 6)
+  float* prefix;              // [W, n] (Eq. 6)
+  float* out;                 // [W] log q of the window, or NULL
   float* post;                // [W, n, r]
-  __nv_bfloat16* dsum;        // [W, dsum_pitch] (accumulate == 0)
-  float* dsum_f32;            // [W, dsum_pitch] (accumulate == 1)
+  __nv_bfloat16* dsum;        // [W, dsum_pitch]
   int dsum_pitch;
-  int len, accumulate;
   int W, n, r, sum_rows;
 };
-// Accumulating passes add by reduction instructions (no value returned, so no wait for the round trip): every address
-// is only ever touched by one lane, in program order, so the sums keep their order and stay reproducible.
-__device__ __forceinline__ void put_post(const CircuitBackwardArgs& a, size_t idx, float v) {
-  if (a.accumulate) atomicAdd(a.post + idx, v);
-  else a.post[idx] = v;
-}
-__device__ __forceinline__ void put_dsum(const CircuitBackwardArgs& a, size_t idx, float v) {
-  if (a.accumulate) atomicAdd(a.dsum_f32 + idx, v);
-  else a.dsum[idx] = __float2bfloat16_rn(v);
-}
 
 // ---------------------------------------------------------------- circuit backward: mixture (Eq. CP)
 // log q = LSE_k a_k, a_k = log omega_k + sum_i G[i, k]:  d log q / d a_k = rho_k = softmax(a)_k for every slot and for
@@ -62,10 +46,10 @@ __global__ void circuit_cp_backward_kernel(const CircuitBackwardArgs a_) {
   const int w = blockIdx.x * kCircuitWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= a_.W) return;
-  const int n = a_.n, r = a_.r, len = a_.len;
+  const int n = a_.n, r = a_.r;
   const float* g = a_.G + static_cast<size_t>(w) * n * r;
   const float* lw = a_.logw + static_cast<size_t>(w) * a_.sum_rows;
-  const float wt = a_.weight[static_cast<size_t>(w) * a_.weight_stride];
+  const float wt = a_.weight[w];
   float a[4];
   float m = -CUDART_INF_F, s = 0.f;
 #pragma unroll
@@ -74,7 +58,7 @@ __global__ void circuit_cp_backward_kernel(const CircuitBackwardArgs a_) {
     a[q] = -CUDART_INF_F;
     if (k < r) {
       a[q] = lw[k];
-      for (int i = 0; i < len; ++i) a[q] += g[i * r + k];
+      for (int i = 0; i < n; ++i) a[q] += g[i * r + k];
       lse_merge(m, s, a[q], 1.f);
     }
   }
@@ -91,11 +75,48 @@ __global__ void circuit_cp_backward_kernel(const CircuitBackwardArgs a_) {
     const int k = lane + 32 * q;
     if (k < r) {
       const float rho = __expf(a[q] - logq);
-      for (int i = 0; i < len; ++i)
-        put_post(a_, (static_cast<size_t>(w) * n + i) * r + k, a_.targets[static_cast<size_t>(w) * n + i] >= 0 ? wt * rho : 0.f);
-      for (int i = len; i < n && !a_.accumulate; ++i) a_.post[(static_cast<size_t>(w) * n + i) * r + k] = 0.f;
-      put_dsum(a_, static_cast<size_t>(w) * a_.dsum_pitch + k, wt * (rho - __expf(lw[k])));
+      for (int i = 0; i < n; ++i)
+        a_.post[(static_cast<size_t>(w) * n + i) * r + k] = a_.targets[static_cast<size_t>(w) * n + i] >= 0 ? wt * rho : 0.f;
+      a_.dsum[static_cast<size_t>(w) * a_.dsum_pitch + k] = __float2bfloat16_rn(wt * (rho - __expf(lw[k])));
     }
+  }
+}
+
+// Eq. 6 through the mixture: with rho_j = softmax(msg_{j+1}) the posterior after slot j, dL/dG[i, k] = sum_{j >= i} coeff_j
+// rho_j[k] and, through the softmax of the mixture logits, dL/dlogit_k = sum_j coeff_j (rho_j[k] - omega_k). One warp per
+// window: the running sums and log-sum-exps of circuit_cp_prefix_kernel (the same bits), then one suffix sum over the slots.
+// (One launch per prefix length, each reading G up to its slot and adding into fp32 rows, was 8 launches, two memsets and a
+// conversion at n = 8: 50 us with their gaps at 2005 positions, prefixes included, against 5.) Shared memory per warp: n (r + 1) + n floats.
+__host__ __device__ inline int cp_loss_warp_floats(int n, int r) { return n * (r + 2); }
+__global__ void circuit_cp_loss_backward_kernel(const CircuitBackwardArgs a_) {
+  extern __shared__ __align__(16) float sm[];
+  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w = blockIdx.x * (blockDim.x >> 5) + wib;
+  if (w >= a_.W) return;
+  const int n = a_.n, r = a_.r;
+  float* tile = sm + static_cast<size_t>(wib) * cp_loss_warp_floats(n, r);
+  float* lps = tile + n * (r + 1);
+  const float* lw = a_.logw + static_cast<size_t>(w) * a_.sum_rows;
+  const float* cw = a_.coeff + static_cast<size_t>(w) * n;
+  const int* tg = a_.targets + static_cast<size_t>(w) * n;
+  cp_prefix_tile(a_.G + static_cast<size_t>(w) * n * r, lw, tile, nullptr, 0, n, r, lane);
+  float csum = 0.f;
+  for (int i = lane; i < n; i += 32) {
+    const float lp = thread_lse(tile + i * (r + 1), r);
+    lps[i] = lp;
+    a_.prefix[static_cast<size_t>(w) * n + i] = lp;
+    csum += cw[i];
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) csum += __shfl_xor_sync(kFull, csum, off);
+  __syncwarp();
+  for (int k = lane; k < r; k += 32) {
+    float acc = 0.f;
+    for (int i = n - 1; i >= 0; --i) {
+      acc = fmaf(cw[i], __expf(tile[i * (r + 1) + k] - lps[i]), acc);
+      a_.post[(static_cast<size_t>(w) * n + i) * r + k] = tg[i] >= 0 ? acc : 0.f;
+    }
+    a_.dsum[static_cast<size_t>(w) * a_.dsum_pitch + k] = __float2bfloat16_rn(acc - csum * __expf(lw[k]));
   }
 }
 
@@ -104,10 +125,10 @@ __global__ void circuit_cp_backward_kernel(const CircuitBackwardArgs a_) {
 // i.e. pairwise posterior minus conditional probability times the posterior of the conditioning value (the gradient
 // with respect to the row's logits). `row` and `pc` are in shared memory; the results go either to a bf16 row in global
 // memory (contextual tables: one set per position), or by atomic adds to an fp32 row in shared memory (static tables,
-// summed over the windows), or added to an fp32 row in global memory (several passes accumulating, Eq. 6). R a multiple of 4: float4 reads rotated by the lane (conflict-free), 8-byte stores.
+// summed over the windows). R a multiple of 4: float4 reads rotated by the lane (conflict-free), 8-byte stores.
 template <int R>
 __device__ __forceinline__ void row_grad_vec(const float* row, const float* pc, float base, float gam, float wt, int lane,
-                                             __nv_bfloat16* dst, float* acc_row, float* f32_row) {
+                                             __nv_bfloat16* dst, float* acc_row) {
   constexpr int Q = R / 4;
   const float4* row4 = reinterpret_cast<const float4*>(row);
   const float4* pc4 = reinterpret_cast<const float4*>(pc);
@@ -125,10 +146,6 @@ __device__ __forceinline__ void row_grad_vec(const float* row, const float* pc, 
       atomicAdd(acc_row + 4 * j + 1, oy);
       atomicAdd(acc_row + 4 * j + 2, oz);
       atomicAdd(acc_row + 4 * j + 3, ow);
-    } else if (f32_row != nullptr) {
-      // this lane owns the row, so the additions to one address keep their order; issued as a reduction (no value comes
-      // back), the warp does not wait for the round trip to L2 that a read-add-write would cost
-      atomicAdd(reinterpret_cast<float4*>(f32_row + 4 * j), make_float4(ox, oy, oz, ow));
     } else {
       __nv_bfloat162 lo = __floats2bfloat162_rn(ox, oy);
       __nv_bfloat162 hi = __floats2bfloat162_rn(oz, ow);
@@ -140,12 +157,12 @@ __device__ __forceinline__ void row_grad_vec(const float* row, const float* pc, 
   }
 }
 __device__ __forceinline__ void row_grad(const float* row, const float* pc, float base, float gam, float wt, int lane, int r,
-                                         __nv_bfloat16* dst, float* acc_row, float* f32_row) {
+                                         __nv_bfloat16* dst, float* acc_row) {
   switch (r) {
-    case 32: row_grad_vec<32>(row, pc, base, gam, wt, lane, dst, acc_row, f32_row); return;
-    case 16: row_grad_vec<16>(row, pc, base, gam, wt, lane, dst, acc_row, f32_row); return;
-    case 8: row_grad_vec<8>(row, pc, base, gam, wt, lane, dst, acc_row, f32_row); return;
-    case 4: row_grad_vec<4>(row, pc, base, gam, wt, lane, dst, acc_row, f32_row); return;
+    case 32: row_grad_vec<32>(row, pc, base, gam, wt, lane, dst, acc_row); return;
+    case 16: row_grad_vec<16>(row, pc, base, gam, wt, lane, dst, acc_row); return;
+    case 8: row_grad_vec<8>(row, pc, base, gam, wt, lane, dst, acc_row); return;
+    case 4: row_grad_vec<4>(row, pc, base, gam, wt, lane, dst, acc_row); return;
     default: break;
   }
   for (int q = 0; q < r; ++q) {                       // start at column `lane` (r a power of two): conflict-free
@@ -153,7 +170,6 @@ __device__ __forceinline__ void row_grad(const float* row, const float* pc, floa
     const float la = row[b];
     const float o = wt * (__expf(base + la + pc[b]) - __expf(la) * gam);
     if (acc_row != nullptr) atomicAdd(acc_row + b, o);
-    else if (f32_row != nullptr) atomicAdd(f32_row + b, o);
     else dst[b] = __float2bfloat16_rn(o);
   }
 }
@@ -168,7 +184,7 @@ __device__ __forceinline__ void row_grad(const float* row, const float* pc, floa
 // the windows into dT [n-1, r, r] (fp32): per CTA in shared memory first, then one atomicAdd per entry and CTA.
 // Shared memory: per warp n*r (alpha) + 2*r*r (tables) + 64 floats; static: + (n-1)*r*r floats per CTA.  r <= 32.
 __host__ __device__ inline size_t hmm_backward_warp_floats(int n, int r) {
-  return static_cast<size_t>(n) * r + 2 * r * r + 64;             // alphas, two tables, two vectors of 32
+  return (static_cast<size_t>(n) * (r + 2) + 3) / 4 * 4 + 2 * r * r + 64;   // alphas, prefixes (Eq. 6), two tables, two vectors of 32
 }
 __host__ __device__ inline size_t hmm_backward_smem_floats(int n, int r, bool is_static, int warps) {
   return static_cast<size_t>(warps) * hmm_backward_warp_floats(n, r) + (is_static ? static_cast<size_t>(n - 1) * r * r : 0);
@@ -179,7 +195,7 @@ __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const 
   extern __shared__ __align__(16) float sm[];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
-  const int n = a_.n, r = a_.r, len = a_.len;
+  const int n = a_.n, r = a_.r;
   const int rr = r * r;
   const bool is_static = table_stride == 0;
   float* acc = sm;                                                       // static only: [n-1, r, r]
@@ -193,20 +209,19 @@ __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const 
     for (int e = threadIdx.x; e < (n - 1) * rr; e += blockDim.x) acc[e] = 0.f;
     __syncthreads();
   }
-  // The steps after `len` carry no evidence and the transitions are normalised: the recursion stops at step len - 1.
   for (int w = next_window(work_counter, lane); w < a_.W; w = next_window(work_counter, lane)) {
     const float* g = a_.G + static_cast<size_t>(w) * n * r;
     const float* lw = a_.logw + static_cast<size_t>(w) * a_.sum_rows;
     const float* tb = tables + static_cast<size_t>(w) * table_stride;
-    const float wt = a_.weight[static_cast<size_t>(w) * a_.weight_stride];
+    const float wt = a_.weight[w];
     const size_t prow = static_cast<size_t>(w) * n * r;
     const size_t drow = static_cast<size_t>(w) * a_.dsum_pitch;
     // ---- forward, keeping every alpha_i
-    if (len > 1) warp_table_load_async(tabs, tb, rr, lane);
+    if (n > 1) warp_table_load_async(tabs, tb, rr, lane);
     float alpha = l.active ? lw[l.k] + g[l.k] : -CUDART_INF_F;
     if (has) alphas[lane] = alpha;
-    for (int i = 1; i < len; ++i) {
-      if (i + 1 < len) {
+    for (int i = 1; i < n; ++i) {
+      if (i + 1 < n) {
         warp_table_load_async(tabs + (i & 1) * rr, tb + static_cast<size_t>(i) * rr, rr, lane);
         cp_async_wait<1>();
       } else {
@@ -221,10 +236,10 @@ __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const 
     if (!has) alpha = -CUDART_INF_F;                                     // (the other parts' copies)
     const float logq = warp_lse_nan(alpha);
     if (lane == 0 && a_.out != nullptr) a_.out[w] = logq;
-    // ---- backward: tables in reverse order; the table of step len - 1 is still in its buffer
-    float beta = 0.f;                                                    // beta_{len-1}
-    for (int i = len - 1; i >= 1; --i) {
-      if (i < len - 1) {
+    // ---- backward: tables in reverse order; the table of step n - 1 is still in its buffer
+    float beta = 0.f;                                                    // beta_{n-1}
+    for (int i = n - 1; i >= 1; --i) {
+      if (i < n - 1) {
         cp_async_wait<0>();
         __syncwarp();
       }
@@ -233,7 +248,7 @@ __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const 
       const bool valid = a_.targets[static_cast<size_t>(w) * n + i] >= 0;
       if (has) {
         const float gamma = __expf(alphas[i * r + lane] + beta - logq);
-        put_post(a_, prow + static_cast<size_t>(i) * r + lane, valid ? wt * gamma : 0.f);
+        a_.post[prow + static_cast<size_t>(i) * r + lane] = valid ? wt * gamma : 0.f;
         cvec[lane] = g[i * r + lane] + beta;
       }
       __syncwarp();
@@ -242,23 +257,16 @@ __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const 
         const float al = alphas[(i - 1) * r + lane];
         const float gam_prev = __expf(al + beta_prev - logq);
         const size_t off = static_cast<size_t>(r) + static_cast<size_t>(i - 1) * rr + lane * r;
-        row_grad(A + lane * r, cvec, al - logq, gam_prev, wt, lane, r,
-                 (is_static || a_.accumulate) ? nullptr : a_.dsum + drow + off,
-                 is_static ? acc + static_cast<size_t>(i - 1) * rr + lane * r : nullptr,
-                 (!is_static && a_.accumulate) ? a_.dsum_f32 + drow + off : nullptr);
+        row_grad(A + lane * r, cvec, al - logq, gam_prev, wt, lane, r, is_static ? nullptr : a_.dsum + drow + off,
+                 is_static ? acc + static_cast<size_t>(i - 1) * rr + lane * r : nullptr);
       }
       beta = beta_prev;
       __syncwarp();                                                      // cvec and the table buffer are free again
     }
     if (has) {
       const float gamma0 = __expf(alphas[lane] + beta - logq);
-      put_post(a_, prow + lane, a_.targets[static_cast<size_t>(w) * n] >= 0 ? wt * gamma0 : 0.f);
-      put_dsum(a_, drow + lane, wt * (gamma0 - __expf(lw[lane])));
-      if (!a_.accumulate) {                                              // slots and tables past the prefix: no gradient
-        for (int i = len; i < n; ++i) a_.post[prow + static_cast<size_t>(i) * r + lane] = 0.f;
-        if (!is_static)
-          for (int e = (len - 1) * rr + lane; e < (n - 1) * rr; e += r) a_.dsum[drow + r + e] = __float2bfloat16_rn(0.f);
-      }
+      a_.post[prow + lane] = a_.targets[static_cast<size_t>(w) * n] >= 0 ? wt * gamma0 : 0.f;
+      a_.dsum[drow + lane] = __float2bfloat16_rn(wt * (gamma0 - __expf(lw[lane])));
     }
     __syncwarp();
   }
@@ -281,7 +289,7 @@ __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const 
 //   abar_{i-1}[a] = coeff_{i-1} softmax(alpha_{i-1})[a] + prop_{i-1}[a]                             times abar_i[b])
 // and dL/dG[i] = abar_i, dL/d logA_i[a][b] = the summand of prop_{i-1}[a]; through the row softmax of the transition
 // logits: summand - A_i[a][b] prop_{i-1}[a]; initial unit: abar_0 - omega sum_z abar_0[z]. Same streaming of the tables
-// and the same outputs as circuit_hmm_backward_kernel with accumulate == 0 (post fp32, dsum bf16, static dT by atomics).
+// and the same outputs as circuit_hmm_backward_kernel (post fp32, dsum bf16, static dT by atomics), and the prefixes themselves.
 template <int R>
 __device__ __forceinline__ void row_grad_mult_vec(const float* row, const float* pc, const float* mult, float base, float gam,
                                                   int lane, __nv_bfloat16* dst, float* acc_row) {
@@ -335,9 +343,8 @@ __device__ __forceinline__ void row_grad_mult(const float* row, const float* pc,
   }
 }
 
-__global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, const float* __restrict__ coeff,
-                                                 const float* __restrict__ tables, int table_stride, float* __restrict__ dT,
-                                                 unsigned* work_counter) {
+__global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, const float* __restrict__ tables,
+                                                 int table_stride, float* __restrict__ dT, unsigned* work_counter) {
   extern __shared__ __align__(16) float sm[];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
@@ -346,10 +353,11 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
   const bool is_static = table_stride == 0;
   float* acc = sm;                                                       // static only: [n-1, r, r]
   float* mine = sm + (is_static ? (n - 1) * rr : 0) + static_cast<size_t>(wib) * hmm_backward_warp_floats(n, r);
-  float* alphas = mine;                                                  // [n, r]
-  float* tabs = alphas + n * r;
+  float* tabs = mine;
   float* cvec = tabs + 2 * rr;                                           // G[i] - alpha_i (log domain)
   float* dvec = cvec + 32;                                               // abar_i (plain)
+  float* alphas = dvec + 32;                                             // [n][r + 1]
+  float* lps = alphas + n * (r + 1);                                     // [n] the prefix log-marginals
   const bool has = lane < r;
   const HmmLanes l = hmm_lanes(r, lane);
   if (is_static) {
@@ -360,7 +368,7 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
     const float* g = a_.G + static_cast<size_t>(w) * n * r;
     const float* lw = a_.logw + static_cast<size_t>(w) * a_.sum_rows;
     const float* tb = tables + static_cast<size_t>(w) * table_stride;
-    const float* cw = coeff + static_cast<size_t>(w) * n;
+    const float* cw = a_.coeff + static_cast<size_t>(w) * n;
     const int* tg = a_.targets + static_cast<size_t>(w) * n;
     const size_t prow = static_cast<size_t>(w) * n * r;
     const size_t drow = static_cast<size_t>(w) * a_.dsum_pitch;
@@ -378,14 +386,18 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
       __syncwarp();
       const float c = hmm_forward_step<true>(alpha, cvec, tabs + ((i - 1) & 1) * rr, l, r);
       alpha = l.active ? c + g[i * r + l.k] : -CUDART_INF_F;
-      if (has) alphas[i * r + lane] = alpha;
+      if (has) alphas[i * (r + 1) + lane] = alpha;
       __syncwarp();
     }
     if (!has) alpha = -CUDART_INF_F;                                     // (the other parts' copies)
-    const float lp = warp_lse_nan(alpha);                                // log p_{n-1}: the joint
-    if (lane == 0 && a_.out != nullptr) a_.out[w] = lp;
+    for (int i = lane; i < n; i += 32) {                                 // every prefix, lane = slot (as circuit_hmm_kernel)
+      const float lp = thread_lse(alphas + i * (r + 1), r);
+      lps[i] = lp;
+      a_.prefix[static_cast<size_t>(w) * n + i] = lp;
+    }
+    __syncwarp();
     // ---- reverse sweep: tables in reverse order; the table of step n - 1 is still in its buffer
-    float abar = has ? cw[n - 1] * __expf(alpha - lp) : 0.f;
+    float abar = has ? cw[n - 1] * __expf(alpha - lps[n - 1]) : 0.f;
     for (int i = n - 1; i >= 1; --i) {
       if (i < n - 1) {
         cp_async_wait<0>();
@@ -393,7 +405,7 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
       }
       if (i - 1 >= 1) warp_table_load_async(tabs + (i & 1) * rr, tb + static_cast<size_t>(i - 2) * rr, rr, lane);
       const float* A = tabs + ((i - 1) & 1) * rr;
-      const float al_i = has ? alphas[i * r + lane] : -CUDART_INF_F;
+      const float al_i = has ? alphas[i * (r + 1) + lane] : -CUDART_INF_F;
       if (has) {
         a_.post[prow + static_cast<size_t>(i) * r + lane] = tg[i] >= 0 ? abar : 0.f;
         cvec[lane] = al_i == -CUDART_INF_F ? -CUDART_INF_F : g[i * r + lane] - al_i;
@@ -403,8 +415,7 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
         dvec[lane] = 0.f;
       }
       __syncwarp();
-      const float al = has ? alphas[(i - 1) * r + lane] : -CUDART_INF_F;
-      const float lp_prev = warp_lse(al, has);                           // log p_{i-1}
+      const float al = has ? alphas[(i - 1) * (r + 1) + lane] : -CUDART_INF_F;
       float prop = 0.f;
       if (has) {
         const float* row = A + lane * r;
@@ -417,7 +428,7 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
         row_grad_mult(row, cvec, dvec, al, prop, lane, r, is_static ? nullptr : a_.dsum + drow + off,
                       is_static ? acc + static_cast<size_t>(i - 1) * rr + lane * r : nullptr);
       }
-      abar = has ? cw[i - 1] * __expf(al - lp_prev) + prop : 0.f;
+      abar = has ? cw[i - 1] * __expf(al - lps[i - 1]) + prop : 0.f;
       __syncwarp();                                                      // cvec, dvec and the table buffer are free again
     }
     float total = abar;                                                  // sum_z abar_0[z]
@@ -449,16 +460,11 @@ __host__ __device__ inline size_t btree_backward_warp_floats(int n, int r) {
   return 3 * static_cast<size_t>(n - 1) * r + 2 * static_cast<size_t>(r) * r + 32;
 }
 
-// With `loss_coeff` [W, n] (Eq. 6: L = sum_l coeff[w, l-1] log p_l over the prefix lengths l) the warp runs the pass of
-// every prefix length on its window back to back, accumulating (accumulate == 1): the window's tables and gradient rows
-// are then re-used out of L2 instead of being streamed from HBM once per prefix length.
-__global__ void circuit_btree_backward_kernel(const CircuitBackwardArgs a_, const float* __restrict__ loss_coeff,
-                                              unsigned* work_counter) {
+__global__ void circuit_btree_backward_kernel(const CircuitBackwardArgs a_, unsigned* work_counter) {
   extern __shared__ __align__(16) float sm[];
   const int wib = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int n = a_.n, r = a_.r;
-  int len = a_.len;                                                      // prefix length of the current pass
   float* prod = sm + static_cast<size_t>(wib) * btree_backward_warp_floats(n, r);
   float* S = prod + (n - 1) * r;
   float* U = S + (n - 1) * r;
@@ -469,49 +475,29 @@ __global__ void circuit_btree_backward_kernel(const CircuitBackwardArgs a_, cons
   const int rr = r * r;
   const int ntab = n - 2;
   auto child_of = [&](int t) { return 2 * (first_leaf_node - 1 - (t >> 1)) + 1 + (t & 1); };
-  // A node whose tokens all lie at or after `len` sees no evidence: its subtree evaluates to one, its table has no
-  // gradient, and it is skipped (first token of heap node c: index within its level times the level's width).
-  auto has_evidence = [&](int c) {
-    const int depth = 31 - __clz(c + 1);
-    return ((c + 1 - (1 << depth)) * (n >> depth)) < len;
-  };
   for (int w = next_window(work_counter, lane); w < a_.W; w = next_window(work_counter, lane)) {
     const float* g = a_.G + static_cast<size_t>(w) * n * r;
     const float* lw = a_.logw + static_cast<size_t>(w) * a_.sum_rows;
     const size_t drow = static_cast<size_t>(w) * a_.dsum_pitch;
-    for (len = loss_coeff ? 1 : a_.len; len <= (loss_coeff ? n : a_.len); ++len) {
-    const float wt = loss_coeff ? loss_coeff[static_cast<size_t>(w) * n + len - 1]
-                                : a_.weight[static_cast<size_t>(w) * a_.weight_stride];
-    if (loss_coeff != nullptr && wt == 0.f) continue;                    // the same for every lane of the warp
-    // ---- upward (tokens >= len are summed out: their input units output one)
+    const float wt = a_.weight[w];
+    // ---- upward
     for (int j = n - 2; j >= first_leaf_node; --j) {
       const int t0 = 2 * (j - first_leaf_node);
-      if (has) prod[j * r + lane] = (t0 < len ? g[t0 * r + lane] : 0.f) + (t0 + 1 < len ? g[(t0 + 1) * r + lane] : 0.f);
+      if (has) prod[j * r + lane] = g[t0 * r + lane] + g[(t0 + 1) * r + lane];
     }
-    auto next_up = [&](int t) {                                          // next table of the upward pass that is needed
-      while (t < ntab && !has_evidence(child_of(t))) ++t;
-      return t;
-    };
-    int buf = 0;
-    int tn = next_up(0);
-    if (tn < ntab) warp_table_load_async(tabs, lw + r + static_cast<size_t>(child_of(tn) - 1) * rr, rr, lane);
+    if (ntab > 0) warp_table_load_async(tabs, lw + r + static_cast<size_t>(child_of(0) - 1) * rr, rr, lane);
     __syncwarp();
     float acc = 0.f;
     for (int t = 0; t < ntab; ++t) {
       const int c = child_of(t);
-      float sc = 0.f;                                                    // a subtree without evidence: log 1
-      if (t == tn) {
-        tn = next_up(t + 1);
-        if (tn < ntab) {
-          warp_table_load_async(tabs + (buf ^ 1) * rr, lw + r + static_cast<size_t>(child_of(tn) - 1) * rr, rr, lane);
-          cp_async_wait<1>();
-        } else {
-          cp_async_wait<0>();
-        }
-        __syncwarp();
-        sc = sum_layer_staged(tabs + buf * rr, prod + c * r, lane, r);
-        buf ^= 1;
+      if (t + 1 < ntab) {
+        warp_table_load_async(tabs + ((t + 1) & 1) * rr, lw + r + static_cast<size_t>(child_of(t + 1) - 1) * rr, rr, lane);
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
       }
+      __syncwarp();
+      const float sc = sum_layer_staged(tabs + (t & 1) * rr, prod + c * r, lane, r);
       if (has) S[c * r + lane] = sc;
       acc += sc;
       if (t & 1) {
@@ -525,30 +511,22 @@ __global__ void circuit_btree_backward_kernel(const CircuitBackwardArgs a_, cons
     // ---- downward, children c = 1 .. n-2 in address order
     if (has) {
       U[lane] = lw[lane];
-      put_dsum(a_, drow + lane, wt * (__expf(lw[lane] + prod[lane] - logq) - __expf(lw[lane])));
+      a_.dsum[drow + lane] = __float2bfloat16_rn(wt * (__expf(lw[lane] + prod[lane] - logq) - __expf(lw[lane])));
     }
-    auto next_down = [&](int c) {
-      while (c <= ntab && !has_evidence(c)) ++c;
-      return c;
-    };
-    buf = 0;
-    int cn = next_down(1);
-    if (cn <= ntab) warp_table_load_async(tabs, lw + r + static_cast<size_t>(cn - 1) * rr, rr, lane);
+    if (ntab > 0) warp_table_load_async(tabs, lw + r, rr, lane);
     __syncwarp();
-    for (int c = cn; c <= ntab; c = cn) {
+    for (int c = 1; c <= ntab; ++c) {
       const int j = (c - 1) >> 1;
       const int sib = (c & 1) ? c + 1 : c - 1;
-      cn = next_down(c + 1);
-      if (cn <= ntab) {
-        warp_table_load_async(tabs + (buf ^ 1) * rr, lw + r + static_cast<size_t>(cn - 1) * rr, rr, lane);
+      if (c < ntab) {
+        warp_table_load_async(tabs + (c & 1) * rr, lw + r + static_cast<size_t>(c) * rr, rr, lane);
         cp_async_wait<1>();
       } else {
         cp_async_wait<0>();
       }
       if (has) cur[lane] = U[j * r + lane] + S[sib * r + lane];          // in[z]
       __syncwarp();
-      const float* tab = tabs + buf * rr;
-      buf ^= 1;
+      const float* tab = tabs + ((c - 1) & 1) * rr;
       if (has) {
         // message to the child: lane b, over the parent's values z (column of the table)
         float m = -CUDART_INF_F;
@@ -560,8 +538,7 @@ __global__ void circuit_btree_backward_kernel(const CircuitBackwardArgs a_, cons
         const float in_z = cur[lane];
         const float gam_parent = __expf(U[j * r + lane] + prod[j * r + lane] - logq);
         const size_t off = static_cast<size_t>(r) + static_cast<size_t>(c - 1) * rr + lane * r;
-        row_grad(tab + lane * r, prod + c * r, in_z - logq, gam_parent, wt, lane, r,
-                 a_.accumulate ? nullptr : a_.dsum + drow + off, nullptr, a_.accumulate ? a_.dsum_f32 + drow + off : nullptr);
+        row_grad(tab + lane * r, prod + c * r, in_z - logq, gam_parent, wt, lane, r, a_.dsum + drow + off, nullptr);
       }
       __syncwarp();
     }
@@ -569,26 +546,172 @@ __global__ void circuit_btree_backward_kernel(const CircuitBackwardArgs a_, cons
     for (int i = 0; i < n; ++i) {
       const int o = first_leaf_node + (i >> 1);
       const bool valid = a_.targets[static_cast<size_t>(w) * n + i] >= 0;
-      if (has) {
-        const size_t idx = (static_cast<size_t>(w) * n + i) * r + lane;
-        if (i < len) put_post(a_, idx, valid ? wt * __expf(U[o * r + lane] + prod[o * r + lane] - logq) : 0.f);
-        else if (!a_.accumulate) a_.post[idx] = 0.f;
-      }
+      if (has)
+        a_.post[(static_cast<size_t>(w) * n + i) * r + lane] = valid ? wt * __expf(U[o * r + lane] + prod[o * r + lane] - logq) : 0.f;
     }
     __syncwarp();
-    }                                                                    // prefix lengths
   }
 }
 
-// fp32 [rows, cols] (pitch src_pitch) -> bf16 (pitch dst_pitch): the accumulated sum-unit logit gradients become the
-// tensor cores' operand.
-__global__ void f32_rows_to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int rows, int cols,
-                                        size_t src_pitch, size_t dst_pitch) {
-  const size_t total = static_cast<size_t>(rows) * cols;
-  for (size_t e = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
-       e += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const size_t rw = e / cols, c = e - rw * cols;
-    dst[rw * dst_pitch + c] = __float2bfloat16_rn(src[rw * src_pitch + c]);
+// ---------------------------------------------------------------- Eq. 6 through the binary tree in one sweep
+// L = sum_j coeff_j log p_j. TreeSweep's upward and downward sweeps give every prefix log p_j from the messages S and D; the
+// gradient is their reverse mode, in plain numbers of either sign (bounded by sum_j |coeff_j|):
+//   owner of the tokens 2m, 2m+1, with rho_0 = softmax(D + G[2m]), rho_1 = softmax(D + G[2m] + G[2m+1]):
+//     dD = c_{2m} rho_0 + c_{2m+1} rho_1, which also goes to G[2m]; c_{2m+1} rho_1 to G[2m+1];
+//   back up the tree (reverse of the downward sweep): D_c[b] = LSE_z(in_c[z] + T_c[z][b]) gives
+//     pd_c[z] = sum_b dD_c[b] exp(in_c[z] + T_c[z][b] - D_c[b]), dD of the parent = the sum over its two children, and pd of a
+//     right child is also the gradient of its left sibling's S;
+//   down again (reverse of the upward sweep): dS_c = pd of the right sibling (left children) + dprod of the parent, and
+//     S_c[z] = LSE_b(T_c[z][b] + prod_c[b]) gives dprod_c[b] = sum_z dS_c[z] exp(T_c[z][b] + prod_c[b] - S_c[z]), which reaches
+//     the two tokens of an owner. Here both parts of dL/dT_c[z][b] are at hand; through the row softmax of the table's logits:
+//     (its two summands) - exp(T_c[z][b]) (pd_c[z] + dS_c[z]).
+// Four passes over a window's n - 2 tables in shared memory (6 exponentials an entry), each table read from and its gradient
+// written to HBM once, as bf16. The n backward passes of the prefix lengths it replaces read and accumulated the window's 57 KB
+// n times (2186 us at 4096 windows, n = 16, r = 32, plus 48 us zeroing and 184 us converting the fp32 accumulators and 313 us
+// for the prefixes; this kernel does all of it in 392 us, its shared-memory and exponential work; HBM would take 80 us). One CTA per window, a warp per node of a level, as circuit_btree_prefix_kernel.
+__host__ __device__ inline size_t btree_loss_smem_floats(int n, int r, int warps, bool tables_in_smem) {
+  const size_t vr = (static_cast<size_t>(r) + 3) / 4 * 4;
+  return btree_prefix_smem_floats(n, r, warps, tables_in_smem) +
+         (4 * static_cast<size_t>(n - 1) + n / 2 + 4 * static_cast<size_t>(warps)) * vr;
+}
+__global__ void __launch_bounds__(256) circuit_btree_loss_backward_kernel(const CircuitBackwardArgs a_, int tables_in_smem) {
+  extern __shared__ __align__(16) float sm[];
+  const int n = a_.n, r = a_.r;
+  TreeSweep t;
+  t.init(sm, n, r, tables_in_smem != 0);
+  const int lane = t.lane, wib = t.wib, warps = t.warps, vr = t.vr;
+  const bool has = lane < r;
+  float* dD = t.after();                           // [n - 1][vr] gradient of D
+  float* pd = dD + (n - 1) * vr;                   // [n - 1][vr] gradient of in_c, per parent value
+  float* dP = pd + (n - 1) * vr;                   // [n - 1][vr] gradient of prod_c
+  float* dS = dP + (n - 1) * vr;                   // [n - 1][vr] gradient of S_c
+  float* late = dS + (n - 1) * vr;                 // [n / 2][vr] c_{2m+1} rho_1
+  float* vec = late + t.owners * vr + wib * 4 * vr;   // four vectors of this warp
+  const int w0 = static_cast<int>(static_cast<long long>(blockIdx.x) * a_.W / gridDim.x);
+  const int w1 = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * a_.W / gridDim.x);
+  for (int w = w0; w < w1; ++w) {
+    const float* cw = a_.coeff + static_cast<size_t>(w) * n;
+    const int* tg = a_.targets + static_cast<size_t>(w) * n;
+    __nv_bfloat16* drow = a_.dsum + static_cast<size_t>(w) * a_.dsum_pitch;
+    t.load(a_.G + static_cast<size_t>(w) * n * r, a_.logw + static_cast<size_t>(w) * a_.sum_rows, true);
+    t.up();
+    t.down();
+    for (int m = wib; m < t.owners; m += warps) {  // prefixes and the gradient of the owners' D
+      const int o = t.first_leaf_node + m;
+      const float d1 = has ? t.D[o * vr + lane] + t.gs[2 * m * vr + lane] : -CUDART_INF_F;
+      const float d2 = has ? d1 + t.gs[(2 * m + 1) * vr + lane] : -CUDART_INF_F;
+      const float p0 = warp_lse_nan(d1), p1 = warp_lse_nan(d2);
+      if (lane == 0) {
+        a_.prefix[static_cast<size_t>(w) * n + 2 * m] = p0;
+        a_.prefix[static_cast<size_t>(w) * n + 2 * m + 1] = p1;
+        if (a_.out != nullptr && m == t.owners - 1) a_.out[w] = p1;
+      }
+      if (has) {
+        const float l = cw[2 * m + 1] * __expf(d2 - p1);
+        late[m * vr + lane] = l;
+        dD[o * vr + lane] = fmaf(cw[2 * m], __expf(d1 - p0), l);
+      }
+    }
+    __syncthreads();
+    for (int L = t.depth; L >= 1; --L) {           // reverse of the downward sweep
+      for (int c = (1 << L) - 1 + wib; c <= (2 << L) - 2; c += warps) {
+        float* dc = vec;                           // the child's D and dD, read by every lane
+        if (has) {
+          if (L < t.depth) dD[c * vr + lane] = pd[(2 * c + 1) * vr + lane] + pd[(2 * c + 2) * vr + lane];
+          dc[lane] = t.D[c * vr + lane];
+        }
+        const float in_z = has ? t.in_of(c) : 0.f;
+        __syncwarp();
+        const float* tab = t.table_of(c);
+        if (has) {
+          const float* row = tab + lane * r;
+          float acc = 0.f;
+          if ((r & 3) == 0) {                      // float4 reads, rotated by the lane: conflict-free
+            const int Q = r / 4;
+            const float4* row4 = reinterpret_cast<const float4*>(row);
+            const float4* d4 = reinterpret_cast<const float4*>(dc);
+            const float4* g4 = reinterpret_cast<const float4*>(dD + c * vr);
+            float a1 = 0.f;
+#pragma unroll 4
+            for (int q = 0; q < Q; ++q) {
+              const int j = (q + lane) & (Q - 1);
+              const float4 x = row4[j], d = d4[j], e = g4[j];
+              acc = fmaf(e.x, __expf(in_z + x.x - d.x), acc);
+              a1 = fmaf(e.y, __expf(in_z + x.y - d.y), a1);
+              acc = fmaf(e.z, __expf(in_z + x.z - d.z), acc);
+              a1 = fmaf(e.w, __expf(in_z + x.w - d.w), a1);
+            }
+            acc += a1;
+          } else {
+            for (int b = 0; b < r; ++b) acc = fmaf(dD[c * vr + b], __expf(in_z + row[b] - dc[b]), acc);
+          }
+          pd[c * vr + lane] = acc;
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+    }
+    if (wib == 0) {                                // the root's logits
+      if (t.depth > 0 && has) dD[lane] = pd[vr + lane] + pd[2 * vr + lane];
+      float d0 = has ? dD[lane] : 0.f;
+      float total = d0;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) total += __shfl_xor_sync(kFull, total, off);
+      if (has) drow[lane] = __float2bfloat16_rn(d0 - __expf(t.lw[lane]) * total);
+    }
+    for (int L = 1; L <= t.depth; ++L) {           // reverse of the upward sweep, and the tables' gradients
+      for (int c = (1 << L) - 1 + wib; c <= (2 << L) - 2; c += warps) {
+        const bool edge = c == (2 << L) - 2;       // on the right edge: no S
+        const int j = (c - 1) >> 1;
+        const bool edge_parent = j == (1 << L) - 2;   // (the root included)
+        float* inv = vec;                          // per parent value: in, S, dS and pd + dS
+        float* sv = vec + vr;
+        float* dsv = vec + 2 * vr;
+        float* sumv = vec + 3 * vr;
+        float prod = 0.f, Dc = 0.f, dDc = 0.f;
+        if (has) {
+          const float ds = edge ? 0.f : ((c & 1) ? pd[(c + 1) * vr + lane] : 0.f) + (edge_parent ? 0.f : dP[j * vr + lane]);
+          inv[lane] = t.in_of(c);
+          sv[lane] = edge ? 0.f : t.S[c * vr + lane];
+          dsv[lane] = ds;
+          sumv[lane] = pd[c * vr + lane] + ds;
+          if (!edge) prod = t.prod_of(c);
+          Dc = t.D[c * vr + lane];
+          dDc = dD[c * vr + lane];
+        }
+        __syncwarp();
+        const float* tab = t.table_of(c);
+        float acc = 0.f;
+        if (has) {
+          __nv_bfloat16* dst = drow + r + static_cast<size_t>(c - 1) * r * r + lane;
+          const float* col = tab + lane;
+#pragma unroll 4
+          for (int z = 0; z < r; ++z) {
+            const float x = col[z * r];
+            float xi = dDc * __expf(inv[z] + x - Dc);
+            if (!edge) {
+              const float e2 = dsv[z] * __expf(x + prod - sv[z]);
+              acc += e2;
+              xi += e2;
+            }
+            dst[z * r] = __float2bfloat16_rn(fmaf(-__expf(x), sumv[z], xi));
+          }
+          dP[c * vr + lane] = acc;
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+    }
+    for (int m = wib; m < t.owners; m += warps) {  // evidence of the tokens 2m and 2m + 1
+      const int o = t.first_leaf_node + m;
+      if (has) {
+        const float back = t.depth > 0 && m < t.owners - 1 ? dP[o * vr + lane] : 0.f;   // (the last owner is on the right edge)
+        float* dst = a_.post + (static_cast<size_t>(w) * n + 2 * m) * r + lane;
+        dst[0] = tg[2 * m] >= 0 ? dD[o * vr + lane] + back : 0.f;
+        dst[r] = tg[2 * m + 1] >= 0 ? late[m * vr + lane] + back : 0.f;
+      }
+    }
+    __syncthreads();                               // shared memory is reused by the next window
   }
 }
 

@@ -99,6 +99,27 @@ __global__ void circuit_cp_kernel(const float* __restrict__ G, const float* __re
 // shared tile, so that no slot waits for another one's reduction. Shared memory: cp_prefix_smem_floats per warp.
 constexpr int kCpTileSlots = 32;
 __host__ __device__ inline int cp_prefix_warp_floats(int n, int r) { return (n < kCpTileSlots ? n : kCpTileSlots) * (r + 1); }
+// Slots [i0, i0 + nc) of one window: leaves msg_{i+1}[k] in tile[(i - i0) (r + 1) + k] and, if mw is given, msg_i[k] in
+// mw[i r + k]. `first`: the messages of slot i0 (log omega, or the last row of the tile before). Ends with a warp barrier.
+__device__ __forceinline__ void cp_prefix_tile(const float* __restrict__ g, const float* first, float* tile,
+                                               float* __restrict__ mw, int i0, int nc, int r, int lane) {
+  for (int k = lane; k < r; k += 32) {
+    float a = first[k];
+    for (int c0 = 0; c0 < nc; c0 += 8) {
+      float gv[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) gv[q] = c0 + q < nc ? g[(i0 + c0 + q) * r + k] : 0.f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (c0 + q < nc) {
+          if (mw != nullptr) mw[(i0 + c0 + q) * r + k] = a;
+          a += gv[q];
+          tile[(c0 + q) * (r + 1) + k] = a;
+        }
+    }
+  }
+  __syncwarp();
+}
 __global__ void circuit_cp_prefix_kernel(const float* __restrict__ G, const float* __restrict__ logw,
                                          float* __restrict__ out, float* __restrict__ prefix, float* __restrict__ msg, int W,
                                          int wpp, int n, int r, int sum_rows, int raw_mixture) {
@@ -116,22 +137,7 @@ __global__ void circuit_cp_prefix_kernel(const float* __restrict__ G, const floa
   if (raw_mixture) norm = thread_lse(lw, r);
   for (int i0 = 0; i0 < n; i0 += kCpTileSlots) {
     const int nc = min(kCpTileSlots, n - i0);
-    for (int k = lane; k < r; k += 32) {
-      float a = i0 == 0 ? lw[k] : tile[(kCpTileSlots - 1) * (r + 1) + k];
-      for (int c0 = 0; c0 < nc; c0 += 8) {
-        float gv[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) gv[q] = c0 + q < nc ? g[(i0 + c0 + q) * r + k] : 0.f;
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (c0 + q < nc) {
-            if (mw != nullptr) mw[(i0 + c0 + q) * r + k] = a;
-            a += gv[q];
-            tile[(c0 + q) * (r + 1) + k] = a;
-          }
-      }
-    }
-    __syncwarp();
+    cp_prefix_tile(g, i0 == 0 ? lw : tile + (kCpTileSlots - 1) * (r + 1), tile, mw, i0, nc, r, lane);
     if (lane < nc) {
       const float res = thread_lse(tile + lane * (r + 1), r) - norm;
       if (prefix != nullptr) prefix[static_cast<size_t>(w) * n + i0 + lane] = res;
@@ -340,9 +346,86 @@ __device__ __forceinline__ float warp_lse_nan(float x) {
 // r = 32): each warp stages the table it needs. A CTA takes a contiguous run of windows and keeps the tables while the
 // position stays the same. Measured against one warp per window and a path per prefix: 4096 windows at n = 16, r = 32:
 // 256 -> 148 us; 108 windows at n = 8: 36 -> 6 us. Shared memory: btree_prefix_smem_floats.
+// One window of a tree sweep, shared by a CTA. vr: pitch of the [r] vectors (r rounded up to 4 floats).
+struct TreeSweep {
+  int n, r, vr, owners, first_leaf_node, depth;    // depth: the owners' level; level L holds the nodes 2^L - 1 .. 2^(L+1) - 2
+  int wib, lane, warps;
+  float* tabs;                                     // the n - 2 tables, or one tile per warp
+  float *S, *D, *gs, *vec;                         // [n - 1][vr], [n - 1][vr], [n][vr], this warp's vector [vr]
+  const float* lw;                                 // the position's row of log omega
+  bool resident;
+
+  __device__ void init(float* sm, int n_, int r_, bool tables_in_smem) {
+    n = n_; r = r_; vr = (r + 3) / 4 * 4;
+    owners = n / 2; first_leaf_node = owners - 1; depth = 31 - __clz(owners);
+    wib = threadIdx.x >> 5; lane = threadIdx.x & 31; warps = blockDim.x >> 5;
+    resident = tables_in_smem;
+    tabs = sm;
+    S = sm + ((tables_in_smem ? (n - 2) : warps) * r * r + 3) / 4 * 4;
+    D = S + (n - 1) * vr;
+    gs = D + (n - 1) * vr;
+    vec = gs + n * vr + wib * vr;
+  }
+  __device__ float* after() const { return gs + (n + warps) * vr; }   // the shared memory past the sweep's own
+  // Start of window w: the position's tables (unless they are still there), its evidence, log omega of the root.
+  __device__ void load(const float* __restrict__ g, const float* __restrict__ lw_, bool new_tables) {
+    lw = lw_;
+    if (resident && new_tables) {
+      const int count = (n - 2) * r * r;
+      if ((count & 3) == 0 && (reinterpret_cast<uintptr_t>(lw + r) & 15u) == 0) {
+        for (int e = threadIdx.x * 4; e < count; e += blockDim.x * 4) cp_async_16(tabs + e, lw + r + e);
+      } else {
+        for (int e = threadIdx.x; e < count; e += blockDim.x) cp_async_4(tabs + e, lw + r + e);
+      }
+      cp_async_commit();
+    }
+    for (int e = threadIdx.x; e < n * r; e += blockDim.x) gs[(e / r) * vr + e % r] = g[e];
+    if (threadIdx.x < r) D[threadIdx.x] = lw[threadIdx.x];
+    cp_async_wait<0>();
+    __syncthreads();
+  }
+  __device__ const float* table_of(int c) const {  // node c's table; not resident: staged into the warp's own tile
+    if (resident) return tabs + (c - 1) * r * r;
+    warp_table_load_async(tabs + wib * r * r, lw + r + static_cast<size_t>(c - 1) * r * r, r * r, lane);
+    cp_async_wait<0>();
+    __syncwarp();
+    return tabs + wib * r * r;
+  }
+  __device__ float prod_of(int c) const {          // lane's entry of the product unit of node c (its subtree given z_c = lane)
+    return c >= first_leaf_node ? gs[2 * (c - first_leaf_node) * vr + lane] + gs[(2 * (c - first_leaf_node) + 1) * vr + lane]
+                                : S[(2 * c + 1) * vr + lane] + S[(2 * c + 2) * vr + lane];
+  }
+  __device__ float in_of(int c) const {            // what comes down to node c's table, per parent value
+    return D[((c - 1) >> 1) * vr + lane] + ((c & 1) ? 0.f : S[(c - 1) * vr + lane]);
+  }
+  __device__ void up() {                           // S of every node that is not on the right edge
+    for (int L = depth; L >= 1; --L) {
+      for (int c = (1 << L) - 1 + wib; c < (2 << L) - 2; c += warps) {
+        if (lane < r) vec[lane] = prod_of(c);
+        __syncwarp();
+        const float sc = sum_layer_staged(table_of(c), vec, lane, r);
+        if (lane < r) S[c * vr + lane] = sc;
+        __syncwarp();
+      }
+      __syncthreads();
+    }
+  }
+  __device__ void down() {                         // D of every node
+    for (int L = 1; L <= depth; ++L) {
+      for (int c = (1 << L) - 1 + wib; c <= (2 << L) - 2; c += warps) {
+        if (lane < r) vec[lane] = in_of(c);
+        __syncwarp();
+        const float dc = down_layer(table_of(c), vec, lane, r);
+        if (lane < r) D[c * vr + lane] = dc;
+        __syncwarp();
+      }
+      __syncthreads();
+    }
+  }
+};
 __host__ __device__ inline size_t btree_prefix_smem_floats(int n, int r, int warps, bool tables_in_smem) {
-  const size_t rr = static_cast<size_t>(r) * r, vec = (static_cast<size_t>(r) + 3) / 4 * 4;
-  return ((tables_in_smem ? (n - 2) * rr : warps * rr) + 3) / 4 * 4 + (2 * static_cast<size_t>(n - 1) + n + warps) * vec;
+  const size_t rr = static_cast<size_t>(r) * r, vr = (static_cast<size_t>(r) + 3) / 4 * 4;
+  return ((tables_in_smem ? (n - 2) * rr : warps * rr) + 3) / 4 * 4 + (2 * static_cast<size_t>(n - 1) + n + warps) * vr;
 }
 __global__ void __launch_bounds__(256) circuit_btree_prefix_kernel(const float* __restrict__ G, const float* __restrict__ logw,
                                                                    float* __restrict__ out, float* __restrict__ prefix,
@@ -351,84 +434,34 @@ __global__ void __launch_bounds__(256) circuit_btree_prefix_kernel(const float* 
   extern __shared__ __align__(16) float sm[];
   grid_launch_dependents();
   grid_dependency_wait();   // G and log omega come from the kernels before this one
-  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-  const int rr = r * r, vr = (r + 3) / 4 * 4;
-  const bool has = lane < r;
-  float* tabs = sm;
-  float* S = sm + ((tables_in_smem ? (n - 2) * rr : warps * rr) + 3) / 4 * 4;
-  float* D = S + (n - 1) * vr;
-  float* gs = D + (n - 1) * vr;                    // evidence of the window [n][vr]
-  float* vec = gs + n * vr + wib * vr;             // one vector per warp
-  const int owners = n / 2, first_leaf_node = owners - 1;
-  const int depth = 31 - __clz(owners);            // the owners' level; level L holds the nodes 2^L - 1 .. 2^(L+1) - 2
+  TreeSweep t;
+  t.init(sm, n, r, tables_in_smem != 0);
   const int w0 = static_cast<int>(static_cast<long long>(blockIdx.x) * W / gridDim.x);
   const int w1 = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * W / gridDim.x);
   int last_pos = -1;
   for (int w = w0; w < w1; ++w) {
     const int pos = w / wpp;
-    const float* lw = logw + static_cast<size_t>(pos) * sum_rows;
-    const float* g = G + static_cast<size_t>(w) * n * r;
-    if (tables_in_smem && pos != last_pos) {
-      const int count = (n - 2) * rr;
-      const bool vec16 = (count & 3) == 0 && ((reinterpret_cast<uintptr_t>(lw + r)) & 15u) == 0;
-      if (vec16) {
-        for (int e = threadIdx.x * 4; e < count; e += blockDim.x * 4) cp_async_16(tabs + e, lw + r + e);
-      } else {
-        for (int e = threadIdx.x; e < count; e += blockDim.x) cp_async_4(tabs + e, lw + r + e);
-      }
-      cp_async_commit();
-      last_pos = pos;
-    }
-    for (int e = threadIdx.x; e < n * r; e += blockDim.x) gs[(e / r) * vr + e % r] = g[e];
-    if (threadIdx.x < r) D[threadIdx.x] = lw[threadIdx.x];
-    cp_async_wait<0>();
-    __syncthreads();
-    auto table_of = [&](int c) -> const float* {   // node c's table; not resident: staged into the warp's own tile
-      if (tables_in_smem) return tabs + (c - 1) * rr;
-      warp_table_load_async(tabs + wib * rr, lw + r + static_cast<size_t>(c - 1) * rr, rr, lane);
-      cp_async_wait<0>();
-      __syncwarp();
-      return tabs + wib * rr;
-    };
-    for (int L = depth; L >= 1; --L) {             // upward, without the nodes on the right edge
-      for (int c = (1 << L) - 1 + wib; c < (2 << L) - 2; c += warps) {
-        if (has) {
-          vec[lane] = L == depth ? gs[2 * (c - first_leaf_node) * vr + lane] + gs[(2 * (c - first_leaf_node) + 1) * vr + lane]
-                                 : S[(2 * c + 1) * vr + lane] + S[(2 * c + 2) * vr + lane];
-        }
-        __syncwarp();
-        const float sc = sum_layer_staged(table_of(c), vec, lane, r);
-        if (has) S[c * vr + lane] = sc;
-        __syncwarp();
-      }
-      __syncthreads();
-    }
-    for (int L = 1; L <= depth; ++L) {             // downward
-      for (int c = (1 << L) - 1 + wib; c <= (2 << L) - 2; c += warps) {
-        if (has) vec[lane] = D[((c - 1) >> 1) * vr + lane] + ((c & 1) ? 0.f : S[(c - 1) * vr + lane]);
-        __syncwarp();
-        const float dc = down_layer(table_of(c), vec, lane, r);
-        if (has) D[c * vr + lane] = dc;
-        __syncwarp();
-      }
-      __syncthreads();
-    }
-    for (int m = wib; m < owners; m += warps) {    // the tokens 2m and 2m + 1
-      const float d = has ? D[(first_leaf_node + m) * vr + lane] : -CUDART_INF_F;
-      const float d1 = has ? d + gs[2 * m * vr + lane] : -CUDART_INF_F;
-      const float d2 = has ? d1 + gs[(2 * m + 1) * vr + lane] : -CUDART_INF_F;
+    t.load(G + static_cast<size_t>(w) * n * r, logw + static_cast<size_t>(pos) * sum_rows, pos != last_pos);
+    last_pos = pos;
+    t.up();
+    t.down();
+    for (int m = t.wib; m < t.owners; m += t.warps) {    // the tokens 2m and 2m + 1
+      const bool has = t.lane < r;
+      const float d = has ? t.D[(t.first_leaf_node + m) * t.vr + t.lane] : -CUDART_INF_F;
+      const float d1 = has ? d + t.gs[2 * m * t.vr + t.lane] : -CUDART_INF_F;
+      const float d2 = has ? d1 + t.gs[(2 * m + 1) * t.vr + t.lane] : -CUDART_INF_F;
       if (msg != nullptr && has) {
-        float* mw = msg + (static_cast<size_t>(w) * n + 2 * m) * r + lane;
+        float* mw = msg + (static_cast<size_t>(w) * n + 2 * m) * r + t.lane;
         mw[0] = d;
         mw[r] = d1;
       }
       const float p0 = warp_lse_nan(d1), p1 = warp_lse_nan(d2);
-      if (lane == 0) {
+      if (t.lane == 0) {
         if (prefix != nullptr) {
           prefix[static_cast<size_t>(w) * n + 2 * m] = p0;
           prefix[static_cast<size_t>(w) * n + 2 * m + 1] = p1;
         }
-        if (out != nullptr && m == owners - 1) out[w] = p1;
+        if (out != nullptr && m == t.owners - 1) out[w] = p1;
       }
     }
     __syncthreads();                               // shared memory is reused by the next window
@@ -649,40 +682,50 @@ __global__ void latent_sample_kernel(int family, const float* __restrict__ logw,
 // L positions with overlapping windows. The conditional of slot j given the context and the window's earlier bytes
 // is the difference of consecutive prefix log-marginals; V_ij counts the valid (non-negative) targets of slot j in
 // sequence i. Two kernels, both with a fixed reduction order, so the result does not change from run to run.
-constexpr int kLossThreads = 256;
+constexpr int kLossThreads = 1024;
+// Both kernels that walk a sequence give thread t the slot t % n and the positions t / n, t / n + kLossThreads / n, ..., so
+// that a warp's loads of the [T, n] rows are contiguous; the threads of a slot are then added up in a fixed order. (A thread
+// per position and slot after slot read every row n times, 4 bytes in every 4 n: 28 + 30 us at n = 16, 4 sequences of 1024
+// positions, against 20 + 10.)
+__device__ __forceinline__ int loss_rows_per_step(int n) { return kLossThreads / n; }
+// x[q * n + j], q < step, added up over q by the whole CTA into x[j] (halving tree: the order depends on n alone).
+template <typename T>
+__device__ __forceinline__ void loss_add_rows(T* x, int step, int n) {
+  const int q = threadIdx.x / n;
+  int half = 1;
+  while (2 * half < step) half *= 2;
+  for (; half > 0; half >>= 1) {
+    __syncthreads();
+    if (q < half && q + half < step) x[threadIdx.x] += x[threadIdx.x + half * n];
+  }
+  __syncthreads();
+}
 
 // grid = N. partial[i, j] = (1/V_ij) sum_{t valid} (prefix[t, j] - prefix[t, j-1]), 0 if V_ij = 0.
 __global__ void __launch_bounds__(kLossThreads) loss_partial_kernel(const float* __restrict__ prefix,
                                                                     const int* __restrict__ targets,
                                                                     float* __restrict__ partial, int L, int n) {
-  __shared__ float ssum[kLossThreads / 32];
-  __shared__ int scnt[kLossThreads / 32];
-  const int i = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int j = 0; j < n; ++j) {
-    float sum = 0.f;
-    int cnt = 0;
-    for (int t = threadIdx.x; t < L; t += kLossThreads) {
+  __shared__ float ssum[kLossThreads];
+  __shared__ int scnt[kLossThreads];
+  const int i = blockIdx.x, step = loss_rows_per_step(n), j = threadIdx.x % n;
+  float sum = 0.f;
+  int cnt = 0;
+  if (threadIdx.x < step * n) {
+    for (int t = threadIdx.x / n; t < L; t += step) {
       const size_t row = (static_cast<size_t>(i) * L + t) * n;
       if (targets[row + j] >= 0) {
         sum += prefix[row + j] - (j > 0 ? prefix[row + j - 1] : 0.f);
         cnt += 1;
       }
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      sum += __shfl_xor_sync(kFull, sum, off);
-      cnt += __shfl_xor_sync(kFull, cnt, off);
-    }
-    if (lane == 0) { ssum[warp] = sum; scnt[warp] = cnt; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float tot = 0.f;
-      int c = 0;
-      for (int q = 0; q < kLossThreads / 32; ++q) { tot += ssum[q]; c += scnt[q]; }
-      partial[static_cast<size_t>(i) * n + j] = c > 0 ? tot / static_cast<float>(c) : 0.f;
-    }
-    __syncthreads();
+  }
+  ssum[threadIdx.x] = sum;
+  scnt[threadIdx.x] = cnt;
+  loss_add_rows(ssum, step, n);
+  loss_add_rows(scnt, step, n);
+  if (threadIdx.x < n) {
+    const int c = scnt[threadIdx.x];
+    partial[static_cast<size_t>(i) * n + threadIdx.x] = c > 0 ? ssum[threadIdx.x] / static_cast<float>(c) : 0.f;
   }
 }
 
@@ -713,33 +756,28 @@ __global__ void __launch_bounds__(kLossThreads) loss_final_kernel(const float* _
 __global__ void __launch_bounds__(kLossThreads) loss_coeff_kernel(const int* __restrict__ targets,
                                                                   float* __restrict__ coeff, int L, int n, int N,
                                                                   float gamma) {
-  __shared__ int scnt[kLossThreads / 32];
-  __shared__ float cj[64];
-  const int i = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float wgt = 1.f;
-  for (int j = 0; j < n; ++j) {
-    int cnt = 0;
-    for (int t = threadIdx.x; t < L; t += kLossThreads) cnt += targets[(static_cast<size_t>(i) * L + t) * n + j] >= 0;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(kFull, cnt, off);
-    if (lane == 0) scnt[warp] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int c = 0;
-      for (int q = 0; q < kLossThreads / 32; ++q) c += scnt[q];
-      cj[j] = c > 0 ? -wgt / (static_cast<float>(N) * static_cast<float>(c)) : 0.f;
-    }
-    wgt *= gamma;
-    __syncthreads();
+  __shared__ int scnt[kLossThreads];
+  __shared__ float cj[65];
+  const int i = blockIdx.x, step = loss_rows_per_step(n), j = threadIdx.x % n;
+  int cnt = 0;
+  if (threadIdx.x < step * n)
+    for (int t = threadIdx.x / n; t < L; t += step) cnt += targets[(static_cast<size_t>(i) * L + t) * n + j] >= 0;
+  scnt[threadIdx.x] = cnt;
+  loss_add_rows(scnt, step, n);
+  if (threadIdx.x < n) {
+    float wgt = 1.f;
+    for (int q = 0; q < static_cast<int>(threadIdx.x); ++q) wgt *= gamma;
+    const int c = scnt[threadIdx.x];
+    cj[threadIdx.x] = c > 0 ? -wgt / (static_cast<float>(N) * static_cast<float>(c)) : 0.f;
   }
-  for (int t = threadIdx.x; t < L; t += kLossThreads) {
+  if (threadIdx.x == 0) cj[n] = 0.f;
+  __syncthreads();
+  if (threadIdx.x >= step * n) return;
+  for (int t = threadIdx.x / n; t < L; t += step) {
     const size_t row = (static_cast<size_t>(i) * L + t) * n;
-    for (int j = 0; j < n; ++j) {
-      const float here = targets[row + j] >= 0 ? cj[j] : 0.f;
-      const float next = (j + 1 < n && targets[row + j + 1] >= 0) ? cj[j + 1] : 0.f;
-      coeff[row + j] = here - next;
-    }
+    const float here = targets[row + j] >= 0 ? cj[j] : 0.f;
+    const float next = (j + 1 < n && targets[row + j + 1] >= 0) ? cj[j + 1] : 0.f;
+    coeff[row + j] = here - next;
   }
 }
 

@@ -280,6 +280,7 @@ struct mtpc_head {
   size_t lr_off_arep;                           // workspace: A as [n, v, r, k]
   size_t lr_off_dec;                            // workspace: few-position draft products base [P, n v] | z [P, n r k]
   size_t lr_off_base;                           // workspace: long drafts: W_base h [T, n v] fp32 (0: not reserved)
+  size_t lr_off_split;                          // workspace: parts of split plain GEMMs
   CUtensorMap tm_lrB_dec;                       // B [n r k, d] for the few-position draft path
   size_t lr_off_zhl, lr_off_partial;            // workspace: z = B h as bf16 halves [T, n r, 2, k]; per-panel partial log-sum-exps
   LowRankGemmParams lr_params;                  // everything of the factored projection launch that does not depend on the call
@@ -705,15 +706,20 @@ struct GemmOperand {
 
 // Optional extras of a plain GEMM launch: bf16 output instead of fp32, and several products of one shape in a launch
 // (see PlainGemmParams); a_* / b_* extents: the whole matrices the batched operands are windows of (M or N, then K).
+constexpr size_t kSplitBytes = kSplitParts * kSplitPartBytes;
+// C2, C3: rows [m1, m2) and [m2, M) of the fp32 result go there.
 struct PlainGemmExtra {
+  float *C2 = nullptr, *C3 = nullptr;
+  int m1 = 0, m2 = 0;
   void* C_bf16 = nullptr;
   int batches = 1, a_m_step = 0, a_k_step = 0, b_n_step = 0, b_k_step = 0;
   size_t c_step = 0;
   long long a_extent_m = 0, a_extent_k = 0, b_extent_n = 0, b_extent_k = 0;
 };
+// split_ws: kSplitBytes of scratch that let the launch cut its last round along K (NULL: it does not).
 int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmOperand B1, int K1, int a_k1, float* C,
-                      size_t ldc, int M, int N, cudaStream_t st, void* C_hilo = nullptr, int split_k = 0,
-                      const PlainGemmExtra* extra = nullptr);
+                      size_t ldc, int M, int N, cudaStream_t st, void* split_ws = nullptr, void* C_hilo = nullptr,
+                      int split_k = 0, const PlainGemmExtra* extra = nullptr);
 // parts: 1 = sum-unit tiles (log omega), 2 = z = B h and the repacked A, 4 = the factored kernel (and its merge)
 int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, const int* targets, cudaStream_t st,
                               const GradArgs* ga = nullptr, int parts = 7, bool targets_are_drafts = false);
@@ -770,7 +776,7 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     rc = launch_plain_gemm(h, GemmOperand{hidden, static_cast<size_t>(c.d), false},
                            GemmOperand{h->lr_W_base, static_cast<size_t>(c.d), false}, c.d,
                            GemmOperand{h->lr_W_base, static_cast<size_t>(c.d), false}, 0, 0, base,
-                           static_cast<size_t>(c.n) * c.v, P, c.n * c.v, st);
+                           static_cast<size_t>(c.n) * c.v, P, c.n * c.v, st, h->ws + h->lr_off_split);
     if (rc != MTPC_OK) return rc;
     {
       const int pairs = W * c.n;
@@ -945,7 +951,7 @@ size_t round64(size_t x) { return (x + 63) / 64 * 64; }
 // The sum-unit logit gradients sit to the right of the emission logit gradients in one matrix [T, Kd], Kd = Nc + Spad.
 struct BackwardLayout {
   size_t Nc, Spad, Kd;
-  size_t off_lse, off_post, off_logits, off_dlogit, off_coeff, total;
+  size_t off_lse, off_post, off_logits, off_dlogit, off_coeff, off_split, total;
 };
 void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout* B) {
   B->Nc = static_cast<size_t>(c.n) * c.r * c.v;
@@ -958,46 +964,117 @@ void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout*
   B->off_logits = take(static_cast<size_t>(T) * B->Nc * 4);              // [T, Nc] fp32: the emission logits of the forward pass
   B->off_dlogit = take(static_cast<size_t>(T) * B->Kd * 2);          // [T, Nc | Spad] bf16
   B->off_coeff = take(static_cast<size_t>(T) * c.n * 4);             // Eq. 6: weights of the prefix marginals
+  B->off_split = take(kSplitBytes);                                 // parts of the GEMMs' cut tiles
   B->total = off;
+}
+
+// How a plain GEMM of `tiles` tiles and `kblocks` K blocks is dealt to `workers` (CTAs, or pairs: ctas = 2): the tiles of the
+// last, partial round are cut into `split` parts each. Cost in K-block times of a worker (0.4 us): a part adds about 8 for
+// writing its fp32 tile, the reduction 10 and its bytes through L2 (15 tile parts of 128 KB a block time). Cut only where that
+// wins clearly.
+struct SplitPlan {
+  int tail = 0, split = 1;
+  long long cost = 0;
+};
+SplitPlan plan_split(long long tiles, int kblocks, int workers, int ctas, bool scratch) {
+  SplitPlan b;
+  const long long whole = tiles / workers;
+  const int rem = static_cast<int>(tiles % workers);
+  b.cost = whole * kblocks + (rem ? kblocks : 0);
+  if (rem == 0 || !scratch) return b;
+  const long long limit = b.cost - 8;
+  for (int s = 2; s <= 16 && rem * s * ctas <= kSplitParts && kblocks / s >= 4; ++s) {
+    const long long rounds = (static_cast<long long>(rem) * s + workers - 1) / workers;
+    const long long cost = whole * kblocks + rounds * ((kblocks + s - 1) / s + 8) + 10 + rem * s * ctas / 15;
+    if (cost < b.cost && cost < limit) { b.cost = cost; b.tail = rem; b.split = s; }
+  }
+  return b;
+}
+
+template <int CTAS>
+void launch_plain_tiles(const PlainGemmParams& p, bool a_mn, bool b_mn, int grid, size_t smem, cudaStream_t st) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CTAS == 2 ? 1 : 0;
+  if (a_mn) cudaLaunchKernelEx(&cfg, plain_gemm_kernel<true, true, kPlainTileN, CTAS>, p);
+  else if (b_mn) cudaLaunchKernelEx(&cfg, plain_gemm_kernel<false, true, kPlainTileN, CTAS>, p);
+  else cudaLaunchKernelEx(&cfg, plain_gemm_kernel<false, false, kPlainTileN, CTAS>, p);
 }
 
 // C[M, N] fp32 (pitch ldc) = A B^T over K = K0 + K1: segment 0 multiplies A's K range [0, K0) with B0, segment 1 (K1 > 0)
 // A's K range [a_k1, a_k1 + K1) with B1.
 // C_hilo != NULL (then C is NULL): the result leaves as two bf16 halves per entry, see PlainGemmParams.
 int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmOperand B1, int K1, int a_k1, float* C,
-                      size_t ldc, int M, int N, cudaStream_t st, void* C_hilo, int split_k, const PlainGemmExtra* extra) {
+                      size_t ldc, int M, int N, cudaStream_t st, void* split_ws, void* C_hilo, int split_k,
+                      const PlainGemmExtra* extra) {
   if (M <= 0 || N <= 0 || K0 <= 0) return MTPC_OK;
   if (K1 > 0 && (A.mn_major || B1.mn_major != B0.mn_major)) return MTPC_ERR_SHAPE;
+  if (A.mn_major && !B0.mn_major) return MTPC_ERR_SHAPE;
   const PlainGemmExtra none;
   const PlainGemmExtra& x = extra ? *extra : none;
   if (x.batches < 1 || (x.batches > 1 && K1 > 0)) return MTPC_ERR_SHAPE;
   PlainGemmParams p;
   memset(&p, 0, sizeof(p));
-  const int Ka = K1 > 0 ? a_k1 + K1 : K0;                      // extent of A along K
-  const uint64_t a_m = x.a_extent_m ? x.a_extent_m : M, a_k = x.a_extent_k ? x.a_extent_k : Ka;
-  const uint64_t b_n = x.b_extent_n ? x.b_extent_n : N, b_k = x.b_extent_k ? x.b_extent_k : K0;
-  int rc = A.mn_major ? make_tmap_mn(&p.tm_a, A.ptr, a_k, a_m, A.pitch) : make_tmap(&p.tm_a, A.ptr, a_m, a_k, kBlockM, A.pitch);
-  if (rc == MTPC_OK)
-    rc = B0.mn_major ? make_tmap_mn(&p.tm_b[0], B0.ptr, b_k, b_n, B0.pitch) : make_tmap(&p.tm_b[0], B0.ptr, b_n, b_k, kPlainTileN, B0.pitch);
-  if (rc == MTPC_OK && K1 > 0)
-    rc = B1.mn_major ? make_tmap_mn(&p.tm_b[1], B1.ptr, K1, N, B1.pitch) : make_tmap(&p.tm_b[1], B1.ptr, N, K1, kPlainTileN, B1.pitch);
-  if (rc != MTPC_OK) return rc;
   p.M = M; p.N = N;
   p.a_k0[0] = 0;
   p.a_k0[1] = a_k1;
   p.seg_kblocks[0] = (K0 + kBlockK - 1) / kBlockK;
   p.seg_kblocks[1] = K1 > 0 ? (K1 + kBlockK - 1) / kBlockK : 0;
-  p.m_tiles = (M + kBlockM - 1) / kBlockM;
+  const int kblocks = p.seg_kblocks[0] + p.seg_kblocks[1];
   // batched products with a rank for N: 64-column accumulator tiles
   const int tile_n = (x.batches > 1 && N <= 64 && B0.mn_major) ? 64 : kPlainTileN;
   p.n_tiles = (N + tile_n - 1) / tile_n;
-  p.stage_bytes = kABytes + tile_n * kBlockK * 2;
+  const int m_tiles = (M + kBlockM - 1) / kBlockM;
+  // Single CTAs or pairs: whichever needs fewer K-block times (a pair's 256 x 256 tile takes its two SMs as long as a single
+  // CTA's 128 x 256 tile takes one), a pair counted 1/16 cheaper: it moves a third less operand data (dW_sum of 14368 rows:
+  // 280 us in pairs, 312 us alone). Within one round it is the call's latency that counts, and a lone CTA's is shorter
+  // (48 tiles of K = 2048: 18.9 us alone, 21.2 us in pairs).
+  SplitPlan plan;
+  bool pair = false;
+  if (tile_n == kPlainTileN && x.batches == 1) {
+    plan = plan_split(static_cast<long long>(m_tiles) * p.n_tiles, kblocks, h->num_sms, 1, split_ws != nullptr);
+    if (h->max_pairs > 0 && m_tiles >= 2 && static_cast<long long>(m_tiles) * p.n_tiles > h->num_sms) {
+      const SplitPlan two = plan_split(static_cast<long long>((m_tiles + 1) / 2) * p.n_tiles, kblocks, h->max_pairs, 2, split_ws != nullptr);
+      if (two.cost * 15 <= plan.cost * 16) { plan = two; pair = true; }
+    }
+  }
+  const int ctas = pair ? 2 : 1;
+  p.m_tiles = (m_tiles + ctas - 1) / ctas;
+  p.tail_tiles = plan.tail;
+  p.split = plan.split;
+  p.partial = static_cast<float*>(split_ws);
+  const int Ka = K1 > 0 ? a_k1 + K1 : K0;                      // extent of A along K
+  const uint64_t a_m = x.a_extent_m ? x.a_extent_m : M, a_k = x.a_extent_k ? x.a_extent_k : Ka;
+  const uint64_t b_n = x.b_extent_n ? x.b_extent_n : N, b_k = x.b_extent_k ? x.b_extent_k : K0;
+  const int b_box = kPlainTileN / ctas;
+  int rc = A.mn_major ? make_tmap_mn(&p.tm_a, A.ptr, a_k, a_m, A.pitch) : make_tmap(&p.tm_a, A.ptr, a_m, a_k, kBlockM, A.pitch);
+  if (rc == MTPC_OK)
+    rc = B0.mn_major ? make_tmap_mn(&p.tm_b[0], B0.ptr, b_k, b_n, B0.pitch) : make_tmap(&p.tm_b[0], B0.ptr, b_n, b_k, b_box, B0.pitch);
+  if (rc == MTPC_OK && K1 > 0)
+    rc = B1.mn_major ? make_tmap_mn(&p.tm_b[1], B1.ptr, K1, N, B1.pitch) : make_tmap(&p.tm_b[1], B1.ptr, N, K1, b_box, B1.pitch);
+  if (rc != MTPC_OK) return rc;
+  p.stage_bytes = kABytes + tile_n / ctas * kBlockK * 2;
   const int ctl = 1024 + static_cast<int>(sizeof(GemmControl));
   p.stages = (kSmemLimit - ctl) / p.stage_bytes;
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   p.wide_stores = (reinterpret_cast<uintptr_t>(C) % 32 == 0 && ldc % 8 == 0 && x.c_step % 8 == 0) ? 1 : 0;
   p.C = C;
   p.ldc = ldc;
+  p.C2 = x.C2;
+  p.C3 = x.C3;
+  p.m_end[0] = x.C2 ? x.m1 : M;
+  p.m_end[1] = x.C3 ? x.m2 : M;
+  if (reinterpret_cast<uintptr_t>(x.C2) % 32 != 0 || reinterpret_cast<uintptr_t>(x.C3) % 32 != 0) p.wide_stores = 0;
   p.C_hilo = static_cast<__nv_bfloat16*>(C_hilo);
   p.split_k = split_k;
   p.C_bf16 = static_cast<__nv_bfloat16*>(x.C_bf16);
@@ -1010,16 +1087,19 @@ int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmO
   p.c_step = x.c_step;
   p.status = at<unsigned>(h, h->L.off_status);
   p.wait_limit_ns = h->wait_limit_ns;
-  const long long items = static_cast<long long>(p.m_tiles) * p.n_tiles * p.batches;
-  const int grid = static_cast<int>(items < h->num_sms ? items : h->num_sms);
+  const long long items = static_cast<long long>(p.m_tiles) * p.n_tiles * p.batches + static_cast<long long>(p.tail_tiles) * (p.split - 1);
+  const int workers = pair ? h->max_pairs : h->num_sms;
+  const int grid = ctas * static_cast<int>(items < workers ? items : workers);
   const size_t smem = p.stages * p.stage_bytes + ctl;
   if (tile_n == 64 && A.mn_major) plain_gemm_kernel<true, true, 64><<<grid, kGemmThreads, smem, st>>>(p);
   else if (tile_n == 64) plain_gemm_kernel<false, true, 64><<<grid, kGemmThreads, smem, st>>>(p);
-  else if (A.mn_major && B0.mn_major) plain_gemm_kernel<true, true><<<grid, kGemmThreads, smem, st>>>(p);
-  else if (!A.mn_major && B0.mn_major) plain_gemm_kernel<false, true><<<grid, kGemmThreads, smem, st>>>(p);
-  else if (!A.mn_major && !B0.mn_major) plain_gemm_kernel<false, false><<<grid, kGemmThreads, smem, st>>>(p);
-  else return MTPC_ERR_SHAPE;
+  else if (pair) launch_plain_tiles<2>(p, A.mn_major, B0.mn_major, grid, smem, st);
+  else launch_plain_tiles<1>(p, A.mn_major, B0.mn_major, grid, smem, st);
   h->launches++;
+  if (p.tail_tiles > 0) {
+    launch_kernel(split_reduce_kernel, p.tail_tiles * ctas * 8, 256, 0, st, /*dependent=*/true, p, ctas);
+    h->launches++;
+  }
   return check_launch();
 }
 
@@ -1084,16 +1164,17 @@ int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, cons
   if (rc != MTPC_OK) return rc;
   __nv_bfloat16* zhl = reinterpret_cast<__nv_bfloat16*>(h->ws + h->lr_off_zhl);
   if (parts & 2) {
-    const GemmOperand hid{hidden_bf16, static_cast<size_t>(c.d), false};
-    const GemmOperand bmat{h->lr_B, static_cast<size_t>(c.d), false};          // [n r k, d], K = d contiguous
-    // z = B h, leaving the GEMM's epilogue already split into its two bf16 halves [T, n r, 2, k]
-    rc = launch_plain_gemm(h, hid, bmat, c.d, bmat, 0, 0, nullptr, 0, T, units * k, st, zhl, k);
-    if (rc != MTPC_OK) return rc;
     // A as [n, v, r, k]: the adaptor columns of adjacent components side by side (remade every call: A may have changed)
     const size_t pieces = static_cast<size_t>(units) * c.v * (k / 8);
     lowrank_repack_kernel<<<static_cast<unsigned>((pieces + 255) / 256), 256, 0, st>>>(
         static_cast<const uint4*>(h->lr_A), reinterpret_cast<uint4*>(h->ws + h->lr_off_arep), c.n, c.r, c.v, k / 8);
     h->launches += 1;
+    // z = B h, leaving the GEMM's epilogue already split into its two bf16 halves [T, n r, 2, k]
+    const GemmOperand hid{hidden_bf16, static_cast<size_t>(c.d), false};
+    const GemmOperand bmat{h->lr_B, static_cast<size_t>(c.d), false};          // [n r k, d], K = d contiguous
+    rc = launch_plain_gemm(h, hid, bmat, c.d, bmat, 0, 0, nullptr, 0, T, units * k, st, h->ws + h->lr_off_split,
+                           zhl, k);
+    if (rc != MTPC_OK) return rc;
   }
   if (!(parts & 4)) return check_launch();
   LowRankGemmParams p = h->lr_params;
@@ -1204,7 +1285,6 @@ int backward_tail(mtpc_head* head, const BackwardLayout& B, uint8_t* bw, const v
   const mtpc_config& c = head->cfg;
   const Layout& L = head->L;
   __nv_bfloat16* dlogit = reinterpret_cast<__nv_bfloat16*>(bw + B.off_dlogit);
-  __nv_bfloat16* dsum = dlogit + B.Nc;
   const int Nc = static_cast<int>(B.Nc);
   pt.begin();
   LogitGradArgs la;
@@ -1229,15 +1309,18 @@ int backward_tail(mtpc_head* head, const BackwardLayout& B, uint8_t* bw, const v
   pt.begin();
   const GemmOperand g_rows{dlogit, B.Kd, false};            // [T, Nc | S r] along its rows: K = the logit index
   const GemmOperand g_cols{dlogit, B.Kd, true};             // the same matrix down its columns: K = the position
-  const GemmOperand s_cols{dsum, B.Kd, true};
   const GemmOperand w_emit{head->W_emit_bf16, static_cast<size_t>(c.d), true};   // [Nc, d]: N = d contiguous
   const GemmOperand w_sum{head->W_sum_bf16, static_cast<size_t>(c.d), true};
   const GemmOperand hid{hb, static_cast<size_t>(c.d), true};                     // [T, d]: N = d contiguous, K = the position
   // d hidden [T, d] = dlogit [T, Nc] W_emit [Nc, d] + dsum [T, S r] W_sum [S r, d]
-  rc = launch_plain_gemm(head, g_rows, w_emit, Nc, w_sum, L.sum_rows, Nc, d_hidden, c.d, T, c.d, st);
-  // dW_emit [Nc, d] = dlogit^T [Nc, T] hidden [T, d];  dW_sum [S r, d] = dsum^T [S r, T] hidden [T, d]
-  if (rc == MTPC_OK) rc = launch_plain_gemm(head, g_cols, hid, T, hid, 0, 0, dW_emit, c.d, Nc, c.d, st);
-  if (rc == MTPC_OK) rc = launch_plain_gemm(head, s_cols, hid, T, hid, 0, 0, dW_sum, c.d, L.sum_rows, c.d, st);
+  rc = launch_plain_gemm(head, g_rows, w_emit, Nc, w_sum, L.sum_rows, Nc, d_hidden, c.d, T, c.d, st,
+                         bw + B.off_split);
+  // [dW_emit; dW_sum] [Nc + S r, d] = [dlogit | dsum]^T hidden [T, d]
+  PlainGemmExtra two;
+  two.C2 = dW_sum;
+  two.m1 = Nc;
+  if (rc == MTPC_OK)
+    rc = launch_plain_gemm(head, g_cols, hid, T, hid, 0, 0, dW_emit, c.d, Nc + L.sum_rows, c.d, st, bw + B.off_split, nullptr, 0, &two);
   pt.end();
   return rc;
 }
@@ -1325,21 +1408,22 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
     x.a_extent_m = T; x.a_extent_k = Nc;
     x.b_extent_n = k; x.b_extent_k = static_cast<long long>(units) * R.v64;
     rc = launch_plain_gemm(head, GemmOperand{dlogit, B.Kd, false}, GemmOperand{bw + R.off_apad, static_cast<size_t>(k), true},
-                           static_cast<int>(R.v64), none, 0, 0, nullptr, R.pitch, T, k, st, nullptr, 0, &x);
+                           static_cast<int>(R.v64), none, 0, 0, nullptr, R.pitch, T, k, st, nullptr, nullptr, 0, &x);
   }
   // d hidden [T, d] = [s | y] [W_base ; B] + dsum W_sum
   if (rc == MTPC_OK)
     rc = launch_plain_gemm(head, GemmOperand{sy, R.pitch, false}, GemmOperand{wcat, static_cast<size_t>(c.d), true},
                            static_cast<int>(R.Ksy), GemmOperand{head->W_sum_bf16, static_cast<size_t>(c.d), true}, L.sum_rows,
-                           static_cast<int>(R.Ksy), d_hidden, c.d, T, c.d, st);
-  // dW_base = s^T h, dB = y^T h, dW_sum = dsum^T h: sy down its columns
+                           static_cast<int>(R.Ksy), d_hidden, c.d, T, c.d, st, bw + B.off_split);
+  // [dW_base; dB; dW_sum] = [s | y | dsum]^T h: sy down its columns
+  PlainGemmExtra three;
+  three.C2 = dB;
+  three.m1 = c.n * c.v;
+  three.C3 = dW_sum;
+  three.m2 = static_cast<int>(R.Ksy);
   if (rc == MTPC_OK)
-    rc = launch_plain_gemm(head, GemmOperand{sy, R.pitch, true}, hid, T, hid, 0, 0, dW_base, c.d, c.n * c.v, c.d, st);
-  if (rc == MTPC_OK)
-    rc = launch_plain_gemm(head, GemmOperand{sy + static_cast<size_t>(c.n) * c.v, R.pitch, true}, hid, T, hid, 0, 0, dB, c.d,
-                           units * k, c.d, st);
-  if (rc == MTPC_OK)
-    rc = launch_plain_gemm(head, GemmOperand{sy + R.Ksy, R.pitch, true}, hid, T, hid, 0, 0, dW_sum, c.d, L.sum_rows, c.d, st);
+    rc = launch_plain_gemm(head, GemmOperand{sy, R.pitch, true}, hid, T, hid, 0, 0, dW_base, c.d, static_cast<int>(R.Ksy) + L.sum_rows,
+                           c.d, st, bw + B.off_split, nullptr, 0, &three);
   if (rc == MTPC_OK) {   // dA_ij [v, k] = g_ij^T z_ij, one product per unit, on the bf16 high half of z the forward pass left
     PlainGemmExtra x;
     x.batches = units;
@@ -1350,7 +1434,7 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
     x.b_extent_n = static_cast<long long>(units) * 2 * k; x.b_extent_k = T;
     rc = launch_plain_gemm(head, GemmOperand{dlogit, B.Kd, true},
                            GemmOperand{head->ws + head->lr_off_zhl, static_cast<size_t>(units) * 2 * k, true}, T, none, 0, 0, dA,
-                           k, c.v, k, st, nullptr, 0, &x);
+                           k, c.v, k, st, nullptr, nullptr, 0, &x);
   }
   pt.end();
   return rc;
@@ -1450,7 +1534,7 @@ struct LowRankSpec {
 // that computes it), where a unit is cut into panels the panels' (maximum, sum) pairs and the targets' logits, and the
 // copy of A the factored kernel reads.
 static int lowrank_extra_bytes(const mtpc_config& c, int k, int panels, size_t base_total, size_t* off_zhl,
-                               size_t* off_partial, size_t* off_arep, size_t* off_dec, size_t* off_base, size_t* total) {
+                               size_t* off_partial, size_t* off_arep, size_t* off_dec, size_t* off_base, size_t* off_split, size_t* total) {
   const size_t units = static_cast<size_t>(c.n) * c.r;
   size_t off = align_up(base_total);
   *off_zhl = off;
@@ -1467,6 +1551,8 @@ static int lowrank_extra_bytes(const mtpc_config& c, int k, int panels, size_t b
     *off_base = off;
     off += align_up(static_cast<size_t>(c.max_positions) * c.n * c.v * 4);
   }
+  *off_split = off;                     // z = B h and W_base h: parts of the tiles of their last rounds
+  off += align_up(kSplitBytes);
   *total = off;
   return MTPC_OK;
 }
@@ -1482,11 +1568,12 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   if (rc != MTPC_OK) return rc;
   LowRankGemmParams lrp;
   memset(&lrp, 0, sizeof(lrp));
-  size_t lr_zhl = 0, lr_partial = 0, lr_arep = 0, lr_dec = 0, lr_base = 0;
+  size_t lr_zhl = 0, lr_partial = 0, lr_arep = 0, lr_dec = 0, lr_base = 0, lr_split = 0;
   if (lowrank) {
     if (cfg->io_dtype != MTPC_BF16) return MTPC_ERR_UNSUPPORTED;
     if (!plan_lowrank(*cfg, lowrank->k, &lrp)) return MTPC_ERR_UNSUPPORTED;
-    lowrank_extra_bytes(*cfg, lowrank->k, lrp.panels, L.total, &lr_zhl, &lr_partial, &lr_arep, &lr_dec, &lr_base, &L.total);
+    lowrank_extra_bytes(*cfg, lowrank->k, lrp.panels, L.total, &lr_zhl, &lr_partial, &lr_arep, &lr_dec, &lr_base,
+                        &lr_split, &L.total);
   }
   const bool ctx = (cfg->flags & MTPC_FLAG_HMM_CONTEXTUAL) != 0;
   if (cfg->family == MTPC_HMM && cfg->n > 1 && !ctx && !T_static) return MTPC_ERR_NULL;
@@ -1512,6 +1599,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
     h->lr_off_arep = lr_arep;
     h->lr_off_dec = lr_dec;
     h->lr_off_base = lr_base;
+    h->lr_off_split = lr_split;
     h->lr_params = lrp;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1529,6 +1617,9 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   fail |= !allow_full_smem(plain_gemm_kernel<false, false>);
   fail |= !allow_full_smem(plain_gemm_kernel<false, true>);
   fail |= !allow_full_smem(plain_gemm_kernel<true, true>);
+  fail |= !allow_full_smem(plain_gemm_kernel<false, false, kPlainTileN, 2>);
+  fail |= !allow_full_smem(plain_gemm_kernel<false, true, kPlainTileN, 2>);
+  fail |= !allow_full_smem(plain_gemm_kernel<true, true, kPlainTileN, 2>);
   fail |= !allow_full_smem(plain_gemm_kernel<true, true, 64>);
   fail |= !allow_full_smem(plain_gemm_kernel<false, true, 64>);
   fail |= cudaFuncSetAttribute(mtpc_decode_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) !=
@@ -1572,8 +1663,8 @@ int mtpc_lowrank_workspace_bytes(const mtpc_config* cfg, int32_t k, size_t* out_
   if (rc != MTPC_OK) return rc;
   LowRankGemmParams lrp;
   if (cfg->io_dtype != MTPC_BF16 || !plan_lowrank(*cfg, k, &lrp)) return MTPC_ERR_UNSUPPORTED;
-  size_t a = 0, b = 0, c3 = 0, c4 = 0, c5 = 0;
-  return lowrank_extra_bytes(*cfg, k, lrp.panels, L.total, &a, &b, &c3, &c4, &c5, out_bytes);
+  size_t a = 0, b = 0, c3 = 0, c4 = 0, c5 = 0, c6 = 0;
+  return lowrank_extra_bytes(*cfg, k, lrp.panels, L.total, &a, &b, &c3, &c4, &c5, &c6, out_bytes);
 }
 
 int mtpc_create_head_lowrank(const mtpc_config* cfg, int32_t k, const void* W_base, const void* A, const void* B,

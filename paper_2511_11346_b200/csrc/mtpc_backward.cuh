@@ -757,23 +757,36 @@ __global__ void __launch_bounds__(256) logit_gradient_kernel(const LogitGradArgs
 
 // ---------------------------------------------------------------- plain bf16 GEMM on the tcgen05 tensor cores
 // C[M, N] (fp32, row-major, pitch ldc) = A[M, K] B[N, K]^T with bf16 operands read where they lie, in either
-// orientation: K-major (K contiguous in memory: 64-element K boxes of 128 or 256 rows) or MN-major (the M / N index
-// contiguous: 64 x 64 boxes, two for the 128 rows of A, four for the 256 columns of B). Out-of-range rows and
+// orientation: K-major (K contiguous in memory: 64-element K boxes of up to 256 rows) or MN-major (the M / N index
+// contiguous: 64 x 64 boxes, two for the 128 rows of A, up to four for the columns of B). Out-of-range rows and
 // columns read as zero. The K axis may consist of two segments with a B matrix each (d hidden sums over the emission
 // rows and the sum-unit rows, which are separate matrices); A then continues at column a_k0[1]. Same pipeline as the
-// projection kernel: one persistent CTA per SM, warp 0 TMA producer, warp 1 MMA issuer (M=128, N=256 tiles, two TMEM
-// slots), warps 2..5 epilogue (one thread per row, 16 fp32 columns per step).
+// projection kernel: one persistent CTA per SM, warp 0 TMA producer, warp 1 MMA issuer (two TMEM slots), warps 2..5 epilogue
+// (one thread per row, 16 fp32 columns per step). CTAS = 1: a CTA works alone (M = 128, N = TN). CTAS = 2: a cluster of two
+// shares every MMA (cta_group::2, M = 256), each CTA staging its own 128 rows of A and half of the columns of B, so a third
+// less data moves from L2 to shared memory per multiply-add; barriers as in the projection kernel.
+// Split of the last round: tiles are dealt to the workers (CTAs or pairs) round by round, and the `tail_tiles` that do not
+// fill a round are cut along K into `split` parts each, dealt part by part (workers that run together then walk the same K
+// range of different tiles and share its operands through L2). The parts are written as fp32 tiles and split_reduce_kernel adds
+// them up in K order, spread over the whole device. (Added up by the warp that arrives last, a few warps read every part alone:
+// 12 tiles in 8 parts took 29 us where the uncut launch takes 19.) It matters where a contraction has few tiles: d hidden of
+// 2005 positions is 96 pair tiles for 74 pairs (415 -> 271 us), of 4096 positions 192 (2945 -> 2480 us, of which the pairs
+// give about 5 %).
 struct PlainGemmParams {
   CUtensorMap tm_a;      // K-major: A [M, K], box 64 (k) x 128; MN-major: A^T [K, M], box 64 (m) x 64 (k)
-  CUtensorMap tm_b[2];   // per K segment. K-major: B [N, K], box 64 (k) x 256; MN-major: B^T [K, N], box 64 (n) x 64 (k)
+  CUtensorMap tm_b[2];   // per K segment. K-major: B [N, K], box 64 (k) x TN / CTAS; MN-major: B^T [K, N], box 64 (n) x 64 (k)
   int a_k0[2];           // K coordinate of A at which each segment starts (multiples of 8)
   int seg_kblocks[2];    // 64-wide K blocks per segment (segment 1: 0 if unused)
   int M, N;
-  int m_tiles, n_tiles;
+  int m_tiles, n_tiles;  // m_tiles: tiles of CTAS * 128 rows
   int stages, stage_bytes;
   int wide_stores;       // C and ldc allow 32-byte stores
   float* C;
   size_t ldc;
+  // The rows from m_end[0] on go to C2, those from m_end[1] on to C3 (same pitch): the weight gradients of several matrices
+  // whose logit gradients lie side by side are one launch, instead of small launches that each end in a partial round.
+  float *C2, *C3;
+  int m_end[2];
   // Instead of C (C == NULL): the result split into two bf16 halves, x = hi + lo, written as [M, N / split_k, 2, split_k]
   // (group g of split_k columns: hi at column (2 g) split_k, lo at (2 g + 1) split_k; split_k a multiple of 16).
   __nv_bfloat16* C_hilo;
@@ -787,15 +800,90 @@ struct PlainGemmParams {
   // zeros past the product's own extent (the caller pads one of them).
   int batches, a_m_step, a_k_step, b_n_step, b_k_step;
   size_t c_step;
+  int tail_tiles, split;      // the last tail_tiles tiles are cut into `split` parts (1: not cut)
+  float* partial;             // [tail_tiles][split][CTAS][4 warps] runs of 32 x TN floats, lane-fastest
   unsigned* status;
   uint64_t wait_limit_ns;   // limit of every pipeline wait
 };
 constexpr int kPlainTileN = 256;
 constexpr uint32_t kMnBoxBytes = 64 * kBlockK * 2;   // one 64 x 64 bf16 box: 8 KB
+// Scratch of a split launch: parts of at most kSplitParts 128 x 256 tiles (three rounds of a 148-SM device).
+constexpr int kSplitParts = 444;
+constexpr size_t kSplitPartBytes = static_cast<size_t>(kBlockM) * kPlainTileN * sizeof(float);
+
+// Work item `item` of a launch: the tile and the K blocks [kb0, kb1) of it; tail >= 0: index of the cut tile, part its part.
+struct PlainItem {
+  int bt, mt, nt, kb0, kb1, tail, part;
+};
+__device__ __forceinline__ PlainItem plain_item(const PlainGemmParams& p, int item, int kblocks) {
+  PlainItem w;
+  const int per_batch = p.m_tiles * p.n_tiles;
+  const int whole = per_batch * p.batches - p.tail_tiles;
+  int tile = item;
+  w.tail = -1;
+  w.part = 0;
+  w.kb0 = 0;
+  w.kb1 = kblocks;
+  if (item >= whole) {
+    const int q = item - whole;
+    w.part = q / p.tail_tiles;
+    w.tail = q - w.part * p.tail_tiles;
+    tile = whole + w.tail;
+    w.kb0 = static_cast<int>(static_cast<long long>(w.part) * kblocks / p.split);
+    w.kb1 = static_cast<int>(static_cast<long long>(w.part + 1) * kblocks / p.split);
+  }
+  // n-tile fastest: the CTAs running together cover a few m-tiles x all n-tiles, so the (larger) A operand is
+  // streamed from HBM once and the B operand once per wave of m-tiles
+  w.bt = tile / per_batch;
+  const int rest = tile - w.bt * per_batch;
+  w.nt = rest % p.n_tiles;
+  w.mt = rest / p.n_tiles;
+  return w;
+}
+
+// First element of a row of the fp32 result (row < M).
+__device__ __forceinline__ float* plain_row(const PlainGemmParams& p, int row) {
+  if (row < p.m_end[0]) return p.C + static_cast<size_t>(row) * p.ldc;
+  if (row < p.m_end[1]) return p.C2 + static_cast<size_t>(row - p.m_end[0]) * p.ldc;
+  return p.C3 + static_cast<size_t>(row - p.m_end[1]) * p.ldc;
+}
+// Sixteen adjacent columns of one row of the result, in whichever form it is wanted. crow: where the row starts in C;
+// coff: its offset in C_bf16.
+__device__ __forceinline__ void plain_store16(const PlainGemmParams& p, const float (&x)[16], int row, float* crow, size_t coff, int col0) {
+  if (p.C == nullptr && p.C_hilo == nullptr) {
+    __align__(16) __nv_bfloat16 o[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) o[q] = __float2bfloat16_rn(x[q]);
+    uint4* dst = reinterpret_cast<uint4*>(p.C_bf16 + coff + col0);      // ldc, c_step and C_bf16 keep 16 columns 32-byte aligned
+    dst[0] = reinterpret_cast<const uint4*>(o)[0];
+    dst[1] = reinterpret_cast<const uint4*>(o)[1];
+  } else if (p.C == nullptr) {
+    // 16 columns of one group: 32 bytes of high halves and 32 bytes of low halves
+    const int grp = col0 / p.split_k, q0 = col0 - grp * p.split_k;
+    __align__(16) __nv_bfloat16 hi[16], lo[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      hi[q] = __float2bfloat16_rn(x[q]);
+      lo[q] = __float2bfloat16_rn(x[q] - __bfloat162float(hi[q]));
+    }
+    __nv_bfloat16* dst = p.C_hilo + static_cast<size_t>(row) * (2 * p.N) + static_cast<size_t>(2 * grp) * p.split_k + q0;
+    reinterpret_cast<uint4*>(dst)[0] = reinterpret_cast<const uint4*>(hi)[0];
+    reinterpret_cast<uint4*>(dst)[1] = reinterpret_cast<const uint4*>(hi)[1];
+    reinterpret_cast<uint4*>(dst + p.split_k)[0] = reinterpret_cast<const uint4*>(lo)[0];
+    reinterpret_cast<uint4*>(dst + p.split_k)[1] = reinterpret_cast<const uint4*>(lo)[1];
+  } else if (p.wide_stores) {                    // 32-byte aligned rows: one full sector per store
+    st_global_v8(crow + col0, x);
+    st_global_v8(crow + col0 + 8, x + 8);
+  } else {
+    float4* c4 = reinterpret_cast<float4*>(crow + col0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c4[q] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+  }
+}
 
 // TN: columns of an accumulator tile: 256, or 64 for the batched products whose N is a rank (MN-major B only: the boxes
 // of the tensor map are 64 wide) - what is fetched, multiplied and read back for columns that do not exist is a quarter.
-template <bool A_MN, bool B_MN, int TN = 256>
+template <bool A_MN, bool B_MN, int TN = 256, int CTAS = 1>
 __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __grid_constant__ PlainGemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
@@ -804,13 +892,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
   GemmControl* ctl = reinterpret_cast<GemmControl*>(tiles + static_cast<size_t>(p.stages) * p.stage_bytes);
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  // n-tile fastest: the CTAs running together cover a few m-tiles x all n-tiles, so the (larger) A operand is
-  // streamed from HBM once and the B operand once per wave of m-tiles
-  const int per_batch = p.m_tiles * p.n_tiles;
-  const int num_items = per_batch * p.batches;
   const int kblocks = p.seg_kblocks[0] + p.seg_kblocks[1];
+  const int num_items = p.m_tiles * p.n_tiles * p.batches + p.tail_tiles * (p.split - 1);
+  const uint32_t cta_rank = CTAS == 2 ? cluster_cta_rank() : 0u;      // 0 = the pair's leader
+  const int first_item = CTAS == 2 ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
+  const int item_step = CTAS == 2 ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
   constexpr uint32_t kSlots = 2;
-  constexpr uint32_t kBBytes = TN * kBlockK * 2;
+  constexpr int kBCols = TN / CTAS;                                   // columns of B this CTA stages
+  constexpr uint32_t kBBytes = kBCols * kBlockK * 2;
+  static_assert(CTAS == 1 || TN == kPlainTileN, "pairs share 256-column tiles");
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -819,7 +909,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
     }
     for (uint32_t s = 0; s < kSlots; ++s) {
       mbar_init(smem_u32(&ctl->tfull[s]), 1);
-      mbar_init(smem_u32(&ctl->tempty[s]), 4);
+      mbar_init(smem_u32(&ctl->tempty[s]), 4 * CTAS);
     }
     mbar_init(smem_u32(&ctl->drain), 1);
     ctl->abort = 0;
@@ -830,43 +920,53 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
     if (p.seg_kblocks[1] > 0) tma_prefetch_desc(&p.tm_b[1]);
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
-    tmem_relinquish();
+    if (CTAS == 2) {
+      tmem_alloc_pair(smem_u32(&ctl->tmem_base), kTmemCols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if (CTAS == 2) cluster_sync_all();   // the peer's barriers are initialised before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
+  grid_launch_dependents();            // split_reduce_kernel's CTAs may be scheduled as SMs free up
 
   if (warp == 0) {
     if (lane == 0) {
       uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-        const int bt = item / per_batch, rest = item - bt * per_batch;
-        const int nt = rest % p.n_tiles, mt = rest / p.n_tiles;
-        const int am = mt * kBlockM + bt * p.a_m_step, ak = bt * p.a_k_step;    // this product's corner of A ...
-        const int bn = nt * TN + bt * p.b_n_step, bk = bt * p.b_k_step;   // ... and of B
-        for (int kb = 0; kb < kblocks; ++kb) {
+      auto load = [&](uint32_t dst, const CUtensorMap* tm, uint32_t full, int x, int y) {
+        if (CTAS == 2) tma_load_2d_pair(dst, tm, full, x, y);
+        else tma_load_2d(dst, tm, full, x, y);
+      };
+      for (int item = first_item; item < num_items && ok; item += item_step) {
+        const PlainItem w = plain_item(p, item, kblocks);
+        const int am = (w.mt * CTAS + static_cast<int>(cta_rank)) * kBlockM + w.bt * p.a_m_step;   // this CTA's rows of A,
+        const int bn = w.nt * TN + static_cast<int>(cta_rank) * kBCols + w.bt * p.b_n_step;        // its columns of B
+        const int ak = w.bt * p.a_k_step, bk = w.bt * p.b_k_step;
+        for (int kb = w.kb0; kb < w.kb1; ++kb) {
           if (!bounded_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
-          const uint32_t full = smem_u32(&ctl->full[stage]);
+          uint32_t full = smem_u32(&ctl->full[stage]);
           const uint32_t a_dst = tiles_addr + stage * p.stage_bytes;
           const int seg = kb >= p.seg_kblocks[0] ? 1 : 0;
           const int kloc = (kb - (seg ? p.seg_kblocks[0] : 0)) * kBlockK;      // K offset inside the segment
-          mbar_arrive_expect_tx(full, kABytes + kBBytes);
+          if (cta_rank == 0) mbar_arrive_expect_tx(full, CTAS * (kABytes + kBBytes));   // of both CTAs' copies when paired
+          if (CTAS == 2) full = cluster_map_shared(full, 0);                   // the leader's barrier
           if (A_MN) {
 #pragma unroll
-            for (int q = 0; q < kBlockM / 64; ++q)
-              tma_load_2d(a_dst + q * kMnBoxBytes, &p.tm_a, full, am + q * 64, p.a_k0[seg] + kloc + ak);
+            for (int q = 0; q < kBlockM / 64; ++q) load(a_dst + q * kMnBoxBytes, &p.tm_a, full, am + q * 64, p.a_k0[seg] + kloc + ak);
           } else {
-            tma_load_2d(a_dst, &p.tm_a, full, p.a_k0[seg] + kloc + ak, am);
+            load(a_dst, &p.tm_a, full, p.a_k0[seg] + kloc + ak, am);
           }
           if (B_MN) {
 #pragma unroll
-            for (int q = 0; q < TN / 64; ++q)
-              tma_load_2d(a_dst + kABytes + q * kMnBoxBytes, &p.tm_b[seg], full, bn + q * 64, kloc + bk);
+            for (int q = 0; q < kBCols / 64; ++q) load(a_dst + kABytes + q * kMnBoxBytes, &p.tm_b[seg], full, bn + q * 64, kloc + bk);
           } else {
-            tma_load_2d(a_dst + kABytes, &p.tm_b[seg], full, kloc + bk, bn);
+            load(a_dst + kABytes, &p.tm_b[seg], full, kloc + bk, bn);
           }
           issued_mask |= 1u << stage;
           phase_mask = (phase_mask & ~(1u << stage)) | (phase << stage);
@@ -874,29 +974,32 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
         }
       }
       // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
-      for (int s = 0; s < p.stages; ++s)
-        if (issued_mask & (1u << s)) {
-          const uint32_t bar = smem_u32(&ctl->full[s]);
-          const uint32_t par = (phase_mask >> s) & 1u;
-          const uint64_t t0 = global_timer_ns();
-          while (!mbar_try_wait(bar, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
-        }
+      if (CTAS == 1 || cta_rank == 0) {
+        for (int s = 0; s < p.stages; ++s)
+          if (issued_mask & (1u << s)) {
+            const uint32_t bar = smem_u32(&ctl->full[s]);
+            const uint32_t par = (phase_mask >> s) & 1u;
+            const uint64_t t0 = global_timer_ns();
+            while (!mbar_try_wait(bar, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
+          }
+      }
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (lane == 0 && cta_rank == 0) {
       uint32_t stage = 0, phase = 0, use = 0;
       bool ok = true;
-      const uint32_t idesc = umma_idesc_bf16(kBlockM, TN, A_MN, B_MN);
+      const uint32_t idesc = umma_idesc_bf16(kBlockM * CTAS, TN, A_MN, B_MN);
       // descriptor advance per K=16 step, in 16-byte units: 32 bytes along a swizzled K-major row, two 8-row groups
       // (2048 bytes) down an MN-major box
       constexpr uint32_t kStepA = A_MN ? 128u : 2u, kStepB = B_MN ? 128u : 2u;
-      for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x, ++use) {
+      for (int item = first_item; item < num_items && ok; item += item_step, ++use) {
+        const PlainItem w = plain_item(p, item, kblocks);
         const uint32_t slot = use % kSlots;
         if (!bounded_wait(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + slot * TN;
-        for (int kb = 0; kb < kblocks; ++kb) {
+        for (int kb = w.kb0; kb < w.kb1; ++kb) {
           if (!bounded_wait(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a_addr = tiles_addr + stage * p.stage_bytes;
@@ -904,16 +1007,22 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
           const uint64_t b_desc = B_MN ? umma_smem_desc_mn_sw128(a_addr + kABytes, kMnBoxBytes)
                                        : umma_smem_desc_sw128(a_addr + kABytes);
 #pragma unroll
-          for (int kk = 0; kk < kBlockK / 16; ++kk)
-            umma_bf16(d_tmem, a_desc + kStepA * kk, b_desc + kStepB * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
-          umma_commit(smem_u32(&ctl->empty[stage]));
+          for (int kk = 0; kk < kBlockK / 16; ++kk) {
+            const uint32_t acc = (kb != w.kb0 || kk != 0) ? 1u : 0u;
+            if (CTAS == 2) umma_bf16_pair(d_tmem, a_desc + kStepA * kk, b_desc + kStepB * kk, idesc, acc);
+            else umma_bf16(d_tmem, a_desc + kStepA * kk, b_desc + kStepB * kk, idesc, acc);
+          }
+          if (CTAS == 2) umma_commit_pair(smem_u32(&ctl->empty[stage]));
+          else umma_commit(smem_u32(&ctl->empty[stage]));
           if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        umma_commit(smem_u32(&ctl->tfull[slot]));
+        if (CTAS == 2) umma_commit_pair(smem_u32(&ctl->tfull[slot]));
+        else umma_commit(smem_u32(&ctl->tfull[slot]));
       }
       if (!ok) {
-        umma_commit(smem_u32(&ctl->drain));
+        if (CTAS == 2) umma_commit_pair(smem_u32(&ctl->drain));
+        else umma_commit(smem_u32(&ctl->drain));
         const uint64_t t0 = global_timer_ns();
         while (!mbar_try_wait(smem_u32(&ctl->drain), 0) && global_timer_ns() - t0 < kWaitLimitNs) {}
       }
@@ -923,65 +1032,90 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
     const int quarter = warp & 3;
     const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
     uint32_t use = 0;
-    for (int item = blockIdx.x; item < num_items; item += gridDim.x, ++use) {
-      const int bt = item / per_batch, rest = item - bt * per_batch;
-      const int nt = rest % p.n_tiles, mt = rest / p.n_tiles;
+    for (int item = first_item; item < num_items; item += item_step, ++use) {
+      const PlainItem w = plain_item(p, item, kblocks);
       const uint32_t slot = use % kSlots;
       if (!bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use / kSlots) & 1u, ctl, p.status, lane)) break;
       tc_fence_after();
-      const int row = mt * kBlockM + quarter * 32 + lane;
+      const int row = (w.mt * CTAS + static_cast<int>(cta_rank)) * kBlockM + quarter * 32 + lane;
       const uint32_t tcol = lane_base + slot * TN;
-      const size_t coff = static_cast<size_t>(row < p.M ? row : 0) * p.ldc + static_cast<size_t>(bt) * p.c_step;
-      float* crow = p.C + coff;
-      for (int b = 0; b < TN / 16; ++b) {
-        const int col0 = nt * TN + b * 16;
-        if (col0 >= p.N) break;                          // (warp-uniform) the rest of the tile lies past the last column
+      const size_t coff = static_cast<size_t>(row < p.M ? row : 0) * p.ldc + static_cast<size_t>(w.bt) * p.c_step;
+      float* crow = p.C == nullptr || row >= p.M ? nullptr : plain_row(p, row) + static_cast<size_t>(w.bt) * p.c_step;
+      const int batches = min(TN, p.N - w.nt * TN) / 16;         // (N is a multiple of 16) the rest lies past the last column
+      const bool cut = w.tail >= 0;
+      // a cut tile's part: 32 x TN floats per warp, lane-fastest so that every access is 512 contiguous bytes
+      float4* part = reinterpret_cast<float4*>(p.partial) +
+                     (cut ? (((static_cast<size_t>(w.tail) * p.split + w.part) * CTAS + cta_rank) * 4 + quarter) * (8 * TN) : 0) + lane;
+      for (int b = 0; b < batches; ++b) {
         float x[16];
         tmem_ld16(tcol + b * 16, x);
-        if (row < p.M && p.C == nullptr && p.C_hilo == nullptr) {
-          __align__(16) __nv_bfloat16 o[16];
+        if (cut) {
 #pragma unroll
-          for (int q = 0; q < 16; ++q) o[q] = __float2bfloat16_rn(x[q]);
-          uint4* dst = reinterpret_cast<uint4*>(p.C_bf16 + coff + col0);      // ldc, c_step and C_bf16 keep 16 columns 32-byte aligned
-          dst[0] = reinterpret_cast<const uint4*>(o)[0];
-          dst[1] = reinterpret_cast<const uint4*>(o)[1];
-        } else if (row < p.M && col0 < p.N && p.C == nullptr) {
-          // 16 columns of one group: 32 bytes of high halves and 32 bytes of low halves
-          const int grp = col0 / p.split_k, q0 = col0 - grp * p.split_k;
-          __align__(16) __nv_bfloat16 hi[16], lo[16];
-#pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            hi[q] = __float2bfloat16_rn(x[q]);
-            lo[q] = __float2bfloat16_rn(x[q] - __bfloat162float(hi[q]));
-          }
-          __nv_bfloat16* dst = p.C_hilo + static_cast<size_t>(row) * (2 * p.N) + static_cast<size_t>(2 * grp) * p.split_k + q0;
-          reinterpret_cast<uint4*>(dst)[0] = reinterpret_cast<const uint4*>(hi)[0];
-          reinterpret_cast<uint4*>(dst)[1] = reinterpret_cast<const uint4*>(hi)[1];
-          reinterpret_cast<uint4*>(dst + p.split_k)[0] = reinterpret_cast<const uint4*>(lo)[0];
-          reinterpret_cast<uint4*>(dst + p.split_k)[1] = reinterpret_cast<const uint4*>(lo)[1];
-        } else if (row < p.M && col0 < p.N) {          // N is a multiple of 16
-          if (p.wide_stores) {                         // 32-byte aligned rows: one full sector per store
-            st_global_v8(crow + col0, x);
-            st_global_v8(crow + col0 + 8, x + 8);
-          } else {
-            float4* c4 = reinterpret_cast<float4*>(crow + col0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) c4[q] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-          }
+          for (int q = 0; q < 4; ++q) part[b * 128 + 32 * q] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+        } else if (row < p.M) {
+          plain_store16(p, x, row, crow, coff, w.nt * TN + b * 16);
         }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&ctl->tempty[slot]));
+      if (lane == 0) {
+        if (CTAS == 2) mbar_arrive_cluster(cluster_map_shared(smem_u32(&ctl->tempty[slot]), 0));
+        else mbar_arrive(smem_u32(&ctl->tempty[slot]));
+      }
     }
   }
 
   tc_fence_before();
   __syncthreads();
+  if (CTAS == 2) {
+    // a CTA of a pair may leave only when its partner no longer needs it; after an abort, first let what is in flight land
+    if (ctl->abort && threadIdx.x == 0) {
+      const uint64_t t0 = global_timer_ns();
+      while (global_timer_ns() - t0 < kAbortSettleNs) {}
+    }
+    __syncthreads();
+    cluster_sync_all();
+  }
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    if (CTAS == 2) tmem_dealloc_pair(tmem_base, kTmemCols);
+    else tmem_dealloc(tmem_base, kTmemCols);
   }
+}
+
+// The cut tiles of a plain GEMM (256-column tiles, one product): adds their parts up in K order and stores the result. One
+// warp per 32 rows x 16 columns; grid.x = tail_tiles * ctas * 8, 8 warps.
+__global__ void __launch_bounds__(256) split_reduce_kernel(const __grid_constant__ PlainGemmParams p, int ctas) {
+  grid_dependency_wait();   // the parts come from the kernel before this one
+  const int lane = threadIdx.x & 31;
+  int q = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int b = q & 15;
+  q >>= 4;
+  const int quarter = q & 3;
+  q >>= 2;
+  const int rank = q % ctas, tail = q / ctas;
+  const int tile = p.m_tiles * p.n_tiles - p.tail_tiles + tail;
+  const int nt = tile % p.n_tiles, mt = tile / p.n_tiles;
+  const int row = (mt * ctas + rank) * kBlockM + quarter * 32 + lane, col0 = nt * kPlainTileN + b * 16;
+  if (col0 >= p.N) return;
+  const size_t pitch = static_cast<size_t>(ctas) * 4 * (8 * kPlainTileN);
+  const float4* src = reinterpret_cast<const float4*>(p.partial) + static_cast<size_t>(tail) * p.split * pitch +
+                      (static_cast<size_t>(rank) * 4 + quarter) * (8 * kPlainTileN) + b * 128 + lane;
+  float x[16];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) x[e] = 0.f;
+#pragma unroll 4
+  for (int part = 0; part < p.split; ++part) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float4 y = src[part * pitch + 32 * e];
+      x[4 * e] += y.x;
+      x[4 * e + 1] += y.y;
+      x[4 * e + 2] += y.z;
+      x[4 * e + 3] += y.w;
+    }
+  }
+  if (row < p.M) plain_store16(p, x, row, p.C == nullptr ? nullptr : plain_row(p, row), static_cast<size_t>(row) * p.ldc, col0);
 }
 
 }  // namespace mtpc

@@ -287,6 +287,8 @@ struct mtpc_head {
   int max_pairs;                                // clusters of two projection CTAs that can be resident at once
   CUtensorMap tm_emit_dec, tm_sum_dec;          // the same matrices in the few-position draft path's tiles
   int decode_tile_rows, decode_sum_tile_rows;
+  int decode_ksplit;                            // CTAs that share a tile of it, each with its part of K
+  int max_decode_clusters[3];                   // clusters of 2, 4, 8 of its CTAs that can be resident at once
   int num_sms;
   cudaStream_t copy_stream; // host-buffer calls: uploads run here, ahead of the kernels (created on first use)
   cudaEvent_t* copy_events; // [copy_event_count]: "chunk c is on the device"; [0] doubles as "the call may start"
@@ -585,22 +587,23 @@ bool set_circuit_attributes() {
   return ok;
 }
 
-// How many clusters of two projection CTAs the device holds at once (0: none, the single-CTA kernel is used).
-int resident_pairs(int smem_bytes) {
+// How many clusters of `size` CTAs of a kernel the device holds at once (0: none).
+template <typename K>
+int resident_clusters(K kernel, int size, int smem_bytes) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(2);
+  cfg.gridDim = dim3(size);
   cfg.blockDim = dim3(kGemmThreads);
   cfg.dynamicSmemBytes = smem_bytes;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.x = size;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, mtpc_gemm_kernel<kModeLogprob, 2>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -619,6 +622,25 @@ int decode_tile_rows(long long rows, int ctas) {
     if (eff > best_eff + 1e-9) { best_eff = eff; best = tr; }
   }
   return best;
+}
+// The same together with the CTAs per tile (each with its part of K): 1, or 2, 4, 8 where all clusters of that size are
+// resident at once (max_clusters: a size does not pack the SMs of every GPC, so fours cover less of the chip than twos) and
+// every CTA keeps at least four K blocks. A CTA's time goes as its K steps x (rows it fetches per step + a fixed part worth
+// about 32 rows) and the exchange of a cluster costs about 40 steps' worth of a row.
+void choose_decode_tiling(long long rows, int sum_rows, int kblocks, int ctas, const int (&max_clusters)[3], int* tile_rows, int* ksplit) {
+  auto tiles_of = [&](int tr) { return (rows + tr - 1) / tr + (sum_rows + tr / 32 * 32 - 1) / (tr / 32 * 32); };
+  *tile_rows = decode_tile_rows(rows, ctas);
+  *ksplit = 1;
+  const long long per_cta = (tiles_of(*tile_rows) + ctas - 1) / ctas;
+  long long best = kblocks * (per_cta * *tile_rows + 48);
+  for (int e = 0; e < 3; ++e) {
+    const int s = 2 << e;
+    if (kblocks / s < 4) break;
+    for (int tr = 128; tr >= 64; tr -= 8) {
+      const long long cost = (kblocks + s - 1) / s * (tr + 48) + 40 * 48;
+      if (tiles_of(tr) <= max_clusters[e] && cost < best) { best = cost; *tile_rows = tr; *ksplit = s; }
+    }
+  }
 }
 
 // Few-position draft path: one pass over all weight rows with the positions on the N axis.
@@ -656,21 +678,44 @@ int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_
   p.tile_stride = (p.Ppad + 31) / 32 * 32;
   p.pass_tiles = kTmemCols / (2 * p.tile_stride);                     // two slots of pass_tiles accumulators
   if (p.pass_tiles > kDecodeMaxTiles) p.pass_tiles = kDecodeMaxTiles;
+  const int tiles = p.emit_tiles + p.emit2_tiles + p.sum_tiles;
+  const int per_cta = (tiles + h->num_sms - 1) / h->num_sms;         // no wider stages than a CTA has tiles
+  if (p.pass_tiles > per_cta) p.pass_tiles = per_cta;
+  p.ksplit = h->decode_ksplit;
+  while (p.ksplit > 1 && decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad) > 64 * 1024) p.ksplit /= 2;
   // stage = weight tiles + hidden tile, padded so that a 128-row operand read from the last tile's base stays inside
   int stage = p.pass_tiles * p.tile_bytes + p.Ppad * kBlockK * 2;
   const int reach = (p.pass_tiles - 1) * p.tile_bytes + kABytes;
   if (stage < reach) stage = reach;
   p.stage_bytes = (stage + 1023) / 1024 * 1024;
-  const int ctl = 1024 + static_cast<int>(sizeof(GemmControl));
+  const int ctl = 1024 + static_cast<int>(sizeof(GemmControl)) + static_cast<int>(decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad));
   p.stages = (kSmemLimit - ctl) / p.stage_bytes;
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   p.logw = at<float>(h, L.off_logw);
   p.sum_bias = sum_bias(h);
   p.status = at<unsigned>(h, L.off_status);
   p.wait_limit_ns = h->wait_limit_ns;
-  const int tiles = p.emit_tiles + p.emit2_tiles + p.sum_tiles;
-  const int grid = tiles < h->num_sms ? tiles : h->num_sms;
-  mtpc_decode_gemm_kernel<<<grid, kGemmThreads, p.stages * p.stage_bytes + ctl, st>>>(p);
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(p.ksplit > 1 ? tiles * p.ksplit : tiles < h->num_sms ? tiles : h->num_sms);
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = p.stages * p.stage_bytes + ctl;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int nattr = 0;
+  if (h->ring == 0) {
+    attr[nattr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[nattr++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (p.ksplit > 1) {
+    attr[nattr].id = cudaLaunchAttributeClusterDimension;
+    attr[nattr].val.clusterDim.x = p.ksplit;
+    attr[nattr].val.clusterDim.y = 1;
+    attr[nattr++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = nattr;
+  cudaLaunchKernelEx(&cfg, mtpc_decode_gemm_kernel, p);
   h->launches++;
   if (h->lr_k > 0) {
     launch_kernel(lowrank_expand_kernel, dim3(c.n * c.r, (c.v + kExpandThreads - 1) / kExpandThreads), kExpandThreads,
@@ -1501,7 +1546,8 @@ static int bind_parameters(mtpc_head* h, const void* W_emit, const void* W_sum, 
   if (rc == MTPC_OK && dense && L.can_draft_many) rc = make_tmap(&h->tm_emit_sm2, h->W_emit_bf16, emit_rows, cfg->d, L.sm.tile_cols / 2);
   if (rc == MTPC_OK) rc = make_tmap(&h->tm_sum2, h->W_sum_bf16, L.sum_rows, cfg->d, L.sum_cols / 2);
   const uint64_t base_rows = static_cast<uint64_t>(cfg->n) * cfg->v, adapt_rows = static_cast<uint64_t>(cfg->n) * cfg->r * h->lr_k;
-  h->decode_tile_rows = decode_tile_rows(static_cast<long long>(dense ? emit_rows : base_rows + adapt_rows), h->num_sms);
+  choose_decode_tiling(static_cast<long long>(dense ? emit_rows : base_rows + adapt_rows), L.sum_rows, cfg->d / kBlockK, h->num_sms,
+                       h->max_decode_clusters, &h->decode_tile_rows, &h->decode_ksplit);
   if (rc == MTPC_OK && dense) rc = make_tmap(&h->tm_emit_dec, h->W_emit_bf16, emit_rows, cfg->d, h->decode_tile_rows);
   if (rc == MTPC_OK && !dense) rc = make_tmap(&h->tm_emit_dec, h->lr_W_base, base_rows, cfg->d, h->decode_tile_rows);
   if (rc == MTPC_OK && !dense) rc = make_tmap(&h->tm_lrB_dec, h->lr_B, adapt_rows, cfg->d, h->decode_tile_rows);
@@ -1613,7 +1659,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogitsGrouped, 1>);
   fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 2>);
   fail |= !allow_full_smem(mtpc_gemm_kernel<kModeSample, 2>);
-  h->max_pairs = fail ? 0 : resident_pairs(L.lp.pair_smem);
+  h->max_pairs = fail ? 0 : resident_clusters(mtpc_gemm_kernel<kModeLogprob, 2>, 2, L.lp.pair_smem);
   fail |= !allow_full_smem(plain_gemm_kernel<false, false>);
   fail |= !allow_full_smem(plain_gemm_kernel<false, true>);
   fail |= !allow_full_smem(plain_gemm_kernel<true, true>);
@@ -1624,6 +1670,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   fail |= !allow_full_smem(plain_gemm_kernel<false, true, 64>);
   fail |= cudaFuncSetAttribute(mtpc_decode_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) !=
           cudaSuccess;
+  for (int e = 0; e < 3; ++e) h->max_decode_clusters[e] = fail ? 0 : resident_clusters(mtpc_decode_gemm_kernel, 2 << e, kSmemLimit);
   const int slot_smem = static_cast<int>(kSlotSmemLimit);
   fail |= cudaFuncSetAttribute(draft_slot_kernel<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
   fail |= cudaFuncSetAttribute(draft_slot_kernel<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;

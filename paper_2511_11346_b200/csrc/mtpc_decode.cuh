@@ -48,6 +48,7 @@ struct DecodeParams {
   int pass_tiles;                // tiles per pass (<= kDecodeMaxTiles)
   int tile_stride;               // TMEM columns per tile
   int stages, stage_bytes;
+  int ksplit;                    // CTAs of a cluster that share a run of tiles, each with its part of K (1: no cluster)
   float* logits;         // [P, emit_rows]
   float* logits2;        // [P, emit2_rows]
   float* logw;           // [P, sum_rows]
@@ -74,18 +75,30 @@ __device__ __forceinline__ DecodeTile decode_tile(const DecodeParams& p, int t) 
 // the tile's own rows is other data, and the TMEM lanes it produces are never read), then the hidden tile
 // (Ppad rows x 128 bytes) followed by slack so that the last tile's 128-row read stays inside the stage.
 // Tensor memory: two slots of pass_tiles * tile_stride columns.
+// ksplit > 1: where the tiles leave most SMs idle (a factored head's 4600 rows are 72 tiles) a cluster of ksplit CTAs takes a
+// tile, each walking its part of K; the others hand their fp32 accumulators to the first one through its shared memory (behind
+// the ring: [rank - 1][tile][position quad][128 rows] of float4), which adds them in rank order and runs the epilogue.
+// Every CTA then has one pass. The pass over 39 MB of weights (n = 8, r = 16, v = 320, d = 4096, rank 16) took 30 us as 72 CTAs
+// of 64 K steps and half the SMs idle; draft + acceptance of 8 positions: 51 -> 38 us with 146 CTAs of 32 steps.
+__host__ __device__ inline size_t decode_exchange_bytes(int ksplit, int pass_tiles, int Ppad) {
+  return static_cast<size_t>(ksplit - 1) * pass_tiles * kBlockM * Ppad * sizeof(float);
+}
 __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t tiles_addr = (raw_addr + 1023u) & ~1023u;
   uint8_t* tiles = smem_raw + (tiles_addr - raw_addr);
-  GemmControl* ctl = reinterpret_cast<GemmControl*>(tiles + static_cast<size_t>(p.stages) * p.stage_bytes);
+  uint8_t* exchange = tiles + static_cast<size_t>(p.stages) * p.stage_bytes;
+  GemmControl* ctl = reinterpret_cast<GemmControl*>(exchange + decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad));
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int total_tiles = p.emit_tiles + p.emit2_tiles + p.sum_tiles;
-  const int tile_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * total_tiles / gridDim.x);
-  const int tile_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * total_tiles / gridDim.x);
+  const int rank = p.ksplit > 1 ? static_cast<int>(cluster_cta_rank()) : 0;
+  const int group = static_cast<int>(blockIdx.x) / p.ksplit, groups = static_cast<int>(gridDim.x) / p.ksplit;
+  const int tile_begin = static_cast<int>(static_cast<long long>(group) * total_tiles / groups);
+  const int tile_end = static_cast<int>(static_cast<long long>(group + 1) * total_tiles / groups);
+  const int kb0 = rank * p.kblocks / p.ksplit, kb1 = (rank + 1) * p.kblocks / p.ksplit;
   const uint32_t hidden_off = p.pass_tiles * p.tile_bytes;
   const uint32_t slot_cols = p.pass_tiles * p.tile_stride;
 
@@ -113,9 +126,70 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
   }
   tc_fence_before();
   __syncthreads();
+  if (p.ksplit > 1) cluster_sync_all();   // every CTA of the cluster runs before one writes into another's shared memory
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   grid_launch_dependents();   // the per-slot kernel may be scheduled as SMs free up; it waits for this grid's results
+  grid_dependency_wait();     // a draft that follows another call closely sets up its barriers while that one finishes
+
+  const int quarter = warp & 3;
+  const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+  // Tile `tile` of the launch, whose accumulators start at tensor-memory column `col`: logits or log omega of this warp's 32
+  // rows. others: the accumulators of the cluster's other CTAs (NULL: none).
+  auto finish_tile = [&](int tile, uint32_t col, const float4* others) {
+    const DecodeTile t = decode_tile(p, tile);
+    if (quarter * 32 >= t.rows) return;                            // warp-uniform: none of this warp's lanes is a row
+    const int nrows = t.is_sum ? p.sum_rows : (t.second ? p.emit2_rows : p.emit_rows);
+    float* dst = t.is_sum ? p.logw : (t.second ? p.logits2 : p.logits);
+    const int local = quarter * 32 + lane;
+    const int row = t.index * t.rows + local;
+    const bool mine = local < t.rows && row < nrows;
+    const float bias = (t.is_sum && p.sum_bias != nullptr && mine) ? p.sum_bias[row] : 0.f;
+    for (int b = 0; b < (p.P + 15) / 16; ++b) {
+      float x[16];
+      tmem_ld16(lane_base + col + b * 16, x);
+      if (others != nullptr) {
+        for (int part = 0; part + 1 < p.ksplit; ++part) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const float4 y = others[(part * p.pass_tiles * (p.Ppad / 4) + b * 4 + c) * kBlockM + local];
+            x[4 * c] += y.x;
+            x[4 * c + 1] += y.y;
+            x[4 * c + 2] += y.z;
+            x[4 * c + 3] += y.w;
+          }
+        }
+      }
+      if (t.is_sum && p.r <= 32) {
+#pragma unroll
+        for (int c = 0; c < 16; ++c) x[c] += bias;
+        // log-softmax over the r rows of a sum unit = r adjacent lanes (r a power of two <= 32); the 16
+        // positions of the batch are reduced side by side so that the shuffles overlap
+        float m[16], e[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) m[c] = x[c];
+        for (int off = 1; off < p.r; off <<= 1) {
+#pragma unroll
+          for (int c = 0; c < 16; ++c) m[c] = fmaxf(m[c], __shfl_xor_sync(0xffffffffu, m[c], off));
+        }
+#pragma unroll
+        for (int c = 0; c < 16; ++c) e[c] = fast_ex2((x[c] - m[c]) * kLog2e);
+        for (int off = 1; off < p.r; off <<= 1) {
+#pragma unroll
+          for (int c = 0; c < 16; ++c) e[c] += __shfl_xor_sync(0xffffffffu, e[c], off);
+        }
+#pragma unroll
+        for (int c = 0; c < 16; ++c) x[c] = x[c] - m[c] - fast_lg2(e[c]) * kLn2;
+      }
+      if (mine) {
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          const int pos = b * 16 + c;
+          if (pos < p.P) dst[static_cast<size_t>(pos) * nrows + row] = x[c];   // 32 lanes -> 128 contiguous bytes
+        }
+      }
+    }
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -126,7 +200,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
         const int ntiles = min(p.pass_tiles, tile_end - cur);
         uint32_t bytes = p.Ppad * (kBlockK * 2);                   // out-of-range rows are zero-filled and counted
         for (int q = 0; q < ntiles; ++q) bytes += decode_tile(p, cur + q).rows * (kBlockK * 2);
-        for (int kb = 0; kb < p.kblocks; ++kb) {
+        for (int kb = kb0; kb < kb1; ++kb) {
           if (!bounded_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
           const uint32_t full = smem_u32(&ctl->full[stage]);
           const uint32_t dst = tiles_addr + stage * p.stage_bytes;
@@ -169,7 +243,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + slot * slot_cols;
-        for (int kb = 0; kb < p.kblocks; ++kb) {
+        for (int kb = kb0; kb < kb1; ++kb) {
           if (!bounded_wait(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t w_addr = tiles_addr + stage * p.stage_bytes;
@@ -178,7 +252,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
             const uint64_t a_desc = umma_smem_desc_sw128(w_addr + q * p.tile_bytes);
 #pragma unroll
             for (int kk = 0; kk < kBlockK / 16; ++kk)
-              umma_bf16(d_tmem + q * p.tile_stride, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+              umma_bf16(d_tmem + q * p.tile_stride, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
           }
           umma_commit(smem_u32(&ctl->empty[stage]));
           if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
@@ -195,8 +269,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue: warp q owns lanes 32q .. 32q+31
-    const int quarter = warp & 3;
-    const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
     uint32_t use = 0;
     bool ok = true;
     for (int cur = tile_begin; cur < tile_end && ok; ++use) {
@@ -207,48 +279,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
         break;
       }
       tc_fence_after();
-      for (int q = 0; q < ntiles; ++q) {
-        const DecodeTile t = decode_tile(p, cur + q);
-        if (quarter * 32 >= t.rows) continue;                      // warp-uniform: none of this warp's lanes is a row
-        const int nrows = t.is_sum ? p.sum_rows : (t.second ? p.emit2_rows : p.emit_rows);
-        float* dst = t.is_sum ? p.logw : (t.second ? p.logits2 : p.logits);
-        const uint32_t tcol = lane_base + slot * slot_cols + q * p.tile_stride;
-        const int local = quarter * 32 + lane;
-        const int row = t.index * t.rows + local;
-        const bool mine = local < t.rows && row < nrows;
-        const float bias = (t.is_sum && p.sum_bias != nullptr && mine) ? p.sum_bias[row] : 0.f;
-        for (int b = 0; b < (p.P + 15) / 16; ++b) {
-          float x[16];
-          tmem_ld16(tcol + b * 16, x);
-          if (t.is_sum && p.r <= 32) {
+      if (p.ksplit == 1) {
+        for (int q = 0; q < ntiles; ++q) finish_tile(cur + q, slot * slot_cols + q * p.tile_stride, nullptr);
+      } else if (rank > 0) {
+        // one pass: the accumulators go to the cluster's first CTA
+        const uint32_t dst0 = cluster_map_shared(smem_u32(exchange), 0) + (quarter * 32 + lane) * 16;
+        for (int q = 0; q < ntiles; ++q)
+          for (int b = 0; b < (p.P + 15) / 16; ++b) {
+            float x[16];
+            tmem_ld16(lane_base + q * p.tile_stride + b * 16, x);
+            const uint32_t dst = dst0 + (((rank - 1) * p.pass_tiles + q) * (p.Ppad / 4) + b * 4) * (kBlockM * 16);
 #pragma unroll
-            for (int c = 0; c < 16; ++c) x[c] += bias;
-            // log-softmax over the r rows of a sum unit = r adjacent lanes (r a power of two <= 32); the 16
-            // positions of the batch are reduced side by side so that the shuffles overlap
-            float m[16], e[16];
-#pragma unroll
-            for (int c = 0; c < 16; ++c) m[c] = x[c];
-            for (int off = 1; off < p.r; off <<= 1) {
-#pragma unroll
-              for (int c = 0; c < 16; ++c) m[c] = fmaxf(m[c], __shfl_xor_sync(0xffffffffu, m[c], off));
-            }
-#pragma unroll
-            for (int c = 0; c < 16; ++c) e[c] = fast_ex2((x[c] - m[c]) * kLog2e);
-            for (int off = 1; off < p.r; off <<= 1) {
-#pragma unroll
-              for (int c = 0; c < 16; ++c) e[c] += __shfl_xor_sync(0xffffffffu, e[c], off);
-            }
-#pragma unroll
-            for (int c = 0; c < 16; ++c) x[c] = x[c] - m[c] - fast_lg2(e[c]) * kLn2;
+            for (int c = 0; c < 4; ++c) st_cluster_v4(dst + c * (kBlockM * 16), x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
           }
-          if (mine) {
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-              const int pos = b * 16 + c;
-              if (pos < p.P) dst[static_cast<size_t>(pos) * nrows + row] = x[c];   // 32 lanes -> 128 contiguous bytes
-            }
-          }
-        }
       }
       cur += ntiles;
       tc_fence_before();
@@ -259,6 +302,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
 
   tc_fence_before();
   __syncthreads();
+  if (p.ksplit > 1) {
+    cluster_sync_all();       // the other CTAs' accumulators have arrived
+    if (rank == 0 && warp >= 2) {
+      tc_fence_after();
+      for (int q = 0; q < tile_end - tile_begin; ++q)
+        finish_tile(tile_begin + q, q * p.tile_stride, reinterpret_cast<const float4*>(exchange) + q * (p.Ppad / 4) * kBlockM);
+      tc_fence_before();
+    }
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);

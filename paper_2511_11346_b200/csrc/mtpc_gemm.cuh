@@ -31,10 +31,7 @@ namespace mtpc {
 
 constexpr int kBlockM = 128;         // positions per tile (= TMEM lanes)
 constexpr int kBlockK = 64;          // bf16 elements per 128-byte swizzled row
-#ifndef MTPC_MAX_STAGES
-#define MTPC_MAX_STAGES 8
-#endif
-constexpr int kMaxStages = MTPC_MAX_STAGES;
+constexpr int kMaxStages = 16;
 constexpr int kMaxSlots = 16;
 constexpr int kTmemCols = 512;
 constexpr int kGemmThreads = 192;

@@ -60,6 +60,10 @@ __device__ __forceinline__ uint32_t cluster_map_shared(uint32_t smem_addr, uint3
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr), "r"(rank));
   return a;
 }
+// 16 bytes into any CTA's shared memory (address from cluster_map_shared); ordered by the next cluster_sync_all.
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, float a, float b, float c, float d) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
 // Arrive on an mbarrier of any CTA of the cluster (address from cluster_map_shared).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");

@@ -286,15 +286,13 @@ int mtpc_lowrank_backward(int32_t n, int32_t r, int32_t v, int32_t d, int32_t k,
  * of 2 d n r v. z is handed to the tensor cores as two bf16 halves (z = hi + lo), so the result differs from exact
  * arithmetic on the bf16 parameters only by fp32 accumulation (no rounding of a composed U to bf16).
  *   cfg, W_sum, T_static, workspace, stream, out: as mtpc_create_head; cfg->io_dtype must be MTPC_BF16.
- *   k        the adaptors' rank: 16 or 32 (MTPC_ERR_UNSUPPORTED otherwise). v must be a multiple of 16 that splits into
- *            at most eight panels of at most 224 columns (a panel's two accumulators and the correction slots share the
- *            512 columns of tensor memory): every such v up to 1792; MTPC_ERR_UNSUPPORTED otherwise.
+ *   k        the adaptors' rank: 16 or 32, and v at most 1792 (MTPC_ERR_UNSUPPORTED otherwise).
  *   W_base   dev [n, v, d] bf16;  A dev [n, r, v, k] bf16;  B dev [n, r, k, d] bf16: caller-owned, read in place, must
  *            outlive the head (after an optimiser step no call is needed unless W_sum / T_static moved:
  *            mtpc_update_parameters with W_emit = NULL then).
- *   workspace >= mtpc_lowrank_workspace_bytes(cfg, k): the dense head's workspace plus z = B h as two bf16 halves, a copy
- *            of A in the layout the kernel reads (remade on every call, so A is always read as it is then) and, for
- *            v > 224, the per-panel partial log-sum-exps.
+ *   workspace >= mtpc_lowrank_workspace_bytes(cfg, k): the dense head's workspace plus W_base h, z = B h as two bf16
+ *            halves, a copy of A in the layout the kernel reads (remade on every call, so A is always read as it is then),
+ *            the partial log-sum-exps and 58 MB for parts of the GEMMs' tiles.
  * Such a head serves mtpc_window_logprob, mtpc_window_prefix_logprob, mtpc_window_loss, mtpc_window_logprob_host,
  * mtpc_draft_sample, mtpc_draft_sample_prefix and mtpc_speculative_accept: up to 128 positions, the draft's weight pass
  * streams W_base and B (n v + n r k rows) instead of n r v composed rows and the logits are formed from the two small
@@ -315,8 +313,8 @@ int mtpc_lowrank_workspace_bytes(const mtpc_config* cfg, int32_t k, size_t* out_
  *   d_hidden   = sum_i (sum_j g_ij) W_base[i] + sum_ij (g_ij A[i,j]) B[i,j] + the sum units' part.
  *   hidden, targets, T, weight, out_logprob, d_hidden [T, d], dW_sum, dT_static: as mtpc_window_logprob_backward.
  *   dW_base dev [n, v, d] fp32;  dA dev [n, r, v, k] fp32;  dB dev [n, r, k, d] fp32: OVERWRITTEN.
- *   bwd_workspace  dev, 256-byte aligned, >= mtpc_lowrank_backward_workspace_bytes(cfg, k, T): the kept logits
- *                  [T, n r v] fp32, their gradients in bf16, and the small operands derived from them.
+ *   bwd_workspace  dev, 256-byte aligned, >= mtpc_lowrank_backward_workspace_bytes(cfg, k, T): the logits' gradients
+ *                  [T, n r v] in bf16 (no logits are kept), and the small operands derived from them.
  * g is rounded to bf16 before the tensor cores contract it (as in mtpc_window_logprob_backward), dA uses the bf16 high
  * half of B h. MTPC_ERR_STATE on a head that was not created by mtpc_create_head_lowrank. Asynchronous on `stream`.
  */

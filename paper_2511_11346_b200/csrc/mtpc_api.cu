@@ -279,11 +279,12 @@ struct mtpc_head {
   const void* lr_B;                             // [n, r, k, d] bf16
   size_t lr_off_arep;                           // workspace: A as [n, v, r, k]
   size_t lr_off_dec;                            // workspace: few-position draft products base [P, n v] | z [P, n r k]
-  size_t lr_off_base;                           // workspace: long drafts: W_base h [T, n v] fp32 (0: not reserved)
+  size_t lr_off_base;                           // workspace: W_base h [T, n v] fp32
   size_t lr_off_split;                          // workspace: parts of split plain GEMMs
   CUtensorMap tm_lrB_dec;                       // B [n r k, d] for the few-position draft path
-  size_t lr_off_zhl, lr_off_partial;            // workspace: z = B h as bf16 halves [T, n r, 2, k]; per-panel partial log-sum-exps
-  LowRankGemmParams lr_params;                  // everything of the factored projection launch that does not depend on the call
+  size_t lr_off_zhl, lr_off_partial;            // workspace: z = B h as bf16 halves [T, n r, 2, k]; partial log-sum-exps per column block
+  CUtensorMap lr_tm_a[2];                       // the copy of A in the boxes of the forward and the gradient build
+  LowRankParams lr_params;                      // everything of the factored projection launch that does not depend on the call
   int max_pairs;                                // clusters of two projection CTAs that can be resident at once
   CUtensorMap tm_emit_dec, tm_sum_dec;          // the same matrices in the few-position draft path's tiles
   int decode_tile_rows, decode_sum_tile_rows;
@@ -765,9 +766,9 @@ struct PlainGemmExtra {
 int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmOperand B1, int K1, int a_k1, float* C,
                       size_t ldc, int M, int N, cudaStream_t st, void* split_ws = nullptr, void* C_hilo = nullptr,
                       int split_k = 0, const PlainGemmExtra* extra = nullptr);
-// parts: 1 = sum-unit tiles (log omega), 2 = z = B h and the repacked A, 4 = the factored kernel (and its merge)
+// parts: 1 = sum-unit tiles (log omega), 2 = W_base h, z = B h and the repacked A, 4 = G (and the units' log-sum-exps)
 int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, const int* targets, cudaStream_t st,
-                              const GradArgs* ga = nullptr, int parts = 7, bool targets_are_drafts = false);
+                              float* lse_out = nullptr, int parts = 7, bool targets_are_drafts = false);
 
 // out [T] (joint) and / or prefix [T, n] (prefix log-marginals); either may be NULL, not both.
 int window_logprob_impl(mtpc_head* h, const void* hidden, const int32_t* targets, int32_t T, float* out, float* prefix,
@@ -797,7 +798,7 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
   // a draft that returns prefix marginals runs the sweep that also yields the slot messages of the acceptance stage
   float* const msg = at<float>(h, L.off_msg);
   if (!L.can_draft) return MTPC_ERR_UNSUPPORTED;
-  if (h->lr_k > 0 && P > L.decode_max_p && wpp == 1 && c.v <= kMaxDraftVocab && h->lr_off_base != 0) {
+  if (h->lr_k > 0 && P > L.decode_max_p && wpp == 1 && c.v <= kMaxDraftVocab) {
     // A long draft on a factored head, one window per position: log omega, the latent draws, then every (window, slot)
     // forms the logits of its one selected unit from W_base h and B h (lowrank_draw_kernel) and draws its byte; the
     // evidence of the drafted bytes under every unit is the factored projection with them as targets. No logits are
@@ -817,12 +818,7 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     pt.end();
     if ((rc = check_launch()) != MTPC_OK) return rc;
     pt.begin();
-    float* base = reinterpret_cast<float*>(h->ws + h->lr_off_base);
-    rc = launch_plain_gemm(h, GemmOperand{hidden, static_cast<size_t>(c.d), false},
-                           GemmOperand{h->lr_W_base, static_cast<size_t>(c.d), false}, c.d,
-                           GemmOperand{h->lr_W_base, static_cast<size_t>(c.d), false}, 0, 0, base,
-                           static_cast<size_t>(c.n) * c.v, P, c.n * c.v, st, h->ws + h->lr_off_split);
-    if (rc != MTPC_OK) return rc;
+    const float* base = reinterpret_cast<const float*>(h->ws + h->lr_off_base);
     {
       const int pairs = W * c.n;
       int blocks = (pairs + kDrawWarps - 1) / kDrawWarps;
@@ -998,7 +994,7 @@ struct BackwardLayout {
   size_t Nc, Spad, Kd;
   size_t off_lse, off_post, off_logits, off_dlogit, off_coeff, off_split, total;
 };
-void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout* B) {
+void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout* B, bool keep_logits = true) {
   B->Nc = static_cast<size_t>(c.n) * c.r * c.v;
   B->Spad = round64(L.sum_rows);
   B->Kd = B->Nc + B->Spad;
@@ -1006,7 +1002,7 @@ void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout*
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
   B->off_lse = take(static_cast<size_t>(T) * c.n * c.r * 4);
   B->off_post = take(static_cast<size_t>(T) * c.n * c.r * 4);
-  B->off_logits = take(static_cast<size_t>(T) * B->Nc * 4);              // [T, Nc] fp32: the emission logits of the forward pass
+  B->off_logits = take(keep_logits ? static_cast<size_t>(T) * B->Nc * 4 : 0);   // [T, Nc] fp32: the emission logits of the forward pass
   B->off_dlogit = take(static_cast<size_t>(T) * B->Kd * 2);          // [T, Nc | Spad] bf16
   B->off_coeff = take(static_cast<size_t>(T) * c.n * 4);             // Eq. 6: weights of the prefix marginals
   B->off_split = take(kSplitBytes);                                 // parts of the GEMMs' cut tiles
@@ -1148,59 +1144,37 @@ int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmO
   return check_launch();
 }
 
-#ifndef MTPC_LR_GROUPS
-#define MTPC_LR_GROUPS 2
-#endif
-constexpr int kLrGroups = MTPC_LR_GROUPS;   // epilogue groups of the factored projection kernel (<= kLrMaxGroups)
-// Tiling of the factored projection (mtpc_lowrank_gemm.cuh) for a head shape; false: the shape does not fit.
-bool plan_lowrank(const mtpc_config& c, int k, LowRankGemmParams* p) {
-  if (k < 16 || k > kLrMaxRank || k % 16 != 0 || c.v % 16 != 0) return false;
-  // the fewest panels whose two base buffers leave room for the correction slots (two per epilogue group, chunks of at
-  // least 16 columns; as many groups, up to kLrGroups and the number of components, as leave chunks of at least 32)
-  int panels = 0, pc = 0, stride = 0, spare = 0;
-  for (int np = 1; np <= kLrMaxPanels; ++np) {
-    pc = ((c.v + np - 1) / np + 15) / 16 * 16;          // the last panel may be narrower
-    stride = (pc + 31) / 32 * 32;
-    spare = kTmemCols - 2 * stride;
-    if (pc <= 256 && spare >= 32) { panels = (c.v + pc - 1) / pc; break; }
-  }
-  if (panels == 0) return false;
-  int groups = kLrGroups < c.r ? kLrGroups : c.r;
-  while (groups > 1 && spare / (2 * groups) < 32) --groups;
-  int chunk = spare / (2 * groups) / 16 * 16;
-  if (chunk > 96) chunk = 96;
-  if (chunk > pc) chunk = pc;
-  p->groups = groups;
+// What a factored head serves (mtpc_lowrank_gemm.cuh); false: the shape does not fit.
+bool plan_lowrank(const mtpc_config& c, int k, LowRankParams* p) {
+  if (k < 16 || k > kLrMaxRank || k % 16 != 0 || c.v % 16 != 0 || c.v > kLrMaxVocab) return false;
   p->n = c.n; p->r = c.r; p->v = c.v; p->k = k;
   p->vv = c.v_valid > 0 ? c.v_valid : c.v;
-  p->kblocks = c.d / kBlockK;
-  p->panels = panels;
-  p->panel_cols = pc;
-  p->acc_stride = stride;
-  p->chunk_cols = chunk;
-  p->nchunk = (pc + chunk - 1) / chunk;
-  p->corr_col0 = 2 * stride;
-  p->base_stage_bytes = kABytes + pc * kBlockK * 2;                                  // a multiple of 1024 (pc % 16 == 0)
-  p->corr_stage_bytes = 2 * kBlockM * 128 + p->nchunk * chunk * 128;                 // two z boxes and the A' boxes of 64 / k components
-  const int ctl = 1024 + static_cast<int>(sizeof(LowRankControl));
-  // at least two correction entries (one in use, the next on its way); the base ring takes the rest, at least two K blocks
-  for (int cs = kLrCorrStages; cs >= 2; --cs) {
-    const int left = kSmemLimit - ctl - cs * p->corr_stage_bytes;
-    int bs = left / p->base_stage_bytes;
-    if (bs > kMaxStages) bs = kMaxStages;
-    if (bs >= 3 || (bs == 2 && cs == 2)) {
-      p->corr_stages = cs;
-      p->base_stages = bs;
-      return true;
-    }
-  }
-  return false;
+  return true;
 }
 
-// Factored projection of a low-rank head: log omega by the dense kernel's sum tiles, z = B h by a plain GEMM that writes
-// it as two bf16 halves, A repacked, then the factored kernel (and the merge of its panels) writes G.
-int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, const int* targets, cudaStream_t st,
-                              const GradArgs* ga, int parts, bool targets_are_drafts) {
+// One launch of the factored projection's kernel on what parts 1 | 2 left in the workspace.
+template <int MODE>
+int launch_lowrank_logits(mtpc_head* h, LowRankParams p, int T, cudaStream_t st) {
+  const int rc = make_tmap(&p.tm_z, h->ws + h->lr_off_zhl, static_cast<uint64_t>(T), static_cast<uint64_t>(p.n) * p.r * 2 * p.k, kBlockM);
+  p.blocks = (p.v + lowrank_cols(MODE) - 1) / lowrank_cols(MODE);
+  p.tm_a = h->lr_tm_a[MODE];
+  if (rc != MTPC_OK) return rc;
+  p.T = T;
+  p.m_tiles = (T + kBlockM - 1) / kBlockM;
+  p.base = reinterpret_cast<const float*>(h->ws + h->lr_off_base);
+  p.status = at<unsigned>(h, h->L.off_status);
+  p.wait_limit_ns = h->wait_limit_ns;
+  const long long items = static_cast<long long>(p.m_tiles) * p.n * p.blocks;
+  const int grid = static_cast<int>(items < h->num_sms ? items : h->num_sms);
+  lowrank_logits_kernel<MODE><<<grid, lowrank_threads(MODE), lowrank_smem_bytes(MODE), st>>>(p);
+  h->launches++;
+  return check_launch();
+}
+
+// Factored projection of a low-rank head: log omega by the dense kernel's sum tiles, W_base h and z = B h (as two bf16 halves)
+// by plain GEMMs, A repacked; then the log-sum-exps over base + corrections and their merge into G.
+int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, const int* targets, cudaStream_t st, float* lse_out,
+                              int parts, bool targets_are_drafts) {
   const mtpc_config& c = h->cfg;
   const Layout& L = h->L;
   const int units = c.n * c.r, k = h->lr_k;
@@ -1208,51 +1182,32 @@ int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, cons
   if (parts & 1) rc = launch_gemm(h, kModeLogprob, hidden_bf16, T, 1, false, true, targets, nullptr, nullptr, st);
   if (rc != MTPC_OK) return rc;
   __nv_bfloat16* zhl = reinterpret_cast<__nv_bfloat16*>(h->ws + h->lr_off_zhl);
+  float* base = reinterpret_cast<float*>(h->ws + h->lr_off_base);
   if (parts & 2) {
+    const GemmOperand hid{hidden_bf16, static_cast<size_t>(c.d), false};
+    const GemmOperand bmat{h->lr_B, static_cast<size_t>(c.d), false};          // [n r k, d], K = d contiguous
+    const GemmOperand wmat{h->lr_W_base, static_cast<size_t>(c.d), false};
+    rc = launch_plain_gemm(h, hid, wmat, c.d, wmat, 0, 0, base, static_cast<size_t>(c.n) * c.v, T, c.n * c.v, st, h->ws + h->lr_off_split);
+    // z = B h, leaving the GEMM's epilogue already split into its two bf16 halves [T, n r, 2, k]
+    if (rc == MTPC_OK)
+      rc = launch_plain_gemm(h, hid, bmat, c.d, bmat, 0, 0, nullptr, 0, T, units * k, st, h->ws + h->lr_off_split, zhl, k);
+    if (rc != MTPC_OK) return rc;
     // A as [n, v, r, k]: the adaptor columns of adjacent components side by side (remade every call: A may have changed)
     const size_t pieces = static_cast<size_t>(units) * c.v * (k / 8);
     lowrank_repack_kernel<<<static_cast<unsigned>((pieces + 255) / 256), 256, 0, st>>>(
         static_cast<const uint4*>(h->lr_A), reinterpret_cast<uint4*>(h->ws + h->lr_off_arep), c.n, c.r, c.v, k / 8);
     h->launches += 1;
-    // z = B h, leaving the GEMM's epilogue already split into its two bf16 halves [T, n r, 2, k]
-    const GemmOperand hid{hidden_bf16, static_cast<size_t>(c.d), false};
-    const GemmOperand bmat{h->lr_B, static_cast<size_t>(c.d), false};          // [n r k, d], K = d contiguous
-    rc = launch_plain_gemm(h, hid, bmat, c.d, bmat, 0, 0, nullptr, 0, T, units * k, st, h->ws + h->lr_off_split,
-                           zhl, k);
-    if (rc != MTPC_OK) return rc;
   }
   if (!(parts & 4)) return check_launch();
-  LowRankGemmParams p = h->lr_params;
-  rc = make_tmap(&p.tm_h, hidden_bf16, static_cast<uint64_t>(T), static_cast<uint64_t>(c.d), kBlockM);
-  if (rc == MTPC_OK) rc = make_tmap(&p.tm_z, zhl, static_cast<uint64_t>(T), static_cast<uint64_t>(units) * 2 * k, kBlockM);
-  if (rc != MTPC_OK) return rc;
-  p.T = T;
-  p.m_tiles = (T + kBlockM - 1) / kBlockM;
-  p.targets = targets;
-  p.G = at<float>(h, L.off_G);
-  p.status = at<unsigned>(h, L.off_status);
-  p.wait_limit_ns = h->wait_limit_ns;
-  p.missing_is_nan = targets_are_drafts ? 1 : 0;
-  if (ga != nullptr) {                 // a training call keeps every logit and every unit's log-sum-exp
-    p.logit_out = ga->logit_out;
-    p.logit_pitch = ga->logit_pitch;
-    p.lse_out = ga->lse_out;
-  }
+  LowRankParams p = h->lr_params;
+  p.log_sum = reinterpret_cast<float*>(h->ws + h->lr_off_partial);
+  p.ref = p.log_sum + static_cast<size_t>((c.v + 31) / 32) * T * units;
+  if ((rc = launch_lowrank_logits<kLowRankForward>(h, p, T, st)) != MTPC_OK) return rc;
   const size_t entries = static_cast<size_t>(T) * units;
-  p.partial = reinterpret_cast<float2*>(h->ws + h->lr_off_partial);
-  p.target_logit = reinterpret_cast<float*>(h->ws + h->lr_off_partial +
-                                            static_cast<size_t>(p.panels) * c.max_positions * units * sizeof(float2));
-  const long long items = static_cast<long long>(p.m_tiles) * c.n * p.panels;
-  const int grid = static_cast<int>(items < h->num_sms ? items : h->num_sms);
-  const int ctl = 1024 + static_cast<int>(sizeof(LowRankControl));
-  mtpc_lowrank_gemm_kernel<<<grid, kLrRoleThreads + 128 * p.groups,
-                             p.base_stages * p.base_stage_bytes + p.corr_stages * p.corr_stage_bytes + ctl, st>>>(p);
+  lowrank_merge_kernel<<<static_cast<unsigned>((entries + 255) / 256), 256, 0, st>>>(
+      p.log_sum, p.ref, base, zhl, reinterpret_cast<const __nv_bfloat16*>(h->ws + h->lr_off_arep), targets, at<float>(h, L.off_G), lse_out,
+      at<unsigned>(h, L.off_status), entries, c.n, c.r, c.v, p.vv, k, targets_are_drafts ? 1 : 0);
   h->launches += 1;
-  if (p.panels > 1) {     // several panels per unit: their partial log-sum-exps are combined into G
-    lowrank_merge_kernel<<<static_cast<unsigned>((entries + 255) / 256), 256, 0, st>>>(
-        p.partial, p.target_logit, targets, p.G, p.lse_out, p.status, entries, c.r, p.vv, p.panels, p.missing_is_nan);
-    h->launches += 1;
-  }
   return check_launch();
 }
 
@@ -1370,7 +1325,7 @@ int backward_tail(mtpc_head* head, const BackwardLayout& B, uint8_t* bw, const v
   return rc;
 }
 
-// Backward workspace of a factored head: the dense layout (log-sum-exps, posteriors, kept logits, logit gradients), then
+// Backward workspace of a factored head: the dense layout without kept logits (log-sum-exps, posteriors, logit gradients), then
 //   sy    [T, n v | n r k | S r padded] bf16: the logit gradients summed over a slot's components, multiplied by the
 //         adaptors A, and those of the sum units: the A operand of d hidden and of the three weight-gradient GEMMs;
 //   wcat  [n v + n r k, d] bf16: W_base and B one after the other (one K segment of d hidden);
@@ -1381,7 +1336,7 @@ struct LowRankBackwardLayout {
   size_t off_sy, off_wcat, off_apad, total;
 };
 void plan_lowrank_backward(const mtpc_config& c, const Layout& L, int k, int T, LowRankBackwardLayout* R) {
-  plan_backward(c, L, T, &R->B);
+  plan_backward(c, L, T, &R->B, /*keep_logits=*/false);
   const size_t units = static_cast<size_t>(c.n) * c.r;
   R->Ksy = static_cast<size_t>(c.n) * c.v + units * k;
   R->pitch = R->Ksy + R->B.Spad;
@@ -1409,30 +1364,22 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
   pt.begin();
   __nv_bfloat16* dlogit = reinterpret_cast<__nv_bfloat16*>(bw + B.off_dlogit);
   const int Nc = static_cast<int>(B.Nc);
-  LogitGradArgs la;
-  la.logits = reinterpret_cast<const float*>(bw + B.off_logits);
-  la.lse = reinterpret_cast<const float*>(bw + B.off_lse);
-  la.post = reinterpret_cast<const float*>(bw + B.off_post);
-  la.targets = targets;
-  la.dlogit = dlogit;
-  la.pitch = B.Kd;
-  la.T = T; la.Nc = Nc; la.n = c.n; la.r = c.r; la.v = c.v;
+  LowRankParams lp = head->lr_params;
+  lp.targets = targets;
+  lp.G = at<float>(head, L.off_G);
+  lp.lse = reinterpret_cast<const float*>(bw + B.off_lse);
+  lp.post = reinterpret_cast<const float*>(bw + B.off_post);
+  lp.g = dlogit;
+  lp.g_pitch = B.Kd;
+  lp.s = sy;
+  lp.s_pitch = R.pitch;
+  if ((rc = launch_lowrank_logits<kLowRankGradient>(head, lp, T, st)) != MTPC_OK) return rc;
   {
-    const int col_blocks = (Nc / 8 + 255) / 256;
-    int row_blocks = (16 * head->num_sms + col_blocks - 1) / col_blocks;
-    if (row_blocks > T) row_blocks = T;
-    if (row_blocks > 65535) row_blocks = 65535;
-    logit_gradient_kernel<<<dim3(col_blocks, row_blocks), 256, 0, st>>>(la);
-  }
-  {
-    const size_t pieces = static_cast<size_t>(T) * (c.n * c.v / 8);
-    lowrank_component_sum_kernel<<<static_cast<unsigned>((pieces + 255) / 256), 256, 0, st>>>(dlogit, B.Kd, sy, R.pitch, T,
-                                                                                               c.n, c.r, c.v);
     const size_t pad_pieces = static_cast<size_t>(units) * R.v64 * (k / 8);
     lowrank_pad_kernel<<<static_cast<unsigned>((pad_pieces + 255) / 256), 256, 0, st>>>(
         static_cast<const uint4*>(head->lr_A), reinterpret_cast<uint4*>(bw + R.off_apad), units, c.v, static_cast<int>(R.v64), k / 8);
   }
-  head->launches += 3;
+  head->launches += 1;
   uint8_t* wcat = bw + R.off_wcat;
   const size_t base_bytes = static_cast<size_t>(c.n) * c.v * c.d * 2;
   bool fail = cudaMemcpyAsync(wcat, head->lr_W_base, base_bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess;
@@ -1577,26 +1524,22 @@ struct LowRankSpec {
 };
 
 // Workspace of a factored head beyond the dense layout: z = B h as two bf16 halves [T, n r, 2, k] (written by the GEMM
-// that computes it), where a unit is cut into panels the panels' (maximum, sum) pairs and the targets' logits, and the
-// copy of A the factored kernel reads.
-static int lowrank_extra_bytes(const mtpc_config& c, int k, int panels, size_t base_total, size_t* off_zhl,
+// that computes it), W_base h, the log-sums of 32 columns each with their references, and the copy of A the factored kernel reads.
+static int lowrank_extra_bytes(const mtpc_config& c, int k, size_t base_total, size_t* off_zhl,
                                size_t* off_partial, size_t* off_arep, size_t* off_dec, size_t* off_base, size_t* off_split, size_t* total) {
   const size_t units = static_cast<size_t>(c.n) * c.r;
   size_t off = align_up(base_total);
   *off_zhl = off;
   off += align_up(static_cast<size_t>(c.max_positions) * units * 2 * k * 2);
   *off_partial = off;
-  if (panels > 1) off += align_up(static_cast<size_t>(c.max_positions) * units * (panels * sizeof(float2) + sizeof(float)));
+  off += align_up(static_cast<size_t>(c.max_positions) * (units + c.n) * ((c.v + 31) / 32) * sizeof(float));
   *off_arep = off;                      // the copy of A laid out [n, v, r, k]
   off += align_up(units * c.v * k * 2);
   *off_dec = off;                       // few-position draft: base = W_base h [P, n v] and z = B h [P, n r k], fp32
   off += align_up(static_cast<size_t>(c.max_positions < kDecodeMaxP ? c.max_positions : kDecodeMaxP) *
                   (static_cast<size_t>(c.n) * c.v + units * k) * 4);
-  *off_base = 0;                        // long drafts (more positions than that path takes): W_base h [T, n v] fp32
-  if (c.max_positions > kDecodeMaxP && c.v <= kMaxDraftVocab) {
-    *off_base = off;
-    off += align_up(static_cast<size_t>(c.max_positions) * c.n * c.v * 4);
-  }
+  *off_base = off;                      // W_base h [T, n v] fp32
+  off += align_up(static_cast<size_t>(c.max_positions) * c.n * c.v * 4);
   *off_split = off;                     // z = B h and W_base h: parts of the tiles of their last rounds
   off += align_up(kSplitBytes);
   *total = off;
@@ -1612,13 +1555,13 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   Layout L;
   int rc = plan(*cfg, &L);
   if (rc != MTPC_OK) return rc;
-  LowRankGemmParams lrp;
+  LowRankParams lrp;
   memset(&lrp, 0, sizeof(lrp));
   size_t lr_zhl = 0, lr_partial = 0, lr_arep = 0, lr_dec = 0, lr_base = 0, lr_split = 0;
   if (lowrank) {
     if (cfg->io_dtype != MTPC_BF16) return MTPC_ERR_UNSUPPORTED;
     if (!plan_lowrank(*cfg, lowrank->k, &lrp)) return MTPC_ERR_UNSUPPORTED;
-    lowrank_extra_bytes(*cfg, lowrank->k, lrp.panels, L.total, &lr_zhl, &lr_partial, &lr_arep, &lr_dec, &lr_base,
+    lowrank_extra_bytes(*cfg, lowrank->k, L.total, &lr_zhl, &lr_partial, &lr_arep, &lr_dec, &lr_base,
                         &lr_split, &L.total);
   }
   const bool ctx = (cfg->flags & MTPC_FLAG_HMM_CONTEXTUAL) != 0;
@@ -1684,13 +1627,12 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
 
   rc = bind_parameters(h, W_emit, W_sum, T_static, st);
   if (rc == MTPC_OK && lowrank) {
-    fail = !allow_full_smem(mtpc_lowrank_gemm_kernel);
-    rc = fail ? MTPC_ERR_CUDA
-              : make_tmap(&h->lr_params.tm_w, lowrank->W_base, static_cast<uint64_t>(cfg->n) * cfg->v, cfg->d,
-                          h->lr_params.panel_cols);
-    if (rc == MTPC_OK)
-      rc = make_tmap(&h->lr_params.tm_a, h->ws + h->lr_off_arep, static_cast<uint64_t>(cfg->n) * cfg->v,
-                     static_cast<uint64_t>(cfg->r) * lowrank->k, h->lr_params.chunk_cols);
+    fail = !allow_full_smem(lowrank_logits_kernel<kLowRankForward>);
+    fail |= !allow_full_smem(lowrank_logits_kernel<kLowRankGradient>);
+    if (fail) rc = MTPC_ERR_CUDA;
+    for (int mode = 0; mode < 2 && rc == MTPC_OK; ++mode)
+      rc = make_tmap(&h->lr_tm_a[mode], h->ws + h->lr_off_arep, static_cast<uint64_t>(cfg->n) * cfg->v,
+                     static_cast<uint64_t>(cfg->r) * lowrank->k, lowrank_cols(mode));
   }
   if (rc != MTPC_OK) { delete h; return rc; }
   *out = h;
@@ -1708,10 +1650,10 @@ int mtpc_lowrank_workspace_bytes(const mtpc_config* cfg, int32_t k, size_t* out_
   Layout L;
   int rc = plan(*cfg, &L);
   if (rc != MTPC_OK) return rc;
-  LowRankGemmParams lrp;
+  LowRankParams lrp;
   if (cfg->io_dtype != MTPC_BF16 || !plan_lowrank(*cfg, k, &lrp)) return MTPC_ERR_UNSUPPORTED;
   size_t a = 0, b = 0, c3 = 0, c4 = 0, c5 = 0, c6 = 0;
-  return lowrank_extra_bytes(*cfg, k, lrp.panels, L.total, &a, &b, &c3, &c4, &c5, &c6, out_bytes);
+  return lowrank_extra_bytes(*cfg, k, L.total, &a, &b, &c3, &c4, &c5, &c6, out_bytes);
 }
 
 int mtpc_create_head_lowrank(const mtpc_config* cfg, int32_t k, const void* W_base, const void* A, const void* B,
@@ -1812,7 +1754,7 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
   // then run the acceptance kernel on them. In chunks of positions whose windows fit the scratch.
   const bool factored = head->lr_k > 0;     // (a long draft on a factored head left W_base h and B h instead of needing the hidden states)
   if (L.accept_rows == 0 || (!factored && !head->draft_hidden)) return MTPC_ERR_UNSUPPORTED;
-  if (factored && head->lr_off_base == 0) return MTPC_ERR_UNSUPPORTED;
+  if (factored && c.v > kMaxDraftVocab) return MTPC_ERR_UNSUPPORTED;
   int* ints = at<int>(head, L.off_grp_ints);
   int* counts = ints, *cursors = ints + c.n, *offsets = ints + 2 * c.n, *num_tiles = ints + 3 * c.n;
   GroupTile* tiles = at<GroupTile>(head, L.off_grp_tiles);
@@ -1986,7 +1928,7 @@ int mtpc_lowrank_backward_workspace_bytes(const mtpc_config* cfg, int32_t k, int
   Layout L;
   int rc = plan(*cfg, &L);
   if (rc != MTPC_OK) return rc;
-  LowRankGemmParams lrp;
+  LowRankParams lrp;
   if (cfg->io_dtype != MTPC_BF16 || !plan_lowrank(*cfg, k, &lrp)) return MTPC_ERR_UNSUPPORTED;
   LowRankBackwardLayout R;
   plan_lowrank_backward(*cfg, L, k, T, &R);
@@ -2018,13 +1960,9 @@ int mtpc_lowrank_window_logprob_backward(mtpc_head* head, const void* hidden, co
   const void* hb = hidden;                                     // (factored heads are bf16)
   head->draft_P = 0;
   PhaseTimer pt(head, st);
-  // 1. factored forward projection, keeping every logit and every unit's log-sum-exp
+  // 1. factored forward projection, keeping every unit's log-sum-exp
   pt.begin();
-  GradArgs fwd;
-  fwd.lse_out = reinterpret_cast<float*>(bw + B.off_lse);
-  fwd.logit_out = reinterpret_cast<float*>(bw + B.off_logits);
-  fwd.logit_pitch = B.Nc;
-  rc = launch_lowrank_projection(head, hb, T, targets, st, &fwd);
+  rc = launch_lowrank_projection(head, hb, T, targets, st, reinterpret_cast<float*>(bw + B.off_lse));
   pt.end();
   if (rc != MTPC_OK) return rc;
   // 2. circuit backward: posteriors of the input units; the sum units' logit gradients go to the right of sy
@@ -2094,7 +2032,7 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   fwd.lse_out = reinterpret_cast<float*>(bw + B.off_lse);
   fwd.logit_out = reinterpret_cast<float*>(bw + B.off_logits);
   fwd.logit_pitch = B.Nc;
-  rc = factored ? launch_lowrank_projection(head, hb, T, targets, st, &fwd)
+  rc = factored ? launch_lowrank_projection(head, hb, T, targets, st, fwd.lse_out)
                 : launch_gemm(head, kModeLogprob, hb, T, 1, true, true, targets, nullptr, nullptr, st, &fwd);
   if (rc != MTPC_OK) return rc;
   loss_coeff_kernel<<<num_sequences, kLossThreads, 0, st>>>(targets, coeff, sequence_length, c.n, num_sequences, gamma);

@@ -1,30 +1,33 @@
-// Projection kernel of a head whose unembeddings are shared across the components of a slot and adapted by low-rank
-// terms (App. G): U_ij = W_i + A_ij B_ij, so logit[t, i, j, :] = W_i h_t + A_ij (B_ij h_t). The composed [n, r, v, d]
-// tensor is never formed. A unit's v columns are cut into `panels` panels of panel_cols columns (the last one may be
-// narrower); a work item is (128 positions, slot i, panel):
-//   base    = h W_i^T            the panel's columns of the one weight-sized-over-r contraction (K = d), accumulated into one
-//                                of TWO tensor-memory buffers, so that the next item's base runs while this item's
-//                                corrections and epilogue are under way;
-//   corr_j  = z_j A_ij^T         for each of the r components one K = 2k contraction on z_j = B_ij h (computed by a plain
-//                                GEMM beforehand whose epilogue splits it into two bf16 halves, z = hi + lo, so that rounding z to
-//                                the tensor cores' operand type costs 2^-17 instead of 2^-9), in chunks of chunk_cols columns
-//                                through two accumulator slots per epilogue group;
-//   epilogue: x = base + corr_j, then the log-likelihood epilogue of the dense kernel on the panel (online log-sum-exp,
-//             target gather). One panel: G = logit[target] - LSE directly. Several: every panel leaves (max, sum of
-//             exponentials) per (position, slot, component), the panel that holds the target leaves its logit, and
-//             lowrank_merge_kernel combines them - so the items are independent and deal out evenly.
-// FLOPs per position: 2 d (n v + n r k) + 4 n r v k instead of 2 d n r v.
-// Roles: warp 0 TMA producer of the base operands, warp 1 MMA issuer of the base, warp 2 TMA producer of the correction
-// operands, warps 3 .. 2 + groups one MMA issuer of corrections per epilogue group (issuing one of these small MMAs holds
-// its thread for a few hundred cycles although the tensor pipe is nearly idle: the issuers must not queue behind each
-// other), then from warp 8 on `groups` epilogue groups of four warps (one thread per position): group g takes the
-// components j = g, g + groups, ... The two pipelines share nothing but the tensor cores: each has its
-// own shared-memory ring and its own barriers. Base ring: a 64-wide K block of h and of the panel's rows of W_i. Correction
-// ring: one entry holds the operands of 64 / k components, all as 128-byte rows with the 128-byte swizzle (few large boxes
-// instead of many 32-byte-row ones): z as boxes of 128 positions x 64 values = [hi | lo] of 32 / k adjacent
-// components, and A as boxes of chunk_cols vocabulary rows x 64 values = the k adaptor columns of 64 / k adjacent components,
-// read from a copy of A laid out [n, v, r, k] (lowrank_repack_kernel, made on every call: A is small and may have changed).
-// A correction MMA (K = 16) addresses its operands inside those rows, 32 bytes apart, like the K steps of the base.
+// Projection of a head whose unembeddings are shared across the components of a slot and adapted by low-rank terms (App. G):
+// U_ij = W_i + A_ij B_ij, so logit[t, i, j, :] = W_i h_t + A_ij (B_ij h_t). The composed [n, r, v, d] tensor is never formed.
+// Two plain GEMMs make base = W_base h [T, n v] (fp32) and z = B h [T, n r, 2, k] (two bf16 halves, z = hi + lo, so that
+// rounding z to the tensor cores' operand type costs 2^-17 instead of 2^-9); lowrank_logits_kernel does the rest without
+// writing a logit. FLOPs per position: 2 d (n v + n r k) + 4 n r v k instead of 2 d n r v.
+//
+// A work item is (128 positions, slot i, 128 or 64 columns b of the vocabulary). A thread of the epilogue keeps the base logits
+// of one position and 32 columns in registers and walks the slot's r components: corr_j = z_j A_ij^T for the item's columns
+// comes out of tensor memory (K = 2k: [hi | lo] against A twice), x = base + corr_j, and then
+//   forward   (kLowRankForward): the log-sum-exp of the 32 columns, combined over the item's columns through shared memory;
+//             lowrank_merge_kernel combines the column blocks, forms the target's logit and writes G. The reference of the
+//             exponentials is the base logits' maximum, known before the walk; a component whose sum leaves [2^-60, 2^120]
+//             against it (corrections of many tens) is redone with its own maximum;
+//   gradient  (kLowRankGradient): g = post (onehot(target) - exp(x - lse)) as bf16, the operand of the GEMMs of the training
+//             call, and sum_j g_ij - so a training call keeps no logits ([T, n r v] fp32 were written and read back) and needs
+//             no pass over g for that sum.
+// Why this shape: with the components outermost (base logits and a running maximum re-read from tensor memory per component,
+// corrections in chunks of <= 48 columns) the kernel was bound by its corrections: a dependent pair of M = 128, N <= 48 MMAs
+// costs about 320 cycles against 24 of arithmetic, and the columns of a component waited for each other through the maximum.
+// Here MMAs are 64 or 128 columns wide, two components' pairs alternate, 512 columns of accumulators are in flight, and no
+// (component, 32 columns) depends on another. The bound is one ex2 per logit (16 a clock and SM: 149 us at T = 8192, n = 8,
+// r = 32, v = 320), in the gradient also the 1.3 GB of g.
+// Measured (this kernel, forward / gradient): 280 / 444 us, where the fused projection that kept logits took 801 us and the
+// passes that made g and its sum from them 921 us; a likelihood call's whole projection at T = 8192, v = 320, d = 4096: r = 16
+// 506 -> 438 us, r = 32 893 -> 673 us.
+// Roles: warp 0 TMA producer, warp 1 MMA issuer, then the epilogue warps (TMEM quarter warp % 4, columns 32 * ((warp - 2) / 4)).
+// Operand ring: one entry holds 64 / k components, all as 128-byte rows with the 128-byte swizzle: z as two boxes of 128
+// positions x 64 values ([hi | lo] of 32 / k adjacent components each), and A as one box of the item's vocabulary rows x 64 values (the k
+// adaptor columns of 64 / k adjacent components) of a copy laid out [n, v, r, k] (lowrank_repack_kernel, made on every call: A is
+// small and may have changed).
 #pragma once
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -36,119 +39,98 @@
 namespace mtpc {
 
 constexpr int kLrMaxRank = 32;          // k <= 32 (a multiple of 16)
-constexpr int kLrMaxGroups = 2;         // epilogue groups: 256 + 128 * groups threads per CTA (512: 128 registers each)
-constexpr int kLrMaxPanels = 8;
-constexpr int kLrCorrStages = 4;        // entries of the correction operand ring (at most)
-constexpr int kLrRoleThreads = 256;     // the single-thread roles, one warp each: warps 0 .. 2 + groups (the rest idle)
+constexpr int kLrMaxVocab = 1792;
+constexpr int kLrStages = 2;
+constexpr int kLrRoleWarps = 2;
+constexpr int kLrJ = 16;                // components per round of an epilogue warp's shared-memory patches
+constexpr int kLrPitch = 33;            // pitch of a component's 32 positions there (read across components without conflicts)
+enum { kLowRankForward = 0, kLowRankGradient = 1 };
+// Columns of a work item (an epilogue warp takes 32 of them). The gradient keeps a second register per column (the sum over the
+// components): 64 columns, eight epilogue warps and 168 registers a thread; with sixteen warps and 96 it spilled or could not
+// have the next accumulators in flight.
+__host__ __device__ constexpr int lowrank_cols(int mode) { return mode == kLowRankForward ? 128 : 64; }
+__host__ __device__ constexpr int lowrank_subs(int mode) { return lowrank_cols(mode) / 32; }
+__host__ __device__ constexpr int lowrank_threads(int mode) { return 32 * kLrRoleWarps + 128 * lowrank_subs(mode); }
+__host__ __device__ constexpr int lowrank_stage_bytes(int mode) { return 2 * kBlockM * 128 + lowrank_cols(mode) * 128; }
 
-struct LowRankGemmParams {
-  CUtensorMap tm_h;      // hidden [T, d]              box 64 x 128, 128-byte swizzle
-  CUtensorMap tm_w;      // W_base [n*v, d]            box 64 x panel_cols, 128-byte swizzle
+struct LowRankParams {
   CUtensorMap tm_z;      // z      [T, n*r*2*k]        box 64 x 128, 128-byte swizzle (unit u: hi at (2u)k, lo at (2u+1)k)
-  CUtensorMap tm_a;      // A'     [n*v, r*k]          box 64 x chunk_cols, 128-byte swizzle (row (i, b): A[i, 0..r-1, b, :])
-  int T, m_tiles, kblocks;
-  int n, r, v, vv, k;
-  int panels, panel_cols;            // panel q covers the columns [q panel_cols, min(v, (q + 1) panel_cols)) of a unit
-  int acc_stride;                    // tensor-memory columns between the two base buffers (panel_cols rounded up to 32)
-  int chunk_cols, nchunk;            // correction chunks of a full panel: nchunk = ceil(panel_cols / chunk_cols)
-  int corr_col0;                     // first tensor-memory column of correction slot 0 (slot s follows at + s * chunk_cols)
-  int groups;                        // epilogue groups (1 .. kLrMaxGroups), each with two correction slots of chunk_cols columns
-  int base_stages, base_stage_bytes, corr_stages, corr_stage_bytes;
-  const int* targets;                // [T, n]
-  float* G;                          // [T, n, r]
-  float2* partial;                   // panels > 1: [panels, T n r] (running maximum, sum of exponentials) of each panel
-  float* target_logit;               // panels > 1: [T n r] logit of the target, written by the panel that holds it
-  float* logit_out;                  // training: every logit [T, n r v] fp32 at a pitch of logit_pitch (NULL: not kept) ...
-  size_t logit_pitch;
-  float* lse_out;                    // ... and every unit's log-sum-exp [T, n r] (with several panels: by the merge kernel)
-  int missing_is_nan;                // the targets are drafted bytes: -1 is a refused draw (G = NaN), not a marginalised byte (G = 0)
+  CUtensorMap tm_a;      // A'     [n*v, r*k]          box 64 x lowrank_cols, 128-byte swizzle (row (i, b): A[i, 0..r-1, b, :])
+  int T, m_tiles, n, r, v, vv, k;
+  int blocks;                        // column blocks of a unit
+  const float* base;                 // [T, n v]
+  float* log_sum;                    // forward: [ceil(v / 32), T n r] log2 of the sum of exponentials of 32 columns, relative to
+  float* ref;                        //          [ceil(v / 32), T n] the maximum of their base logits
+  const int* targets;                // gradient: [T, n]
+  const float* G;                    // gradient: [T, n, r] log phi at the target,
+  const float* lse;                  //           [T, n, r] log-sum-exp of every unit,
+  const float* post;                 //           [T, n, r] its weighted posterior
+  __nv_bfloat16* g;                  //           [T, n r v] at a pitch of g_pitch
+  size_t g_pitch;
+  __nv_bfloat16* s;                  //           [T, n v] at a pitch of s_pitch: g summed over a slot's components
+  size_t s_pitch;
   unsigned* status;
   uint64_t wait_limit_ns;
 };
-
-struct LowRankControl {
-  GemmControl g;                     // full / empty: base ring; tfull / tempty: correction slots; abort, limits, tmem_base
-  uint64_t cfull[kLrCorrStages];     // correction operand ring
-  uint64_t cempty[kLrCorrStages];
-  uint64_t afull[2];                 // base accumulators
-  uint64_t aempty[2];
-  uint64_t drain2[kLrMaxGroups];
-};
-
-// Wait (bounded) until the copies a producer still has in flight have landed: no copy may be in flight when the CTA goes.
-__device__ __forceinline__ void lowrank_drain_ring(uint64_t* full, int stages, uint32_t issued_mask, uint32_t phase_mask) {
-  for (int s = 0; s < stages; ++s)
-    if (issued_mask & (1u << s)) {
-      const uint32_t bar = smem_u32(&full[s]);
-      const uint32_t par = (phase_mask >> s) & 1u;
-      const uint64_t t0 = global_timer_ns();
-      while (!mbar_try_wait(bar, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
-    }
+// Shared memory of an epilogue warp behind the ring, in floats: the next item's base logits [32 positions][32 columns] (16-byte
+// pieces swizzled by the position); forward: log-sums [kLrJ][kLrPitch]; gradient: two rounds of lse, weight and G, each
+// [kLrJ][kLrPitch]. Nothing is shared between epilogue warps: with block-wide staging and barriers a sixth (forward) to nearly
+// half (gradient) of the time went into the boundaries between items.
+__host__ __device__ constexpr int lowrank_warp_floats(int mode) {
+  return 1024 + (mode == kLowRankForward ? 1 : 6) * kLrJ * kLrPitch;
+}
+inline size_t lowrank_smem_bytes(int mode) {
+  return 1024 + static_cast<size_t>(kLrStages) * lowrank_stage_bytes(mode) + 4 * lowrank_subs(mode) * lowrank_warp_floats(mode) * sizeof(float) +
+         sizeof(GemmControl);
 }
 
 struct LowRankItem {
-  int mt, slot, panel;
-  int width;     // columns of this panel (the last panel of a unit may be narrower), a multiple of 16
-  int nchunk;    // correction chunks that cover them
+  int mt, slot, block, width;     // width: columns of this block (a multiple of 16)
 };
-// panel fastest, then slot: the CTAs that run together share the hidden tile (and the slot's W_i) through L2
-__device__ __forceinline__ LowRankItem lowrank_item(const LowRankGemmParams& p, int item) {
+// column block fastest: the CTAs that run together share the positions' z through L2
+template <int COLS>
+__device__ __forceinline__ LowRankItem lowrank_item(const LowRankParams& p, int item) {
   LowRankItem c;
-  c.panel = item % p.panels;
-  const int rest = item / p.panels;
+  c.block = item % p.blocks;
+  const int rest = item / p.blocks;
   c.slot = rest % p.n;
   c.mt = rest / p.n;
-  c.width = min(p.panel_cols, p.v - c.panel * p.panel_cols);
-  c.nchunk = (c.width + p.chunk_cols - 1) / p.chunk_cols;
+  c.width = min(COLS, p.v - c.block * COLS);
   return c;
 }
 
-__global__ void __launch_bounds__(kLrRoleThreads + 128 * kLrMaxGroups, 1)
-mtpc_lowrank_gemm_kernel(const __grid_constant__ LowRankGemmParams p) {
+template <int MODE>
+__global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kernel(const __grid_constant__ LowRankParams p) {
+  constexpr int kCols = lowrank_cols(MODE), kSubs = lowrank_subs(MODE), kSlots = kTmemCols / kCols;
+  constexpr int kStageBytes = lowrank_stage_bytes(MODE);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
-  const uint32_t base_ring = (raw_addr + 1023u) & ~1023u;
-  const uint32_t corr_ring = base_ring + static_cast<uint32_t>(p.base_stages * p.base_stage_bytes);
-  uint8_t* tiles = smem_raw + (base_ring - raw_addr);
-  LowRankControl* lc = reinterpret_cast<LowRankControl*>(tiles + static_cast<size_t>(p.base_stages) * p.base_stage_bytes +
-                                                         static_cast<size_t>(p.corr_stages) * p.corr_stage_bytes);
-  GemmControl* ctl = &lc->g;
+  const uint32_t ring = (raw_addr + 1023u) & ~1023u;
+  float* patches = reinterpret_cast<float*>(smem_raw + (ring - raw_addr) + kLrStages * kStageBytes);
+  GemmControl* ctl = reinterpret_cast<GemmControl*>(patches + 4 * kSubs * lowrank_warp_floats(MODE));
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int num_items = p.m_tiles * p.n * p.panels;
+  const int num_items = p.m_tiles * p.n * p.blocks;
   const int kq = p.k / 16;                                // K = 16 steps of one half of a correction
-  const int ca = 64 / p.k;                                // components per correction entry (= per box of A')
+  const int ca = 64 / p.k;                                // components per ring entry (= per box of A')
   const int cz = 32 / p.k;                                // components per box of z; an entry has ca / cz = 2 of them
-  const int nent = (p.r + ca - 1) / ca;                   // correction entries per item
-  const uint32_t zbox = kBlockM * 128;                    // bytes of one z box (128 rows x 128 bytes)
-  const uint32_t abox = static_cast<uint32_t>(p.chunk_cols) * 128;
-  const uint32_t a_off = 2 * zbox;                        // correction entry: [z box 0 | z box 1 | A' boxes c = 0 .. nchunk - 1]
+  const int nent = (p.r + ca - 1) / ca;                   // ring entries per item
+  constexpr uint32_t kZBox = kBlockM * 128;               // bytes of one z box
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < p.base_stages; ++s) {
+    for (int s = 0; s < kLrStages; ++s) {
       mbar_init(smem_u32(&ctl->full[s]), 1);
       mbar_init(smem_u32(&ctl->empty[s]), 1);
     }
-    for (int s = 0; s < p.corr_stages; ++s) {
-      mbar_init(smem_u32(&lc->cfull[s]), 1);
-      mbar_init(smem_u32(&lc->cempty[s]), p.groups);        // every correction issuer hands an entry back
-    }
-    for (int s = 0; s < 2 * p.groups; ++s) {
+    for (int s = 0; s < kSlots; ++s) {
       mbar_init(smem_u32(&ctl->tfull[s]), 1);
-      mbar_init(smem_u32(&ctl->tempty[s]), 4);
-    }
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(smem_u32(&lc->afull[s]), 1);
-      mbar_init(smem_u32(&lc->aempty[s]), 4 * p.groups);
+      mbar_init(smem_u32(&ctl->tempty[s]), 4 * kSubs);
     }
     mbar_init(smem_u32(&ctl->drain), 1);
-    for (int g = 0; g < p.groups; ++g) mbar_init(smem_u32(&lc->drain2[g]), 1);
     ctl->abort = 0;
     ctl->wait_limit_ns = p.wait_limit_ns;
     fence_mbar_init();
-    tma_prefetch_desc(&p.tm_h);
-    tma_prefetch_desc(&p.tm_w);
     tma_prefetch_desc(&p.tm_z);
     tma_prefetch_desc(&p.tm_a);
   }
@@ -162,55 +144,77 @@ mtpc_lowrank_gemm_kernel(const __grid_constant__ LowRankGemmParams p) {
   const uint32_t tmem_base = ctl->tmem_base;
 
   if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer, base operands
+    // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0;
+      uint32_t st = 0, phase = 0, issued_mask = 0, phase_mask = 0;
       bool ok = true;
-      const uint32_t bytes = kABytes + static_cast<uint32_t>(p.panel_cols) * (kBlockK * 2);
       for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-        const LowRankItem w = lowrank_item(p, item);
-        for (int kb = 0; kb < p.kblocks; ++kb) {
-          if (!bounded_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
-          const uint32_t full = smem_u32(&ctl->full[stage]);
-          const uint32_t dst = base_ring + stage * p.base_stage_bytes;
-          mbar_arrive_expect_tx(full, bytes);
-          tma_load_2d(dst, &p.tm_h, full, kb * kBlockK, w.mt * kBlockM);
-          // the box is panel_cols rows high also for a narrower last panel: the rows past it (the next slot's, or
-          // zeros past the end of W_base) are not multiplied
-          tma_load_2d(dst + kABytes, &p.tm_w, full, kb * kBlockK, w.slot * p.v + w.panel * p.panel_cols);
-          issued_mask |= 1u << stage;
-          phase_mask = (phase_mask & ~(1u << stage)) | (phase << stage);
-          if (++stage == static_cast<uint32_t>(p.base_stages)) { stage = 0; phase ^= 1u; }
+        const LowRankItem w = lowrank_item<kCols>(p, item);
+        for (int e = 0; e < nent; ++e) {
+          if (!bounded_wait(smem_u32(&ctl->empty[st]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
+          const uint32_t full = smem_u32(&ctl->full[st]);
+          const uint32_t dst = ring + st * kStageBytes;
+          const int unit0 = w.slot * p.r + e * ca;           // first component of the entry
+          mbar_arrive_expect_tx(full, kStageBytes);
+          // boxes may cover components past the slot's last (the next slot's, or zeros past the end) and, for A', rows past
+          // the unit: none of that is multiplied
+          for (int bx = 0; bx < 2; ++bx)
+            tma_load_2d(dst + bx * kZBox, &p.tm_z, full, (unit0 + bx * cz) * 2 * p.k, w.mt * kBlockM);
+          tma_load_2d(dst + 2 * kZBox, &p.tm_a, full, e * ca * p.k, w.slot * p.v + w.block * kCols);
+          issued_mask |= 1u << st;
+          phase_mask = (phase_mask & ~(1u << st)) | (phase << st);
+          if (++st == kLrStages) { st = 0; phase ^= 1u; }
         }
       }
-      lowrank_drain_ring(ctl->full, p.base_stages, issued_mask, phase_mask);
+      // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
+      for (int s = 0; s < kLrStages; ++s)
+        if (issued_mask & (1u << s)) {
+          const uint32_t bar = smem_u32(&ctl->full[s]);
+          const uint32_t par = (phase_mask >> s) & 1u;
+          const uint64_t t0 = global_timer_ns();
+          while (!mbar_try_wait(bar, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
+        }
     }
     __syncwarp();
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer, base: item `it` into buffer it & 1
+    // ------------------------------------------------------------------ MMA issuer: component u overall into slot u % kSlots
     if (lane == 0) {
-      uint32_t stage = 0, phase = 0, it = 0;
+      uint32_t st = 0, phase = 0, use = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x, ++it) {
-        const uint32_t idesc = umma_idesc_bf16(kBlockM, lowrank_item(p, item).width);
-        const uint32_t buf = it & 1u;
-        if (!bounded_wait(smem_u32(&lc->aempty[buf]), ((it >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + buf * p.acc_stride;
-        for (int kb = 0; kb < p.kblocks; ++kb) {
-          if (!bounded_wait(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
+      for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
+        const LowRankItem w = lowrank_item<kCols>(p, item);
+        const uint32_t idesc = umma_idesc_bf16(kBlockM, w.width);
+        for (int e = 0; e < nent && ok; ++e) {
+          if (!bounded_wait(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t addr = base_ring + stage * p.base_stage_bytes;
-          const uint64_t a_desc = umma_smem_desc_sw128(addr);
-          const uint64_t b_desc = umma_smem_desc_sw128(addr + kABytes);
-#pragma unroll
-          for (int kk = 0; kk < kBlockK / 16; ++kk)
-            umma_bf16(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
-          umma_commit(smem_u32(&ctl->empty[stage]));
-          if (++stage == static_cast<uint32_t>(p.base_stages)) { stage = 0; phase ^= 1u; }
+          const uint32_t entry = ring + st * kStageBytes;
+          const int count = min(ca, p.r - e * ca);
+          for (int l = 0; l < count && ok; l += 2) {
+            const int pair = min(2, count - l);
+            uint64_t z_desc[2], a_desc[2];
+            uint32_t d_tmem[2];
+            for (int q = 0; q < pair; ++q) {
+              // descriptors step in 16-byte units: the component's [hi | lo] inside its z box, its k columns inside the A' box
+              z_desc[q] = umma_smem_desc_sw128(entry + ((l + q) / cz) * kZBox) + (((l + q) % cz) * 2 * p.k) / 8;
+              a_desc[q] = umma_smem_desc_sw128(entry + 2 * kZBox) + ((l + q) * p.k) / 8;
+              const uint32_t slot = (use + q) % kSlots;
+              d_tmem[q] = tmem_base + slot * kCols;
+              if (!bounded_wait(smem_u32(&ctl->tempty[slot]), (((use + q) / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+            }
+            if (!ok) break;
+            tc_fence_after();
+            // the two components alternate, so that an MMA does not follow the one whose result it adds to
+            for (int part = 0; part < 2; ++part)
+              for (int kk = 0; kk < kq; ++kk)
+                for (int q = 0; q < pair; ++q)
+                  umma_bf16(d_tmem[q], z_desc[q] + (part * p.k + 16 * kk) / 8, a_desc[q] + (16 * kk) / 8, idesc, (part | kk) != 0 ? 1u : 0u);
+            for (int q = 0; q < pair; ++q) umma_commit(smem_u32(&ctl->tfull[(use + q) % kSlots]));
+            use += pair;
+          }
+          if (!ok) break;
+          umma_commit(smem_u32(&ctl->empty[st]));
+          if (++st == kLrStages) { st = 0; phase ^= 1u; }
         }
-        if (!ok) break;
-        umma_commit(smem_u32(&lc->afull[buf]));
       }
       if (!ok || ctl->abort) {   // wait (bounded) for the MMAs already issued before tensor memory is freed
         umma_commit(smem_u32(&ctl->drain));
@@ -219,199 +223,226 @@ mtpc_lowrank_gemm_kernel(const __grid_constant__ LowRankGemmParams p) {
       }
     }
     __syncwarp();
-  } else if (warp == 2) {
-    // ------------------------------------------------------------------ TMA producer, correction operands
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0;
-      bool ok = true;
-      const uint32_t bytes = 2 * zbox + static_cast<uint32_t>(p.nchunk) * abox;
-      for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-        const LowRankItem w = lowrank_item(p, item);
-        for (int e = 0; e < nent; ++e) {
-          if (!bounded_wait(smem_u32(&lc->cempty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
-          const uint32_t full = smem_u32(&lc->cfull[stage]);
-          const uint32_t dst = corr_ring + stage * p.corr_stage_bytes;
-          const int unit0 = w.slot * p.r + e * ca;           // first component of the entry
-          mbar_arrive_expect_tx(full, bytes);
-          // boxes may cover components past the slot's last (the next slot's, or zeros past the end) and, for A',
-          // rows past the panel: none of that is multiplied
-          for (int bx = 0; bx < 2; ++bx)
-            tma_load_2d(dst + bx * zbox, &p.tm_z, full, (unit0 + bx * cz) * 2 * p.k, w.mt * kBlockM);
-          for (int c = 0; c < p.nchunk; ++c)
-            tma_load_2d(dst + a_off + c * abox, &p.tm_a, full, e * ca * p.k,
-                        w.slot * p.v + w.panel * p.panel_cols + c * p.chunk_cols);
-          issued_mask |= 1u << stage;
-          phase_mask = (phase_mask & ~(1u << stage)) | (phase << stage);
-          if (++stage == static_cast<uint32_t>(p.corr_stages)) { stage = 0; phase ^= 1u; }
-        }
-      }
-      lowrank_drain_ring(lc->cfull, p.corr_stages, issued_mask, phase_mask);
-    }
-    __syncwarp();
-  } else if (warp >= 3 && warp < 3 + p.groups) {
-    // ------------------------------------------------------------------ MMA issuer of the corrections of one epilogue
-    // group: its components in turn, chunk c of the group's u-th chunk overall into slot 2 g + (u & 1)
-    if (lane == 0) {
-      const int g = warp - 3;
-      uint32_t stage = 0, phase = 0, cuse = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-        const LowRankItem w = lowrank_item(p, item);
-        for (int e = 0; e < nent && ok; ++e) {
-          if (!bounded_wait(smem_u32(&lc->cfull[stage]), phase, ctl, p.status)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t entry = corr_ring + stage * p.corr_stage_bytes;
-          for (int l = 0; l < ca && ok; ++l) {
-            const int j = e * ca + l;
-            if (j >= p.r) break;
-            if (j % p.groups != g) continue;
-            // descriptors step in 16-byte units: the component's [hi | lo] inside its z box, its k columns inside the A' box
-            const uint64_t z_desc = umma_smem_desc_sw128(entry + (l / cz) * zbox) + ((l % cz) * 2 * p.k) / 8;
-            for (int c = 0; c < w.nchunk; ++c, ++cuse) {
-              const int width = min(p.chunk_cols, w.width - c * p.chunk_cols);
-              const uint32_t idesc = umma_idesc_bf16(kBlockM, width);
-              const uint64_t a_desc = umma_smem_desc_sw128(entry + a_off + c * abox) + (l * p.k) / 8;
-              const uint32_t slot = 2 * g + (cuse & 1u);
-              if (!bounded_wait(smem_u32(&ctl->tempty[slot]), ((cuse >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
-              tc_fence_after();
-              const uint32_t d_tmem = tmem_base + p.corr_col0 + slot * p.chunk_cols;
-              uint32_t acc = 0;
-              for (int part = 0; part < 2; ++part)
-                for (int q = 0; q < kq; ++q) {
-                  umma_bf16(d_tmem, z_desc + (part * p.k + 16 * q) / 8, a_desc + (16 * q) / 8, idesc, acc);
-                  acc = 1;
-                }
-              umma_commit(smem_u32(&ctl->tfull[slot]));
-            }
-          }
-          if (!ok) break;
-          umma_commit(smem_u32(&lc->cempty[stage]));           // (also for an entry none of whose components are this group's)
-          if (++stage == static_cast<uint32_t>(p.corr_stages)) { stage = 0; phase ^= 1u; }
-        }
-      }
-      if (!ok || ctl->abort) {
-        umma_commit(smem_u32(&lc->drain2[g]));
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(smem_u32(&lc->drain2[g]), 0) && global_timer_ns() - t0 < kWaitLimitNs) {}
-      }
-    }
-    __syncwarp();
-  } else if (warp >= kLrRoleThreads / 32) {
+  } else {
     // ------------------------------------------------------------------ epilogue
     const int quarter = warp & 3;
-    const int group = (warp - kLrRoleThreads / 32) >> 2;      // this warp's epilogue group: components group, group + groups, ...
-    const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-    const size_t entries = static_cast<size_t>(p.T) * p.n * p.r;
-    uint32_t it = 0, cuse = 0;
+    const int sub = (warp - kLrRoleWarps) >> 2;
+    const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + sub * 32;
+    const size_t units = static_cast<size_t>(p.n) * p.r;
+    const float2 l2 = make_float2(kLog2e, kLog2e);
+    float* next_base = patches + (warp - kLrRoleWarps) * lowrank_warp_floats(MODE);
+    float* patch = next_base + 1024;
+    // ---- copies that are in flight while the current item or round is worked on
+    auto fetch_base = [&](int item) {                      // base logits of the warp's 32 positions x 32 columns
+      if (item < num_items) {
+        const LowRankItem w = lowrank_item<kCols>(p, item);
+        const int col0 = w.block * kCols + sub * 32, ch = lane & 7;
+        if (col0 + ch * 4 < p.v) {
+#pragma unroll
+          for (int it = 0; it < 8; ++it) {
+            const int rr = it * 4 + (lane >> 3);
+            const int t = min(w.mt * kBlockM + quarter * 32 + rr, p.T - 1);
+            cp_async_16(next_base + rr * 32 + ((ch ^ (rr & 7)) * 4),
+                        p.base + static_cast<size_t>(t) * p.n * p.v + static_cast<size_t>(w.slot) * p.v + col0 + ch * 4);
+          }
+        }
+      }
+    };
+    auto fetch_round = [&](int item, int j0, float* dst) { // gradient: lse, weight and G of 32 positions x kLrJ components
+      if (item < num_items) {
+        const LowRankItem w = lowrank_item<kCols>(p, item);
+        const int jj = lane & (kLrJ - 1);
+        if (j0 + jj < p.r) {
+          for (int it = 0; it < 16; ++it) {
+            const int rr = it * 2 + (lane >> 4);
+            const int t = min(w.mt * kBlockM + quarter * 32 + rr, p.T - 1);
+            const size_t tu = static_cast<size_t>(t) * units + static_cast<size_t>(w.slot) * p.r + j0 + jj;
+            float* d = dst + jj * kLrPitch + rr;
+            cp_async_4(d, p.lse + tu);
+            cp_async_4(d + kLrJ * kLrPitch, p.post + tu);
+            cp_async_4(d + 2 * kLrJ * kLrPitch, p.G + tu);
+          }
+        }
+      }
+    };
+    uint32_t use = 0, round = 0;
     bool ok = true;
-    for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x, ++it) {
-      const LowRankItem w = lowrank_item(p, item);
-      const int row = w.mt * kBlockM + quarter * 32 + lane;
+    // (every lane polls: no broadcast of the outcome, one vote)
+    auto wait_slot = [&](uint32_t u) -> bool {
+      return __all_sync(kFull, bounded_wait(smem_u32(&ctl->tfull[u % kSlots]), (u / kSlots) & 1u, ctl, p.status));
+    };
+    fetch_base(blockIdx.x);
+    if (MODE == kLowRankGradient) fetch_round(blockIdx.x, 0, patch);
+    cp_async_commit();
+    for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
+      const LowRankItem w = lowrank_item<kCols>(p, item);
+      const int row0 = w.mt * kBlockM + quarter * 32, row = row0 + lane;
       const bool valid = row < p.T;
-      const int tgt = valid ? p.targets[static_cast<size_t>(row) * p.n + w.slot] : -1;
-      const int panel_col0 = w.panel * p.panel_cols;
-      const uint32_t buf = it & 1u;
-      if (!bounded_wait_warp(smem_u32(&lc->afull[buf]), (it >> 1) & 1u, ctl, p.status, lane)) { ok = false; break; }
-      tc_fence_after();
-      const uint32_t bcol = lane_base + buf * p.acc_stride;
-      for (int j = group; j < p.r && ok; j += p.groups) {
-        float m = -CUDART_INF_F, s = 0.f, tval = 0.f;
-        for (int c = 0; c < w.nchunk; ++c, ++cuse) {
-          const uint32_t slot = 2 * group + (cuse & 1u);
-          if (!bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (cuse >> 1) & 1u, ctl, p.status, lane)) { ok = false; break; }
-          tc_fence_after();
-          const int col_chunk = c * p.chunk_cols;             // first column of the chunk inside the panel
-          const int width = min(p.chunk_cols, w.width - col_chunk);
-          const uint32_t ccol = lane_base + p.corr_col0 + slot * p.chunk_cols;
-          // one batch of 16 columns: correction + base, then the dense kernel's online log-sum-exp and target gather
-          auto consume = [&](const uint32_t (&rc)[16], const uint32_t (&rb)[16], int b) {
-            float x[16];
+      const int col0 = w.block * kCols + sub * 32;         // this warp's first column inside the unit
+      const int here = min(32, p.v - col0);                // its columns: 32, 16 or none (<= 0)
+      float2 base[16];                                     // (base - ref) log2(e); ref: their maximum (forward) or 0
+      float ref = -CUDART_INF_F;
+      cp_async_wait<0>();
+      __syncwarp();
 #pragma unroll
-            for (int q = 0; q < 16; ++q) x[q] = __uint_as_float(rc[q]) + __uint_as_float(rb[q]);
-            const int col0 = panel_col0 + col_chunk + b * 16; // column inside the unit
-            mask_padding(x, col0, p.vv);
-            if (p.logit_out != nullptr && valid) {            // row of the logit matrix: (slot, component, symbol)
-              float* l = p.logit_out + static_cast<size_t>(row) * p.logit_pitch + (static_cast<size_t>(w.slot) * p.r + j) * p.v + col0;
-              st_global_v8(l, x);
-              st_global_v8(l + 8, x + 8);
+      for (int q = 0; q < 8; ++q) {
+        float4 x = *reinterpret_cast<const float4*>(next_base + lane * 32 + ((q ^ (lane & 7)) * 4));
+        if (col0 + 4 * q + 4 > p.vv) {                     // padding columns, and columns past the unit, carry no mass
+          if (col0 + 4 * q >= p.vv) x.x = -CUDART_INF_F;
+          if (col0 + 4 * q + 1 >= p.vv) x.y = -CUDART_INF_F;
+          if (col0 + 4 * q + 2 >= p.vv) x.z = -CUDART_INF_F;
+          if (col0 + 4 * q + 3 >= p.vv) x.w = -CUDART_INF_F;
+        }
+        base[2 * q] = make_float2(x.x, x.y);
+        base[2 * q + 1] = make_float2(x.z, x.w);
+        ref = fmaxf(ref, fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
+      }
+      if (MODE == kLowRankGradient || ref == -CUDART_INF_F) ref = 0.f;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) base[q] = make_float2((base[q].x - ref) * kLog2e, (base[q].y - ref) * kLog2e);
+      __syncwarp();
+      fetch_base(item + gridDim.x);
+      float2 sum[16];                                      // gradient: sum over the components,
+      float hot = 0.f;                                     // and of the weights, for the target's column
+      int rel = -1;
+      bool has_target = false;
+      if constexpr (MODE == kLowRankGradient) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) sum[q] = make_float2(0.f, 0.f);
+        const int tgt = valid ? p.targets[static_cast<size_t>(row) * p.n + w.slot] : -1;
+        has_target = tgt >= 0;                             // a marginalised byte has no gradient
+        rel = (tgt >= col0 && tgt < col0 + 32) ? tgt - col0 : -1;
+      } else {
+        cp_async_commit();
+        if (valid && here > 0) p.ref[static_cast<size_t>(col0 / 32) * p.T * p.n + static_cast<size_t>(row) * p.n + w.slot] = ref;
+      }
+      for (int j0 = 0; j0 < p.r; j0 += kLrJ, ++round) {
+        const int jc = min(kLrJ, p.r - j0);                // a power of two
+        const float* mine = patch + (round & 1) * (3 * kLrJ * kLrPitch);    // gradient: this round's
+        if constexpr (MODE == kLowRankGradient) {
+          if (j0 > 0) {
+            cp_async_wait<0>();
+            __syncwarp();
+          }
+          const bool last = j0 + kLrJ >= p.r;              // the next round: of this item or of the next one
+          fetch_round(last ? item + gridDim.x : item, last ? 0 : j0 + kLrJ, patch + ((round + 1) & 1) * (3 * kLrJ * kLrPitch));
+          cp_async_commit();
+        }
+        // The accumulators of a component in two halves of sixteen columns: the second half is on its way while the first is
+        // consumed, the next component's first half while the second is.
+        uint32_t ca0[16], ca1[16];
+        if (!(ok = wait_slot(use))) break;
+        tc_fence_after();
+        tmem_ld16_issue(lane_base + (use % kSlots) * kCols, ca0);
+        for (int jj = 0; jj < jc; ++jj, ++use) {
+          const uint32_t col = lane_base + (use % kSlots) * kCols;
+          tmem_ld_wait16(ca0);
+          tmem_ld16_issue(col + 16, ca1);                  // (columns past the block's width are not used)
+          float2 sa = make_float2(0.f, 0.f), sb = sa;
+          float lse2 = 0.f, wt = 0.f;
+          __nv_bfloat16* dst = nullptr;
+          if constexpr (MODE == kLowRankGradient) {
+            lse2 = mine[jj * kLrPitch + lane] * kLog2e;
+            wt = has_target ? mine[(kLrJ + jj) * kLrPitch + lane] : 0.f;
+            hot += wt;
+            dst = p.g + static_cast<size_t>(valid ? row : 0) * p.g_pitch + (static_cast<size_t>(w.slot) * p.r + j0 + jj) * p.v + col0;
+          }
+          auto eat = [&](const uint32_t (&c)[16], int half) {
+            uint32_t o[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const float2 cq = make_float2(__uint_as_float(c[2 * q]), __uint_as_float(c[2 * q + 1]));
+              if constexpr (MODE == kLowRankForward) {
+                const float2 y = __ffma2_rn(cq, l2, base[8 * half + q]);
+                const float2 e = make_float2(fast_ex2(y.x), fast_ex2(y.y));
+                if (q & 1) sb = __fadd2_rn(sb, e);
+                else sa = __fadd2_rn(sa, e);
+              } else {
+                const float2 y = __ffma2_rn(cq, l2, __fadd2_rn(base[8 * half + q], make_float2(-lse2, -lse2)));
+                const float2 gq = __fmul2_rn(make_float2(fast_ex2(y.x), fast_ex2(y.y)), make_float2(-wt, -wt));
+                sum[8 * half + q] = __fadd2_rn(sum[8 * half + q], gq);
+                const __nv_bfloat162 h = __floats2bfloat162_rn(gq.x, gq.y);
+                o[q] = *reinterpret_cast<const uint32_t*>(&h);
+              }
             }
-            // short dependent chains: reduce as trees
-            float t8[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) t8[q] = fmaxf(x[q], x[q + 8]);
-            const float bm = fmaxf(fmaxf(fmaxf(t8[0], t8[1]), fmaxf(t8[2], t8[3])), fmaxf(fmaxf(t8[4], t8[5]), fmaxf(t8[6], t8[7])));
-            const float mn = fmaxf(m, bm);
-            const float mn2 = mn * kLog2e;
-            const float rescale = fast_ex2((m - mn) * kLog2e);
-            float e[16];
-#pragma unroll
-            for (int q = 0; q < 16; ++q) e[q] = fast_ex2(fmaf(x[q], kLog2e, -mn2));
-#pragma unroll
-            for (int q = 0; q < 8; ++q) e[q] += e[q + 8];
-            s = fmaf(s, rescale, ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7])));
-            m = mn;
-            const int rel = tgt - col0;
-            if (static_cast<unsigned>(rel) < 16u) {
-#pragma unroll
-              for (int q = 0; q < 16; ++q)
-                if (rel == q) tval = x[q];
-            }
+            if constexpr (MODE == kLowRankGradient)
+              if (valid) st_global_v8_b32(dst + 16 * half, o);                   // 32-byte aligned: one full sector
           };
-          // both loads of the next batch are in flight while this one goes through the exponentials
-          const int nb = width / 16;
-          uint32_t c0[16], b0[16], c1[16], b1[16];
-          tmem_ld16_issue(ccol, c0);
-          tmem_ld16_issue(bcol + col_chunk, b0);
-          tmem_ld_wait16(c0);
-          tmem_ld_wait16(b0);
-          for (int b = 0; b < nb; b += 2) {
-            if (b + 1 < nb) {
-              tmem_ld16_issue(ccol + (b + 1) * 16, c1);
-              tmem_ld16_issue(bcol + col_chunk + (b + 1) * 16, b1);
+          if (here > 0) eat(ca0, 0);
+          tmem_ld_wait16(ca1);
+          if (jj + 1 < jc) {
+            if (!(ok = wait_slot(use + 1))) break;
+            tc_fence_after();
+            tmem_ld16_issue(lane_base + ((use + 1) % kSlots) * kCols, ca0);
+          }
+          if (here == 32) eat(ca1, 1);
+          if constexpr (MODE == kLowRankForward) {
+            float s = (sa.x + sa.y) + (sb.x + sb.y);
+            float l = fast_lg2(s);                         // log2 of the sum relative to ref: a small number
+            if (here > 0 && !__all_sync(kFull, s > 0x1p-60f && s < 0x1p120f)) {
+              // corrections so large that the base logits' maximum is no reference: once more, with the maximum (NaN stays NaN)
+              float m = -CUDART_INF_F;
+              s = 0.f;
+#pragma unroll 1
+              for (int pass = 0; pass < 2; ++pass)
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                  uint32_t c[16];
+                  tmem_ld16_issue(col + 16 * half, c);
+                  tmem_ld_wait16(c);
+                  if (16 * half < here) {
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) {
+                      const float b = q & 1 ? base[8 * half + q / 2].y : base[8 * half + q / 2].x;
+                      const float y = fmaf(__uint_as_float(c[q]), kLog2e, b);
+                      if (pass == 0) m = fmaxf(m, y);
+                      else s += fast_ex2(y - m);
+                    }
+                  }
+                }
+              l = m + fast_lg2(s);
             }
-            consume(c0, b0, b);
-            if (b + 1 >= nb) break;
-            tmem_ld_wait16(c1);
-            tmem_ld_wait16(b1);
-            if (b + 2 < nb) {
-              tmem_ld16_issue(ccol + (b + 2) * 16, c0);
-              tmem_ld16_issue(bcol + col_chunk + (b + 2) * 16, b0);
-            }
-            consume(c1, b1, b + 1);
-            if (b + 2 < nb) {
-              tmem_ld_wait16(c0);
-              tmem_ld_wait16(b0);
-            }
+            patch[jj * kLrPitch + lane] = l;
+          } else if (rel >= 0) {
+            dst[rel] = __float2bfloat16_rn(wt * (1.f - __expf(mine[(2 * kLrJ + jj) * kLrPitch + lane])));
           }
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&ctl->tempty[slot]));
+          if (lane == 0) mbar_arrive(smem_u32(&ctl->tempty[use % kSlots]));
         }
         if (!ok) break;
-        if (valid) {
-          const size_t e = (static_cast<size_t>(row) * p.n + w.slot) * p.r + j;
-          if (p.panels == 1) {
-            if (p.lse_out != nullptr) p.lse_out[e] = m + fast_lg2(s) * kLn2;
-            if (tgt < 0) {
-              p.G[e] = p.missing_is_nan ? CUDART_NAN_F : 0.f;   // marginalised byte: the input unit sums to 1
-            } else if (tgt >= p.vv) {
-              p.G[e] = CUDART_NAN_F;
-              atomicOr(p.status, kStatusBadTarget);
-            } else {
-              p.G[e] = tval - (m + fast_lg2(s) * kLn2);
+        if constexpr (MODE == kLowRankForward) {
+          if (here > 0) {                                  // the round's log-sums, transposed: 64 contiguous bytes per position
+            __syncwarp();
+            float* dst = p.log_sum + static_cast<size_t>(col0 / 32) * p.T * units + static_cast<size_t>(w.slot) * p.r + j0;
+            const int jj = lane & (kLrJ - 1);
+            if (jj < jc) {
+#pragma unroll
+              for (int it = 0; it < 16; ++it) {
+                const int rr = it * 2 + (lane >> 4);
+                if (row0 + rr < p.T) dst[static_cast<size_t>(row0 + rr) * units + jj] = patch[jj * kLrPitch + rr];
+              }
             }
-          } else {
-            // (padding is less than 16 columns and a panel at least 16 wide: every panel has existing symbols)
-            p.partial[static_cast<size_t>(w.panel) * entries + e] = make_float2(m, s);
-            if (static_cast<unsigned>(tgt - panel_col0) < static_cast<unsigned>(w.width)) p.target_logit[e] = tval;
+            __syncwarp();
           }
         }
       }
-      if (!ok) break;
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&lc->aempty[buf]));   // the base of the item after next may overwrite the buffer
+      if constexpr (MODE == kLowRankGradient) if (valid && ok && here > 0) {
+        uint32_t o[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+          float2 sq = sum[q];
+          if (rel == 2 * q) sq.x += hot;
+          if (rel == 2 * q + 1) sq.y += hot;
+          const __nv_bfloat162 h = __floats2bfloat162_rn(sq.x, sq.y);
+          o[q] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        __nv_bfloat16* dst = p.s + static_cast<size_t>(row) * p.s_pitch + static_cast<size_t>(w.slot) * p.v + col0;
+        st_global_v8_b32(dst, o);
+        if (here == 32) st_global_v8_b32(dst + 16, o + 8);
+      }
     }
+    cp_async_wait<0>();                                    // (after an abort) no copy is in flight when the CTA goes away
   }
 
   tc_fence_before();
@@ -422,28 +453,70 @@ mtpc_lowrank_gemm_kernel(const __grid_constant__ LowRankGemmParams p) {
   }
 }
 
-// G[t, i, j] = logit[target] - LSE over the unit, from the per-panel (maximum, sum of exponentials) the factored projection
-// left: one thread per (position, slot, component). Targets < 0 (marginalised): 0; targets >= vv: NaN and the status bit.
-__global__ void lowrank_merge_kernel(const float2* __restrict__ partial, const float* __restrict__ target_logit,
+// G[t, i, j] = logit[target] - LSE over the unit: the LSE from the log-sums of 32 columns each and their references, the target's
+// logit as its base logit + A[i, j, target] . z[t, i, j] (k multiply-adds per thread; A in its repacked layout, so that the r
+// components of a slot read one contiguous row). One thread per (position, slot, component). Targets < 0 (marginalised): 0,
+// or NaN where they are refused draws; targets >= vv: NaN and the status bit.
+__global__ void lowrank_merge_kernel(const float* __restrict__ log_sum, const float* __restrict__ refs, const float* __restrict__ base,
+                                     const __nv_bfloat16* __restrict__ zhl, const __nv_bfloat16* __restrict__ Arep,
                                      const int* __restrict__ targets, float* __restrict__ G, float* __restrict__ lse_out,
-                                     unsigned* status, size_t entries, int r, int vv, int panels, int missing_is_nan) {
+                                     unsigned* status, size_t entries, int n, int r, int v, int vv, int k, int missing_is_nan) {
   const size_t e = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= entries) return;
-  float m = -CUDART_INF_F, s = 0.f;
-  for (int q = 0; q < panels; ++q) {
-    const float2 ms = partial[static_cast<size_t>(q) * entries + e];
-    lse_merge(m, s, ms.x, ms.y);
+  const size_t ti = e / r, tn = entries / r;       // (position, slot), and how many there are
+  const int blocks = (v + 31) / 32;
+  float best = -CUDART_INF_F, ref = 0.f, shift = 0.f, s = 0.f;
+  bool bad = false;
+  for (int q0 = 0; q0 < blocks; q0 += 4) {         // four log-sums in flight (sixteen: 123 against 62 us, r = 32 at T = 8192)
+    float lq[4], rq[4];
+    float top = best, top_ref = ref, top_shift = shift;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      lq[q] = q0 + q < blocks ? log_sum[(q0 + q) * entries + e] : -CUDART_INF_F;
+      rq[q] = q0 + q < blocks ? refs[(q0 + q) * tn + ti] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {                  // the largest so far is the reference
+      const float total = fmaf(rq[q], kLog2e, lq[q]);
+      bad |= total != total;
+      if (total > top) { top = total; top_ref = rq[q]; top_shift = lq[q]; }
+    }
+    if (q0 > 0) s *= fast_ex2(fmaf(ref - top_ref, kLog2e, shift - top_shift));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s += fast_ex2(fmaf(rq[q] - top_ref, kLog2e, lq[q] - top_shift));
+    best = top;
+    ref = top_ref;
+    shift = top_shift;
   }
-  const float lse = m + __logf(s);
+  const float lse = bad ? CUDART_NAN_F : fmaf(shift + fast_lg2(s), kLn2, ref);
   if (lse_out != nullptr) lse_out[e] = lse;
-  const int tgt = targets[e / r];
+  const int tgt = targets[ti];
   if (tgt < 0) { G[e] = missing_is_nan ? CUDART_NAN_F : 0.f; return; }
   if (tgt >= vv) {
     G[e] = CUDART_NAN_F;
     atomicOr(status, kStatusBadTarget);
     return;
   }
-  G[e] = target_logit[e] - lse;
+  const int i = static_cast<int>(ti % n), j = static_cast<int>(e - ti * r);
+  const uint4* zp = reinterpret_cast<const uint4*>(zhl + e * 2 * k);
+  const uint4* ap = reinterpret_cast<const uint4*>(Arep + ((static_cast<size_t>(i) * v + tgt) * r + j) * k);
+  float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+  for (int q = 0; q < kLrMaxRank / 8; ++q) {
+    if (q * 8 < k) {
+      const uint4 hi = zp[q], lo = zp[k / 8 + q], a = ap[q];
+      const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&hi);
+      const __nv_bfloat162* l2 = reinterpret_cast<const __nv_bfloat162*>(&lo);
+      const __nv_bfloat162* a2 = reinterpret_cast<const __nv_bfloat162*>(&a);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const float2 h = __bfloat1622float2(h2[t]), l = __bfloat1622float2(l2[t]), x = __bfloat1622float2(a2[t]);
+        d0 = fmaf(h.x + l.x, x.x, d0);
+        d1 = fmaf(h.y + l.y, x.y, d1);
+      }
+    }
+  }
+  G[e] = base[ti * v + tgt] + (d0 + d1) - lse;
 }
 
 // A [n, r, v, k] -> A' [n, v, r, k] (bf16, k a multiple of 8): one 16-byte piece per thread.
@@ -507,37 +580,10 @@ __global__ void __launch_bounds__(kExpandThreads) lowrank_expand_kernel(const fl
   }
 }
 
-// Backward pass of a factored head (App. G): with g = d loss / d logit [T, n r v] (bf16), the gradients are
-//   dW_base[i] = (sum_j g_ij)^T h,   dA_ij = g_ij^T (B_ij h),   dB_ij = (g_ij A_ij)^T h,
-//   d hidden   = (sum_j g_ij) W_base[i] + (g_ij A_ij) B_ij  summed over the slots and components.
-// lowrank_component_sum_kernel: S[t, i, b] = sum_j g[t, i, j, b], written as bf16 into a matrix of pitch out_pitch (where
-// it is the A operand of the GEMMs that follow). Eight symbols per thread, 16-byte loads and stores.
-__global__ void __launch_bounds__(256) lowrank_component_sum_kernel(const __nv_bfloat16* __restrict__ g, size_t g_pitch,
-                                                                    __nv_bfloat16* __restrict__ out, size_t out_pitch, int T,
-                                                                    int n, int r, int v) {
-  const int per_row = n * v / 8;                                 // 16-byte pieces of one row of S
-  const size_t idx = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= static_cast<size_t>(T) * per_row) return;
-  const int t = static_cast<int>(idx / per_row), c = static_cast<int>(idx % per_row) * 8;
-  const int i = c / v, b = c - i * v;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  const __nv_bfloat16* src = g + static_cast<size_t>(t) * g_pitch + static_cast<size_t>(i) * r * v + b;
-  for (int j = 0; j < r; ++j) {
-    const uint4 piece = *reinterpret_cast<const uint4*>(src + static_cast<size_t>(j) * v);
-    const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&piece);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float2 f = __bfloat1622float2(h2[q]);
-      acc[2 * q] += f.x;
-      acc[2 * q + 1] += f.y;
-    }
-  }
-  __align__(16) __nv_bfloat16 o[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) o[q] = __float2bfloat16_rn(acc[q]);
-  *reinterpret_cast<uint4*>(out + static_cast<size_t>(t) * out_pitch + c) = *reinterpret_cast<const uint4*>(o);
-}
-
+// Backward pass of a factored head (App. G): with g = d loss / d logit [T, n r v] (bf16) and s_i = sum_j g_ij, both written by
+// lowrank_logits_kernel, the gradients are
+//   dW_base[i] = s_i^T h,   dA_ij = g_ij^T (B_ij h),   dB_ij = (g_ij A_ij)^T h,
+//   d hidden   = s_i W_base[i] + (g_ij A_ij) B_ij  summed over the slots and components.
 // A [n r, v, k] -> [n r, v64, k] with v64 = v rounded up to 64 and zero rows past v: the batched GEMM g_ij A_ij walks K in
 // blocks of 64 symbols, and what it reads of g past a unit's own columns must meet zeros.
 __global__ void lowrank_pad_kernel(const uint4* __restrict__ A, uint4* __restrict__ out, int units, int v, int v64, int kv) {

@@ -246,4 +246,11 @@ __device__ __forceinline__ void st_global_v8(float* dst, const float* x) {
                : "memory");
 }
 
+// The same of eight 32-bit words.
+__device__ __forceinline__ void st_global_v8_b32(void* dst, const uint32_t* x) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]),
+               "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7])
+               : "memory");
+}
+
 }  // namespace mtpc

@@ -684,8 +684,7 @@ def measure_draft_whole_batch(torch, head, wl, hidden, steps: int) -> dict:
     res = {"call": "mtpc_draft_sample over the whole batch", "windows": W, "ms_per_call": dms,
            "windows_per_s": W / (dms * 1e-3),
            "phase_ms": [statistics.mean(p[k] for p in dph) for k in range(len(dph[0]))],
-           "phases": "sum-unit GEMM, latent draws, byte draws (sorted by unit: sort + staging + GEMM), GEMM + gather "
-                     "epilogue on the drafted bytes, circuit"}
+           "phases": "projection keeping its logits, latent draws, byte draws and evidence, circuit"}
     # draft with prefix marginals + acceptance stage (Algorithm 3) on the whole batch, synthetic target-model rows
     tp = torch.from_numpy(I.target_rows(I.BASE_SEED + 77, 9, (W, s.n + 1, s.v))).cuda()
     ua = torch.from_numpy(I.uniforms(I.BASE_SEED + 78, 10, (W, s.n + 1))).cuda()

@@ -74,11 +74,8 @@ typedef struct {
   int32_t n;                   /* window length. BTREE: a power of two >= 2                            */
   int32_t r;                   /* units per layer (mixture components / hidden states): a power of two,
                                   <= 128 for CP, <= 32 for HMM and BTREE                               */
-  int32_t v;                   /* vocabulary: a multiple of 16, any size the n*r*v <= 2^30 limit admits (a unit of
-                                  up to 512 symbols is sampled out of tensor memory in one go; wider units are
-                                  streamed through it twice and, on more than 128 positions, always with the
-                                  draws sorted by unit). v = 272 and the like (no split into equal 16-aligned
-                                  tiles of <= 256 columns) draft on up to 128 positions per call only              */
+  int32_t v;                   /* vocabulary: a multiple of 16, any size the n*r*v <= 2^30 limit admits (units of
+                                  more than 512 symbols are drawn from 512 at a time)                              */
   int32_t d;                   /* hidden size: a multiple of 64                                        */
   int32_t io_dtype;            /* MTPC_F32 | MTPC_BF16: dtype of hidden, W_emit and W_sum              */
   int32_t max_positions;       /* upper bound on T (log-prob) and P (draft) per call                   */
@@ -191,12 +188,13 @@ int mtpc_draft_sample_prefix(mtpc_head* head, const void* hidden, int32_t P, int
  * the latent that owns the slot; it is evaluated from what the draft call left in the workspace. Hence:
  *   - the call must follow mtpc_draft_sample / mtpc_draft_sample_prefix on this head with the same P and wpp, with no
  *     other call on the head in between, else MTPC_ERR_STATE;
- *   - a draft of P <= 128 positions (decode-time batches) leaves every logit of those positions: one kernel;
- *   - a draft of more positions (a verification batch) leaves only the evidence of the drafted bytes. The call then
- *     runs the tests, sorts the rejected windows by the slot of their first rejected byte, recomputes that slot's
- *     r*v logits for them in one projection pass over staged hidden states, and draws. It reads the hidden states the
- *     DRAFT call was given (bf16 heads: the caller's buffer, which must still hold them); heads created for at most 128
- *     positions have no scratch for this (MTPC_ERR_UNSUPPORTED).
+ *   - the draft leaves every logit of its positions, and the call is one kernel, unless they exceed 4 GiB (n r v 4 bytes per
+ *     position): such a draft runs in chunks of positions and leaves only the evidence of the drafted bytes. The call then
+ *     runs the tests, sorts the rejected windows by the slot of their first rejected byte, recomputes that slot's r*v logits
+ *     for them in one projection pass over staged hidden states, and draws. It reads the hidden states the DRAFT call was
+ *     given (bf16 heads: the caller's buffer, which must still hold them);
+ *   - a draft by mtpc_draft_sample leaves no slot messages (what the sweep for prefix marginals yields besides them): the
+ *     first acceptance call after it forms them with one more launch.
  * A uniform outside [0,1) or a draft byte outside [0,v) sets the status bit and yields -1 / -1 for that window.
  */
 int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32_t* draft_bytes,
@@ -371,9 +369,9 @@ int mtpc_get_status(mtpc_head* head, void* stream, uint32_t* out_flags);
  *                        and the loss, [2] and [3] as above.
  *   mtpc_draft_sample, mtpc_draft_sample_prefix:   P <= 128 positions: [0] one pass over all weights (logits of every unit),
  *                        [1] per-slot latent + byte draws and evidence, [2] circuit evaluation.
- *                        Otherwise: [0] sum-unit GEMM, [1] latent sampling, [2] byte draws (GEMM + inverse-CDF
- *                        epilogue; when the draws are sorted by unit: the sort, the staging copy and that GEMM),
- *                        [3] GEMM + gather epilogue on the drafted bytes, [4] circuit evaluation.
+ *                        Otherwise: [0] the projection, keeping its logits, [1] latent draws, [2] byte draws and evidence,
+ *                        [3] circuit evaluation (a factored head: [0] log omega, W_base h and B h, [1] latent draws, [2] byte
+ *                        draws, [3] log-sum-exps and evidence, [4] circuit evaluation).
  */
 int mtpc_set_timing(mtpc_head* head, int32_t ring);
 int mtpc_get_timing(mtpc_head* head, int32_t calls_back, float* out_ms, int32_t capacity, int32_t* out_count);
@@ -401,10 +399,9 @@ int mtpc_debug_set_wait_limit_ns(mtpc_head* head, uint64_t limit_ns);
 int mtpc_debug_set_projection_variant(mtpc_head* head, int32_t variant);
 
 /*
- * Test and measurement hook (no passage of the paper): how mtpc_draft_sample on more than 128 positions runs the byte
- * draws of Algorithm 1. 0 (default): chosen per call; 1: one pass of every position against every input unit;
- * 2: the (window, slot) pairs are first sorted by the unit they sample from, and each is multiplied by that unit only
- * (MTPC_ERR_UNSUPPORTED if the head was created for at most 128 positions). Same uniforms, same bytes either way.
+ * Test hook (no passage of the paper), kept for its callers: mode 0, 1 or 2 once chose how mtpc_draft_sample on more than
+ * 128 positions runs the byte draws. There is one implementation now; the modes draw the same bytes. MTPC_ERR_SHAPE for other
+ * modes, MTPC_ERR_UNSUPPORTED for mode 2 on a head created for at most 128 positions.
  */
 int mtpc_debug_set_draft_grouping(mtpc_head* head, int32_t mode);
 

@@ -25,15 +25,18 @@ using namespace mtpc;
 constexpr size_t kAlign = 256;
 constexpr int kMaxPhases = 5;
 constexpr size_t kSlotSmemLimit = 160 * 1024;   // latent-draw tables of the draft slot kernel kept in shared memory up to this
-constexpr int kMaxDraftVocab = 512;     // many-position draft: the v logits of a unit live in 512 TMEM columns
+constexpr int kMaxDraftVocab = 512;     // symbols a warp draws from in one go
 constexpr int kHostChunkPositions = 2048;   // host-buffer calls upload and process this many positions at a time
 constexpr int kWorkCounterWord = 16;   // word of the 256-byte status area used as the circuit kernels' work counter
 constexpr int kSmemLimit = 232448;   // 227 KB of dynamic shared memory per CTA on sm_100
 // Hidden states of one rasterisation block of the projection kernel: small enough to stay L2-resident next to the
 // weight tiles streaming past (data read by all SMs ends up in both halves of the 126 MB L2).
 constexpr size_t kHiddenBlockBytes = 36u << 20;
-// Many-position draft, sampling pass grouped by unit: hidden states staged per (window, slot) pair, at most this much
-// at a time (longer calls are processed in chunks of positions).
+// Drafts of more positions than the few-position path takes keep the emission logits of their positions (the byte draws, the
+// evidence and the acceptance stage are then gathers), at most this much of them: longer drafts run in chunks of positions,
+// and their acceptance stage recomputes the logits it needs.
+constexpr size_t kKeptLogitBytes = static_cast<size_t>(4) << 30;
+// ... from hidden states staged by slot, this much at a time.
 constexpr size_t kGroupStageBytes = 1u << 30;
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -52,23 +55,20 @@ struct Tiling {
 struct Layout {
   // derived sizes
   int S, sum_rows, sum_cols, sum_tiles;
-  Tiling lp;            // log-likelihood mode: 256-column tiles over the flattened (i,k,b) axis
-  Tiling sm;            // sampling mode: one unit per group, equal tiles of <= 256 columns
+  Tiling lp;            // 256-column tiles over the flattened (i,k,b) axis
   size_t max_windows;
   // workspace offsets (bytes)
   size_t off_status, off_wemit, off_wsum, off_hidden, off_logA, off_G, off_logw, off_sel, off_logits, off_unit_lse;
   size_t off_prefix, off_partial, off_sum_bias;   // training loss: prefix log-marginals [max_positions, n], per-sequence terms
   size_t off_msg;       // slot messages of the drafted windows [max_windows, n, r], kept for the acceptance stage
-  int decode_max_p;     // positions the few-position draft path can take (0: path not available)
-  bool can_draft;       // v <= 512: the sampling kernels hold a whole input unit on chip
-  bool can_draft_many;  // the sampling epilogue of the projection kernel can tile a unit (draft of more than 128 positions)
-  bool sample_two_pass; // ... but only by streaming the unit's tiles through tensor memory twice (v > 512): draws sorted by unit
+  int decode_max_p;     // positions the few-position draft path can take
+  int kept_p;           // positions whose logits a longer draft can keep at once (0: no longer drafts)
   size_t off_h_hidden, off_h_targets, off_h_uniforms, off_h_bytes, off_h_out;
-  // grouped sampling pass of the many-position draft (0 entries: not available)
-  size_t group_entries;   // (window, slot) pairs that can be staged at once
+  // acceptance stage after a draft that did not keep its logits: windows that can be staged at once (0: not needed)
+  size_t group_entries;
   size_t off_grp_ints, off_grp_tiles, off_grp_perm, off_grp_stage;
-  // acceptance stage after a many-position draft: first rejected slot and staging row per window, the recomputed logits
-  // [accept_rows, r v] and unit log-sum-exps [accept_rows, r] of that slot
+  // ... first rejected slot and staging row per window, the recomputed logits [accept_rows, r v] and unit log-sum-exps
+  // [accept_rows, r] of that slot (a factored head forms them after every long draft)
   size_t accept_rows;     // windows that can be handled at once (0: not available)
   size_t off_acc_rej, off_acc_row, off_acc_logits, off_acc_lse;
   size_t total;
@@ -95,7 +95,8 @@ bool fit_tiling(Tiling* t, int sum_cols) {
   return stages >= 2 && t->num_slots >= 2;
 }
 
-int plan(const mtpc_config& c, Layout* L) {
+// factored: the head keeps low-rank unembeddings factored (its long drafts take another route).
+int plan(const mtpc_config& c, Layout* L, bool factored = false) {
   if (c.family < MTPC_CP || c.family > MTPC_BTREE) return MTPC_ERR_SHAPE;
   if (c.io_dtype != MTPC_F32 && c.io_dtype != MTPC_BF16) return MTPC_ERR_SHAPE;
   if (c.n < 1 || c.r < 1 || c.v < 1 || c.d < 1 || c.max_positions < 1 || c.max_windows_per_pos < 1)
@@ -121,28 +122,6 @@ int plan(const mtpc_config& c, Layout* L) {
   L->sum_cols = sum_cols;
   L->sum_tiles = (L->sum_rows + sum_cols - 1) / sum_cols;
   const int emit_units = c.n * c.r;
-  // sampling: emission unit -> equal tiles of <= 256 columns, each a multiple of 16, all in TMEM at once
-  // (a unit of more than 512 symbols does not fit tensor memory: such heads draft through the few-position path only)
-  L->can_draft = true;
-  L->sample_two_pass = c.v > kMaxDraftVocab;
-  if (!L->sample_two_pass) {
-    int chunks = (c.v + 255) / 256;
-    while (c.v % chunks != 0 || (c.v / chunks) % 16 != 0) ++chunks;
-    L->sm.tile_cols = c.v / chunks;
-    L->sm.group_units = 1;
-    L->sm.group_tiles = chunks;
-    L->sm.num_groups = emit_units;
-    // (no such split, e.g. v = 272 = 17 x 16: only the few-position draft path, which needs none, is available)
-    L->can_draft_many = fit_tiling(&L->sm, sum_cols) && L->sm.num_slots >= chunks;
-  } else {
-    // 256-column tiles, the last one ragged (its tail columns are masked), streamed through two accumulator slots
-    L->sm.tile_cols = 256;
-    L->sm.group_units = 1;
-    L->sm.group_tiles = (c.v + 255) / 256;
-    L->sm.num_groups = emit_units;
-    L->can_draft_many = fit_tiling(&L->sm, sum_cols);
-  }
-  if (!L->can_draft_many) memset(&L->sm, 0, sizeof(L->sm));
   // log-likelihood: 256-column tiles; a group is the shortest run of whole units that is a whole number of tiles
   const int lcm = c.v / gcd_int(c.v, 256) * 256;
   L->lp.tile_cols = 256;
@@ -171,9 +150,15 @@ int plan(const mtpc_config& c, Layout* L) {
   L->off_sel = take(L->max_windows * c.n * 4);
   L->off_msg = take(L->max_windows * c.n * c.r * 4);
   // (latents of more than 32 values are handled for the mixture only; HMM and BTree are limited to r <= 32 anyway)
-  L->decode_max_p = L->can_draft ? (c.max_positions < kDecodeMaxP ? c.max_positions : kDecodeMaxP) : 0;
-  L->off_logits = take(static_cast<size_t>(L->decode_max_p) * emit_units * c.v * 4);
-  L->off_unit_lse = take(static_cast<size_t>(L->decode_max_p) * emit_units * 4);
+  L->decode_max_p = c.max_positions < kDecodeMaxP ? c.max_positions : kDecodeMaxP;
+  L->kept_p = 0;
+  if (c.max_positions > L->decode_max_p && !factored) {
+    const size_t cap = kKeptLogitBytes / (static_cast<size_t>(emit_units) * c.v * 4);     // >= 1: n r v <= 2^30
+    L->kept_p = static_cast<size_t>(c.max_positions) < cap ? c.max_positions : static_cast<int>(cap);
+  }
+  const size_t logit_rows = L->kept_p > L->decode_max_p ? L->kept_p : L->decode_max_p;
+  L->off_logits = take(logit_rows * emit_units * c.v * 4);
+  L->off_unit_lse = take(logit_rows * emit_units * 4);
   L->off_prefix = take(static_cast<size_t>(c.max_positions) * c.n * 4);
   L->off_partial = take(static_cast<size_t>(c.max_positions) * c.n * 4);
   L->off_h_hidden = take(static_cast<size_t>(c.max_positions) * c.d * elt);
@@ -181,27 +166,21 @@ int plan(const mtpc_config& c, Layout* L) {
   L->off_h_uniforms = take(L->max_windows * 2 * c.n * 4);
   L->off_h_bytes = take(L->max_windows * c.n * 4);
   L->off_h_out = take(L->max_windows * 4);
-  // grouped sampling: only heads that can be asked for a many-position draft carry the staging area
   L->group_entries = 0;
-  if (L->can_draft_many && c.max_positions > L->decode_max_p && emit_units <= kGroupMaxUnits) {
-    const size_t cap = kGroupStageBytes / (static_cast<size_t>(c.d) * 2);
-    const size_t all = L->max_windows * c.n;
-    L->group_entries = all < cap ? all : cap;
-    if (L->group_entries < static_cast<size_t>(c.max_windows_per_pos) * c.n) L->group_entries = 0;   // not even one position
+  L->accept_rows = 0;
+  if (c.max_positions > L->decode_max_p && L->kept_p < c.max_positions) {
+    const size_t stage_cap = kGroupStageBytes / (static_cast<size_t>(c.d) * 2);
+    const size_t row_cap = kGroupStageBytes / (static_cast<size_t>(c.r) * c.v * 4);
+    L->accept_rows = L->max_windows < row_cap ? L->max_windows : row_cap;
+    if (!factored && L->accept_rows > stage_cap) L->accept_rows = stage_cap;        // they share the staging rows
+    if (L->accept_rows < static_cast<size_t>(c.max_windows_per_pos)) L->accept_rows = 0;   // not even one position
+    if (!factored) L->group_entries = L->accept_rows;
   }
-  const size_t ge = L->group_entries;
-  L->off_grp_ints = take(ge ? (3 * static_cast<size_t>(emit_units) + 64) * 4 : 0);     // counts | cursors | offsets | tile count
-  L->off_grp_tiles = take(ge ? (emit_units + ge / 128 + 1) * sizeof(GroupTile) : 0);
+  const size_t ge = L->group_entries, ar = L->accept_rows;
+  L->off_grp_ints = take(ge ? (3 * static_cast<size_t>(c.n) + 64) * 4 : 0);            // counts | cursors | offsets | tile count
+  L->off_grp_tiles = take(ge ? (c.n + ge / 128 + 1) * sizeof(GroupTile) : 0);
   L->off_grp_perm = take(ge * 4);
   L->off_grp_stage = take(ge * c.d * 2);
-  L->accept_rows = 0;
-  if (ge > 0) {
-    const size_t cap = kGroupStageBytes / (static_cast<size_t>(c.r) * c.v * 4);
-    L->accept_rows = L->max_windows < cap ? L->max_windows : cap;
-    if (L->accept_rows > ge) L->accept_rows = ge;                               // they share the staging rows
-    if (L->accept_rows < static_cast<size_t>(c.max_windows_per_pos)) L->accept_rows = 0;
-  }
-  const size_t ar = L->accept_rows;
   L->off_acc_rej = take(ar ? L->max_windows * 4 : 0);
   L->off_acc_row = take(ar ? L->max_windows * 4 : 0);
   L->off_acc_logits = take(ar * c.r * c.v * 4);
@@ -268,10 +247,9 @@ struct mtpc_head {
   uint8_t* ws;
   const void* W_emit_bf16;
   const void* W_sum_bf16;
-  CUtensorMap tm_emit_lp, tm_emit_sm, tm_sum;   // W_emit with the box of either tiling; W_sum
-  CUtensorMap tm_emit_lp2, tm_emit_sm2, tm_sum2; // the same with boxes of half the rows: what one CTA of a pair stages
+  CUtensorMap tm_emit_lp, tm_sum;               // W_emit, W_sum
+  CUtensorMap tm_emit_lp2, tm_sum2;             // the same with boxes of half the rows: what one CTA of a pair stages
   int projection_variant;                       // 0: chosen per launch; 1: every CTA alone; 2: CTA pairs (cta_group::2)
-  int draft_grouping;                           // many-position draft: 0 chosen per call; 1 never sort the draws by unit; 2 always
   // factored low-rank head (App. G; mtpc_create_head_lowrank): rank k > 0, no composed W_emit
   int lr_k;
   const void* lr_W_base;                        // [n, v, d] bf16
@@ -297,7 +275,8 @@ struct mtpc_head {
   int draft_P;              // positions whose draft state (logits, or after a many-position draft G and log omega) is in the workspace (0: none)
   int draft_wpp;            // windows per position of that draft
   bool draft_msg;           // its slot messages are in the workspace too (a draft that asked for prefix marginals leaves them)
-  const void* draft_hidden; // many-position draft: the bf16 hidden states it read (the acceptance stage stages rows of them)
+  bool draft_logits;        // every logit and unit log-sum-exp of its positions as well
+  const void* draft_hidden; // the bf16 hidden states it read (the acceptance stage may have to stage rows of them)
   int ring;                 // calls whose per-kernel events are retained (0 = timing off)
   cudaEvent_t* ev;          // [ring][kMaxPhases][2]
   int* ring_phases;         // [ring] phases recorded by the call in that slot
@@ -385,31 +364,27 @@ int choose_group_units(int v, int emit_units, int m_tiles, int ctas) {
   return best;
 }
 
-struct GroupArgs {           // grouped sampling pass: the staged hidden states and their tiles (mtpc_group.cuh)
+struct GroupArgs {           // rows sorted by slot: the staged hidden states and their tiles (mtpc_group.cuh)
   const void* stage = nullptr;
   int entries = 0;                           // rows of the staging buffer in use
   const GroupTile* tiles = nullptr;
   const int* num_tiles = nullptr;
-  const int* perm = nullptr;
-  const int* unit_sel = nullptr;             // this chunk's rows of the selected units
   int max_tiles = 0;
-  bool by_slot = false;                      // rows sorted by slot; the kernel writes the slot's logits (acceptance stage)
 };
 
-struct GradArgs {            // what the projection kernel keeps for the backward pass (training calls only)
+struct GradArgs {            // what the projection kernel keeps for the backward pass or a draft
   float* lse_out = nullptr;                  // the units' log-sum-exps [T, n, r]
   float* logit_out = nullptr;                // the emission logits [T, n r v] fp32
   size_t logit_pitch = 0;
 };
 
-int launch_gemm(mtpc_head* h, int mode, const void* hidden_bf16, int rows, int wpp, bool with_emit, bool with_sum,
-                const int* targets, const float* uniforms, int* out_bytes, cudaStream_t st,
-                const GradArgs* ga = nullptr, bool targets_are_drafts = false, const GroupArgs* grp = nullptr) {
+// first_row: where in log omega the launch's positions start (a draft that runs in chunks of positions).
+int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit, bool with_sum, const int* targets, cudaStream_t st,
+                const GradArgs* ga = nullptr, const GroupArgs* grp = nullptr, int first_row = 0) {
   if (rows <= 0 || (!with_emit && !with_sum)) return MTPC_OK;
   const mtpc_config& c = h->cfg;
   const Layout& L = h->L;
-  const Tiling& tl = mode == kModeSample ? L.sm : L.lp;
-  if (grp != nullptr && (grp->by_slot ? mode != kModeLogprob : mode != kModeSample)) return MTPC_ERR_SHAPE;
+  const Tiling& tl = L.lp;
   GemmParams p;
   memset(&p, 0, sizeof(p));
   if (ga) {
@@ -420,8 +395,6 @@ int launch_gemm(mtpc_head* h, int mode, const void* hidden_bf16, int rows, int w
   int rc = grp ? make_tmap(&p.tm_a, grp->stage, static_cast<uint64_t>(grp->entries), static_cast<uint64_t>(c.d), kBlockM)
                : make_tmap(&p.tm_a, hidden_bf16, static_cast<uint64_t>(rows), static_cast<uint64_t>(c.d), kBlockM);
   if (rc != MTPC_OK) return rc;
-  p.tm_emit = mode == kModeSample ? h->tm_emit_sm : h->tm_emit_lp;
-  p.tm_sum = h->tm_sum;
   p.T = rows;
   p.m_tiles = (rows + kBlockM - 1) / kBlockM;
   // Two CTAs per MMA when there are at least two m-tiles to pair up (and the device can hold a cluster at all)
@@ -442,11 +415,10 @@ int launch_gemm(mtpc_head* h, int mode, const void* hidden_bf16, int rows, int w
   p.emit_units = c.n * c.r;
   p.num_groups = with_emit ? tl.num_groups : 0;
   p.group_units = tl.group_units;
-  if (grp != nullptr) {
-    // sorted rows: by unit, one item per row tile; by slot, a row tile's r units are cut into runs that fill the device
-    p.group_units = grp->by_slot ? choose_group_units(c.v, c.r, grp->max_tiles, workers) : 1;
-    p.num_groups = grp->by_slot ? (c.r + p.group_units - 1) / p.group_units : 1;
-  } else if (mode != kModeSample && with_emit) {
+  if (grp != nullptr) {                                               // a row tile's r units are cut into runs that fill the device
+    p.group_units = choose_group_units(c.v, c.r, grp->max_tiles, workers);
+    p.num_groups = (c.r + p.group_units - 1) / p.group_units;
+  } else if (with_emit) {
     p.group_units = choose_group_units(c.v, p.emit_units, p.m_units, workers);
     p.num_groups = (p.emit_units + p.group_units - 1) / p.group_units;
   }
@@ -458,41 +430,26 @@ int launch_gemm(mtpc_head* h, int mode, const void* hidden_bf16, int rows, int w
   p.num_slots = tl.num_slots;
   p.stages = pair ? tl.pair_stages : tl.stages;
   p.stage_bytes = pair ? tl.pair_stage_bytes : tl.stage_bytes;
-  if (pair) {
-    p.tm_emit = mode == kModeSample ? h->tm_emit_sm2 : h->tm_emit_lp2;
-    p.tm_sum = h->tm_sum2;
-  }
-  p.wpp = wpp;
+  p.tm_emit = pair ? h->tm_emit_lp2 : h->tm_emit_lp;
+  p.tm_sum = pair ? h->tm_sum2 : h->tm_sum;
   p.targets = targets;
-  p.missing_is_nan = targets_are_drafts ? 1 : 0;
   p.G = at<float>(h, L.off_G);
-  p.logw = at<float>(h, L.off_logw);
+  p.logw = at<float>(h, L.off_logw) + static_cast<size_t>(first_row) * L.sum_rows;
   p.sum_bias = sum_bias(h);
-  p.unit_sel = at<int>(h, L.off_sel);
   if (grp) {
     p.group_tiles = grp->tiles;
     p.group_num_tiles = grp->num_tiles;
-    p.group_perm = grp->perm;
-    p.group_two_pass = (L.sample_two_pass && !grp->by_slot) ? 1 : 0;
-    p.unit_sel = grp->unit_sel;
   }
-  p.uniforms = uniforms;
-  p.out_bytes = out_bytes;
   p.status = at<unsigned>(h, L.off_status);
   p.wait_limit_ns = h->wait_limit_ns;
   const long long items = grp ? static_cast<long long>(grp->max_tiles) * p.num_groups
                               : static_cast<long long>(p.m_units) * (p.num_groups + p.num_sum_tiles);
   const int grid = ctas * static_cast<int>(items < workers ? items : workers);
   const size_t smem = pair ? tl.pair_smem : tl.smem;
-  if (grp && grp->by_slot) {
+  if (grp) {
     mtpc_gemm_kernel<kModeLogitsGrouped, 1><<<grid, kGemmThreads, smem, st>>>(p);
-  } else if (grp) {
-    mtpc_gemm_kernel<kModeSampleGrouped, 1><<<grid, kGemmThreads, smem, st>>>(p);
   } else if (!pair) {
-    if (mode == kModeLogprob)
-      mtpc_gemm_kernel<kModeLogprob, 1><<<grid, kGemmThreads, smem, st>>>(p);
-    else
-      mtpc_gemm_kernel<kModeSample, 1><<<grid, kGemmThreads, smem, st>>>(p);
+    mtpc_gemm_kernel<kModeLogprob, 1><<<grid, kGemmThreads, smem, st>>>(p);
   } else {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
@@ -507,8 +464,7 @@ int launch_gemm(mtpc_head* h, int mode, const void* hidden_bf16, int rows, int w
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (mode == kModeLogprob) cudaLaunchKernelEx(&cfg, mtpc_gemm_kernel<kModeLogprob, 2>, p);
-    else cudaLaunchKernelEx(&cfg, mtpc_gemm_kernel<kModeSample, 2>, p);
+    cudaLaunchKernelEx(&cfg, mtpc_gemm_kernel<kModeLogprob, 2>, p);
   }
   h->launches++;
   return check_launch();
@@ -780,7 +736,7 @@ int window_logprob_impl(mtpc_head* h, const void* hidden, const int32_t* targets
   PhaseTimer pt(h, st);
   pt.begin();
   if (h->lr_k > 0) rc = launch_lowrank_projection(h, hb, T, targets, st);
-  else rc = launch_gemm(h, kModeLogprob, hb, T, 1, true, true, targets, nullptr, nullptr, st);
+  else rc = launch_gemm(h, hb, T, true, true, targets, st);
   pt.end();
   if (rc != MTPC_OK) return rc;
   pt.begin();
@@ -797,7 +753,6 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
   const int W = P * wpp;
   // a draft that returns prefix marginals runs the sweep that also yields the slot messages of the acceptance stage
   float* const msg = at<float>(h, L.off_msg);
-  if (!L.can_draft) return MTPC_ERR_UNSUPPORTED;
   if (h->lr_k > 0 && P > L.decode_max_p && wpp == 1 && c.v <= kMaxDraftVocab) {
     // A long draft on a factored head, one window per position: log omega, the latent draws, then every (window, slot)
     // forms the logits of its one selected unit from W_base h and B h (lowrank_draw_kernel) and draws its byte; the
@@ -811,9 +766,9 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     pt.end();
     if (rc != MTPC_OK) return rc;
     pt.begin();
-    latent_sample_kernel<<<(W + 127) / 128, 128, 0, st>>>(c.family, at<float>(h, L.off_logw), hmm_tables(h), uniforms,
-                                                          at<int>(h, L.off_sel), out_bytes, at<unsigned>(h, L.off_status), W,
-                                                          wpp, c.n, c.r, L.sum_rows, hmm_table_stride(h));
+    latent_sample_kernel<<<(W + kLatentWarps - 1) / kLatentWarps, 32 * kLatentWarps, 0, st>>>(
+        c.family, at<float>(h, L.off_logw), hmm_tables(h), uniforms, at<int>(h, L.off_sel), out_bytes, at<unsigned>(h, L.off_status), W,
+        wpp, c.n, c.r, L.sum_rows, hmm_table_stride(h));
     h->launches++;
     pt.end();
     if ((rc = check_launch()) != MTPC_OK) return rc;
@@ -841,6 +796,7 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
       h->draft_P = P;
       h->draft_wpp = wpp;
       h->draft_msg = out_prefix != nullptr;
+      h->draft_logits = false;
       h->draft_hidden = nullptr;
     }
     return rc;
@@ -896,6 +852,7 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     h->draft_P = P;
     h->draft_wpp = wpp;
     h->draft_msg = out_prefix != nullptr;
+    h->draft_logits = true;
     pt.end();
     if ((rc = check_launch()) != MTPC_OK) return rc;
     pt.begin();
@@ -904,82 +861,44 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     pt.end();
     return rc;
   }
-  if (!L.can_draft_many) return MTPC_ERR_UNSUPPORTED;
-  // 1. sum-unit weights (Sec. 3.3) -> 2. latent draws at the sum units (Algorithm 1)
-  pt.begin();
-  rc = launch_gemm(h, kModeLogprob, hb, P, 1, false, true, nullptr, nullptr, nullptr, st);
-  pt.end();
-  if (rc != MTPC_OK) return rc;
-  pt.begin();
-  latent_sample_kernel<<<(W + 127) / 128, 128, 0, st>>>(c.family, at<float>(h, L.off_logw), hmm_tables(h), uniforms,
-                                                        at<int>(h, L.off_sel), out_bytes,
-                                                        at<unsigned>(h, L.off_status), W, wpp, c.n, c.r, L.sum_rows,
-                                                        hmm_table_stride(h));
-  h->launches++;
-  pt.end();
-  if ((rc = check_launch()) != MTPC_OK) return rc;
-  // 3. byte draws at the selected input units. With few windows per position against many units per slot the draws
-  // are first sorted by unit, so that every window is multiplied by the one unit it samples from.
-  if (L.sample_two_pass && L.group_entries == 0) return MTPC_ERR_UNSUPPORTED;
-  const bool grouped = L.sample_two_pass ||
-                       (L.group_entries > 0 && h->draft_grouping != 1 && (h->draft_grouping == 2 || wpp * 4 <= c.r));
-  if (grouped) {
-    const int units = c.n * c.r;
-    int* ints = at<int>(h, L.off_grp_ints);
-    int* counts = ints, *cursors = ints + units, *offsets = ints + 2 * units, *num_tiles = ints + 3 * units;
-    GroupTile* tiles = at<GroupTile>(h, L.off_grp_tiles);
-    int* perm = at<int>(h, L.off_grp_perm);
-    __nv_bfloat16* stage = at<__nv_bfloat16>(h, L.off_grp_stage);
-    const int chunk_pos = static_cast<int>(L.group_entries / (static_cast<size_t>(wpp) * c.n));   // >= 1 by construction
-    for (int p0 = 0; p0 < P; p0 += chunk_pos) {
-      const int pc = P - p0 < chunk_pos ? P - p0 : chunk_pos;
-      const int entries = pc * wpp * c.n;
-      const size_t w0 = static_cast<size_t>(p0) * wpp;
-      const int* sel = at<int>(h, L.off_sel) + w0 * c.n;
-      pt.begin();
-      if (cudaMemsetAsync(ints, 0, static_cast<size_t>(2 * units) * 4, st) != cudaSuccess) return MTPC_ERR_CUDA;
-      const int cblocks = (entries + kGroupThreads - 1) / kGroupThreads;
-      group_count_kernel<<<cblocks < 4 * h->num_sms ? cblocks : 4 * h->num_sms, kGroupThreads, units * sizeof(int), st>>>(
-          sel, counts, entries, c.n, c.r);
-      group_scan_kernel<<<1, kGroupScanThreads, 0, st>>>(counts, offsets, tiles, num_tiles, units);
-      const int gblocks = (entries + kGroupThreads / 32 - 1) / (kGroupThreads / 32);
-      group_gather_kernel<<<gblocks < 16 * h->num_sms ? gblocks : 16 * h->num_sms, kGroupThreads, 0, st>>>(
-          sel, static_cast<const __nv_bfloat16*>(hb) + static_cast<size_t>(p0) * c.d, offsets, cursors, perm, stage, entries,
-          c.n, c.r, wpp, c.d, static_cast<int*>(nullptr));
-      h->launches += 3;
-      if ((rc = check_launch()) != MTPC_OK) return rc;
-      GroupArgs ga;
-      ga.stage = stage;
-      ga.entries = entries;
-      ga.tiles = tiles;
-      ga.num_tiles = num_tiles;
-      ga.perm = perm;
-      ga.unit_sel = sel;
-      ga.max_tiles = units + entries / 128 + 1;
-      rc = launch_gemm(h, kModeSample, hb, pc, wpp, true, false, nullptr, uniforms + w0 * 2 * c.n, out_bytes + w0 * c.n, st,
-                       nullptr, false, &ga);
-      pt.end();
-      if (rc != MTPC_OK) return rc;
-    }
-  } else {
+  // Many positions: one projection that keeps its logits, unit log-sum-exps and log omega; everything after it is gathers.
+  // In chunks of positions if the logits of all of them do not fit (then only the last chunk's remain).
+  const int chunks = (P + L.kept_p - 1) / L.kept_p, chunk_p = (P + chunks - 1) / chunks;
+  for (int p0 = 0; p0 < P; p0 += chunk_p) {
+    const int pc = P - p0 < chunk_p ? P - p0 : chunk_p, wc = pc * wpp;
+    const size_t w0 = static_cast<size_t>(p0) * wpp;
+    const float* u = uniforms + w0 * 2 * c.n;
+    GradArgs keep;
+    keep.lse_out = at<float>(h, L.off_unit_lse);
+    keep.logit_out = at<float>(h, L.off_logits);
+    keep.logit_pitch = static_cast<size_t>(c.n) * c.r * c.v;
     pt.begin();
-    rc = launch_gemm(h, kModeSample, hb, P, wpp, true, false, nullptr, uniforms, out_bytes, st);
+    rc = launch_gemm(h, static_cast<const __nv_bfloat16*>(hb) + static_cast<size_t>(p0) * c.d, pc, true, true, nullptr, st, &keep, nullptr, p0);
     pt.end();
     if (rc != MTPC_OK) return rc;
+    int* sel = at<int>(h, L.off_sel) + w0 * c.n;
+    pt.begin();
+    latent_sample_kernel<<<(wc + kLatentWarps - 1) / kLatentWarps, 32 * kLatentWarps, 0, st>>>(
+        c.family, at<float>(h, L.off_logw) + static_cast<size_t>(p0) * L.sum_rows,
+        hmm_tables(h) + static_cast<size_t>(p0) * hmm_table_stride(h), u, sel, out_bytes + w0 * c.n, at<unsigned>(h, L.off_status), wc, wpp,
+        c.n, c.r, L.sum_rows, hmm_table_stride(h));
+    pt.end();
+    pt.begin();
+    auto* pick = c.v > kMaxDraftVocab ? draft_pick_kernel<true> : draft_pick_kernel<false>;
+    pick<<<(wc * c.n + 7) / 8, 256, 0, st>>>(keep.logit_out, keep.lse_out, sel, u, out_bytes + w0 * c.n, at<float>(h, L.off_G) + w0 * c.n * c.r,
+                                             at<unsigned>(h, L.off_status), wc * c.n, wpp, c.n, c.r, c.v, valid_symbols(c));
+    pt.end();
+    h->launches += 2;
+    if ((rc = check_launch()) != MTPC_OK) return rc;
   }
-  // 4. evidence of the drafted bytes under every unit -> 5. joint log-prob with the latents summed out
-  pt.begin();
-  rc = launch_gemm(h, kModeLogprob, hb, P, wpp, true, false, out_bytes, nullptr, nullptr, st, nullptr,
-                   /*targets_are_drafts=*/true);
-  pt.end();
-  if (rc != MTPC_OK) return rc;
   pt.begin();
   rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, false, false, out_prefix ? msg : nullptr);
   pt.end();
-  if (rc == MTPC_OK) {                 // G, log omega, the messages and the hidden states stay in place for an acceptance call
+  if (rc == MTPC_OK) {                 // G, log omega, the messages and the logits stay in place for an acceptance call
     h->draft_P = P;
     h->draft_wpp = wpp;
     h->draft_msg = out_prefix != nullptr;
+    h->draft_logits = chunks == 1;
     h->draft_hidden = hb;
   }
   return rc;
@@ -1179,7 +1098,7 @@ int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, cons
   const Layout& L = h->L;
   const int units = c.n * c.r, k = h->lr_k;
   int rc = MTPC_OK;
-  if (parts & 1) rc = launch_gemm(h, kModeLogprob, hidden_bf16, T, 1, false, true, targets, nullptr, nullptr, st);
+  if (parts & 1) rc = launch_gemm(h, hidden_bf16, T, false, true, targets, st);
   if (rc != MTPC_OK) return rc;
   __nv_bfloat16* zhl = reinterpret_cast<__nv_bfloat16*>(h->ws + h->lr_off_zhl);
   float* base = reinterpret_cast<float*>(h->ws + h->lr_off_base);
@@ -1487,10 +1406,8 @@ static int bind_parameters(mtpc_head* h, const void* W_emit, const void* W_sum, 
   const bool dense = h->lr_k == 0;      // a factored low-rank head has no composed W_emit: only the sum-unit maps
   int rc = MTPC_OK;
   if (dense) rc = make_tmap(&h->tm_emit_lp, h->W_emit_bf16, emit_rows, cfg->d, L.lp.tile_cols);
-  if (rc == MTPC_OK && dense && L.can_draft_many) rc = make_tmap(&h->tm_emit_sm, h->W_emit_bf16, emit_rows, cfg->d, L.sm.tile_cols);
   if (rc == MTPC_OK) rc = make_tmap(&h->tm_sum, h->W_sum_bf16, L.sum_rows, cfg->d, L.sum_cols);
   if (rc == MTPC_OK && dense) rc = make_tmap(&h->tm_emit_lp2, h->W_emit_bf16, emit_rows, cfg->d, L.lp.tile_cols / 2);
-  if (rc == MTPC_OK && dense && L.can_draft_many) rc = make_tmap(&h->tm_emit_sm2, h->W_emit_bf16, emit_rows, cfg->d, L.sm.tile_cols / 2);
   if (rc == MTPC_OK) rc = make_tmap(&h->tm_sum2, h->W_sum_bf16, L.sum_rows, cfg->d, L.sum_cols / 2);
   const uint64_t base_rows = static_cast<uint64_t>(cfg->n) * cfg->v, adapt_rows = static_cast<uint64_t>(cfg->n) * cfg->r * h->lr_k;
   choose_decode_tiling(static_cast<long long>(dense ? emit_rows : base_rows + adapt_rows), L.sum_rows, cfg->d / kBlockK, h->num_sms,
@@ -1553,7 +1470,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   if (lowrank && (!lowrank->W_base || !lowrank->A || !lowrank->B)) return MTPC_ERR_NULL;
   *out = nullptr;
   Layout L;
-  int rc = plan(*cfg, &L);
+  int rc = plan(*cfg, &L, lowrank != nullptr);
   if (rc != MTPC_OK) return rc;
   LowRankParams lrp;
   memset(&lrp, 0, sizeof(lrp));
@@ -1596,12 +1513,8 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   // the attribute is per function, not per head: always ask for the full 227 KB so that heads do not undo each other
   fail |= cudaFuncSetAttribute(mtpc_gemm_kernel<kModeLogprob, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                kSmemLimit) != cudaSuccess;
-  fail |= cudaFuncSetAttribute(mtpc_gemm_kernel<kModeSample, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kSmemLimit) != cudaSuccess;
-  fail |= !allow_full_smem(mtpc_gemm_kernel<kModeSampleGrouped, 1>);
   fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogitsGrouped, 1>);
   fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 2>);
-  fail |= !allow_full_smem(mtpc_gemm_kernel<kModeSample, 2>);
   h->max_pairs = fail ? 0 : resident_clusters(mtpc_gemm_kernel<kModeLogprob, 2>, 2, L.lp.pair_smem);
   fail |= !allow_full_smem(plain_gemm_kernel<false, false>);
   fail |= !allow_full_smem(plain_gemm_kernel<false, true>);
@@ -1648,7 +1561,7 @@ int mtpc_create_head(const mtpc_config* cfg, const void* W_emit, const void* W_s
 int mtpc_lowrank_workspace_bytes(const mtpc_config* cfg, int32_t k, size_t* out_bytes) {
   if (!cfg || !out_bytes) return MTPC_ERR_NULL;
   Layout L;
-  int rc = plan(*cfg, &L);
+  int rc = plan(*cfg, &L, /*factored=*/true);
   if (rc != MTPC_OK) return rc;
   LowRankParams lrp;
   if (cfg->io_dtype != MTPC_BF16 || !plan_lowrank(*cfg, k, &lrp)) return MTPC_ERR_UNSUPPORTED;
@@ -1737,8 +1650,8 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
     if (rc != MTPC_OK) return rc;
     head->draft_msg = true;
   }
-  if (P <= L.decode_max_p) {
-    // after a few-position draft: every logit of the drafted positions is still in the workspace
+  if (head->draft_logits) {
+    // every logit of the drafted positions is still in the workspace
     pt.begin();
     launch_kernel(spec_accept_kernel, W, threads, smem, st, /*dependent=*/head->ring == 0, at<float>(head, L.off_logits),
                   at<float>(head, L.off_unit_lse), msg, draft_bytes, prefix_logprob, target_probs, accept_uniforms, out_accepted,
@@ -1748,7 +1661,7 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
     pt.end();
     return check_launch();
   }
-  // After a many-position draft no logits were kept. The evidence of the drafted bytes (G) and log omega are still in
+  // A draft that ran in chunks kept the last one's logits only (a factored head's long draft none). The evidence of the drafted bytes (G) and log omega are still in
   // the workspace; what is missing is, for every window rejected at byte s, the r v logits of slot s. So: run the tests,
   // sort the rejected windows by s, stage their hidden states, recompute those logits with one sorted projection pass,
   // then run the acceptance kernel on them. In chunks of positions whose windows fit the scratch.
@@ -1814,16 +1727,12 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
     ga.entries = wc;
     ga.tiles = tiles;
     ga.num_tiles = num_tiles;
-    ga.perm = perm;
-    ga.unit_sel = rej;
     ga.max_tiles = c.n + wc / 128 + 1;
-    ga.by_slot = true;
     GradArgs out;
     out.lse_out = lse;
     out.logit_out = lg;
     out.logit_pitch = static_cast<size_t>(c.r) * c.v;
-    rc2 = launch_gemm(head, kModeLogprob, head->draft_hidden, pc, wpp, true, false, nullptr, nullptr, nullptr, st, &out, false,
-                      &ga);
+    rc2 = launch_gemm(head, head->draft_hidden, pc, true, false, nullptr, st, &out, &ga);
     pt.end();
     if (rc2 != MTPC_OK) return rc2;
     pt.begin();
@@ -1899,7 +1808,7 @@ int mtpc_window_logprob_backward(mtpc_head* head, const void* hidden, const int3
   fwd.lse_out = reinterpret_cast<float*>(bw + B.off_lse);
   fwd.logit_out = reinterpret_cast<float*>(bw + B.off_logits);
   fwd.logit_pitch = B.Nc;
-  rc = launch_gemm(head, kModeLogprob, hb, T, 1, true, true, targets, nullptr, nullptr, st, &fwd);
+  rc = launch_gemm(head, hb, T, true, true, targets, st, &fwd);
   pt.end();
   if (rc != MTPC_OK) return rc;
   // 2. circuit backward: posteriors of the input units and of the sum units
@@ -2033,7 +1942,7 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   fwd.logit_out = reinterpret_cast<float*>(bw + B.off_logits);
   fwd.logit_pitch = B.Nc;
   rc = factored ? launch_lowrank_projection(head, hb, T, targets, st, fwd.lse_out)
-                : launch_gemm(head, kModeLogprob, hb, T, 1, true, true, targets, nullptr, nullptr, st, &fwd);
+                : launch_gemm(head, hb, T, true, true, targets, st, &fwd);
   if (rc != MTPC_OK) return rc;
   loss_coeff_kernel<<<num_sequences, kLossThreads, 0, st>>>(targets, coeff, sequence_length, c.n, num_sequences, gamma);
   head->launches++;
@@ -2297,9 +2206,8 @@ int mtpc_debug_set_projection_variant(mtpc_head* head, int32_t variant) {
 int mtpc_debug_set_draft_grouping(mtpc_head* head, int32_t mode) {
   if (!head) return MTPC_ERR_NULL;
   if (mode < 0 || mode > 2) return MTPC_ERR_SHAPE;
-  if (mode == 2 && head->L.group_entries == 0) return MTPC_ERR_UNSUPPORTED;
-  head->draft_grouping = mode;
-  return MTPC_OK;
+  if (mode == 2 && head->cfg.max_positions <= head->L.decode_max_p) return MTPC_ERR_UNSUPPORTED;
+  return MTPC_OK;                      // one implementation: the modes draw the same bytes
 }
 
 int mtpc_launch_count(mtpc_head* head, uint64_t* out_count) {

@@ -1,5 +1,4 @@
-// Circuit evaluation in log space (Eq. CP, Eq. HMM, Eq. BTree), latent ancestral sampling (Algorithm 1, sum
-// units) and the small preparation kernels. One warp evaluates one window; lane = latent value.
+// Circuit evaluation in log space (Eq. CP, Eq. HMM, Eq. BTree) and the small preparation kernels.
 #pragma once
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -623,57 +622,6 @@ __global__ void __launch_bounds__(32 * kHmmWarps) circuit_hmm_kernel(
         if (lane == 0) out[w] = res;
       }
     }
-  }
-}
-
-// ---------------------------------------------------------------- latent draws (Algorithm 1, sum units)
-// Inverse CDF over r log-probabilities: the smallest j with u < p_0 + ... + p_j, else r - 1.
-__device__ __forceinline__ int inv_cdf_logp(const float* __restrict__ logp, int r, float u) {
-  float cum = 0.f;
-  int found = r - 1;
-  bool hit = false;
-  for (int j = 0; j < r; ++j) {
-    cum += expf(logp[j]);
-    if (!hit && u < cum) { hit = true; found = j; }
-  }
-  return found;
-}
-
-// One thread per window. Writes unit_sel[w, i] = the input unit chosen for token i and presets out_bytes to -1.
-__global__ void latent_sample_kernel(int family, const float* __restrict__ logw, const float* __restrict__ logA,
-                                     const float* __restrict__ uniforms, int* __restrict__ unit_sel,
-                                     int* __restrict__ out_bytes, unsigned* status, int W, int wpp, int n, int r,
-                                     int sum_rows, int logA_stride) {
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= W) return;
-  const float* lw = logw + static_cast<size_t>(w / wpp) * sum_rows;
-  const float* u = uniforms + static_cast<size_t>(w) * 2 * n;
-  int* sel = unit_sel + static_cast<size_t>(w) * n;
-  bool bad = false;
-  for (int i = 0; i < n; ++i) out_bytes[static_cast<size_t>(w) * n + i] = -1;
-  const int nlat = (family == 0) ? 1 : (family == 1 ? n : n - 1);
-  for (int i = 0; i < nlat; ++i) bad |= !(u[i] >= 0.f && u[i] < 1.f);
-  if (bad) {
-    atomicOr(status, 2u);
-    for (int i = 0; i < n; ++i) sel[i] = -1;
-    return;
-  }
-  if (family == 0) {
-    const int z = inv_cdf_logp(lw, r, u[0]);
-    for (int i = 0; i < n; ++i) sel[i] = z;
-  } else if (family == 1) {
-    int z = inv_cdf_logp(lw, r, u[0]);
-    sel[0] = z;
-    for (int i = 1; i < n; ++i) {
-      z = inv_cdf_logp(logA + static_cast<size_t>(w / wpp) * logA_stride + (static_cast<size_t>(i - 1) * r + z) * r, r, u[i]);
-      sel[i] = z;
-    }
-  } else {
-    int zs[63];
-    zs[0] = inv_cdf_logp(lw, r, u[0]);
-    for (int j = 1; j < n - 1; ++j)
-      zs[j] = inv_cdf_logp(lw + r + (static_cast<size_t>(j - 1) * r + zs[(j - 1) >> 1]) * r, r, u[j]);
-    for (int i = 0; i < n; ++i) sel[i] = zs[n / 2 - 1 + (i >> 1)];
   }
 }
 

@@ -594,6 +594,98 @@ __global__ void __launch_bounds__(kSlotThreads, 2) draft_slot_kernel(
   }
 }
 
+// ---------------------------------------------------------------- draft of many positions
+// Latent draws (Algorithm 1 at the sum units), one warp per window, lane = latent value. Writes unit_sel[w, i] = the input unit
+// chosen for token i and presets out_bytes to -1; a window with a uniform outside [0,1) gets -1 throughout. (One thread per
+// window walking r entries per draw took 57 us for 4096 windows of a 16-leaf tree, 15 dependent draws each; this 14 us.)
+constexpr int kLatentWarps = 4;
+__global__ void __launch_bounds__(32 * kLatentWarps) latent_sample_kernel(
+    int family, const float* __restrict__ logw, const float* __restrict__ logA, const float* __restrict__ uniforms,
+    int* __restrict__ unit_sel, int* __restrict__ out_bytes, unsigned* status, int W, int wpp, int n, int r, int sum_rows,
+    int logA_stride) {
+  __shared__ int zs[kLatentWarps][64];
+  const int w = blockIdx.x * kLatentWarps + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (w >= W) return;
+  int* z = zs[threadIdx.x >> 5];
+  const float* lw = logw + static_cast<size_t>(w / wpp) * sum_rows;
+  const float* u = uniforms + static_cast<size_t>(w) * 2 * n;
+  const int nlat = (family == 0) ? 1 : (family == 1 ? n : n - 1);
+  bool bad = false;
+  for (int c = lane; c < nlat; c += 32) bad |= !(u[c] >= 0.f && u[c] < 1.f);
+  bad = __any_sync(kFull, bad);
+  if (bad) {
+    if (lane == 0) atomicOr(status, 2u);
+  } else {
+    const int root = r > 32 ? warp_inv_cdf_logits_wide(lw, r, u[0], lane) : warp_inv_cdf_logp(lane < r ? lw[lane] : 0.f, r, u[0], lane);
+    if (lane == 0) z[0] = root;
+    int prev = root;
+    for (int j = 1; j < nlat; ++j) {
+      const float* tab = family == 1 ? logA + static_cast<size_t>(w / wpp) * logA_stride + (static_cast<size_t>(j - 1) * r + prev) * r
+                                     : lw + r + (static_cast<size_t>(j - 1) * r + z[(j - 1) >> 1]) * r;
+      prev = warp_inv_cdf_logp(lane < r ? tab[lane] : 0.f, r, u[j], lane);
+      if (lane == 0) z[j] = prev;
+      __syncwarp();
+    }
+    __syncwarp();
+  }
+  for (int i = lane; i < n; i += 32) {
+    unit_sel[static_cast<size_t>(w) * n + i] = bad ? -1 : (family == 0 ? z[0] : family == 1 ? z[i] : z[n / 2 - 1 + (i >> 1)]);
+    out_bytes[static_cast<size_t>(w) * n + i] = -1;
+  }
+}
+
+// Byte draws of a draft whose logits were kept by the projection kernel: one warp per (window, slot) draws the byte by inverse
+// CDF from the logits of the unit the latent draw selected and gathers its evidence G[w, i, k] = log phi_k(byte) from the
+// slot's r units. 4 v + 36 r bytes per pair; bound by three dependent trips to memory. (The projection of the drafted bytes'
+// evidence, and a sampling projection on hidden states sorted by unit before it, are what keeping the logits replaces: 2232 +
+// 217 + 74 us at 4096 positions of the n = 16, r = 32, v = 256 tree, against 206 us more for the projection that keeps them
+// and 67 us here.)
+template <bool WIDE>   // units of more than 512 symbols: 512 at a time, as in draft_slot_kernel
+__global__ void __launch_bounds__(256) draft_pick_kernel(const float* __restrict__ logits, const float* __restrict__ unit_lse,
+                                                         const int* __restrict__ unit_sel, const float* __restrict__ uniforms,
+                                                         int* __restrict__ out_bytes, float* __restrict__ G, unsigned* status,
+                                                         int pairs, int wpp, int n, int r, int v, int vv) {
+  const int e = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (e >= pairs) return;
+  const int w = e / n, i = e - w * n;
+  const size_t unit0 = (static_cast<size_t>(w / wpp) * n + i) * r;
+  const float* row = logits + unit0 * v;                   // [r, v] logits of this slot
+  const int z = unit_sel[e];
+  const float ub = uniforms[static_cast<size_t>(w) * 2 * n + n + i];
+  int byte = -1;
+  if (z >= 0) {
+    if (!(ub >= 0.f && ub < 1.f)) {
+      if (lane == 0) atomicOr(status, 2u);
+    } else {
+      const float* x = row + static_cast<size_t>(z) * v;
+      const float m = unit_lse[unit0 + z];                 // the weights are then probabilities
+      if (!WIDE) {
+        byte = warp_inv_cdf_chunk<kSlotMaxPerLane>(x, 0, (v + 31) / 32, vv, m, ub, true, lane);
+      } else {
+        constexpr int kChunk = kSlotMaxPerLane * 32;
+        double total = 0.0;
+        for (int c0 = 0; c0 < v; c0 += kChunk) total += static_cast<double>(warp_chunk_sum(x, c0, vv, m, lane));
+        const double thr = static_cast<double>(ub) * total;
+        double before = 0.0;
+        byte = vv - 1;                                     // rounding may leave no index: the last one
+        for (int c0 = 0; c0 < v; c0 += kChunk) {
+          const float cs = warp_chunk_sum(x, c0, vv, m, lane);
+          if (thr < before + static_cast<double>(cs)) {
+            byte = warp_inv_cdf_chunk<kSlotMaxPerLane>(x, c0, kSlotMaxPerLane, vv, m, static_cast<float>(thr - before), false, lane);
+            break;
+          }
+          before += static_cast<double>(cs);
+        }
+      }
+    }
+  }
+  if (lane == 0) out_bytes[e] = byte;
+  for (int k = lane; k < r; k += 32)
+    G[static_cast<size_t>(e) * r + k] = byte < 0 ? CUDART_NAN_F : row[static_cast<size_t>(k) * v + byte] - unit_lse[unit0 + k];
+}
+
 // ---------------------------------------------------------------- acceptance stage (Algorithm 3)
 constexpr int kAcceptMaxThreads = 512;
 
@@ -616,7 +708,7 @@ inline int accept_threads(int v) { return v >= kAcceptMaxThreads ? kAcceptMaxThr
 // memory), a thread then has all the logits of its byte in flight, and the scan over the bytes is one warp scan plus the
 // warps' totals. With the recursions gone from it (they were one warp's serial chain through the tables) and launched as a
 // programmatic dependent the kernel went from 59 to 6 us at HMM n = 16, 128 windows; 12 to 5 us for one mixture window; 569 to
-// 49 us for 4096 tree windows of n = 16. row_of != NULL (after a many-position draft): `logits` [rows, r v] and `unit_lse` [rows, r] hold only the
+// 49 us for 4096 tree windows of n = 16. row_of != NULL (logits recomputed after a long draft): `logits` [rows, r v] and `unit_lse` [rows, r] hold only the
 // slot of each rejected window's first rejected byte, at row row_of[w].
 __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
     const float* __restrict__ logits, const float* __restrict__ unit_lse, const float* __restrict__ msg,

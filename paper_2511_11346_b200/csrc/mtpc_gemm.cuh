@@ -1,8 +1,7 @@
 // Projection kernel of the MtPC head (Sec. 3.3): logits = h W^T on the tcgen05 tensor cores, with the softmax
-// over the vocabulary, the evidence gather (log phi at the target byte) or the inverse-CDF byte draw
-// (Algorithm 1, input units), and the log-softmax of the sum-unit logits all done in the epilogue straight
-// out of tensor memory. The [positions, n, r, v] logit tensor never exists in HBM, except when a training call asks the
-// epilogue to keep it for the backward pass (logit_out).
+// over the vocabulary, the evidence gather (log phi at the target byte) and the log-softmax of the sum-unit logits all done
+// in the epilogue straight out of tensor memory. The [positions, n, r, v] logit tensor never exists in HBM, except when a
+// training call or a draft of many positions asks the epilogue to keep it (logit_out).
 //
 // One persistent CTA per SM, 6 warps:
 //   warp 0      TMA producer: per 64-wide K block, one 128-row tile of h and the v rows of one emission unit
@@ -15,8 +14,7 @@
 // boundary, covered by accumulator tiles of `tile_cols` columns. The log-likelihood mode uses 256-column tiles
 // whatever v is (v=320: 4 units = 1280 rows = 5 tiles; v=256: 1 unit = 1 tile): a tile may then hold the end
 // of one unit and the start of the next, and the epilogue carries its running max / sum across tiles and
-// closes a unit whenever its v-th column has been consumed. The sampling mode needs a whole unit on chip at
-// once and uses one unit per group (v=320 -> 2 tiles of 160). Sum-unit rows form work items of their own
+// closes a unit whenever its v-th column has been consumed. Sum-unit rows form work items of their own
 // (one tile of `sum_cols` columns). Accumulators live in a ring of TMEM slots, so the epilogue of one tile
 // overlaps the MMAs of the next. Every barrier wait is bounded: when one runs out the CTA raises
 // MTPC_STATUS_TIMEOUT in the status word, drains its copies, frees its TMEM and returns.
@@ -40,13 +38,11 @@ constexpr uint64_t kAbortSettleNs = 200ull * 1000ull;            // 0.2 ms: far 
 constexpr int kABytes = kBlockM * kBlockK * 2;                   // 16 KB
 constexpr uint32_t kStatusBadTarget = 1u, kStatusBadUniform = 2u, kStatusTimeout = 4u;
 
-// kModeSampleGrouped: the byte draws again, on rows that were sorted by the unit they sample from (mtpc_group.cuh):
-// a work item is one GroupTile instead of (m-tile, unit).
 // kModeLogitsGrouped: rows sorted by SLOT (the acceptance stage after a many-position draft): a work item is a GroupTile
 // whose `unit` is a slot and a run of group_units of the slot's r units; their logits and log-sum-exps are written out per
 // staged row. (There are only about n + rows / 128 tiles: without the split over units a batch of 4096 windows of 16 slots
 // is 45 items for 148 SMs, each r v columns long: 623 us against 213.)
-enum { kModeLogprob = 0, kModeSample = 1, kModeSampleGrouped = 2, kModeLogitsGrouped = 3 };
+enum { kModeLogprob = 0, kModeLogitsGrouped = 1 };
 
 struct GemmParams {
   CUtensorMap tm_a;      // hidden  [T, d]        box 64 x 128
@@ -65,22 +61,15 @@ struct GemmParams {
   int sum_cols, sum_rows;            // sum tile width; S * r
   int slot_stride, num_slots;
   int stages, stage_bytes;
-  int wpp;                           // windows (target rows) per position
-  const int* targets;                // [T*wpp, n]
-  int missing_is_nan;                // a negative target is a refused draw (G = NaN), not a byte to sum out (G = 0)
-  float* G;                          // [T*wpp, n, r]   log phi at the target
+  const int* targets;                // [T, n] or NULL (a draft: no evidence yet, the logits are kept)
+  float* G;                          // [T, n, r]       log phi at the target
   float* logw;                       // [T, S*r]        log-softmaxed sum-unit weights
   const float* sum_bias;             // [S*r] or NULL   added to the sum-unit logits before their softmax
-  float* lse_out;                    // [T, n, r] or NULL: log-sum-exp of every input unit, kept for the backward pass
+  float* lse_out;                    // [T, n, r] or NULL: log-sum-exp of every input unit, kept for the backward pass or a draft
   float* logit_out;                  // [T, n*r*v] fp32 with row pitch logit_pitch, or NULL: the emission logits themselves,
-  size_t logit_pitch;                // kept for the backward pass (padding columns as -inf); wpp == 1 only
-  const int* unit_sel;               // [T*wpp, n]      selected input unit per token (sample mode)
-  const float* uniforms;             // [T*wpp, 2n]
-  int* out_bytes;                    // [T*wpp, n]
-  const GroupTile* group_tiles;      // grouped sampling: the work items, ...
-  const int* group_num_tiles;        // ... how many there are (device memory: written by the kernel that made them), ...
-  const int* group_perm;             // ... and which (window, slot) pair every row of the staged hidden states (tm_a) holds
-  int group_two_pass;                // grouped sampling of a unit too wide for tensor memory: its tiles are computed twice
+  size_t logit_pitch;                // kept for the backward pass or a draft (padding columns as -inf)
+  const GroupTile* group_tiles;      // sorted rows: the work items, and ...
+  const int* group_num_tiles;        // ... how many there are (device memory: written by the kernel that made them)
   unsigned* status;
   uint64_t wait_limit_ns;            // limit of every pipeline wait (kWaitLimitNs unless a test shortened it)
 };
@@ -136,23 +125,20 @@ __device__ __forceinline__ bool bounded_wait_warp(uint32_t bar, uint32_t parity,
 struct TileCoord {
   int mt, is_sum, ntiles, cols, brow0, unit0, nunits;
   int arow, count;   // first row of the A operand and the rows that count (set by the caller for ungrouped items)
-  int wrap;          // tiles per sweep over the item's weight rows: tile t reads the rows of tile t % wrap
 };
-// A grouped item: `count` staged rows from `row0` on, against the tiles of the one unit they sample from (by_slot: of
-// group_units of the r units of the one slot whose logits they need; the runs of one row tile follow each other).
-__device__ __forceinline__ TileCoord group_coord(const GemmParams& p, int item, bool by_slot) {
-  const int runs = by_slot ? p.num_groups : 1;
-  const int tile = item / runs, first = (item - tile * runs) * p.group_units;
+// A grouped item: `count` staged rows from `row0` on, against the tiles of group_units of the r units of the one slot whose
+// logits they need; the runs of one row tile follow each other.
+__device__ __forceinline__ TileCoord group_coord(const GemmParams& p, int item) {
+  const int tile = item / p.num_groups, first = (item - tile * p.num_groups) * p.group_units;
   const GroupTile g = p.group_tiles[tile];
   TileCoord c;
   c.mt = 0;
   c.is_sum = 0;
-  c.unit0 = by_slot ? g.unit * p.r + first : g.unit;
-  c.nunits = by_slot ? min(p.group_units, p.r - first) : 1;
+  c.unit0 = g.unit * p.r + first;
+  c.nunits = min(p.group_units, p.r - first);
   c.cols = p.tile_cols;
   c.brow0 = c.unit0 * p.v;
-  c.wrap = (c.nunits * p.v + p.tile_cols - 1) / p.tile_cols;
-  c.ntiles = p.group_two_pass ? 2 * c.wrap : c.wrap;
+  c.ntiles = (c.nunits * p.v + p.tile_cols - 1) / p.tile_cols;
   c.arow = g.row0;
   c.count = g.count;
   return c;
@@ -242,17 +228,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  constexpr bool kGrouped = MODE == kModeSampleGrouped || MODE == kModeLogitsGrouped;
+  constexpr bool kGrouped = MODE == kModeLogitsGrouped;
   static_assert(!kGrouped || CTAS == 1, "grouped tiles are ragged: no pairing");
-  const int num_items = kGrouped ? *p.group_num_tiles * (MODE == kModeLogitsGrouped ? p.num_groups : 1)
-                                 : (p.num_groups + p.num_sum_tiles) * p.m_units;
+  const int num_items = kGrouped ? *p.group_num_tiles * p.num_groups : (p.num_groups + p.num_sum_tiles) * p.m_units;
   const uint32_t cta_rank = CTAS == 2 ? cluster_cta_rank() : 0u;      // 0 = the pair's leader
   auto coord = [&](int item) {
-    if (kGrouped) return group_coord(p, item, MODE == kModeLogitsGrouped);
+    if (kGrouped) return group_coord(p, item);
     TileCoord c = tile_coord(p, item);
     c.arow = (c.mt * CTAS + static_cast<int>(cta_rank)) * kBlockM;
     c.count = min(kBlockM, p.T - c.arow);                             // <= 0: a pair's second CTA past the last position
-    c.wrap = c.ntiles;
     return c;
   };
   const int first_item = CTAS == 2 ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
@@ -305,7 +289,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
           for (int kb = 0; kb < p.kblocks; ++kb) {
             if (!bounded_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
             const uint32_t a_dst = tiles_addr + stage * p.stage_bytes;
-            const int brow = tc.brow0 + (t % tc.wrap) * tc.cols + static_cast<int>(cta_rank) * brows;
+            const int brow = tc.brow0 + t * tc.cols + static_cast<int>(cta_rank) * brows;
             if (CTAS == 2) {
               const uint32_t full = cluster_map_shared(smem_u32(&ctl->full[stage]), 0);   // the leader's barrier
               if (cta_rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[stage]), bytes);
@@ -519,16 +503,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
           if (lane == 0) release_slot(slot);
         }
         if (!ok) break;
-      } else if (MODE == kModeLogprob) {
+      } else {
         // ---- log phi at the target byte: online log-sum-exp over the v columns of each unit + gather. The
         // running (m, s) and the gathered logit live across tile boundaries; a unit is closed when its v-th
         // column has been consumed.
-        const size_t wrow0 = static_cast<size_t>(valid ? row : 0) * p.wpp;
+        const int* tgts = (valid && p.targets != nullptr) ? p.targets + static_cast<size_t>(row) * p.n : nullptr;
         const int units_end = tc.unit0 + tc.nunits;
         int unit = tc.unit0, col_in_unit = 0;
         int slot_i = unit / p.r, k = unit - slot_i * p.r;
         float m = -CUDART_INF_F, s = 0.f, tval = 0.f;
-        int tgt = (p.wpp == 1 && valid) ? p.targets[wrow0 * p.n + slot_i] : -1;
+        int tgt = tgts != nullptr ? tgts[slot_i] : -1;
         for (int t = 0; t < tc.ntiles && ok; ++t, ++use) {
           const uint32_t slot = use % p.num_slots;
           if (!bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use / p.num_slots) & 1u, ctl, p.status, lane)) {
@@ -557,24 +541,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
 #pragma unroll
             for (int q = 0; q < 16; ++q) s += fast_ex2(fmaf(x[q], kLog2e, -mn2));
             m = mn;
-            if (p.wpp == 1) {
-              const int rel = tgt - col_in_unit;
-              if (static_cast<unsigned>(rel) < 16u) {
+            const int rel = tgt - col_in_unit;
+            if (static_cast<unsigned>(rel) < 16u) {
 #pragma unroll
-                for (int q = 0; q < 16; ++q)
-                  if (rel == q) tval = x[q];
-              }
-            } else if (valid) {
-              for (int j = 0; j < p.wpp; ++j) {
-                const int rel = p.targets[(wrow0 + j) * p.n + slot_i] - col_in_unit;
-                if (static_cast<unsigned>(rel) < 16u) {
-                  float val = 0.f;
-#pragma unroll
-                  for (int q = 0; q < 16; ++q)
-                    if (rel == q) val = x[q];
-                  p.G[((wrow0 + j) * p.n + slot_i) * p.r + k] = val;   // raw logit; normalised below
-                }
-              }
+              for (int q = 0; q < 16; ++q)
+                if (rel == q) tval = x[q];
             }
             col_in_unit += 16;
             if (col_in_unit == p.v) {
@@ -582,18 +553,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
               const float lse = m + fast_lg2(s) * kLn2;
               if (valid && p.lse_out != nullptr)
                 p.lse_out[(static_cast<size_t>(row) * p.n + slot_i) * p.r + k] = lse;
-              if (valid) {
-                for (int j = 0; j < p.wpp; ++j) {
-                  const int tj = (p.wpp == 1) ? tgt : p.targets[(wrow0 + j) * p.n + slot_i];
-                  float* g = p.G + ((wrow0 + j) * p.n + slot_i) * p.r + k;
-                  if (tj < 0) {
-                    *g = p.missing_is_nan ? CUDART_NAN_F : 0.f;   // marginalised byte: the input unit sums to 1
-                  } else if (tj >= p.vv) {
-                    *g = CUDART_NAN_F;
-                    atomicOr(p.status, kStatusBadTarget);
-                  } else {
-                    *g = ((p.wpp == 1) ? tval : *g) - lse;
-                  }
+              if (tgts != nullptr) {
+                float* g = p.G + (static_cast<size_t>(row) * p.n + slot_i) * p.r + k;
+                if (tgt < 0) {
+                  *g = 0.f;                              // marginalised byte: the input unit sums to 1
+                } else if (tgt >= p.vv) {
+                  *g = CUDART_NAN_F;
+                  atomicOr(p.status, kStatusBadTarget);
+                } else {
+                  *g = tval - lse;
                 }
               }
               ++unit;
@@ -602,7 +570,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
               if (unit < units_end) {
                 slot_i = unit / p.r;
                 k = unit - slot_i * p.r;
-                tgt = (p.wpp == 1 && valid) ? p.targets[wrow0 * p.n + slot_i] : -1;
+                tgt = tgts != nullptr ? tgts[slot_i] : -1;
               }
             }
             return unit < units_end;
@@ -630,157 +598,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
           if (lane == 0) release_slot(slot);
         }
         if (!ok) break;
-      } else {
-        // ---- byte draws (Algorithm 1, input units): inverse CDF of softmax(logits) for every window of this
-        // row whose selected unit for this slot is k. One unit per group: all its tiles stay in TMEM until the end.
-        const int slot_i = tc.unit0 / p.r;
-        const int k = tc.unit0 - slot_i * p.r;
-        unsigned long long pending = 0ull;
-        size_t wrow0 = 0;
-        int nwin = p.wpp;
-        if (MODE == kModeSampleGrouped) {
-          // the row holds one (window, slot) pair, and the slot is this tile's
-          if (valid) { wrow0 = static_cast<size_t>(p.group_perm[row] / p.n); pending = 1ull; }
-          nwin = 1;
-        } else {
-          wrow0 = static_cast<size_t>(valid ? row : 0) * p.wpp;
-          if (valid)
-            for (int j = 0; j < nwin; ++j)
-              if (p.unit_sel[(wrow0 + j) * p.n + slot_i] == k) pending |= 1ull << j;
-        }
-        if (MODE == kModeSampleGrouped && p.group_two_pass) {
-          // ---- a unit wider than tensor memory: its tiles stream through the accumulator ring twice. Sweep 1: running
-          // maximum and sum of exponentials (the sum in fp64, 16 terms at a time, so that tens of thousands of terms
-          // keep the precision the draw needs). Sweep 2: the scan u * total < running sum over the recomputed tiles.
-          const float uval = valid ? p.uniforms[wrow0 * (2 * p.n) + p.n + slot_i] : 0.f;
-          float m = -CUDART_INF_F;
-          double total = 0.0, cum = 0.0, thr = 0.0;
-          int found = p.vv - 1;   // rounding may leave no index: the last one
-          bool hit = false;
-          for (int t = 0; t < tc.ntiles && ok; ++t, ++use) {
-            const uint32_t slot = use % p.num_slots;
-            if (!bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use / p.num_slots) & 1u, ctl, p.status, lane)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t tcol = lane_base + slot * p.slot_stride;
-            const bool second = t >= tc.wrap;
-            if (t == tc.wrap) thr = static_cast<double>(uval) * total;
-            const int col_tile = (t % tc.wrap) * tc.cols;
-            for (int b = 0; b < nbatch && col_tile + b * 16 < p.vv; ++b) {
-              float x[16];
-              tmem_ld16(tcol + b * 16, x);
-              const int col0 = col_tile + b * 16;
-              mask_padding(x, col0, p.vv);
-              if (!second) {
-                float bm = x[0];
-#pragma unroll
-                for (int q = 1; q < 16; ++q) bm = fmaxf(bm, x[q]);
-                if (bm > m) {                                   // rescale what was summed so far to the new maximum
-                  total *= static_cast<double>(fast_ex2((m - bm) * kLog2e));
-                  m = bm;
-                }
-                const float m2 = m * kLog2e;
-                float part = 0.f;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) part += fast_ex2(fmaf(x[q], kLog2e, -m2));
-                total += static_cast<double>(part);
-              } else if (!hit) {
-                const float m2 = m * kLog2e;
-                const float rest = static_cast<float>(thr - cum);   // what the threshold still needs inside this batch
-                float part = 0.f;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                  part += fast_ex2(fmaf(x[q], kLog2e, -m2));
-                  if (!hit && rest < part) { hit = true; found = col0 + q; }
-                }
-                cum += static_cast<double>(part);
-              }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) release_slot(slot);
-          }
-          if (!ok) break;
-          if (valid) {
-            if (!(uval >= 0.f && uval < 1.f)) {
-              found = -1;
-              atomicOr(p.status, kStatusBadUniform);
-            }
-            p.out_bytes[wrow0 * p.n + slot_i] = found;
-          }
-          continue;
-        }
-        for (int c = 0; c < tc.ntiles && ok; ++c) {
-          const uint32_t u = use + c;
-          if (!bounded_wait_warp(smem_u32(&ctl->tfull[u % p.num_slots]), (u / p.num_slots) & 1u, ctl, p.status,
-                                 lane))
-            ok = false;
-        }
-        if (!ok) break;
-        tc_fence_after();
-        if (__any_sync(0xffffffffu, pending != 0ull)) {
-          float m = -CUDART_INF_F;
-          for (int c = 0; c < tc.ntiles; ++c) {
-            const uint32_t tcol = lane_base + ((use + c) % p.num_slots) * p.slot_stride;
-            for (int b = 0; b < nbatch; ++b) {
-              float x[16];
-              tmem_ld16(tcol + b * 16, x);
-              mask_padding(x, c * tc.cols + b * 16, p.vv);
-#pragma unroll
-              for (int q = 0; q < 16; ++q) m = fmaxf(m, x[q]);
-            }
-          }
-          const float m2 = m * kLog2e;
-          float total = 0.f;   // same terms in the same order as the running sum of the scan below
-          for (int c = 0; c < tc.ntiles; ++c) {
-            const uint32_t tcol = lane_base + ((use + c) % p.num_slots) * p.slot_stride;
-            for (int b = 0; b < nbatch; ++b) {
-              float x[16];
-              tmem_ld16(tcol + b * 16, x);
-              mask_padding(x, c * tc.cols + b * 16, p.vv);
-#pragma unroll
-              for (int q = 0; q < 16; ++q) total += fast_ex2(fmaf(x[q], kLog2e, -m2));
-            }
-          }
-          while (__any_sync(0xffffffffu, pending != 0ull)) {
-            const int j = pending ? __ffsll(static_cast<long long>(pending)) - 1 : -1;
-            float uval = 0.f;
-            if (j >= 0) uval = p.uniforms[(wrow0 + j) * (2 * p.n) + p.n + slot_i];
-            const float thr = uval * total;
-            float cum = 0.f;
-            int found = p.vv - 1;   // rounding may leave no index: the last one
-            bool hit = false;
-            for (int c = 0; c < tc.ntiles; ++c) {
-              const uint32_t tcol = lane_base + ((use + c) % p.num_slots) * p.slot_stride;
-              for (int b = 0; b < nbatch; ++b) {
-                float x[16];
-                tmem_ld16(tcol + b * 16, x);
-                const int col0 = c * tc.cols + b * 16;
-                mask_padding(x, col0, p.vv);
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                  cum += fast_ex2(fmaf(x[q], kLog2e, -m2));
-                  if (!hit && thr < cum) { hit = true; found = col0 + q; }
-                }
-              }
-            }
-            if (j >= 0) {
-              if (!(uval >= 0.f && uval < 1.f)) {
-                found = -1;
-                atomicOr(p.status, kStatusBadUniform);
-              }
-              p.out_bytes[(wrow0 + j) * p.n + slot_i] = found;
-              pending &= pending - 1ull;
-            }
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0)
-          for (int c = 0; c < tc.ntiles; ++c) release_slot((use + c) % p.num_slots);
-        use += tc.ntiles;
       }
     }
   }

@@ -1,13 +1,12 @@
-// Grouping of the byte draws of a many-position draft by the input unit they sample from (Algorithm 1, input-unit
-// step). After the latent draws every (window, slot) pair knows its unit (i, z). A counting sort over the n*r units
-// packs the hidden states of the pairs that share a unit into consecutive rows of a staging buffer, so that the
-// sampling pass of the projection kernel multiplies each pair by the one unit it samples from: windows * n * v * d
-// multiply-adds instead of positions * n * r * v * d.
-//   group_count_kernel   histogram of the pairs over the units
-//   group_scan_kernel    exclusive scan -> first staging row of every unit, and the list of 128-row tiles
-//   group_gather_kernel  every pair takes the next free row of its unit and copies its hidden state there
-// The order of the pairs inside a unit depends on the order of the atomic increments; nothing downstream depends on it
-// (every row is sampled on its own, with its own uniform).
+// Sorting of the rejected windows of a long draft by the slot of their first rejected byte (Algorithm 3), for drafts whose
+// logits did not fit the workspace: the acceptance stage recomputes that slot's logits. A counting sort over the n slots packs
+// the hidden states of the windows that share a slot into consecutive rows of a staging buffer, so that one pass of the
+// projection kernel multiplies each by the r units of its slot only.
+//   group_count_kernel   histogram of the windows over the slots
+//   group_scan_kernel    exclusive scan -> first staging row of every slot, and the list of 128-row tiles
+//   group_gather_kernel  every window takes the next free row of its slot and copies its hidden state there
+// The order inside a slot depends on the order of the atomic increments; nothing downstream depends on it. (The kernels sort
+// entries e by the key (e % n) * r + unit_sel[e]; the acceptance stage calls them with n = 1 and r slots.)
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -18,8 +17,7 @@ constexpr int kGroupThreads = 256;
 constexpr int kGroupScanThreads = 1024;
 constexpr int kGroupMaxUnits = 8192;    // n <= 64 slots x r <= 128 units
 
-// One tile of the grouped sampling pass: `count` <= 128 staging rows starting at `row0`, all sampling from emission
-// unit `unit` (= slot * r + component).
+// One tile of the sorted pass: `count` <= 128 staging rows starting at `row0`, all of key `unit` (a slot).
 struct GroupTile {
   int unit, row0, count, pad;
 };

@@ -326,23 +326,39 @@ struct PhaseTimer {
 int check_launch() { return cudaGetLastError() == cudaSuccess ? MTPC_OK : MTPC_ERR_CUDA; }
 
 // Launch `kernel`, optionally allowed to start before the kernel ahead of it in the stream has finished (programmatic
-// dependent launch): such a kernel calls grid_dependency_wait() before it touches the earlier kernel's results.
+// dependent launch): such a kernel calls grid_dependency_wait() before it touches global memory, so what overlaps is its launch and
+// set-up (about 2 us a kernel). cluster > 1: in clusters of that many CTAs.
 template <typename... Params, typename... Args>
-void launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent,
-                   Args&&... args) {
+void launch_clusters(void (*kernel)(Params...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent,
+                     Args&&... args) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (dependent) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = cluster;
+    attr[n].val.clusterDim.y = 1;
+    attr[n++].val.clusterDim.z = 1;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = dependent ? 1 : 0;
+  cfg.numAttrs = n;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
+template <typename... Params, typename... Args>
+void launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent, Args&&... args) {
+  launch_clusters(kernel, 1, grid, block, smem, st, dependent, args...);
+}
+// The kernels of a call follow each other as dependents, unless events are recorded between them.
+bool overlapped(const mtpc_head* h) { return h->ring == 0; }
 
 // Launch the projection kernel for `rows` positions over the emission groups (with_emit) and / or the sum tiles.
 // Units per work item of the log-likelihood mode. An item covers its units with 256-column tiles; unless the
@@ -397,9 +413,13 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
   if (rc != MTPC_OK) return rc;
   p.T = rows;
   p.m_tiles = (rows + kBlockM - 1) / kBlockM;
-  // Two CTAs per MMA when there are at least two m-tiles to pair up (and the device can hold a cluster at all)
-  const bool pair = grp == nullptr &&
-                    (h->projection_variant == 2 || (h->projection_variant == 0 && p.m_tiles >= 2 && h->max_pairs > 0));
+  // Two CTAs per MMA when there are at least two m-tiles to pair up (and the device can hold a cluster at all) and K is long
+  // enough for the halved operand traffic to count: with few K steps the epilogue bounds a tile, and a lone CTA need not wait
+  // for its partner's. Alone / in pairs, us, CP: d = 256, 32 units of 256 symbols, 256 positions 11.6 / 12.8; 128 units of 320,
+  // 8192 positions 375 / 400; d = 1024, 64 x 320, 256 positions 19.9 / 20.8; 128 x 320, 2048 positions 138.8 / 139.3; d = 1536,
+  // 128 x 320, 1024 positions 107.8 / 105.8; d = 2048, 256 positions 52.0 / 47.6; d = 4096, 64 x 320, 256 positions 67.3 / 60.7.
+  const bool pair = grp == nullptr && (h->projection_variant == 2 || (h->projection_variant == 0 && p.m_tiles >= 2 &&
+                                                                      h->max_pairs > 0 && c.d > 1024));
   const int ctas = pair ? 2 : 1;
   const int workers = pair ? h->max_pairs : h->num_sms;               // CTAs, or CTA pairs, resident at once
   p.m_units = (p.m_tiles + ctas - 1) / ctas;
@@ -446,26 +466,10 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
                               : static_cast<long long>(p.m_units) * (p.num_groups + p.num_sum_tiles);
   const int grid = ctas * static_cast<int>(items < workers ? items : workers);
   const size_t smem = pair ? tl.pair_smem : tl.smem;
-  if (grp) {
-    mtpc_gemm_kernel<kModeLogitsGrouped, 1><<<grid, kGemmThreads, smem, st>>>(p);
-  } else if (!pair) {
-    mtpc_gemm_kernel<kModeLogprob, 1><<<grid, kGemmThreads, smem, st>>>(p);
-  } else {
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, mtpc_gemm_kernel<kModeLogprob, 2>, p);
-  }
+  p.work_counter = with_sum ? p.status + kWorkCounterWord : nullptr;    // (the first launch of every call that needs it zeroed)
+  if (grp) launch_kernel(mtpc_gemm_kernel<kModeLogitsGrouped, 1>, grid, kGemmThreads, smem, st, overlapped(h), p);
+  else if (!pair) launch_kernel(mtpc_gemm_kernel<kModeLogprob, 1>, grid, kGemmThreads, smem, st, overlapped(h), p);
+  else launch_clusters(mtpc_gemm_kernel<kModeLogprob, 2>, 2, grid, kGemmThreads, smem, st, overlapped(h), p);
   h->launches++;
   return check_launch();
 }
@@ -481,9 +485,10 @@ int sms_times_resident(const mtpc_head* h, size_t smem) {
 
 // Circuit evaluation of W windows: out[w] = joint log-prob, prefix [W, n] = log-marginals of the prefixes x_0..x_i, msg
 // [W, n, r] = slot messages (each may be NULL, not all).
-// dependent: the launch directly follows draft_slot_kernel, which has zeroed the work counter, and may overlap its tail.
-int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cudaStream_t st, bool dependent = false,
-                   bool raw_mixture = false, float* msg = nullptr) {
+// (The tree's joint kernel hands out windows through a counter next to the status word, which the projection or
+// draft_slot_kernel before it has zeroed.)
+int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cudaStream_t st, bool raw_mixture = false,
+                   float* msg = nullptr) {
   if (W <= 0) return MTPC_OK;
   const mtpc_config& c = h->cfg;
   const Layout& L = h->L;
@@ -495,10 +500,10 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
   if (c.family == MTPC_CP && sweep) {
     const size_t per_warp = cp_prefix_warp_floats(c.n, c.r) * sizeof(float);
     const int warps = W <= h->num_sms || per_warp > 8192 ? 1 : 4;       // few windows: one per SM
-    launch_kernel(circuit_cp_prefix_kernel, (W + warps - 1) / warps, warps * 32, warps * per_warp, st, dependent, G, logw, out,
+    launch_kernel(circuit_cp_prefix_kernel, (W + warps - 1) / warps, warps * 32, warps * per_warp, st, overlapped(h), G, logw, out,
                   prefix, msg, W, wpp, c.n, c.r, L.sum_rows, raw_mixture ? 1 : 0);
   } else if (c.family == MTPC_CP) {
-    launch_kernel(circuit_cp_kernel, blocks, threads, 0, st, dependent, G, logw, out, W, wpp, c.n, c.r, L.sum_rows,
+    launch_kernel(circuit_cp_kernel, blocks, threads, 0, st, overlapped(h), G, logw, out, W, wpp, c.n, c.r, L.sum_rows,
                   raw_mixture ? 1 : 0);
   } else if (c.family == MTPC_HMM) {
     // as many tables as fit beside the warps' vectors (all of them but for very long windows)
@@ -508,21 +513,19 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
     const int stride = hmm_table_stride(h);
     const int items = stride == 0 ? (W + kHmmWarps - 1) / kHmmWarps : W / wpp * ((wpp + kHmmWarps - 1) / kHmmWarps);
     const int resident = sms_times_resident(h, smem);
-    launch_kernel(circuit_hmm_kernel, items < resident ? items : resident, kHmmWarps * 32, smem, st, dependent, G, logw,
+    launch_kernel(circuit_hmm_kernel, items < resident ? items : resident, kHmmWarps * 32, smem, st, overlapped(h), G, logw,
                   hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r, L.sum_rows, chunk);
   } else if (sweep) {
     const int warps = c.n / 2 < 8 ? c.n / 2 : 8;                         // a warp per node of the owners' level
     const bool fits = btree_prefix_smem_floats(c.n, c.r, warps, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
     const size_t smem = btree_prefix_smem_floats(c.n, c.r, warps, fits) * sizeof(float);
     const int resident = sms_times_resident(h, smem);
-    launch_kernel(circuit_btree_prefix_kernel, W < resident ? W : resident, warps * 32, smem, st, dependent, G, logw, out, prefix,
-                  msg, W, wpp, c.n, c.r, L.sum_rows, fits ? 1 : 0);
+    launch_kernel(circuit_btree_prefix_kernel, W < resident ? W : resident, warps * 32, smem, st, overlapped(h), G, logw, out,
+                  prefix, msg, W, wpp, c.n, c.r, L.sum_rows, fits ? 1 : 0);
   } else {
-    // windows are handed out through a counter next to the status word
     unsigned* counter = at<unsigned>(h, L.off_status) + kWorkCounterWord;
     const int resident = blocks < 8 * h->num_sms ? blocks : 8 * h->num_sms;   // more CTAs than an SM can hold do no harm
-    if (!dependent && cudaMemsetAsync(counter, 0, sizeof(unsigned), st) != cudaSuccess) return MTPC_ERR_CUDA;
-    launch_kernel(circuit_btree_kernel, resident, threads, btree_smem_bytes(c.n, c.r), st, dependent, G, logw, out, counter, W,
+    launch_kernel(circuit_btree_kernel, resident, threads, btree_smem_bytes(c.n, c.r), st, overlapped(h), G, logw, out, counter, W,
                   wpp, c.n, c.r, L.sum_rows);
   }
   h->launches++;
@@ -652,35 +655,23 @@ int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_
   p.sum_bias = sum_bias(h);
   p.status = at<unsigned>(h, L.off_status);
   p.wait_limit_ns = h->wait_limit_ns;
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(p.ksplit > 1 ? tiles * p.ksplit : tiles < h->num_sms ? tiles : h->num_sms);
-  cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = p.stages * p.stage_bytes + ctl;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  int nattr = 0;
-  if (h->ring == 0) {
-    attr[nattr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[nattr++].val.programmaticStreamSerializationAllowed = 1;
-  }
-  if (p.ksplit > 1) {
-    attr[nattr].id = cudaLaunchAttributeClusterDimension;
-    attr[nattr].val.clusterDim.x = p.ksplit;
-    attr[nattr].val.clusterDim.y = 1;
-    attr[nattr++].val.clusterDim.z = 1;
-  }
-  cfg.attrs = attr;
-  cfg.numAttrs = nattr;
-  cudaLaunchKernelEx(&cfg, mtpc_decode_gemm_kernel, p);
+  launch_clusters(mtpc_decode_gemm_kernel, p.ksplit, p.ksplit > 1 ? tiles * p.ksplit : tiles < h->num_sms ? tiles : h->num_sms,
+                  kGemmThreads, p.stages * p.stage_bytes + ctl, st, overlapped(h), p);
   h->launches++;
   if (h->lr_k > 0) {
     launch_kernel(lowrank_expand_kernel, dim3(c.n * c.r, (c.v + kExpandThreads - 1) / kExpandThreads), kExpandThreads,
-                  static_cast<size_t>(P) * h->lr_k * sizeof(float), st, h->ring == 0, p.logits, p.logits2,
+                  static_cast<size_t>(P) * h->lr_k * sizeof(float), st, overlapped(h), p.logits, p.logits2,
                   static_cast<const __nv_bfloat16*>(h->lr_A), at<float>(h, L.off_logits), P, c.n, c.r, c.v, h->lr_k);
     h->launches++;
   }
   return check_launch();
+}
+
+void round_to_bf16(const float* src, __nv_bfloat16* dst, size_t count, cudaStream_t st, bool dependent) {
+  const int vec = count % 8 == 0 && reinterpret_cast<uintptr_t>(src) % 16 == 0 && reinterpret_cast<uintptr_t>(dst) % 16 == 0;
+  const size_t blocks = ((vec ? count / 8 : count) + 255) / 256;
+  launch_kernel(f32_to_bf16_kernel, static_cast<unsigned>(blocks < 4096 ? blocks : 4096), 256, 0, st, dependent, src, dst,
+                count, vec);
 }
 
 // hidden (io_dtype, device) -> bf16 device pointer the GEMM reads
@@ -689,8 +680,7 @@ int stage_hidden(mtpc_head* h, const void* hidden, int rows, const void** out_bf
   __nv_bfloat16* dst = at<__nv_bfloat16>(h, h->L.off_hidden);
   const size_t count = static_cast<size_t>(rows) * h->cfg.d;
   if (count) {
-    const int blocks = static_cast<int>((count + 255) / 256 < 4096 ? (count + 255) / 256 : 4096);
-    f32_to_bf16_kernel<<<blocks, 256, 0, st>>>(static_cast<const float*>(hidden), dst, count);
+    round_to_bf16(static_cast<const float*>(hidden), dst, count, st, overlapped(h));
     h->launches++;
     if (check_launch() != MTPC_OK) return MTPC_ERR_CUDA;
   }
@@ -766,9 +756,9 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     pt.end();
     if (rc != MTPC_OK) return rc;
     pt.begin();
-    latent_sample_kernel<<<(W + kLatentWarps - 1) / kLatentWarps, 32 * kLatentWarps, 0, st>>>(
-        c.family, at<float>(h, L.off_logw), hmm_tables(h), uniforms, at<int>(h, L.off_sel), out_bytes, at<unsigned>(h, L.off_status), W,
-        wpp, c.n, c.r, L.sum_rows, hmm_table_stride(h));
+    launch_kernel(latent_sample_kernel, (W + kLatentWarps - 1) / kLatentWarps, 32 * kLatentWarps, 0, st, overlapped(h),
+                  c.family, at<float>(h, L.off_logw), hmm_tables(h), uniforms, at<int>(h, L.off_sel), out_bytes,
+                  at<unsigned>(h, L.off_status), W, wpp, c.n, c.r, L.sum_rows, hmm_table_stride(h));
     h->launches++;
     pt.end();
     if ((rc = check_launch()) != MTPC_OK) return rc;
@@ -778,9 +768,10 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
       const int pairs = W * c.n;
       int blocks = (pairs + kDrawWarps - 1) / kDrawWarps;
       if (blocks > 32 * h->num_sms) blocks = 32 * h->num_sms;
-      lowrank_draw_kernel<<<blocks, 32 * kDrawWarps, static_cast<size_t>(kDrawWarps) * c.v * sizeof(float), st>>>(
-          base, reinterpret_cast<const __nv_bfloat16*>(h->ws + h->lr_off_zhl), static_cast<const __nv_bfloat16*>(h->lr_A),
-          at<int>(h, L.off_sel), uniforms, out_bytes, at<unsigned>(h, L.off_status), W, wpp, c.n, c.r, c.v, valid_symbols(c), k);
+      launch_kernel(lowrank_draw_kernel, blocks, 32 * kDrawWarps, static_cast<size_t>(kDrawWarps) * c.v * sizeof(float), st,
+                    overlapped(h), base, reinterpret_cast<const __nv_bfloat16*>(h->ws + h->lr_off_zhl),
+                    static_cast<const __nv_bfloat16*>(h->lr_A), at<int>(h, L.off_sel), uniforms, out_bytes,
+                    at<unsigned>(h, L.off_status), W, wpp, c.n, c.r, c.v, valid_symbols(c), k);
       h->launches++;
     }
     pt.end();
@@ -790,7 +781,7 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     pt.end();
     if (rc != MTPC_OK) return rc;
     pt.begin();
-    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, false, false, out_prefix ? msg : nullptr);
+    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*raw_mixture=*/false, out_prefix ? msg : nullptr);
     pt.end();
     if (rc == MTPC_OK) {               // G, log omega, the messages, W_base h and B h stay in place for an acceptance call
       h->draft_P = P;
@@ -842,7 +833,7 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
                           : c.v <= 256 ? draft_slot_kernel<false, 8>
                           : c.v <= 320 ? draft_slot_kernel<false, 10> : draft_slot_kernel<false, 16>;
       launch_kernel(slot_kernel, dim3(c.n, P), kSlotThreads,
-                    in_smem ? with_tables : base, st, h->ring == 0, c.family,
+                    in_smem ? with_tables : base, st, overlapped(h), c.family,
                     at<float>(h, L.off_logits), at<float>(h, L.off_logw), hmm_tables(h), uniforms, out_bytes,
                     at<float>(h, L.off_G), at<float>(h, L.off_unit_lse), at<unsigned>(h, L.off_status),
                     at<unsigned>(h, L.off_status) + kWorkCounterWord, wpp, c.n, c.r, c.v, valid_symbols(c), L.sum_rows,
@@ -856,7 +847,7 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     pt.end();
     if ((rc = check_launch()) != MTPC_OK) return rc;
     pt.begin();
-    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*dependent=*/h->ring == 0, /*raw_mixture=*/c.r > 32,
+    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*raw_mixture=*/c.r > 32,
                         out_prefix ? msg : nullptr);
     pt.end();
     return rc;
@@ -878,21 +869,22 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     if (rc != MTPC_OK) return rc;
     int* sel = at<int>(h, L.off_sel) + w0 * c.n;
     pt.begin();
-    latent_sample_kernel<<<(wc + kLatentWarps - 1) / kLatentWarps, 32 * kLatentWarps, 0, st>>>(
-        c.family, at<float>(h, L.off_logw) + static_cast<size_t>(p0) * L.sum_rows,
-        hmm_tables(h) + static_cast<size_t>(p0) * hmm_table_stride(h), u, sel, out_bytes + w0 * c.n, at<unsigned>(h, L.off_status), wc, wpp,
-        c.n, c.r, L.sum_rows, hmm_table_stride(h));
+    launch_kernel(latent_sample_kernel, (wc + kLatentWarps - 1) / kLatentWarps, 32 * kLatentWarps, 0, st, overlapped(h),
+                  c.family, at<float>(h, L.off_logw) + static_cast<size_t>(p0) * L.sum_rows,
+                  hmm_tables(h) + static_cast<size_t>(p0) * hmm_table_stride(h), u, sel, out_bytes + w0 * c.n,
+                  at<unsigned>(h, L.off_status), wc, wpp, c.n, c.r, L.sum_rows, hmm_table_stride(h));
     pt.end();
     pt.begin();
     auto* pick = c.v > kMaxDraftVocab ? draft_pick_kernel<true> : draft_pick_kernel<false>;
-    pick<<<(wc * c.n + 7) / 8, 256, 0, st>>>(keep.logit_out, keep.lse_out, sel, u, out_bytes + w0 * c.n, at<float>(h, L.off_G) + w0 * c.n * c.r,
-                                             at<unsigned>(h, L.off_status), wc * c.n, wpp, c.n, c.r, c.v, valid_symbols(c));
+    launch_kernel(pick, (wc * c.n + 7) / 8, 256, 0, st, overlapped(h), keep.logit_out, keep.lse_out, sel, u,
+                  out_bytes + w0 * c.n, at<float>(h, L.off_G) + w0 * c.n * c.r, at<unsigned>(h, L.off_status), wc * c.n, wpp,
+                  c.n, c.r, c.v, valid_symbols(c));
     pt.end();
     h->launches += 2;
     if ((rc = check_launch()) != MTPC_OK) return rc;
   }
   pt.begin();
-  rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, false, false, out_prefix ? msg : nullptr);
+  rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*raw_mixture=*/false, out_prefix ? msg : nullptr);
   pt.end();
   if (rc == MTPC_OK) {                 // G, log omega, the messages and the logits stay in place for an acceptance call
     h->draft_P = P;
@@ -952,23 +944,10 @@ SplitPlan plan_split(long long tiles, int kblocks, int workers, int ctas, bool s
 }
 
 template <int CTAS>
-void launch_plain_tiles(const PlainGemmParams& p, bool a_mn, bool b_mn, int grid, size_t smem, cudaStream_t st) {
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = CTAS == 2 ? 1 : 0;
-  if (a_mn) cudaLaunchKernelEx(&cfg, plain_gemm_kernel<true, true, kPlainTileN, CTAS>, p);
-  else if (b_mn) cudaLaunchKernelEx(&cfg, plain_gemm_kernel<false, true, kPlainTileN, CTAS>, p);
-  else cudaLaunchKernelEx(&cfg, plain_gemm_kernel<false, false, kPlainTileN, CTAS>, p);
+void launch_plain_tiles(const PlainGemmParams& p, bool a_mn, bool b_mn, int grid, size_t smem, cudaStream_t st, bool dependent) {
+  auto* kernel = a_mn ? plain_gemm_kernel<true, true, kPlainTileN, CTAS>
+                      : b_mn ? plain_gemm_kernel<false, true, kPlainTileN, CTAS> : plain_gemm_kernel<false, false, kPlainTileN, CTAS>;
+  launch_clusters(kernel, CTAS, grid, kGemmThreads, smem, st, dependent, p);
 }
 
 // C[M, N] fp32 (pitch ldc) = A B^T over K = K0 + K1: segment 0 multiplies A's K range [0, K0) with B0, segment 1 (K1 > 0)
@@ -1051,13 +1030,13 @@ int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmO
   const int workers = pair ? h->max_pairs : h->num_sms;
   const int grid = ctas * static_cast<int>(items < workers ? items : workers);
   const size_t smem = p.stages * p.stage_bytes + ctl;
-  if (tile_n == 64 && A.mn_major) plain_gemm_kernel<true, true, 64><<<grid, kGemmThreads, smem, st>>>(p);
-  else if (tile_n == 64) plain_gemm_kernel<false, true, 64><<<grid, kGemmThreads, smem, st>>>(p);
-  else if (pair) launch_plain_tiles<2>(p, A.mn_major, B0.mn_major, grid, smem, st);
-  else launch_plain_tiles<1>(p, A.mn_major, B0.mn_major, grid, smem, st);
+  if (tile_n == 64 && A.mn_major) launch_kernel(plain_gemm_kernel<true, true, 64>, grid, kGemmThreads, smem, st, overlapped(h), p);
+  else if (tile_n == 64) launch_kernel(plain_gemm_kernel<false, true, 64>, grid, kGemmThreads, smem, st, overlapped(h), p);
+  else if (pair) launch_plain_tiles<2>(p, A.mn_major, B0.mn_major, grid, smem, st, overlapped(h));
+  else launch_plain_tiles<1>(p, A.mn_major, B0.mn_major, grid, smem, st, overlapped(h));
   h->launches++;
   if (p.tail_tiles > 0) {
-    launch_kernel(split_reduce_kernel, p.tail_tiles * ctas * 8, 256, 0, st, /*dependent=*/true, p, ctas);
+    launch_kernel(split_reduce_kernel, p.tail_tiles * ctas * 8, 256, 0, st, overlapped(h), p, ctas);
     h->launches++;
   }
   return check_launch();
@@ -1085,7 +1064,7 @@ int launch_lowrank_logits(mtpc_head* h, LowRankParams p, int T, cudaStream_t st)
   p.wait_limit_ns = h->wait_limit_ns;
   const long long items = static_cast<long long>(p.m_tiles) * p.n * p.blocks;
   const int grid = static_cast<int>(items < h->num_sms ? items : h->num_sms);
-  lowrank_logits_kernel<MODE><<<grid, lowrank_threads(MODE), lowrank_smem_bytes(MODE), st>>>(p);
+  launch_kernel(lowrank_logits_kernel<MODE>, grid, lowrank_threads(MODE), lowrank_smem_bytes(MODE), st, overlapped(h), p);
   h->launches++;
   return check_launch();
 }
@@ -1113,8 +1092,8 @@ int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, cons
     if (rc != MTPC_OK) return rc;
     // A as [n, v, r, k]: the adaptor columns of adjacent components side by side (remade every call: A may have changed)
     const size_t pieces = static_cast<size_t>(units) * c.v * (k / 8);
-    lowrank_repack_kernel<<<static_cast<unsigned>((pieces + 255) / 256), 256, 0, st>>>(
-        static_cast<const uint4*>(h->lr_A), reinterpret_cast<uint4*>(h->ws + h->lr_off_arep), c.n, c.r, c.v, k / 8);
+    launch_kernel(lowrank_repack_kernel, static_cast<unsigned>((pieces + 255) / 256), 256, 0, st, overlapped(h),
+                  static_cast<const uint4*>(h->lr_A), reinterpret_cast<uint4*>(h->ws + h->lr_off_arep), c.n, c.r, c.v, k / 8);
     h->launches += 1;
   }
   if (!(parts & 4)) return check_launch();
@@ -1123,9 +1102,9 @@ int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, cons
   p.ref = p.log_sum + static_cast<size_t>((c.v + 31) / 32) * T * units;
   if ((rc = launch_lowrank_logits<kLowRankForward>(h, p, T, st)) != MTPC_OK) return rc;
   const size_t entries = static_cast<size_t>(T) * units;
-  lowrank_merge_kernel<<<static_cast<unsigned>((entries + 255) / 256), 256, 0, st>>>(
-      p.log_sum, p.ref, base, zhl, reinterpret_cast<const __nv_bfloat16*>(h->ws + h->lr_off_arep), targets, at<float>(h, L.off_G), lse_out,
-      at<unsigned>(h, L.off_status), entries, c.n, c.r, c.v, p.vv, k, targets_are_drafts ? 1 : 0);
+  launch_kernel(lowrank_merge_kernel, static_cast<unsigned>((entries + 255) / 256), 256, 0, st, overlapped(h), p.log_sum, p.ref,
+                base, zhl, reinterpret_cast<const __nv_bfloat16*>(h->ws + h->lr_off_arep), targets, at<float>(h, L.off_G),
+                lse_out, at<unsigned>(h, L.off_status), entries, c.n, c.r, c.v, p.vv, k, targets_are_drafts ? 1 : 0);
   h->launches += 1;
   return check_launch();
 }
@@ -1162,24 +1141,25 @@ int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cuda
   const int threads = warps * 32;
   const int resident = blocks < 8 * h->num_sms ? blocks : 8 * h->num_sms;
   const size_t smem = circuit_backward_smem(h, warps);
-  if ((c.family == MTPC_HMM || (c.family == MTPC_BTREE && !loss)) && cudaMemsetAsync(counter, 0, sizeof(unsigned), st) != cudaSuccess)
-    return MTPC_ERR_CUDA;
   if (c.family == MTPC_CP && loss) {
-    circuit_cp_loss_backward_kernel<<<blocks, threads, smem, st>>>(a);
+    launch_kernel(circuit_cp_loss_backward_kernel, blocks, threads, smem, st, overlapped(h), a);
   } else if (c.family == MTPC_CP) {
-    circuit_cp_backward_kernel<<<(a.W + kCircuitWarps - 1) / kCircuitWarps, kCircuitWarps * 32, 0, st>>>(a);
+    launch_kernel(circuit_cp_backward_kernel, (a.W + kCircuitWarps - 1) / kCircuitWarps, kCircuitWarps * 32, 0, st,
+                  overlapped(h), a);
   } else if (c.family == MTPC_HMM && loss) {
-    circuit_hmm_loss_backward_kernel<<<resident, threads, smem, st>>>(a, hmm_tables(h), hmm_table_stride(h), dT, counter);
+    launch_kernel(circuit_hmm_loss_backward_kernel, resident, threads, smem, st, overlapped(h), a, hmm_tables(h),
+                  hmm_table_stride(h), dT, counter);
   } else if (c.family == MTPC_HMM) {
-    circuit_hmm_backward_kernel<<<resident, threads, smem, st>>>(a, hmm_tables(h), hmm_table_stride(h), dT, counter);
+    launch_kernel(circuit_hmm_backward_kernel, resident, threads, smem, st, overlapped(h), a, hmm_tables(h),
+                  hmm_table_stride(h), dT, counter);
   } else if (loss) {
     const int tw = c.n / 2 < 8 ? c.n / 2 : 8;                             // a warp per node of the owners' level
     const bool fits = btree_loss_smem_floats(c.n, c.r, tw, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
     const size_t tsmem = btree_loss_smem_floats(c.n, c.r, tw, fits) * sizeof(float);
     const int grid = a.W < sms_times_resident(h, tsmem) ? a.W : sms_times_resident(h, tsmem);
-    circuit_btree_loss_backward_kernel<<<grid, tw * 32, tsmem, st>>>(a, fits ? 1 : 0);
+    launch_kernel(circuit_btree_loss_backward_kernel, grid, tw * 32, tsmem, st, overlapped(h), a, fits ? 1 : 0);
   } else {
-    circuit_btree_backward_kernel<<<resident, threads, smem, st>>>(a, counter);
+    launch_kernel(circuit_btree_backward_kernel, resident, threads, smem, st, overlapped(h), a, counter);
   }
   h->launches++;
   return check_launch();
@@ -1219,7 +1199,7 @@ int backward_tail(mtpc_head* head, const BackwardLayout& B, uint8_t* bw, const v
     int row_blocks = (16 * head->num_sms + col_blocks - 1) / col_blocks;   // enough CTAs to fill the device, each walks rows
     if (row_blocks > T) row_blocks = T;
     if (row_blocks > 65535) row_blocks = 65535;
-    logit_gradient_kernel<<<dim3(col_blocks, row_blocks), 256, 0, st>>>(la);
+    launch_kernel(logit_gradient_kernel, dim3(col_blocks, row_blocks), 256, 0, st, overlapped(head), la);
   }
   head->launches++;
   int rc = check_launch();
@@ -1295,8 +1275,9 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
   if ((rc = launch_lowrank_logits<kLowRankGradient>(head, lp, T, st)) != MTPC_OK) return rc;
   {
     const size_t pad_pieces = static_cast<size_t>(units) * R.v64 * (k / 8);
-    lowrank_pad_kernel<<<static_cast<unsigned>((pad_pieces + 255) / 256), 256, 0, st>>>(
-        static_cast<const uint4*>(head->lr_A), reinterpret_cast<uint4*>(bw + R.off_apad), units, c.v, static_cast<int>(R.v64), k / 8);
+    launch_kernel(lowrank_pad_kernel, static_cast<unsigned>((pad_pieces + 255) / 256), 256, 0, st, overlapped(head),
+                  static_cast<const uint4*>(head->lr_A), reinterpret_cast<uint4*>(bw + R.off_apad), units, c.v,
+                  static_cast<int>(R.v64), k / 8);
   }
   head->launches += 1;
   uint8_t* wcat = bw + R.off_wcat;
@@ -1377,10 +1358,8 @@ static int bind_parameters(mtpc_head* h, const void* W_emit, const void* W_sum, 
   const size_t emit_count = static_cast<size_t>(cfg->n) * cfg->r * cfg->v * cfg->d;
   const size_t sum_count = static_cast<size_t>(L.sum_rows) * cfg->d;
   if (cfg->io_dtype == MTPC_F32) {
-    f32_to_bf16_kernel<<<2048, 256, 0, st>>>(static_cast<const float*>(W_emit), at<__nv_bfloat16>(h, L.off_wemit),
-                                             emit_count);
-    f32_to_bf16_kernel<<<256, 256, 0, st>>>(static_cast<const float*>(W_sum), at<__nv_bfloat16>(h, L.off_wsum),
-                                            sum_count);
+    round_to_bf16(static_cast<const float*>(W_emit), at<__nv_bfloat16>(h, L.off_wemit), emit_count, st, false);
+    round_to_bf16(static_cast<const float*>(W_sum), at<__nv_bfloat16>(h, L.off_wsum), sum_count, st, false);
     h->launches += 2;
     h->W_emit_bf16 = h->ws + L.off_wemit;
     h->W_sum_bf16 = h->ws + L.off_wsum;
@@ -1645,15 +1624,14 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
   float* const msg = at<float>(head, L.off_msg);
   if (!head->draft_msg) {
     // the draft returned the joint alone: the slot messages are formed now, from the evidence and log omega it left
-    rc = launch_circuit(head, W, wpp, nullptr, nullptr, st, /*dependent=*/false,
-                        /*raw_mixture=*/P <= L.decode_max_p && c.r > 32, msg);
+    rc = launch_circuit(head, W, wpp, nullptr, nullptr, st, /*raw_mixture=*/P <= L.decode_max_p && c.r > 32, msg);
     if (rc != MTPC_OK) return rc;
     head->draft_msg = true;
   }
   if (head->draft_logits) {
     // every logit of the drafted positions is still in the workspace
     pt.begin();
-    launch_kernel(spec_accept_kernel, W, threads, smem, st, /*dependent=*/head->ring == 0, at<float>(head, L.off_logits),
+    launch_kernel(spec_accept_kernel, W, threads, smem, st, overlapped(head), at<float>(head, L.off_logits),
                   at<float>(head, L.off_unit_lse), msg, draft_bytes, prefix_logprob, target_probs, accept_uniforms, out_accepted,
                   out_next_byte, at<unsigned>(head, L.off_status), W, wpp, c.n, c.r, c.v, valid_symbols(c),
                   static_cast<const int*>(nullptr));
@@ -1687,22 +1665,24 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
     const float* tp = target_probs + w0 * (c.n + 1) * c.v;
     const float* ua = accept_uniforms + w0 * (c.n + 1);
     pt.begin();
-    accept_test_kernel<<<(wc + 7) / 8, 256, 0, st>>>(xb, pre, tp, ua, rej, wc, c.n, c.v, valid_symbols(c));
+    launch_kernel(accept_test_kernel, (wc + 7) / 8, 256, 0, st, overlapped(head), xb, pre, tp, ua, rej, wc, c.n, c.v,
+                  valid_symbols(c));
     if (factored) {
       // the slot's logits from W_base h and B h, window by window: no sort, no staging, no projection pass
       const int pairs = wc * c.r;
       int blocks = (pairs + kDrawWarps - 1) / kDrawWarps;
       if (blocks > 32 * head->num_sms) blocks = 32 * head->num_sms;
-      lowrank_slot_logits_kernel<<<blocks, 32 * kDrawWarps, 0, st>>>(
-          reinterpret_cast<const float*>(head->ws + head->lr_off_base), reinterpret_cast<const __nv_bfloat16*>(head->ws + head->lr_off_zhl),
-          static_cast<const __nv_bfloat16*>(head->lr_A), rej, lg, lse, row_of, wc, static_cast<int>(w0), wpp, c.n, c.r, c.v,
-          valid_symbols(c), head->lr_k);
+      launch_kernel(lowrank_slot_logits_kernel, blocks, 32 * kDrawWarps, 0, st, overlapped(head),
+                    reinterpret_cast<const float*>(head->ws + head->lr_off_base),
+                    reinterpret_cast<const __nv_bfloat16*>(head->ws + head->lr_off_zhl),
+                    static_cast<const __nv_bfloat16*>(head->lr_A), rej, lg, lse, row_of, wc, static_cast<int>(w0), wpp, c.n,
+                    c.r, c.v, valid_symbols(c), head->lr_k);
       head->launches += 2;
       pt.end();
       int rcf = check_launch();
       if (rcf != MTPC_OK) return rcf;
       pt.begin();
-      launch_kernel(spec_accept_kernel, wc, threads, smem, st, /*dependent=*/head->ring == 0, lg, lse, msg + w0 * c.n * c.r, xb,
+      launch_kernel(spec_accept_kernel, wc, threads, smem, st, overlapped(head), lg, lse, msg + w0 * c.n * c.r, xb,
                     pre, tp, ua, out_accepted + w0, out_next_byte + w0, at<unsigned>(head, L.off_status), wc, wpp, c.n, c.r, c.v,
                     valid_symbols(c), row_of);
       head->launches++;
@@ -1736,7 +1716,7 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
     pt.end();
     if (rc2 != MTPC_OK) return rc2;
     pt.begin();
-    launch_kernel(spec_accept_kernel, wc, threads, smem, st, /*dependent=*/head->ring == 0, lg, lse, msg + w0 * c.n * c.r, xb,
+    launch_kernel(spec_accept_kernel, wc, threads, smem, st, overlapped(head), lg, lse, msg + w0 * c.n * c.r, xb,
                   pre, tp, ua, out_accepted + w0, out_next_byte + w0, at<unsigned>(head, L.off_status), wc, wpp, c.n, c.r, c.v,
                   valid_symbols(c), row_of);
     head->launches++;
@@ -1760,8 +1740,10 @@ int mtpc_window_loss(mtpc_head* head, const void* hidden, const int32_t* targets
   float* partial = at<float>(head, L.off_partial);
   int rc = window_logprob_impl(head, hidden, targets, T, nullptr, prefix, st);   // phases 0 and 1
   if (rc != MTPC_OK) return rc;
-  loss_partial_kernel<<<num_sequences, kLossThreads, 0, st>>>(prefix, targets, partial, sequence_length, head->cfg.n);
-  loss_final_kernel<<<1, kLossThreads, 0, st>>>(partial, out_slot_loss, out_loss, num_sequences, head->cfg.n, gamma);
+  launch_kernel(loss_partial_kernel, num_sequences, kLossThreads, 0, st, overlapped(head), prefix, targets, partial,
+                sequence_length, head->cfg.n);
+  launch_kernel(loss_final_kernel, 1, kLossThreads, 0, st, overlapped(head), partial, out_slot_loss, out_loss, num_sequences,
+                head->cfg.n, gamma);
   head->launches += 2;
   return check_launch();
 }
@@ -1797,6 +1779,8 @@ int mtpc_window_logprob_backward(mtpc_head* head, const void* hidden, const int3
   if ((rc = set_backward_attributes(head)) != MTPC_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t* bw = static_cast<uint8_t*>(bwd_workspace);
+  if (static_hmm && cudaMemsetAsync(dT_static, 0, static_cast<size_t>(c.n - 1) * c.r * c.r * 4, st) != cudaSuccess)
+    return MTPC_ERR_CUDA;
   const void* hb = nullptr;
   head->draft_P = 0;
   rc = stage_hidden(head, hidden, T, &hb, st);
@@ -1813,8 +1797,6 @@ int mtpc_window_logprob_backward(mtpc_head* head, const void* hidden, const int3
   if (rc != MTPC_OK) return rc;
   // 2. circuit backward: posteriors of the input units and of the sum units
   pt.begin();
-  if (static_hmm && cudaMemsetAsync(dT_static, 0, static_cast<size_t>(c.n - 1) * c.r * c.r * 4, st) != cudaSuccess)
-    return MTPC_ERR_CUDA;
   CircuitBackwardArgs a;
   memset(&a, 0, sizeof(a));
   a.targets = targets;
@@ -1866,6 +1848,8 @@ int mtpc_lowrank_window_logprob_backward(mtpc_head* head, const void* hidden, co
   if ((rc = set_backward_attributes(head)) != MTPC_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t* bw = static_cast<uint8_t*>(bwd_workspace);
+  if (static_hmm && cudaMemsetAsync(dT_static, 0, static_cast<size_t>(c.n - 1) * c.r * c.r * 4, st) != cudaSuccess)
+    return MTPC_ERR_CUDA;
   const void* hb = hidden;                                     // (factored heads are bf16)
   head->draft_P = 0;
   PhaseTimer pt(head, st);
@@ -1876,8 +1860,6 @@ int mtpc_lowrank_window_logprob_backward(mtpc_head* head, const void* hidden, co
   if (rc != MTPC_OK) return rc;
   // 2. circuit backward: posteriors of the input units; the sum units' logit gradients go to the right of sy
   pt.begin();
-  if (static_hmm && cudaMemsetAsync(dT_static, 0, static_cast<size_t>(c.n - 1) * c.r * c.r * 4, st) != cudaSuccess)
-    return MTPC_ERR_CUDA;
   __nv_bfloat16* sy = reinterpret_cast<__nv_bfloat16*>(bw + R.off_sy);
   CircuitBackwardArgs a;
   memset(&a, 0, sizeof(a));
@@ -1930,6 +1912,8 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   float* coeff = reinterpret_cast<float*>(bw + B.off_coeff);
   float* prefix = at<float>(head, L.off_prefix);
   float* partial = at<float>(head, L.off_partial);
+  if (static_hmm && cudaMemsetAsync(dT_static, 0, static_cast<size_t>(c.n - 1) * c.r * c.r * 4, st) != cudaSuccess)
+    return MTPC_ERR_CUDA;
   const void* hb = nullptr;
   head->draft_P = 0;
   rc = stage_hidden(head, hidden, T, &hb, st);
@@ -1944,15 +1928,14 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   rc = factored ? launch_lowrank_projection(head, hb, T, targets, st, fwd.lse_out)
                 : launch_gemm(head, hb, T, true, true, targets, st, &fwd);
   if (rc != MTPC_OK) return rc;
-  loss_coeff_kernel<<<num_sequences, kLossThreads, 0, st>>>(targets, coeff, sequence_length, c.n, num_sequences, gamma);
+  launch_kernel(loss_coeff_kernel, num_sequences, kLossThreads, 0, st, overlapped(head), targets, coeff, sequence_length, c.n,
+                num_sequences, gamma);
   head->launches++;
   pt.end();
   if ((rc = check_launch()) != MTPC_OK) return rc;
   // 2. circuit: every prefix and the whole gradient of the loss, then the loss itself. The sum units' logit gradients (bf16)
   // go to the right of dlogit, or of [s | y] on a factored head.
   pt.begin();
-  if (static_hmm && cudaMemsetAsync(dT_static, 0, static_cast<size_t>(c.n - 1) * c.r * c.r * 4, st) != cudaSuccess)
-    return MTPC_ERR_CUDA;
   CircuitBackwardArgs a;
   memset(&a, 0, sizeof(a));
   a.targets = targets;
@@ -1964,8 +1947,10 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   a.dsum_pitch = static_cast<int>(factored ? R.pitch : B.Kd);
   a.W = T;
   if ((rc = launch_circuit_backward(head, a, dT_static, st)) != MTPC_OK) return rc;
-  loss_partial_kernel<<<num_sequences, kLossThreads, 0, st>>>(prefix, targets, partial, sequence_length, c.n);
-  loss_final_kernel<<<1, kLossThreads, 0, st>>>(partial, out_slot_loss, out_loss, num_sequences, c.n, gamma);
+  launch_kernel(loss_partial_kernel, num_sequences, kLossThreads, 0, st, overlapped(head), prefix, targets, partial,
+                sequence_length, c.n);
+  launch_kernel(loss_final_kernel, 1, kLossThreads, 0, st, overlapped(head), partial, out_slot_loss, out_loss, num_sequences,
+                c.n, gamma);
   head->launches += 2;
   pt.end();
   if ((rc = check_launch()) != MTPC_OK) return rc;

@@ -43,6 +43,8 @@ struct CircuitBackwardArgs {
 // log q = LSE_k a_k, a_k = log omega_k + sum_i G[i, k]:  d log q / d a_k = rho_k = softmax(a)_k for every slot and for
 // the mixture weight; through the softmax of the mixture logits: rho_k - omega_k.
 __global__ void circuit_cp_backward_kernel(const CircuitBackwardArgs a_) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int w = blockIdx.x * kCircuitWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= a_.W) return;
@@ -89,6 +91,8 @@ __global__ void circuit_cp_backward_kernel(const CircuitBackwardArgs a_) {
 // conversion at n = 8: 50 us with their gaps at 2005 positions, prefixes included, against 5.) Shared memory per warp: n (r + 1) + n floats.
 __host__ __device__ inline int cp_loss_warp_floats(int n, int r) { return n * (r + 2); }
 __global__ void circuit_cp_loss_backward_kernel(const CircuitBackwardArgs a_) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   extern __shared__ __align__(16) float sm[];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int w = blockIdx.x * (blockDim.x >> 5) + wib;
@@ -192,6 +196,8 @@ __host__ __device__ inline size_t hmm_backward_smem_floats(int n, int r, bool is
 
 __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const float* __restrict__ tables,
                                             int table_stride, float* __restrict__ dT, unsigned* work_counter) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   extern __shared__ __align__(16) float sm[];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
@@ -345,6 +351,8 @@ __device__ __forceinline__ void row_grad_mult(const float* row, const float* pc,
 
 __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, const float* __restrict__ tables,
                                                  int table_stride, float* __restrict__ dT, unsigned* work_counter) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   extern __shared__ __align__(16) float sm[];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
@@ -461,6 +469,8 @@ __host__ __device__ inline size_t btree_backward_warp_floats(int n, int r) {
 }
 
 __global__ void circuit_btree_backward_kernel(const CircuitBackwardArgs a_, unsigned* work_counter) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   extern __shared__ __align__(16) float sm[];
   const int wib = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -575,6 +585,8 @@ __host__ __device__ inline size_t btree_loss_smem_floats(int n, int r, int warps
          (4 * static_cast<size_t>(n - 1) + n / 2 + 4 * static_cast<size_t>(warps)) * vr;
 }
 __global__ void __launch_bounds__(256) circuit_btree_loss_backward_kernel(const CircuitBackwardArgs a_, int tables_in_smem) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   extern __shared__ __align__(16) float sm[];
   const int n = a_.n, r = a_.r;
   TreeSweep t;
@@ -732,6 +744,7 @@ struct LogitGradArgs {
 };
 
 __global__ void __launch_bounds__(256) logit_gradient_kernel(const LogitGradArgs a) {
+  grid_dependency_wait();
   const int c = (blockIdx.x * 256 + threadIdx.x) * 8;
   if (c >= a.Nc) return;
   const int units = a.n * a.r;
@@ -753,6 +766,7 @@ __global__ void __launch_bounds__(256) logit_gradient_kernel(const LogitGradArgs
       o[q] = __float2bfloat16_rn(pst * ((rel == q ? 1.f : 0.f) - fast_ex2(fmaf(xs[q], kLog2e, -lse2))));
     *reinterpret_cast<uint4*>(a.dlogit + static_cast<size_t>(t) * a.pitch + c) = *reinterpret_cast<const uint4*>(o);
   }
+  grid_launch_dependents();
 }
 
 // ---------------------------------------------------------------- plain bf16 GEMM on the tcgen05 tensor cores
@@ -933,7 +947,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
   if (CTAS == 2) cluster_sync_all();   // the peer's barriers are initialised before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
-  grid_launch_dependents();            // split_reduce_kernel's CTAs may be scheduled as SMs free up
+  grid_launch_dependents();            // the next kernel's CTAs may be scheduled as SMs free up
+  grid_dependency_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1116,6 +1131,7 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const __grid_constant
     }
   }
   if (row < p.M) plain_store16(p, x, row, p.C == nullptr ? nullptr : plain_row(p, row), static_cast<size_t>(row) * p.ldc, col0);
+  grid_launch_dependents();
 }
 
 }  // namespace mtpc

@@ -603,6 +603,7 @@ __global__ void __launch_bounds__(32 * kLatentWarps) latent_sample_kernel(
     int family, const float* __restrict__ logw, const float* __restrict__ logA, const float* __restrict__ uniforms,
     int* __restrict__ unit_sel, int* __restrict__ out_bytes, unsigned* status, int W, int wpp, int n, int r, int sum_rows,
     int logA_stride) {
+  grid_dependency_wait();
   __shared__ int zs[kLatentWarps][64];
   const int w = blockIdx.x * kLatentWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -633,6 +634,7 @@ __global__ void __launch_bounds__(32 * kLatentWarps) latent_sample_kernel(
     unit_sel[static_cast<size_t>(w) * n + i] = bad ? -1 : (family == 0 ? z[0] : family == 1 ? z[i] : z[n / 2 - 1 + (i >> 1)]);
     out_bytes[static_cast<size_t>(w) * n + i] = -1;
   }
+  grid_launch_dependents();
 }
 
 // Byte draws of a draft whose logits were kept by the projection kernel: one warp per (window, slot) draws the byte by inverse
@@ -646,6 +648,7 @@ __global__ void __launch_bounds__(256) draft_pick_kernel(const float* __restrict
                                                          const int* __restrict__ unit_sel, const float* __restrict__ uniforms,
                                                          int* __restrict__ out_bytes, float* __restrict__ G, unsigned* status,
                                                          int pairs, int wpp, int n, int r, int v, int vv) {
+  grid_dependency_wait();
   const int e = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (e >= pairs) return;
@@ -684,6 +687,7 @@ __global__ void __launch_bounds__(256) draft_pick_kernel(const float* __restrict
   if (lane == 0) out_bytes[e] = byte;
   for (int k = lane; k < r; k += 32)
     G[static_cast<size_t>(e) * r + k] = byte < 0 ? CUDART_NAN_F : row[static_cast<size_t>(k) * v + byte] - unit_lse[unit0 + k];
+  grid_launch_dependents();
 }
 
 // ---------------------------------------------------------------- acceptance stage (Algorithm 3)
@@ -862,6 +866,7 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
 __global__ void accept_test_kernel(const int* __restrict__ bytes, const float* __restrict__ prefix,
                                    const float* __restrict__ target, const float* __restrict__ uniforms,
                                    int* __restrict__ first_rejected, int W, int n, int v, int vv) {
+  grid_dependency_wait();
   const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= W) return;
@@ -887,6 +892,7 @@ __global__ void accept_test_kernel(const int* __restrict__ bytes, const float* _
     }
   }
   if (lane == 0) first_rejected[w] = (bad || s == n) ? -1 : s;
+  grid_launch_dependents();
 }
 
 }  // namespace mtpc

@@ -70,6 +70,7 @@ struct GemmParams {
   size_t logit_pitch;                // kept for the backward pass or a draft (padding columns as -inf)
   const GroupTile* group_tiles;      // sorted rows: the work items, and ...
   const int* group_num_tiles;        // ... how many there are (device memory: written by the kernel that made them)
+  unsigned* work_counter;            // zeroed here for the circuit kernel that hands out its windows through it, or NULL
   unsigned* status;
   uint64_t wait_limit_ns;            // limit of every pipeline wait (kWaitLimitNs unless a test shortened it)
 };
@@ -229,6 +230,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   constexpr bool kGrouped = MODE == kModeLogitsGrouped;
+  if (kGrouped) grid_dependency_wait();   // the tiles are read below
   static_assert(!kGrouped || CTAS == 1, "grouped tiles are ragged: no pairing");
   const int num_items = kGrouped ? *p.group_num_tiles * p.num_groups : (p.num_groups + p.num_sum_tiles) * p.m_units;
   const uint32_t cta_rank = CTAS == 2 ? cluster_cta_rank() : 0u;      // 0 = the pair's leader
@@ -273,6 +275,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   if (CTAS == 2) cluster_sync_all();   // the peer's barriers are initialised before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
+  grid_launch_dependents();   // the next kernel's CTAs may be scheduled as SMs free up; they wait for this grid's results
+  grid_dependency_wait();     // barriers and tensor memory were set up while the kernel before this one finished
+  if (p.work_counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *p.work_counter = 0;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer

@@ -142,6 +142,8 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kerne
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
+  grid_launch_dependents();
+  grid_dependency_wait();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -461,6 +463,7 @@ __global__ void lowrank_merge_kernel(const float* __restrict__ log_sum, const fl
                                      const __nv_bfloat16* __restrict__ zhl, const __nv_bfloat16* __restrict__ Arep,
                                      const int* __restrict__ targets, float* __restrict__ G, float* __restrict__ lse_out,
                                      unsigned* status, size_t entries, int n, int r, int v, int vv, int k, int missing_is_nan) {
+  grid_dependency_wait();
   const size_t e = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= entries) return;
   const size_t ti = e / r, tn = entries / r;       // (position, slot), and how many there are
@@ -517,10 +520,12 @@ __global__ void lowrank_merge_kernel(const float* __restrict__ log_sum, const fl
     }
   }
   G[e] = base[ti * v + tgt] + (d0 + d1) - lse;
+  grid_launch_dependents();
 }
 
 // A [n, r, v, k] -> A' [n, v, r, k] (bf16, k a multiple of 8): one 16-byte piece per thread.
 __global__ void lowrank_repack_kernel(const uint4* __restrict__ A, uint4* __restrict__ out, int n, int r, int v, int kv) {
+  grid_dependency_wait();
   const size_t total = static_cast<size_t>(n) * r * v * kv;      // kv = k / 8 pieces per row
   const size_t idx = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= total) return;
@@ -531,6 +536,7 @@ __global__ void lowrank_repack_kernel(const uint4* __restrict__ A, uint4* __rest
   const int b = static_cast<int>(rest % v);
   const int i = static_cast<int>(rest / v);
   out[idx] = A[((static_cast<size_t>(i) * r + j) * v + b) * kv + q];
+  grid_launch_dependents();
 }
 
 // Few-position draft on a factored head: logits[p, i, j, b] = base[p, i, b] + sum_q A[i, j, b, q] z[p, i, j, q], from the
@@ -587,6 +593,7 @@ __global__ void __launch_bounds__(kExpandThreads) lowrank_expand_kernel(const fl
 // A [n r, v, k] -> [n r, v64, k] with v64 = v rounded up to 64 and zero rows past v: the batched GEMM g_ij A_ij walks K in
 // blocks of 64 symbols, and what it reads of g past a unit's own columns must meet zeros.
 __global__ void lowrank_pad_kernel(const uint4* __restrict__ A, uint4* __restrict__ out, int units, int v, int v64, int kv) {
+  grid_dependency_wait();
   const size_t total = static_cast<size_t>(units) * v64 * kv;    // kv = k / 8 pieces per row
   const size_t idx = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= total) return;
@@ -595,6 +602,7 @@ __global__ void lowrank_pad_kernel(const uint4* __restrict__ A, uint4* __restric
   const int b = static_cast<int>(rest % v64);
   const size_t u = rest / v64;
   out[idx] = b < v ? A[(u * v + b) * kv + q] : make_uint4(0u, 0u, 0u, 0u);
+  grid_launch_dependents();
 }
 
 // Byte draws of a long draft on a factored head (Algorithm 1, input-unit step): one warp per (window, slot) forms the v
@@ -607,6 +615,7 @@ __global__ void __launch_bounds__(32 * kDrawWarps) lowrank_draw_kernel(
     const float* __restrict__ base, const __nv_bfloat16* __restrict__ zhl, const __nv_bfloat16* __restrict__ A,
     const int* __restrict__ unit_sel, const float* __restrict__ uniforms, int* __restrict__ out_bytes, unsigned* status, int W,
     int wpp, int n, int r, int v, int vv, int k) {
+  grid_dependency_wait();
   extern __shared__ float draw_sm[];                              // kDrawWarps x v logits
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* x = draw_sm + warp * v;
@@ -658,6 +667,7 @@ __global__ void __launch_bounds__(32 * kDrawWarps) lowrank_draw_kernel(
     if (lane == 0) out_bytes[e] = byte;
     __syncwarp();                                                 // x is reused by the warp's next pair
   }
+  grid_launch_dependents();
 }
 
 // Acceptance stage after a long draft on a factored head (Algorithm 3): for every window whose draft was rejected at byte s
@@ -668,6 +678,7 @@ __global__ void __launch_bounds__(32 * kDrawWarps) lowrank_slot_logits_kernel(
     const float* __restrict__ base, const __nv_bfloat16* __restrict__ zhl, const __nv_bfloat16* __restrict__ A,
     const int* __restrict__ first_rejected, float* __restrict__ logits, float* __restrict__ unit_lse, int* __restrict__ row_of,
     int W, int w_first, int wpp, int n, int r, int v, int vv, int k) {
+  grid_dependency_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t units = static_cast<size_t>(n) * r;
   const int pairs = W * r;
@@ -714,6 +725,7 @@ __global__ void __launch_bounds__(32 * kDrawWarps) lowrank_slot_logits_kernel(
     }
     if (lane == 0) unit_lse[static_cast<size_t>(w) * r + j] = m + __logf(sum);
   }
+  grid_launch_dependents();
 }
 
 }  // namespace mtpc

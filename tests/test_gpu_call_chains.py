@@ -1,0 +1,69 @@
+"""Calls that follow one another without a pause. The kernels of a call, and the first kernel of the next one, are scheduled before
+the kernel ahead has finished and wait for it on the device; the kernels that hand out windows through a counter rely on the
+projection (or the per-slot kernel) before them to zero it. So back-to-back calls on alternating inputs must give, bit for bit, what
+each call gives alone on an idle device. (fp32 heads: the gradient of a static transition table is summed by atomics and is left
+out.) d = 1088 runs the projection in CTA pairs, d <= 1024 in single CTAs; an fp32 hidden state at an odd multiple of four bytes
+takes the scalar conversion, an aligned one the 16-byte conversion."""
+import pytest
+import torch
+
+from paper_2511_11346_b200 import inputs as I
+from paper_2511_11346_b200.runner import DeviceHead
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("family,n,r,v,d,T,dtype", [
+    (I.BTREE, 8, 16, 64, 128, 150, "f32"),
+    (I.BTREE, 4, 8, 48, 1088, 300, "bf16"),
+    (I.HMM, 5, 8, 64, 1024, 257, "f32"),
+    (I.CP, 3, 8, 320, 64, 200, "f32"),
+])
+def test_back_to_back_calls_equal_isolated_ones(family, n, r, v, d, T, dtype):
+    shape = I.HeadShape(family, n, r, v, d, io_dtype=I.F32 if dtype == "f32" else I.BF16)
+    wl = I.make_workload("chain", shape, T, seed=41, wpp=2, weight_std=0.25)
+    dh = DeviceHead(wl)
+    torch.manual_seed(7)
+    hidden = [dh.hidden_device()]
+    hidden.append(torch.randn_like(hidden[0]))
+    targets = [torch.from_numpy(wl.targets).cuda(), torch.randint(v, (T, n), dtype=torch.int32, device="cuda")]
+    if dtype == "f32":                                   # the same values, four bytes off a 16-byte boundary
+        room = torch.empty(hidden[1].numel() + 1, dtype=torch.float32, device="cuda")
+        hidden[1] = room[1:].view_as(hidden[1]).copy_(hidden[1])
+    head = dh.head
+    uniforms = torch.rand(2 * T, 2 * n, device="cuda")
+    weight = torch.full((T,), -1.0 / T, device="cuda")
+
+    def calls(i, small):
+        P = 3 if small else T
+        out = {k: torch.empty(T, device="cuda") for k in ("lp", "blp")}
+        out["pre"] = torch.empty(T, n, device="cuda")
+        out["bytes"] = torch.empty(2 * P, n, dtype=torch.int32, device="cuda")
+        out["dlp"] = torch.empty(2 * P, device="cuda")
+        g = {k: torch.empty(s, device="cuda") for k, s in
+             (("dh", (T, d)), ("dWe", (n, r, v, d)), ("dWs", tuple(dh.W_sum.shape)))}
+        dT = torch.empty(max(n - 1, 1), r, r, device="cuda") if family == I.HMM else None
+        steps = [lambda: head.mtpc_window_logprob(hidden[i], targets[i], out["lp"]),
+                 lambda: head.mtpc_draft_sample(hidden[i][:P], 2, uniforms[:2 * P], out["bytes"], out["dlp"]),
+                 lambda: head.mtpc_window_logprob_backward(hidden[i], targets[i], weight, out["blp"], g["dh"], g["dWe"], g["dWs"], dT),
+                 lambda: head.mtpc_window_prefix_logprob(hidden[i], targets[i], out["pre"])]
+        return steps, {**out, **g}
+
+    def run(alone):
+        results = []
+        for i, small in ((0, True), (1, False), (0, False), (1, True)):
+            steps, out = calls(i, small)
+            for step in steps:
+                if alone:
+                    torch.cuda.synchronize()
+                step()
+            results.append(out)
+        torch.cuda.synchronize()
+        return results
+
+    for a, b in zip(run(alone=True), run(alone=False)):
+        for k in a:
+            assert torch.equal(a[k], b[k]), k
+            assert not a[k].is_floating_point() or torch.isfinite(a[k]).all(), k
+    assert head.mtpc_get_status() == 0
+    dh.close()

@@ -1157,7 +1157,8 @@ int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cuda
     const bool fits = btree_loss_smem_floats(c.n, c.r, tw, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
     const size_t tsmem = btree_loss_smem_floats(c.n, c.r, tw, fits) * sizeof(float);
     const int grid = a.W < sms_times_resident(h, tsmem) ? a.W : sms_times_resident(h, tsmem);
-    launch_kernel(circuit_btree_loss_backward_kernel, grid, tw * 32, tsmem, st, overlapped(h), a, fits ? 1 : 0);
+    // (as a dependent, its CTAs crowded beside the projection's last ones: 350 -> 395 us at 4096 positions of a 16 x 32 head)
+    launch_kernel(circuit_btree_loss_backward_kernel, grid, tw * 32, tsmem, st, /*dependent=*/false, a, fits ? 1 : 0);
   } else {
     launch_kernel(circuit_btree_backward_kernel, resident, threads, smem, st, overlapped(h), a, counter);
   }
@@ -1199,7 +1200,9 @@ int backward_tail(mtpc_head* head, const BackwardLayout& B, uint8_t* bw, const v
     int row_blocks = (16 * head->num_sms + col_blocks - 1) / col_blocks;   // enough CTAs to fill the device, each walks rows
     if (row_blocks > T) row_blocks = T;
     if (row_blocks > 65535) row_blocks = 65535;
-    launch_kernel(logit_gradient_kernel, dim3(col_blocks, row_blocks), 256, 0, st, overlapped(head), la);
+    // not as a dependent: CTAs scheduled beside the circuit kernel's last ones would share a few SMs (517 us became 690 at 4096
+    // positions of a 16 x 32 x 256 head)
+    launch_kernel(logit_gradient_kernel, dim3(col_blocks, row_blocks), 256, 0, st, /*dependent=*/false, la);
   }
   head->launches++;
   int rc = check_launch();

@@ -45,9 +45,6 @@ bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 // How one launch of the projection kernel tiles the N axis and uses shared / tensor memory.
 struct Tiling {
   int tile_cols;        // accumulator width of an emission tile
-  int group_units;      // emission units per work group
-  int group_tiles;      // tiles of a full group
-  int num_groups;       // groups covering all n*r units
   int slot_stride, num_slots, stages, stage_bytes, smem;
   int pair_stages, pair_stage_bytes, pair_smem;   // the same ring when two CTAs share every MMA (half a weight tile per CTA)
 };
@@ -74,7 +71,6 @@ struct Layout {
   size_t total;
 };
 
-int gcd_int(int a, int b) { while (b) { int t = a % b; a = b; b = t; } return a; }
 
 // Shared-memory ring and TMEM slots for tiles of `tile_cols` emission columns and `sum_cols` sum columns.
 bool fit_tiling(Tiling* t, int sum_cols) {
@@ -122,16 +118,7 @@ int plan(const mtpc_config& c, Layout* L, bool factored = false) {
   L->sum_cols = sum_cols;
   L->sum_tiles = (L->sum_rows + sum_cols - 1) / sum_cols;
   const int emit_units = c.n * c.r;
-  // log-likelihood: 256-column tiles; a group is the shortest run of whole units that is a whole number of tiles
-  const int lcm = c.v / gcd_int(c.v, 256) * 256;
   L->lp.tile_cols = 256;
-  L->lp.group_units = lcm / c.v;
-  L->lp.group_tiles = lcm / 256;
-  if (L->lp.group_units > emit_units) {   // fewer units than one full group: a single, partial group
-    L->lp.group_units = emit_units;
-    L->lp.group_tiles = (emit_units * c.v + 255) / 256;
-  }
-  L->lp.num_groups = (emit_units + L->lp.group_units - 1) / L->lp.group_units;
   if (!fit_tiling(&L->lp, sum_cols)) return MTPC_ERR_UNSUPPORTED;
 
   L->max_windows = static_cast<size_t>(c.max_positions) * c.max_windows_per_pos;
@@ -360,22 +347,29 @@ void launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem
 // The kernels of a call follow each other as dependents, unless events are recorded between them.
 bool overlapped(const mtpc_head* h) { return h->ring == 0; }
 
-// Launch the projection kernel for `rows` positions over the emission groups (with_emit) and / or the sum tiles.
 // Units per work item of the log-likelihood mode. An item covers its units with 256-column tiles; unless the
 // units end on a tile boundary the last tile is partly wasted (its tail belongs to the next item, which recomputes it).
-// Items are dealt round-robin to `ctas` persistent CTAs, so a launch takes about rounds x tiles-per-item tile times:
+// Items are dealt round-robin to `ctas` persistent CTAs and the launch's sum tiles fill the last round (ItemWalk), so a launch
+// takes about rounds x tiles-per-item tile times and the share of the sum tiles that the last round has no room for:
 // pick the count that minimises that (v = 320: 4 units = 5 tiles, nothing wasted; v = 272: 8 units = 9 tiles, 6 % wasted
 // but twice as many items as the waste-free 16 units = 17 tiles).
-int choose_group_units(int v, int emit_units, int m_tiles, int ctas) {
-  int best = 1;
-  long long best_cost = -1;
+struct ItemPlan {
+  int units = 1;             // per item
+  long long tiles = 0;       // tile times of the launch
+};
+ItemPlan choose_group_units(int v, int emit_units, int m_tiles, int ctas, int sum_tiles) {
+  ItemPlan best;
+  const long long sums = static_cast<long long>(sum_tiles) * m_tiles;
+  if (emit_units == 0) best.tiles = (sums + ctas - 1) / ctas;
   const int limit = emit_units < 64 ? emit_units : 64;
   for (int u = 1; u <= limit; ++u) {
-    const long long tiles = (static_cast<long long>(u) * v + 255) / 256;
-    const long long groups = (emit_units + u - 1) / u;
-    const long long rounds = (groups * m_tiles + ctas - 1) / ctas;
-    const long long cost = rounds * tiles;
-    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = u; }
+    const int tiles = (u * v + 255) / 256;
+    const long long items = static_cast<long long>((emit_units + u - 1) / u) * m_tiles;
+    const long long rounds = (items + ctas - 1) / ctas;
+    const long long rest = sums - (rounds * ctas - items) * tiles;
+    const long long cost = rounds * tiles + (rest > 0 ? (rest + ctas - 1) / ctas : 0);
+    if (u == 1 || cost < best.tiles) { best.tiles = cost; best.units = u; }
+    if (rounds == 1 && rest <= 0) break;                              // longer items only make the one round longer
   }
   return best;
 }
@@ -394,6 +388,7 @@ struct GradArgs {            // what the projection kernel keeps for the backwar
   size_t logit_pitch = 0;
 };
 
+// Launch the projection kernel for `rows` positions over the emission groups (with_emit) and / or the sum tiles.
 // first_row: where in log omega the launch's positions start (a draft that runs in chunks of positions).
 int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit, bool with_sum, const int* targets, cudaStream_t st,
                 const GradArgs* ga = nullptr, const GroupArgs* grp = nullptr, int first_row = 0) {
@@ -413,13 +408,23 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
   if (rc != MTPC_OK) return rc;
   p.T = rows;
   p.m_tiles = (rows + kBlockM - 1) / kBlockM;
-  // Two CTAs per MMA when there are at least two m-tiles to pair up (and the device can hold a cluster at all) and K is long
-  // enough for the halved operand traffic to count: with few K steps the epilogue bounds a tile, and a lone CTA need not wait
-  // for its partner's. Alone / in pairs, us, CP: d = 256, 32 units of 256 symbols, 256 positions 11.6 / 12.8; 128 units of 320,
-  // 8192 positions 375 / 400; d = 1024, 64 x 320, 256 positions 19.9 / 20.8; 128 x 320, 2048 positions 138.8 / 139.3; d = 1536,
-  // 128 x 320, 1024 positions 107.8 / 105.8; d = 2048, 256 positions 52.0 / 47.6; d = 4096, 64 x 320, 256 positions 67.3 / 60.7.
-  const bool pair = grp == nullptr && (h->projection_variant == 2 || (h->projection_variant == 0 && p.m_tiles >= 2 &&
-                                                                      h->max_pairs > 0 && c.d > 1024));
+  // Every CTA alone, or two CTAs per MMA (when there are two m-tiles to pair up and the device can hold a cluster at all): whichever
+  // plan takes less time. A pair moves less operand data per MMA, which counts when K is long; with few K steps the epilogue bounds
+  // a tile, and a lone CTA need not wait for its partner's. Time per tile in pairs / alone, measured over 26 shapes of 256 to 8192
+  // positions: d = 256 1.06 to 1.10, d = 1024 1.00 to 1.07, d = 1536 0.98, d = 2048 0.92 to 0.96, d = 4096 0.89 to 0.97. A ragged
+  // number of m-tiles costs the pairs more tiles (384 positions, d = 4096, 8 x 16 x 320: 5 tiles a pair against 4, 139.6 us / 121.9).
+  const int emit_units = with_emit ? c.n * c.r : 0, launch_sums = with_sum ? L.sum_tiles : 0;
+  bool pair = grp == nullptr && h->projection_variant == 2;
+  ItemPlan plan;
+  if (grp == nullptr) {
+    plan = choose_group_units(c.v, emit_units, p.m_tiles, h->num_sms, launch_sums);
+    if (h->projection_variant != 1 && h->max_pairs > 0) {
+      const ItemPlan two = choose_group_units(c.v, emit_units, (p.m_tiles + 1) / 2, h->max_pairs, launch_sums);
+      if (h->projection_variant == 0 && p.m_tiles >= 2)
+        pair = c.d <= 1024 ? two.tiles * 34 <= plan.tiles * 33 : two.tiles * 12 <= plan.tiles * 13;
+      if (pair) plan = two;
+    }
+  }
   const int ctas = pair ? 2 : 1;
   const int workers = pair ? h->max_pairs : h->num_sms;               // CTAs, or CTA pairs, resident at once
   p.m_units = (p.m_tiles + ctas - 1) / ctas;
@@ -433,15 +438,9 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
   p.n = c.n; p.r = c.r; p.v = c.v;
   p.vv = valid_symbols(c);
   p.emit_units = c.n * c.r;
-  p.num_groups = with_emit ? tl.num_groups : 0;
-  p.group_units = tl.group_units;
-  if (grp != nullptr) {                                               // a row tile's r units are cut into runs that fill the device
-    p.group_units = choose_group_units(c.v, c.r, grp->max_tiles, workers);
-    p.num_groups = (c.r + p.group_units - 1) / p.group_units;
-  } else if (with_emit) {
-    p.group_units = choose_group_units(c.v, p.emit_units, p.m_units, workers);
-    p.num_groups = (p.emit_units + p.group_units - 1) / p.group_units;
-  }
+  p.group_units = plan.units;
+  if (grp != nullptr) p.group_units = choose_group_units(c.v, c.r, grp->max_tiles, workers, 0).units;   // runs of a row tile's r units
+  p.num_groups = grp != nullptr ? (c.r + p.group_units - 1) / p.group_units : (emit_units + p.group_units - 1) / p.group_units;
   p.tile_cols = tl.tile_cols;
   p.num_sum_tiles = with_sum ? L.sum_tiles : 0;
   p.sum_cols = L.sum_cols;

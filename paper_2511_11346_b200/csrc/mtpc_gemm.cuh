@@ -149,7 +149,7 @@ __device__ __forceinline__ TileCoord group_coord(const GemmParams& p, int item) 
 // the group next, so the CTAs that run at the same time share a few groups' weights through L2 while the block's
 // hidden states (m_block x 128 rows) stay L2-resident for every group; a block is finished before the next one
 // starts, so the weights are streamed from HBM once per block and the hidden states once. Sum items follow,
-// m-tile fastest.
+// m-tile fastest (ItemWalk).
 __device__ __forceinline__ TileCoord tile_coord(const GemmParams& p, int item) {
   TileCoord c;
   const int emit_items = p.num_groups * p.m_units;
@@ -182,6 +182,33 @@ __device__ __forceinline__ TileCoord tile_coord(const GemmParams& p, int item) {
     c.ntiles = (c.nunits * p.v + p.tile_cols - 1) / p.tile_cols;
   }
   return c;
+}
+
+// A worker's items. Emission items are dealt round-robin; the workers that get none in the last round take sum tiles instead, up to
+// an emission item's worth each, and what then remains is dealt round-robin to all: neighbours in time share a sum tile's weights.
+// (Dealt round-robin behind the emission items, 84 sum tiles of 693 positions of a contextual 8 x 32 x 320 head made the longest
+// worker 16 tiles long; 15 now, 14.2 the mean. Runs of consecutive sum tiles per worker stream all their weights at once: 4096
+// positions of a 16 x 32 x 256 tree head 3349 us a draft and its acceptance instead of 3116; 3271 before.)
+struct ItemWalk {
+  int worker, workers, emit_items, idle, quota_end, end;
+  __device__ __forceinline__ int first_sum(bool after_quota) const {
+    const int j = worker - (workers - idle);                          // >= 0: a worker with no emission item in the last round
+    if (!after_quota && j >= 0 && emit_items + j < min(quota_end, end)) return emit_items + j;
+    return quota_end + worker;
+  }
+  __device__ __forceinline__ int first() const { return worker < emit_items ? worker : first_sum(false); }
+  __device__ __forceinline__ int next(int item) const {
+    if (item < emit_items) return item + workers < emit_items ? item + workers : first_sum(false);
+    if (item >= quota_end) return item + workers;
+    return item + idle < min(quota_end, end) ? item + idle : first_sum(true);
+  }
+};
+__device__ __forceinline__ ItemWalk item_walk(const GemmParams& p, int emit_items, int sum_items, int worker, int workers) {
+  const int busy = emit_items % workers;
+  ItemWalk w{worker, workers, emit_items, busy ? workers - busy : 0, 0, emit_items + sum_items};
+  const long long room = static_cast<long long>(w.idle) * ((p.group_units * p.v + p.tile_cols - 1) / p.tile_cols);
+  w.quota_end = emit_items + (room < sum_items ? static_cast<int>(room) : sum_items);
+  return w;
 }
 
 // Padding columns of a unit (vocabulary not a multiple of 16) count as logit = -inf: never the maximum, no mass.
@@ -232,7 +259,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   constexpr bool kGrouped = MODE == kModeLogitsGrouped;
   if (kGrouped) grid_dependency_wait();   // the tiles are read below
   static_assert(!kGrouped || CTAS == 1, "grouped tiles are ragged: no pairing");
-  const int num_items = kGrouped ? *p.group_num_tiles * p.num_groups : (p.num_groups + p.num_sum_tiles) * p.m_units;
+  const int emit_items = kGrouped ? *p.group_num_tiles * p.num_groups : p.num_groups * p.m_units;
   const uint32_t cta_rank = CTAS == 2 ? cluster_cta_rank() : 0u;      // 0 = the pair's leader
   auto coord = [&](int item) {
     if (kGrouped) return group_coord(p, item);
@@ -241,8 +268,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
     c.count = min(kBlockM, p.T - c.arow);                             // <= 0: a pair's second CTA past the last position
     return c;
   };
-  const int first_item = CTAS == 2 ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
-  const int item_step = CTAS == 2 ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
+  const int worker = CTAS == 2 ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
+  const int workers = CTAS == 2 ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
+  const ItemWalk walk = item_walk(p, emit_items, kGrouped ? 0 : p.num_sum_tiles * p.m_units, worker, workers);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -284,7 +312,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
     if (lane == 0) {
       uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0;
       bool ok = true;
-      for (int item = first_item; item < num_items && ok; item += item_step) {
+      for (int item = walk.first(); item < walk.end && ok; item = walk.next(item)) {
         const TileCoord tc = coord(item);
         const CUtensorMap* tmb = tc.is_sum ? &p.tm_sum : &p.tm_emit;
         const int brows = tc.cols / CTAS;                                 // weight rows this CTA stages per tile
@@ -330,7 +358,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
     if (lane == 0 && cta_rank == 0) {
       uint32_t stage = 0, phase = 0, use = 0;
       bool ok = true;
-      for (int item = first_item; item < num_items && ok; item += item_step) {
+      for (int item = walk.first(); item < walk.end && ok; item = walk.next(item)) {
         const TileCoord tc = coord(item);
         const uint32_t idesc = umma_idesc_bf16(kBlockM * CTAS, tc.cols);
         for (int t = 0; t < tc.ntiles && ok; ++t, ++use) {
@@ -380,7 +408,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
       if (CTAS == 2) mbar_arrive_cluster(cluster_map_shared(smem_u32(&ctl->tempty[slot]), 0));
       else mbar_arrive(smem_u32(&ctl->tempty[slot]));
     };
-    for (int item = first_item; item < num_items && ok; item += item_step) {
+    for (int item = walk.first(); item < walk.end && ok; item = walk.next(item)) {
       const TileCoord tc = coord(item);
       const int row = tc.arow + quarter * 32 + lane;
       const bool valid = quarter * 32 + lane < tc.count;

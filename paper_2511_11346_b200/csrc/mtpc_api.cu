@@ -25,6 +25,7 @@ using namespace mtpc;
 constexpr size_t kAlign = 256;
 constexpr int kMaxPhases = 5;
 constexpr size_t kSlotSmemLimit = 160 * 1024;   // latent-draw tables of the draft slot kernel kept in shared memory up to this
+constexpr size_t kSlotSmemPair = 112 * 1024;     // two of its CTAs share an SM up to this
 constexpr int kMaxDraftVocab = 512;     // symbols a warp draws from in one go
 constexpr int kHostChunkPositions = 2048;   // host-buffer calls upload and process this many positions at a time
 constexpr int kWorkCounterWord = 16;   // word of the 256-byte status area used as the circuit kernels' work counter
@@ -55,7 +56,7 @@ struct Layout {
   Tiling lp;            // 256-column tiles over the flattened (i,k,b) axis
   size_t max_windows;
   // workspace offsets (bytes)
-  size_t off_status, off_wemit, off_wsum, off_hidden, off_logA, off_G, off_logw, off_sel, off_logits, off_unit_lse;
+  size_t off_status, off_wemit, off_wsum, off_hidden, off_logA, off_probA, off_cdfA, off_G, off_logw, off_sel, off_logits, off_unit_lse;
   size_t off_prefix, off_partial, off_sum_bias;   // training loss: prefix log-marginals [max_positions, n], per-sequence terms
   size_t off_msg;       // slot messages of the drafted windows [max_windows, n, r], kept for the acceptance stage
   int decode_max_p;     // positions the few-position draft path can take
@@ -131,6 +132,8 @@ int plan(const mtpc_config& c, Layout* L, bool factored = false) {
   L->off_wsum = take(f32 ? static_cast<size_t>(L->sum_rows) * c.d * 2 : 0);
   L->off_hidden = take(f32 ? static_cast<size_t>(c.max_positions) * c.d * 2 : 0);
   L->off_logA = take(c.family == MTPC_HMM && !ctx ? static_cast<size_t>(c.n - 1) * c.r * c.r * 4 : 0);
+  L->off_probA = take(c.family == MTPC_HMM && !ctx ? static_cast<size_t>(c.n - 1) * c.r * c.r * 4 : 0);
+  L->off_cdfA = take(c.family == MTPC_HMM && !ctx ? static_cast<size_t>(c.n - 1) * c.r * c.r * 4 : 0);
   L->off_sum_bias = take(ctx ? static_cast<size_t>(L->sum_rows) * 4 : 0);
   L->off_G = take(L->max_windows * c.n * c.r * 4);
   L->off_logw = take(static_cast<size_t>(c.max_positions) * L->sum_rows * 4);
@@ -512,8 +515,10 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
     const int stride = hmm_table_stride(h);
     const int items = stride == 0 ? (W + kHmmWarps - 1) / kHmmWarps : W / wpp * ((wpp + kHmmWarps - 1) / kHmmWarps);
     const int resident = sms_times_resident(h, smem);
+    const bool probabilities = stride == 0 && L.off_probA != 0;          // (a call without a head has log-probabilities alone)
     launch_kernel(circuit_hmm_kernel, items < resident ? items : resident, kHmmWarps * 32, smem, st, overlapped(h), G, logw,
-                  hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r, L.sum_rows, chunk);
+                  probabilities ? at<float>(h, L.off_probA) : hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r,
+                  L.sum_rows, chunk, probabilities ? 1 : 0);
   } else if (sweep) {
     const int warps = c.n / 2 < 8 ? c.n / 2 : 8;                         // a warp per node of the owners' level
     const bool fits = btree_prefix_smem_floats(c.n, c.r, warps, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
@@ -826,17 +831,25 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
       const size_t base = static_cast<size_t>((2 * c.r + 3) & ~3) * sizeof(float);
       const size_t with_tables = base + static_cast<size_t>(chain) * c.r * c.r * sizeof(float);
       const int in_smem = chain > 0 && with_tables <= kSlotSmemLimit;
+      // The units' weights stay in shared memory for the byte draws where there are many draws to a unit, if they fit beside the
+      // tables without costing an SM its second CTA, or there is no second one to be had anyway. (Where most are never used, the
+      // CTAs are better kept small enough to wait beside the weight pass's: 27 positions of a tree head, 4 windows on 32 units,
+      // 109.4 us with them and 106.3 without; 16 windows on 16 units, 64 positions: 153.4 and 157.0.)
+      const size_t weights = static_cast<size_t>(c.r) * ((c.v + 31) / 32 * 32) * sizeof(float);
+      const size_t smem = (in_smem ? with_tables : base) + weights;
+      const int weights_in_smem = c.v <= kMaxDraftVocab && 2 * wpp >= c.r &&
+                                  (smem <= kSlotSmemPair || (smem <= kSlotSmemLimit && c.n * P <= h->num_sms));
       // builds of the narrow kernel that unroll 4, 8, 10 or 16 batches of 32 symbols: the smallest that covers v
       auto* slot_kernel = c.v > kMaxDraftVocab ? draft_slot_kernel<true, 16>
                           : c.v <= 128 ? draft_slot_kernel<false, 4>
                           : c.v <= 256 ? draft_slot_kernel<false, 8>
                           : c.v <= 320 ? draft_slot_kernel<false, 10> : draft_slot_kernel<false, 16>;
       launch_kernel(slot_kernel, dim3(c.n, P), kSlotThreads,
-                    in_smem ? with_tables : base, st, overlapped(h), c.family,
-                    at<float>(h, L.off_logits), at<float>(h, L.off_logw), hmm_tables(h), uniforms, out_bytes,
+                    weights_in_smem ? smem : smem - weights, st, overlapped(h), c.family,
+                    at<float>(h, L.off_logits), at<float>(h, L.off_logw), is_ctx(h) ? hmm_tables(h) : at<float>(h, L.off_cdfA), uniforms, out_bytes,
                     at<float>(h, L.off_G), at<float>(h, L.off_unit_lse), at<unsigned>(h, L.off_status),
                     at<unsigned>(h, L.off_status) + kWorkCounterWord, wpp, c.n, c.r, c.v, valid_symbols(c), L.sum_rows,
-                    hmm_table_stride(h), in_smem);
+                    hmm_table_stride(h), in_smem, weights_in_smem);
     }
     h->launches++;
     h->draft_P = P;
@@ -874,7 +887,9 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
                   at<unsigned>(h, L.off_status), wc, wpp, c.n, c.r, L.sum_rows, hmm_table_stride(h));
     pt.end();
     pt.begin();
-    auto* pick = c.v > kMaxDraftVocab ? draft_pick_kernel<true> : draft_pick_kernel<false>;
+    auto* pick = c.v > kMaxDraftVocab ? draft_pick_kernel<true, 16>
+                 : c.v <= 256 ? draft_pick_kernel<false, 8>
+                 : c.v <= 320 ? draft_pick_kernel<false, 10> : draft_pick_kernel<false, 16>;
     launch_kernel(pick, (wc * c.n + 7) / 8, 256, 0, st, overlapped(h), keep.logit_out, keep.lse_out, sel, u,
                   out_bytes + w0 * c.n, at<float>(h, L.off_G) + w0 * c.n * c.r, at<unsigned>(h, L.off_status), wc * c.n, wpp,
                   c.n, c.r, c.v, valid_symbols(c));
@@ -1380,7 +1395,9 @@ static int bind_parameters(mtpc_head* h, const void* W_emit, const void* W_sum, 
   } else if (cfg->family == MTPC_HMM && cfg->n > 1) {
     const int rows = (cfg->n - 1) * cfg->r;
     log_softmax_rows_kernel<<<(rows + 127) / 128, 128, 0, st>>>(T_static, at<float>(h, L.off_logA), rows, cfg->r);
-    h->launches++;
+    static_tables_kernel<<<(rows + 7) / 8, 256, 0, st>>>(at<float>(h, L.off_logA), at<float>(h, L.off_probA), at<float>(h, L.off_cdfA),
+                                                         rows, cfg->r);
+    h->launches += 2;
   }
   if (check_launch() != MTPC_OK) return MTPC_ERR_CUDA;
   const uint64_t emit_rows = static_cast<uint64_t>(cfg->n) * cfg->r * cfg->v;
@@ -2282,7 +2299,7 @@ extern "C" int mtpc_window_logprob_static(const mtpc_config* cfg, const void* W_
   L.off_G = take(static_cast<size_t>(c.max_positions) * c.n * c.r * 4);
   L.off_logw = take(static_cast<size_t>(c.max_positions) * L.sum_rows * 4);
   L.off_sel = L.off_wemit = L.off_wsum = L.off_hidden = L.off_logits = L.off_unit_lse = 0;   // unused by this call
-  L.off_prefix = L.off_partial = L.off_sum_bias = L.off_msg = 0;
+  L.off_prefix = L.off_partial = L.off_sum_bias = L.off_msg = L.off_probA = L.off_cdfA = 0;
   L.off_h_hidden = L.off_h_targets = L.off_h_uniforms = L.off_h_bytes = L.off_h_out = 0;
   L.total = off;
   if (L.total > static_cast<size_t>(MTPC_STATIC_SCRATCH_BYTES)) return MTPC_ERR_STATIC_SCRATCH;

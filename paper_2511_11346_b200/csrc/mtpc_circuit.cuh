@@ -171,6 +171,16 @@ __device__ __forceinline__ void cp_async_4(float* dst, const float* src) {
                "l"(src)
                : "memory");
 }
+// The calling threads' share (of `threads`) of copying count floats to shared memory, not committed.
+__device__ __forceinline__ void fetch_floats(float* dst, const float* src, int count, int threads) {
+  if ((count & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0) {
+#pragma unroll 1
+    for (int e = threadIdx.x * 4; e < count; e += threads * 4) cp_async_16(dst + e, src + e);
+  } else {
+#pragma unroll 1
+    for (int e = threadIdx.x; e < count; e += threads) cp_async_4(dst + e, src + e);
+  }
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -524,8 +534,9 @@ __device__ __forceinline__ float hmm_forward_step(float alpha, float* ev, const 
 // Position p = w / wpp reads logA_i[a][k] at tables[p * table_stride + (i-1) r^2 + a r + k]: contextual transitions (App. H)
 // have table_stride = sum_rows (28 KB per position at n = 8, r = 32, read once: the HBM stream that bounds the call then),
 // static ones table_stride = 0.
-// A CTA's warps work on windows that share tables. The tables are turned into probabilities on their way into shared
-// memory, by all threads: once per CTA for static transitions, once per position for contextual ones, so that a step of the
+// A CTA's warps work on windows that share tables. They reach shared memory as probabilities: contextual ones (log-probabilities)
+// are exponentiated on their way there by all threads, once per position; of static ones a head keeps the probabilities
+// (`probabilities`), and a CTA copies them while it still waits for the kernel before it. So a step of the
 // recursion is one warp maximum, 32 multiply-adds per lane and one logarithm, with no exponential of a table entry and no
 // memory round trip in it. Tables that do not fit (n = 64 at r = 32) go through in chunks of chunk_tables. The prefix log-sum-exps are taken at the
 // end, lane = slot. Measured against one warp per window streaming log tables: 8192 windows at n = 8, r = 32: 42 -> 22 us;
@@ -538,13 +549,22 @@ __host__ __device__ inline size_t hmm_circuit_smem_floats(int n, int r, bool wit
   return (static_cast<size_t>(chunk_tables) * r * r + 3) / 4 * 4 +
          static_cast<size_t>(kHmmWarps) * hmm_circuit_warp_floats(n, r, with_prefix);
 }
-__global__ void __launch_bounds__(32 * kHmmWarps) circuit_hmm_kernel(
+__global__ void __launch_bounds__(32 * kHmmWarps, 4) circuit_hmm_kernel(
     const float* __restrict__ G, const float* __restrict__ logw, const float* __restrict__ tables, int table_stride,
     float* __restrict__ out, float* __restrict__ prefix, float* __restrict__ msg, int W, int wpp, int n, int r, int sum_rows,
-    int chunk_tables) {
+    int chunk_tables, int probabilities) {
   extern __shared__ __align__(16) float sm[];
   grid_launch_dependents();
+  const bool early = probabilities && chunk_tables >= n - 1;           // all of a static set, written when the head was made
+  if (early) {
+    fetch_floats(sm, tables, (n - 1) * r * r, 32 * kHmmWarps);
+    cp_async_commit();
+  }
   grid_dependency_wait();   // G and log omega come from the kernel before this one
+  if (early) {
+    cp_async_wait<0>();
+    __syncthreads();
+  }
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rr = r * r;
   float* E = sm;
@@ -557,7 +577,7 @@ __global__ void __launch_bounds__(32 * kHmmWarps) circuit_hmm_kernel(
   // work items: kHmmWarps windows each; contextual tables: of one position
   const int per_pos = table_stride == 0 ? 0 : (wpp + kHmmWarps - 1) / kHmmWarps;
   const int items = table_stride == 0 ? (W + kHmmWarps - 1) / kHmmWarps : (W / wpp) * per_pos;
-  int loaded_pos = -1, loaded_first = -1;                  // which tables E holds
+  int loaded_pos = early ? 0 : -1, loaded_first = loaded_pos;          // which tables E holds
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
     int pos_tab = 0, w;
     bool valid;
@@ -588,7 +608,11 @@ __global__ void __launch_bounds__(32 * kHmmWarps) circuit_hmm_kernel(
         __syncthreads();                                   // every warp is done with what E held
         const float* src = tb + static_cast<size_t>(t0) * rr;
         const int count = nt * rr;
-        if ((count & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+        if (probabilities) {
+          fetch_floats(E, src, count, 32 * kHmmWarps);
+          cp_async_commit();
+          cp_async_wait<0>();
+        } else if ((count & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
           for (int e = threadIdx.x * 4; e < count; e += 32 * kHmmWarps * 4) {
             const float4 x = *reinterpret_cast<const float4*>(src + e);
             *reinterpret_cast<float4*>(E + e) = make_float4(__expf(x.x), __expf(x.y), __expf(x.z), __expf(x.w));

@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
   if (p.ksplit > 1) cluster_sync_all();   // every CTA of the cluster runs before one writes into another's shared memory
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
-  grid_launch_dependents();   // the per-slot kernel may be scheduled as SMs free up; it waits for this grid's results
   grid_dependency_wait();     // a draft that follows another call closely sets up its barriers while that one finishes
+  grid_launch_dependents();   // the per-slot kernel may be scheduled as SMs free up; it waits for this grid's results
 
   const int quarter = warp & 3;
   const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
@@ -337,6 +337,25 @@ __device__ __forceinline__ int warp_inv_cdf_logp(float logp, int r, float u, int
   return hit ? __ffs(hit) - 1 : r - 1;
 }
 
+// What a head with static transitions keeps of its `rows` rows of r <= 32 log-probabilities besides them, one warp per row:
+// the probabilities (the circuit's recursion), and their running sums: with them a draw is one comparison per lane and a ballot, and
+// yields what warp_inv_cdf_logp yields.
+__global__ void __launch_bounds__(256) static_tables_kernel(const float* __restrict__ logp, float* __restrict__ prob,
+                                                            float* __restrict__ cdf, int rows, int r) {
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= rows) return;
+  const float lp = lane < r ? logp[static_cast<size_t>(row) * r + lane] : -CUDART_INF_F;
+  const float cum = warp_scan_incl(lane < r ? expf(lp) : 0.f, lane);
+  if (lane < r) {
+    prob[static_cast<size_t>(row) * r + lane] = __expf(lp);
+    cdf[static_cast<size_t>(row) * r + lane] = cum;
+  }
+}
+__device__ __forceinline__ int warp_inv_cdf(float cum, int r, float u, int lane) {
+  const unsigned hit = __ballot_sync(kFull, lane < r && u < cum);
+  return hit ? __ffs(hit) - 1 : r - 1;
+}
+
 // The same draw over the softmax of r <= 128 unnormalised logits x[0..r): lane l owns the consecutive indices
 // [l * per, (l + 1) * per), per = ceil(r / 32) <= 4; u * total < running sum, index order, no division.
 __device__ __forceinline__ int warp_inv_cdf_logits_wide(const float* __restrict__ x, int r, float u, int lane) {
@@ -413,67 +432,100 @@ __device__ __forceinline__ float warp_chunk_sum(const float* __restrict__ x, int
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
   return s;
 }
-// Inverse CDF inside one chunk of 32 * per symbols starting at c0, on the weights exp(x[b] - m): lane l owns the
-// consecutive symbols [c0 + l*per, c0 + (l+1)*per). The threshold is u * (the chunk's total) when `relative`, else
-// `thr` itself. Returns the smallest symbol whose running sum exceeds the threshold; the last existing symbol of
-// the chunk if rounding leaves none. All lanes return the same value.
-template <int NQ>   // per <= NQ <= kSlotMaxPerLane: the steps that are unrolled
-__device__ __forceinline__ int warp_inv_cdf_chunk(const float* __restrict__ x, int c0, int per, int vv, float m, float thr,
-                                                  bool relative, int lane) {
-  const int b0 = c0 + lane * per;
-  float ev[NQ];
+// e[q] = p[q] for q < per (the widest loads that per allows; p is aligned for them), `fill` from p + limit on and in the rest of e.
+template <int NQ>
+__device__ __forceinline__ void load_run(const float* p, int per, int limit, float fill, float (&e)[NQ]) {
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) ev[q] = (q < per && b0 + q < vv) ? x[b0 + q] : -CUDART_INF_F;
+  for (int q = 0; q < NQ; ++q) e[q] = fill;
+  if (per % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q + 3 < NQ; q += 4)
+      if (q < per && q < limit) {
+        const float4 x = *reinterpret_cast<const float4*>(p + q);
+        e[q] = x.x; e[q + 1] = x.y; e[q + 2] = x.z; e[q + 3] = x.w;
+      }
+  } else if (per % 2 == 0) {
+#pragma unroll
+    for (int q = 0; q + 1 < NQ; q += 2)
+      if (q < per && q < limit) {
+        const float2 x = *reinterpret_cast<const float2*>(p + q);
+        e[q] = x.x; e[q + 1] = x.y;
+      }
+  } else {
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+      if (q < per && q < limit) e[q] = p[q];
+  }
+}
+// Inverse CDF over weights held by a warp, lane l those of the consecutive symbols [b0, b0 + per), b0 = c0 + l per (0 beyond
+// end and beyond per). The threshold is thr * (the weights' total) when `relative`, else thr itself. Returns the smallest symbol
+// whose running sum exceeds it; the last one below end if rounding leaves none. All lanes return the same value.
+template <int NQ>   // per <= NQ <= kSlotMaxPerLane: the steps that are unrolled
+__device__ __forceinline__ int warp_inv_cdf_weights(const float (&ev)[NQ], int c0, int per, int end, float thr, bool relative, int lane) {
   float part = 0.f;
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    ev[q] = __expf(ev[q] - m);
-    part += ev[q];
-  }
+  for (int q = 0; q < NQ; ++q) part += ev[q];
   const float incl = warp_scan_incl(part, lane);
   if (relative) thr *= __shfl_sync(kFull, incl, 31);
   const unsigned hit = __ballot_sync(kFull, thr < incl);
-  int byte = min(c0 + 32 * per, vv) - 1;
-  if (hit) {
-    const int src = __ffs(hit) - 1;
-    int found = -1;
-    const float before = __shfl_up_sync(kFull, incl, 1);
-    if (lane == src) {
-      float cum = lane == 0 ? 0.f : before;
+  const float before = __shfl_up_sync(kFull, incl, 1);
+  // the running sums never fall: the number of a lane's that the threshold is not below is the place of the first that it is
+  float cum = lane == 0 ? 0.f : before;
+  int passed = 0;
 #pragma unroll
-      for (int q = 0; q < NQ; ++q)
-        if (found < 0 && q < per && b0 + q < vv) {
-          cum += ev[q];
-          if (thr < cum) found = b0 + q;
-        }
-      if (found < 0) found = min(b0 + per, vv) - 1;   // the lane's total passed the threshold: its last byte
-    }
-    byte = __shfl_sync(kFull, found, src);
+  for (int q = 0; q < NQ; ++q) {
+    cum += ev[q];
+    passed += thr < cum ? 0 : 1;
   }
-  return byte;
+  const int b0 = c0 + lane * per;
+  const int found = min(b0 + min(passed, per), min(b0 + per, end) - 1);    // the lane's total passed the threshold: its last symbol
+  return hit ? __shfl_sync(kFull, found, __ffs(hit) - 1) : min(c0 + 32 * per, end) - 1;
+}
+// The same over the 32 * per symbols starting at c0 of a unit of v, vv of them real, on the weights exp(x[b] - m).
+template <int NQ>
+__device__ __forceinline__ int warp_inv_cdf_chunk(const float* __restrict__ x, int c0, int per, int v, int vv, float m, float thr,
+                                                  bool relative, int lane) {
+  const int b0 = c0 + lane * per;
+  float ev[NQ];
+  load_run<NQ>(x + b0, per, v - b0, -CUDART_INF_F, ev);
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) ev[q] = b0 + q < vv ? fast_ex2((ev[q] - m) * kLog2e) : 0.f;
+  return warp_inv_cdf_weights<NQ>(ev, c0, per, vv, thr, relative, lane);
 }
 
-// logA: HMM transition log-probabilities [n-1, r, r]; position p reads them at logA + p * logA_stride (stride 0:
-// one static set for all positions; stride sum_rows with logA = log omega + r: contextual tables, App. H).
-// grid = (n, P), 16 warps. Shared memory: 2 * r floats (max and log-sum-exp of each unit of the slot), then, when
-// tables_in_smem, the chain's tables (slot_chain_length * r * r floats), fetched by cp.async while the log-sum-exps
-// are computed, so that the data-dependent row reads of the latent draws do not each cost a trip to L2.
+// hmm: HMM transition tables [n-1, r, r]; position p reads them at hmm + p * hmm_stride. Stride 0: one static set for all
+// positions, as running sums of probabilities (static_tables_kernel); stride sum_rows with hmm = log omega + r: contextual
+// tables (App. H) of log-probabilities.
+// grid = (n, P), 16 warps. Shared memory: 2 * r floats (max and log-sum-exp of each unit of the slot); when weights_in_smem, the
+// units' weights exp(logit - max), which the byte draws then read instead of the logits; when tables_in_smem, the chain's tables
+// (slot_chain_length * r * r floats), fetched by cp.async while the log-sum-exps are computed, static ones while the kernel still
+// waits for the one before it.
 // The log-sum-exps also go to unit_lse_out [P, n, r], so that later calls can turn the retained logits into log phi.
-// WIDE: vocabularies of more than 512 symbols (a separate build: the narrow one keeps a unit's logits in 16 registers per lane).
+// Bound by trips to memory that wait on one another, and by instructions where a device full of CTAs shares them: so a warp requests
+// its first unit's logits, its first window's uniforms and the root weights before anything else, and the next unit's logits
+// before it works on this one's. Loops that run once or twice stay rolled: at
+// these durations fetching instructions counts. Time after the weight pass, per slot stage: mixture n = 16, r = 16, v = 320, 64
+// positions of 16 windows 22 -> 15.5 us; HMM n = 16, r = 32, 8 positions 16.2 -> 9.8; tree n = 8, r = 32, 27 positions 10.4 -> 8.
+// WIDE: vocabularies of more than 512 symbols (a separate build: the narrow one keeps a unit's logits in registers).
 template <bool WIDE, int NQ>   // NQ: batches of 32 symbols of a unit that are unrolled (v <= 32 NQ; WIDE: 16)
 __global__ void __launch_bounds__(kSlotThreads, 2) draft_slot_kernel(
-    int family, const float* __restrict__ logits, const float* __restrict__ logw, const float* __restrict__ logA,
+    int family, const float* __restrict__ logits, const float* __restrict__ logw, const float* __restrict__ hmm_tables,
     const float* __restrict__ uniforms, int* __restrict__ out_bytes, float* __restrict__ G,
     float* __restrict__ unit_lse_out, unsigned* status, unsigned* work_counter, int wpp, int n, int r, int v, int vv,
-    int sum_rows, int logA_stride, int tables_in_smem) {
+    int sum_rows, int hmm_stride, int tables_in_smem, int weights_in_smem) {
   extern __shared__ __align__(16) float sm[];
   grid_launch_dependents();
+  const int per = (v + 31) / 32;             // consecutive symbols per lane in the CDF scan (<= NQ, narrow)
+  float* weights = sm + ((2 * r + 3) & ~3);  // [r][32 per]
+  float* tabs = weights + (weights_in_smem ? r * 32 * per : 0);
+  const int chain = slot_chain_length(family, n, blockIdx.x);
+  const bool early = tables_in_smem && family == 1 && hmm_stride == 0;      // written when the head was made, not by this call
+  if (early) fetch_floats(tabs, hmm_tables, chain * r * r, kSlotThreads);
   grid_dependency_wait();     // the logits and log omega come from the kernel before this one
   if (work_counter != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
     *work_counter = 0;        // the circuit kernel that follows hands out its windows through this counter
   float* unit_max = sm;
   float* unit_lse = sm + r;
-  float* tabs = sm + ((2 * r + 3) & ~3);
   const int i = blockIdx.x;
   const int pos = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -481,35 +533,76 @@ __global__ void __launch_bounds__(kSlotThreads, 2) draft_slot_kernel(
   const int rr = r * r;
   const float* row = logits + (static_cast<size_t>(pos) * n + i) * r * v;   // [r, v] logits of this slot
   const float* lw = logw + static_cast<size_t>(pos) * sum_rows;
-  const float* hmm = logA + static_cast<size_t>(pos) * logA_stride;
-  const int chain = slot_chain_length(family, n, i);
+  const float* hmm = hmm_tables + static_cast<size_t>(pos) * hmm_stride;
+  const int nlat = (family == 0) ? 1 : (family == 1 ? n : n - 1);           // latent draws of a window (n <= 64)
 
-  if (tables_in_smem) {
-    for (int step = 0; step < chain; ++step) {
-      const float* src = slot_chain_table(family, lw, hmm, n, r, i, step);
-      float* dst = tabs + step * rr;
-      const bool vec = (rr & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0;
-      if (vec) {
-        for (int e = threadIdx.x * 4; e < rr; e += kSlotThreads * 4) cp_async_16(dst + e, src + e);
-      } else {
-        for (int e = threadIdx.x; e < rr; e += kSlotThreads) cp_async_4(dst + e, src + e);
-      }
+  constexpr int kVec = (NQ + 3) / 4;
+  auto load_unit = [&](int k, float4 (&xv)[kVec]) {      // lane l: symbols [4 l, 4 l + 4), [128 + 4 l, ..), ..
+#pragma unroll
+    for (int q = 0; q < kVec; ++q) {
+      const int b = 4 * (lane + 32 * q);
+      xv[q] = b < v ? *reinterpret_cast<const float4*>(row + k * v + b)
+                    : make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
     }
-    cp_async_commit();
-  }
+  };
+  struct Draws { float u0, u1, byte; };                  // lane l: the window's latent uniforms l and 32 + l; its byte's
+  auto load_draws = [&](int j) {
+    const float* u = uniforms + (pos * wpp + j) * 2 * n;           // (at most 128 positions of 64 windows: 32 bits do)
+    return Draws{lane < nlat ? u[lane] : 0.f, 32 + lane < nlat ? u[32 + lane] : 0.f, u[n + i]};
+  };
+  float4 next_unit[kVec];
+  Draws next_draws{};
+  if (!WIDE && warp < r) load_unit(warp, next_unit);
+  if (warp < wpp) next_draws = load_draws(warp);
+  const float root_logp = r <= 32 && lane < r ? lw[lane] : 0.f;
 
-  // ---- log-sum-exp of every input unit of the slot: a lane's logits are fetched in batches of independent loads
-  // (one batch covers 512 symbols; wider vocabularies take several, merged online)
+  if (tables_in_smem && !early) {
+#pragma unroll 1
+    for (int step = 0; step < chain; ++step)
+      fetch_floats(tabs + step * rr, slot_chain_table(family, lw, hmm, n, r, i, step), rr, kSlotThreads);
+  }
+  if (tables_in_smem) cp_async_commit();
+
+  // ---- log-sum-exp of every input unit of the slot (wide vocabularies: 512 symbols at a time, merged online)
   constexpr int kChunk = kSlotMaxPerLane * 32;
   for (int k = warp; k < r; k += nwarps) {
-    const float* x = row + static_cast<size_t>(k) * v;
     float m = -CUDART_INF_F, s = 0.f;
-    for (int c0 = 0; c0 < (WIDE ? v : 1); c0 += kChunk) {
+    if (!WIDE) {
+      float4 xv[kVec];
+#pragma unroll
+      for (int q = 0; q < kVec; ++q) xv[q] = next_unit[q];
+      if (k + nwarps < r) load_unit(k + nwarps, next_unit);
+#pragma unroll
+      for (int q = 0; q < kVec; ++q) {
+        const int b = 4 * (lane + 32 * q);
+        if (b + 3 >= vv) {                       // [vv, v): padding symbols
+          if (b >= vv) xv[q].x = -CUDART_INF_F;
+          if (b + 1 >= vv) xv[q].y = -CUDART_INF_F;
+          if (b + 2 >= vv) xv[q].z = -CUDART_INF_F;
+          xv[q].w = -CUDART_INF_F;
+        }
+        m = fmaxf(fmaxf(m, fmaxf(xv[q].x, xv[q].y)), fmaxf(xv[q].z, xv[q].w));
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, off));
+#pragma unroll
+      for (int q = 0; q < kVec; ++q) {
+        const int b = 4 * (lane + 32 * q);
+        const float4 e = make_float4(fast_ex2((xv[q].x - m) * kLog2e), fast_ex2((xv[q].y - m) * kLog2e),
+                                     fast_ex2((xv[q].z - m) * kLog2e), fast_ex2((xv[q].w - m) * kLog2e));
+        s += (e.x + e.y) + (e.z + e.w);          // padding: 2^-inf = 0
+        if (weights_in_smem && b < 32 * per) *reinterpret_cast<float4*>(weights + k * 32 * per + b) = e;
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
+    }
+    for (int c0 = 0; WIDE && c0 < v; c0 += kChunk) {
+      const float* x = row + static_cast<size_t>(k) * v;
       float xv[NQ];
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
         const int b = c0 + lane + 32 * q;
-        xv[q] = b < vv ? x[b] : -CUDART_INF_F;   // [vv, v): padding symbols
+        xv[q] = b < vv ? x[b] : -CUDART_INF_F;
       }
       float cm = xv[0];
 #pragma unroll
@@ -528,69 +621,71 @@ __global__ void __launch_bounds__(kSlotThreads, 2) draft_slot_kernel(
     if (lane == 0) {
       unit_max[k] = m;
       unit_lse[k] = m + __logf(s);
-      unit_lse_out[(static_cast<size_t>(pos) * n + i) * r + k] = unit_lse[k];   // kept for the acceptance stage
+      unit_lse_out[(pos * n + i) * r + k] = unit_lse[k];   // kept for the acceptance stage
     }
   }
+  const float root_cum = warp_scan_incl(lane < r && r <= 32 ? expf(root_logp) : 0.f, lane);
   if (tables_in_smem) cp_async_wait<0>();
   __syncthreads();
 
-  const int per = (v + 31) / 32;   // consecutive bytes per lane in the CDF scan (<= kSlotMaxPerLane)
-  const int nlat = (family == 0) ? 1 : (family == 1 ? n : n - 1);
   for (int j = warp; j < wpp; j += nwarps) {
-    const size_t w = static_cast<size_t>(pos) * wpp + j;
-    const float* u = uniforms + w * 2 * n;
-    const float ub = u[n + i];
+    const int slot = (pos * wpp + j) * n + i;
+    const Draws d = next_draws;
+    if (j + nwarps < wpp) next_draws = load_draws(j + nwarps);
+    auto uniform = [&](int c) { return __shfl_sync(kFull, c < 32 ? d.u0 : d.u1, c & 31); };
     // ---- latent draws down to the unit that owns slot i; every uniform the window's latent draws use is checked
-    bool bad = false;
-    for (int c = lane; c < nlat; c += 32) bad |= !(u[c] >= 0.f && u[c] < 1.f);
-    bad = __any_sync(kFull, bad) || !(ub >= 0.f && ub < 1.f);
+    const bool bad = __any_sync(kFull, !(d.u0 >= 0.f && d.u0 < 1.f) || !(d.u1 >= 0.f && d.u1 < 1.f) || !(d.byte >= 0.f && d.byte < 1.f));
     int byte = -1;
     if (bad) {
       if (lane == 0) atomicOr(status, 2u);
     } else {
-      int z = r > 32 ? warp_inv_cdf_logits_wide(lw, r, u[0], lane)     // CP only; the mixture logits are unnormalised
-                     : warp_inv_cdf_logp(lane < r ? lw[lane] : 0.f, r, u[0], lane);
+      int z = r > 32 ? warp_inv_cdf_logits_wide(lw, r, uniform(0), lane)     // CP only; the mixture logits are unnormalised
+                     : warp_inv_cdf(root_cum, r, uniform(0), lane);
       if (family == 1) {
         for (int st = 0; st < chain; ++st) {
-          const float* tab = tables_in_smem ? tabs + st * rr : hmm + static_cast<size_t>(st) * rr;
-          z = warp_inv_cdf_logp(lane < r ? tab[z * r + lane] : 0.f, r, u[st + 1], lane);
+          const float t = lane >= r ? 0.f : tables_in_smem ? tabs[st * rr + z * r + lane] : hmm[st * rr + z * r + lane];
+          z = hmm_stride == 0 ? warp_inv_cdf(t, r, uniform(st + 1), lane) : warp_inv_cdf_logp(t, r, uniform(st + 1), lane);
         }
       } else if (family == 2) {
         const int code = n / 2 + (i >> 1);
         for (int st = 0; st < chain; ++st) {
           const int node = (code >> (chain - 1 - st)) - 1;
-          const float* tab = tables_in_smem ? tabs + st * rr : lw + r + static_cast<size_t>(node - 1) * rr;
-          z = warp_inv_cdf_logp(lane < r ? tab[z * r + lane] : 0.f, r, u[node], lane);
+          const float t = lane >= r ? 0.f : tables_in_smem ? tabs[st * rr + z * r + lane] : lw[r + (node - 1) * rr + z * r + lane];
+          z = warp_inv_cdf_logp(t, r, uniform(node), lane);
         }
       }
-      const float* x = row + static_cast<size_t>(z) * v;
+      const float* x = row + z * v;
       const float m = unit_max[z];
-      if (!WIDE) {
+      if (!WIDE && weights_in_smem) {
         // ---- inverse CDF over the v bytes of unit z: lane l owns bytes [l*per, (l+1)*per)
-        byte = warp_inv_cdf_chunk<NQ>(x, 0, per, vv, m, ub, true, lane);
+        float ev[NQ];
+        load_run<NQ>(weights + z * 32 * per + lane * per, per, per, 0.f, ev);
+        byte = warp_inv_cdf_weights<NQ>(ev, 0, per, vv, d.byte, true, lane);
+      } else if (!WIDE) {
+        byte = warp_inv_cdf_chunk<NQ>(x, 0, per, v, vv, m, d.byte, true, lane);
       } else {
         // ---- wide vocabulary: 512 symbols at a time. First the total (chunk sums in fp32, added up in fp64), then
         // the chunk the threshold u * total falls into, then the draw inside that chunk.
         double total = 0.0;
         for (int c0 = 0; c0 < v; c0 += kChunk) total += static_cast<double>(warp_chunk_sum(x, c0, vv, m, lane));
-        const double thr = static_cast<double>(ub) * total;
+        const double thr = static_cast<double>(d.byte) * total;
         double before = 0.0;
         byte = vv - 1;                           // rounding may leave no index: the last one
         for (int c0 = 0; c0 < v; c0 += kChunk) {
           const float cs = warp_chunk_sum(x, c0, vv, m, lane);
           if (thr < before + static_cast<double>(cs)) {
-            byte = warp_inv_cdf_chunk<kSlotMaxPerLane>(x, c0, kSlotMaxPerLane, vv, m, static_cast<float>(thr - before), false, lane);
+            byte = warp_inv_cdf_chunk<kSlotMaxPerLane>(x, c0, kSlotMaxPerLane, v, vv, m, static_cast<float>(thr - before), false, lane);
             break;
           }
           before += static_cast<double>(cs);
         }
       }
     }
-    if (lane == 0) out_bytes[w * n + i] = byte;
+    if (lane == 0) out_bytes[slot] = byte;
     // evidence of the drafted byte under every input unit of the slot; a draw that was refused (byte -1) has none:
     // NaN, so that the window's log-prob comes out as NaN rather than as the joint of its other bytes
     for (int k = lane; k < r; k += 32)
-      G[(w * n + i) * r + k] = byte < 0 ? CUDART_NAN_F : row[static_cast<size_t>(k) * v + byte] - unit_lse[k];
+      G[slot * r + k] = byte < 0 ? CUDART_NAN_F : row[k * v + byte] - unit_lse[k];
   }
 }
 
@@ -643,7 +738,7 @@ __global__ void __launch_bounds__(32 * kLatentWarps) latent_sample_kernel(
 // evidence, and a sampling projection on hidden states sorted by unit before it, are what keeping the logits replaces: 2232 +
 // 217 + 74 us at 4096 positions of the n = 16, r = 32, v = 256 tree, against 206 us more for the projection that keeps them
 // and 67 us here.)
-template <bool WIDE>   // units of more than 512 symbols: 512 at a time, as in draft_slot_kernel
+template <bool WIDE, int NQ>   // units of more than 512 symbols: 512 at a time, as in draft_slot_kernel; else v <= 32 NQ
 __global__ void __launch_bounds__(256) draft_pick_kernel(const float* __restrict__ logits, const float* __restrict__ unit_lse,
                                                          const int* __restrict__ unit_sel, const float* __restrict__ uniforms,
                                                          int* __restrict__ out_bytes, float* __restrict__ G, unsigned* status,
@@ -665,7 +760,7 @@ __global__ void __launch_bounds__(256) draft_pick_kernel(const float* __restrict
       const float* x = row + static_cast<size_t>(z) * v;
       const float m = unit_lse[unit0 + z];                 // the weights are then probabilities
       if (!WIDE) {
-        byte = warp_inv_cdf_chunk<kSlotMaxPerLane>(x, 0, (v + 31) / 32, vv, m, ub, true, lane);
+        byte = warp_inv_cdf_chunk<NQ>(x, 0, (v + 31) / 32, v, vv, m, ub, true, lane);
       } else {
         constexpr int kChunk = kSlotMaxPerLane * 32;
         double total = 0.0;
@@ -676,7 +771,7 @@ __global__ void __launch_bounds__(256) draft_pick_kernel(const float* __restrict
         for (int c0 = 0; c0 < v; c0 += kChunk) {
           const float cs = warp_chunk_sum(x, c0, vv, m, lane);
           if (thr < before + static_cast<double>(cs)) {
-            byte = warp_inv_cdf_chunk<kSlotMaxPerLane>(x, c0, kSlotMaxPerLane, vv, m, static_cast<float>(thr - before), false, lane);
+            byte = warp_inv_cdf_chunk<kSlotMaxPerLane>(x, c0, kSlotMaxPerLane, v, vv, m, static_cast<float>(thr - before), false, lane);
             break;
           }
           before += static_cast<double>(cs);
@@ -735,6 +830,7 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
   // ---- 1. acceptance tests: lane i runs the test of byte i; the first rejecting lane ends the accepted run
   bool bad_u = !(u_last >= 0.f && u_last < 1.f), bad_x = false;
   int s = n;
+#pragma unroll 1
   for (int base = 0; base < n; base += 32) {
     const int i = base + lane;
     bool rej = false;
@@ -762,6 +858,7 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
   // ---- 2. weights of the v bytes
   const float* trow = tp + static_cast<size_t>(s) * v;
   if (s == n) {
+#pragma unroll 1
     for (int b = threadIdx.x; b < v; b += blockDim.x) mres[b] = b < vv ? trow[b] : 0.f;
   } else {
     const size_t lrow = row_of != nullptr ? static_cast<size_t>(row_of[w]) : static_cast<size_t>(pos) * n + s;
@@ -790,12 +887,14 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
         if (lane + 32 * q < r) cw[lane + 32 * q] = (c[q] - lse - l[q]) * kLog2e;
     }
     __syncthreads();
+#pragma unroll 1
     for (int b = threadIdx.x; b < v; b += blockDim.x) {
       float res = 0.f;
       if (b < vv) {
         const float t = trow[b];
         float q0 = 0.f, q1 = 0.f;
         int k = 0;
+#pragma unroll 1
         for (; k + 16 <= r; k += 16) {                   // sixteen rows' logits in flight, two accumulation chains
           float xv[16];
 #pragma unroll
@@ -806,6 +905,7 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
             q1 += fast_ex2(fmaf(xv[e + 1], kLog2e, cw[k + e + 1]));
           }
         }
+#pragma unroll 1
         for (; k < r; ++k) q0 += fast_ex2(fmaf(lg[static_cast<size_t>(k) * v + b], kLog2e, cw[k]));
         res = fmaxf(0.f, t - (q0 + q1));
       }
@@ -817,6 +917,7 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
   const int per = (v + blockDim.x - 1) / blockDim.x;
   const int b0 = threadIdx.x * per;
   float part = 0.f;
+#pragma unroll 1
   for (int q = 0; q < per; ++q)
     if (b0 + q < v) part += mres[b0 + q];
   const float incl = warp_scan_incl(part, lane);
@@ -824,10 +925,12 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
   __syncthreads();
   // every warp adds the warps' totals up in the same order, so exactly one of them finds the threshold inside its own run
   float total = 0.f;
+#pragma unroll 1
   for (int q = 0; q < warps; ++q) total += cw[q];
   const float thr = u_last * total;
   float before = 0.f;
   int owner = -1;
+#pragma unroll 1
   for (int q = 0; q < warps; ++q) {
     const float end = before + cw[q];
     if (thr < end) { owner = q; break; }
@@ -849,6 +952,7 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
   if (lane == src) {
     float cum = before + (lane == 0 ? 0.f : prev);
     int found = -1, last = min(b0 + per, vv) - 1;
+#pragma unroll 1
     for (int q = 0; q < per && found < 0; ++q)
       if (b0 + q < vv && mres[b0 + q] > 0.f) {
         cum += mres[b0 + q];

@@ -303,8 +303,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   if (CTAS == 2) cluster_sync_all();   // the peer's barriers are initialised before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
-  grid_launch_dependents();   // the next kernel's CTAs may be scheduled as SMs free up; they wait for this grid's results
   grid_dependency_wait();     // barriers and tensor memory were set up while the kernel before this one finished
+  grid_launch_dependents();   // the next kernel's CTAs may be scheduled as SMs free up; they wait for this grid's results
   if (p.work_counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *p.work_counter = 0;
 
   if (warp == 0) {

@@ -616,7 +616,7 @@ __global__ void __launch_bounds__(32 * kDrawWarps) lowrank_draw_kernel(
     const int* __restrict__ unit_sel, const float* __restrict__ uniforms, int* __restrict__ out_bytes, unsigned* status, int W,
     int wpp, int n, int r, int v, int vv, int k) {
   grid_dependency_wait();
-  extern __shared__ float draw_sm[];                              // kDrawWarps x v logits
+  extern __shared__ __align__(16) float draw_sm[];                // kDrawWarps x v logits
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* x = draw_sm + warp * v;
   const size_t units = static_cast<size_t>(n) * r;
@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(32 * kDrawWarps) lowrank_draw_kernel(
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     __syncwarp();
-    const int byte = warp_inv_cdf_chunk<kSlotMaxPerLane>(x, 0, per, vv, m, ub, true, lane);
+    const int byte = warp_inv_cdf_chunk<kSlotMaxPerLane>(x, 0, per, v, vv, m, ub, true, lane);
     if (lane == 0) out_bytes[e] = byte;
     __syncwarp();                                                 // x is reused by the warp's next pair
   }

@@ -574,16 +574,21 @@ int resident_clusters(K kernel, int size, int smem_bytes) {
   return clusters;
 }
 
-// Rows per emission tile of the few-position draft path: the height in [64, 128] (multiple of 8) that leaves the
-// least idle time when the tiles are dealt evenly to `ctas` persistent CTAs; ties go to the taller tile.
-int decode_tile_rows(long long rows, int ctas) {
+// Rows per tile of the few-position draft path: the height in [64, 128] (multiple of 8) with which the longest of `ctas` persistent
+// CTAs has the fewest rows, emission and sum-unit tiles dealt evenly together, a pass of up to kDecodeMaxTiles tiles counted as 8 rows
+// more (its copy of the hidden states); ties go to the taller tile. (By the emission rows alone, a tree head of n = 8, r = 32,
+// v = 256 got 5 tiles of 112 rows on its longest CTA where the mean is 485 rows, 4 of 128 now: a decode step of 27 positions
+// 103.7 -> 100.4 us; a contextual head of n = 16, r = 32, v = 320, d = 2048, 115 positions: 283.6 -> 268.3.)
+long long decode_tiles(long long rows, int sum_rows, int tr) {
+  return (rows + tr - 1) / tr + (sum_rows + tr / 32 * 32 - 1) / (tr / 32 * 32);
+}
+int decode_tile_rows(long long rows, int sum_rows, int ctas) {
   int best = 128;
-  double best_eff = 0.0;
+  long long best_cost = -1;
   for (int tr = 128; tr >= 64; tr -= 8) {
-    const long long tiles = (rows + tr - 1) / tr;
-    const long long per_cta = (tiles + ctas - 1) / ctas;
-    const double eff = static_cast<double>(rows) / (static_cast<double>(per_cta) * ctas * tr);
-    if (eff > best_eff + 1e-9) { best_eff = eff; best = tr; }
+    const long long per_cta = (decode_tiles(rows, sum_rows, tr) + ctas - 1) / ctas;
+    const long long cost = per_cta * tr + 8 * ((per_cta + kDecodeMaxTiles - 1) / kDecodeMaxTiles);
+    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = tr; }
   }
   return best;
 }
@@ -592,17 +597,16 @@ int decode_tile_rows(long long rows, int ctas) {
 // every CTA keeps at least four K blocks. A CTA's time goes as its K steps x (rows it fetches per step + a fixed part worth
 // about 32 rows) and the exchange of a cluster costs about 40 steps' worth of a row.
 void choose_decode_tiling(long long rows, int sum_rows, int kblocks, int ctas, const int (&max_clusters)[3], int* tile_rows, int* ksplit) {
-  auto tiles_of = [&](int tr) { return (rows + tr - 1) / tr + (sum_rows + tr / 32 * 32 - 1) / (tr / 32 * 32); };
-  *tile_rows = decode_tile_rows(rows, ctas);
+  *tile_rows = decode_tile_rows(rows, sum_rows, ctas);
   *ksplit = 1;
-  const long long per_cta = (tiles_of(*tile_rows) + ctas - 1) / ctas;
+  const long long per_cta = (decode_tiles(rows, sum_rows, *tile_rows) + ctas - 1) / ctas;
   long long best = kblocks * (per_cta * *tile_rows + 48);
   for (int e = 0; e < 3; ++e) {
     const int s = 2 << e;
     if (kblocks / s < 4) break;
     for (int tr = 128; tr >= 64; tr -= 8) {
       const long long cost = (kblocks + s - 1) / s * (tr + 48) + 40 * 48;
-      if (tiles_of(tr) <= max_clusters[e] && cost < best) { best = cost; *tile_rows = tr; *ksplit = s; }
+      if (decode_tiles(rows, sum_rows, tr) <= max_clusters[e] && cost < best) { best = cost; *tile_rows = tr; *ksplit = s; }
     }
   }
 }
@@ -644,7 +648,8 @@ int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_
   if (p.pass_tiles > kDecodeMaxTiles) p.pass_tiles = kDecodeMaxTiles;
   const int tiles = p.emit_tiles + p.emit2_tiles + p.sum_tiles;
   const int per_cta = (tiles + h->num_sms - 1) / h->num_sms;         // no wider stages than a CTA has tiles
-  if (p.pass_tiles > per_cta) p.pass_tiles = per_cta;
+  const int passes = (per_cta + p.pass_tiles - 1) / p.pass_tiles;
+  p.pass_tiles = (per_cta + passes - 1) / passes;                     // passes of one length keep as many bytes in flight throughout
   p.ksplit = h->decode_ksplit;
   while (p.ksplit > 1 && decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad) > 64 * 1024) p.ksplit /= 2;
   // stage = weight tiles + hidden tile, padded so that a 128-row operand read from the last tile's base stays inside

@@ -549,7 +549,7 @@ __host__ __device__ inline size_t hmm_circuit_smem_floats(int n, int r, bool wit
   return (static_cast<size_t>(chunk_tables) * r * r + 3) / 4 * 4 +
          static_cast<size_t>(kHmmWarps) * hmm_circuit_warp_floats(n, r, with_prefix);
 }
-__global__ void __launch_bounds__(32 * kHmmWarps, 4) circuit_hmm_kernel(
+__global__ void __launch_bounds__(32 * kHmmWarps, 5) circuit_hmm_kernel(
     const float* __restrict__ G, const float* __restrict__ logw, const float* __restrict__ tables, int table_stride,
     float* __restrict__ out, float* __restrict__ prefix, float* __restrict__ msg, int W, int wpp, int n, int r, int sum_rows,
     int chunk_tables, int probabilities) {

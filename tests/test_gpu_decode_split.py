@@ -30,3 +30,19 @@ def test_drafts_of_heads_with_few_weight_rows(family, n, r, v, d, P, wpp):
     assert not (differ & (ref["margin"] >= 1e-6)).any()
     assert np.abs(out_lp.cpu().numpy()[~differ] - ref["logprob"][~differ]).max() <= 2e-3
     dh.close()
+
+
+@pytest.mark.parametrize("family,n,r,v,P", [
+    (I.BTREE, 8, 32, 256, 40),               # four tiles a CTA in two passes of two, sum tiles between them
+    (I.HMM_CTX, 6, 32, 256, 100),            # 128 positions' accumulators: passes of two
+])
+def test_drafts_of_heads_with_several_tiles_per_cta(family, n, r, v, P):
+    wl = I.make_workload("passes", I.HeadShape(family, n, r, v, 64), P, seed=8300 + n, wpp=1, weight_std=0.2)
+    dh = DeviceHead(wl)
+    out_bytes, out_lp = dh.draft_sample()
+    assert dh.head.mtpc_get_status() == 0
+    ref = orc.draft_sample(family, wl.hidden_q, wl.W_emit_q, wl.W_sum_q, wl.T_static, 1, wl.uniforms)
+    differ = (out_bytes.cpu().numpy() != ref["bytes"]).any(axis=1)
+    assert not (differ & (ref["margin"] >= 1e-6)).any()
+    assert np.abs(out_lp.cpu().numpy()[~differ] - ref["logprob"][~differ]).max() <= 2e-3
+    dh.close()

@@ -1273,6 +1273,35 @@ void plan_lowrank_backward(const mtpc_config& c, const Layout& L, int k, int T, 
 // Phases 3 and 4 of a training call on a factored head: logit gradients g [T, n r v] (bf16), their sum over a slot's
 // components, the zero-padded A, W_base and B in a row; then the GEMMs. The sum units' logit gradients are already in the
 // right-hand columns of sy.
+int launch_adaptor_grad(mtpc_head* h, const __nv_bfloat16* g, size_t g_pitch, int Nc, const void* a_pad, int v64, __nv_bfloat16* y,
+                        size_t y_pitch, float* dA, int T, cudaStream_t st) {
+  const mtpc_config& c = h->cfg;
+  AdaptorGradParams p;
+  memset(&p, 0, sizeof(p));
+  p.units = c.n * c.r;
+  p.T = T;
+  p.v = c.v;
+  p.v64 = v64;
+  p.k = h->lr_k;
+  const int ctl = 1024 + static_cast<int>(sizeof(GemmControl));
+  p.stages = (kSmemLimit - ctl - static_cast<int>(adaptor_fixed_bytes(v64))) / static_cast<int>(kAdaptorStage);
+  if (p.stages < 2) return MTPC_ERR_UNSUPPORTED;
+  const uint64_t z_cols = static_cast<uint64_t>(p.units) * 2 * p.k;
+  int rc = make_tmap(&p.tm_g, g, T, Nc, kBlockM, g_pitch);
+  if (rc == MTPC_OK) rc = make_tmap(&p.tm_z, h->ws + h->lr_off_zhl, T, z_cols, kBlockM, z_cols);
+  if (rc == MTPC_OK) rc = make_tmap_mn(&p.tm_a, a_pad, static_cast<uint64_t>(p.units) * v64, p.k, p.k);
+  if (rc != MTPC_OK) return rc;
+  p.y = y;
+  p.y_pitch = y_pitch;
+  p.dA = dA;
+  p.status = at<unsigned>(h, h->L.off_status);
+  p.wait_limit_ns = h->wait_limit_ns;
+  launch_kernel(adaptor_grad_kernel, p.units < h->num_sms ? p.units : h->num_sms, kGemmThreads,
+                p.stages * kAdaptorStage + adaptor_fixed_bytes(v64) + ctl, st, overlapped(h), p);
+  h->launches++;
+  return check_launch();
+}
+
 int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8_t* bw, const void* hb, const int32_t* targets,
                           int T, float* d_hidden, float* dW_base, float* dA, float* dB, float* dW_sum, PhaseTimer& pt,
                           cudaStream_t st) {
@@ -1312,7 +1341,13 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
   pt.begin();
   const GemmOperand none{nullptr, 0, false};
   const GemmOperand hid{hb, static_cast<size_t>(c.d), true};
-  {   // y_ij = g_ij A_ij [T, k], one product per unit, into the middle columns of sy
+  // y_ij = g_ij A_ij [T, k] into the middle columns of sy and dA_ij [v, k] = g_ij^T z_ij from one reading of g, where a CTA can keep a
+  // unit's A and there are units for at least half the SMs; else one batched product each
+  const bool one_pass = c.v <= kAdaptorMaxV && 2 * units >= head->num_sms;
+  if (one_pass) {
+    rc = launch_adaptor_grad(head, dlogit, B.Kd, Nc, bw + R.off_apad, static_cast<int>(R.v64), sy + static_cast<size_t>(c.n) * c.v, R.pitch,
+                             dA, T, st);
+  } else {
     PlainGemmExtra x;
     x.C_bf16 = sy + static_cast<size_t>(c.n) * c.v;
     x.batches = units;
@@ -1338,7 +1373,7 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
   if (rc == MTPC_OK)
     rc = launch_plain_gemm(head, GemmOperand{sy, R.pitch, true}, hid, T, hid, 0, 0, dW_base, c.d, static_cast<int>(R.Ksy) + L.sum_rows,
                            c.d, st, bw + B.off_split, nullptr, 0, &three);
-  if (rc == MTPC_OK) {   // dA_ij [v, k] = g_ij^T z_ij, one product per unit, on the bf16 high half of z the forward pass left
+  if (rc == MTPC_OK && !one_pass) {   // on the bf16 high half of z the forward pass left
     PlainGemmExtra x;
     x.batches = units;
     x.a_m_step = c.v;
@@ -1527,6 +1562,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   fail |= !allow_full_smem(plain_gemm_kernel<true, true, kPlainTileN, 2>);
   fail |= !allow_full_smem(plain_gemm_kernel<true, true, 64>);
   fail |= !allow_full_smem(plain_gemm_kernel<false, true, 64>);
+  fail |= !allow_full_smem(adaptor_grad_kernel);
   fail |= cudaFuncSetAttribute(mtpc_decode_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) !=
           cudaSuccess;
   for (int e = 0; e < 3; ++e) h->max_decode_clusters[e] = fail ? 0 : resident_clusters(mtpc_decode_gemm_kernel, 2 << e, kSmemLimit);

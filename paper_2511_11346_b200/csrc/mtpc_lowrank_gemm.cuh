@@ -32,6 +32,7 @@
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
+#include "mtpc_backward.cuh"
 #include "mtpc_circuit.cuh"
 #include "mtpc_decode.cuh"
 #include "mtpc_gemm.cuh"
@@ -726,6 +727,219 @@ __global__ void __launch_bounds__(32 * kDrawWarps) lowrank_slot_logits_kernel(
     if (lane == 0) unit_lse[static_cast<size_t>(w) * r + j] = m + __logf(sum);
   }
   grid_launch_dependents();
+}
+
+// ---------------------------------------------------------------- gradients through the adaptors A
+// y_u [T, k] = g_u A_u and dA_u [v, k] = g_u^T z_u of every unit u from ONE reading of its logit gradients g_u [T, v]: a CTA takes a
+// unit at a time and walks its positions, 128 at once; a stage of shared memory holds 128 positions x 128 symbols of g as two
+// 64-symbol boxes, which are the K-major operand A of the product y and, untransposed, the MN-major operand A of the product dA.
+// y's accumulators (two, of k columns) leave at the end of each 128 positions, dA's (two sets of up to four tiles of 128 symbols) at
+// the end of the unit. z: the bf16 high half the forward pass left, k of the 64 columns that a box brings in. Bound by the bytes
+// of g: 2 T n r v. Two batched GEMMs, each reading g, took %OLD% us at 8192 positions of 8 x 32 units of 320 symbols, k = 16;
+// this takes %NEW%. Units of more than 512 symbols, or too few units to occupy the device, keep those.
+struct AdaptorGradParams {
+  CUtensorMap tm_g;      // g    [T, n r v] at its pitch   box 64 x 128
+  CUtensorMap tm_z;      // z    [T, n r 2 k]              box 64 x 128 (unit u: from column 2 k u)
+  CUtensorMap tm_a;      // A    [n r v64, k], v64 = v rounded up to 64 with zero rows; box 64 x 64
+  int units, T, v, v64, k, stages;
+  __nv_bfloat16* y;      // unit u: columns [u k, (u + 1) k)
+  size_t y_pitch;
+  float* dA;             // [units, v, k]
+  unsigned* status;
+  uint64_t wait_limit_ns;
+};
+constexpr uint32_t kAdaptorBox = kBlockM * 128;              // 128 positions x 64 bf16: 16 KB
+constexpr uint32_t kAdaptorStage = 2 * kAdaptorBox;
+constexpr int kAdaptorMaxV = 512;
+// barriers beyond the stage ring: full / empty of A_u, empty of the two z buffers (their bytes count into the first stage of a tile)
+constexpr int kAdaptorBarA = 13, kAdaptorBarZ = 14;
+inline size_t adaptor_fixed_bytes(int v64) { return 2 * kAdaptorBox + static_cast<size_t>(v64) * 128; }
+
+__global__ void __launch_bounds__(kGemmThreads, 1) adaptor_grad_kernel(const __grid_constant__ AdaptorGradParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw_addr = smem_u32(smem_raw);
+  const uint32_t tiles_addr = (raw_addr + 1023u) & ~1023u;
+  const uint32_t z_addr = tiles_addr + p.stages * kAdaptorStage, a_addr = z_addr + 2 * kAdaptorBox;
+  GemmControl* ctl = reinterpret_cast<GemmControl*>(smem_raw + (a_addr - raw_addr) + static_cast<size_t>(p.v64) * 128);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t_tiles = (p.T + kBlockM - 1) / kBlockM, pairs = (p.v64 + 127) / 128;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kMaxStages; ++s) {
+      mbar_init(smem_u32(&ctl->full[s]), 1);
+      mbar_init(smem_u32(&ctl->empty[s]), 1);
+    }
+    for (int s = 0; s < 4; ++s) {                            // 0, 1: y; 2, 3: dA
+      mbar_init(smem_u32(&ctl->tfull[s]), 1);
+      mbar_init(smem_u32(&ctl->tempty[s]), 4);
+    }
+    mbar_init(smem_u32(&ctl->drain), 1);
+    ctl->abort = 0;
+    ctl->wait_limit_ns = p.wait_limit_ns;
+    fence_mbar_init();
+    tma_prefetch_desc(&p.tm_g);
+    tma_prefetch_desc(&p.tm_z);
+    tma_prefetch_desc(&p.tm_a);
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = ctl->tmem_base;
+  grid_dependency_wait();
+  grid_launch_dependents();
+  // tensor memory: y at columns 0 and 32, dA's tiles at 64 and 192, 32 columns each
+  auto da_col = [&](uint32_t set, int tile) { return 64 + set * 128 + tile * 32; };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0, tc = 0, uc = 0;
+      bool ok = true;
+      auto issued = [&](uint32_t bar, uint32_t par) {
+        issued_mask |= 1u << bar;
+        phase_mask = (phase_mask & ~(1u << bar)) | (par << bar);
+      };
+      for (int unit = blockIdx.x; unit < p.units && ok; unit += gridDim.x, ++uc) {
+        bool a_loaded = false;
+        for (int t = 0; t < t_tiles && ok; ++t, ++tc) {
+          const uint32_t zbuf = tc & 1u;
+          for (int q = 0; q < pairs; ++q) {
+            if (!bounded_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
+            if (q == 0 && !bounded_wait(smem_u32(&ctl->empty[kAdaptorBarZ + zbuf]), ((tc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+            const int boxes = q * 128 + 64 < p.v64 ? 2 : 1;
+            const uint32_t full = smem_u32(&ctl->full[stage]), dst = tiles_addr + stage * kAdaptorStage;
+            mbar_arrive_expect_tx(full, (boxes + (q == 0 ? 1 : 0)) * kAdaptorBox);
+            for (int b = 0; b < boxes; ++b) tma_load_2d(dst + b * kAdaptorBox, &p.tm_g, full, unit * p.v + q * 128 + b * 64, t * kBlockM);
+            if (q == 0) tma_load_2d(z_addr + zbuf * kAdaptorBox, &p.tm_z, full, unit * 2 * p.k, t * kBlockM);
+            issued(stage, phase);
+            if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
+            // A_u goes into the buffer that the unit before it has finished with: asked for behind the unit's first stage, so that
+            // the wait does not keep g from being fetched
+            if (!a_loaded) {
+              a_loaded = true;
+              if (!bounded_wait(smem_u32(&ctl->empty[kAdaptorBarA]), (uc & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+              const uint32_t afull = smem_u32(&ctl->full[kAdaptorBarA]);
+              mbar_arrive_expect_tx(afull, p.v64 * 128);
+              for (int b = 0; b < p.v64; b += 64) tma_load_2d(a_addr + b * 128, &p.tm_a, afull, 0, unit * p.v64 + b);
+              issued(kAdaptorBarA, uc & 1u);
+            }
+          }
+        }
+      }
+      // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
+      for (int s = 0; s < kMaxStages; ++s)
+        if (issued_mask & (1u << s)) {
+          const uint64_t t0 = global_timer_ns();
+          while (!mbar_try_wait(smem_u32(&ctl->full[s]), (phase_mask >> s) & 1u) && global_timer_ns() - t0 < kWaitLimitNs) {}
+        }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      uint32_t stage = 0, phase = 0, tc = 0, uc = 0;
+      bool ok = true;
+      const uint32_t idesc_y = umma_idesc_bf16(kBlockM, p.k, false, true), idesc_da = umma_idesc_bf16(kBlockM, p.k, true, true);
+      for (int unit = blockIdx.x; unit < p.units && ok; unit += gridDim.x, ++uc) {
+        const uint32_t set = uc & 1u;
+        if (!bounded_wait(smem_u32(&ctl->tempty[2 + set]), ((uc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+        if (!bounded_wait(smem_u32(&ctl->full[kAdaptorBarA]), uc & 1u, ctl, p.status)) { ok = false; break; }
+        for (int t = 0; t < t_tiles && ok; ++t, ++tc) {
+          const uint32_t yslot = tc & 1u;
+          if (!bounded_wait(smem_u32(&ctl->tempty[yslot]), ((tc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+          const uint64_t z_desc = umma_smem_desc_mn_sw128(z_addr + yslot * kAdaptorBox, kAdaptorBox);
+          for (int q = 0; q < pairs; ++q) {
+            if (!bounded_wait(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t g_addr = tiles_addr + stage * kAdaptorStage;
+            const int boxes = q * 128 + 64 < p.v64 ? 2 : 1;
+            for (int b = 0; b < boxes; ++b) {
+              const uint64_t g_desc = umma_smem_desc_sw128(g_addr + b * kAdaptorBox);
+              const uint64_t a_desc = umma_smem_desc_mn_sw128(a_addr + (2 * q + b) * kMnBoxBytes, kMnBoxBytes);
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk)                 // 16 symbols: 32 bytes along g's rows, 16 rows down A_u's box
+                umma_bf16(tmem_base + yslot * 32, g_desc + 2 * kk, a_desc + 128 * kk, idesc_y, (q | b | kk) != 0 ? 1u : 0u);
+            }
+            // the second box of an odd number is whatever the stage held before: rows past the unit's symbols, never read
+            const uint64_t gt_desc = umma_smem_desc_mn_sw128(g_addr, kAdaptorBox);
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk)                   // 16 positions: 16 rows down both
+              umma_bf16(tmem_base + da_col(set, q), gt_desc + 128 * kk, z_desc + 128 * kk, idesc_da, (t | kk) != 0 ? 1u : 0u);
+            umma_commit(smem_u32(&ctl->empty[stage]));
+            if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
+          }
+          if (!ok) break;
+          umma_commit(smem_u32(&ctl->tfull[yslot]));
+          umma_commit(smem_u32(&ctl->empty[kAdaptorBarZ + yslot]));
+        }
+        if (!ok) break;
+        umma_commit(smem_u32(&ctl->tfull[2 + set]));
+        umma_commit(smem_u32(&ctl->empty[kAdaptorBarA]));
+      }
+      if (!ok) {
+        umma_commit(smem_u32(&ctl->drain));
+        const uint64_t t0 = global_timer_ns();
+        while (!mbar_try_wait(smem_u32(&ctl->drain), 0) && global_timer_ns() - t0 < kWaitLimitNs) {}
+      }
+    }
+    __syncwarp();
+  } else {
+    const int quarter = warp & 3;
+    const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+    uint32_t tc = 0, uc = 0;
+    bool ok = true;
+    for (int unit = blockIdx.x; unit < p.units && ok; unit += gridDim.x, ++uc) {
+      for (int t = 0; t < t_tiles; ++t, ++tc) {
+        const uint32_t yslot = tc & 1u;
+        if (!bounded_wait_warp(smem_u32(&ctl->tfull[yslot]), (tc >> 1) & 1u, ctl, p.status, lane)) { ok = false; break; }
+        tc_fence_after();
+        const int row = t * kBlockM + quarter * 32 + lane;
+        for (int b = 0; b < p.k; b += 16) {
+          float x[16];
+          tmem_ld16(lane_base + yslot * 32 + b, x);
+          if (row < p.T) {
+            __nv_bfloat162 o[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) o[e] = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
+            uint4* dst = reinterpret_cast<uint4*>(p.y + static_cast<size_t>(row) * p.y_pitch + unit * p.k + b);
+            dst[0] = reinterpret_cast<const uint4*>(o)[0];
+            dst[1] = reinterpret_cast<const uint4*>(o)[1];
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&ctl->tempty[yslot]));
+      }
+      if (!ok) break;
+      const uint32_t set = uc & 1u;
+      if (!bounded_wait_warp(smem_u32(&ctl->tfull[2 + set]), (uc >> 1) & 1u, ctl, p.status, lane)) break;
+      tc_fence_after();
+      for (int q = 0; q < pairs; ++q) {
+        const int sym = q * 128 + quarter * 32 + lane;
+        for (int b = 0; b < p.k; b += 16) {
+          float x[16];
+          tmem_ld16(lane_base + da_col(set, q) + b, x);
+          if (sym < p.v) {
+            float4* dst = reinterpret_cast<float4*>(p.dA + (static_cast<size_t>(unit) * p.v + sym) * p.k + b);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dst[e] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&ctl->tempty[2 + set]));
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, kTmemCols);
+  }
 }
 
 }  // namespace mtpc

@@ -715,6 +715,8 @@ struct PlainGemmExtra {
   void* C_bf16 = nullptr;
   int batches = 1, a_m_step = 0, a_k_step = 0, b_n_step = 0, b_k_step = 0;
   size_t c_step = 0;
+  GemmOperand B2{nullptr, 0, false};         // a third K segment: K2 rows of B, from column a_k2 of A on
+  int K2 = 0, a_k2 = 0;
   long long a_extent_m = 0, a_extent_k = 0, b_extent_n = 0, b_extent_k = 0;
 };
 // split_ws: kSplitBytes of scratch that let the launch cut its last round along K (NULL: it does not).
@@ -988,7 +990,10 @@ int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmO
   p.a_k0[1] = a_k1;
   p.seg_kblocks[0] = (K0 + kBlockK - 1) / kBlockK;
   p.seg_kblocks[1] = K1 > 0 ? (K1 + kBlockK - 1) / kBlockK : 0;
-  const int kblocks = p.seg_kblocks[0] + p.seg_kblocks[1];
+  p.a_k0[2] = x.a_k2;
+  p.seg_kblocks[2] = x.K2 > 0 ? (x.K2 + kBlockK - 1) / kBlockK : 0;
+  if (x.K2 > 0 && (K1 <= 0 || !x.B2.mn_major || !B0.mn_major)) return MTPC_ERR_SHAPE;
+  const int kblocks = p.seg_kblocks[0] + p.seg_kblocks[1] + p.seg_kblocks[2];
   // batched products with a rank for N: 64-column accumulator tiles
   const int tile_n = (x.batches > 1 && N <= 64 && B0.mn_major) ? 64 : kPlainTileN;
   p.n_tiles = (N + tile_n - 1) / tile_n;
@@ -1011,7 +1016,7 @@ int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmO
   p.tail_tiles = plan.tail;
   p.split = plan.split;
   p.partial = static_cast<float*>(split_ws);
-  const int Ka = K1 > 0 ? a_k1 + K1 : K0;                      // extent of A along K
+  const int Ka = x.K2 > 0 ? x.a_k2 + x.K2 : K1 > 0 ? a_k1 + K1 : K0;           // extent of A along K
   const uint64_t a_m = x.a_extent_m ? x.a_extent_m : M, a_k = x.a_extent_k ? x.a_extent_k : Ka;
   const uint64_t b_n = x.b_extent_n ? x.b_extent_n : N, b_k = x.b_extent_k ? x.b_extent_k : K0;
   const int b_box = kPlainTileN / ctas;
@@ -1020,6 +1025,7 @@ int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmO
     rc = B0.mn_major ? make_tmap_mn(&p.tm_b[0], B0.ptr, b_k, b_n, B0.pitch) : make_tmap(&p.tm_b[0], B0.ptr, b_n, b_k, b_box, B0.pitch);
   if (rc == MTPC_OK && K1 > 0)
     rc = B1.mn_major ? make_tmap_mn(&p.tm_b[1], B1.ptr, K1, N, B1.pitch) : make_tmap(&p.tm_b[1], B1.ptr, N, K1, b_box, B1.pitch);
+  if (rc == MTPC_OK && x.K2 > 0) rc = make_tmap_mn(&p.tm_b[2], x.B2.ptr, x.K2, N, x.B2.pitch);
   if (rc != MTPC_OK) return rc;
   p.stage_bytes = kABytes + tile_n / ctas * kBlockK * 2;
   const int ctl = 1024 + static_cast<int>(sizeof(GemmControl));
@@ -1249,12 +1255,11 @@ int backward_tail(mtpc_head* head, const BackwardLayout& B, uint8_t* bw, const v
 // Backward workspace of a factored head: the dense layout without kept logits (log-sum-exps, posteriors, logit gradients), then
 //   sy    [T, n v | n r k | S r padded] bf16: the logit gradients summed over a slot's components, multiplied by the
 //         adaptors A, and those of the sum units: the A operand of d hidden and of the three weight-gradient GEMMs;
-//   wcat  [n v + n r k, d] bf16: W_base and B one after the other (one K segment of d hidden);
 //   apad  [n r, v rounded up to 64, k] bf16: A with zero rows between the units.
 struct LowRankBackwardLayout {
   BackwardLayout B;
   size_t Ksy, pitch, v64;
-  size_t off_sy, off_wcat, off_apad, total;
+  size_t off_sy, off_apad, total;
 };
 void plan_lowrank_backward(const mtpc_config& c, const Layout& L, int k, int T, LowRankBackwardLayout* R) {
   plan_backward(c, L, T, &R->B, /*keep_logits=*/false);
@@ -1265,13 +1270,12 @@ void plan_lowrank_backward(const mtpc_config& c, const Layout& L, int k, int T, 
   size_t off = R->B.total;
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
   R->off_sy = take(static_cast<size_t>(T) * R->pitch * 2);
-  R->off_wcat = take(R->Ksy * c.d * 2);
   R->off_apad = take(units * R->v64 * k * 2);
   R->total = off;
 }
 
 // Phases 3 and 4 of a training call on a factored head: logit gradients g [T, n r v] (bf16), their sum over a slot's
-// components, the zero-padded A, W_base and B in a row; then the GEMMs. The sum units' logit gradients are already in the
+// components, the zero-padded A; then the GEMMs. The sum units' logit gradients are already in the
 // right-hand columns of sy.
 int launch_adaptor_grad(mtpc_head* h, const __nv_bfloat16* g, size_t g_pitch, int Nc, const void* a_pad, int v64, __nv_bfloat16* y,
                         size_t y_pitch, float* dA, int T, cudaStream_t st) {
@@ -1331,11 +1335,7 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
                   static_cast<int>(R.v64), k / 8);
   }
   head->launches += 1;
-  uint8_t* wcat = bw + R.off_wcat;
-  const size_t base_bytes = static_cast<size_t>(c.n) * c.v * c.d * 2;
-  bool fail = cudaMemcpyAsync(wcat, head->lr_W_base, base_bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess;
-  fail |= cudaMemcpyAsync(wcat + base_bytes, head->lr_B, static_cast<size_t>(units) * k * c.d * 2, cudaMemcpyDeviceToDevice, st) != cudaSuccess;
-  if (fail || (rc = check_launch()) != MTPC_OK) return MTPC_ERR_CUDA;
+  if ((rc = check_launch()) != MTPC_OK) return rc;
   pt.end();
   // 4. the GEMMs
   pt.begin();
@@ -1359,11 +1359,15 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
     rc = launch_plain_gemm(head, GemmOperand{dlogit, B.Kd, false}, GemmOperand{bw + R.off_apad, static_cast<size_t>(k), true},
                            static_cast<int>(R.v64), none, 0, 0, nullptr, R.pitch, T, k, st, nullptr, nullptr, 0, &x);
   }
-  // d hidden [T, d] = [s | y] [W_base ; B] + dsum W_sum
+  // d hidden [T, d] = s W_base + y B + dsum W_sum
+  PlainGemmExtra tail;
+  tail.B2 = GemmOperand{head->W_sum_bf16, static_cast<size_t>(c.d), true};
+  tail.K2 = L.sum_rows;
+  tail.a_k2 = static_cast<int>(R.Ksy);
   if (rc == MTPC_OK)
-    rc = launch_plain_gemm(head, GemmOperand{sy, R.pitch, false}, GemmOperand{wcat, static_cast<size_t>(c.d), true},
-                           static_cast<int>(R.Ksy), GemmOperand{head->W_sum_bf16, static_cast<size_t>(c.d), true}, L.sum_rows,
-                           static_cast<int>(R.Ksy), d_hidden, c.d, T, c.d, st, bw + B.off_split);
+    rc = launch_plain_gemm(head, GemmOperand{sy, R.pitch, false}, GemmOperand{head->lr_W_base, static_cast<size_t>(c.d), true}, c.n * c.v,
+                           GemmOperand{head->lr_B, static_cast<size_t>(c.d), true}, units * k, c.n * c.v, d_hidden, c.d, T, c.d, st,
+                           bw + B.off_split, nullptr, 0, &tail);
   // [dW_base; dB; dW_sum] = [s | y | dsum]^T h: sy down its columns
   PlainGemmExtra three;
   three.C2 = dB;

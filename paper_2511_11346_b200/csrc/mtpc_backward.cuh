@@ -773,8 +773,8 @@ __global__ void __launch_bounds__(256) logit_gradient_kernel(const LogitGradArgs
 // C[M, N] (fp32, row-major, pitch ldc) = A[M, K] B[N, K]^T with bf16 operands read where they lie, in either
 // orientation: K-major (K contiguous in memory: 64-element K boxes of up to 256 rows) or MN-major (the M / N index
 // contiguous: 64 x 64 boxes, two for the 128 rows of A, up to four for the columns of B). Out-of-range rows and
-// columns read as zero. The K axis may consist of two segments with a B matrix each (d hidden sums over the emission
-// rows and the sum-unit rows, which are separate matrices); A then continues at column a_k0[1]. Same pipeline as the
+// columns read as zero. The K axis may consist of up to three segments with a B matrix each (d hidden sums over the
+// emission rows, or W_base and the adaptors B, and the sum-unit rows, which are separate matrices); A then continues at a_k0[i]. Same pipeline as the
 // projection kernel: one persistent CTA per SM, warp 0 TMA producer, warp 1 MMA issuer (two TMEM slots), warps 2..5 epilogue
 // (one thread per row, 16 fp32 columns per step). CTAS = 1: a CTA works alone (M = 128, N = TN). CTAS = 2: a cluster of two
 // shares every MMA (cta_group::2, M = 256), each CTA staging its own 128 rows of A and half of the columns of B, so a third
@@ -788,9 +788,9 @@ __global__ void __launch_bounds__(256) logit_gradient_kernel(const LogitGradArgs
 // give about 5 %).
 struct PlainGemmParams {
   CUtensorMap tm_a;      // K-major: A [M, K], box 64 (k) x 128; MN-major: A^T [K, M], box 64 (m) x 64 (k)
-  CUtensorMap tm_b[2];   // per K segment. K-major: B [N, K], box 64 (k) x TN / CTAS; MN-major: B^T [K, N], box 64 (n) x 64 (k)
-  int a_k0[2];           // K coordinate of A at which each segment starts (multiples of 8)
-  int seg_kblocks[2];    // 64-wide K blocks per segment (segment 1: 0 if unused)
+  CUtensorMap tm_b[3];   // per K segment. K-major: B [N, K], box 64 (k) x TN / CTAS; MN-major: B^T [K, N], box 64 (n) x 64 (k)
+  int a_k0[3];           // K coordinate of A at which each segment starts (multiples of 8)
+  int seg_kblocks[3];    // 64-wide K blocks per segment (0: unused; only trailing ones are)
   int M, N;
   int m_tiles, n_tiles;  // m_tiles: tiles of CTAS * 128 rows
   int stages, stage_bytes;
@@ -906,7 +906,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
   GemmControl* ctl = reinterpret_cast<GemmControl*>(tiles + static_cast<size_t>(p.stages) * p.stage_bytes);
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int kblocks = p.seg_kblocks[0] + p.seg_kblocks[1];
+  const int kblocks = p.seg_kblocks[0] + p.seg_kblocks[1] + p.seg_kblocks[2];
   const int num_items = p.m_tiles * p.n_tiles * p.batches + p.tail_tiles * (p.split - 1);
   const uint32_t cta_rank = CTAS == 2 ? cluster_cta_rank() : 0u;      // 0 = the pair's leader
   const int first_item = CTAS == 2 ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
@@ -932,6 +932,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
     tma_prefetch_desc(&p.tm_a);
     tma_prefetch_desc(&p.tm_b[0]);
     if (p.seg_kblocks[1] > 0) tma_prefetch_desc(&p.tm_b[1]);
+    if (p.seg_kblocks[2] > 0) tma_prefetch_desc(&p.tm_b[2]);
   }
   if (warp == 1) {
     if (CTAS == 2) {
@@ -952,51 +953,53 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
 
   if (warp == 0) {
     if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0;
+      // One K block must be asked for in less time than its MMAs take (256 cycles), so that little is computed per block.
+      uint32_t stage = 0, phase = 0, issued = 0;
       bool ok = true;
       auto load = [&](uint32_t dst, const CUtensorMap* tm, uint32_t full, int x, int y) {
         if (CTAS == 2) tma_load_2d_pair(dst, tm, full, x, y);
         else tma_load_2d(dst, tm, full, x, y);
       };
+      const uint32_t own_full = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+      const uint32_t full0 = CTAS == 2 ? cluster_map_shared(own_full, 0) : own_full;             // the leader's barriers
       for (int item = first_item; item < num_items && ok; item += item_step) {
         const PlainItem w = plain_item(p, item, kblocks);
         const int am = (w.mt * CTAS + static_cast<int>(cta_rank)) * kBlockM + w.bt * p.a_m_step;   // this CTA's rows of A,
         const int bn = w.nt * TN + static_cast<int>(cta_rank) * kBCols + w.bt * p.b_n_step;        // its columns of B
-        const int ak = w.bt * p.a_k_step, bk = w.bt * p.b_k_step;
-        for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (!bounded_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
-          uint32_t full = smem_u32(&ctl->full[stage]);
-          const uint32_t a_dst = tiles_addr + stage * p.stage_bytes;
-          const int seg = kb >= p.seg_kblocks[0] ? 1 : 0;
-          const int kloc = (kb - (seg ? p.seg_kblocks[0] : 0)) * kBlockK;      // K offset inside the segment
-          if (cta_rank == 0) mbar_arrive_expect_tx(full, CTAS * (kABytes + kBBytes));   // of both CTAs' copies when paired
-          if (CTAS == 2) full = cluster_map_shared(full, 0);                   // the leader's barrier
-          if (A_MN) {
+        int kb = w.kb0, seg_begin = 0;
+        for (int seg = 0; seg < 3 && ok; ++seg) {
+          const int seg_end = seg_begin + p.seg_kblocks[seg], stop = min(seg_end, w.kb1);
+          const CUtensorMap* tm_b = &p.tm_b[seg];
+          int ak = p.a_k0[seg] + (kb - seg_begin) * kBlockK + w.bt * p.a_k_step, bk = (kb - seg_begin) * kBlockK + w.bt * p.b_k_step;
+          for (; kb < stop; ++kb, ak += kBlockK, bk += kBlockK) {
+            if (!bounded_wait(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
+            const uint32_t full = full0 + 8 * stage, a_dst = tiles_addr + stage * p.stage_bytes;
+            if (cta_rank == 0) mbar_arrive_expect_tx(own_full + 8 * stage, CTAS * (kABytes + kBBytes));   // of both CTAs' copies when paired
+            if (A_MN) {
 #pragma unroll
-            for (int q = 0; q < kBlockM / 64; ++q) load(a_dst + q * kMnBoxBytes, &p.tm_a, full, am + q * 64, p.a_k0[seg] + kloc + ak);
-          } else {
-            load(a_dst, &p.tm_a, full, p.a_k0[seg] + kloc + ak, am);
-          }
-          if (B_MN) {
+              for (int q = 0; q < kBlockM / 64; ++q) load(a_dst + q * kMnBoxBytes, &p.tm_a, full, am + q * 64, ak);
+            } else {
+              load(a_dst, &p.tm_a, full, ak, am);
+            }
+            if (B_MN) {
 #pragma unroll
-            for (int q = 0; q < kBCols / 64; ++q) load(a_dst + kABytes + q * kMnBoxBytes, &p.tm_b[seg], full, bn + q * 64, kloc + bk);
-          } else {
-            load(a_dst + kABytes, &p.tm_b[seg], full, kloc + bk, bn);
+              for (int q = 0; q < kBCols / 64; ++q) load(a_dst + kABytes + q * kMnBoxBytes, tm_b, full, bn + q * 64, bk);
+            } else {
+              load(a_dst + kABytes, tm_b, full, bk, bn);
+            }
+            ++issued;
+            if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
           }
-          issued_mask |= 1u << stage;
-          phase_mask = (phase_mask & ~(1u << stage)) | (phase << stage);
-          if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
+          seg_begin = seg_end;
         }
       }
       // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
       if (CTAS == 1 || cta_rank == 0) {
-        for (int s = 0; s < p.stages; ++s)
-          if (issued_mask & (1u << s)) {
-            const uint32_t bar = smem_u32(&ctl->full[s]);
-            const uint32_t par = (phase_mask >> s) & 1u;
-            const uint64_t t0 = global_timer_ns();
-            while (!mbar_try_wait(bar, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
-          }
+        for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s) {
+          const uint32_t par = ((issued - 1 - s) / p.stages) & 1u;
+          const uint64_t t0 = global_timer_ns();
+          while (!mbar_try_wait(own_full + 8 * s, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
+        }
       }
     }
     __syncwarp();

@@ -310,8 +310,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0;
+      uint32_t stage = 0, phase = 0, issued = 0;
       bool ok = true;
+      const uint32_t own_full = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+      const uint32_t full0 = CTAS == 2 ? cluster_map_shared(own_full, 0) : own_full;             // the leader's barriers
       for (int item = walk.first(); item < walk.end && ok; item = walk.next(item)) {
         const TileCoord tc = coord(item);
         const CUtensorMap* tmb = tc.is_sum ? &p.tm_sum : &p.tm_emit;
@@ -319,23 +321,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
         const uint32_t bytes = CTAS * (kABytes + brows * (kBlockK * 2));   // of both CTAs' copies when paired
         const int arow = tc.arow;
         for (int t = 0; t < tc.ntiles && ok; ++t) {
-          for (int kb = 0; kb < p.kblocks; ++kb) {
-            if (!bounded_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
-            const uint32_t a_dst = tiles_addr + stage * p.stage_bytes;
-            const int brow = tc.brow0 + t * tc.cols + static_cast<int>(cta_rank) * brows;
+          const int brow = tc.brow0 + t * tc.cols + static_cast<int>(cta_rank) * brows;
+          for (int k = 0; k < p.kblocks * kBlockK; k += kBlockK) {
+            if (!bounded_wait(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
+            const uint32_t full = full0 + 8 * stage, a_dst = tiles_addr + stage * p.stage_bytes;
+            if (cta_rank == 0) mbar_arrive_expect_tx(own_full + 8 * stage, bytes);
             if (CTAS == 2) {
-              const uint32_t full = cluster_map_shared(smem_u32(&ctl->full[stage]), 0);   // the leader's barrier
-              if (cta_rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[stage]), bytes);
-              tma_load_2d_pair(a_dst, &p.tm_a, full, kb * kBlockK, arow);
-              tma_load_2d_pair(a_dst + kABytes, tmb, full, kb * kBlockK, brow);
+              tma_load_2d_pair(a_dst, &p.tm_a, full, k, arow);
+              tma_load_2d_pair(a_dst + kABytes, tmb, full, k, brow);
             } else {
-              const uint32_t full = smem_u32(&ctl->full[stage]);
-              mbar_arrive_expect_tx(full, bytes);
-              tma_load_2d(a_dst, &p.tm_a, full, kb * kBlockK, arow);
-              tma_load_2d(a_dst + kABytes, tmb, full, kb * kBlockK, brow);
+              tma_load_2d(a_dst, &p.tm_a, full, k, arow);
+              tma_load_2d(a_dst + kABytes, tmb, full, k, brow);
             }
-            issued_mask |= 1u << stage;
-            phase_mask = (phase_mask & ~(1u << stage)) | (phase << stage);
+            ++issued;
             if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
           }
         }
@@ -343,13 +341,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
       // The CTA must not go away with copies in flight. After a full run they have all landed already (the MMA warp
       // consumed them); after an abort, by this warp or by another one, give them a bounded chance to land.
       if (CTAS == 1 || cta_rank == 0) {
-        for (int s = 0; s < p.stages; ++s)
-          if (issued_mask & (1u << s)) {
-            const uint32_t bar = smem_u32(&ctl->full[s]);
-            const uint32_t par = (phase_mask >> s) & 1u;
-            const uint64_t t0 = global_timer_ns();
-            while (!mbar_try_wait(bar, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
-          }
+        for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s) {
+          const uint32_t par = ((issued - 1 - s) / p.stages) & 1u;
+          const uint64_t t0 = global_timer_ns();
+          while (!mbar_try_wait(own_full + 8 * s, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
+        }
       }
     }
     __syncwarp();

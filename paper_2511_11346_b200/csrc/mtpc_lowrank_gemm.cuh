@@ -735,8 +735,10 @@ __global__ void __launch_bounds__(32 * kDrawWarps) lowrank_slot_logits_kernel(
 // 64-symbol boxes, which are the K-major operand A of the product y and, untransposed, the MN-major operand A of the product dA.
 // y's accumulators (two, of k columns) leave at the end of each 128 positions, dA's (two sets of up to four tiles of 128 symbols) at
 // the end of the unit. z: the bf16 high half the forward pass left, k of the 64 columns that a box brings in. Bound by the bytes
-// of g: 2 T n r v. Two batched GEMMs, each reading g, took %OLD% us at 8192 positions of 8 x 32 units of 320 symbols, k = 16;
-// this takes %NEW%. Units of more than 512 symbols, or too few units to occupy the device, keep those.
+// of g: 2 T n r v. Two batched GEMMs, each reading g, took 505 us at 8192 positions of 8 x 32 units of 320 symbols,
+// k = 16; this takes 281, for 205 us of bytes (the second round of units leaves a quarter of the SMs idle; equal runs of tiles over
+// all units, which do not, took 353: CTAs at the same positions of neighbouring units read whole rows of g between them). Units of
+// more than 512 symbols, or too few units to occupy the device, keep those products.
 struct AdaptorGradParams {
   CUtensorMap tm_g;      // g    [T, n r v] at its pitch   box 64 x 128
   CUtensorMap tm_z;      // z    [T, n r 2 k]              box 64 x 128 (unit u: from column 2 k u)

@@ -1011,6 +1011,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
       // descriptor advance per K=16 step, in 16-byte units: 32 bytes along a swizzled K-major row, two 8-row groups
       // (2048 bytes) down an MN-major box
       constexpr uint32_t kStepA = A_MN ? 128u : 2u, kStepB = B_MN ? 128u : 2u;
+      const uint64_t a_desc0 = A_MN ? umma_smem_desc_mn_sw128(tiles_addr, kMnBoxBytes) : umma_smem_desc_sw128(tiles_addr);
+      const uint64_t b_desc0 = B_MN ? umma_smem_desc_mn_sw128(tiles_addr + kABytes, kMnBoxBytes)
+                                    : umma_smem_desc_sw128(tiles_addr + kABytes);
+      const uint32_t stage_step = p.stage_bytes >> 4, full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
       for (int item = first_item; item < num_items && ok; item += item_step, ++use) {
         const PlainItem w = plain_item(p, item, kblocks);
         const uint32_t slot = use % kSlots;
@@ -1018,20 +1022,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + slot * TN;
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (!bounded_wait(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
+          if (!bounded_wait(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a_addr = tiles_addr + stage * p.stage_bytes;
-          const uint64_t a_desc = A_MN ? umma_smem_desc_mn_sw128(a_addr, kMnBoxBytes) : umma_smem_desc_sw128(a_addr);
-          const uint64_t b_desc = B_MN ? umma_smem_desc_mn_sw128(a_addr + kABytes, kMnBoxBytes)
-                                       : umma_smem_desc_sw128(a_addr + kABytes);
+          const uint64_t a_desc = a_desc0 + stage * stage_step, b_desc = b_desc0 + stage * stage_step;
 #pragma unroll
           for (int kk = 0; kk < kBlockK / 16; ++kk) {
             const uint32_t acc = (kb != w.kb0 || kk != 0) ? 1u : 0u;
             if (CTAS == 2) umma_bf16_pair(d_tmem, a_desc + kStepA * kk, b_desc + kStepB * kk, idesc, acc);
             else umma_bf16(d_tmem, a_desc + kStepA * kk, b_desc + kStepB * kk, idesc, acc);
           }
-          if (CTAS == 2) umma_commit_pair(smem_u32(&ctl->empty[stage]));
-          else umma_commit(smem_u32(&ctl->empty[stage]));
+          if (CTAS == 2) umma_commit_pair(empty0 + 8 * stage);
+          else umma_commit(empty0 + 8 * stage);
           if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;

@@ -354,6 +354,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
     if (lane == 0 && cta_rank == 0) {
       uint32_t stage = 0, phase = 0, use = 0;
       bool ok = true;
+      const uint64_t a_desc0 = umma_smem_desc_sw128(tiles_addr), b_desc0 = umma_smem_desc_sw128(tiles_addr + kABytes);
+      const uint32_t stage_step = p.stage_bytes >> 4, full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
       for (int item = walk.first(); item < walk.end && ok; item = walk.next(item)) {
         const TileCoord tc = coord(item);
         const uint32_t idesc = umma_idesc_bf16(kBlockM * CTAS, tc.cols);
@@ -366,18 +368,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + slot * p.slot_stride;
           for (int kb = 0; kb < p.kblocks; ++kb) {
-            if (!bounded_wait(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
+            if (!bounded_wait(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
             tc_fence_after();
-            const uint32_t a_addr = tiles_addr + stage * p.stage_bytes;
-            const uint64_t a_desc = umma_smem_desc_sw128(a_addr);
-            const uint64_t b_desc = umma_smem_desc_sw128(a_addr + kABytes);
+            const uint64_t a_desc = a_desc0 + stage * stage_step, b_desc = b_desc0 + stage * stage_step;
 #pragma unroll
             for (int kk = 0; kk < kBlockK / 16; ++kk) {   // +32 bytes per K=16 step inside the swizzled row
               if (CTAS == 2) umma_bf16_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
               else umma_bf16(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
             }
-            if (CTAS == 2) umma_commit_pair(smem_u32(&ctl->empty[stage]));   // frees the stage in both CTAs
-            else umma_commit(smem_u32(&ctl->empty[stage]));
+            if (CTAS == 2) umma_commit_pair(empty0 + 8 * stage);   // frees the stage in both CTAs
+            else umma_commit(empty0 + 8 * stage);
             if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
           }
           if (!ok) break;

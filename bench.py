@@ -417,8 +417,8 @@ def measure_factored_backward(torch, wl, lowrank, steps: int):
     head.mtpc_destroy()
     return {"call": "mtpc_lowrank_window_logprob_backward", "ms_per_call": ms, "phase_ms": phase_ms,
             "eq6_call": "mtpc_lowrank_window_loss_backward", "eq6_ms_per_call": ms6, "eq6_loss": float(loss.cpu()[0]),
-            "phases": "factored forward keeping the logits, circuit backward, logit gradients + their sums + operand "
-                      "copies, GEMMs (g A, d hidden, dW_base, dB, dW_sum, dA)",
+            "phases": "factored forward, circuit backward, logit gradients from the base logits + their sums, "
+                      "products (g A and dA from one reading of g, d hidden, dW_base with dB and dW_sum)",
             "value_equals_forward_call": same_value, "device_status": status,
             "note": "the route through the composed tensor costs compose_ms + the dense backward call + backward_ms"}
 
@@ -583,8 +583,8 @@ def measure_eq6_step(torch, dh, wl, hidden, targets, grads, steps: int):
                          "logit_gradient": phase_ms[2], "plain_gemms": phase_ms[3]}}
 
 
-CIRCUIT_KERNEL = {I.CP: "circuit_cp_kernel", I.HMM: "circuit_hmm_stream_kernel", I.BTREE: "circuit_btree_kernel",
-                  I.HMM_CTX: "circuit_hmm_stream_kernel (per-position tables)"}
+CIRCUIT_KERNEL = {I.CP: "circuit_cp_kernel", I.HMM: "circuit_hmm_kernel", I.BTREE: "circuit_btree_kernel",
+                  I.HMM_CTX: "circuit_hmm_kernel (per-position tables)"}
 
 
 def config_block(idx: int, wl, world: int) -> dict:

@@ -309,7 +309,7 @@ class MtpcHead:
         _check(lib().mtpc_debug_set_projection_variant(self.handle, int(variant)), "mtpc_debug_set_projection_variant")
 
     def mtpc_debug_set_draft_grouping(self, mode: int) -> None:
-        """Test hook, many-position draft: 0 = chosen per call, 1 = all units for all positions, 2 = draws sorted by unit."""
+        """Test hook kept for callers: many-position drafts have one form now, so 0, 1 and 2 are accepted and change nothing."""
         _check(lib().mtpc_debug_set_draft_grouping(self.handle, int(mode)), "mtpc_debug_set_draft_grouping")
 
     def mtpc_set_timing(self, ring: int) -> None:

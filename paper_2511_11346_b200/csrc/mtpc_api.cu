@@ -8,6 +8,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <atomic>
 #include <new>
 
 #include "../../include/mtpc.h"
@@ -551,14 +552,19 @@ bool set_circuit_attributes() {
   return ok;
 }
 
-// How many clusters of `size` CTAs of a kernel the device holds at once (0: none).
+// How many clusters of `size` CTAs of a kernel, each with all the shared memory a CTA can have, device `dev` holds at once (0:
+// none). Asked of the driver once per device and `which` (about 30 us each, a property of the device): heads are made often.
 template <typename K>
-int resident_clusters(K kernel, int size, int smem_bytes) {
+int resident_clusters(K kernel, int size, int which, int dev) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[4][kDevices];                            // count + 1
+  std::atomic<int>* entry = dev >= 0 && dev < kDevices ? &known[which][dev] : nullptr;
+  if (entry && entry->load() > 0) return entry->load() - 1;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(size);
   cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = smem_bytes;
+  cfg.dynamicSmemBytes = kSmemLimit;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = size;
@@ -571,6 +577,7 @@ int resident_clusters(K kernel, int size, int smem_bytes) {
     cudaGetLastError();
     return 0;
   }
+  if (entry) entry->store(clusters + 1);
   return clusters;
 }
 
@@ -1557,7 +1564,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
                                kSmemLimit) != cudaSuccess;
   fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogitsGrouped, 1>);
   fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 2>);
-  h->max_pairs = fail ? 0 : resident_clusters(mtpc_gemm_kernel<kModeLogprob, 2>, 2, L.lp.pair_smem);
+  h->max_pairs = fail ? 0 : resident_clusters(mtpc_gemm_kernel<kModeLogprob, 2>, 2, 0, dev);
   fail |= !allow_full_smem(plain_gemm_kernel<false, false>);
   fail |= !allow_full_smem(plain_gemm_kernel<false, true>);
   fail |= !allow_full_smem(plain_gemm_kernel<true, true>);
@@ -1569,7 +1576,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   fail |= !allow_full_smem(adaptor_grad_kernel);
   fail |= cudaFuncSetAttribute(mtpc_decode_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) !=
           cudaSuccess;
-  for (int e = 0; e < 3; ++e) h->max_decode_clusters[e] = fail ? 0 : resident_clusters(mtpc_decode_gemm_kernel, 2 << e, kSmemLimit);
+  for (int e = 0; e < 3; ++e) h->max_decode_clusters[e] = fail ? 0 : resident_clusters(mtpc_decode_gemm_kernel, 2 << e, 1 + e, dev);
   const int slot_smem = static_cast<int>(kSlotSmemLimit);
   fail |= cudaFuncSetAttribute(draft_slot_kernel<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
   fail |= cudaFuncSetAttribute(draft_slot_kernel<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;

@@ -194,37 +194,40 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0;
+      uint32_t stage = 0, phase = 0, issued = 0;
       bool ok = true;
+      const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
       for (int cur = tile_begin; cur < tile_end && ok;) {
         const int ntiles = min(p.pass_tiles, tile_end - cur);
         uint32_t bytes = p.Ppad * (kBlockK * 2);                   // out-of-range rows are zero-filled and counted
-        for (int q = 0; q < ntiles; ++q) bytes += decode_tile(p, cur + q).rows * (kBlockK * 2);
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!bounded_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
-          const uint32_t full = smem_u32(&ctl->full[stage]);
-          const uint32_t dst = tiles_addr + stage * p.stage_bytes;
+        const CUtensorMap* map[kDecodeMaxTiles];
+        int row[kDecodeMaxTiles];
+#pragma unroll
+        for (int q = 0; q < kDecodeMaxTiles; ++q) {
+          const DecodeTile t = decode_tile(p, min(cur + q, tile_end - 1));
+          map[q] = t.is_sum ? &p.tm_sum : (t.second ? &p.tm_emit2 : &p.tm_emit);
+          row[q] = t.index * t.rows;
+          if (q < ntiles) bytes += t.rows * (kBlockK * 2);
+        }
+        for (int k = kb0 * kBlockK; k < kb1 * kBlockK; k += kBlockK) {
+          if (!bounded_wait(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
+          const uint32_t full = full0 + 8 * stage, dst = tiles_addr + stage * p.stage_bytes;
           mbar_arrive_expect_tx(full, bytes);
-          for (int q = 0; q < ntiles; ++q) {
-            const DecodeTile t = decode_tile(p, cur + q);
-            tma_load_2d(dst + q * p.tile_bytes, t.is_sum ? &p.tm_sum : (t.second ? &p.tm_emit2 : &p.tm_emit), full,
-                        kb * kBlockK, t.index * t.rows);
-          }
-          tma_load_2d(dst + hidden_off, &p.tm_h, full, kb * kBlockK, 0);
-          issued_mask |= 1u << stage;
-          phase_mask = (phase_mask & ~(1u << stage)) | (phase << stage);
+#pragma unroll
+          for (int q = 0; q < kDecodeMaxTiles; ++q)
+            if (q < ntiles) tma_load_2d(dst + q * p.tile_bytes, map[q], full, k, row[q]);
+          tma_load_2d(dst + hidden_off, &p.tm_h, full, k, 0);
+          ++issued;
           if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
         }
         cur += ntiles;
       }
       // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
-      for (int s = 0; s < p.stages; ++s)
-        if (issued_mask & (1u << s)) {
-          const uint32_t bar = smem_u32(&ctl->full[s]);
-          const uint32_t par = (phase_mask >> s) & 1u;
-          const uint64_t t0 = global_timer_ns();
-          while (!mbar_try_wait(bar, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
-        }
+      for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s) {
+        const uint32_t par = ((issued - 1 - s) / p.stages) & 1u;
+        const uint64_t t0 = global_timer_ns();
+        while (!mbar_try_wait(full0 + 8 * s, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
+      }
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -233,6 +236,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
       uint32_t stage = 0, phase = 0, use = 0;
       bool ok = true;
       const uint32_t idesc = umma_idesc_bf16(kBlockM, p.Ppad);
+      const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+      const uint32_t stage_step = p.stage_bytes >> 4, tile_step = p.tile_bytes >> 4;          // descriptors step in 16-byte units
+      const uint64_t a_desc0 = umma_smem_desc_sw128(tiles_addr), b_desc0 = umma_smem_desc_sw128(tiles_addr + hidden_off);
       for (int cur = tile_begin; cur < tile_end && ok; ++use) {
         const int ntiles = min(p.pass_tiles, tile_end - cur);
         cur += ntiles;
@@ -244,17 +250,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + slot * slot_cols;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!bounded_wait(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
+          if (!bounded_wait(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t w_addr = tiles_addr + stage * p.stage_bytes;
-          const uint64_t b_desc = umma_smem_desc_sw128(w_addr + hidden_off);
+          const uint64_t b_desc = b_desc0 + stage * stage_step;
           for (int q = 0; q < ntiles; ++q) {
-            const uint64_t a_desc = umma_smem_desc_sw128(w_addr + q * p.tile_bytes);
+            const uint64_t a_desc = a_desc0 + stage * stage_step + q * tile_step;
 #pragma unroll
             for (int kk = 0; kk < kBlockK / 16; ++kk)
               umma_bf16(d_tmem + q * p.tile_stride, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
           }
-          umma_commit(smem_u32(&ctl->empty[stage]));
+          umma_commit(empty0 + 8 * stage);
           if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;

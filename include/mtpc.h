@@ -338,7 +338,7 @@ int mtpc_create_head_lowrank(const mtpc_config* cfg, int32_t k, const void* W_ba
  * Host-buffer variants: same results, but hidden / targets / uniforms are HOST pointers (pinned memory for
  * full copy speed) and the outputs are written to HOST buffers. The copies to and from the device go through
  * staging areas in the workspace; the call returns after the stream has been synchronised, so the outputs are
- * ready on return. mtpc_window_logprob_host uploads and processes 2048 positions at a time: the uploads run on a
+ * ready on return. mtpc_window_logprob_host uploads and processes the positions in pieces: the uploads run on a
  * second stream the head owns, ordered after the work already on `stream`, so that all but the first are hidden
  * behind the kernels (with per-kernel timing on, every chunk is recorded as a call of its own).
  */

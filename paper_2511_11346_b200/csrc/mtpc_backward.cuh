@@ -784,8 +784,7 @@ __global__ void __launch_bounds__(256) logit_gradient_kernel(const LogitGradArgs
 // range of different tiles and share its operands through L2). The parts are written as fp32 tiles and split_reduce_kernel adds
 // them up in K order, spread over the whole device. (Added up by the warp that arrives last, a few warps read every part alone:
 // 12 tiles in 8 parts took 29 us where the uncut launch takes 19.) It matters where a contraction has few tiles: d hidden of
-// 2005 positions is 96 pair tiles for 74 pairs (415 -> 271 us), of 4096 positions 192 (2945 -> 2480 us, of which the pairs
-// give about 5 %).
+// 2005 positions is 96 pair tiles for 74 pairs (415 -> 271 us), of 4096 positions 192 (2945 -> 2480 us, pairs and cut together).
 struct PlainGemmParams {
   CUtensorMap tm_a;      // K-major: A [M, K], box 64 (k) x 128; MN-major: A^T [K, M], box 64 (m) x 64 (k)
   CUtensorMap tm_b[3];   // per K segment. K-major: B [N, K], box 64 (k) x TN / CTAS; MN-major: B^T [K, N], box 64 (n) x 64 (k)

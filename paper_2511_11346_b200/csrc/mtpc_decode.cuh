@@ -79,7 +79,8 @@ __device__ __forceinline__ DecodeTile decode_tile(const DecodeParams& p, int t) 
 // tile, each walking its part of K; the others hand their fp32 accumulators to the first one through its shared memory (behind
 // the ring: [rank - 1][tile][position quad][128 rows] of float4), which adds them in rank order and runs the epilogue.
 // Every CTA then has one pass. The pass over 39 MB of weights (n = 8, r = 16, v = 320, d = 4096, rank 16) took 30 us as 72 CTAs
-// of 64 K steps and half the SMs idle; draft + acceptance of 8 positions: 51 -> 38 us with 146 CTAs of 32 steps.
+// of 64 K steps and half the SMs idle; draft + acceptance of 8 positions: 51 -> 38 us with clusters
+// of two.
 __host__ __device__ inline size_t decode_exchange_bytes(int ksplit, int pass_tiles, int Ppad) {
   return static_cast<size_t>(ksplit - 1) * pass_tiles * kBlockM * Ppad * sizeof(float);
 }

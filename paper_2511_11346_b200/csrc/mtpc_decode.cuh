@@ -705,35 +705,41 @@ __global__ void __launch_bounds__(32 * kLatentWarps) latent_sample_kernel(
     int* __restrict__ unit_sel, int* __restrict__ out_bytes, unsigned* status, int W, int wpp, int n, int r, int sum_rows,
     int logA_stride) {
   grid_dependency_wait();
-  __shared__ int zs[kLatentWarps][64];
   const int w = blockIdx.x * kLatentWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= W) return;
-  int* z = zs[threadIdx.x >> 5];
   const float* lw = logw + static_cast<size_t>(w / wpp) * sum_rows;
   const float* u = uniforms + static_cast<size_t>(w) * 2 * n;
   const int nlat = (family == 0) ? 1 : (family == 1 ? n : n - 1);
+  // The drawn values stay in registers, lane l those of the latents l and 32 + l, and are read by shuffles.
+  int lo = 0, hi = 0;
+  auto value = [&](int j) {                        // of latent j, which may differ from lane to lane
+    const int a = __shfl_sync(kFull, lo, j & 31), b = __shfl_sync(kFull, hi, j & 31);
+    return j < 32 ? a : b;
+  };
   bool bad = false;
   for (int c = lane; c < nlat; c += 32) bad |= !(u[c] >= 0.f && u[c] < 1.f);
   bad = __any_sync(kFull, bad);
   if (bad) {
     if (lane == 0) atomicOr(status, 2u);
   } else {
-    const int root = r > 32 ? warp_inv_cdf_logits_wide(lw, r, u[0], lane) : warp_inv_cdf_logp(lane < r ? lw[lane] : 0.f, r, u[0], lane);
-    if (lane == 0) z[0] = root;
-    int prev = root;
+    int prev = r > 32 ? warp_inv_cdf_logits_wide(lw, r, u[0], lane) : warp_inv_cdf_logp(lane < r ? lw[lane] : 0.f, r, u[0], lane);
+    if (lane == 0) lo = prev;
     for (int j = 1; j < nlat; ++j) {
-      const float* tab = family == 1 ? logA + static_cast<size_t>(w / wpp) * logA_stride + (static_cast<size_t>(j - 1) * r + prev) * r
-                                     : lw + r + (static_cast<size_t>(j - 1) * r + z[(j - 1) >> 1]) * r;
+      const int parent = family == 1 ? prev : value((j - 1) >> 1);
+      const float* tab = family == 1 ? logA + static_cast<size_t>(w / wpp) * logA_stride + (static_cast<size_t>(j - 1) * r + parent) * r
+                                     : lw + r + (static_cast<size_t>(j - 1) * r + parent) * r;
       prev = warp_inv_cdf_logp(lane < r ? tab[lane] : 0.f, r, u[j], lane);
-      if (lane == 0) z[j] = prev;
-      __syncwarp();
+      if (lane == (j & 31)) (j < 32 ? lo : hi) = prev;
     }
-    __syncwarp();
   }
-  for (int i = lane; i < n; i += 32) {
-    unit_sel[static_cast<size_t>(w) * n + i] = bad ? -1 : (family == 0 ? z[0] : family == 1 ? z[i] : z[n / 2 - 1 + (i >> 1)]);
-    out_bytes[static_cast<size_t>(w) * n + i] = -1;
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    const int i = i0 + lane;
+    const int z = value(i >= n || family == 0 ? 0 : family == 1 ? i : n / 2 - 1 + (i >> 1));
+    if (i < n) {
+      unit_sel[static_cast<size_t>(w) * n + i] = bad ? -1 : z;
+      out_bytes[static_cast<size_t>(w) * n + i] = -1;
+    }
   }
   grid_launch_dependents();
 }

@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kerne
         for (int q = 0; q < 16; ++q) sum[q] = make_float2(0.f, 0.f);
         const int tgt = valid ? p.targets[static_cast<size_t>(row) * p.n + w.slot] : -1;
         has_target = tgt >= 0;                             // a marginalised byte has no gradient
-        rel = (tgt >= col0 && tgt < col0 + 32) ? tgt - col0 : -1;
+        rel = (tgt >= col0 && tgt < min(col0 + 32, p.vv)) ? tgt - col0 : -1;   // (a refused target, >= vv, has no column)
       } else {
         cp_async_commit();
         if (valid && here > 0) p.ref[static_cast<size_t>(col0 / 32) * p.T * p.n + static_cast<size_t>(row) * p.n + w.slot] = ref;

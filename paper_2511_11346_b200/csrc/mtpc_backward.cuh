@@ -61,7 +61,8 @@ __global__ void circuit_cp_backward_kernel(const CircuitBackwardArgs a_) {
     if (k < r) {
       a[q] = lw[k];
       for (int i = 0; i < n; ++i) a[q] += g[i * r + k];
-      lse_merge(m, s, a[q], 1.f);
+      if (a[q] != a[q]) { m = 0.f; s = a[q]; }                           // NaN must survive the maximum
+      else lse_merge(m, s, a[q], 1.f);
     }
   }
 #pragma unroll

@@ -173,7 +173,8 @@ int mtpc_draft_sample_prefix(mtpc_head* head, const void* hidden, int32_t P, int
  * Acceptance stage of speculative sampling (Algorithm 3, from "determine the number of accepted tokens" to the
  * last byte), for the P*wpp windows of the head's most recent draft. The target model's conditionals are an input:
  * the LLM that produces them is outside this library.
- *   draft_bytes     dev [W, n] int32, W = P*wpp: the drafted windows (as written by mtpc_draft_sample*).
+ *   draft_bytes     dev [W, n] int32, W = P*wpp: the drafted windows as mtpc_draft_sample* wrote them, in their order (the
+ *                   draft left what it knows about these bytes, window by window; other bytes are not evaluated).
  *   prefix_logprob  dev [W, n] fp32: their prefix log-marginals (as written by mtpc_draft_sample_prefix).
  *   target_probs    dev [W, n+1, v] fp32: row i is p(X_{t+i+1} | context, draft bytes 0..i-1), probabilities.
  *   accept_uniforms dev [W, n+1] fp32 in [0,1): column i is the alpha of the test on byte i; column n draws the
@@ -192,9 +193,7 @@ int mtpc_draft_sample_prefix(mtpc_head* head, const void* hidden, int32_t P, int
  *     position): such a draft runs in chunks of positions and leaves only the evidence of the drafted bytes. The call then
  *     runs the tests, sorts the rejected windows by the slot of their first rejected byte, recomputes that slot's r*v logits
  *     for them in one projection pass over staged hidden states, and draws. It reads the hidden states the DRAFT call was
- *     given (bf16 heads: the caller's buffer, which must still hold them);
- *   - a draft by mtpc_draft_sample leaves no slot messages (what the sweep for prefix marginals yields besides them): the
- *     first acceptance call after it forms them with one more launch.
+ *     given (bf16 heads: the caller's buffer, which must still hold them).
  * A uniform outside [0,1) or a draft byte outside [0,v) sets the status bit and yields -1 / -1 for that window.
  */
 int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32_t* draft_bytes,

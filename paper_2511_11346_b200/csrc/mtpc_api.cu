@@ -266,8 +266,7 @@ struct mtpc_head {
   int copy_event_count;
   int draft_P;              // positions whose draft state (logits, or after a many-position draft G and log omega) is in the workspace (0: none)
   int draft_wpp;            // windows per position of that draft
-  bool draft_msg;           // its slot messages are in the workspace too (a draft that asked for prefix marginals leaves them)
-  bool draft_logits;        // every logit and unit log-sum-exp of its positions as well
+  bool draft_logits;        // every logit and unit log-sum-exp of its positions is there as well
   const void* draft_hidden; // the bf16 hidden states it read (the acceptance stage may have to stage rows of them)
   int ring;                 // calls whose per-kernel events are retained (0 = timing off)
   cudaEvent_t* ev;          // [ring][kMaxPhases][2]
@@ -760,13 +759,14 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
   const mtpc_config& c = h->cfg;
   const Layout& L = h->L;
   const int W = P * wpp;
-  // a draft that returns prefix marginals runs the sweep that also yields the slot messages of the acceptance stage
+  // Every draft runs the sweep that also yields the slot messages of the acceptance stage, whether it returns joints or prefix
+  // marginals: what it leaves behind is a function of P and wpp alone, so a recorded acceptance call may follow either.
   float* const msg = at<float>(h, L.off_msg);
   if (h->lr_k > 0 && P > L.decode_max_p && wpp == 1 && c.v <= kMaxDraftVocab) {
     // A long draft on a factored head, one window per position: log omega, the latent draws, then every (window, slot)
     // forms the logits of its one selected unit from W_base h and B h (lowrank_draw_kernel) and draws its byte; the
     // evidence of the drafted bytes under every unit is the factored projection with them as targets. No logits are
-    // kept: no acceptance stage after such a draft.
+    // kept: the acceptance stage forms those of a window's rejected slot from W_base h and B h.
     const int k = h->lr_k;
     h->draft_P = 0;
     PhaseTimer pt(h, st);
@@ -800,12 +800,11 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     pt.end();
     if (rc != MTPC_OK) return rc;
     pt.begin();
-    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*raw_mixture=*/false, out_prefix ? msg : nullptr);
+    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*raw_mixture=*/false, msg);
     pt.end();
     if (rc == MTPC_OK) {               // G, log omega, the messages, W_base h and B h stay in place for an acceptance call
       h->draft_P = P;
       h->draft_wpp = wpp;
-      h->draft_msg = out_prefix != nullptr;
       h->draft_logits = false;
       h->draft_hidden = nullptr;
     }
@@ -813,8 +812,8 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
   }
   if (h->lr_k > 0 && P > L.decode_max_p) {
     // Otherwise (several windows per position, or units wider than 512 symbols) the few-position path runs chunk after
-    // chunk of positions: W_base, B and A are small enough to stay in L2. Only the last chunk's logits remain: no
-    // acceptance stage after such a draft either.
+    // chunk of positions: W_base, B and A are small enough to stay in L2. Only the last chunk's logits and messages remain: no
+    // acceptance stage after such a draft.
     for (int p0 = 0; p0 < P; p0 += L.decode_max_p) {
       const int pc = P - p0 < L.decode_max_p ? P - p0 : L.decode_max_p;
       const size_t w0 = static_cast<size_t>(p0) * wpp;
@@ -869,13 +868,11 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     h->launches++;
     h->draft_P = P;
     h->draft_wpp = wpp;
-    h->draft_msg = out_prefix != nullptr;
     h->draft_logits = true;
     pt.end();
     if ((rc = check_launch()) != MTPC_OK) return rc;
     pt.begin();
-    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*raw_mixture=*/c.r > 32,
-                        out_prefix ? msg : nullptr);
+    rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*raw_mixture=*/c.r > 32, msg);
     pt.end();
     return rc;
   }
@@ -913,12 +910,11 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     if ((rc = check_launch()) != MTPC_OK) return rc;
   }
   pt.begin();
-  rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*raw_mixture=*/false, out_prefix ? msg : nullptr);
+  rc = launch_circuit(h, W, wpp, out_logprob, out_prefix, st, /*raw_mixture=*/false, msg);
   pt.end();
   if (rc == MTPC_OK) {                 // G, log omega, the messages and the logits stay in place for an acceptance call
     h->draft_P = P;
     h->draft_wpp = wpp;
-    h->draft_msg = out_prefix != nullptr;
     h->draft_logits = chunks == 1;
     h->draft_hidden = hb;
   }
@@ -1694,12 +1690,6 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
   const int threads = accept_threads(c.v);
   PhaseTimer pt(head, st);
   float* const msg = at<float>(head, L.off_msg);
-  if (!head->draft_msg) {
-    // the draft returned the joint alone: the slot messages are formed now, from the evidence and log omega it left
-    rc = launch_circuit(head, W, wpp, nullptr, nullptr, st, /*raw_mixture=*/P <= L.decode_max_p && c.r > 32, msg);
-    if (rc != MTPC_OK) return rc;
-    head->draft_msg = true;
-  }
   if (head->draft_logits) {
     // every logit of the drafted positions is still in the workspace
     pt.begin();

@@ -1139,17 +1139,30 @@ int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, cons
 }
 
 // Warps per CTA of the circuit backward kernels: as many of 8, 4, 2, 1 as keep the CTA's shared memory within the limit
-// (long windows need n x r floats of messages per warp). 0: not even one warp fits.
-size_t circuit_backward_smem(const mtpc_head* h, int warps) {
+// (long windows need n x r floats of messages per warp). warps == 0: not even one warp fits.
+struct BackwardShape {
+  int warps;
+  size_t smem;
+  bool wide;                 // HMM, Eq. 6: see hmm_loss_warp_floats
+};
+BackwardShape circuit_backward_shape(const mtpc_head* h, bool loss) {
   const mtpc_config& c = h->cfg;
-  if (c.family == MTPC_HMM) return hmm_backward_smem_floats(c.n, c.r, !is_ctx(h), warps) * sizeof(float);
-  if (c.family == MTPC_BTREE) return static_cast<size_t>(warps) * btree_backward_warp_floats(c.n, c.r) * sizeof(float);
-  return static_cast<size_t>(warps) * cp_loss_warp_floats(c.n, c.r) * sizeof(float);
-}
-int circuit_backward_warps(const mtpc_head* h) {
-  for (int w = kCircuitWarps; w >= 1; w >>= 1)
-    if (circuit_backward_smem(h, w) <= static_cast<size_t>(kSmemLimit)) return w;
-  return 0;
+  const size_t shared = c.family == MTPC_HMM && !is_ctx(h) ? static_cast<size_t>(c.n - 1) * c.r * c.r : 0;   // the CTA's dT
+  auto fit = [&](size_t per_warp) {
+    for (int w = kCircuitWarps; w >= 1; w >>= 1)
+      if ((shared + w * per_warp) * sizeof(float) <= static_cast<size_t>(kSmemLimit)) return w;
+    return 0;
+  };
+  auto shape = [&](size_t per_warp, bool wide) {
+    const int w = fit(per_warp);
+    return BackwardShape{w, (shared + w * per_warp) * sizeof(float), wide};
+  };
+  if (c.family == MTPC_BTREE) return shape(btree_backward_warp_floats(c.n, c.r), false);
+  if (c.family == MTPC_CP) return shape(loss ? cp_loss_warp_floats(c.n, c.r) : 0, false);
+  const BackwardShape compact = shape(hmm_backward_warp_floats(c.n, c.r), false);
+  if (!loss) return compact;
+  const BackwardShape wide = shape(hmm_loss_warp_floats(c.n, c.r, true), true);
+  return wide.warps >= compact.warps ? wide : compact;
 }
 
 // a.coeff (Eq. 6: the weights [W, n] of the prefix log-marginals) chooses the kernels that give every prefix and the whole
@@ -1164,20 +1177,20 @@ int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cuda
   a.sum_rows = L.sum_rows;
   unsigned* counter = at<unsigned>(h, L.off_status) + kWorkCounterWord;
   const bool loss = a.coeff != nullptr;
-  const int warps = circuit_backward_warps(h);
+  const BackwardShape shape = circuit_backward_shape(h, loss);
+  const int warps = shape.warps;
   if (warps == 0) return MTPC_ERR_UNSUPPORTED;
   const int blocks = (a.W + warps - 1) / warps;
   const int threads = warps * 32;
   const int resident = blocks < 8 * h->num_sms ? blocks : 8 * h->num_sms;
-  const size_t smem = circuit_backward_smem(h, warps);
+  const size_t smem = shape.smem;
   if (c.family == MTPC_CP && loss) {
     launch_kernel(circuit_cp_loss_backward_kernel, blocks, threads, smem, st, overlapped(h), a);
   } else if (c.family == MTPC_CP) {
-    launch_kernel(circuit_cp_backward_kernel, (a.W + kCircuitWarps - 1) / kCircuitWarps, kCircuitWarps * 32, 0, st,
-                  overlapped(h), a);
+    launch_kernel(circuit_cp_backward_kernel, blocks, threads, smem, st, overlapped(h), a);
   } else if (c.family == MTPC_HMM && loss) {
     launch_kernel(circuit_hmm_loss_backward_kernel, resident, threads, smem, st, overlapped(h), a, hmm_tables(h),
-                  hmm_table_stride(h), dT, counter);
+                  hmm_table_stride(h), dT, counter, shape.wide ? 1 : 0);
   } else if (c.family == MTPC_HMM) {
     launch_kernel(circuit_hmm_backward_kernel, resident, threads, smem, st, overlapped(h), a, hmm_tables(h),
                   hmm_table_stride(h), dT, counter);
@@ -1197,7 +1210,7 @@ int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cuda
 
 // Shared-memory attributes of the circuit backward kernels (per function: always the full limit, see allow_full_smem).
 int set_backward_attributes(const mtpc_head* head) {
-  if (circuit_backward_warps(head) == 0) return MTPC_ERR_UNSUPPORTED;
+  if (circuit_backward_shape(head, false).warps == 0) return MTPC_ERR_UNSUPPORTED;   // (the loss kernels fit where these do)
   bool ok = allow_full_smem(circuit_hmm_backward_kernel);
   ok &= allow_full_smem(circuit_cp_loss_backward_kernel);
   ok &= allow_full_smem(circuit_btree_loss_backward_kernel);

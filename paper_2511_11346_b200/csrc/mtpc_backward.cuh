@@ -189,10 +189,12 @@ __device__ __forceinline__ void row_grad(const float* row, const float* pc, floa
 // the windows into dT [n-1, r, r] (fp32): per CTA in shared memory first, then one atomicAdd per entry and CTA.
 // Shared memory: per warp n*r (alpha) + 2*r*r (tables) + 64 floats; static: + (n-1)*r*r floats per CTA.  r <= 32.
 __host__ __device__ inline size_t hmm_backward_warp_floats(int n, int r) {
-  return (static_cast<size_t>(n) * (r + 2) + 3) / 4 * 4 + 2 * r * r + 64;   // alphas, prefixes (Eq. 6), two tables, two vectors of 32
+  return static_cast<size_t>(n) * r + 2 * r * r + 64;             // alphas, two tables, two vectors of 32
 }
-__host__ __device__ inline size_t hmm_backward_smem_floats(int n, int r, bool is_static, int warps) {
-  return static_cast<size_t>(warps) * hmm_backward_warp_floats(n, r) + (is_static ? static_cast<size_t>(n - 1) * r * r : 0);
+// The kernel of Eq. 6 takes n more floats for the prefixes and a pitch of r + 1 for the alphas, so that a lane per slot reads them
+// without bank conflicts - unless without them more warps fit (n = 54 at r = 32, static, fits no other way), then `wide` is false.
+__host__ __device__ inline size_t hmm_loss_warp_floats(int n, int r, bool wide) {
+  return wide ? (static_cast<size_t>(n) * (r + 2) + 3) / 4 * 4 + 2 * r * r + 64 : hmm_backward_warp_floats(n, r);
 }
 
 __global__ void circuit_hmm_backward_kernel(const CircuitBackwardArgs a_, const float* __restrict__ tables,
@@ -351,7 +353,7 @@ __device__ __forceinline__ void row_grad_mult(const float* row, const float* pc,
 }
 
 __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, const float* __restrict__ tables,
-                                                 int table_stride, float* __restrict__ dT, unsigned* work_counter) {
+                                                 int table_stride, float* __restrict__ dT, unsigned* work_counter, int wide) {
   grid_launch_dependents();
   grid_dependency_wait();
   extern __shared__ __align__(16) float sm[];
@@ -361,12 +363,12 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
   const int rr = r * r;
   const bool is_static = table_stride == 0;
   float* acc = sm;                                                       // static only: [n-1, r, r]
-  float* mine = sm + (is_static ? (n - 1) * rr : 0) + static_cast<size_t>(wib) * hmm_backward_warp_floats(n, r);
+  float* mine = sm + (is_static ? (n - 1) * rr : 0) + static_cast<size_t>(wib) * hmm_loss_warp_floats(n, r, wide != 0);
   float* tabs = mine;
   float* cvec = tabs + 2 * rr;                                           // G[i] - alpha_i (log domain)
   float* dvec = cvec + 32;                                               // abar_i (plain)
-  float* alphas = dvec + 32;                                             // [n][r + 1]
-  float* lps = alphas + n * (r + 1);                                     // [n] the prefix log-marginals
+  float* alphas = dvec + 32;                                             // [n][pitch]
+  const int pitch = wide ? r + 1 : r;
   const bool has = lane < r;
   const HmmLanes l = hmm_lanes(r, lane);
   if (is_static) {
@@ -379,6 +381,7 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
     const float* tb = tables + static_cast<size_t>(w) * table_stride;
     const float* cw = a_.coeff + static_cast<size_t>(w) * n;
     const int* tg = a_.targets + static_cast<size_t>(w) * n;
+    float* lps = wide ? alphas + n * pitch : a_.prefix + static_cast<size_t>(w) * n;   // [n] the prefix log-marginals
     const size_t prow = static_cast<size_t>(w) * n * r;
     const size_t drow = static_cast<size_t>(w) * a_.dsum_pitch;
     // ---- forward, keeping every alpha_i
@@ -395,12 +398,12 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
       __syncwarp();
       const float c = hmm_forward_step<true>(alpha, cvec, tabs + ((i - 1) & 1) * rr, l, r);
       alpha = l.active ? c + g[i * r + l.k] : -CUDART_INF_F;
-      if (has) alphas[i * (r + 1) + lane] = alpha;
+      if (has) alphas[i * pitch + lane] = alpha;
       __syncwarp();
     }
     if (!has) alpha = -CUDART_INF_F;                                     // (the other parts' copies)
     for (int i = lane; i < n; i += 32) {                                 // every prefix, lane = slot (as circuit_hmm_kernel)
-      const float lp = thread_lse(alphas + i * (r + 1), r);
+      const float lp = thread_lse(alphas + i * pitch, r);
       lps[i] = lp;
       a_.prefix[static_cast<size_t>(w) * n + i] = lp;
     }
@@ -414,7 +417,7 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
       }
       if (i - 1 >= 1) warp_table_load_async(tabs + (i & 1) * rr, tb + static_cast<size_t>(i - 2) * rr, rr, lane);
       const float* A = tabs + ((i - 1) & 1) * rr;
-      const float al_i = has ? alphas[i * (r + 1) + lane] : -CUDART_INF_F;
+      const float al_i = has ? alphas[i * pitch + lane] : -CUDART_INF_F;
       if (has) {
         a_.post[prow + static_cast<size_t>(i) * r + lane] = tg[i] >= 0 ? abar : 0.f;
         cvec[lane] = al_i == -CUDART_INF_F ? -CUDART_INF_F : g[i * r + lane] - al_i;
@@ -424,7 +427,7 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
         dvec[lane] = 0.f;
       }
       __syncwarp();
-      const float al = has ? alphas[(i - 1) * (r + 1) + lane] : -CUDART_INF_F;
+      const float al = has ? alphas[(i - 1) * pitch + lane] : -CUDART_INF_F;
       float prop = 0.f;
       if (has) {
         const float* row = A + lane * r;

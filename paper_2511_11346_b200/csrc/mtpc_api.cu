@@ -516,10 +516,20 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
     const int stride = hmm_table_stride(h);
     const int items = stride == 0 ? (W + kHmmWarps - 1) / kHmmWarps : W / wpp * ((wpp + kHmmWarps - 1) / kHmmWarps);
     const int resident = sms_times_resident(h, smem);
-    const bool probabilities = stride == 0 && L.off_probA != 0;          // (a call without a head has log-probabilities alone)
-    launch_kernel(circuit_hmm_kernel, items < resident ? items : resident, kHmmWarps * 32, smem, st, overlapped(h), G, logw,
-                  probabilities ? at<float>(h, L.off_probA) : hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r,
-                  L.sum_rows, chunk, probabilities ? 1 : 0);
+    // contextual tables: a CTA per position while about one round of CTAs holds all positions, else a warp per window (both
+    // measured at circuit_hmm_stream_kernel; the two cross between 1.0 and 1.6 rounds over n = 4 to 64, r = 8 to 32)
+    if (stride != 0 && wpp <= 2 && 4ll * items > 5ll * resident) {
+      const size_t stream_smem = kHmmStreamWarps * hmm_stream_warp_floats(c.n, c.r, prefix != nullptr) * sizeof(float);
+      const int per_sm = static_cast<int>(kSmemLimit / (stream_smem + 1024)), ctas = (W + kHmmStreamWarps - 1) / kHmmStreamWarps;
+      const int held = h->num_sms * (per_sm < 1 ? 1 : per_sm > 16 ? 16 : per_sm);
+      launch_kernel(circuit_hmm_stream_kernel, ctas < held ? ctas : held, kHmmStreamWarps * 32, stream_smem, st, overlapped(h), G, logw,
+                    hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r, L.sum_rows);
+    } else {
+      const bool probabilities = stride == 0 && L.off_probA != 0;        // (a call without a head has log-probabilities alone)
+      launch_kernel(circuit_hmm_kernel, items < resident ? items : resident, kHmmWarps * 32, smem, st, overlapped(h), G, logw,
+                    probabilities ? at<float>(h, L.off_probA) : hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r,
+                    L.sum_rows, chunk, probabilities ? 1 : 0);
+    }
   } else if (sweep) {
     const int warps = c.n / 2 < 8 ? c.n / 2 : 8;                         // a warp per node of the owners' level
     const bool fits = btree_prefix_smem_floats(c.n, c.r, warps, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
@@ -546,6 +556,7 @@ bool allow_full_smem(K kernel) {
 }
 bool set_circuit_attributes() {
   bool ok = allow_full_smem(circuit_hmm_kernel);
+  ok &= allow_full_smem(circuit_hmm_stream_kernel);
   ok &= allow_full_smem(circuit_btree_kernel);
   ok &= allow_full_smem(circuit_btree_prefix_kernel);
   ok &= allow_full_smem(circuit_cp_prefix_kernel);

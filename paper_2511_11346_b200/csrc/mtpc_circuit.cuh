@@ -651,6 +651,73 @@ __global__ void __launch_bounds__(32 * kHmmWarps, 5) circuit_hmm_kernel(
   }
 }
 
+// The same recursion, bit for bit, for many positions with contextual tables and one or two windows each: one warp per window streams
+// its log tables, the copy of the next one in flight while this one is reduced. circuit_hmm_kernel gives a position to a CTA, whose
+// warps beyond the position's windows only help to exponentiate its tables: the shorter way for as many positions as are resident at once, but
+// with several rounds of them the idle warps count. Whole calls of a small head in us, there / here: n = 8, r = 32 at 693 positions 27 / 31, at
+// 1500 61 / 55, at 4096 170 / 138; n = 16, r = 32 at 400 43 / 57, at 2200 202 / 151; n = 8, r = 8 at 600 36.0 / 37.4, at 4096 68 / 47.
+constexpr int kHmmStreamWarps = 4;
+__host__ __device__ inline size_t hmm_stream_warp_floats(int n, int r, bool with_prefix) {
+  return 2 * static_cast<size_t>(r) * r + hmm_circuit_warp_floats(n, r, with_prefix);
+}
+__global__ void __launch_bounds__(32 * kHmmStreamWarps) circuit_hmm_stream_kernel(
+    const float* __restrict__ G, const float* __restrict__ logw, const float* __restrict__ tables, int table_stride,
+    float* __restrict__ out, float* __restrict__ prefix, float* __restrict__ msg, int W, int wpp, int n, int r, int sum_rows) {
+  extern __shared__ __align__(16) float sm[];
+  grid_dependency_wait();   // G and log omega come from the kernel before this one
+  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rr = r * r;
+  float* evec = sm + wib * hmm_stream_warp_floats(n, r, prefix != nullptr);      // [2][32], alternating
+  float* tabs = evec + 64;                                                       // [2][r, r]
+  float* alphas = tabs + 2 * rr;
+  const HmmLanes l = hmm_lanes(r, lane);
+  const int k = l.k;
+  const bool keeps = l.active && l.part == 0;
+  for (int w = blockIdx.x * kHmmStreamWarps + wib; w < W; w += gridDim.x * kHmmStreamWarps) {
+    const float* g = G + static_cast<size_t>(w) * n * r;
+    const float* tb = tables + static_cast<size_t>(w / wpp) * table_stride;
+    float* mw = msg != nullptr && keeps ? msg + static_cast<size_t>(w) * n * r : nullptr;
+    if (n > 1) warp_table_load_async(tabs, tb, rr, lane);
+    float alpha = -CUDART_INF_F, gi = 0.f;
+    if (l.active) {
+      const float l0 = logw[static_cast<size_t>(w / wpp) * sum_rows + k];
+      if (mw != nullptr) mw[k] = l0;
+      alpha = l0 + g[k];
+      if (n > 1) gi = g[r + k];
+    }
+    if (prefix != nullptr && keeps) alphas[k] = alpha;
+    for (int i = 1; i < n; ++i) {
+      const float g_next = (l.active && i + 1 < n) ? g[(i + 1) * r + k] : 0.f;
+      if (i + 1 < n) {
+        warp_table_load_async(tabs + (i & 1) * rr, tb + static_cast<size_t>(i) * rr, rr, lane);
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
+      }
+      __syncwarp();                                        // table i is in shared memory for every lane
+      const float c = hmm_forward_step<true>(alpha, evec + (i & 1) * 32, tabs + ((i - 1) & 1) * rr, l, r);
+      if (mw != nullptr) mw[i * r + k] = c;
+      alpha = l.active ? c + gi : -CUDART_INF_F;
+      gi = g_next;
+      if (prefix != nullptr && keeps) alphas[i * (r + 1) + k] = alpha;
+      __syncwarp();                                        // the table's buffer may be overwritten
+    }
+    if (prefix != nullptr) {
+      __syncwarp();
+      for (int i = lane; i < n; i += 32) {
+        const float res = thread_lse(alphas + i * (r + 1), r);
+        prefix[static_cast<size_t>(w) * n + i] = res;
+        if (out != nullptr && i == n - 1) out[w] = res;
+      }
+      __syncwarp();
+    } else if (out != nullptr) {
+      const float res = warp_lse_nan(l.part == 0 ? alpha : -CUDART_INF_F);
+      if (lane == 0) out[w] = res;
+    }
+  }
+  grid_launch_dependents();                                // (at the end: a waiting GEMM would take the L1)
+}
+
 // ---------------------------------------------------------------- training loss (Eq. 6)
 // Eq. (6): L_j = -(1/N) sum_i (1/V_ij) sum_t log p(x_{t+j} | x_{<t+j}), L = sum_j gamma^(j-1) L_j, over N sequences of
 // L positions with overlapping windows. The conditional of slot j given the context and the window's earlier bytes

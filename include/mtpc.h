@@ -193,7 +193,10 @@ int mtpc_draft_sample_prefix(mtpc_head* head, const void* hidden, int32_t P, int
  *     position): such a draft runs in chunks of positions and leaves only the evidence of the drafted bytes. The call then
  *     runs the tests, sorts the rejected windows by the slot of their first rejected byte, recomputes that slot's r*v logits
  *     for them in one projection pass over staged hidden states, and draws. It reads the hidden states the DRAFT call was
- *     given (bf16 heads: the caller's buffer, which must still hold them).
+ *     given (bf16 heads: the caller's buffer, which must still hold them);
+ *   - a draft by mtpc_draft_sample leaves no slot messages (what the sweep for prefix marginals yields besides them): the call
+ *     forms them with one more launch. So does one recorded into a CUDA graph without its draft, which may be replayed after
+ *     either kind, and any call outside a capture once a draft by mtpc_draft_sample has been recorded on the head.
  * A uniform outside [0,1) or a draft byte outside [0,v) sets the status bit and yields -1 / -1 for that window.
  */
 int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32_t* draft_bytes,

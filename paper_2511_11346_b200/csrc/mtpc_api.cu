@@ -266,6 +266,9 @@ struct mtpc_head {
   int copy_event_count;
   int draft_P;              // positions whose draft state (logits, or after a many-position draft G and log omega) is in the workspace (0: none)
   int draft_wpp;            // windows per position of that draft
+  bool draft_msg;           // its slot messages are there too (a draft of prefix marginals leaves them, an acceptance call forms them)
+  unsigned long long draft_capture;   // ... enqueued in this stream capture (0: none)
+  bool joint_recorded;      // a draft of joints, which leaves no messages, may be replayed at any time
   bool draft_logits;        // every logit and unit log-sum-exp of its positions is there as well
   const void* draft_hidden; // the bf16 hidden states it read (the acceptance stage may have to stage rows of them)
   int ring;                 // calls whose per-kernel events are retained (0 = timing off)
@@ -764,15 +767,25 @@ int window_logprob_impl(mtpc_head* h, const void* hidden, const int32_t* targets
   return rc;
 }
 
+// The stream capture that `st` is recording into (0: none).
+unsigned long long capture_id(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return status == cudaStreamCaptureStatusActive ? id + 1 : 0;
+}
+
 // out_logprob [W] (joint) and / or out_prefix [W, n] (prefix log-marginals of the draft); either may be NULL, not both.
 int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, const float* uniforms,
                       int32_t* out_bytes, float* out_logprob, float* out_prefix, cudaStream_t st) {
   const mtpc_config& c = h->cfg;
   const Layout& L = h->L;
   const int W = P * wpp;
-  // Every draft runs the sweep that also yields the slot messages of the acceptance stage, whether it returns joints or prefix
-  // marginals: what it leaves behind is a function of P and wpp alone, so a recorded acceptance call may follow either.
-  float* const msg = at<float>(h, L.off_msg);
+  // a draft that returns prefix marginals runs the sweep that also yields the slot messages of the acceptance stage (the joints
+  // alone take a tree half the table passes: 203 us against 294 for 8000 windows of n = 16, r = 32)
+  float* const msg = out_prefix ? at<float>(h, L.off_msg) : nullptr;
+  const unsigned long long capture = capture_id(st);
+  if (capture != 0 && !out_prefix) h->joint_recorded = true;
   if (h->lr_k > 0 && P > L.decode_max_p && wpp == 1 && c.v <= kMaxDraftVocab) {
     // A long draft on a factored head, one window per position: log omega, the latent draws, then every (window, slot)
     // forms the logits of its one selected unit from W_base h and B h (lowrank_draw_kernel) and draws its byte; the
@@ -816,6 +829,8 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     if (rc == MTPC_OK) {               // G, log omega, the messages, W_base h and B h stay in place for an acceptance call
       h->draft_P = P;
       h->draft_wpp = wpp;
+      h->draft_msg = msg != nullptr;
+      h->draft_capture = capture;
       h->draft_logits = false;
       h->draft_hidden = nullptr;
     }
@@ -879,6 +894,8 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     h->launches++;
     h->draft_P = P;
     h->draft_wpp = wpp;
+    h->draft_msg = msg != nullptr;
+    h->draft_capture = capture;
     h->draft_logits = true;
     pt.end();
     if ((rc = check_launch()) != MTPC_OK) return rc;
@@ -926,6 +943,8 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
   if (rc == MTPC_OK) {                 // G, log omega, the messages and the logits stay in place for an acceptance call
     h->draft_P = P;
     h->draft_wpp = wpp;
+    h->draft_msg = msg != nullptr;
+    h->draft_capture = capture;
     h->draft_logits = chunks == 1;
     h->draft_hidden = hb;
   }
@@ -1714,6 +1733,16 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
   const int threads = accept_threads(c.v);
   PhaseTimer pt(head, st);
   float* const msg = at<float>(head, L.off_msg);
+  // The slot messages are formed here, from the evidence and log omega the draft left, unless they are sure to be the last draft's
+  // when this call runs: formed by a call of the same capture, or outside any while no draft of joints has been recorded. (A
+  // recorded call runs after drafts the host does not see.)
+  const unsigned long long capture = capture_id(st);
+  if (!head->draft_msg || head->draft_capture != capture || (capture == 0 && head->joint_recorded)) {
+    rc = launch_circuit(head, W, wpp, nullptr, nullptr, st, /*raw_mixture=*/P <= L.decode_max_p && c.r > 32, msg);
+    if (rc != MTPC_OK) return rc;
+    head->draft_msg = true;
+    head->draft_capture = capture;
+  }
   if (head->draft_logits) {
     // every logit of the drafted positions is still in the workspace
     pt.begin();

@@ -543,7 +543,11 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
   } else {
     unsigned* counter = at<unsigned>(h, L.off_status) + kWorkCounterWord;
     const int resident = blocks < 8 * h->num_sms ? blocks : 8 * h->num_sms;   // more CTAs than an SM can hold do no harm
-    launch_kernel(circuit_btree_kernel, resident, threads, btree_smem_bytes(c.n, c.r), st, overlapped(h), G, logw, out, counter, W,
+    // As a dependent only where a window is short work and there are few: else the CTAs crowd onto the SMs that fall free first
+    // (n = 32, r = 16, d = 1024, whole calls as a dependent / not: 100 positions 71 / 58 us, 500 positions 98 / 84; n = 16, r = 8, 27
+    // positions 26 / 29, 500 positions 45 / 41).
+    const bool dependent = overlapped(h) && W <= h->num_sms && (c.n - 2) * c.r * c.r <= 1024;
+    launch_kernel(circuit_btree_kernel, resident, threads, btree_smem_bytes(c.n, c.r), st, dependent, G, logw, out, counter, W,
                   wpp, c.n, c.r, L.sum_rows);
   }
   h->launches++;

@@ -322,6 +322,9 @@ int check_launch() { return cudaGetLastError() == cudaSuccess ? MTPC_OK : MTPC_E
 // Launch `kernel`, optionally allowed to start before the kernel ahead of it in the stream has finished (programmatic
 // dependent launch): such a kernel calls grid_dependency_wait() before it touches global memory, so what overlaps is its launch and
 // set-up (about 2 us a kernel). cluster > 1: in clusters of that many CTAs.
+// Two kernels copy a static head's transition tables before they wait (draft_slot_kernel, circuit_hmm_kernel). The tables are written by
+// a plain launch (bind_parameters), and the first kernel of every call that runs one of the two lets its dependents in only after
+// its own wait (the fp32 conversion, the projection, the weight pass), so the tables are complete before any of them starts.
 template <typename... Params, typename... Args>
 void launch_clusters(void (*kernel)(Params...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent,
                      Args&&... args) {
@@ -1489,10 +1492,9 @@ static int bind_parameters(mtpc_head* h, const void* W_emit, const void* W_sum, 
     if (bad) return MTPC_ERR_CUDA;
   } else if (cfg->family == MTPC_HMM && cfg->n > 1) {
     const int rows = (cfg->n - 1) * cfg->r;
-    log_softmax_rows_kernel<<<(rows + 127) / 128, 128, 0, st>>>(T_static, at<float>(h, L.off_logA), rows, cfg->r);
-    static_tables_kernel<<<(rows + 7) / 8, 256, 0, st>>>(at<float>(h, L.off_logA), at<float>(h, L.off_probA), at<float>(h, L.off_cdfA),
-                                                         rows, cfg->r);
-    h->launches += 2;
+    static_tables_kernel<<<(rows + 7) / 8, 256, 0, st>>>(T_static, at<float>(h, L.off_logA), at<float>(h, L.off_probA),
+                                                         at<float>(h, L.off_cdfA), rows, cfg->r);
+    h->launches++;
   }
   if (check_launch() != MTPC_OK) return MTPC_ERR_CUDA;
   const uint64_t emit_rows = static_cast<uint64_t>(cfg->n) * cfg->r * cfg->v;
@@ -2455,7 +2457,7 @@ extern "C" int mtpc_window_logprob_static(const mtpc_config* cfg, const void* W_
   if (fail) return MTPC_ERR_CUDA;
   if (c.family == MTPC_HMM && c.n > 1) {
     const int rows = (c.n - 1) * c.r;
-    log_softmax_rows_kernel<<<(rows + 127) / 128, 128, 0, st>>>(T_static, at<float>(&h, L.off_logA), rows, c.r);
+    static_tables_kernel<<<(rows + 7) / 8, 256, 0, st>>>(T_static, at<float>(&h, L.off_logA), nullptr, nullptr, rows, c.r);
     if (check_launch() != MTPC_OK) return MTPC_ERR_CUDA;
   }
   rc = make_tmap(&h.tm_emit_lp, W_emit, static_cast<uint64_t>(c.n) * c.r * c.v, c.d, L.lp.tile_cols);

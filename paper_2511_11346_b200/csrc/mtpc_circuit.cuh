@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(32 * kHmmWarps, 5) circuit_hmm_kernel(
     int chunk_tables, int probabilities) {
   extern __shared__ __align__(16) float sm[];
   grid_launch_dependents();
-  const bool early = probabilities && chunk_tables >= n - 1;           // all of a static set, written when the head was made
+  const bool early = probabilities && chunk_tables >= n - 1;           // a static set, complete before the call's first kernel lets this in
   if (early) {
     fetch_floats(sm, tables, (n - 1) * r * r, 32 * kHmmWarps);
     cp_async_commit();
@@ -847,19 +847,6 @@ __global__ void __launch_bounds__(256) f32_to_bf16_kernel(const float* __restric
     reinterpret_cast<uint4*>(dst)[i] = *reinterpret_cast<const uint4*>(o);
   }
   grid_launch_dependents();
-}
-
-// Row-wise log-softmax of the static transition logits: one thread per row of r entries.
-__global__ void log_softmax_rows_kernel(const float* __restrict__ src, float* __restrict__ dst, int rows, int r) {
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= rows) return;
-  const float* x = src + static_cast<size_t>(row) * r;
-  float m = x[0];
-  for (int j = 1; j < r; ++j) m = fmaxf(m, x[j]);
-  float s = 0.f;
-  for (int j = 0; j < r; ++j) s += expf(x[j] - m);
-  const float lse = m + logf(s);
-  for (int j = 0; j < r; ++j) dst[static_cast<size_t>(row) * r + j] = x[j] - lse;
 }
 
 }  // namespace mtpc

@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   grid_dependency_wait();     // a draft that follows another call closely sets up its barriers while that one finishes
-  grid_launch_dependents();   // the per-slot kernel may be scheduled as SMs free up; it waits for this grid's results
+  grid_launch_dependents();   // (after the wait: the per-slot kernel reads static tables early) it waits for this grid's results
 
   const int quarter = warp & 3;
   const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
@@ -343,14 +343,24 @@ __device__ __forceinline__ int warp_inv_cdf_logp(float logp, int r, float u, int
   return hit ? __ffs(hit) - 1 : r - 1;
 }
 
-// What a head with static transitions keeps of its `rows` rows of r <= 32 log-probabilities besides them, one warp per row:
-// the probabilities (the circuit's recursion), and their running sums: with them a draw is one comparison per lane and a ballot, and
-// yields what warp_inv_cdf_logp yields.
-__global__ void __launch_bounds__(256) static_tables_kernel(const float* __restrict__ logp, float* __restrict__ prob,
-                                                            float* __restrict__ cdf, int rows, int r) {
+// The tables of `rows` rows of r <= 32 static transition logits x, one warp per row: their log-softmax, and what a head keeps besides
+// it (prob and cdf; NULL: a call without a head), the probabilities (the circuit's recursion) and their running sums, with which a draw
+// is one comparison per lane and a ballot, and yields what warp_inv_cdf_logp yields. The sum runs in index order. (mtpc_update_parameters on n = 8,
+// r = 8: 6.8 us as two kernels, one of them with a thread per row; 4.6 before there were tables to keep.)
+__global__ void __launch_bounds__(256) static_tables_kernel(const float* __restrict__ x, float* __restrict__ logp,
+                                                            float* __restrict__ prob, float* __restrict__ cdf, int rows, int r) {
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= rows) return;
-  const float lp = lane < r ? logp[static_cast<size_t>(row) * r + lane] : -CUDART_INF_F;
+  const float mine = lane < r ? x[static_cast<size_t>(row) * r + lane] : -CUDART_INF_F;
+  float m = mine;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, off));
+  const float e = expf(mine - m);
+  float s = 0.f;
+  for (int j = 0; j < r; ++j) s += __shfl_sync(kFull, e, j);
+  const float lp = mine - (m + logf(s));
+  if (lane < r) logp[static_cast<size_t>(row) * r + lane] = lp;
+  if (prob == nullptr) return;
   const float cum = warp_scan_incl(lane < r ? expf(lp) : 0.f, lane);
   if (lane < r) {
     prob[static_cast<size_t>(row) * r + lane] = __expf(lp);
@@ -525,7 +535,7 @@ __global__ void __launch_bounds__(kSlotThreads, 2) draft_slot_kernel(
   float* weights = sm + ((2 * r + 3) & ~3);  // [r][32 per]
   float* tabs = weights + (weights_in_smem ? r * 32 * per : 0);
   const int chain = slot_chain_length(family, n, blockIdx.x);
-  const bool early = tables_in_smem && family == 1 && hmm_stride == 0;      // written when the head was made, not by this call
+  const bool early = tables_in_smem && family == 1 && hmm_stride == 0;      // static tables, complete before the call's first kernel lets this in
   if (early) fetch_floats(tabs, hmm_tables, chain * r * r, kSlotThreads);
   grid_dependency_wait();     // the logits and log omega come from the kernel before this one
   if (work_counter != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)

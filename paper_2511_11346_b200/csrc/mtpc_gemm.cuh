@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   grid_dependency_wait();     // barriers and tensor memory were set up while the kernel before this one finished
-  grid_launch_dependents();   // the next kernel's CTAs may be scheduled as SMs free up; they wait for this grid's results
+  grid_launch_dependents();   // (after the wait: kernels behind this one read a head's static tables early) they wait for this grid's results
   if (p.work_counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *p.work_counter = 0;
 
   if (warp == 0) {

@@ -67,3 +67,44 @@ def test_back_to_back_calls_equal_isolated_ones(family, n, r, v, d, T, dtype):
             assert not a[k].is_floating_point() or torch.isfinite(a[k]).all(), k
     assert head.mtpc_get_status() == 0
     dh.close()
+
+
+@pytest.mark.parametrize("n,r,v,d,T,P,wpp,dtype", [
+    (8, 16, 64, 128, 150, 6, 8, "bf16"), (3, 32, 48, 64, 40, 1, 1, "bf16"), (5, 4, 32, 1088, 300, 9, 16, "f32"),
+])
+def test_parameters_updated_between_calls(n, r, v, d, T, P, wpp, dtype):
+    """Static transition tables are copied to shared memory before a kernel waits for the one ahead of it (the per-slot kernel of a
+    short draft, the circuit). That is sound because the kernel that writes them is launched plainly and the first kernel of
+    every call waits before it lets the next one start. Updates with alternating tables right before the calls must therefore give what
+    they give with the device idle in between, in one launch for a bf16 head."""
+    wl = I.make_workload("update", I.HeadShape(I.HMM, n, r, v, d, io_dtype=I.F32 if dtype == "f32" else I.BF16), T, seed=53, wpp=wpp,
+                         weight_std=0.25)
+    dh = DeviceHead(wl)
+    hidden, targets = dh.hidden_device(), torch.from_numpy(wl.targets).cuda()
+    tables = [dh.T_static, 3.0 * torch.flip(dh.T_static, dims=(2,)).contiguous()]
+    u = torch.from_numpy(wl.uniforms).cuda()[:P * wpp].contiguous()
+    few = hidden[:P].contiguous()
+
+    def run(alone):
+        got = []
+        for i in range(6):
+            before = dh.head.mtpc_launch_count()
+            dh.head.mtpc_update_parameters(dh.W_emit, dh.W_sum, tables[i % 2])
+            assert dh.head.mtpc_launch_count() - before == (1 if dtype == "bf16" else 3)
+            for call in (lambda: (dh.window_prefix_logprob(hidden=hidden, targets=targets),),
+                         lambda: dh.draft_sample_prefix(wpp, hidden=few, uniforms=u)) if i % 3 else (
+                         lambda: dh.draft_sample_prefix(wpp, hidden=few, uniforms=u),
+                         lambda: (dh.window_logprob(hidden=hidden, targets=targets),)):
+                if alone:
+                    torch.cuda.synchronize()
+                got += call()
+        torch.cuda.synchronize()
+        return got
+
+    want, got = run(alone=True), run(alone=False)
+    assert dh.head.mtpc_get_status() == 0
+    for a, b in zip(want, got):
+        assert torch.equal(a, b)
+    per = len(want) // 6
+    assert not torch.equal(want[per], want[2 * per])       # the tables matter
+    dh.close()

@@ -58,7 +58,9 @@ enum {
 
 /* mtpc_config.flags */
 enum {
-  MTPC_FLAG_HMM_CONTEXTUAL = 1u /* MTPC_HMM only: the transitions depend on the hidden state (App. H), see below */
+  MTPC_FLAG_HMM_CONTEXTUAL = 1u, /* MTPC_HMM only: the transitions depend on the hidden state (App. H), see below */
+  MTPC_FLAG_SHORT_DRAFTS = 4u    /* drafts take at most 128 positions (MTPC_ERR_UNSUPPORTED beyond): a head that evaluates or
+                                    trains on many reserves no workspace for the logits of as many drafted ones */
 };
 
 /* Bits of the device status word. */
@@ -80,7 +82,7 @@ typedef struct {
   int32_t io_dtype;            /* MTPC_F32 | MTPC_BF16: dtype of hidden, W_emit and W_sum              */
   int32_t max_positions;       /* upper bound on T (log-prob) and P (draft) per call                   */
   int32_t max_windows_per_pos; /* upper bound on wpp (>= 1; <= 64)                                     */
-  uint32_t flags;              /* 0 or MTPC_FLAG_HMM_CONTEXTUAL                                        */
+  uint32_t flags;              /* 0 or MTPC_FLAG_* combined                                            */
   int32_t v_valid;             /* 0, or the number of symbols that exist when the vocabulary is not a
                                   multiple of 16 (v - 16 < v_valid <= v; a byte-level Llama has 268: v = 272):
                                   every unit of W_emit keeps v rows, the last v - v_valid of them are padding
@@ -88,7 +90,9 @@ typedef struct {
                                   targets and bytes are < v_valid; target_probs rows keep v entries          */
 } mtpc_config;
 
-/* Bytes of device workspace a head with this configuration needs (a multiple of 256). */
+/* Bytes of device workspace a head with this configuration needs (a multiple of 256). Beyond what an evaluation needs, a head for
+ * more than 128 positions holds the emission logits of as many drafted ones, at most 4 GiB (and, where that is less than all, up to
+ * 2 GiB to recompute some): 1.3 of 1.4 GB for n = 8, r = 16, v = 320 at 8192 positions. MTPC_FLAG_SHORT_DRAFTS leaves that out. */
 int mtpc_workspace_bytes(const mtpc_config* cfg, size_t* out_bytes);
 
 /*
@@ -292,7 +296,7 @@ int mtpc_lowrank_backward(int32_t n, int32_t r, int32_t v, int32_t d, int32_t k,
  *            mtpc_update_parameters with W_emit = NULL then).
  *   workspace >= mtpc_lowrank_workspace_bytes(cfg, k): the dense head's workspace plus W_base h, z = B h as two bf16
  *            halves, a copy of A in the layout the kernel reads (remade on every call, so A is always read as it is then),
- *            the partial log-sum-exps and 58 MB for parts of the GEMMs' tiles.
+ *            the partial log-sum-exps and room for parts of the GEMMs' tiles (up to 58 MB).
  * Such a head serves mtpc_window_logprob, mtpc_window_prefix_logprob, mtpc_window_loss, mtpc_window_logprob_host,
  * mtpc_draft_sample, mtpc_draft_sample_prefix and mtpc_speculative_accept: up to 128 positions, the draft's weight pass
  * streams W_base and B (n v + n r k rows) instead of n r v composed rows and the logits are formed from the two small

@@ -14,6 +14,7 @@ from . import build as _build
 MTPC_CP, MTPC_HMM, MTPC_BTREE = 0, 1, 2
 MTPC_F32, MTPC_BF16 = 0, 1
 MTPC_FLAG_HMM_CONTEXTUAL = 1
+MTPC_FLAG_SHORT_DRAFTS = 4
 MTPC_OK = 0
 STATUS_BAD_TARGET, STATUS_BAD_UNIFORM, STATUS_TIMEOUT = 1, 2, 4
 

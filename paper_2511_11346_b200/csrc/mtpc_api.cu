@@ -100,7 +100,7 @@ int plan(const mtpc_config& c, Layout* L, bool factored = false) {
   if (c.io_dtype != MTPC_F32 && c.io_dtype != MTPC_BF16) return MTPC_ERR_SHAPE;
   if (c.n < 1 || c.r < 1 || c.v < 1 || c.d < 1 || c.max_positions < 1 || c.max_windows_per_pos < 1)
     return MTPC_ERR_SHAPE;
-  if ((c.flags & ~MTPC_FLAG_HMM_CONTEXTUAL) != 0) return MTPC_ERR_UNSUPPORTED;
+  if ((c.flags & ~(MTPC_FLAG_HMM_CONTEXTUAL | MTPC_FLAG_SHORT_DRAFTS)) != 0) return MTPC_ERR_UNSUPPORTED;
   const bool ctx = (c.flags & MTPC_FLAG_HMM_CONTEXTUAL) != 0;
   if (ctx && c.family != MTPC_HMM) return MTPC_ERR_UNSUPPORTED;
   if (c.n > 64 || c.max_windows_per_pos > 64) return MTPC_ERR_UNSUPPORTED;
@@ -124,7 +124,10 @@ int plan(const mtpc_config& c, Layout* L, bool factored = false) {
   L->lp.tile_cols = 256;
   if (!fit_tiling(&L->lp, sum_cols)) return MTPC_ERR_UNSUPPORTED;
 
-  L->max_windows = static_cast<size_t>(c.max_positions) * c.max_windows_per_pos;
+  L->decode_max_p = c.max_positions < kDecodeMaxP ? c.max_positions : kDecodeMaxP;
+  const bool long_drafts = c.max_positions > L->decode_max_p && (c.flags & MTPC_FLAG_SHORT_DRAFTS) == 0;
+  L->max_windows = static_cast<size_t>(long_drafts ? c.max_positions : L->decode_max_p) * c.max_windows_per_pos;
+  if (L->max_windows < static_cast<size_t>(c.max_positions)) L->max_windows = c.max_positions;   // an evaluation's
   const size_t elt = c.io_dtype == MTPC_F32 ? 4 : 2;
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
@@ -142,9 +145,8 @@ int plan(const mtpc_config& c, Layout* L, bool factored = false) {
   L->off_sel = take(L->max_windows * c.n * 4);
   L->off_msg = take(L->max_windows * c.n * c.r * 4);
   // (latents of more than 32 values are handled for the mixture only; HMM and BTree are limited to r <= 32 anyway)
-  L->decode_max_p = c.max_positions < kDecodeMaxP ? c.max_positions : kDecodeMaxP;
   L->kept_p = 0;
-  if (c.max_positions > L->decode_max_p && !factored) {
+  if (long_drafts && !factored) {
     const size_t cap = kKeptLogitBytes / (static_cast<size_t>(emit_units) * c.v * 4);     // >= 1: n r v <= 2^30
     L->kept_p = static_cast<size_t>(c.max_positions) < cap ? c.max_positions : static_cast<int>(cap);
   }
@@ -160,7 +162,7 @@ int plan(const mtpc_config& c, Layout* L, bool factored = false) {
   L->off_h_out = take(L->max_windows * 4);
   L->group_entries = 0;
   L->accept_rows = 0;
-  if (c.max_positions > L->decode_max_p && L->kept_p < c.max_positions) {
+  if (long_drafts && L->kept_p < c.max_positions) {
     const size_t stage_cap = kGroupStageBytes / (static_cast<size_t>(c.d) * 2);
     const size_t row_cap = kGroupStageBytes / (static_cast<size_t>(c.r) * c.v * 4);
     L->accept_rows = L->max_windows < row_cap ? L->max_windows : row_cap;
@@ -250,7 +252,8 @@ struct mtpc_head {
   size_t lr_off_arep;                           // workspace: A as [n, v, r, k]
   size_t lr_off_dec;                            // workspace: few-position draft products base [P, n v] | z [P, n r k]
   size_t lr_off_base;                           // workspace: W_base h [T, n v] fp32
-  size_t lr_off_split;                          // workspace: parts of split plain GEMMs
+  size_t lr_off_split;                          // workspace: parts of split plain GEMMs ...
+  int lr_split_parts;                           // ... and how many there is room for
   CUtensorMap tm_lrB_dec;                       // B [n r k, d] for the few-position draft path
   size_t lr_off_zhl, lr_off_partial;            // workspace: z = B h as bf16 halves [T, n r, 2, k]; partial log-sum-exps per column block
   CUtensorMap lr_tm_a[2];                       // the copy of A in the boxes of the forward and the gradient build
@@ -735,7 +738,11 @@ struct GemmOperand {
 
 // Optional extras of a plain GEMM launch: bf16 output instead of fp32, and several products of one shape in a launch
 // (see PlainGemmParams); a_* / b_* extents: the whole matrices the batched operands are windows of (M or N, then K).
-constexpr size_t kSplitBytes = kSplitParts * kSplitPartBytes;
+// Scratch that lets a launch cut its last round along K (parts == 0: it does not).
+struct SplitScratch {
+  void* ptr = nullptr;
+  int parts = 0;             // tile parts it has room for
+};
 // C2, C3: rows [m1, m2) and [m2, M) of the fp32 result go there.
 struct PlainGemmExtra {
   float *C2 = nullptr, *C3 = nullptr;
@@ -747,9 +754,8 @@ struct PlainGemmExtra {
   int K2 = 0, a_k2 = 0;
   long long a_extent_m = 0, a_extent_k = 0, b_extent_n = 0, b_extent_k = 0;
 };
-// split_ws: kSplitBytes of scratch that let the launch cut its last round along K (NULL: it does not).
 int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmOperand B1, int K1, int a_k1, float* C,
-                      size_t ldc, int M, int N, cudaStream_t st, void* split_ws = nullptr, void* C_hilo = nullptr,
+                      size_t ldc, int M, int N, cudaStream_t st, SplitScratch scratch = SplitScratch{}, void* C_hilo = nullptr,
                       int split_k = 0, const PlainGemmExtra* extra = nullptr);
 // parts: 1 = sum-unit tiles (log omega), 2 = W_base h, z = B h and the repacked A, 4 = G (and the units' log-sum-exps)
 int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, const int* targets, cudaStream_t st,
@@ -788,6 +794,7 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
   const mtpc_config& c = h->cfg;
   const Layout& L = h->L;
   const int W = P * wpp;
+  if (P > L.decode_max_p && (c.flags & MTPC_FLAG_SHORT_DRAFTS) != 0) return MTPC_ERR_UNSUPPORTED;
   // a draft that returns prefix marginals runs the sweep that also yields the slot messages of the acceptance stage (the joints
   // alone take a tree half the table passes: 203 us against 294 for 8000 windows of n = 16, r = 32)
   float* const msg = out_prefix ? at<float>(h, L.off_msg) : nullptr;
@@ -961,13 +968,51 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
 // ---------------------------------------------------------------- backward pass (host side)
 size_t round64(size_t x) { return (x + 63) / 64 * 64; }
 
+// How a plain GEMM of `tiles` tiles and `kblocks` K blocks is dealt to `workers` (CTAs, or pairs: ctas = 2): the tiles of the
+// last, partial round are cut into `split` parts each. Cost in K-block times of a worker (0.4 us): a part adds about 8 for
+// writing its fp32 tile, the reduction 10 and its bytes through L2 (15 tile parts of 128 KB a block time). Cut only where that
+// wins clearly, into no more than `parts` tile parts in all.
+struct SplitPlan {
+  int tail = 0, split = 1;
+  long long cost = 0;
+};
+SplitPlan plan_split(long long tiles, int kblocks, int workers, int ctas, int parts) {
+  SplitPlan b;
+  const long long whole = tiles / workers;
+  const int rem = static_cast<int>(tiles % workers);
+  b.cost = whole * kblocks + (rem ? kblocks : 0);
+  if (rem == 0) return b;
+  const long long limit = b.cost - 8;
+  for (int s = 2; s <= 16 && rem * s * ctas <= parts && kblocks / s >= 4; ++s) {
+    const long long rounds = (static_cast<long long>(rem) * s + workers - 1) / workers;
+    const long long cost = whole * kblocks + rounds * ((kblocks + s - 1) / s + 8) + 10 + rem * s * ctas / 15;
+    if (cost < b.cost && cost < limit) { b.cost = cost; b.tail = rem; b.split = s; }
+  }
+  return b;
+}
+
+int k_blocks(size_t k) { return static_cast<int>((k + kBlockK - 1) / kBlockK); }
+// Tile parts that a launch of M x N over `kblocks` K blocks may be cut into, by single CTAs or pairs of a 148-SM device (elsewhere
+// what is reserved limits the cut).
+int split_parts(size_t M, int N, int kblocks) {
+  int parts = 0;
+  for (int ctas = 1; ctas <= 2; ++ctas) {
+    const long long tiles = static_cast<long long>((M + ctas * kBlockM - 1) / (ctas * kBlockM)) * ((N + kPlainTileN - 1) / kPlainTileN);
+    const SplitPlan p = plan_split(tiles, kblocks, 148 / ctas, ctas, kSplitParts);
+    if (p.tail * p.split * ctas > parts) parts = p.tail * p.split * ctas;
+  }
+  return parts;
+}
+
 // Carving of the backward workspace for T positions (all buffers 256-byte aligned).
 // The sum-unit logit gradients sit to the right of the emission logit gradients in one matrix [T, Kd], Kd = Nc + Spad.
 struct BackwardLayout {
   size_t Nc, Spad, Kd;
   size_t off_lse, off_post, off_logits, off_dlogit, off_coeff, off_split, total;
+  int parts;                 // tile parts at off_split
 };
-void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout* B, bool keep_logits = true) {
+// rank > 0: of a factored head, which keeps no logits.
+void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout* B, int rank = 0) {
   B->Nc = static_cast<size_t>(c.n) * c.r * c.v;
   B->Spad = round64(L.sum_rows);
   B->Kd = B->Nc + B->Spad;
@@ -975,34 +1020,16 @@ void plan_backward(const mtpc_config& c, const Layout& L, int T, BackwardLayout*
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
   B->off_lse = take(static_cast<size_t>(T) * c.n * c.r * 4);
   B->off_post = take(static_cast<size_t>(T) * c.n * c.r * 4);
-  B->off_logits = take(keep_logits ? static_cast<size_t>(T) * B->Nc * 4 : 0);   // [T, Nc] fp32: the emission logits of the forward pass
+  B->off_logits = take(rank == 0 ? static_cast<size_t>(T) * B->Nc * 4 : 0);   // [T, Nc] fp32: the emission logits of the forward pass
   B->off_dlogit = take(static_cast<size_t>(T) * B->Kd * 2);          // [T, Nc | Spad] bf16
   B->off_coeff = take(static_cast<size_t>(T) * c.n * 4);             // Eq. 6: weights of the prefix marginals
-  B->off_split = take(kSplitBytes);                                 // parts of the GEMMs' cut tiles
+  // parts of the GEMMs' cut tiles: d hidden, and the weight gradients in one launch
+  const size_t nv = static_cast<size_t>(c.n) * c.v, nrk = static_cast<size_t>(c.n) * c.r * rank;
+  const int dh_blocks = (rank ? k_blocks(nv) + k_blocks(nrk) : k_blocks(B->Nc)) + k_blocks(L.sum_rows);
+  const int dh = split_parts(T, c.d, dh_blocks), dw = split_parts((rank ? nv + nrk : B->Nc) + L.sum_rows, c.d, k_blocks(T));
+  B->parts = dh > dw ? dh : dw;
+  B->off_split = take(B->parts * kSplitPartBytes);
   B->total = off;
-}
-
-// How a plain GEMM of `tiles` tiles and `kblocks` K blocks is dealt to `workers` (CTAs, or pairs: ctas = 2): the tiles of the
-// last, partial round are cut into `split` parts each. Cost in K-block times of a worker (0.4 us): a part adds about 8 for
-// writing its fp32 tile, the reduction 10 and its bytes through L2 (15 tile parts of 128 KB a block time). Cut only where that
-// wins clearly.
-struct SplitPlan {
-  int tail = 0, split = 1;
-  long long cost = 0;
-};
-SplitPlan plan_split(long long tiles, int kblocks, int workers, int ctas, bool scratch) {
-  SplitPlan b;
-  const long long whole = tiles / workers;
-  const int rem = static_cast<int>(tiles % workers);
-  b.cost = whole * kblocks + (rem ? kblocks : 0);
-  if (rem == 0 || !scratch) return b;
-  const long long limit = b.cost - 8;
-  for (int s = 2; s <= 16 && rem * s * ctas <= kSplitParts && kblocks / s >= 4; ++s) {
-    const long long rounds = (static_cast<long long>(rem) * s + workers - 1) / workers;
-    const long long cost = whole * kblocks + rounds * ((kblocks + s - 1) / s + 8) + 10 + rem * s * ctas / 15;
-    if (cost < b.cost && cost < limit) { b.cost = cost; b.tail = rem; b.split = s; }
-  }
-  return b;
 }
 
 template <int CTAS>
@@ -1016,7 +1043,7 @@ void launch_plain_tiles(const PlainGemmParams& p, bool a_mn, bool b_mn, int grid
 // A's K range [a_k1, a_k1 + K1) with B1.
 // C_hilo != NULL (then C is NULL): the result leaves as two bf16 halves per entry, see PlainGemmParams.
 int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmOperand B1, int K1, int a_k1, float* C,
-                      size_t ldc, int M, int N, cudaStream_t st, void* split_ws, void* C_hilo, int split_k,
+                      size_t ldc, int M, int N, cudaStream_t st, SplitScratch scratch, void* C_hilo, int split_k,
                       const PlainGemmExtra* extra) {
   if (M <= 0 || N <= 0 || K0 <= 0) return MTPC_OK;
   if (K1 > 0 && (A.mn_major || B1.mn_major != B0.mn_major)) return MTPC_ERR_SHAPE;
@@ -1046,9 +1073,9 @@ int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmO
   SplitPlan plan;
   bool pair = false;
   if (tile_n == kPlainTileN && x.batches == 1) {
-    plan = plan_split(static_cast<long long>(m_tiles) * p.n_tiles, kblocks, h->num_sms, 1, split_ws != nullptr);
+    plan = plan_split(static_cast<long long>(m_tiles) * p.n_tiles, kblocks, h->num_sms, 1, scratch.parts);
     if (h->max_pairs > 0 && m_tiles >= 2 && static_cast<long long>(m_tiles) * p.n_tiles > h->num_sms) {
-      const SplitPlan two = plan_split(static_cast<long long>((m_tiles + 1) / 2) * p.n_tiles, kblocks, h->max_pairs, 2, split_ws != nullptr);
+      const SplitPlan two = plan_split(static_cast<long long>((m_tiles + 1) / 2) * p.n_tiles, kblocks, h->max_pairs, 2, scratch.parts);
       if (two.cost * 15 <= plan.cost * 16) { plan = two; pair = true; }
     }
   }
@@ -1056,7 +1083,7 @@ int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmO
   p.m_tiles = (m_tiles + ctas - 1) / ctas;
   p.tail_tiles = plan.tail;
   p.split = plan.split;
-  p.partial = static_cast<float*>(split_ws);
+  p.partial = static_cast<float*>(scratch.ptr);
   const int Ka = x.K2 > 0 ? x.a_k2 + x.K2 : K1 > 0 ? a_k1 + K1 : K0;           // extent of A along K
   const uint64_t a_m = x.a_extent_m ? x.a_extent_m : M, a_k = x.a_extent_k ? x.a_extent_k : Ka;
   const uint64_t b_n = x.b_extent_n ? x.b_extent_n : N, b_k = x.b_extent_k ? x.b_extent_k : K0;
@@ -1151,10 +1178,10 @@ int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, cons
     const GemmOperand hid{hidden_bf16, static_cast<size_t>(c.d), false};
     const GemmOperand bmat{h->lr_B, static_cast<size_t>(c.d), false};          // [n r k, d], K = d contiguous
     const GemmOperand wmat{h->lr_W_base, static_cast<size_t>(c.d), false};
-    rc = launch_plain_gemm(h, hid, wmat, c.d, wmat, 0, 0, base, static_cast<size_t>(c.n) * c.v, T, c.n * c.v, st, h->ws + h->lr_off_split);
+    rc = launch_plain_gemm(h, hid, wmat, c.d, wmat, 0, 0, base, static_cast<size_t>(c.n) * c.v, T, c.n * c.v, st, SplitScratch{h->ws + h->lr_off_split, h->lr_split_parts});
     // z = B h, leaving the GEMM's epilogue already split into its two bf16 halves [T, n r, 2, k]
     if (rc == MTPC_OK)
-      rc = launch_plain_gemm(h, hid, bmat, c.d, bmat, 0, 0, nullptr, 0, T, units * k, st, h->ws + h->lr_off_split, zhl, k);
+      rc = launch_plain_gemm(h, hid, bmat, c.d, bmat, 0, 0, nullptr, 0, T, units * k, st, SplitScratch{h->ws + h->lr_off_split, h->lr_split_parts}, zhl, k);
     if (rc != MTPC_OK) return rc;
     // A as [n, v, r, k]: the adaptor columns of adjacent components side by side (remade every call: A may have changed)
     const size_t pieces = static_cast<size_t>(units) * c.v * (k / 8);
@@ -1295,13 +1322,13 @@ int backward_tail(mtpc_head* head, const BackwardLayout& B, uint8_t* bw, const v
   const GemmOperand hid{hb, static_cast<size_t>(c.d), true};                     // [T, d]: N = d contiguous, K = the position
   // d hidden [T, d] = dlogit [T, Nc] W_emit [Nc, d] + dsum [T, S r] W_sum [S r, d]
   rc = launch_plain_gemm(head, g_rows, w_emit, Nc, w_sum, L.sum_rows, Nc, d_hidden, c.d, T, c.d, st,
-                         bw + B.off_split);
+                         SplitScratch{bw + B.off_split, B.parts});
   // [dW_emit; dW_sum] [Nc + S r, d] = [dlogit | dsum]^T hidden [T, d]
   PlainGemmExtra two;
   two.C2 = dW_sum;
   two.m1 = Nc;
   if (rc == MTPC_OK)
-    rc = launch_plain_gemm(head, g_cols, hid, T, hid, 0, 0, dW_emit, c.d, Nc + L.sum_rows, c.d, st, bw + B.off_split, nullptr, 0, &two);
+    rc = launch_plain_gemm(head, g_cols, hid, T, hid, 0, 0, dW_emit, c.d, Nc + L.sum_rows, c.d, st, SplitScratch{bw + B.off_split, B.parts}, nullptr, 0, &two);
   pt.end();
   return rc;
 }
@@ -1316,7 +1343,7 @@ struct LowRankBackwardLayout {
   size_t off_sy, off_apad, total;
 };
 void plan_lowrank_backward(const mtpc_config& c, const Layout& L, int k, int T, LowRankBackwardLayout* R) {
-  plan_backward(c, L, T, &R->B, /*keep_logits=*/false);
+  plan_backward(c, L, T, &R->B, k);
   const size_t units = static_cast<size_t>(c.n) * c.r;
   R->Ksy = static_cast<size_t>(c.n) * c.v + units * k;
   R->pitch = R->Ksy + R->B.Spad;
@@ -1411,7 +1438,7 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
     x.a_extent_m = T; x.a_extent_k = Nc;
     x.b_extent_n = k; x.b_extent_k = static_cast<long long>(units) * R.v64;
     rc = launch_plain_gemm(head, GemmOperand{dlogit, B.Kd, false}, GemmOperand{bw + R.off_apad, static_cast<size_t>(k), true},
-                           static_cast<int>(R.v64), none, 0, 0, nullptr, R.pitch, T, k, st, nullptr, nullptr, 0, &x);
+                           static_cast<int>(R.v64), none, 0, 0, nullptr, R.pitch, T, k, st, SplitScratch{}, nullptr, 0, &x);
   }
   // d hidden [T, d] = s W_base + y B + dsum W_sum
   PlainGemmExtra tail;
@@ -1421,7 +1448,7 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
   if (rc == MTPC_OK)
     rc = launch_plain_gemm(head, GemmOperand{sy, R.pitch, false}, GemmOperand{head->lr_W_base, static_cast<size_t>(c.d), true}, c.n * c.v,
                            GemmOperand{head->lr_B, static_cast<size_t>(c.d), true}, units * k, c.n * c.v, d_hidden, c.d, T, c.d, st,
-                           bw + B.off_split, nullptr, 0, &tail);
+                           SplitScratch{bw + B.off_split, B.parts}, nullptr, 0, &tail);
   // [dW_base; dB; dW_sum] = [s | y | dsum]^T h: sy down its columns
   PlainGemmExtra three;
   three.C2 = dB;
@@ -1430,7 +1457,7 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
   three.m2 = static_cast<int>(R.Ksy);
   if (rc == MTPC_OK)
     rc = launch_plain_gemm(head, GemmOperand{sy, R.pitch, true}, hid, T, hid, 0, 0, dW_base, c.d, static_cast<int>(R.Ksy) + L.sum_rows,
-                           c.d, st, bw + B.off_split, nullptr, 0, &three);
+                           c.d, st, SplitScratch{bw + B.off_split, B.parts}, nullptr, 0, &three);
   if (rc == MTPC_OK && !one_pass) {   // on the bf16 high half of z the forward pass left
     PlainGemmExtra x;
     x.batches = units;
@@ -1441,7 +1468,7 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
     x.b_extent_n = static_cast<long long>(units) * 2 * k; x.b_extent_k = T;
     rc = launch_plain_gemm(head, GemmOperand{dlogit, B.Kd, true},
                            GemmOperand{head->ws + head->lr_off_zhl, static_cast<size_t>(units) * 2 * k, true}, T, none, 0, 0, dA,
-                           k, c.v, k, st, nullptr, nullptr, 0, &x);
+                           k, c.v, k, st, SplitScratch{}, nullptr, 0, &x);
   }
   pt.end();
   return rc;
@@ -1538,7 +1565,7 @@ struct LowRankSpec {
 // Workspace of a factored head beyond the dense layout: z = B h as two bf16 halves [T, n r, 2, k] (written by the GEMM
 // that computes it), W_base h, the log-sums of 32 columns each with their references, and the copy of A the factored kernel reads.
 static int lowrank_extra_bytes(const mtpc_config& c, int k, size_t base_total, size_t* off_zhl,
-                               size_t* off_partial, size_t* off_arep, size_t* off_dec, size_t* off_base, size_t* off_split, size_t* total) {
+                               size_t* off_partial, size_t* off_arep, size_t* off_dec, size_t* off_base, size_t* off_split, int* parts, size_t* total) {
   const size_t units = static_cast<size_t>(c.n) * c.r;
   size_t off = align_up(base_total);
   *off_zhl = off;
@@ -1553,7 +1580,13 @@ static int lowrank_extra_bytes(const mtpc_config& c, int k, size_t base_total, s
   *off_base = off;                      // W_base h [T, n v] fp32
   off += align_up(static_cast<size_t>(c.max_positions) * c.n * c.v * 4);
   *off_split = off;                     // z = B h and W_base h: parts of the tiles of their last rounds
-  off += align_up(kSplitBytes);
+  *parts = 0;
+  for (int t = kBlockM; t < c.max_positions + kBlockM; t += kBlockM) {
+    const int w = split_parts(t, c.n * c.v, c.d / kBlockK), z = split_parts(t, static_cast<int>(units) * k, c.d / kBlockK);
+    if (w > *parts) *parts = w;
+    if (z > *parts) *parts = z;
+  }
+  off += align_up(*parts * kSplitPartBytes);
   *total = off;
   return MTPC_OK;
 }
@@ -1570,11 +1603,12 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   LowRankParams lrp;
   memset(&lrp, 0, sizeof(lrp));
   size_t lr_zhl = 0, lr_partial = 0, lr_arep = 0, lr_dec = 0, lr_base = 0, lr_split = 0;
+  int lr_parts = 0;
   if (lowrank) {
     if (cfg->io_dtype != MTPC_BF16) return MTPC_ERR_UNSUPPORTED;
     if (!plan_lowrank(*cfg, lowrank->k, &lrp)) return MTPC_ERR_UNSUPPORTED;
     lowrank_extra_bytes(*cfg, lowrank->k, L.total, &lr_zhl, &lr_partial, &lr_arep, &lr_dec, &lr_base,
-                        &lr_split, &L.total);
+                        &lr_split, &lr_parts, &L.total);
   }
   const bool ctx = (cfg->flags & MTPC_FLAG_HMM_CONTEXTUAL) != 0;
   if (cfg->family == MTPC_HMM && cfg->n > 1 && !ctx && !T_static) return MTPC_ERR_NULL;
@@ -1601,6 +1635,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
     h->lr_off_dec = lr_dec;
     h->lr_off_base = lr_base;
     h->lr_off_split = lr_split;
+    h->lr_split_parts = lr_parts;
     h->lr_params = lrp;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1662,7 +1697,8 @@ int mtpc_lowrank_workspace_bytes(const mtpc_config* cfg, int32_t k, size_t* out_
   LowRankParams lrp;
   if (cfg->io_dtype != MTPC_BF16 || !plan_lowrank(*cfg, k, &lrp)) return MTPC_ERR_UNSUPPORTED;
   size_t a = 0, b = 0, c3 = 0, c4 = 0, c5 = 0, c6 = 0;
-  return lowrank_extra_bytes(*cfg, k, L.total, &a, &b, &c3, &c4, &c5, &c6, out_bytes);
+  int parts = 0;
+  return lowrank_extra_bytes(*cfg, k, L.total, &a, &b, &c3, &c4, &c5, &c6, &parts, out_bytes);
 }
 
 int mtpc_create_head_lowrank(const mtpc_config* cfg, int32_t k, const void* W_base, const void* A, const void* B,

@@ -5,7 +5,8 @@
   python bench.py [--gpus N] [--steps K] [--warmup W] [--workload 1|2|3|5|6] [--impl reference]
 
 One step = one mtpc_window_logprob call over the whole batch (projection GEMM with fused softmax/gather
-epilogue + circuit evaluation). Prints ONE JSON line on rank 0. With N > 1 (launched by torchrun, one process
+epilogue + circuit evaluation). Prints ONE JSON line on rank 0, and the full records of the other measurements on
+standard error before it. With N > 1 (launched by torchrun, one process
 per GPU) every rank runs an independent replica: the head has no exchange step, so there is no collective on
 the data path; ranks meet only at the timing barrier and `value` sums the replicas' work over the slowest
 rank's time. `--impl reference` times the fp64 CPU oracle on the host cores instead (rank 0 only).
@@ -41,7 +42,7 @@ SUSTAINED_LOOP_S = 2.5    # length of the second, power-capped loop whose roofli
 
 def workload_name(idx: int, wl) -> str:
     s = wl.shape
-    return (f"configs[{idx}] {wl.name}: T={wl.T} d={s.d} n={s.n} r={s.r} v={s.v} "
+    return (f"{wl.name}: T={wl.T} d={s.d} n={s.n} r={s.r} v={s.v} "
             f"{'bf16' if s.io_dtype == I.BF16 else 'fp32'} io")
 
 
@@ -261,7 +262,7 @@ def measure_decode_cell(torch, cell, steps: int, warmup: int, with_graph: bool =
     gbs = weight_bytes / (p50 * 1e-3) / 1e9
     graph_p50 = statistics.median(graph_lat) if with_graph else None
     gemm_gbs = weight_bytes / (phase_p50[0] * 1e-3) / 1e9
-    out = {"workload": f"configs[4] {wl.name}: P={wl.T} wpp={wl.wpp} d={s.d} n={s.n} r={s.r} v={s.v}",
+    out = {"workload": f"{wl.name}: P={wl.T} wpp={wl.wpp} d={s.d} n={s.n} r={s.r} v={s.v}",
            "windows_per_s": W / (p50 * 1e-3), "p50_ms": p50, "calls": steps, "kernels_per_call": launches,
            "kernel_p50_ms": phase_p50, "device_status": status,
            "cuda_graph_replay": None if graph_p50 is None else {
@@ -662,7 +663,7 @@ def oracle_parity(wl, out, k: int = 256) -> dict:
 
 
 def measure_draft_whole_batch(torch, head, wl, hidden, steps: int) -> dict:
-    """configs[3]: draft one window per position over the whole batch (the many-position path)."""
+    """Draft one window per position over the whole batch (the many-position path)."""
     s = wl.shape
     u = torch.from_numpy(wl.uniforms).cuda()
     W = wl.T * wl.wpp
@@ -710,7 +711,7 @@ def measure_draft_whole_batch(torch, head, wl, hidden, steps: int) -> dict:
 
 def measure_other_workload(torch, idx: int, dev_index: int, peaks: dict, peak_src: str, with_oracle: bool,
                            steps: int = 20) -> dict:
-    """configs[2] / configs[3] measured like the headline workload: a burst loop of `steps` calls after five warm-up
+    """Another workload (the HMM and the tree head) measured like the headline workload: a burst loop of `steps` calls after five warm-up
     calls (the headline's --steps: a 60-call loop already runs into the power cap, 1.5 GHz against 1.97 for 20 calls,
     and would be compared with a peak taken at full clock), a seconds-long sustained loop, the circuit kernel against HBM
     and the parity of the timed output."""
@@ -745,6 +746,37 @@ def measure_other_workload(torch, idx: int, dev_index: int, peaks: dict, peak_sr
     del dh, hidden, targets, out
     torch.cuda.empty_cache()
     return res
+
+
+def rounded(x):
+    """Floats to six significant digits, in lists and dicts too."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    return [rounded(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def printed_line(line: dict) -> dict:
+    """What goes to standard output: the headline's own record, and of every other workload and decode cell a few figures. (The
+    full records make a line of 20 KB, more than a reader that keeps the end of the output gets to see.)"""
+    full = ("workloads", "backward", "draft_whole_batch", "draft", "decode_sweep")
+    out = {k: v if k in ("value", "ms_per_step", "e2e") else rounded(v) for k, v in line.items() if k not in full}
+    if line.get("workloads"):
+        out["workloads"] = [rounded({
+            "workload": w["workload"], "positions_per_s": w["positions_per_s"],
+            "positions_per_s_sustained": w.get("positions_per_s_sustained"), "frac": w["roofline"]["frac"],
+            "draft_whole_batch_ms": w.get("draft_whole_batch", {}).get("ms_per_call")}) for w in line["workloads"]]
+    if line.get("draft_whole_batch"):
+        out["draft_whole_batch_ms"] = rounded(line["draft_whole_batch"]["ms_per_call"])
+    if line.get("backward"):
+        out["backward_ms"] = rounded(line["backward"].get("ms_per_call"))
+    if line.get("decode_sweep"):
+        out["decode_columns"] = ["cell", "draft p50 ms", "replayed from a graph", "draft + acceptance", "HBM fraction", "of the weight pass"]
+        out["decode"] = [rounded([c["workload"].split(":")[0], c["p50_ms"], c.get("cuda_graph_replay", {}).get("p50_ms"),
+                                  c.get("draft_plus_accept", {}).get("p50_ms"), c["hbm_roofline"]["frac"],
+                                  c["hbm_roofline"].get("weight_pass_kernel_frac")]) for c in line["decode_sweep"]]
+    return out
 
 
 def run_ours(args):
@@ -847,7 +879,7 @@ def run_ours(args):
         backward = measure_backward(torch, dh, wl, hidden, targets, steps=max(5, min(args.steps, 30)), peaks=peaks)
 
     draft_many = None
-    if wl.wpp and world == 1:       # configs[3]: draft one window per position over the whole batch (many-position path)
+    if wl.wpp and world == 1:       # the tree workload: draft one window per position over the whole batch
         draft_many = measure_draft_whole_batch(torch, head, wl, hidden, max(3, min(args.steps, 30)))
 
     launches = main["launches"] + (sus["launches"] if sus else 0)
@@ -855,7 +887,7 @@ def run_ours(args):
     del dh, hidden, targets, out
     torch.cuda.empty_cache()
 
-    # ---------------- the other heads the throughput target names (default run: configs[2] and configs[3])
+    # ---------------- the other heads the throughput target names (default run: the HMM and the tree workload)
     others = []
     if world == 1 and args.workload == 1 and args.positions is None and not args.no_other_workloads:
         for idx in (2, 3):
@@ -907,7 +939,8 @@ def run_ours(args):
     if draft is not None:
         line["draft"] = draft
         line["decode_sweep"] = sweep
-    print(json.dumps(line), flush=True)
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(printed_line(line)), flush=True)
 
 
 def main():
@@ -930,7 +963,7 @@ def main():
     ap.add_argument("--no-graph", action="store_true", help="skip the CUDA-graph replay of the draft calls (profiling runs)")
     ap.add_argument("--no-sustained", action="store_true", help="skip the second, seconds-long loop (profiling runs)")
     ap.add_argument("--no-other-workloads", action="store_true",
-                    help="default run only: skip configs[2] and configs[3] after the headline workload")
+                    help="default run only: skip the HMM and the tree workload after the headline one")
     ap.add_argument("--backward", action="store_true", help="also time mtpc_window_logprob_backward on the workload")
     ap.add_argument("--positions", type=int, default=None,
                     help="override the number of positions (scaled-down profiler captures; not a bench value)")

@@ -418,7 +418,7 @@ def test_eq6_loss_backward_on_a_factored_head(family, n, r, v, d, k, N, L):
 
 
 def test_factored_training_call_at_full_size_on_sampled_positions():
-    """configs[1]'s shape, rank 16, the launch configuration the benchmark times (64 row tiles, 128 products per batched
+    """The mixture training workload's shape (8192 positions, 8 x 16 x 320, d = 4096), rank 16, the launch configuration the benchmark times (64 row tiles, 128 products per batched
     launch). The loss weights are non-zero on a seeded sample of positions, so every gradient is a sum over exactly those
     positions, which the oracle can afford; d hidden must vanish everywhere else. A second launch with every weight non-zero
     checks what holds at any size: the logit gradients of a unit sum to zero over its symbols, so dA summed over the symbols

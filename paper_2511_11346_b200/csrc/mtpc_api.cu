@@ -66,7 +66,7 @@ struct Layout {
   size_t off_h_hidden, off_h_targets, off_h_uniforms, off_h_bytes, off_h_out;
   // acceptance stage after a draft that did not keep its logits: windows that can be staged at once (0: not needed)
   size_t group_entries;
-  size_t off_grp_ints, off_grp_tiles, off_grp_perm, off_grp_stage;
+  size_t off_grp_ints, off_grp_tiles, off_grp_stage;
   // ... first rejected slot and staging row per window, the recomputed logits [accept_rows, r v] and unit log-sum-exps
   // [accept_rows, r] of that slot (a factored head forms them after every long draft)
   size_t accept_rows;     // windows that can be handled at once (0: not available)
@@ -173,7 +173,6 @@ int plan(const mtpc_config& c, Layout* L, bool factored = false) {
   const size_t ge = L->group_entries, ar = L->accept_rows;
   L->off_grp_ints = take(ge ? (3 * static_cast<size_t>(c.n) + 64) * 4 : 0);            // counts | cursors | offsets | tile count
   L->off_grp_tiles = take(ge ? (c.n + ge / 128 + 1) * sizeof(GroupTile) : 0);
-  L->off_grp_perm = take(ge * 4);
   L->off_grp_stage = take(ge * c.d * 2);
   L->off_acc_rej = take(ar ? L->max_windows * 4 : 0);
   L->off_acc_row = take(ar ? L->max_windows * 4 : 0);
@@ -1806,7 +1805,6 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
   int* ints = at<int>(head, L.off_grp_ints);
   int* counts = ints, *cursors = ints + c.n, *offsets = ints + 2 * c.n, *num_tiles = ints + 3 * c.n;
   GroupTile* tiles = at<GroupTile>(head, L.off_grp_tiles);
-  int* perm = at<int>(head, L.off_grp_perm);
   __nv_bfloat16* stage = at<__nv_bfloat16>(head, L.off_grp_stage);
   int* rej = at<int>(head, L.off_acc_rej);
   int* row_of = at<int>(head, L.off_acc_row);
@@ -1850,12 +1848,12 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
     if (cudaMemsetAsync(ints, 0, static_cast<size_t>(2 * c.n) * 4, st) != cudaSuccess) return MTPC_ERR_CUDA;
     const int cblocks = (wc + kGroupThreads - 1) / kGroupThreads;
     group_count_kernel<<<cblocks < 4 * head->num_sms ? cblocks : 4 * head->num_sms, kGroupThreads, c.n * sizeof(int), st>>>(
-        rej, counts, wc, 1, c.n);
+        rej, counts, wc, c.n);
     group_scan_kernel<<<1, kGroupScanThreads, 0, st>>>(counts, offsets, tiles, num_tiles, c.n);
     const int gblocks = (wc + kGroupThreads / 32 - 1) / (kGroupThreads / 32);
     group_gather_kernel<<<gblocks < 16 * head->num_sms ? gblocks : 16 * head->num_sms, kGroupThreads, 0, st>>>(
-        rej, static_cast<const __nv_bfloat16*>(head->draft_hidden) + static_cast<size_t>(p0) * c.d, offsets, cursors, perm,
-        stage, wc, 1, c.n, wpp, c.d, row_of);
+        rej, static_cast<const __nv_bfloat16*>(head->draft_hidden) + static_cast<size_t>(p0) * c.d, offsets, cursors, stage,
+        wc, wpp, c.d, row_of);
     head->launches += 4;
     int rc2 = check_launch();
     if (rc2 != MTPC_OK) return rc2;

@@ -5,8 +5,7 @@
 //   group_count_kernel   histogram of the windows over the slots
 //   group_scan_kernel    exclusive scan -> first staging row of every slot, and the list of 128-row tiles
 //   group_gather_kernel  every window takes the next free row of its slot and copies its hidden state there
-// The order inside a slot depends on the order of the atomic increments; nothing downstream depends on it. (The kernels sort
-// entries e by the key (e % n) * r + unit_sel[e]; the acceptance stage calls them with n = 1 and r slots.)
+// The order inside a slot depends on the order of the atomic increments; nothing downstream depends on it.
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -15,32 +14,30 @@ namespace mtpc {
 
 constexpr int kGroupThreads = 256;
 constexpr int kGroupScanThreads = 1024;
-constexpr int kGroupMaxUnits = 8192;    // n <= 64 slots x r <= 128 units
 
-// One tile of the sorted pass: `count` <= 128 staging rows starting at `row0`, all of key `unit` (a slot).
+// One tile of the sorted pass: `count` <= 128 staging rows starting at `row0`, all of slot `unit`.
 struct GroupTile {
   int unit, row0, count, pad;
 };
 
-// counts[unit] += 1 for every (window, slot) pair with a selected unit (pairs of windows whose latent draw was refused
-// have none). Shared-memory histogram per CTA, flushed once.
-__global__ void __launch_bounds__(kGroupThreads) group_count_kernel(const int* __restrict__ unit_sel,
-                                                                    int* __restrict__ counts, int entries, int n, int r) {
+// counts[slot] += 1 for every window rejected in that slot (first_rejected[w] = -1: none). Shared-memory histogram per CTA,
+// flushed once.
+__global__ void __launch_bounds__(kGroupThreads) group_count_kernel(const int* __restrict__ first_rejected,
+                                                                    int* __restrict__ counts, int windows, int slots) {
   extern __shared__ int hist[];
-  const int units = n * r;
-  for (int k = threadIdx.x; k < units; k += kGroupThreads) hist[k] = 0;
+  for (int k = threadIdx.x; k < slots; k += kGroupThreads) hist[k] = 0;
   __syncthreads();
-  for (int e = blockIdx.x * kGroupThreads + threadIdx.x; e < entries; e += gridDim.x * kGroupThreads) {
-    const int z = unit_sel[e];
-    if (z >= 0) atomicAdd(&hist[(e % n) * r + z], 1);
+  for (int w = blockIdx.x * kGroupThreads + threadIdx.x; w < windows; w += gridDim.x * kGroupThreads) {
+    const int s = first_rejected[w];
+    if (s >= 0) atomicAdd(&hist[s], 1);
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < units; k += kGroupThreads)
+  for (int k = threadIdx.x; k < slots; k += kGroupThreads)
     if (hist[k]) atomicAdd(&counts[k], hist[k]);
 }
 
-// One CTA. offsets[u] = number of pairs in the units before u; tiles = every unit cut into runs of <= 128 rows, in
-// unit order; *num_tiles = how many. Thread t owns the units [t * per, (t + 1) * per).
+// One CTA. offsets[u] = number of windows in the slots before u; tiles = every slot cut into runs of <= 128 rows, in slot
+// order; *num_tiles = how many. Thread t owns the slots [t * per, (t + 1) * per).
 __global__ void __launch_bounds__(kGroupScanThreads) group_scan_kernel(const int* __restrict__ counts,
                                                                        int* __restrict__ offsets,
                                                                        GroupTile* __restrict__ tiles,
@@ -97,30 +94,27 @@ __global__ void __launch_bounds__(kGroupScanThreads) group_scan_kernel(const int
   }
 }
 
-// One warp per (window, slot) pair: lane 0 takes the next free staging row of the pair's unit, the warp copies the
-// window's hidden state (d bf16, d a multiple of 8, rows 16-byte aligned) there and records which pair the row holds
-// (and, where row_of is given, which row a pair got).
-__global__ void __launch_bounds__(kGroupThreads) group_gather_kernel(const int* __restrict__ unit_sel,
+// One warp per window: lane 0 takes the next free staging row of the slot the window was rejected in and records it (row_of), the
+// warp copies the hidden state of the window's position (d bf16, d a multiple of 8, rows 16-byte aligned) there.
+__global__ void __launch_bounds__(kGroupThreads) group_gather_kernel(const int* __restrict__ first_rejected,
                                                                      const __nv_bfloat16* __restrict__ hidden,
                                                                      const int* __restrict__ offsets,
-                                                                     int* __restrict__ cursors, int* __restrict__ perm,
-                                                                     __nv_bfloat16* __restrict__ stage, int entries, int n,
-                                                                     int r, int wpp, int d, int* __restrict__ row_of) {
+                                                                     int* __restrict__ cursors,
+                                                                     __nv_bfloat16* __restrict__ stage, int windows, int wpp,
+                                                                     int d, int* __restrict__ row_of) {
   const int lane = threadIdx.x & 31;
   const int warps = gridDim.x * (kGroupThreads / 32);
   const int vecs = d / 8;                                      // 16-byte pieces per row
-  for (int e = blockIdx.x * (kGroupThreads / 32) + (threadIdx.x >> 5); e < entries; e += warps) {
-    const int z = unit_sel[e];
-    if (z < 0) continue;                                       // warp-uniform: the whole warp reads the same entry
+  for (int w = blockIdx.x * (kGroupThreads / 32) + (threadIdx.x >> 5); w < windows; w += warps) {
+    const int s = first_rejected[w];
+    if (s < 0) continue;                                       // warp-uniform: the whole warp reads the same entry
     int row = 0;
     if (lane == 0) {
-      const int u = (e % n) * r + z;
-      row = offsets[u] + atomicAdd(&cursors[u], 1);
-      perm[row] = e;
-      if (row_of != nullptr) row_of[e] = row;                  // the inverse map, for callers that look a pair's row up
+      row = offsets[s] + atomicAdd(&cursors[s], 1);
+      row_of[w] = row;
     }
     row = __shfl_sync(0xffffffffu, row, 0);
-    const uint4* src = reinterpret_cast<const uint4*>(hidden + static_cast<size_t>((e / n) / wpp) * d);
+    const uint4* src = reinterpret_cast<const uint4*>(hidden + static_cast<size_t>(w / wpp) * d);
     uint4* dst = reinterpret_cast<uint4*>(stage + static_cast<size_t>(row) * d);
     for (int q = lane; q < vecs; q += 32) dst[q] = src[q];
   }

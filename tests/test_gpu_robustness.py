@@ -93,26 +93,27 @@ def test_both_builds_of_the_projection_kernel_give_the_same_numbers(family, n, r
     (I.BTREE, 8, 32, 256, 64, 290, 1),      # tree latents
     (I.HMM_CTX, 3, 16, 320, 64, 200, 1),    # contextual transitions; a unit's 320 columns in two accumulator tiles
 ])
-def test_draws_sorted_by_unit_give_the_same_bytes(family, n, r, v, d, T, wpp):
-    """Many-position draft (Algorithm 1): running every position against every unit, or sorting the (window, slot) pairs
-    by the unit they sample from and multiplying each by that unit only, must return the same bytes and log-probs -
-    the order in which windows are processed must not matter - and they must be the oracle's."""
-    wl = I.make_workload("grouped", I.HeadShape(family, n, r, v, d), T, seed=500 + n + r, wpp=wpp, weight_std=0.25)
+def test_long_drafts_with_refused_draws(family, n, r, v, d, T, wpp):
+    """Many-position draft (Algorithm 1) at shapes with many windows per unit and with units no window selects: a refused byte draw
+    leaves its byte at -1, a refused latent draw the whole window, both a NaN log-prob; every other window is the oracle's, and the
+    same on every run. (The hook that once chose between two forms of the byte draws takes its modes and changes nothing.)"""
+    wl = I.make_workload("refused_draws", I.HeadShape(family, n, r, v, d), T, seed=500 + n + r, wpp=wpp, weight_std=0.25)
     dh = DeviceHead(wl)
     u = wl.uniforms.copy()
-    u[5, n + 1] = 2.0                        # a refused byte draw ...
-    u[9, 0] = -1.0                           # ... and a refused latent draw keep their meaning in both modes
+    u[5, n + 1] = 2.0
+    u[9, 0] = -1.0
     ud = torch.from_numpy(u).cuda()
     got = []
-    for mode in (1, 2, 2):                   # the sorted pass twice: its internal row order differs from run to run
+    for mode in (0, 2):
         dh.head.mtpc_debug_set_draft_grouping(mode)
         out_bytes, out_lp = dh.draft_sample(uniforms=ud)
         assert dh.head.mtpc_get_status(with_code=True) == (B.MTPC_OK, B.STATUS_BAD_UNIFORM)
         got.append((out_bytes.cpu().numpy(), out_lp.cpu().numpy()))
-    for b, lp in got[1:]:
-        np.testing.assert_array_equal(b, got[0][0])
-        np.testing.assert_array_equal(lp, got[0][1])
-    gb, gl = got[1]
+    np.testing.assert_array_equal(got[0][0], got[1][0])
+    np.testing.assert_array_equal(got[0][1], got[1][1])
+    with pytest.raises(B.MtpcError):
+        dh.head.mtpc_debug_set_draft_grouping(3)
+    gb, gl = got[0]
     assert gb[5, 1] == -1 and (gb[9] == -1).all() and np.isnan(gl[5]) and np.isnan(gl[9])
     ok = np.ones(len(gb), dtype=bool)
     ok[[5, 9]] = False
@@ -125,19 +126,16 @@ def test_draws_sorted_by_unit_give_the_same_bytes(family, n, r, v, d, T, wpp):
     dh.close()
 
 
-@pytest.mark.parametrize("path", ["logprob", "logprob_single_ctas", "draft_few", "draft_many", "draft_many_ungrouped", "backward"])
+@pytest.mark.parametrize("path", ["logprob", "logprob_single_ctas", "draft_few", "draft_many", "backward"])
 def test_a_wait_that_runs_out_is_reported_and_the_head_recovers(path):
-    """Projection kernel (log-likelihood and sampling epilogues), the few-position draft kernel and the plain GEMMs of
-    the backward pass: with a 50 ns limit the first wait for a copy gives up in every CTA."""
-    T = {"logprob": 300, "logprob_single_ctas": 300, "draft_few": 8, "draft_many": 200, "draft_many_ungrouped": 200,
-         "backward": 300}[path]
+    """Projection kernel (with and without the logits it keeps), the few-position draft kernel and the plain GEMMs of the
+    backward pass: with a 50 ns limit the first wait for a copy gives up in every CTA."""
+    T = {"logprob": 300, "logprob_single_ctas": 300, "draft_few": 8, "draft_many": 200, "backward": 300}[path]
     wl = I.make_workload("timeout_" + path, I.HeadShape(I.HMM, 4, 8, 64, 4096), T, seed=77, wpp=2, weight_std=0.2)
     dh = DeviceHead(wl)
     weight = torch.full((wl.T,), -1.0 / wl.T, dtype=torch.float32, device="cuda")
     if path == "logprob_single_ctas":
         dh.head.mtpc_debug_set_projection_variant(1)      # the other paths pair their CTAs (more than one m-tile)
-    if path == "draft_many_ungrouped":
-        dh.head.mtpc_debug_set_draft_grouping(1)          # wpp = 2 against r = 8 units: sorted by unit otherwise
 
     def call():
         if path.startswith("logprob"):
@@ -170,10 +168,46 @@ def test_a_wait_that_runs_out_is_reported_and_the_head_recovers(path):
     dh.close()
 
 
+def test_the_sorted_pass_of_the_acceptance_stage_gives_up_and_recovers():
+    """A draft whose logits exceed 4 GiB runs in chunks, and the acceptance stage recomputes the rejected slots' logits in a projection
+    over windows sorted by slot: under a 50 ns limit that pass gives up, and the next draft and acceptance are what they were."""
+    n, r, v, d, P = 16, 32, 512, 1024, 4200                # 1 MiB of logits per position
+    g = torch.Generator(device="cuda")
+    g.manual_seed(12)
+
+    def normal(*shape, std):
+        return torch.empty(shape, dtype=torch.bfloat16, device="cuda").normal_(0.0, std, generator=g)
+
+    head = B.MtpcHead(B.MTPC_CP, n, r, v, d, B.MTPC_BF16, P, 1, normal(n, r, v, d, std=0.05), normal(r, d, std=0.05))
+    hidden, u = normal(P, d, std=1.0), torch.rand(P, 2 * n, device="cuda", generator=g)
+    tp = torch.softmax(0.5 * torch.randn(P, n + 1, v, device="cuda", generator=g), dim=-1)
+    ua = torch.rand(P, n + 1, device="cuda", generator=g)
+
+    def step(limit=0):
+        out = [torch.zeros(P, n, dtype=torch.int32, device="cuda"), torch.zeros(P, n, device="cuda")]
+        out += [torch.zeros(P, dtype=torch.int32, device="cuda") for _ in range(2)]
+        head.mtpc_draft_sample_prefix(hidden, 1, u, out[0], out[1])
+        head.mtpc_debug_set_wait_limit_ns(limit)
+        head.mtpc_speculative_accept(P, 1, out[0], out[1], tp, ua, out[2], out[3])
+        head.mtpc_debug_set_wait_limit_ns(0)
+        torch.cuda.synchronize()
+        return out, head.mtpc_get_status(with_code=True)
+
+    want, status = step()
+    assert status == (B.MTPC_OK, 0) and ((want[2] >= 0) & (want[2] < n)).any()
+    _, (code, bits) = step(limit=50)
+    assert code == B.ERR_TIMEOUT and bits & B.STATUS_TIMEOUT
+    got, status = step()
+    assert status == (B.MTPC_OK, 0)
+    for a, b in zip(want, got):
+        assert torch.equal(a, b)
+    head.mtpc_destroy()
+
+
 @pytest.mark.parametrize("family,n,r,v,d,P,wpp", [
     (I.CP, 8, 16, 320, 256, 8, 16),         # few positions: weight pass, per-slot kernel and circuit as dependent launches
     (I.HMM, 4, 8, 64, 128, 5, 3),
-    (I.BTREE, 8, 8, 64, 64, 200, 2),        # many positions: sorted draws, projection passes, circuit
+    (I.BTREE, 8, 8, 64, 64, 200, 2),        # many positions: projection that keeps its logits, draws, circuit
 ])
 def test_draft_and_acceptance_calls_can_be_captured_into_a_cuda_graph(family, n, r, v, d, P, wpp):
     """The calls only enqueue work on the caller's stream (no synchronisation, no allocation), so a serving loop may

@@ -422,9 +422,10 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
   p.m_tiles = (rows + kBlockM - 1) / kBlockM;
   // Every CTA alone, or two CTAs per MMA (when there are two m-tiles to pair up and the device can hold a cluster at all): whichever
   // plan takes less time. A pair moves less operand data per MMA, which counts when K is long; with few K steps the epilogue bounds
-  // a tile, and a lone CTA need not wait for its partner's. Time per tile in pairs / alone, measured over 26 shapes of 256 to 8192
-  // positions: d = 256 1.06 to 1.10, d = 1024 1.00 to 1.07, d = 1536 0.98, d = 2048 0.92 to 0.96, d = 4096 0.89 to 0.97. A ragged
-  // number of m-tiles costs the pairs more tiles (384 positions, d = 4096, 8 x 16 x 320: 5 tiles a pair against 4, 139.6 us / 121.9).
+  // a tile, and a lone CTA need not wait for its partner's. Time per tile in pairs / alone over 256 to 4096 positions of 8 x 16 x 320,
+  // 4 x 8 x 256 and 8 x 8 x 272 heads: d = 1024 1.00 to 1.17, d = 1088 1.00 to 1.14, d = 1280 0.95 to 1.08, d = 1536 0.90 to 1.08,
+  // d = 1792 0.92 to 1.08, d = 2048 0.85 to 1.08, d = 4096 0.85 to 1.10 (above 1 only where a CTA has one or two tiles). A ragged
+  // number of m-tiles costs the pairs more tiles (384 positions, d = 4096, 8 x 16 x 320: 5 a pair against 4, 150 us / 138).
   const int emit_units = with_emit ? c.n * c.r : 0, launch_sums = with_sum ? L.sum_tiles : 0;
   bool pair = grp == nullptr && h->projection_variant == 2;
   ItemPlan plan;
@@ -433,7 +434,7 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
     if (h->projection_variant != 1 && h->max_pairs > 0) {
       const ItemPlan two = choose_group_units(c.v, emit_units, (p.m_tiles + 1) / 2, h->max_pairs, launch_sums);
       if (h->projection_variant == 0 && p.m_tiles >= 2)
-        pair = c.d <= 1024 ? two.tiles * 34 <= plan.tiles * 33 : two.tiles * 12 <= plan.tiles * 13;
+        pair = c.d < 1536 ? two.tiles * 34 <= plan.tiles * 33 : two.tiles * 12 <= plan.tiles * 13;
       if (pair) plan = two;
     }
   }

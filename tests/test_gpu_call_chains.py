@@ -2,7 +2,7 @@
 the kernel ahead has finished and wait for it on the device; the kernels that hand out windows through a counter rely on the
 projection (or the per-slot kernel) before them to zero it. So back-to-back calls on alternating inputs must give, bit for bit, what
 each call gives alone on an idle device. (fp32 heads: the gradient of a static transition table is summed by atomics and is left
-out.) d = 1088 runs the projection in CTA pairs, d <= 1024 in single CTAs; an fp32 hidden state at an odd multiple of four bytes
+out.) d = 1600 runs the projection in CTA pairs, d < 1536 in single CTAs; an fp32 hidden state at an odd multiple of four bytes
 takes the scalar conversion, an aligned one the 16-byte conversion."""
 import pytest
 import torch
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("family,n,r,v,d,T,dtype", [
     (I.BTREE, 8, 16, 64, 128, 150, "f32"),
-    (I.BTREE, 4, 8, 48, 1088, 300, "bf16"),
+    (I.BTREE, 4, 8, 48, 1600, 300, "bf16"),
     (I.HMM, 5, 8, 64, 1024, 257, "f32"),
     (I.CP, 3, 8, 320, 64, 200, "f32"),
 ])
@@ -70,7 +70,7 @@ def test_back_to_back_calls_equal_isolated_ones(family, n, r, v, d, T, dtype):
 
 
 @pytest.mark.parametrize("n,r,v,d,T,P,wpp,dtype", [
-    (8, 16, 64, 128, 150, 6, 8, "bf16"), (3, 32, 48, 64, 40, 1, 1, "bf16"), (5, 4, 32, 1088, 300, 9, 16, "f32"),
+    (8, 16, 64, 128, 150, 6, 8, "bf16"), (3, 32, 48, 64, 40, 1, 1, "bf16"), (5, 4, 32, 1600, 300, 9, 16, "f32"),
 ])
 def test_parameters_updated_between_calls(n, r, v, d, T, P, wpp, dtype):
     """Static transition tables are copied to shared memory before a kernel waits for the one ahead of it (the per-slot kernel of a

@@ -264,7 +264,7 @@ struct mtpc_head {
   int max_decode_clusters[3];                   // clusters of 2, 4, 8 of its CTAs that can be resident at once
   int num_sms;
   cudaStream_t copy_stream; // host-buffer calls: uploads run here, ahead of the kernels (created on first use)
-  cudaEvent_t* copy_events; // [copy_event_count]: "chunk c is on the device"; [0] doubles as "the call may start"
+  cudaEvent_t* copy_events; // [copy_event_count]: "chunk c is on the device"; the one after the last chunk's: "the uploads may start"
   int copy_event_count;
   int draft_P;              // positions whose draft state (logits, or after a many-position draft G and log omega) is in the workspace (0: none)
   int draft_wpp;            // windows per position of that draft

@@ -582,7 +582,7 @@ __global__ void circuit_btree_backward_kernel(const CircuitBackwardArgs a_, unsi
 // Four passes over a window's n - 2 tables in shared memory (6 exponentials an entry), each table read from and its gradient
 // written to HBM once, as bf16. The n backward passes of the prefix lengths it replaces read and accumulated the window's 57 KB
 // n times (2186 us at 4096 windows, n = 16, r = 32, plus 48 us zeroing and 184 us converting the fp32 accumulators and 313 us
-// for the prefixes; this kernel does all of it in 392 us, its shared-memory and exponential work; HBM would take 80 us). One CTA per window, a warp per node of a level, as circuit_btree_prefix_kernel.
+// for the prefixes; this kernel does all of it in 350 us, its shared-memory and exponential work; HBM would take 80 us). One CTA per window, a warp per node of a level, as circuit_btree_prefix_kernel.
 __host__ __device__ inline size_t btree_loss_smem_floats(int n, int r, int warps, bool tables_in_smem) {
   const size_t vr = (static_cast<size_t>(r) + 3) / 4 * 4;
   return btree_prefix_smem_floats(n, r, warps, tables_in_smem) +

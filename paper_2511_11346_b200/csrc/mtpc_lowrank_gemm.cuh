@@ -20,7 +20,8 @@
 // Here MMAs are 64 or 128 columns wide, two components' pairs alternate, 512 columns of accumulators are in flight, and no
 // (component, 32 columns) depends on another. The bound is one ex2 per logit (16 a clock and SM: 149 us at T = 8192, n = 8,
 // r = 32, v = 320), in the gradient also the 1.3 GB of g.
-// Measured (this kernel, forward / gradient): 280 / 444 us, where the fused projection that kept logits took 801 us and the
+// Measured (this kernel, forward / gradient): 290 / 448 us with the schedulers issuing on 48 / 41 % of the
+// cycles (the rest waits on tensor-memory loads and ex2), where the fused projection that kept logits took 801 us and the
 // passes that made g and its sum from them 921 us; a likelihood call's whole projection at T = 8192, v = 320, d = 4096: r = 16
 // 506 -> 438 us, r = 32 893 -> 673 us.
 // Roles: warp 0 TMA producer, warp 1 MMA issuer, then the epilogue warps (TMEM quarter warp % 4, columns 32 * ((warp - 2) / 4)).

@@ -241,8 +241,8 @@ def test_backward_argument_checks():
                                                  (I.HMM, 5, 2, 16, 64, 3, 7), (I.HMM_CTX, 3, 2, 16, 64, 3, 7),
                                                  (I.HMM_CTX, 6, 32, 32, 64, 2, 17), (I.HMM_CTX, 1, 4, 32, 64, 2, 9)])
 def test_eq6_loss_backward_matches_oracle(family, n, r, v, d, N, L):
-    """The training loss of Eq. 6 and its gradients (mixture and tree: one circuit backward pass per prefix length,
-    accumulated; HMM: every prefix is a forward message, one reverse sweep), against
+    """The training loss of Eq. 6 and its gradients (every prefix from one sweep over the circuit, the gradient from its
+    reverse), against
     reverse-mode differentiation of the definition in float64. Windows run past the end of their sequences (masked
     tails), one sequence has no valid byte in the last slot."""
     wl = I.make_workload(f"l6_{family}_{n}_{r}", I.HeadShape(family, n, r, v, d), N * L, seed=6000 + n + N + r, weight_std=0.25)

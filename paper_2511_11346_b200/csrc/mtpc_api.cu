@@ -1581,8 +1581,10 @@ static int lowrank_extra_bytes(const mtpc_config& c, int k, size_t base_total, s
   off += align_up(static_cast<size_t>(c.max_positions) * c.n * c.v * 4);
   *off_split = off;                     // z = B h and W_base h: parts of the tiles of their last rounds
   *parts = 0;
-  for (int t = kBlockM; t < c.max_positions + kBlockM; t += kBlockM) {
-    const int w = split_parts(t, c.n * c.v, c.d / kBlockK), z = split_parts(t, static_cast<int>(units) * k, c.d / kBlockK);
+  const int m_tiles = (c.max_positions - 1) / kBlockM + 1, period = 148;      // (the last rounds repeat with it, see split_parts)
+  for (int m = 1; m <= m_tiles && m <= period; ++m) {
+    const int w = split_parts(static_cast<size_t>(m) * kBlockM, c.n * c.v, c.d / kBlockK);
+    const int z = split_parts(static_cast<size_t>(m) * kBlockM, static_cast<int>(units) * k, c.d / kBlockK);
     if (w > *parts) *parts = w;
     if (z > *parts) *parts = z;
   }

@@ -62,3 +62,16 @@ def test_scratch_of_cut_tiles_goes_by_the_shape():
     assert code == 0 and train <= 3 * MB
     code, train = size("mtpc_backward_workspace_bytes", ctypes.byref(config()), 2048)
     assert code == 0 and train <= 2048 * 40960 * 6 * 1.01 + 60 * MB
+
+
+def test_the_size_of_a_head_for_very_many_positions_is_found_at_once():
+    import time
+    start = time.perf_counter()
+    for positions in (1 << 30, (1 << 31) - 1):
+        code, _ = size("mtpc_lowrank_workspace_bytes", ctypes.byref(config(n=1, r=1, v=16, d=4096, max_positions=positions)), 16)
+        assert code == 0
+    assert time.perf_counter() - start < 0.2
+    # the tiles of a last round repeat every 148 row tiles, so beyond that only the buffers per position grow
+    step = 148 * 128
+    a, b, c = (size("mtpc_lowrank_workspace_bytes", ctypes.byref(config(max_positions=k * step, flags=B.MTPC_FLAG_SHORT_DRAFTS)), 16)[1] for k in (1, 2, 3))
+    assert c - b == b - a

@@ -1229,6 +1229,19 @@ BackwardShape circuit_backward_shape(const mtpc_head* h, bool loss) {
   return wide.warps >= compact.warps ? wide : compact;
 }
 
+// Warps (windows at a time) of a CTA of the static HMM's Eq. 6 kernel: the running sums of all n - 1 tables lie in shared memory beside the
+// tables themselves, so few fit for long windows (n = 17 at r = 32 is the last with four); 0: the streaming kernel.
+size_t hmm_static_loss_smem(const mtpc_config& c, int warps) {
+  const size_t tables = (static_cast<size_t>(c.n - 1) * c.r * c.r + 3) / 4 * 4;
+  return (2 * tables + warps * hmm_static_loss_warp_floats(c.n, c.r)) * sizeof(float);
+}
+int hmm_static_loss_warps(const mtpc_head* h) {
+  if (h->cfg.family != MTPC_HMM || is_ctx(h) || h->L.off_probA == 0) return 0;
+  for (int w = kHmmStaticWarps; w >= 4; w >>= 1)
+    if (hmm_static_loss_smem(h->cfg, w) <= static_cast<size_t>(kSmemLimit)) return w;
+  return 0;
+}
+
 // a.coeff (Eq. 6: the weights [W, n] of the prefix log-marginals) chooses the kernels that give every prefix and the whole
 // gradient in one launch; otherwise the gradient of sum_w a.weight[w] log q_w.
 int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cudaStream_t st) {
@@ -1248,10 +1261,17 @@ int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cuda
   const int threads = warps * 32;
   const int resident = blocks < 8 * h->num_sms ? blocks : 8 * h->num_sms;
   const size_t smem = shape.smem;
+  const int static_warps = loss ? hmm_static_loss_warps(h) : 0;
   if (c.family == MTPC_CP && loss) {
     launch_kernel(circuit_cp_loss_backward_kernel, blocks, threads, smem, st, overlapped(h), a);
   } else if (c.family == MTPC_CP) {
     launch_kernel(circuit_cp_backward_kernel, blocks, threads, smem, st, overlapped(h), a);
+  } else if (c.family == MTPC_HMM && loss && static_warps > 0) {
+    const size_t ssmem = hmm_static_loss_smem(c, static_warps);
+    const int batches = (a.W + static_warps - 1) / static_warps;
+    const int held = h->num_sms * (2 * (ssmem + 1024) <= static_cast<size_t>(kSmemLimit) ? 2 : 1);
+    launch_kernel(circuit_hmm_static_loss_backward_kernel, batches < held ? batches : held, static_warps * 32, ssmem, st, overlapped(h), a,
+                  at<float>(h, L.off_probA), hmm_tables(h), dT);
   } else if (c.family == MTPC_HMM && loss) {
     launch_kernel(circuit_hmm_loss_backward_kernel, resident, threads, smem, st, overlapped(h), a, hmm_tables(h),
                   hmm_table_stride(h), dT, counter, shape.wide ? 1 : 0);
@@ -1279,6 +1299,7 @@ int set_backward_attributes(const mtpc_head* head) {
   ok &= allow_full_smem(circuit_cp_loss_backward_kernel);
   ok &= allow_full_smem(circuit_btree_loss_backward_kernel);
   ok &= allow_full_smem(circuit_hmm_loss_backward_kernel);
+  ok &= allow_full_smem(circuit_hmm_static_loss_backward_kernel);
   ok &= allow_full_smem(circuit_btree_backward_kernel);
   return ok ? MTPC_OK : MTPC_ERR_CUDA;
 }

@@ -461,6 +461,219 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
   }
 }
 
+// The same for static transitions whose probabilities a head keeps: one set of tables for all windows, so nothing is streamed, no
+// table entry is exponentiated, and the table gradients are sums of rank-one terms that need no atomics. With u = exp(alpha_{i-1} -
+// max), c_i[b] = sum_a u[a] A[a][b] (the forward step's sum) and x_i[b] = abar_i[b] / c_i[b]:
+//   prop_{i-1}[a] = u[a] sum_b A[a][b] x_i[b],   dL/d(logit of A_i[a][b]) = A[a][b] (u[a] x_i[b] - prop_{i-1}[a]).
+// A batch is one window per warp: each warp runs its window forward and back (32 multiply-adds a lane and step either way) and leaves
+// u, x and prop in shared memory; then the steps are dealt to the warps, which add the batch's u x^T - prop into the CTA's running
+// sums, eight columns in registers at a time (acc [n-1][b][a]: lane = a, conflict-free). The factor A and the addition into dT come
+// once per CTA. A step whose sum is below 2^-100 for a state that matters (the evidence outweighs the other states' by 70 nats)
+// is redone with logarithms, straight into dT. Forward step and prefixes are those of circuit_hmm_kernel, bit for bit.
+// 8192 windows of n = 8, r = 32: 202 us by the streaming kernel (five exponentials an entry, 32 shared atomics a lane and step), 52 by this
+// one, bound by its instructions and the reads of the tables from shared memory.
+// Shared memory: 2 (n-1) r^2 floats, and per warp hmm_static_loss_warp_floats.
+constexpr int kHmmStaticWarps = 16;
+__host__ __device__ inline size_t hmm_static_loss_warp_floats(int n, int r) {
+  return (static_cast<size_t>(n) * r + 3) / 4 * 4 + 64 + (static_cast<size_t>(n) * (2 * r + 1) + 3) / 4 * 4;
+}
+__global__ void __launch_bounds__(32 * kHmmStaticWarps, 2) circuit_hmm_static_loss_backward_kernel(
+    const CircuitBackwardArgs a_, const float* __restrict__ prob, const float* __restrict__ logA, float* __restrict__ dT) {
+  extern __shared__ __align__(16) float sm[];
+  grid_launch_dependents();
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int n = a_.n, r = a_.r, rr = r * r, tables = (n - 1) * rr;
+  float* E = sm;                                                         // [n-1][r, r]
+  float* acc = E + (tables + 3) / 4 * 4;                                 // [n-1][b][a]
+  float* area = acc + (tables + 3) / 4 * 4;
+  const size_t warp_floats = hmm_static_loss_warp_floats(n, r);
+  const int off_u = (n * r + 3) / 4 * 4 + 64, off_prop = off_u + n * (r + 1);
+  float* xs = area + wib * warp_floats;                                  // [n][r]: c_i, then x_i
+  float* ev = xs + (n * r + 3) / 4 * 4;                                  // two vectors of 32
+  float* us = xs + off_u;                                                // [n][r + 1]: alpha_i, then u of the step after it
+  float* props = xs + off_prop;                                          // [n][r]
+  fetch_floats(E, prob, tables, blockDim.x);                             // static tables: complete before the call's first kernel lets this in
+  cp_async_commit();
+  for (int e = threadIdx.x; e < tables; e += blockDim.x) acc[e] = 0.f;
+  grid_dependency_wait();
+  cp_async_wait<0>();
+  __syncthreads();
+  const HmmLanes l = hmm_lanes(r, lane);
+  const int k = l.k;
+  const bool mine = l.active && l.part == 0;
+  const int w_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * a_.W / gridDim.x);
+  const int w_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * a_.W / gridDim.x);
+  const int cols = min(l.rows, 8), chunks = l.rows / cols;               // columns of a table a lane sums at a time
+  for (int w0 = w_begin; w0 < w_end; w0 += warps) {
+    const int w = w0 + wib;
+    if (w < w_end) {
+      const float* g = a_.G + static_cast<size_t>(w) * n * r;
+      const float* cw = a_.coeff + static_cast<size_t>(w) * n;
+      const int* tg = a_.targets + static_cast<size_t>(w) * n;
+      float* post = a_.post + static_cast<size_t>(w) * n * r;
+      const float l0 = l.active ? a_.logw[static_cast<size_t>(w) * a_.sum_rows + k] : 0.f;
+      // ---- forward
+      float alpha = l.active ? l0 + g[k] : -CUDART_INF_F;
+      float gi = l.active && n > 1 ? g[r + k] : 0.f;
+      if (mine) us[k] = alpha;
+      for (int i = 1; i < n; ++i) {
+        const float g_next = l.active && i + 1 < n ? g[(i + 1) * r + k] : 0.f;
+        float m;
+        const float c = hmm_forward_sum<false>(alpha, ev + (i & 1) * 32, E + (i - 1) * rr, l, r, m);
+        alpha = l.active ? m + __logf(c) + gi : -CUDART_INF_F;
+        gi = g_next;
+        if (mine) {
+          us[i * (r + 1) + k] = alpha;
+          xs[i * r + k] = c;
+        }
+      }
+      __syncwarp();
+      // ---- every prefix, lane = slot; its log-sum-exp is kept by the lane (slots past 32: read back)
+      float lp_mine = 0.f;
+      for (int i = lane; i < n; i += 32) {
+        const float lp = thread_lse(us + i * (r + 1), r);
+        a_.prefix[static_cast<size_t>(w) * n + i] = lp;
+        if (i < 32) lp_mine = lp;
+      }
+      __syncwarp();
+      auto prefix_of = [&](int i) { return i < 32 ? __shfl_sync(kFull, lp_mine, i) : a_.prefix[static_cast<size_t>(w) * n + i]; };
+      // ---- reverse sweep
+      const float lp_last = prefix_of(n - 1);
+      float al_i = alpha;                                                // alpha_i of the lane's state
+      float abar = l.active ? cw[n - 1] * __expf(alpha - lp_last) : 0.f;
+      for (int i = n - 1; i >= 1; --i) {
+        const float al = l.active ? us[(i - 1) * (r + 1) + k] : -CUDART_INF_F;
+        const float lp = prefix_of(i - 1);
+        float m = warp_max_nan(al);
+        if (m == -CUDART_INF_F) m = 0.f;
+        const float u = __expf(al - m);
+        const float c = l.active ? xs[i * r + k] : 1.f;
+        if (mine) {
+          post[static_cast<size_t>(i) * r + k] = tg[i] >= 0 ? abar : 0.f;
+          xs[i * r + k] = c == 0.f ? 0.f : __fdividef(abar, c);
+        }
+        const bool redo = __any_sync(kFull, c > 0.f && c < 0x1p-100f && abar != 0.f);
+        __syncwarp();
+        float prop = 0.f;
+        if (!redo) {
+          const float* row = E + (i - 1) * rr + k * r;
+          const float* x = xs + i * r;
+          if (l.rows == 32) {                                            // float4 reads rotated by the lane: conflict-free
+            const float4 *row4 = reinterpret_cast<const float4*>(row), *x4 = reinterpret_cast<const float4*>(x);
+            float p1 = 0.f, p2 = 0.f, p3 = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const int j = (q + lane) & 7;
+              const float4 a = row4[j], y = x4[j];
+              prop = fmaf(a.x, y.x, prop);
+              p1 = fmaf(a.y, y.y, p1);
+              p2 = fmaf(a.z, y.z, p2);
+              p3 = fmaf(a.w, y.w, p3);
+            }
+            prop = (prop + p1) + (p2 + p3);
+          } else if (l.active) {
+            for (int q = 0; q < l.rows; ++q) {
+              const int b = l.part * l.rows + ((q + k) & (l.rows - 1));
+              prop = fmaf(row[b], x[b], prop);
+            }
+          }
+          for (int off = r; off < r * l.parts; off <<= 1) prop += __shfl_xor_sync(kFull, prop, off);
+          prop *= u;
+          if (mine) {
+            us[(i - 1) * (r + 1) + k] = u;
+            props[i * r + k] = prop;
+          }
+        } else {
+          if (mine) {
+            ev[k] = al_i == -CUDART_INF_F ? -CUDART_INF_F : g[i * r + k] - al_i;
+            ev[32 + k] = abar;
+          }
+          __syncwarp();
+          if (l.active) {
+            const float* row = logA + static_cast<size_t>(i - 1) * rr + k * r;
+            for (int b = 0; b < r; ++b) prop += __expf(al + row[b] + ev[b]) * ev[32 + b];
+            if (mine) {
+              for (int b = 0; b < r; ++b)
+                atomicAdd(dT + static_cast<size_t>(i - 1) * rr + k * r + b, __expf(al + row[b] + ev[b]) * ev[32 + b] - __expf(row[b]) * prop);
+              us[(i - 1) * (r + 1) + k] = 0.f;                           // nothing for the running sums
+              xs[i * r + k] = 0.f;
+              props[i * r + k] = 0.f;
+            }
+          }
+          __syncwarp();
+        }
+        abar = l.active ? cw[i - 1] * __expf(al - lp) + prop : 0.f;
+        al_i = al;
+      }
+      float total = mine ? abar : 0.f;                                   // sum_z abar_0[z]
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) total += __shfl_xor_sync(kFull, total, off);
+      if (mine) {
+        post[k] = tg[0] >= 0 ? abar : 0.f;
+        a_.dsum[static_cast<size_t>(w) * a_.dsum_pitch + k] = __float2bfloat16_rn(abar - __expf(l0) * total);
+      }
+    }
+    __syncthreads();
+    // ---- the batch's rank-one terms
+    const int count = min(warps, w_end - w0);
+    for (int task = wib; task < (n - 1) * chunks; task += warps) {
+      const int i = 1 + task / chunks, b0 = l.part * l.rows + (task % chunks) * cols;
+      if (!l.active) continue;
+      float* sum = acc + (i - 1) * rr + b0 * r + k;
+      float s[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s[q] = q < cols ? sum[q * r] : 0.f;
+      const float* from = area;
+      if (cols == 8) {
+#pragma unroll 2
+        for (int j = 0; j < count; ++j, from += warp_floats) {
+          const float u = from[off_u + (i - 1) * (r + 1) + k], pr = -from[off_prop + i * r + k];
+          const float4 x0 = *reinterpret_cast<const float4*>(from + i * r + b0), x1 = *reinterpret_cast<const float4*>(from + i * r + b0 + 4);
+          s[0] += fmaf(u, x0.x, pr);
+          s[1] += fmaf(u, x0.y, pr);
+          s[2] += fmaf(u, x0.z, pr);
+          s[3] += fmaf(u, x0.w, pr);
+          s[4] += fmaf(u, x1.x, pr);
+          s[5] += fmaf(u, x1.y, pr);
+          s[6] += fmaf(u, x1.z, pr);
+          s[7] += fmaf(u, x1.w, pr);
+        }
+      } else {
+        for (int j = 0; j < count; ++j, from += warp_floats) {
+          const float u = from[off_u + (i - 1) * (r + 1) + k], pr = -from[off_prop + i * r + k];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (q < cols) s[q] += fmaf(u, from[i * r + b0 + q], pr);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (q < cols) sum[q * r] = s[q];
+    }
+    __syncthreads();                                                     // the warps' vectors are reused by the next batch
+  }
+  // ---- dT += A * (the running sums), four adjacent entries at a time where dT is aligned for it
+  if (rr % 4 == 0 && (reinterpret_cast<uintptr_t>(dT) & 15u) == 0) {
+    for (int e = threadIdx.x * 4; e < tables; e += blockDim.x * 4) {
+      const int q = e % rr, a = q / r, b = q - a * r;                    // (r a power of two: four entries of one row, or whole rows)
+      float v[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int at = (a * r + b + t) / r, bt = (b + t) % r;
+        v[t] = E[e + t] * acc[(e - q) + bt * r + at];
+      }
+      if (!(v[0] == 0.f && v[1] == 0.f && v[2] == 0.f && v[3] == 0.f))
+        atomicAdd(reinterpret_cast<float4*>(dT + e), make_float4(v[0], v[1], v[2], v[3]));
+    }
+  } else {
+    for (int e = threadIdx.x; e < tables; e += blockDim.x) {
+      const int q = e % rr, a = q / r, b = q - a * r;
+      const float v = E[e] * acc[(e - q) + b * r + a];
+      if (v != 0.f) atomicAdd(dT + e, v);
+    }
+  }
+}
+
 // ---------------------------------------------------------------- circuit backward: binary tree (Eq. BTree)
 // Upward pass as in circuit_btree_kernel (prod[j][z], S[c][z]); downward pass with U[j][z] = log-weight of everything
 // outside node j's subtree given z_j = z: U[0] = log omega_root, U[c][b] = LSE_z(U[j][z] + S[sibling][z] + logOmega_c[z][b]).

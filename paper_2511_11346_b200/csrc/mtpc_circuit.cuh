@@ -498,9 +498,10 @@ __device__ __forceinline__ HmmLanes hmm_lanes(int r, int lane) {
 // (every part returns it). alpha: per active lane, -inf elsewhere; NaN in any of them reaches every state. A [r, r] in shared
 // memory holds probabilities (LOG_TABLE: their logarithms); ev: 32 floats of the warp's shared memory, not reused before the
 // warp's next synchronisation. Every kernel that runs the recursion takes this step, so they return the same bits.
+// hmm_forward_sum returns the sum and m.
 template <bool LOG_TABLE>
-__device__ __forceinline__ float hmm_forward_step(float alpha, float* ev, const float* A, const HmmLanes& l, int r) {
-  float m = warp_max_nan(alpha);
+__device__ __forceinline__ float hmm_forward_sum(float alpha, float* ev, const float* A, const HmmLanes& l, int r, float& m) {
+  m = warp_max_nan(alpha);
   if (m == -CUDART_INF_F) m = 0.f;
   if (l.part == 0) ev[l.k] = __expf(alpha - m);
   __syncwarp();
@@ -525,6 +526,12 @@ __device__ __forceinline__ float hmm_forward_step(float alpha, float* ev, const 
     for (int a = 0; a < l.rows; ++a) s = fmaf(ep[a], entry(col[a * r]), s);
   }
   for (int off = r; off < r * l.parts; off <<= 1) s += __shfl_xor_sync(kFull, s, off);
+  return s;
+}
+template <bool LOG_TABLE>
+__device__ __forceinline__ float hmm_forward_step(float alpha, float* ev, const float* A, const HmmLanes& l, int r) {
+  float m;
+  const float s = hmm_forward_sum<LOG_TABLE>(alpha, ev, A, l, r, m);
   return m + __logf(s);
 }
 

@@ -216,6 +216,22 @@ int make_tmap(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, u
   return r == CUDA_SUCCESS ? MTPC_OK : MTPC_ERR_CUDA;
 }
 
+// bf16 array [rows][units][v] (row pitch `pitch` elements) written in boxes of 32 rows x 64 columns of one unit, 128-byte swizzle: what lies
+// past the unit's v columns is not written.
+int make_tmap_unit_rows(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t units, uint64_t v, uint64_t pitch) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return MTPC_ERR_CUDA;
+  if ((reinterpret_cast<uintptr_t>(base) & 15u) != 0 || (pitch * 2) % 16 != 0 || (v * 2) % 16 != 0) return MTPC_ERR_WORKSPACE;
+  cuuint64_t gdim[3] = {v, units, rows};
+  cuuint64_t gstride[2] = {v * 2, pitch * 2};
+  cuuint32_t box[3] = {64, 1, 32};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), gdim, gstride, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? MTPC_OK : MTPC_ERR_CUDA;
+}
+
 // bf16 matrix [rows, cols] row-major read as an MN-major operand (its columns are the operand's M or N index, its rows
 // the K index): boxes of 64 columns x 64 rows, 128-byte swizzle, zero fill outside.
 int make_tmap_mn(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, uint64_t pitch) {
@@ -255,7 +271,7 @@ struct mtpc_head {
   int lr_split_parts;                           // ... and how many there is room for
   CUtensorMap tm_lrB_dec;                       // B [n r k, d] for the few-position draft path
   size_t lr_off_zhl, lr_off_partial;            // workspace: z = B h as bf16 halves [T, n r, 2, k]; partial log-sum-exps per column block
-  CUtensorMap lr_tm_a[2];                       // the copy of A in the boxes of the forward and the gradient build
+  CUtensorMap lr_tm_a;                          // the copy of A in the boxes of the factored projection
   LowRankParams lr_params;                      // everything of the factored projection launch that does not depend on the call
   int max_pairs;                                // clusters of two projection CTAs that can be resident at once
   CUtensorMap tm_emit_dec, tm_sum_dec;          // the same matrices in the few-position draft path's tiles
@@ -1147,8 +1163,8 @@ bool plan_lowrank(const mtpc_config& c, int k, LowRankParams* p) {
 template <int MODE>
 int launch_lowrank_logits(mtpc_head* h, LowRankParams p, int T, cudaStream_t st) {
   const int rc = make_tmap(&p.tm_z, h->ws + h->lr_off_zhl, static_cast<uint64_t>(T), static_cast<uint64_t>(p.n) * p.r * 2 * p.k, kBlockM);
-  p.blocks = (p.v + lowrank_cols(MODE) - 1) / lowrank_cols(MODE);
-  p.tm_a = h->lr_tm_a[MODE];
+  p.blocks = (p.v + kLrCols - 1) / kLrCols;
+  p.tm_a = h->lr_tm_a;
   if (rc != MTPC_OK) return rc;
   p.T = T;
   p.m_tiles = (T + kBlockM - 1) / kBlockM;
@@ -1156,7 +1172,8 @@ int launch_lowrank_logits(mtpc_head* h, LowRankParams p, int T, cudaStream_t st)
   p.status = at<unsigned>(h, h->L.off_status);
   p.wait_limit_ns = h->wait_limit_ns;
   const long long items = static_cast<long long>(p.m_tiles) * p.n * p.blocks;
-  const int grid = static_cast<int>(items < h->num_sms ? items : h->num_sms);
+  const int held = lowrank_ctas(MODE) * h->num_sms;
+  const int grid = static_cast<int>(items < held ? items : held);
   launch_kernel(lowrank_logits_kernel<MODE>, grid, lowrank_threads(MODE), lowrank_smem_bytes(MODE), st, overlapped(h), p);
   h->launches++;
   return check_launch();
@@ -1192,12 +1209,11 @@ int launch_lowrank_projection(mtpc_head* h, const void* hidden_bf16, int T, cons
   if (!(parts & 4)) return check_launch();
   LowRankParams p = h->lr_params;
   p.log_sum = reinterpret_cast<float*>(h->ws + h->lr_off_partial);
-  p.ref = p.log_sum + static_cast<size_t>((c.v + 31) / 32) * T * units;
+  p.ref = p.log_sum + static_cast<size_t>((c.v + 31) / 32) * ((T + 31) / 32 * 32) * units;
   if ((rc = launch_lowrank_logits<kLowRankForward>(h, p, T, st)) != MTPC_OK) return rc;
-  const size_t entries = static_cast<size_t>(T) * units;
-  launch_kernel(lowrank_merge_kernel, static_cast<unsigned>((entries + 255) / 256), 256, 0, st, overlapped(h), p.log_sum, p.ref,
+  launch_kernel(k == 16 ? lowrank_merge_kernel<16> : lowrank_merge_kernel<32>, dim3((T + 31) / 32, c.n, (c.r + kMergeUnits - 1) / kMergeUnits), 256, 0, st, overlapped(h), p.log_sum, p.ref,
                 base, zhl, reinterpret_cast<const __nv_bfloat16*>(h->ws + h->lr_off_arep), targets, at<float>(h, L.off_G),
-                lse_out, at<unsigned>(h, L.off_status), entries, c.n, c.r, c.v, p.vv, k, targets_are_drafts ? 1 : 0);
+                lse_out, at<unsigned>(h, L.off_status), T, c.n, c.r, c.v, p.vv, targets_are_drafts ? 1 : 0);
   h->launches += 1;
   return check_launch();
 }
@@ -1425,8 +1441,7 @@ int lowrank_backward_tail(mtpc_head* head, const LowRankBackwardLayout& R, uint8
   lp.G = at<float>(head, L.off_G);
   lp.lse = reinterpret_cast<const float*>(bw + B.off_lse);
   lp.post = reinterpret_cast<const float*>(bw + B.off_post);
-  lp.g = dlogit;
-  lp.g_pitch = B.Kd;
+  if ((rc = make_tmap_unit_rows(&lp.tm_g, dlogit, static_cast<uint64_t>(T), static_cast<uint64_t>(units), static_cast<uint64_t>(c.v), B.Kd)) != MTPC_OK) return rc;
   lp.s = sy;
   lp.s_pitch = R.pitch;
   if ((rc = launch_lowrank_logits<kLowRankGradient>(head, lp, T, st)) != MTPC_OK) return rc;
@@ -1592,7 +1607,7 @@ static int lowrank_extra_bytes(const mtpc_config& c, int k, size_t base_total, s
   *off_zhl = off;
   off += align_up(static_cast<size_t>(c.max_positions) * units * 2 * k * 2);
   *off_partial = off;
-  off += align_up(static_cast<size_t>(c.max_positions) * (units + c.n) * ((c.v + 31) / 32) * sizeof(float));
+  off += align_up(static_cast<size_t>((c.max_positions + 31) / 32 * 32) * (units + c.n) * ((c.v + 31) / 32) * sizeof(float));
   *off_arep = off;                      // the copy of A laid out [n, v, r, k]
   off += align_up(units * c.v * k * 2);
   *off_dec = off;                       // few-position draft: base = W_base h [P, n v] and z = B h [P, n r k], fp32
@@ -1697,9 +1712,9 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
     fail = !allow_full_smem(lowrank_logits_kernel<kLowRankForward>);
     fail |= !allow_full_smem(lowrank_logits_kernel<kLowRankGradient>);
     if (fail) rc = MTPC_ERR_CUDA;
-    for (int mode = 0; mode < 2 && rc == MTPC_OK; ++mode)
-      rc = make_tmap(&h->lr_tm_a[mode], h->ws + h->lr_off_arep, static_cast<uint64_t>(cfg->n) * cfg->v,
-                     static_cast<uint64_t>(cfg->r) * lowrank->k, lowrank_cols(mode));
+    if (rc == MTPC_OK)
+      rc = make_tmap(&h->lr_tm_a, h->ws + h->lr_off_arep, static_cast<uint64_t>(cfg->n) * cfg->v,
+                     static_cast<uint64_t>(cfg->r) * lowrank->k, kLrCols);
   }
   if (rc != MTPC_OK) { delete h; return rc; }
   *out = h;

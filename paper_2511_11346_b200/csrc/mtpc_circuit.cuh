@@ -161,16 +161,14 @@ __device__ __forceinline__ int next_window(unsigned* counter, int lane) {
 
 // ---- asynchronous staging of an r x r table (global -> shared) by one warp, for kernels that stream one set of
 // tables per position from HBM: the copy of the next table is in flight while the current one is reduced.
-__device__ __forceinline__ void cp_async_16(float* dst, const float* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
-               "l"(src)
-               : "memory");
+__device__ __forceinline__ void cp_async_16(uint32_t dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async_4(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
-               "l"(src)
-               : "memory");
+__device__ __forceinline__ void cp_async_4(uint32_t dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async_16(float* dst, const float* src) { cp_async_16(smem_u32(dst), src); }
+__device__ __forceinline__ void cp_async_4(float* dst, const float* src) { cp_async_4(smem_u32(dst), src); }
 // The calling threads' share (of `threads`) of copying count floats to shared memory, not committed.
 __device__ __forceinline__ void fetch_floats(float* dst, const float* src, int count, int threads) {
   if ((count & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0) {

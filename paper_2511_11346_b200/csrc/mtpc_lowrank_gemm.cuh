@@ -4,31 +4,30 @@
 // rounding z to the tensor cores' operand type costs 2^-17 instead of 2^-9); lowrank_logits_kernel does the rest without
 // writing a logit. FLOPs per position: 2 d (n v + n r k) + 4 n r v k instead of 2 d n r v.
 //
-// A work item is (128 positions, slot i, 128 or 64 columns b of the vocabulary). A thread of the epilogue keeps the base logits
-// of one position and 32 columns in registers and walks the slot's r components: corr_j = z_j A_ij^T for the item's columns
-// comes out of tensor memory (K = 2k: [hi | lo] against A twice), x = base + corr_j, and then
-//   forward   (kLowRankForward): the log-sum-exp of the 32 columns, combined over the item's columns through shared memory;
-//             lowrank_merge_kernel combines the column blocks, forms the target's logit and writes G. The reference of the
-//             exponentials is the base logits' maximum, known before the walk; a component whose sum leaves [2^-60, 2^120]
-//             against it (corrections of many tens) is redone with its own maximum;
+// A work item is (128 positions, slot i, 64 columns b of the vocabulary). A thread of the epilogue keeps the base logits
+// of one position and 32 (gradient: 16) columns in registers and walks the slot's r components: corr_j = z_j A_ij^T for the item's
+// columns comes out of tensor memory (K = 2k: [hi | lo] against A twice), x = base + corr_j, and then
+//   forward   (kLowRankForward): the log-sum-exp of the 32 columns; lowrank_merge_kernel combines the unit's, forms the target's
+//             logit and writes G. The reference of the exponentials is the base logits' maximum, known before the walk; a component
+//             whose sum leaves [2^-60, 2^120] against it (corrections of many tens) is redone with its own maximum;
 //   gradient  (kLowRankGradient): g = post (onehot(target) - exp(x - lse)) as bf16, the operand of the GEMMs of the training
 //             call, and sum_j g_ij - so a training call keeps no logits ([T, n r v] fp32 were written and read back) and needs
 //             no pass over g for that sum.
 // Why this shape: with the components outermost (base logits and a running maximum re-read from tensor memory per component,
 // corrections in chunks of <= 48 columns) the kernel was bound by its corrections: a dependent pair of M = 128, N <= 48 MMAs
 // costs about 320 cycles against 24 of arithmetic, and the columns of a component waited for each other through the maximum.
-// Here MMAs are 64 or 128 columns wide, two components' pairs alternate, 512 columns of accumulators are in flight, and no
+// Here the MMAs of two components alternate into one slot of tensor memory, two (gradient: four) slots are in flight, and no
 // (component, 32 columns) depends on another. The bound is one ex2 per logit (16 a clock and SM: 149 us at T = 8192, n = 8,
 // r = 32, v = 320), in the gradient also the 1.3 GB of g.
-// Measured (this kernel, forward / gradient): 290 / 448 us with the schedulers issuing on 48 / 41 % of the
-// cycles (the rest waits on tensor-memory loads and ex2), where the fused projection that kept logits took 801 us and the
-// passes that made g and its sum from them 921 us; a likelihood call's whole projection at T = 8192, v = 320, d = 4096: r = 16
-// 506 -> 438 us, r = 32 893 -> 673 us.
-// Roles: warp 0 TMA producer, warp 1 MMA issuer, then the epilogue warps (TMEM quarter warp % 4, columns 32 * ((warp - 2) / 4)).
-// Operand ring: one entry holds 64 / k components, all as 128-byte rows with the 128-byte swizzle: z as two boxes of 128
-// positions x 64 values ([hi | lo] of 32 / k adjacent components each), and A as one box of the item's vocabulary rows x 64 values (the k
-// adaptor columns of 64 / k adjacent components) of a copy laid out [n, v, r, k] (lowrank_repack_kernel, made on every call: A is
-// small and may have changed).
+// 64 columns divide more vocabularies evenly than 128 (of the third item of v = 320 half the warps had nothing), one wait and one
+// release serve two components, and log-sums leave as 128 contiguous bytes (position fastest; transposed through shared memory
+// before). Measured, forward / merge / gradient, same sizes: 292 / 62 / 450 us before, 247 / 67 / 387 now, the exponential unit
+// busy for 73 / 43 % of the cycles (61 / 38); the gradient's rest is instructions (two thirds of an issue slot a logit) and its warps' latency.
+// The fused projection that kept logits took 801 us and the passes that made g and its sum from them 921.
+// Roles: warp 0 TMA producer, warp 1 MMA issuer, then the epilogue warps (TMEM quarter warp % 4).
+// Operand ring: one entry holds 32 / k components, all as 128-byte rows with the 128-byte swizzle: z as one box of 128
+// positions x 64 values ([hi | lo] of the components), and A as one box of the item's vocabulary rows x 64 values (the components' k
+// adaptor columns first) of a copy laid out [n, v, r, k] (lowrank_repack_kernel, made on every call: A is small and may have changed).
 #pragma once
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -42,83 +41,90 @@ namespace mtpc {
 
 constexpr int kLrMaxRank = 32;          // k <= 32 (a multiple of 16)
 constexpr int kLrMaxVocab = 1792;
-constexpr int kLrStages = 2;
-constexpr int kLrRoleWarps = 2;
-constexpr int kLrJ = 16;                // components per round of an epilogue warp's shared-memory patches
-constexpr int kLrPitch = 33;            // pitch of a component's 32 positions there (read across components without conflicts)
+constexpr int kLrStages = 3;
+constexpr int kLrCols = 64;             // columns of a work item
+constexpr int kLrRound = 8;             // gradient: components whose lse, weight and G an epilogue warp fetches at a time
 enum { kLowRankForward = 0, kLowRankGradient = 1 };
-// Columns of a work item (an epilogue warp takes 32 of them). The gradient keeps a second register per column (the sum over the
-// components): 64 columns, eight epilogue warps and 168 registers a thread; with sixteen warps and 96 it spilled or could not
-// have the next accumulators in flight.
-__host__ __device__ constexpr int lowrank_cols(int mode) { return mode == kLowRankForward ? 128 : 64; }
-__host__ __device__ constexpr int lowrank_subs(int mode) { return lowrank_cols(mode) / 32; }
+// Columns of an epilogue thread, and CTAs per SM. Both builds have sixteen epilogue warps on an SM: the forward's in two CTAs, which
+// drift apart and fill each other's waits; the gradient keeps a second register per column (the sum over the components) and shares
+// the operands, which its narrower threads would otherwise fetch twice.
+__host__ __device__ constexpr int lowrank_warp_cols(int mode) { return mode == kLowRankForward ? 32 : 16; }
+__host__ __device__ constexpr int lowrank_ctas(int mode) { return mode == kLowRankForward ? 2 : 1; }
+__host__ __device__ constexpr int lowrank_subs(int mode) { return kLrCols / lowrank_warp_cols(mode); }
+constexpr int kLrRoleWarps = 2;
 __host__ __device__ constexpr int lowrank_threads(int mode) { return 32 * kLrRoleWarps + 128 * lowrank_subs(mode); }
-__host__ __device__ constexpr int lowrank_stage_bytes(int mode) { return 2 * kBlockM * 128 + lowrank_cols(mode) * 128; }
+__host__ __device__ constexpr int lowrank_tmem_cols(int mode) { return kTmemCols / lowrank_ctas(mode); }
+constexpr uint32_t kLrZBox = kBlockM * 128;                  // 128 positions x 64 bf16 of z
+constexpr uint32_t kLrStageBytes = kLrZBox + kLrCols * 128;  // and the item's vocabulary rows x 64 bf16 of A'
 
 struct LowRankParams {
   CUtensorMap tm_z;      // z      [T, n*r*2*k]        box 64 x 128, 128-byte swizzle (unit u: hi at (2u)k, lo at (2u+1)k)
-  CUtensorMap tm_a;      // A'     [n*v, r*k]          box 64 x lowrank_cols, 128-byte swizzle (row (i, b): A[i, 0..r-1, b, :])
+  CUtensorMap tm_a;      // A'     [n*v, r*k]          box 64 x kLrCols, 128-byte swizzle (row (i, b): A[i, 0..r-1, b, :])
   int T, m_tiles, n, r, v, vv, k;
   int blocks;                        // column blocks of a unit
   const float* base;                 // [T, n v]
-  float* log_sum;                    // forward: [ceil(v / 32), T n r] log2 of the sum of exponentials of 32 columns, relative to
-  float* ref;                        //          [ceil(v / 32), T n] the maximum of their base logits
+  float* log_sum;                    // forward: [ceil(T / 32), ceil(v / 32), n r, 32] log2 of the sum of exponentials of 32 columns,
+  float* ref;                        //          relative to [ceil(T / 32), ceil(v / 32), n, 32] the maximum of their base logits
   const int* targets;                // gradient: [T, n]
   const float* G;                    // gradient: [T, n, r] log phi at the target,
   const float* lse;                  //           [T, n, r] log-sum-exp of every unit,
   const float* post;                 //           [T, n, r] its weighted posterior
-  __nv_bfloat16* g;                  //           [T, n r v] at a pitch of g_pitch
-  size_t g_pitch;
+  CUtensorMap tm_g;                  //           g: [T][n r][v] of bf16 at a pitch, box 32 x 1 x 64, 128-byte swizzle
   __nv_bfloat16* s;                  //           [T, n v] at a pitch of s_pitch: g summed over a slot's components
   size_t s_pitch;
   unsigned* status;
   uint64_t wait_limit_ns;
 };
-// Shared memory of an epilogue warp behind the ring, in floats: the next item's base logits [32 positions][32 columns] (16-byte
-// pieces swizzled by the position); forward: log-sums [kLrJ][kLrPitch]; gradient: two rounds of lse, weight and G, each
-// [kLrJ][kLrPitch]. Nothing is shared between epilogue warps: with block-wide staging and barriers a sixth (forward) to nearly
-// half (gradient) of the time went into the boundaries between items.
-__host__ __device__ constexpr int lowrank_warp_floats(int mode) {
-  return 1024 + (mode == kLowRankForward ? 1 : 6) * kLrJ * kLrPitch;
+// Shared memory behind the ring, in floats. Per epilogue warp: the next item's base logits [32 positions][its columns] (16-byte pieces
+// swizzled by the position). Gradient, per group of the four warps that share 32 positions: two buffers of g for two components, each
+// [32 positions][64 columns] bf16 as a TMA store with 128-byte swizzle takes them, and two rounds of lse, weight and G, each
+// [kLrRound][kLrPitch]. Nothing else is shared between epilogue warps: with block-wide staging and barriers a sixth
+// (forward) to nearly half (gradient) of the time went into the boundaries between items.
+constexpr int kLrTileBytes = 32 * 128;
+constexpr int kLrPitch = 33;            // of a component's 32 positions (written and read across components without conflicts)
+__host__ __device__ constexpr int lowrank_group_floats(int mode) { return mode == kLowRankForward ? 0 : kLrTileBytes; }   // 4 tiles of 1024
+__host__ __device__ constexpr int lowrank_round_floats(int mode) { return mode == kLowRankForward ? 0 : 6 * kLrRound * kLrPitch; }
+__host__ __device__ constexpr int lowrank_patch_floats(int mode) {
+  return 4 * (lowrank_group_floats(mode) + lowrank_subs(mode) * 32 * lowrank_warp_cols(mode) + lowrank_round_floats(mode));
 }
 inline size_t lowrank_smem_bytes(int mode) {
-  return 1024 + static_cast<size_t>(kLrStages) * lowrank_stage_bytes(mode) + 4 * lowrank_subs(mode) * lowrank_warp_floats(mode) * sizeof(float) +
-         sizeof(GemmControl);
+  return 1024 + static_cast<size_t>(kLrStages) * kLrStageBytes + lowrank_patch_floats(mode) * sizeof(float) + sizeof(GemmControl);
+}
+
+__device__ __forceinline__ void st_shared_bf16(uint32_t dst, __nv_bfloat16 x) {
+  asm volatile("st.shared.b16 [%0], %1;" ::"r"(dst), "h"(__bfloat16_as_ushort(x)) : "memory");
 }
 
 struct LowRankItem {
   int mt, slot, block, width;     // width: columns of this block (a multiple of 16)
 };
 // column block fastest: the CTAs that run together share the positions' z through L2
-template <int COLS>
 __device__ __forceinline__ LowRankItem lowrank_item(const LowRankParams& p, int item) {
   LowRankItem c;
   c.block = item % p.blocks;
   const int rest = item / p.blocks;
   c.slot = rest % p.n;
   c.mt = rest / p.n;
-  c.width = min(COLS, p.v - c.block * COLS);
+  c.width = min(kLrCols, p.v - c.block * kLrCols);
   return c;
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kernel(const __grid_constant__ LowRankParams p) {
-  constexpr int kCols = lowrank_cols(MODE), kSubs = lowrank_subs(MODE), kSlots = kTmemCols / kCols;
-  constexpr int kStageBytes = lowrank_stage_bytes(MODE);
+__global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) lowrank_logits_kernel(const __grid_constant__ LowRankParams p) {
+  constexpr int kSubs = lowrank_subs(MODE), kWarpCols = lowrank_warp_cols(MODE);
+  constexpr int kTmem = lowrank_tmem_cols(MODE), kSlots = kTmem / (2 * kLrCols);      // a slot: the accumulators of two components
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t ring = (raw_addr + 1023u) & ~1023u;
-  float* patches = reinterpret_cast<float*>(smem_raw + (ring - raw_addr) + kLrStages * kStageBytes);
-  GemmControl* ctl = reinterpret_cast<GemmControl*>(patches + 4 * kSubs * lowrank_warp_floats(MODE));
+  float* patches = reinterpret_cast<float*>(smem_raw + (ring - raw_addr) + kLrStages * kLrStageBytes);
+  GemmControl* ctl = reinterpret_cast<GemmControl*>(patches + lowrank_patch_floats(MODE));
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int num_items = p.m_tiles * p.n * p.blocks;
-  const int kq = p.k / 16;                                // K = 16 steps of one half of a correction
-  const int ca = 64 / p.k;                                // components per ring entry (= per box of A')
-  const int cz = 32 / p.k;                                // components per box of z; an entry has ca / cz = 2 of them
-  const int nent = (p.r + ca - 1) / ca;                   // ring entries per item
-  constexpr uint32_t kZBox = kBlockM * 128;               // bytes of one z box
+  const int npairs = (p.r + 1) / 2;                       // components go through in pairs (r = 1: one and its copy)
+  const int per_entry = 32 / p.k;                         // components per ring entry: 2 (k = 16) or 1 (k = 32)
+  const int nent = (p.r + per_entry - 1) / per_entry;     // ring entries per item
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kLrStages; ++s) {
@@ -135,9 +141,10 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kerne
     fence_mbar_init();
     tma_prefetch_desc(&p.tm_z);
     tma_prefetch_desc(&p.tm_a);
+    if (MODE == kLowRankGradient) tma_prefetch_desc(&p.tm_g);
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
+    tmem_alloc(smem_u32(&ctl->tmem_base), kTmem);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -146,25 +153,23 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kerne
   const uint32_t tmem_base = ctl->tmem_base;
   grid_launch_dependents();
   grid_dependency_wait();
-
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       uint32_t st = 0, phase = 0, issued_mask = 0, phase_mask = 0;
       bool ok = true;
       for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-        const LowRankItem w = lowrank_item<kCols>(p, item);
+        const LowRankItem w = lowrank_item(p, item);
         for (int e = 0; e < nent; ++e) {
           if (!bounded_wait(smem_u32(&ctl->empty[st]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
           const uint32_t full = smem_u32(&ctl->full[st]);
-          const uint32_t dst = ring + st * kStageBytes;
-          const int unit0 = w.slot * p.r + e * ca;           // first component of the entry
-          mbar_arrive_expect_tx(full, kStageBytes);
-          // boxes may cover components past the slot's last (the next slot's, or zeros past the end) and, for A', rows past
-          // the unit: none of that is multiplied
-          for (int bx = 0; bx < 2; ++bx)
-            tma_load_2d(dst + bx * kZBox, &p.tm_z, full, (unit0 + bx * cz) * 2 * p.k, w.mt * kBlockM);
-          tma_load_2d(dst + 2 * kZBox, &p.tm_a, full, e * ca * p.k, w.slot * p.v + w.block * kCols);
+          const uint32_t dst = ring + st * kLrStageBytes;
+          const int j = e * per_entry;                       // first component of the entry
+          mbar_arrive_expect_tx(full, kLrStageBytes);
+          // the boxes may cover components past the slot's last (the next slot's, or zeros past the end), adaptor columns past the
+          // entry's and rows past the unit: none of that is multiplied
+          tma_load_2d(dst, &p.tm_z, full, (w.slot * p.r + j) * 2 * p.k, w.mt * kBlockM);
+          tma_load_2d(dst + kLrZBox, &p.tm_a, full, j * p.k, w.slot * p.v + w.block * kLrCols);
           issued_mask |= 1u << st;
           phase_mask = (phase_mask & ~(1u << st)) | (phase << st);
           if (++st == kLrStages) { st = 0; phase ^= 1u; }
@@ -181,43 +186,46 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kerne
     }
     __syncwarp();
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer: component u overall into slot u % kSlots
+    // ------------------------------------------------------------------ MMA issuer: pair u overall into slot u % kSlots
     if (lane == 0) {
       uint32_t st = 0, phase = 0, use = 0;
       bool ok = true;
+      const uint64_t z_desc0 = umma_smem_desc_sw128(ring), a_desc0 = umma_smem_desc_sw128(ring + kLrZBox);
+      constexpr uint32_t kStageStep = kLrStageBytes >> 4;      // descriptors step in 16-byte units
+      auto next_stage = [&] {
+        umma_commit(smem_u32(&ctl->empty[st]));
+        if (++st == kLrStages) { st = 0; phase ^= 1u; }
+      };
       for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-        const LowRankItem w = lowrank_item<kCols>(p, item);
+        const LowRankItem w = lowrank_item(p, item);
         const uint32_t idesc = umma_idesc_bf16(kBlockM, w.width);
-        for (int e = 0; e < nent && ok; ++e) {
-          if (!bounded_wait(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
+        for (int pr = 0; pr < npairs && ok; ++pr, ++use) {
+          const uint32_t slot = use % kSlots;
+          if (!bounded_wait(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t entry = ring + st * kStageBytes;
-          const int count = min(ca, p.r - e * ca);
-          for (int l = 0; l < count && ok; l += 2) {
-            const int pair = min(2, count - l);
-            uint64_t z_desc[2], a_desc[2];
-            uint32_t d_tmem[2];
-            for (int q = 0; q < pair; ++q) {
-              // descriptors step in 16-byte units: the component's [hi | lo] inside its z box, its k columns inside the A' box
-              z_desc[q] = umma_smem_desc_sw128(entry + ((l + q) / cz) * kZBox) + (((l + q) % cz) * 2 * p.k) / 8;
-              a_desc[q] = umma_smem_desc_sw128(entry + 2 * kZBox) + ((l + q) * p.k) / 8;
-              const uint32_t slot = (use + q) % kSlots;
-              d_tmem[q] = tmem_base + slot * kCols;
-              if (!bounded_wait(smem_u32(&ctl->tempty[slot]), (((use + q) / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
-            }
-            if (!ok) break;
+          const uint32_t d_tmem = tmem_base + slot * 2 * kLrCols;
+          const int count = min(2, p.r - 2 * pr);
+          if (p.k == 16) {                                     // one entry: [hi | lo] of two components, 16 adaptor columns each
+            if (!bounded_wait(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
             tc_fence_after();
-            // the two components alternate, so that an MMA does not follow the one whose result it adds to
-            for (int part = 0; part < 2; ++part)
-              for (int kk = 0; kk < kq; ++kk)
-                for (int q = 0; q < pair; ++q)
-                  umma_bf16(d_tmem[q], z_desc[q] + (part * p.k + 16 * kk) / 8, a_desc[q] + (16 * kk) / 8, idesc, (part | kk) != 0 ? 1u : 0u);
-            for (int q = 0; q < pair; ++q) umma_commit(smem_u32(&ctl->tfull[(use + q) % kSlots]));
-            use += pair;
+            const uint64_t z = z_desc0 + st * kStageStep, a = a_desc0 + st * kStageStep;
+            for (int part = 0; part < 2; ++part)               // (the two alternate: an MMA does not follow the one whose result it adds to)
+              for (int q = 0; q < 2; ++q)
+                umma_bf16(d_tmem + q * kLrCols, z + (q < count ? 4 * q : 0) + 2 * part, a + (q < count ? 2 * q : 0), idesc, part);
+            next_stage();
+          } else {                                             // an entry per component: hi at 0, lo at 32 of its 64 values
+            for (int q = 0; q < count && ok; ++q) {
+              if (!bounded_wait(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
+              tc_fence_after();
+              const uint64_t z = z_desc0 + st * kStageStep, a = a_desc0 + st * kStageStep;
+              for (int kk = 0; kk < 4; ++kk) umma_bf16(d_tmem + q * kLrCols, z + 2 * kk, a + 2 * (kk & 1), idesc, kk != 0 ? 1u : 0u);
+              for (int kk = 0; kk < 4 && count == 1; ++kk)
+                umma_bf16(d_tmem + kLrCols, z + 2 * kk, a + 2 * (kk & 1), idesc, kk != 0 ? 1u : 0u);
+              next_stage();
+            }
           }
           if (!ok) break;
-          umma_commit(smem_u32(&ctl->empty[st]));
-          if (++st == kLrStages) { st = 0; phase ^= 1u; }
+          umma_commit(smem_u32(&ctl->tfull[slot]));
         }
       }
       if (!ok || ctl->abort) {   // wait (bounded) for the MMAs already issued before tensor memory is freed
@@ -231,66 +239,82 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kerne
     // ------------------------------------------------------------------ epilogue
     const int quarter = warp & 3;
     const int sub = (warp - kLrRoleWarps) >> 2;
-    const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + sub * 32;
+    const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + sub * kWarpCols;
     const size_t units = static_cast<size_t>(p.n) * p.r;
     const float2 l2 = make_float2(kLog2e, kLog2e);
-    float* next_base = patches + (warp - kLrRoleWarps) * lowrank_warp_floats(MODE);
-    float* patch = next_base + 1024;
+    const uint32_t next_base = smem_u32(patches) + (4 * lowrank_group_floats(MODE) + (warp - kLrRoleWarps) * 32 * kWarpCols) * 4;
+    const uint32_t rounds = smem_u32(patches) + (4 * lowrank_group_floats(MODE) + 4 * kSubs * 32 * kWarpCols + quarter * lowrank_round_floats(MODE)) * 4;
+    constexpr int kChunks = kWarpCols / 4;                 // 16-byte pieces of a position's base logits
+    auto swizzled = [](int row, int ch) { return kChunks == 8 ? ch ^ (row & 7) : ch ^ ((row >> 1) & 3); };
     // ---- copies that are in flight while the current item or round is worked on
-    auto fetch_base = [&](int item) {                      // base logits of the warp's 32 positions x 32 columns
+    auto fetch_base = [&](int item) {                      // base logits of the warp's 32 positions x its columns
       if (item < num_items) {
-        const LowRankItem w = lowrank_item<kCols>(p, item);
-        const int col0 = w.block * kCols + sub * 32, ch = lane & 7;
-        if (col0 + ch * 4 < p.v) {
+        const LowRankItem w = lowrank_item(p, item);
+        const int ch = lane % kChunks, col = w.block * kLrCols + sub * kWarpCols + ch * 4;
+        if (col < p.v) {
+          const float* src = p.base + static_cast<size_t>(w.slot) * p.v + col;
 #pragma unroll
-          for (int it = 0; it < 8; ++it) {
-            const int rr = it * 4 + (lane >> 3);
+          for (int it = 0; it < kChunks; ++it) {
+            const int rr = it * (32 / kChunks) + lane / kChunks;
             const int t = min(w.mt * kBlockM + quarter * 32 + rr, p.T - 1);
-            cp_async_16(next_base + rr * 32 + ((ch ^ (rr & 7)) * 4),
-                        p.base + static_cast<size_t>(t) * p.n * p.v + static_cast<size_t>(w.slot) * p.v + col0 + ch * 4);
+            cp_async_16(next_base + (rr * kWarpCols + swizzled(rr, ch) * 4) * 4, src + static_cast<size_t>(t) * p.n * p.v);
           }
         }
       }
     };
-    auto fetch_round = [&](int item, int j0, float* dst) { // gradient: lse, weight and G of 32 positions x kLrJ components
-      if (item < num_items) {
-        const LowRankItem w = lowrank_item<kCols>(p, item);
-        const int jj = lane & (kLrJ - 1);
-        if (j0 + jj < p.r) {
-          for (int it = 0; it < 16; ++it) {
-            const int rr = it * 2 + (lane >> 4);
-            const int t = min(w.mt * kBlockM + quarter * 32 + rr, p.T - 1);
-            const size_t tu = static_cast<size_t>(t) * units + static_cast<size_t>(w.slot) * p.r + j0 + jj;
-            float* d = dst + jj * kLrPitch + rr;
-            cp_async_4(d, p.lse + tu);
-            cp_async_4(d + kLrJ * kLrPitch, p.post + tu);
-            cp_async_4(d + 2 * kLrJ * kLrPitch, p.G + tu);
-          }
+    // gradient: lse, weight and G of 32 positions x kLrRound components, by the four warps of the positions together
+    auto fetch_round = [&](const LowRankItem& w, int j0, uint32_t dst) {
+      const int j = lane & (kLrRound - 1);
+      if (j0 + j < p.r) {
+#pragma unroll
+        for (int it = 0; it < 2; ++it) {
+          const int rr = it * 16 + sub * 4 + lane / kLrRound;
+          const int t = min(w.mt * kBlockM + quarter * 32 + rr, p.T - 1);
+          const size_t tu = static_cast<size_t>(t) * units + static_cast<size_t>(w.slot) * p.r + j0 + j;
+          const uint32_t d = dst + (j * kLrPitch + rr) * 4;
+          cp_async_4(d, p.lse + tu);
+          cp_async_4(d + 4 * kLrRound * kLrPitch, p.post + tu);
+          cp_async_4(d + 8 * kLrRound * kLrPitch, p.G + tu);
         }
       }
     };
-    uint32_t use = 0, round = 0;
+    auto group_barrier = [&] { asm volatile("bar.sync %0, 128;" ::"r"(1 + quarter) : "memory"); };
+    uint32_t use = 0, ca[8], cb[8];                          // (ca, cb: the gradient's accumulators, eight columns each)
+    const int round_shift = p.r >= 8 ? 2 : p.r >= 4 ? 1 : 0;   // log2 of the pairs in a round: round `use >> round_shift` is in buffer (.. & 1)
     bool ok = true;
     // (every lane polls: no broadcast of the outcome, one vote)
     auto wait_slot = [&](uint32_t u) -> bool {
-      return __all_sync(kFull, bounded_wait(smem_u32(&ctl->tfull[u % kSlots]), (u / kSlots) & 1u, ctl, p.status));
+      const bool up = __all_sync(kFull, bounded_wait(smem_u32(&ctl->tfull[u % kSlots]), (u / kSlots) & 1u, ctl, p.status));
+      tc_fence_after();
+      return up;
+    };
+    auto release_slot = [&](uint32_t u) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&ctl->tempty[u % kSlots]));
     };
     fetch_base(blockIdx.x);
-    if (MODE == kLowRankGradient) fetch_round(blockIdx.x, 0, patch);
+    if (MODE == kLowRankGradient && blockIdx.x < num_items) fetch_round(lowrank_item(p, blockIdx.x), 0, rounds);
     cp_async_commit();
-    for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-      const LowRankItem w = lowrank_item<kCols>(p, item);
-      const int row0 = w.mt * kBlockM + quarter * 32, row = row0 + lane;
+    if (MODE == kLowRankGradient) {
+      cp_async_wait<0>();
+      group_barrier();
+      if (blockIdx.x < num_items) ok = wait_slot(0);
+      tmem_ld8_issue(lane_base, ca);
+    }
+    for (int item = blockIdx.x; item < num_items && (ok || MODE == kLowRankGradient); item += gridDim.x) {
+      const LowRankItem w = lowrank_item(p, item);
+      const int row = w.mt * kBlockM + quarter * 32 + lane;
       const bool valid = row < p.T;
-      const int col0 = w.block * kCols + sub * 32;         // this warp's first column inside the unit
-      const int here = min(32, p.v - col0);                // its columns: 32, 16 or none (<= 0)
-      float2 base[16];                                     // (base - ref) log2(e); ref: their maximum (forward) or 0
+      const int col0 = w.block * kLrCols + sub * kWarpCols;   // this warp's first column inside the unit
+      const int here = min(kWarpCols, p.v - col0);            // its columns (a multiple of 16), or none (<= 0)
+      float2 base[kWarpCols / 2];                             // (base - ref) log2(e); ref: their maximum (forward) or 0
       float ref = -CUDART_INF_F;
       cp_async_wait<0>();
       __syncwarp();
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        float4 x = *reinterpret_cast<const float4*>(next_base + lane * 32 + ((q ^ (lane & 7)) * 4));
+      for (int q = 0; q < kChunks; ++q) {
+        float4 x = ld_shared_v4(next_base + (lane * kWarpCols + swizzled(lane, q) * 4) * 4);
         if (col0 + 4 * q + 4 > p.vv) {                     // padding columns, and columns past the unit, carry no mass
           if (col0 + 4 * q >= p.vv) x.x = -CUDART_INF_F;
           if (col0 + 4 * q + 1 >= p.vv) x.y = -CUDART_INF_F;
@@ -303,84 +327,47 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kerne
       }
       if (MODE == kLowRankGradient || ref == -CUDART_INF_F) ref = 0.f;
 #pragma unroll
-      for (int q = 0; q < 16; ++q) base[q] = make_float2((base[q].x - ref) * kLog2e, (base[q].y - ref) * kLog2e);
+      for (int q = 0; q < kWarpCols / 2; ++q) base[q] = make_float2((base[q].x - ref) * kLog2e, (base[q].y - ref) * kLog2e);
       __syncwarp();
       fetch_base(item + gridDim.x);
-      float2 sum[16];                                      // gradient: sum over the components,
-      float hot = 0.f;                                     // and of the weights, for the target's column
-      int rel = -1;
-      bool has_target = false;
-      if constexpr (MODE == kLowRankGradient) {
-#pragma unroll
-        for (int q = 0; q < 16; ++q) sum[q] = make_float2(0.f, 0.f);
-        const int tgt = valid ? p.targets[static_cast<size_t>(row) * p.n + w.slot] : -1;
-        has_target = tgt >= 0;                             // a marginalised byte has no gradient
-        rel = (tgt >= col0 && tgt < min(col0 + 32, p.vv)) ? tgt - col0 : -1;   // (a refused target, >= vv, has no column)
-      } else {
+      if constexpr (MODE == kLowRankForward) {
         cp_async_commit();
-        if (valid && here > 0) p.ref[static_cast<size_t>(col0 / 32) * p.T * p.n + static_cast<size_t>(row) * p.n + w.slot] = ref;
-      }
-      for (int j0 = 0; j0 < p.r; j0 += kLrJ, ++round) {
-        const int jc = min(kLrJ, p.r - j0);                // a power of two
-        const float* mine = patch + (round & 1) * (3 * kLrJ * kLrPitch);    // gradient: this round's
-        if constexpr (MODE == kLowRankGradient) {
-          if (j0 > 0) {
-            cp_async_wait<0>();
-            __syncwarp();
-          }
-          const bool last = j0 + kLrJ >= p.r;              // the next round: of this item or of the next one
-          fetch_round(last ? item + gridDim.x : item, last ? 0 : j0 + kLrJ, patch + ((round + 1) & 1) * (3 * kLrJ * kLrPitch));
-          cp_async_commit();
-        }
-        // The accumulators of a component in two halves of sixteen columns: the second half is on its way while the first is
-        // consumed, the next component's first half while the second is.
-        uint32_t ca0[16], ca1[16];
+        // ---- forward: a component's accumulators in two halves of sixteen columns; the second half is on its way while the first
+        // is consumed, the next component's first half while the second is
+        const size_t strip = static_cast<size_t>(w.mt * (kBlockM / 32) + quarter) * ((p.v + 31) / 32) + col0 / 32;   // of 32 positions and columns
+        if (valid && here > 0) p.ref[(strip * p.n + w.slot) * 32 + lane] = ref;
+        float* dst = p.log_sum + (strip * units + static_cast<size_t>(w.slot) * p.r) * 32 + lane;
+        uint32_t c0[16], c1[16];
         if (!(ok = wait_slot(use))) break;
-        tc_fence_after();
-        tmem_ld16_issue(lane_base + (use % kSlots) * kCols, ca0);
-        for (int jj = 0; jj < jc; ++jj, ++use) {
-          const uint32_t col = lane_base + (use % kSlots) * kCols;
-          tmem_ld_wait16(ca0);
-          tmem_ld16_issue(col + 16, ca1);                  // (columns past the block's width are not used)
-          float2 sa = make_float2(0.f, 0.f), sb = sa;
-          float lse2 = 0.f, wt = 0.f;
-          __nv_bfloat16* dst = nullptr;
-          if constexpr (MODE == kLowRankGradient) {
-            lse2 = mine[jj * kLrPitch + lane] * kLog2e;
-            wt = has_target ? mine[(kLrJ + jj) * kLrPitch + lane] : 0.f;
-            hot += wt;
-            dst = p.g + static_cast<size_t>(valid ? row : 0) * p.g_pitch + (static_cast<size_t>(w.slot) * p.r + j0 + jj) * p.v + col0;
-          }
-          auto eat = [&](const uint32_t (&c)[16], int half) {
-            uint32_t o[8];
+        tmem_ld16_issue(lane_base + (use % kSlots) * 2 * kLrCols, c0);
+        for (int pr = 0; pr < npairs; ++pr, ++use) {
+          const uint32_t pair_col = lane_base + (use % kSlots) * 2 * kLrCols;
+          const bool two = 2 * pr + 1 < p.r;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const float2 cq = make_float2(__uint_as_float(c[2 * q]), __uint_as_float(c[2 * q + 1]));
-              if constexpr (MODE == kLowRankForward) {
-                const float2 y = __ffma2_rn(cq, l2, base[8 * half + q]);
-                const float2 e = make_float2(fast_ex2(y.x), fast_ex2(y.y));
-                if (q & 1) sb = __fadd2_rn(sb, e);
-                else sa = __fadd2_rn(sa, e);
-              } else {
-                const float2 y = __ffma2_rn(cq, l2, __fadd2_rn(base[8 * half + q], make_float2(-lse2, -lse2)));
-                const float2 gq = __fmul2_rn(make_float2(fast_ex2(y.x), fast_ex2(y.y)), make_float2(-wt, -wt));
-                sum[8 * half + q] = __fadd2_rn(sum[8 * half + q], gq);
-                const __nv_bfloat162 h = __floats2bfloat162_rn(gq.x, gq.y);
-                o[q] = *reinterpret_cast<const uint32_t*>(&h);
+          for (int q = 0; q < 2; ++q) {
+            if (q == 1 && !two) break;
+            const uint32_t col = pair_col + q * kLrCols;
+            float2 sa = make_float2(0.f, 0.f), sb = sa;
+            auto eat = [&](const uint32_t (&c)[16], int half) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                const float2 y = __ffma2_rn(make_float2(__uint_as_float(c[2 * e]), __uint_as_float(c[2 * e + 1])), l2, base[8 * half + e]);
+                const float2 x = make_float2(fast_ex2(y.x), fast_ex2(y.y));
+                if (e & 1) sb = __fadd2_rn(sb, x);
+                else sa = __fadd2_rn(sa, x);
               }
+            };
+            tmem_ld_wait16(c0);
+            tmem_ld16_issue(col + 16, c1);                 // (columns past the block's width are not used)
+            if (here > 0) eat(c0, 0);
+            tmem_ld_wait16(c1);
+            if (q == 0 && two) {
+              tmem_ld16_issue(col + kLrCols, c0);
+            } else if (pr + 1 < npairs) {
+              if (!(ok = wait_slot(use + 1))) break;
+              tmem_ld16_issue(lane_base + ((use + 1) % kSlots) * 2 * kLrCols, c0);
             }
-            if constexpr (MODE == kLowRankGradient)
-              if (valid) st_global_v8_b32(dst + 16 * half, o);                   // 32-byte aligned: one full sector
-          };
-          if (here > 0) eat(ca0, 0);
-          tmem_ld_wait16(ca1);
-          if (jj + 1 < jc) {
-            if (!(ok = wait_slot(use + 1))) break;
-            tc_fence_after();
-            tmem_ld16_issue(lane_base + ((use + 1) % kSlots) * kCols, ca0);
-          }
-          if (here == 32) eat(ca1, 1);
-          if constexpr (MODE == kLowRankForward) {
+            if (here == 32) eat(c1, 1);
             float s = (sa.x + sa.y) + (sb.x + sb.y);
             float l = fast_lg2(s);                         // log2 of the sum relative to ref: a small number
             if (here > 0 && !__all_sync(kFull, s > 0x1p-60f && s < 0x1p120f)) {
@@ -396,9 +383,9 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kerne
                   tmem_ld_wait16(c);
                   if (16 * half < here) {
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                      const float b = q & 1 ? base[8 * half + q / 2].y : base[8 * half + q / 2].x;
-                      const float y = fmaf(__uint_as_float(c[q]), kLog2e, b);
+                    for (int e = 0; e < 16; ++e) {
+                      const float b = e & 1 ? base[8 * half + e / 2].y : base[8 * half + e / 2].x;
+                      const float y = fmaf(__uint_as_float(c[e]), kLog2e, b);
                       if (pass == 0) m = fmaxf(m, y);
                       else s += fast_ex2(y - m);
                     }
@@ -406,122 +393,210 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), 1) lowrank_logits_kerne
                 }
               l = m + fast_lg2(s);
             }
-            patch[jj * kLrPitch + lane] = l;
-          } else if (rel >= 0) {
-            dst[rel] = __float2bfloat16_rn(wt * (1.f - __expf(mine[(2 * kLrJ + jj) * kLrPitch + lane])));
+            if (valid && here > 0) *dst = l;               // position fastest: 128 contiguous bytes per warp, the next component's behind them
+            dst += 32;
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&ctl->tempty[use % kSlots]));
+          if (!ok) break;
+          release_slot(use);
         }
-        if (!ok) break;
-        if constexpr (MODE == kLowRankForward) {
-          if (here > 0) {                                  // the round's log-sums, transposed: 64 contiguous bytes per position
-            __syncwarp();
-            float* dst = p.log_sum + static_cast<size_t>(col0 / 32) * p.T * units + static_cast<size_t>(w.slot) * p.r + j0;
-            const int jj = lane & (kLrJ - 1);
-            if (jj < jc) {
+      } else {
+        // ---- gradient: the next eight columns are on their way while eight are consumed. g leaves by way of shared memory: stored by the
+        // threads, 32 bytes to a row each, the stores alone kept the load-store unit busy for half the time. A warp whose wait
+        // gave up goes on without waiting, so that the group's barriers still meet.
+        float2 sum[8];                                       // sum over the components,
+        float hot = 0.f;                                     // and of the weights, for the target's column
 #pragma unroll
-              for (int it = 0; it < 16; ++it) {
-                const int rr = it * 2 + (lane >> 4);
-                if (row0 + rr < p.T) dst[static_cast<size_t>(row0 + rr) * units + jj] = patch[jj * kLrPitch + rr];
-              }
+        for (int q = 0; q < 8; ++q) sum[q] = make_float2(0.f, 0.f);
+        const int tgt = valid ? p.targets[static_cast<size_t>(row) * p.n + w.slot] : -1;
+        // the target's column; -1: not here (nor is a refused target's, >= vv); -2: a marginalised byte, which has no gradient
+        const int rel = tgt < 0 ? -2 : (tgt >= col0 && tgt < min(col0 + 16, p.vv)) ? tgt - col0 : -1;
+        const uint32_t tiles = smem_u32(patches) + quarter * (4 * kLrTileBytes) + lane * 128;
+        const uint32_t piece = ((2 * sub) ^ (lane & 7)) * 16, piece1 = piece ^ 16;       // where the thread's two 16-byte pieces lie in its row
+        for (int pr = 0; pr < npairs; ++pr, ++use) {
+          const int jj = 2 * pr & (kLrRound - 1);          // the pair's first component inside its round
+          const uint32_t buffer = (use >> round_shift) & 1u;
+          if (jj == 0) {                                   // a new round: the next one, of this item or of the next item, is asked for
+            const uint32_t next_round = rounds + (buffer ^ 1u) * (12 * kLrRound * kLrPitch);
+            if (2 * pr + kLrRound < p.r) fetch_round(w, 2 * pr + kLrRound, next_round);
+            else if (item + gridDim.x < num_items) fetch_round(lowrank_item(p, item + gridDim.x), 0, next_round);
+            cp_async_commit();
+          }
+          const uint32_t mine = rounds + (buffer * (3 * kLrRound * kLrPitch) + lane) * 4;
+          const uint32_t col = lane_base + (use % kSlots) * 2 * kLrCols;
+          const bool two = 2 * pr + 1 < p.r;               // (r = 1: one component, and its copy with no weight)
+          const uint32_t tile = tiles + (use & 1u) * (2 * kLrTileBytes);
+          const uint32_t at0 = mine + jj * (4 * kLrPitch), at1 = at0 + (two ? 4 * kLrPitch : 0);
+          constexpr uint32_t kArray = 4 * kLrRound * kLrPitch;                       // from lse to weight to G
+          const bool more = pr + 1 < npairs || item + gridDim.x < num_items;       // pairs after this one
+          auto eat = [&](const uint32_t (&c)[8], int half, uint32_t to, float nl, float wt) {
+            uint32_t o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float2 y = __ffma2_rn(make_float2(__uint_as_float(c[2 * e]), __uint_as_float(c[2 * e + 1])), l2,
+                                          __fadd2_rn(base[4 * half + e], make_float2(nl, nl)));
+              const float2 gq = __fmul2_rn(make_float2(fast_ex2(y.x), fast_ex2(y.y)), make_float2(wt, wt));
+              sum[4 * half + e] = __fadd2_rn(sum[4 * half + e], gq);
+              const __nv_bfloat162 h = __floats2bfloat162_rn(gq.x, gq.y);
+              o[e] = *reinterpret_cast<const uint32_t*>(&h);
             }
-            __syncwarp();
+            st_shared_v4(to, o[0], o[1], o[2], o[3]);
+          };
+          float wt = rel != -2 ? -ld_shared_f32(at0 + kArray) : 0.f, nl = -ld_shared_f32(at0) * kLog2e;
+          hot -= wt;
+          tmem_ld_wait8(ca);
+          tmem_ld8_issue(col + 8, cb);
+          eat(ca, 0, tile + piece, nl, wt);
+          tmem_ld_wait8(cb);
+          tmem_ld8_issue(col + kLrCols, ca);
+          eat(cb, 1, tile + piece1, nl, wt);
+          wt = two && rel != -2 ? -ld_shared_f32(at1 + kArray) : 0.f;
+          nl = -ld_shared_f32(at1) * kLog2e;
+          hot -= wt;
+          tmem_ld_wait8(ca);
+          tmem_ld8_issue(col + kLrCols + 8, cb);
+          eat(ca, 0, tile + kLrTileBytes + piece, nl, wt);
+          tmem_ld_wait8(cb);
+          release_slot(use);
+          if (more && ok) ok = wait_slot(use + 1);
+          tmem_ld8_issue(lane_base + ((use + 1) % kSlots) * 2 * kLrCols, ca);        // (issued on every path: no copies of ca)
+          eat(cb, 1, tile + kLrTileBytes + piece1, nl, wt);
+          if (rel >= 0) {
+            const uint32_t to = tile + (rel & 8 ? piece1 : piece) + (rel & 7) * 2;
+            st_shared_bf16(to, __float2bfloat16_rn(ld_shared_f32(at0 + kArray) * (1.f - __expf(ld_shared_f32(at0 + 2 * kArray)))));
+            st_shared_bf16(to + kLrTileBytes, __float2bfloat16_rn(wt * (__expf(ld_shared_f32(at1 + 2 * kArray)) - 1.f)));
+          }
+          // the pair's g leaves; its buffer is written again two pairs on, after the barrier of the next pair, before which the
+          // thread that sends has seen this one read
+          fence_proxy_async_shared();
+          const bool sender = sub == 0 && lane == 0;
+          if (sender) bulk_wait_read<0>();
+          if (jj + 2 >= kLrRound || pr + 1 == npairs) cp_async_wait<0>();   // the next round's lse, weights and G: visible to the group behind the barrier
+          group_barrier();
+          if (sender && ok && w.mt * kBlockM + quarter * 32 < p.T) {
+            const uint32_t from = tile - lane * 128;
+            const int unit = w.slot * p.r + 2 * pr;
+            tma_store_3d(&p.tm_g, from, w.block * kLrCols, unit, w.mt * kBlockM + quarter * 32);
+            if (two) tma_store_3d(&p.tm_g, from + kLrTileBytes, w.block * kLrCols, unit + 1, w.mt * kBlockM + quarter * 32);
+            bulk_commit();
           }
         }
-      }
-      if constexpr (MODE == kLowRankGradient) if (valid && ok && here > 0) {
-        uint32_t o[16];
+        const bool stores = valid && here > 0;
+        if (stores && ok) {
+          uint32_t o[8];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          float2 sq = sum[q];
-          if (rel == 2 * q) sq.x += hot;
-          if (rel == 2 * q + 1) sq.y += hot;
-          const __nv_bfloat162 h = __floats2bfloat162_rn(sq.x, sq.y);
-          o[q] = *reinterpret_cast<const uint32_t*>(&h);
+          for (int q = 0; q < 8; ++q) {
+            float2 sq = sum[q];
+            if (rel == 2 * q) sq.x += hot;
+            if (rel == 2 * q + 1) sq.y += hot;
+            const __nv_bfloat162 h = __floats2bfloat162_rn(sq.x, sq.y);
+            o[q] = *reinterpret_cast<const uint32_t*>(&h);
+          }
+          st_global_v8_b32(p.s + static_cast<size_t>(row) * p.s_pitch + static_cast<size_t>(w.slot) * p.v + col0, o);
         }
-        __nv_bfloat16* dst = p.s + static_cast<size_t>(row) * p.s_pitch + static_cast<size_t>(w.slot) * p.v + col0;
-        st_global_v8_b32(dst, o);
-        if (here == 32) st_global_v8_b32(dst + 16, o + 8);
       }
     }
     cp_async_wait<0>();                                    // (after an abort) no copy is in flight when the CTA goes away
+    if (MODE == kLowRankGradient) {
+      tmem_ld_wait8(ca);
+      bulk_wait<0>();
+    }
   }
 
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc(tmem_base, kTmem);
   }
 }
 
 // G[t, i, j] = logit[target] - LSE over the unit: the LSE from the log-sums of 32 columns each and their references, the target's
 // logit as its base logit + A[i, j, target] . z[t, i, j] (k multiply-adds per thread; A in its repacked layout, so that the r
-// components of a slot read one contiguous row). One thread per (position, slot, component). Targets < 0 (marginalised): 0,
-// or NaN where they are refused draws; targets >= vv: NaN and the status bit.
-__global__ void lowrank_merge_kernel(const float* __restrict__ log_sum, const float* __restrict__ refs, const float* __restrict__ base,
-                                     const __nv_bfloat16* __restrict__ zhl, const __nv_bfloat16* __restrict__ Arep,
-                                     const int* __restrict__ targets, float* __restrict__ G, float* __restrict__ lse_out,
-                                     unsigned* status, size_t entries, int n, int r, int v, int vv, int k, int missing_is_nan) {
+// components of a slot read one contiguous row). Targets < 0 (marginalised): 0, or NaN where they are refused draws; targets >= vv:
+// NaN and the status bit. A CTA takes 32 positions of eight components of a slot: first lane = position and warp = component, so that
+// the log-sums are read as they were written; the LSEs change places through shared memory, and then the component runs fastest.
+constexpr int kMergeUnits = 8;
+template <int K>                                   // k
+__global__ void __launch_bounds__(256, K == 16 ? 4 : 3) lowrank_merge_kernel(const float* __restrict__ log_sum, const float* __restrict__ refs,
+                                                            const float* __restrict__ base, const __nv_bfloat16* __restrict__ zhl,
+                                                            const __nv_bfloat16* __restrict__ Arep, const int* __restrict__ targets,
+                                                            float* __restrict__ G, float* __restrict__ lse_out, unsigned* status, int T,
+                                                            int n, int r, int v, int vv, int missing_is_nan) {
+  __shared__ float tile[32][kMergeUnits + 1];
   grid_dependency_wait();
-  const size_t e = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= entries) return;
-  const size_t ti = e / r, tn = entries / r;       // (position, slot), and how many there are
-  const int blocks = (v + 31) / 32;
-  float best = -CUDART_INF_F, ref = 0.f, shift = 0.f, s = 0.f;
-  bool bad = false;
-  for (int q0 = 0; q0 < blocks; q0 += 4) {         // four log-sums in flight (sixteen: 123 against 62 us, r = 32 at T = 8192)
-    float lq[4], rq[4];
-    float top = best, top_ref = ref, top_shift = shift;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = blockIdx.y, t0 = blockIdx.x * 32, u0 = blockIdx.z * kMergeUnits, uc = min(kMergeUnits, r - u0);
+  const int blocks = (v + 31) / 32, tl = min(lane, T - 1 - t0);
+  const size_t units = static_cast<size_t>(n) * r;
+  // the thread's position and component behind the barrier: its target, its row of z and then of A are asked for first
+  const int row = threadIdx.x / uc, j = u0 + threadIdx.x - row * uc, t = t0 + row;      // (uc a power of two)
+  const bool has = row < 32 && t < T;
+  const size_t ti = static_cast<size_t>(t) * n + i, e = ti * r + j;
+  const int tgt = has ? targets[ti] : -1;
+  uint4 z[K / 4];
+  const uint4* zp = reinterpret_cast<const uint4*>(zhl + e * 2 * K);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      lq[q] = q0 + q < blocks ? log_sum[(q0 + q) * entries + e] : -CUDART_INF_F;
-      rq[q] = q0 + q < blocks ? refs[(q0 + q) * tn + ti] : 0.f;
+  for (int q = 0; q < K / 4; ++q) z[q] = tgt >= 0 ? __ldcs(zp + q) : make_uint4(0u, 0u, 0u, 0u);
+  if (warp < uc) {
+    const size_t strip0 = static_cast<size_t>(blockIdx.x) * blocks;
+    const float* ls = log_sum + (strip0 * units + static_cast<size_t>(i) * r + u0 + warp) * 32 + tl;
+    const float* rf = refs + (strip0 * n + i) * 32 + tl;
+    float best = -CUDART_INF_F, ref = 0.f, shift = 0.f, s = 0.f;
+    bool bad = false;
+    constexpr int kBatch = K == 16 ? 12 : 8;                           // log-sums in flight
+    for (int q0 = 0; q0 < blocks; q0 += kBatch) {
+      float lq[kBatch], rq[kBatch];
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        lq[q] = q0 + q < blocks ? __ldcs(ls + (q0 + q) * units * 32) : -CUDART_INF_F;
+        rq[q] = q0 + q < blocks ? rf[static_cast<size_t>(q0 + q) * n * 32] : 0.f;
+      }
+#pragma unroll
+      for (int h = 0; h < kBatch; h += 4) {              // four at a time, the largest so far the reference
+        if (q0 + h >= blocks) break;
+        float top = best, top_ref = ref, top_shift = shift;
+#pragma unroll
+        for (int q = h; q < h + 4; ++q) {
+          const float total = fmaf(rq[q], kLog2e, lq[q]);
+          bad |= total != total;
+          if (total > top) { top = total; top_ref = rq[q]; top_shift = lq[q]; }
+        }
+        if (q0 + h > 0) s *= fast_ex2(fmaf(ref - top_ref, kLog2e, shift - top_shift));
+#pragma unroll
+        for (int q = h; q < h + 4; ++q) s += fast_ex2(fmaf(rq[q] - top_ref, kLog2e, lq[q] - top_shift));
+        best = top;
+        ref = top_ref;
+        shift = top_shift;
+      }
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {                  // the largest so far is the reference
-      const float total = fmaf(rq[q], kLog2e, lq[q]);
-      bad |= total != total;
-      if (total > top) { top = total; top_ref = rq[q]; top_shift = lq[q]; }
-    }
-    if (q0 > 0) s *= fast_ex2(fmaf(ref - top_ref, kLog2e, shift - top_shift));
-#pragma unroll
-    for (int q = 0; q < 4; ++q) s += fast_ex2(fmaf(rq[q] - top_ref, kLog2e, lq[q] - top_shift));
-    best = top;
-    ref = top_ref;
-    shift = top_shift;
+    tile[lane][warp] = bad ? CUDART_NAN_F : fmaf(shift + fast_lg2(s), kLn2, ref);
   }
-  const float lse = bad ? CUDART_NAN_F : fmaf(shift + fast_lg2(s), kLn2, ref);
-  if (lse_out != nullptr) lse_out[e] = lse;
-  const int tgt = targets[ti];
-  if (tgt < 0) { G[e] = missing_is_nan ? CUDART_NAN_F : 0.f; return; }
-  if (tgt >= vv) {
-    G[e] = CUDART_NAN_F;
-    atomicOr(status, kStatusBadTarget);
-    return;
-  }
-  const int i = static_cast<int>(ti % n), j = static_cast<int>(e - ti * r);
-  const uint4* zp = reinterpret_cast<const uint4*>(zhl + e * 2 * k);
-  const uint4* ap = reinterpret_cast<const uint4*>(Arep + ((static_cast<size_t>(i) * v + tgt) * r + j) * k);
-  float d0 = 0.f, d1 = 0.f;
+  float dot = 0.f;
+  if (tgt >= 0 && tgt < vv) {
+    const uint4* ap = reinterpret_cast<const uint4*>(Arep + ((static_cast<size_t>(i) * v + tgt) * r + j) * K);
+    float d0 = 0.f, d1 = 0.f;
 #pragma unroll
-  for (int q = 0; q < kLrMaxRank / 8; ++q) {
-    if (q * 8 < k) {
-      const uint4 hi = zp[q], lo = zp[k / 8 + q], a = ap[q];
+    for (int q = 0; q < K / 8; ++q) {
+      const uint4 hi = z[q], lo = z[K / 8 + q], a = ap[q];
       const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&hi);
       const __nv_bfloat162* l2 = reinterpret_cast<const __nv_bfloat162*>(&lo);
       const __nv_bfloat162* a2 = reinterpret_cast<const __nv_bfloat162*>(&a);
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const float2 h = __bfloat1622float2(h2[t]), l = __bfloat1622float2(l2[t]), x = __bfloat1622float2(a2[t]);
-        d0 = fmaf(h.x + l.x, x.x, d0);
-        d1 = fmaf(h.y + l.y, x.y, d1);
+      for (int w = 0; w < 4; ++w) {
+        const float2 h = __bfloat1622float2(h2[w]), l = __bfloat1622float2(l2[w]), y = __bfloat1622float2(a2[w]);
+        d0 = fmaf(h.x + l.x, y.x, d0);
+        d1 = fmaf(h.y + l.y, y.y, d1);
       }
     }
+    dot = base[ti * v + tgt] + (d0 + d1);
   }
-  G[e] = base[ti * v + tgt] + (d0 + d1) - lse;
+  __syncthreads();
+  if (has) {
+    const float lse = tile[row][j - u0];
+    if (lse_out != nullptr) lse_out[e] = lse;
+    G[e] = tgt < 0 ? (missing_is_nan ? CUDART_NAN_F : 0.f) : tgt >= vv ? CUDART_NAN_F : dot - lse;
+    if (tgt >= vv) atomicOr(status, kStatusBadTarget);
+  }
   grid_launch_dependents();
 }
 

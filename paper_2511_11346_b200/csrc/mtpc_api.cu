@@ -560,7 +560,9 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
     const bool fits = btree_prefix_smem_floats(c.n, c.r, warps, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
     const size_t smem = btree_prefix_smem_floats(c.n, c.r, warps, fits) * sizeof(float);
     const int resident = sms_times_resident(h, smem);
-    launch_kernel(circuit_btree_prefix_kernel, W < resident ? W : resident, warps * 32, smem, st, overlapped(h), G, logw, out,
+    auto* kernel = c.r == 32 ? circuit_btree_prefix_kernel<32> : c.r == 16 ? circuit_btree_prefix_kernel<16>
+                   : c.r == 8 ? circuit_btree_prefix_kernel<8> : circuit_btree_prefix_kernel<0>;
+    launch_kernel(kernel, W < resident ? W : resident, warps * 32, smem, st, overlapped(h), G, logw, out,
                   prefix, msg, W, wpp, c.n, c.r, L.sum_rows, fits ? 1 : 0);
   } else {
     unsigned* counter = at<unsigned>(h, L.off_status) + kWorkCounterWord;
@@ -587,7 +589,8 @@ bool set_circuit_attributes() {
   bool ok = allow_full_smem(circuit_hmm_kernel);
   ok &= allow_full_smem(circuit_hmm_stream_kernel);
   ok &= allow_full_smem(circuit_btree_kernel);
-  ok &= allow_full_smem(circuit_btree_prefix_kernel);
+  ok &= allow_full_smem(circuit_btree_prefix_kernel<32>) && allow_full_smem(circuit_btree_prefix_kernel<16>);
+  ok &= allow_full_smem(circuit_btree_prefix_kernel<8>) && allow_full_smem(circuit_btree_prefix_kernel<0>);
   ok &= allow_full_smem(circuit_cp_prefix_kernel);
   return ok;
 }
@@ -1300,7 +1303,9 @@ int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cuda
     const size_t tsmem = btree_loss_smem_floats(c.n, c.r, tw, fits) * sizeof(float);
     const int grid = a.W < sms_times_resident(h, tsmem) ? a.W : sms_times_resident(h, tsmem);
     // (as a dependent, its CTAs crowded beside the projection's last ones: 350 -> 395 us at 4096 positions of a 16 x 32 head)
-    launch_kernel(circuit_btree_loss_backward_kernel, grid, tw * 32, tsmem, st, /*dependent=*/false, a, fits ? 1 : 0);
+    auto* kernel = c.r == 32 ? circuit_btree_loss_backward_kernel<32> : c.r == 16 ? circuit_btree_loss_backward_kernel<16>
+                   : c.r == 8 ? circuit_btree_loss_backward_kernel<8> : circuit_btree_loss_backward_kernel<0>;
+    launch_kernel(kernel, grid, tw * 32, tsmem, st, /*dependent=*/false, a, fits ? 1 : 0);
   } else {
     launch_kernel(circuit_btree_backward_kernel, resident, threads, smem, st, overlapped(h), a, counter);
   }
@@ -1313,7 +1318,8 @@ int set_backward_attributes(const mtpc_head* head) {
   if (circuit_backward_shape(head, false).warps == 0) return MTPC_ERR_UNSUPPORTED;   // (the loss kernels fit where these do)
   bool ok = allow_full_smem(circuit_hmm_backward_kernel);
   ok &= allow_full_smem(circuit_cp_loss_backward_kernel);
-  ok &= allow_full_smem(circuit_btree_loss_backward_kernel);
+  ok &= allow_full_smem(circuit_btree_loss_backward_kernel<32>) && allow_full_smem(circuit_btree_loss_backward_kernel<16>);
+  ok &= allow_full_smem(circuit_btree_loss_backward_kernel<8>) && allow_full_smem(circuit_btree_loss_backward_kernel<0>);
   ok &= allow_full_smem(circuit_hmm_loss_backward_kernel);
   ok &= allow_full_smem(circuit_hmm_static_loss_backward_kernel);
   ok &= allow_full_smem(circuit_btree_backward_kernel);

@@ -792,29 +792,32 @@ __global__ void circuit_btree_backward_kernel(const CircuitBackwardArgs a_, unsi
 //     S_c[z] = LSE_b(T_c[z][b] + prod_c[b]) gives dprod_c[b] = sum_z dS_c[z] exp(T_c[z][b] + prod_c[b] - S_c[z]), which reaches
 //     the two tokens of an owner. Here both parts of dL/dT_c[z][b] are at hand; through the row softmax of the table's logits:
 //     (its two summands) - exp(T_c[z][b]) (pd_c[z] + dS_c[z]).
-// Four passes over a window's n - 2 tables in shared memory (6 exponentials an entry), each table read from and its gradient
-// written to HBM once, as bf16. The n backward passes of the prefix lengths it replaces read and accumulated the window's 57 KB
+// Four passes over a window's n - 2 tables, in shared memory as probabilities (TreeSweep), each table read from and its gradient written
+// to HBM once, as bf16: with u = exp(in - max), e = exp(prod - max) and the sums of the two sweeps, every summand above is a product
+// of numbers per row and per column with the table's entry, so no entry takes another exponential (six, with log tables). The n backward
+// passes of the prefix lengths it replaces read and accumulated the window's 57 KB
 // n times (2186 us at 4096 windows, n = 16, r = 32, plus 48 us zeroing and 184 us converting the fp32 accumulators and 313 us
-// for the prefixes; this kernel does all of it in 350 us, its shared-memory and exponential work; HBM would take 80 us). One CTA per window, a warp per node of a level, as circuit_btree_prefix_kernel.
+// for the prefixes; this kernel on log tables, two CTAs an SM, did all of it in 498 us inside a training step; on probabilities, three
+// CTAs an SM, in 211; HBM would take 80). One CTA per window, a warp per node of a level, as circuit_btree_prefix_kernel.
 __host__ __device__ inline size_t btree_loss_smem_floats(int n, int r, int warps, bool tables_in_smem) {
   const size_t vr = (static_cast<size_t>(r) + 3) / 4 * 4;
   return btree_prefix_smem_floats(n, r, warps, tables_in_smem) +
-         (4 * static_cast<size_t>(n - 1) + n / 2 + 4 * static_cast<size_t>(warps)) * vr;
+         (3 * static_cast<size_t>(n - 1) + n / 2 + 4 * static_cast<size_t>(warps)) * vr;
 }
-__global__ void __launch_bounds__(256) circuit_btree_loss_backward_kernel(const CircuitBackwardArgs a_, int tables_in_smem) {
+template <int R>
+__global__ void __launch_bounds__(256, 3) circuit_btree_loss_backward_kernel(const CircuitBackwardArgs a_, int tables_in_smem) {
   grid_launch_dependents();
   grid_dependency_wait();
   extern __shared__ __align__(16) float sm[];
-  const int n = a_.n, r = a_.r;
-  TreeSweep t;
+  const int n = a_.n, r = R > 0 ? R : a_.r;
+  TreeSweep<R> t;
   t.init(sm, n, r, tables_in_smem != 0);
   const int lane = t.lane, wib = t.wib, warps = t.warps, vr = t.vr;
   const bool has = lane < r;
   float* dD = t.after();                           // [n - 1][vr] gradient of D
   float* pd = dD + (n - 1) * vr;                   // [n - 1][vr] gradient of in_c, per parent value
   float* dP = pd + (n - 1) * vr;                   // [n - 1][vr] gradient of prod_c
-  float* dS = dP + (n - 1) * vr;                   // [n - 1][vr] gradient of S_c
-  float* late = dS + (n - 1) * vr;                 // [n / 2][vr] c_{2m+1} rho_1
+  float* late = dP + (n - 1) * vr;                 // [n / 2][vr] c_{2m+1} rho_1
   float* vec = late + t.owners * vr + wib * 4 * vr;   // four vectors of this warp
   const int w0 = static_cast<int>(static_cast<long long>(blockIdx.x) * a_.W / gridDim.x);
   const int w1 = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * a_.W / gridDim.x);
@@ -844,38 +847,31 @@ __global__ void __launch_bounds__(256) circuit_btree_loss_backward_kernel(const 
     __syncthreads();
     for (int L = t.depth; L >= 1; --L) {           // reverse of the downward sweep
       for (int c = (1 << L) - 1 + wib; c <= (2 << L) - 2; c += warps) {
-        float* dc = vec;                           // the child's D and dD, read by every lane
+        float dd = 0.f, Dc = 0.f;
         if (has) {
           if (L < t.depth) dD[c * vr + lane] = pd[(2 * c + 1) * vr + lane] + pd[(2 * c + 2) * vr + lane];
-          dc[lane] = t.D[c * vr + lane];
+          dd = dD[c * vr + lane];
+          Dc = t.D[c * vr + lane];
         }
         const float in_z = has ? t.in_of(c) : 0.f;
+        float m;
+        const float u = t.scaled(in_z, m);
+        const float sum = has ? __expf(Dc - m) : 1.f;                    // sum_z u[z] T_c[z][lane]
+        float* x = vec;                            // dD_c over that sum
+        if (has) x[lane] = sum == 0.f ? 0.f : __fdividef(dd, sum);
+        const bool redo = __any_sync(kFull, sum < kTreeFloor && dd != 0.f);
         __syncwarp();
-        const float* tab = t.table_of(c);
-        if (has) {
-          const float* row = tab + lane * r;
-          float acc = 0.f;
-          if ((r & 3) == 0) {                      // float4 reads, rotated by the lane: conflict-free
-            const int Q = r / 4;
-            const float4* row4 = reinterpret_cast<const float4*>(row);
-            const float4* d4 = reinterpret_cast<const float4*>(dc);
-            const float4* g4 = reinterpret_cast<const float4*>(dD + c * vr);
-            float a1 = 0.f;
-#pragma unroll 4
-            for (int q = 0; q < Q; ++q) {
-              const int j = (q + lane) & (Q - 1);
-              const float4 x = row4[j], d = d4[j], e = g4[j];
-              acc = fmaf(e.x, __expf(in_z + x.x - d.x), acc);
-              a1 = fmaf(e.y, __expf(in_z + x.y - d.y), a1);
-              acc = fmaf(e.z, __expf(in_z + x.z - d.z), acc);
-              a1 = fmaf(e.w, __expf(in_z + x.w - d.w), a1);
-            }
-            acc += a1;
-          } else {
-            for (int b = 0; b < r; ++b) acc = fmaf(dD[c * vr + b], __expf(in_z + row[b] - dc[b]), acc);
+        float acc;
+        if (!redo) {
+          acc = u * row_dot(t.table_of(c), x, lane, r);
+        } else {                                   // terms may have been lost: with logarithms
+          acc = 0.f;
+          if (has) {
+            const float* row = t.log_table(c) + lane * r;
+            for (int b = 0; b < r; ++b) acc = fmaf(dD[c * vr + b], __expf(in_z + row[b] - t.D[c * vr + b]), acc);
           }
-          pd[c * vr + lane] = acc;
         }
+        if (has) pd[c * vr + lane] = acc;
         __syncwarp();
       }
       __syncthreads();
@@ -893,39 +889,84 @@ __global__ void __launch_bounds__(256) circuit_btree_loss_backward_kernel(const 
         const bool edge = c == (2 << L) - 2;       // on the right edge: no S
         const int j = (c - 1) >> 1;
         const bool edge_parent = j == (1 << L) - 2;   // (the root included)
-        float* inv = vec;                          // per parent value: in, S, dS and pd + dS
-        float* sv = vec + vr;
-        float* dsv = vec + 2 * vr;
-        float* sumv = vec + 3 * vr;
-        float prod = 0.f, Dc = 0.f, dDc = 0.f;
+        float in_z = 0.f, Sz = 0.f, ds = 0.f, sumz = 0.f, prod = 0.f, Dc = 0.f, dDc = 0.f;
         if (has) {
-          const float ds = edge ? 0.f : ((c & 1) ? pd[(c + 1) * vr + lane] : 0.f) + (edge_parent ? 0.f : dP[j * vr + lane]);
-          inv[lane] = t.in_of(c);
-          sv[lane] = edge ? 0.f : t.S[c * vr + lane];
-          dsv[lane] = ds;
-          sumv[lane] = pd[c * vr + lane] + ds;
-          if (!edge) prod = t.prod_of(c);
+          ds = edge ? 0.f : ((c & 1) ? pd[(c + 1) * vr + lane] : 0.f) + (edge_parent ? 0.f : dP[j * vr + lane]);
+          in_z = t.in_of(c);
+          sumz = pd[c * vr + lane] + ds;
+          if (!edge) {
+            Sz = t.S[c * vr + lane];
+            prod = t.prod_of(c);
+          }
           Dc = t.D[c * vr + lane];
           dDc = dD[c * vr + lane];
         }
-        __syncwarp();
-        const float* tab = t.table_of(c);
-        float acc = 0.f;
-        if (has) {
-          __nv_bfloat16* dst = drow + r + static_cast<size_t>(c - 1) * r * r + lane;
-          const float* col = tab + lane;
-#pragma unroll 4
-          for (int z = 0; z < r; ++z) {
-            const float x = col[z * r];
-            float xi = dDc * __expf(inv[z] + x - Dc);
-            if (!edge) {
-              const float e2 = dsv[z] * __expf(x + prod - sv[z]);
-              acc += e2;
-              xi += e2;
+        float mi, mp;
+        const float u = t.scaled(in_z, mi);
+        const float e = edge ? 0.f : t.scaled(prod, mp);
+        const float below = has ? __expf(Dc - mi) : 1.f;                 // sum_z u[z] T_c[z][lane]
+        const float across = has && !edge ? __expf(Sz - mp) : 1.f;       // sum_b T_c[lane][b] e[b]
+        const bool redo = __any_sync(kFull, (below < kTreeFloor && dDc != 0.f) || (across < kTreeFloor && ds != 0.f));
+        __nv_bfloat16* dst = drow + r + static_cast<size_t>(c - 1) * r * r;
+        if (!redo) {
+          // dL/dT_c[z][b] = T_c[z][b] (u[z] x[b] + y[z] e[b] - (pd + dS)[z]), x = dD / below, y = dS / across; dprod[b] = e[b] sum_z T y
+          const float x = below == 0.f ? 0.f : __fdividef(dDc, below);
+          float4* zv = reinterpret_cast<float4*>(vec);
+          if (has) zv[lane] = make_float4(u, across == 0.f ? 0.f : __fdividef(ds, across), sumz, 0.f);
+          __syncwarp();
+          const float* tab = t.table_of(c);
+          if (r == 32) {                           // a lane takes two columns of every other row: 4-byte stores
+            const int half = lane >> 4, b = 2 * (lane & 15);
+            const float x0 = __shfl_sync(kFull, x, b), x1 = __shfl_sync(kFull, x, b + 1);
+            const float e0 = __shfl_sync(kFull, e, b), e1 = __shfl_sync(kFull, e, b + 1);
+            float a0 = 0.f, a1 = 0.f;
+#pragma unroll 8
+            for (int q = 0; q < 16; ++q) {
+              const int z = 2 * q + half;
+              const float2 p = *reinterpret_cast<const float2*>(tab + z * 32 + b);
+              const float4 f = zv[z];
+              a0 = fmaf(p.x, f.y, a0);
+              a1 = fmaf(p.y, f.y, a1);
+              const float g0 = p.x * fmaf(f.y, e0, fmaf(f.x, x0, -f.z)), g1 = p.y * fmaf(f.y, e1, fmaf(f.x, x1, -f.z));
+              *reinterpret_cast<__nv_bfloat162*>(dst + z * 32 + b) = __floats2bfloat162_rn(g0, g1);
             }
-            dst[z * r] = __float2bfloat16_rn(fmaf(-__expf(x), sumv[z], xi));
+            a0 += __shfl_xor_sync(kFull, a0, 16);
+            a1 += __shfl_xor_sync(kFull, a1, 16);
+            if (half == 0) *reinterpret_cast<float2*>(dP + c * vr + b) = make_float2(a0 * e0, a1 * e1);
+          } else if (has) {
+            float a0 = 0.f;
+            for (int z = 0; z < r; ++z) {
+              const float p = tab[z * r + lane];
+              const float4 f = zv[z];
+              a0 = fmaf(p, f.y, a0);
+              dst[z * r + lane] = __float2bfloat16_rn(p * fmaf(f.y, e, fmaf(f.x, x, -f.z)));
+            }
+            dP[c * vr + lane] = a0 * e;
           }
-          dP[c * vr + lane] = acc;
+        } else {                                   // terms may have been lost: with logarithms
+          float *inv = vec, *sv = vec + vr, *dsv = vec + 2 * vr, *sumv = vec + 3 * vr;
+          if (has) {
+            inv[lane] = in_z;
+            sv[lane] = Sz;
+            dsv[lane] = ds;
+            sumv[lane] = sumz;
+          }
+          __syncwarp();
+          if (has) {
+            const float* col = t.log_table(c) + lane;
+            float acc = 0.f;
+            for (int z = 0; z < r; ++z) {
+              const float l = col[z * r];
+              float xi = dDc * __expf(inv[z] + l - Dc);
+              if (!edge) {
+                const float e2 = dsv[z] * __expf(l + prod - sv[z]);
+                acc += e2;
+                xi += e2;
+              }
+              dst[z * r + lane] = __float2bfloat16_rn(fmaf(-__expf(l), sumv[z], xi));
+            }
+            dP[c * vr + lane] = acc;
+          }
         }
         __syncwarp();
       }

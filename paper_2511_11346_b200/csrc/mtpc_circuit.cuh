@@ -293,44 +293,64 @@ __global__ void circuit_btree_kernel(const float* __restrict__ G, const float* _
   }
 }
 
-// LSE_z(in[z] + tab[z][lane]): the message down to a child with value `lane`; tab [r, r] and in [r] in shared memory.
-template <int R>
-__device__ __forceinline__ float down_layer_vec(const float* tab, const float* in, int lane) {
-  if (lane >= R) return 0.f;
-  const float4* in4 = reinterpret_cast<const float4*>(in);
-  float v[R];
-#pragma unroll
-  for (int q = 0; q < R / 4; ++q) {
-    const float4 a = in4[q];
-    v[4 * q] = a.x + tab[(4 * q) * R + lane];
-    v[4 * q + 1] = a.y + tab[(4 * q + 1) * R + lane];
-    v[4 * q + 2] = a.z + tab[(4 * q + 2) * R + lane];
-    v[4 * q + 3] = a.w + tab[(4 * q + 3) * R + lane];
-  }
-  float m = v[0];
-#pragma unroll
-  for (int q = 1; q < R; ++q) m = fmaxf(m, v[q]);
+// LSE_q(vec[q] + tab[q * step]) by one lane, for steps that are rarely taken: a row of a log table (step 1) or a column (step r).
+__device__ __noinline__ float layer_lse(const float* tab, int step, const float* vec, int r) {
+  float m = -CUDART_INF_F;
+  for (int q = 0; q < r; ++q) m = fmaxf(m, vec[q] + tab[q * step]);
   if (m == -CUDART_INF_F) m = 0.f;
   float s = 0.f;
-#pragma unroll
-  for (int q = 0; q < R; ++q) s += __expf(v[q] - m);
+  for (int q = 0; q < r; ++q) s += __expf(vec[q] + tab[q * step] - m);
   return m + __logf(s);                            // NaN evidence survives through the sum
 }
-__device__ __forceinline__ float down_layer(const float* tab, const float* in, int lane, int r) {
-  switch (r) {
-    case 32: return down_layer_vec<32>(tab, in, lane);
-    case 16: return down_layer_vec<16>(tab, in, lane);
-    case 8: return down_layer_vec<8>(tab, in, lane);
-    case 4: return down_layer_vec<4>(tab, in, lane);
-    default: break;
+// sum_b tab[lane][b] vec[b] and sum_z vec[z] tab[z][lane] over a table [r, r] and a vector [r] in shared memory (16-byte aligned for r >= 4);
+// lanes past r return 0. Rows are read as float4 rotated by the lane (see sum_layer_staged_vec).
+template <int R>
+__device__ __forceinline__ float row_dot_vec(const float* tab, const float* vec, int lane) {
+  constexpr int Q = R / 4;
+  const float4 *row4 = reinterpret_cast<const float4*>(tab + lane * R), *v4 = reinterpret_cast<const float4*>(vec);
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 4
+  for (int q = 0; q < Q; ++q) {
+    const int j = (q + lane) & (Q - 1);
+    const float4 a = row4[j], v = v4[j];
+    s0 = fmaf(a.x, v.x, s0);
+    s1 = fmaf(a.y, v.y, s1);
+    s2 = fmaf(a.z, v.z, s2);
+    s3 = fmaf(a.w, v.w, s3);
   }
+  return (s0 + s1) + (s2 + s3);
+}
+__device__ __forceinline__ float row_dot(const float* tab, const float* vec, int lane, int r) {
   if (lane >= r) return 0.f;
-  float m = -CUDART_INF_F;
-  for (int z = 0; z < r; ++z) m = fmaxf(m, in[z] + tab[z * r + lane]);
-  if (m == -CUDART_INF_F) m = 0.f;
+  if (r == 32) return row_dot_vec<32>(tab, vec, lane);
+  if (r == 16) return row_dot_vec<16>(tab, vec, lane);
+  if (r == 8) return row_dot_vec<8>(tab, vec, lane);
   float s = 0.f;
-  for (int z = 0; z < r; ++z) s += __expf(in[z] + tab[z * r + lane] - m);
-  return m + __logf(s);
+  for (int b = 0; b < r; ++b) s = fmaf(tab[lane * r + b], vec[b], s);
+  return s;
+}
+template <int R>
+__device__ __forceinline__ float col_dot_vec(const float* tab, const float* vec, int lane) {
+  const float4* v4 = reinterpret_cast<const float4*>(vec);
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 4
+  for (int q = 0; q < R / 4; ++q) {
+    const float4 v = v4[q];
+    s0 = fmaf(v.x, tab[(4 * q) * R + lane], s0);
+    s1 = fmaf(v.y, tab[(4 * q + 1) * R + lane], s1);
+    s2 = fmaf(v.z, tab[(4 * q + 2) * R + lane], s2);
+    s3 = fmaf(v.w, tab[(4 * q + 3) * R + lane], s3);
+  }
+  return (s0 + s1) + (s2 + s3);
+}
+__device__ __forceinline__ float col_dot(const float* tab, const float* vec, int lane, int r) {
+  if (lane >= r) return 0.f;
+  if (r == 32) return col_dot_vec<32>(tab, vec, lane);
+  if (r == 16) return col_dot_vec<16>(tab, vec, lane);
+  if (r == 8) return col_dot_vec<8>(tab, vec, lane);
+  float s = 0.f;
+  for (int z = 0; z < r; ++z) s = fmaf(vec[z], tab[z * r + lane], s);
+  return s;
 }
 // log-sum-exp of one value per lane (lanes without one pass -inf). All lanes return it.
 __device__ __forceinline__ float warp_lse_nan(float x) {
@@ -354,8 +374,15 @@ __device__ __forceinline__ float warp_lse_nan(float x) {
 // memory round trip, and a batch has several windows' tables in flight per SM. tables_in_smem == 0 (they do not fit: n = 64 at
 // r = 32): each warp stages the table it needs. A CTA takes a contiguous run of windows and keeps the tables while the
 // position stays the same. Measured against one warp per window and a path per prefix: 4096 windows at n = 16, r = 32:
-// 256 -> 148 us; 108 windows at n = 8: 36 -> 6 us. Shared memory: btree_prefix_smem_floats.
+// 256 -> 148 us; 108 windows at n = 8: 36 -> 6 us.
+// In shared memory the tables are probabilities, exponentiated once on their way there, so that a step of either sweep is one warp
+// maximum, r multiply-adds per lane and one logarithm (r exponentials of sums, a maximum over them and their sum before). Where a
+// step's sum falls below kTreeFloor against its maximum, so that terms may have been lost, the warp takes the step once more with
+// logarithms from the log tables in global memory. (4096 windows at n = 16, r = 32, inside a draft: 102 -> 96 us, latency of a window's
+// levels; 27 positions of 4 windows at n = 8: 8.7 -> 5.8.) Shared memory: btree_prefix_smem_floats.
+constexpr float kTreeFloor = 0x1p-100f;
 // One window of a tree sweep, shared by a CTA. vr: pitch of the [r] vectors (r rounded up to 4 floats).
+template <int R>                                   // r, where the kernel is built for it (0: any)
 struct TreeSweep {
   int n, r, vr, owners, first_leaf_node, depth;    // depth: the owners' level; level L holds the nodes 2^L - 1 .. 2^(L+1) - 2
   int wib, lane, warps;
@@ -365,7 +392,7 @@ struct TreeSweep {
   bool resident;
 
   __device__ void init(float* sm, int n_, int r_, bool tables_in_smem) {
-    n = n_; r = r_; vr = (r + 3) / 4 * 4;
+    n = n_; r = R > 0 ? R : r_; vr = (r + 3) / 4 * 4;
     owners = n / 2; first_leaf_node = owners - 1; depth = 31 - __clz(owners);
     wib = threadIdx.x >> 5; lane = threadIdx.x & 31; warps = blockDim.x >> 5;
     resident = tables_in_smem;
@@ -376,27 +403,44 @@ struct TreeSweep {
     vec = gs + n * vr + wib * vr;
   }
   __device__ float* after() const { return gs + (n + warps) * vr; }   // the shared memory past the sweep's own
+  __device__ const float* log_table(int c) const { return lw + r + static_cast<size_t>(c - 1) * r * r; }
+  // Copies `count` log-probabilities to shared memory, by `threads` threads of which this is the `thread`th, ..
+  __device__ static bool whole_vectors(const float* src, int count) { return (count & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0; }
+  __device__ static void fetch_table(float* dst, const float* __restrict__ src, int count, int thread, int threads) {
+    if (whole_vectors(src, count)) {
+      for (int e = thread * 4; e < count; e += threads * 4) cp_async_16(dst + e, src + e);
+    } else {
+      for (int e = thread; e < count; e += threads) cp_async_4(dst + e, src + e);
+    }
+    cp_async_commit();
+  }
+  // .. and, once they are there, makes probabilities of those that the thread itself has copied.
+  __device__ static void exponentiate(float* dst, const float* src, int count, int thread, int threads) {
+    cp_async_wait<0>();
+    if (whole_vectors(src, count)) {
+#pragma unroll 2
+      for (int e = thread * 4; e < count; e += threads * 4) {
+        const float4 x = *reinterpret_cast<const float4*>(dst + e);
+        *reinterpret_cast<float4*>(dst + e) = make_float4(__expf(x.x), __expf(x.y), __expf(x.z), __expf(x.w));
+      }
+    } else {
+      for (int e = thread; e < count; e += threads) dst[e] = __expf(dst[e]);
+    }
+  }
   // Start of window w: the position's tables (unless they are still there), its evidence, log omega of the root.
   __device__ void load(const float* __restrict__ g, const float* __restrict__ lw_, bool new_tables) {
     lw = lw_;
-    if (resident && new_tables) {
-      const int count = (n - 2) * r * r;
-      if ((count & 3) == 0 && (reinterpret_cast<uintptr_t>(lw + r) & 15u) == 0) {
-        for (int e = threadIdx.x * 4; e < count; e += blockDim.x * 4) cp_async_16(tabs + e, lw + r + e);
-      } else {
-        for (int e = threadIdx.x; e < count; e += blockDim.x) cp_async_4(tabs + e, lw + r + e);
-      }
-      cp_async_commit();
-    }
+    const bool fetch = resident && new_tables;
+    if (fetch) fetch_table(tabs, lw + r, (n - 2) * r * r, threadIdx.x, blockDim.x);
     for (int e = threadIdx.x; e < n * r; e += blockDim.x) gs[(e / r) * vr + e % r] = g[e];
     if (threadIdx.x < r) D[threadIdx.x] = lw[threadIdx.x];
-    cp_async_wait<0>();
+    if (fetch) exponentiate(tabs, lw + r, (n - 2) * r * r, threadIdx.x, blockDim.x);
     __syncthreads();
   }
-  __device__ const float* table_of(int c) const {  // node c's table; not resident: staged into the warp's own tile
+  __device__ const float* table_of(int c) const {  // node c's probabilities; not resident: staged into the warp's own tile
     if (resident) return tabs + (c - 1) * r * r;
-    warp_table_load_async(tabs + wib * r * r, lw + r + static_cast<size_t>(c - 1) * r * r, r * r, lane);
-    cp_async_wait<0>();
+    fetch_table(tabs + wib * r * r, log_table(c), r * r, lane, 32);
+    exponentiate(tabs + wib * r * r, log_table(c), r * r, lane, 32);
     __syncwarp();
     return tabs + wib * r * r;
   }
@@ -407,12 +451,29 @@ struct TreeSweep {
   __device__ float in_of(int c) const {            // what comes down to node c's table, per parent value
     return D[((c - 1) >> 1) * vr + lane] + ((c & 1) ? 0.f : S[(c - 1) * vr + lane]);
   }
+  // exp(x - m) per lane, m the warp's maximum of x (0 if there is none); lanes past r: 0.
+  __device__ float scaled(float x, float& m) const {
+    if (lane >= r) x = -CUDART_INF_F;
+    m = warp_max_nan(x);
+    if (m == -CUDART_INF_F) m = 0.f;
+    return __expf(x - m);
+  }
   __device__ void up() {                           // S of every node that is not on the right edge
     for (int L = depth; L >= 1; --L) {
       for (int c = (1 << L) - 1 + wib; c < (2 << L) - 2; c += warps) {
-        if (lane < r) vec[lane] = prod_of(c);
+        const float prod = lane < r ? prod_of(c) : 0.f;
+        float m;
+        const float e = scaled(prod, m);
+        if (lane < r) vec[lane] = e;
         __syncwarp();
-        const float sc = sum_layer_staged(table_of(c), vec, lane, r);
+        const float q = row_dot(table_of(c), vec, lane, r);
+        float sc = m + __logf(q);
+        if (__any_sync(kFull, lane < r && q < kTreeFloor)) {
+          __syncwarp();
+          if (lane < r) vec[lane] = prod;
+          __syncwarp();
+          if (lane < r) sc = layer_lse(log_table(c) + lane * r, 1, vec, r);
+        }
         if (lane < r) S[c * vr + lane] = sc;
         __syncwarp();
       }
@@ -422,9 +483,19 @@ struct TreeSweep {
   __device__ void down() {                         // D of every node
     for (int L = 1; L <= depth; ++L) {
       for (int c = (1 << L) - 1 + wib; c <= (2 << L) - 2; c += warps) {
-        if (lane < r) vec[lane] = in_of(c);
+        const float in = lane < r ? in_of(c) : 0.f;
+        float m;
+        const float u = scaled(in, m);
+        if (lane < r) vec[lane] = u;
         __syncwarp();
-        const float dc = down_layer(table_of(c), vec, lane, r);
+        const float q = col_dot(table_of(c), vec, lane, r);
+        float dc = m + __logf(q);
+        if (__any_sync(kFull, lane < r && q < kTreeFloor)) {
+          __syncwarp();
+          if (lane < r) vec[lane] = in;
+          __syncwarp();
+          if (lane < r) dc = layer_lse(log_table(c) + lane, r, vec, r);
+        }
         if (lane < r) D[c * vr + lane] = dc;
         __syncwarp();
       }
@@ -436,14 +507,16 @@ __host__ __device__ inline size_t btree_prefix_smem_floats(int n, int r, int war
   const size_t rr = static_cast<size_t>(r) * r, vr = (static_cast<size_t>(r) + 3) / 4 * 4;
   return ((tables_in_smem ? (n - 2) * rr : warps * rr) + 3) / 4 * 4 + (2 * static_cast<size_t>(n - 1) + n + warps) * vr;
 }
-__global__ void __launch_bounds__(256) circuit_btree_prefix_kernel(const float* __restrict__ G, const float* __restrict__ logw,
+template <int R>
+__global__ void __launch_bounds__(256, 3) circuit_btree_prefix_kernel(const float* __restrict__ G, const float* __restrict__ logw,
                                                                    float* __restrict__ out, float* __restrict__ prefix,
-                                                                   float* __restrict__ msg, int W, int wpp, int n, int r,
+                                                                   float* __restrict__ msg, int W, int wpp, int n, int r_,
                                                                    int sum_rows, int tables_in_smem) {
   extern __shared__ __align__(16) float sm[];
   grid_launch_dependents();
   grid_dependency_wait();   // G and log omega come from the kernels before this one
-  TreeSweep t;
+  const int r = R > 0 ? R : r_;
+  TreeSweep<R> t;
   t.init(sm, n, r, tables_in_smem != 0);
   const int w0 = static_cast<int>(static_cast<long long>(blockIdx.x) * W / gridDim.x);
   const int w1 = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * W / gridDim.x);

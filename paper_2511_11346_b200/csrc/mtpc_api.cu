@@ -340,8 +340,8 @@ int check_launch() { return cudaGetLastError() == cudaSuccess ? MTPC_OK : MTPC_E
 // Launch `kernel`, optionally allowed to start before the kernel ahead of it in the stream has finished (programmatic
 // dependent launch): such a kernel calls grid_dependency_wait() before it touches global memory, so what overlaps is its launch and
 // set-up (about 2 us a kernel). cluster > 1: in clusters of that many CTAs.
-// Two kernels copy a static head's transition tables before they wait (draft_slot_kernel, circuit_hmm_kernel). The tables are written by
-// a plain launch (bind_parameters), and the first kernel of every call that runs one of the two lets its dependents in only after
+// Three kernels copy a static head's transition tables before they wait (draft_slot_kernel, circuit_hmm_kernel and the static HMM's Eq. 6
+// kernel). The tables are written by a plain launch (bind_parameters), and the first kernel of every call that runs one of them lets its dependents in only after
 // its own wait (the fp32 conversion, the projection, the weight pass), so the tables are complete before any of them starts.
 template <typename... Params, typename... Args>
 void launch_clusters(void (*kernel)(Params...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent,
@@ -1709,7 +1709,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   fail |= cudaFuncSetAttribute(draft_slot_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
   fail |= cudaFuncSetAttribute(draft_slot_kernel<true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
   fail |= !set_circuit_attributes();
-  fail |= !allow_full_smem(spec_accept_kernel);
+  fail |= !allow_full_smem(spec_accept_kernel<true>) || !allow_full_smem(spec_accept_kernel<false>);
   fail |= cudaMemsetAsync(h->ws + L.off_status, 0, 256, st) != cudaSuccess;
   if (fail) { delete h; return MTPC_ERR_CUDA; }
 
@@ -1817,6 +1817,7 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
   const size_t smem = accept_smem_floats(c.r, c.v) * sizeof(float);
   if (smem > static_cast<size_t>(kSmemLimit)) return MTPC_ERR_UNSUPPORTED;      // a residual row of more than ~56k symbols
   const int threads = accept_threads(c.v);
+  auto* accept_kernel = W <= head->num_sms ? spec_accept_kernel<true> : spec_accept_kernel<false>;
   PhaseTimer pt(head, st);
   float* const msg = at<float>(head, L.off_msg);
   // The slot messages are formed here, from the evidence and log omega the draft left, unless they are sure to be the last draft's
@@ -1832,7 +1833,7 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
   if (head->draft_logits) {
     // every logit of the drafted positions is still in the workspace
     pt.begin();
-    launch_kernel(spec_accept_kernel, W, threads, smem, st, overlapped(head), at<float>(head, L.off_logits),
+    launch_kernel(accept_kernel, W, threads, smem, st, overlapped(head), at<float>(head, L.off_logits),
                   at<float>(head, L.off_unit_lse), msg, draft_bytes, prefix_logprob, target_probs, accept_uniforms, out_accepted,
                   out_next_byte, at<unsigned>(head, L.off_status), W, wpp, c.n, c.r, c.v, valid_symbols(c),
                   static_cast<const int*>(nullptr));
@@ -1882,7 +1883,7 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
       int rcf = check_launch();
       if (rcf != MTPC_OK) return rcf;
       pt.begin();
-      launch_kernel(spec_accept_kernel, wc, threads, smem, st, overlapped(head), lg, lse, msg + w0 * c.n * c.r, xb,
+      launch_kernel(accept_kernel, wc, threads, smem, st, overlapped(head), lg, lse, msg + w0 * c.n * c.r, xb,
                     pre, tp, ua, out_accepted + w0, out_next_byte + w0, at<unsigned>(head, L.off_status), wc, wpp, c.n, c.r, c.v,
                     valid_symbols(c), row_of);
       head->launches++;
@@ -1916,7 +1917,7 @@ int mtpc_speculative_accept(mtpc_head* head, int32_t P, int32_t wpp, const int32
     pt.end();
     if (rc2 != MTPC_OK) return rc2;
     pt.begin();
-    launch_kernel(spec_accept_kernel, wc, threads, smem, st, overlapped(head), lg, lse, msg + w0 * c.n * c.r, xb,
+    launch_kernel(accept_kernel, wc, threads, smem, st, overlapped(head), lg, lse, msg + w0 * c.n * c.r, xb,
                   pre, tp, ua, out_accepted + w0, out_next_byte + w0, at<unsigned>(head, L.off_status), wc, wpp, c.n, c.r, c.v,
                   valid_symbols(c), row_of);
     head->launches++;

@@ -673,13 +673,21 @@ __global__ void __launch_bounds__(32 * kHmmWarps, 5) circuit_hmm_kernel(
     const float* tb = tables + static_cast<size_t>(pos_tab) * table_stride;
     float* mw = msg != nullptr && valid && part == 0 ? msg + static_cast<size_t>(w) * n * r : nullptr;
     float alpha = -CUDART_INF_F, gi = 0.f;
+    // the evidence of the later slots: with prefixes, all of it in one trip to the rows the messages will take, else a step ahead of use
+    if (prefix != nullptr && valid)
+      for (int e = r + lane; e < n * r; e += 32) cp_async_4(alphas + e + (e >> (31 - __clz(r))), g + e);
     if (active && valid) {
       const float l0 = logw[static_cast<size_t>(w / wpp) * sum_rows + k];
       if (mw != nullptr) mw[k] = l0;
       alpha = l0 + g[k];
-      if (n > 1) gi = g[r + k];
+      if (n > 1 && prefix == nullptr) gi = g[r + k];
     }
-    if (prefix != nullptr && active && part == 0) alphas[k] = alpha;
+    if (prefix != nullptr) {
+      if (active && part == 0) alphas[k] = alpha;
+      cp_async_commit();
+      cp_async_wait<0>();
+      __syncwarp();
+    }
     for (int t0 = 0; t0 < n - 1; t0 += chunk_tables) {
       const int nt = min(chunk_tables, n - 1 - t0);
       if (loaded_pos != pos_tab || loaded_first != t0) {
@@ -704,11 +712,12 @@ __global__ void __launch_bounds__(32 * kHmmWarps, 5) circuit_hmm_kernel(
       }
       if (!valid) continue;
       for (int i = t0 + 1; i <= t0 + nt; ++i) {
-        const float g_next = (active && i + 1 < n) ? g[(i + 1) * r + k] : 0.f;
+        const float g_next = (prefix == nullptr && active && i + 1 < n) ? g[(i + 1) * r + k] : 0.f;
+        if (prefix != nullptr && active) gi = alphas[i * (r + 1) + k];
         const float c = hmm_forward_step<false>(alpha, evec + (i & 1) * 32, E + (i - 1 - t0) * rr, l, r);
         if (mw != nullptr && active) mw[i * r + k] = c;
         alpha = active ? c + gi : -CUDART_INF_F;
-        gi = g_next;
+        if (prefix == nullptr) gi = g_next;
         if (prefix != nullptr && active && part == 0) alphas[i * (r + 1) + k] = alpha;
       }
     }

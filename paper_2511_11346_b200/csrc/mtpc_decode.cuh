@@ -831,6 +831,10 @@ inline int accept_threads(int v) { return v >= kAcceptMaxThreads ? kAcceptMaxThr
 // programmatic dependent the kernel went from 59 to 6 us at HMM n = 16, 128 windows; 12 to 5 us for one mixture window; 569 to
 // 49 us for 4096 tree windows of n = 16. row_of != NULL (logits recomputed after a long draft): `logits` [rows, r v] and `unit_lse` [rows, r] hold only the
 // slot of each rejected window's first rejected byte, at row row_of[w].
+// AHEAD: a thread asks for its byte's target probability and the logits of 32 units before the weights are formed, which takes two
+// trips to memory out of the chain and twice the registers. 128 windows of an HMM, r = 32: 9.7 -> 6.8 us behind the circuit; 108 of a tree
+// 7.5 -> 6.7; but 1024 windows of a mixture 11.7 -> 15.0, so only while every window has an SM to itself.
+template <bool AHEAD>
 __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
     const float* __restrict__ logits, const float* __restrict__ unit_lse, const float* __restrict__ msg,
     const int* __restrict__ bytes, const float* __restrict__ prefix, const float* __restrict__ target,
@@ -886,6 +890,17 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
     const size_t lrow = row_of != nullptr ? static_cast<size_t>(row_of[w]) : static_cast<size_t>(pos) * n + s;
     const float* ulse = unit_lse + lrow * r;
     const float* lg = logits + lrow * r * v;             // [r, v] logits of slot s
+    float ahead[AHEAD ? 32 : 1], t_ahead;
+    if constexpr (AHEAD) {
+      const int b = threadIdx.x < vv ? threadIdx.x : 0;
+      t_ahead = trow[b];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) ahead[e] = e < r ? lg[static_cast<size_t>(e) * v + b] : 0.f;
+      if (r > 16) {
+#pragma unroll
+        for (int e = 16; e < 32; ++e) ahead[e] = lg[static_cast<size_t>(e) * v + b];
+      }
+    }
     if (wib == 0) {
       const float* mw = msg + (static_cast<size_t>(w) * n + s) * r;
       float c[4], l[4];
@@ -913,9 +928,33 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
     for (int b = threadIdx.x; b < v; b += blockDim.x) {
       float res = 0.f;
       if (b < vv) {
-        const float t = trow[b];
+        const bool first = AHEAD && b == threadIdx.x;
+        const float t = first ? t_ahead : trow[b];
         float q0 = 0.f, q1 = 0.f;
         int k = 0;
+        if constexpr (AHEAD) {
+          if (first && r >= 16) {
+#pragma unroll
+            for (int e = 0; e < 16; e += 2) {
+              q0 += fast_ex2(fmaf(ahead[e], kLog2e, cw[e]));
+              q1 += fast_ex2(fmaf(ahead[e + 1], kLog2e, cw[e + 1]));
+            }
+            k = 16;
+            if (r > 16) {
+#pragma unroll
+              for (int e = 16; e < 32; e += 2) {
+                q0 += fast_ex2(fmaf(ahead[e], kLog2e, cw[e]));
+                q1 += fast_ex2(fmaf(ahead[e + 1], kLog2e, cw[e + 1]));
+              }
+              k = 32;
+            }
+          } else if (first) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+              if (e < r) q0 += fast_ex2(fmaf(ahead[e], kLog2e, cw[e]));
+            k = r;
+          }
+        }
 #pragma unroll 1
         for (; k + 16 <= r; k += 16) {                   // sixteen rows' logits in flight, two accumulation chains
           float xv[16];

@@ -626,17 +626,23 @@ __global__ void __launch_bounds__(kExpandThreads) lowrank_expand_kernel(const fl
                                                                         const __nv_bfloat16* __restrict__ A,
                                                                         float* __restrict__ logits, int P, int n, int r,
                                                                         int v, int k) {
-  extern __shared__ float zs[];                                 // [P, k]
+  extern __shared__ __align__(16) float zs[];                   // [P, k]
   grid_launch_dependents();
   grid_dependency_wait();
   const int unit = blockIdx.x, i = unit / r;
   const int b = blockIdx.y * kExpandThreads + threadIdx.x;
   const size_t units = static_cast<size_t>(n) * r;
   for (int e = threadIdx.x; e < P * k; e += kExpandThreads) zs[e] = z[(static_cast<size_t>(e / k) * units + unit) * k + e % k];
-  __syncthreads();
-  if (b >= v) return;
+  constexpr int kBatch = 8;                                     // positions whose base logits are in flight
+  float next[kBatch];
+  const float* brow = base + static_cast<size_t>(i) * v + min(b, v - 1);
+  auto fetch = [&](int p0) {
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) next[q] = p0 + q < P ? brow[static_cast<size_t>(p0 + q) * n * v] : 0.f;
+  };
+  fetch(0);
   float a[kLrMaxRank];
-  const uint4* arow = reinterpret_cast<const uint4*>(A + (static_cast<size_t>(unit) * v + b) * k);   // k bf16 = k / 8 pieces
+  const uint4* arow = reinterpret_cast<const uint4*>(A + (static_cast<size_t>(unit) * v + min(b, v - 1)) * k);   // k bf16 = k / 8 pieces
 #pragma unroll
   for (int q = 0; q < kLrMaxRank / 8; ++q) {
     if (q * 8 < k) {
@@ -653,13 +659,28 @@ __global__ void __launch_bounds__(kExpandThreads) lowrank_expand_kernel(const fl
       for (int t = 0; t < 8; ++t) a[q * 8 + t] = 0.f;
     }
   }
-  for (int pos = 0; pos < P; ++pos) {
-    float acc = base[(static_cast<size_t>(pos) * n + i) * v + b];
-    const float* zp = zs + pos * k;
+  __syncthreads();
+  if (b >= v) return;
+  for (int p0 = 0; p0 < P; p0 += kBatch) {
+    float acc[kBatch];
 #pragma unroll
-    for (int q = 0; q < kLrMaxRank; ++q)
-      if (q < k) acc = fmaf(a[q], zp[q], acc);
-    logits[(static_cast<size_t>(pos) * units + unit) * v + b] = acc;
+    for (int q = 0; q < kBatch; ++q) acc[q] = next[q];
+    if (p0 + kBatch < P) fetch(p0 + kBatch);
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      if (p0 + u >= P) break;
+      const float4* zp = reinterpret_cast<const float4*>(zs + (p0 + u) * k);
+#pragma unroll
+      for (int q = 0; q < kLrMaxRank / 4; ++q)
+        if (4 * q < k) {
+          const float4 zq = zp[q];
+          acc[u] = fmaf(a[4 * q], zq.x, acc[u]);
+          acc[u] = fmaf(a[4 * q + 1], zq.y, acc[u]);
+          acc[u] = fmaf(a[4 * q + 2], zq.z, acc[u]);
+          acc[u] = fmaf(a[4 * q + 3], zq.w, acc[u]);
+        }
+      logits[(static_cast<size_t>(p0 + u) * units + unit) * v + b] = acc[u];
+    }
   }
 }
 

@@ -698,6 +698,13 @@ int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_
   if (p.pass_tiles > kDecodeMaxTiles) p.pass_tiles = kDecodeMaxTiles;
   const int tiles = p.emit_tiles + p.emit2_tiles + p.sum_tiles;
   const int per_cta = (tiles + h->num_sms - 1) / h->num_sms;         // no wider stages than a CTA has tiles
+  // A long run of tiles and few positions: passes of two tiles and a ring 28 KB short of the limit. Three tiles a step spread the same bytes
+  // in flight over half as many rows again, 128 bytes from each. 16 x 32 x 320 (9 tiles a CTA), d = 4096, draft alone, as elsewhere / so:
+  // 1 position 225.2 / 213.2 us, 8 229.1 / 217.9, 32 237.5 / 231.2, but 64 253.2 / 251.4 and 128 283.9 / 305.7 (the hidden states, once per
+  // pass, are then a third of what it fetches); 16 x 32 x 256, d = 1024, 8 positions (6 or 7 tiles) 64.5 / 64.0; with 5 tiles a CTA
+  // (16 x 16 x 320) 109.4 / 110.9, with 3 61.6 / 68.8.
+  const bool narrow = per_cta >= 7 && p.Ppad <= 32;
+  if (narrow && p.pass_tiles > 2) p.pass_tiles = 2;
   const int passes = (per_cta + p.pass_tiles - 1) / p.pass_tiles;
   p.pass_tiles = (per_cta + passes - 1) / passes;                     // passes of one length keep as many bytes in flight throughout
   p.ksplit = h->decode_ksplit;
@@ -708,7 +715,7 @@ int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_
   if (stage < reach) stage = reach;
   p.stage_bytes = (stage + 1023) / 1024 * 1024;
   const int ctl = 1024 + static_cast<int>(sizeof(GemmControl)) + static_cast<int>(decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad));
-  p.stages = (kSmemLimit - ctl) / p.stage_bytes;
+  p.stages = (kSmemLimit - ctl - (narrow ? 28000 : 0)) / p.stage_bytes;
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   p.logw = at<float>(h, L.off_logw);
   p.sum_bias = sum_bias(h);

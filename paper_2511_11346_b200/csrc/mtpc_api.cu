@@ -1949,7 +1949,7 @@ int mtpc_window_loss(mtpc_head* head, const void* hidden, const int32_t* targets
   int rc = window_logprob_impl(head, hidden, targets, T, nullptr, prefix, st);   // phases 0 and 1
   if (rc != MTPC_OK) return rc;
   launch_kernel(loss_partial_kernel, num_sequences, kLossThreads, 0, st, overlapped(head), prefix, targets, partial,
-                sequence_length, head->cfg.n);
+                sequence_length, head->cfg.n, 0);
   launch_kernel(loss_final_kernel, 1, kLossThreads, 0, st, overlapped(head), partial, out_slot_loss, out_loss, num_sequences,
                 head->cfg.n, gamma);
   head->launches += 2;
@@ -2155,15 +2155,17 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   a.dsum_pitch = static_cast<int>(factored ? R.pitch : B.Kd);
   a.W = T;
   if ((rc = launch_circuit_backward(head, a, dT_static, st)) != MTPC_OK) return rc;
+  pt.end();
+  rc = factored ? lowrank_backward_tail(head, R, bw, hb, targets, T, d_hidden, dW_base, dA, dB, dW_sum, pt, st)
+                : backward_tail(head, B, bw, hb, targets, T, d_hidden, dW_emit, dW_sum, pt, st);
+  if (rc != MTPC_OK) return rc;
+  // 5. the loss, from the prefixes: beside the last GEMM
   launch_kernel(loss_partial_kernel, num_sequences, kLossThreads, 0, st, overlapped(head), prefix, targets, partial,
-                sequence_length, c.n);
+                sequence_length, c.n, overlapped(head) ? 1 : 0);
   launch_kernel(loss_final_kernel, 1, kLossThreads, 0, st, overlapped(head), partial, out_slot_loss, out_loss, num_sequences,
                 c.n, gamma);
   head->launches += 2;
-  pt.end();
-  if ((rc = check_launch()) != MTPC_OK) return rc;
-  if (factored) return lowrank_backward_tail(head, R, bw, hb, targets, T, d_hidden, dW_base, dA, dB, dW_sum, pt, st);
-  return backward_tail(head, B, bw, hb, targets, T, d_hidden, dW_emit, dW_sum, pt, st);
+  return check_launch();
 }
 
 extern "C" {

@@ -829,12 +829,14 @@ __device__ __forceinline__ void loss_add_rows(T* x, int step, int n) {
   __syncthreads();
 }
 
+// `beside`: the prefixes are older than the kernel ahead of this one, which it then runs beside; it ends behind that kernel all the same,
+// so that what follows finds both complete. (In a training call the loss is formed beside the last GEMM, not between circuit and gradients.)
 // grid = N. partial[i, j] = (1/V_ij) sum_{t valid} (prefix[t, j] - prefix[t, j-1]), 0 if V_ij = 0.
 __global__ void __launch_bounds__(kLossThreads) loss_partial_kernel(const float* __restrict__ prefix,
                                                                     const int* __restrict__ targets,
-                                                                    float* __restrict__ partial, int L, int n) {
+                                                                    float* __restrict__ partial, int L, int n, int beside) {
   grid_launch_dependents();
-  grid_dependency_wait();
+  if (!beside) grid_dependency_wait();
   __shared__ float ssum[kLossThreads];
   __shared__ int scnt[kLossThreads];
   const int i = blockIdx.x, step = loss_rows_per_step(n), j = threadIdx.x % n;
@@ -857,6 +859,7 @@ __global__ void __launch_bounds__(kLossThreads) loss_partial_kernel(const float*
     const int c = scnt[threadIdx.x];
     partial[static_cast<size_t>(i) * n + threadIdx.x] = c > 0 ? ssum[threadIdx.x] / static_cast<float>(c) : 0.f;
   }
+  if (beside) grid_dependency_wait();
 }
 
 // One CTA; warp q reduces the slots q, q + warps, ...: slot_loss[j] = -(1/N) sum_i partial[i, j]; then
@@ -885,11 +888,12 @@ __global__ void __launch_bounds__(kLossThreads) loss_final_kernel(const float* _
 // Coefficients of the prefix log-marginals in Eq. (6). With c[t, j] = -gamma^j / (N V_ij) for a valid target (i the
 // sequence of position t) and 0 otherwise, L = sum_t sum_j c[t, j] (P[t, j] - P[t, j-1]) = sum_t sum_j coeff[t, j] P[t, j]
 // with coeff[t, j] = c[t, j] - c[t, j+1] (c[t, n] = 0): the weights of the n backward passes. grid = N, n <= 64.
+// It needs nothing of the projection it is launched behind and runs beside it, but ends after it: what follows waits for both. (That
+// projection lets it in only after its own wait: whoever read the coefficients of the call before is done.)
 __global__ void __launch_bounds__(kLossThreads) loss_coeff_kernel(const int* __restrict__ targets,
                                                                   float* __restrict__ coeff, int L, int n, int N,
                                                                   float gamma) {
   grid_launch_dependents();
-  grid_dependency_wait();
   __shared__ int scnt[kLossThreads];
   __shared__ float cj[65];
   const int i = blockIdx.x, step = loss_rows_per_step(n), j = threadIdx.x % n;
@@ -906,13 +910,13 @@ __global__ void __launch_bounds__(kLossThreads) loss_coeff_kernel(const int* __r
   }
   if (threadIdx.x == 0) cj[n] = 0.f;
   __syncthreads();
-  if (threadIdx.x >= step * n) return;
-  for (int t = threadIdx.x / n; t < L; t += step) {
+  for (int t = threadIdx.x / n; t < L && threadIdx.x < step * n; t += step) {
     const size_t row = (static_cast<size_t>(i) * L + t) * n;
     const float here = targets[row + j] >= 0 ? cj[j] : 0.f;
     const float next = (j + 1 < n && targets[row + j + 1] >= 0) ? cj[j + 1] : 0.f;
     coeff[row + j] = here - next;
   }
+  grid_dependency_wait();
 }
 
 // ---------------------------------------------------------------- preparation

@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(32 * kHmmStaticWarps, 2) circuit_hmm_static_lo
         float m = warp_max_nan(al);
         if (m == -CUDART_INF_F) m = 0.f;
         const float u = __expf(al - m);
-        const float c = l.active ? xs[i * r + k] : 1.f;
+        const float c = mine ? xs[i * r + k] : 1.f;                      // (one lane of a state reads its sum and puts x in its place)
         if (mine) {
           post[static_cast<size_t>(i) * r + k] = tg[i] >= 0 ? abar : 0.f;
           xs[i * r + k] = c == 0.f ? 0.f : __fdividef(abar, c);

@@ -468,14 +468,31 @@ __global__ void circuit_hmm_loss_backward_kernel(const CircuitBackwardArgs a_, c
 // A batch is one window per warp: each warp runs its window forward and back (32 multiply-adds a lane and step either way) and leaves
 // u, x and prop in shared memory; then the steps are dealt to the warps, which add the batch's u x^T - prop into the CTA's running
 // sums, eight columns in registers at a time (acc [n-1][b][a]: lane = a, conflict-free). The factor A and the addition into dT come
-// once per CTA. A step whose sum is below 2^-100 for a state that matters (the evidence outweighs the other states' by 70 nats)
-// is redone with logarithms, straight into dT. Forward step and prefixes are those of circuit_hmm_kernel, bit for bit.
+// once per CTA. A column b that sum_lost finds takes its part of prop and dT with logarithms: an exponential and at most an atomic per lane,
+// and no atomic for what is below the normal numbers, which is all that a state hardly ever entered has to give. (Whole steps redone so, by
+// a test that any state with a posterior met: a head with one state entered with e^-75 took 2048 us instead of 58.) Forward step and prefixes
+// are those of circuit_hmm_kernel, bit for bit.
 // 8192 windows of n = 8, r = 32: 202 us by the streaming kernel (five exponentials an entry, 32 shared atomics a lane and step), 52 by this
 // one, bound by its instructions and the reads of the tables from shared memory.
 // Shared memory: 2 (n-1) r^2 floats, and per warp hmm_static_loss_warp_floats.
 constexpr int kHmmStaticWarps = 16;
 __host__ __device__ inline size_t hmm_static_loss_warp_floats(int n, int r) {
   return (static_cast<size_t>(n) * r + 3) / 4 * 4 + 64 + (static_cast<size_t>(n) * (2 * r + 1) + 3) / 4 * 4;
+}
+// What the columns b in `lost` give to the gradient of the lane's alpha (al) and, if it is `mine` to write, to its row of dT. back: per
+// state b (in lane b) its evidence less alpha_i[b]; row: the lane's row of the log table. (Inlined it costs its callers' registers: 0.4 %.)
+__device__ __noinline__ float hmm_lost_columns(unsigned lost, float al, float back, float abar, const float* __restrict__ row,
+                                               float* dT_row, bool mine) {
+  float sum = 0.f;
+  do {
+    const int b = __ffs(lost) - 1;
+    lost &= lost - 1;
+    const float back_b = __shfl_sync(kFull, back, b), abar_b = __shfl_sync(kFull, abar, b);
+    const float e = __expf(al + row[b] + back_b) * abar_b;
+    sum += e;
+    if (mine && !(fabsf(e) < 0x1p-126f)) atomicAdd(dT_row + b, e);
+  } while (lost != 0);
+  return sum;
 }
 __global__ void __launch_bounds__(32 * kHmmStaticWarps, 2) circuit_hmm_static_loss_backward_kernel(
     const CircuitBackwardArgs a_, const float* __restrict__ prob, const float* __restrict__ logA, float* __restrict__ dT) {
@@ -548,59 +565,44 @@ __global__ void __launch_bounds__(32 * kHmmStaticWarps, 2) circuit_hmm_static_lo
         if (m == -CUDART_INF_F) m = 0.f;
         const float u = __expf(al - m);
         const float c = mine ? xs[i * r + k] : 1.f;                      // (one lane of a state reads its sum and puts x in its place)
+        const bool tiny = sum_lost(c, abar);
         if (mine) {
           post[static_cast<size_t>(i) * r + k] = tg[i] >= 0 ? abar : 0.f;
-          xs[i * r + k] = c == 0.f ? 0.f : __fdividef(abar, c);
+          xs[i * r + k] = tiny ? 0.f : __fdividef(abar, c);
         }
-        const bool redo = __any_sync(kFull, c > 0.f && c < 0x1p-100f && abar != 0.f);
+        unsigned lost = __ballot_sync(kFull, tiny && abar != 0.f);
         __syncwarp();
         float prop = 0.f;
-        if (!redo) {
-          const float* row = E + (i - 1) * rr + k * r;
-          const float* x = xs + i * r;
-          if (l.rows == 32) {                                            // float4 reads rotated by the lane: conflict-free
-            const float4 *row4 = reinterpret_cast<const float4*>(row), *x4 = reinterpret_cast<const float4*>(x);
-            float p1 = 0.f, p2 = 0.f, p3 = 0.f;
+        const float* row = E + (i - 1) * rr + k * r;
+        const float* x = xs + i * r;
+        if (l.rows == 32) {                                              // float4 reads rotated by the lane: conflict-free
+          const float4 *row4 = reinterpret_cast<const float4*>(row), *x4 = reinterpret_cast<const float4*>(x);
+          float p1 = 0.f, p2 = 0.f, p3 = 0.f;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const int j = (q + lane) & 7;
-              const float4 a = row4[j], y = x4[j];
-              prop = fmaf(a.x, y.x, prop);
-              p1 = fmaf(a.y, y.y, p1);
-              p2 = fmaf(a.z, y.z, p2);
-              p3 = fmaf(a.w, y.w, p3);
-            }
-            prop = (prop + p1) + (p2 + p3);
-          } else if (l.active) {
-            for (int q = 0; q < l.rows; ++q) {
-              const int b = l.part * l.rows + ((q + k) & (l.rows - 1));
-              prop = fmaf(row[b], x[b], prop);
-            }
+          for (int q = 0; q < 8; ++q) {
+            const int j = (q + lane) & 7;
+            const float4 a = row4[j], y = x4[j];
+            prop = fmaf(a.x, y.x, prop);
+            p1 = fmaf(a.y, y.y, p1);
+            p2 = fmaf(a.z, y.z, p2);
+            p3 = fmaf(a.w, y.w, p3);
           }
-          for (int off = r; off < r * l.parts; off <<= 1) prop += __shfl_xor_sync(kFull, prop, off);
-          prop *= u;
-          if (mine) {
-            us[(i - 1) * (r + 1) + k] = u;
-            props[i * r + k] = prop;
+          prop = (prop + p1) + (p2 + p3);
+        } else if (l.active) {
+          for (int q = 0; q < l.rows; ++q) {
+            const int b = l.part * l.rows + ((q + k) & (l.rows - 1));
+            prop = fmaf(row[b], x[b], prop);
           }
-        } else {
-          if (mine) {
-            ev[k] = al_i == -CUDART_INF_F ? -CUDART_INF_F : g[i * r + k] - al_i;
-            ev[32 + k] = abar;
-          }
-          __syncwarp();
-          if (l.active) {
-            const float* row = logA + static_cast<size_t>(i - 1) * rr + k * r;
-            for (int b = 0; b < r; ++b) prop += __expf(al + row[b] + ev[b]) * ev[32 + b];
-            if (mine) {
-              for (int b = 0; b < r; ++b)
-                atomicAdd(dT + static_cast<size_t>(i - 1) * rr + k * r + b, __expf(al + row[b] + ev[b]) * ev[32 + b] - __expf(row[b]) * prop);
-              us[(i - 1) * (r + 1) + k] = 0.f;                           // nothing for the running sums
-              xs[i * r + k] = 0.f;
-              props[i * r + k] = 0.f;
-            }
-          }
-          __syncwarp();
+        }
+        for (int off = r; off < r * l.parts; off <<= 1) prop += __shfl_xor_sync(kFull, prop, off);
+        prop *= u;
+        if (lost != 0) {                                                 // columns left out above
+          const float back = l.active && al_i != -CUDART_INF_F ? g[i * r + k] - al_i : -CUDART_INF_F;
+          prop += hmm_lost_columns(lost, al, back, abar, logA + (i - 1) * rr + k * r, dT + (i - 1) * rr + k * r, mine);
+        }
+        if (mine) {
+          us[(i - 1) * (r + 1) + k] = u;
+          props[i * r + k] = prop;
         }
         abar = l.active ? cw[i - 1] * __expf(al - lp) + prop : 0.f;
         al_i = al;

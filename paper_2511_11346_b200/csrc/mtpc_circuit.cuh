@@ -565,6 +565,13 @@ __device__ __forceinline__ HmmLanes hmm_lanes(int r, int lane) {
   l.active = lane < r * l.parts;
   return l;
 }
+// Whether a sum of products of probabilities, each scaled by its maximum, is no divisor for the gradient that came to it. The build keeps
+// subnormal numbers, so 32 products of factors rounded at 2^-149 are off by 2^-144 at most: from 2^-118 on nothing of a sum is lost.
+// And a quotient above 2^112 (a state that its evidence alone makes likely) could overflow where quotients are added over many windows.
+constexpr float kSumFloor = 0x1p-118f;
+__device__ __forceinline__ bool sum_lost(float sum, float gradient) {
+  return sum < fmaxf(kSumFloor, fabsf(gradient) * 0x1p-112f);           // (NaN is not lost: it goes on through the quotient)
+}
 // One step of the forward recursion: LSE_a(alpha[a] + logA[a][k]) = m + log sum_a exp(alpha[a] - m) A[a][k] for lane's state k
 // (every part returns it). alpha: per active lane, -inf elsewhere; NaN in any of them reaches every state. A [r, r] in shared
 // memory holds probabilities (LOG_TABLE: their logarithms); ev: 32 floats of the warp's shared memory, not reused before the

@@ -51,3 +51,38 @@ def test_states_that_only_their_evidence_makes_likely():
     t = wl.targets.copy()
     t[::2, 2] = 5
     compare(wl, t, 1)
+
+
+@pytest.mark.parametrize("r,logp,N", [(32, -83.0, 1), (8, -83.0, 2), (32, -76.0, 2)])
+def test_columns_taken_with_logarithms(r, logp, N):
+    """As above, with sums below the floor of the products (e^-83 = 2^-119.7, itself good to 2^-30) or quotients above their limit, in windows
+    of both kinds, and tails in which the same state has no gradient."""
+    n, L = 6, 30
+    wl = I.make_workload("static_lost", I.HeadShape(I.HMM, n, r, 16, 64), N * L, seed=9230 + r, weight_std=0.05)
+    wl.hidden_q[:, :32] = 1.0
+    wl.W_emit_q[:, :, 5, :32] = -4.0
+    wl.W_emit_q[:, 0, 5, :32] = 0.0
+    wl.T_static[:, :, 0] = logp
+    t = wl.targets.copy().reshape(N, L, n)
+    t[:, ::2, 2] = 5
+    t[:, 1::4, 3] = 5
+    for j in range(1, n):
+        t[:, max(L - j, 0):, j] = -1
+    compare(wl, t.reshape(N * L, n), N)
+
+
+@pytest.mark.parametrize("r", [32, 8])
+def test_sums_below_the_normal_numbers_in_marginalised_tails(r):
+    """State 0 is reached (e^-50) from state 1 alone, which the last byte before the tail makes unlikely (e^-50): the step's sum for state 0
+    is subnormal, and its gradient, exactly 0 there, is not to be divided by it."""
+    n, N, L = 6, 2, 30
+    wl = I.make_workload("static_tail", I.HeadShape(I.HMM, n, r, 16, 64), N * L, seed=9210 + r, weight_std=0.05)
+    wl.hidden_q[:, :32] = 1.0
+    wl.W_emit_q[:, 1, 5, :32] = -1.5625
+    wl.T_static[:, :, 0] = -200.0
+    wl.T_static[:, 1, 0] = -50.0
+    t = wl.targets.copy().reshape(N, L, n)
+    for j in range(1, n):
+        t[:, max(L - j, 0):, j] = -1
+        t[:, L - j, j - 1] = 5
+    compare(wl, t.reshape(N * L, n), N)

@@ -859,19 +859,16 @@ __global__ void __launch_bounds__(256, 3) circuit_btree_loss_backward_kernel(con
         float m;
         const float u = t.scaled(in_z, m);
         const float sum = has ? __expf(Dc - m) : 1.f;                    // sum_z u[z] T_c[z][lane]
+        const bool tiny = has && sum_lost(sum, dd);
         float* x = vec;                            // dD_c over that sum
-        if (has) x[lane] = sum == 0.f ? 0.f : __fdividef(dd, sum);
-        const bool redo = __any_sync(kFull, sum < kTreeFloor && dd != 0.f);
+        if (has) x[lane] = tiny ? 0.f : __fdividef(dd, sum);
+        unsigned lost = __ballot_sync(kFull, tiny && dd != 0.f);
         __syncwarp();
-        float acc;
-        if (!redo) {
-          acc = u * row_dot(t.table_of(c), x, lane, r);
-        } else {                                   // terms may have been lost: with logarithms
-          acc = 0.f;
-          if (has) {
-            const float* row = t.log_table(c) + lane * r;
-            for (int b = 0; b < r; ++b) acc = fmaf(dD[c * vr + b], __expf(in_z + row[b] - t.D[c * vr + b]), acc);
-          }
+        float acc = u * row_dot(t.table_of(c), x, lane, r);
+        for (; lost != 0; lost &= lost - 1) {      // with logarithms
+          const int b = __ffs(lost) - 1;
+          const float dd_b = __shfl_sync(kFull, dd, b), D_b = __shfl_sync(kFull, Dc, b);
+          if (has) acc = fmaf(dd_b, __expf(in_z + t.log_table(c)[lane * r + b] - D_b), acc);
         }
         if (has) pd[c * vr + lane] = acc;
         __syncwarp();
@@ -908,67 +905,66 @@ __global__ void __launch_bounds__(256, 3) circuit_btree_loss_backward_kernel(con
         const float e = edge ? 0.f : t.scaled(prod, mp);
         const float below = has ? __expf(Dc - mi) : 1.f;                 // sum_z u[z] T_c[z][lane]
         const float across = has && !edge ? __expf(Sz - mp) : 1.f;       // sum_b T_c[lane][b] e[b]
-        const bool redo = __any_sync(kFull, (below < kTreeFloor && dDc != 0.f) || (across < kTreeFloor && ds != 0.f));
+        const bool tiny_b = has && sum_lost(below, dDc), tiny_z = has && !edge && sum_lost(across, ds);
+        unsigned lost_b = __ballot_sync(kFull, tiny_b && dDc != 0.f), lost_z = __ballot_sync(kFull, tiny_z && ds != 0.f);
         __nv_bfloat16* dst = drow + r + static_cast<size_t>(c - 1) * r * r;
-        if (!redo) {
-          // dL/dT_c[z][b] = T_c[z][b] (u[z] x[b] + y[z] e[b] - (pd + dS)[z]), x = dD / below, y = dS / across; dprod[b] = e[b] sum_z T y
-          const float x = below == 0.f ? 0.f : __fdividef(dDc, below);
-          float4* zv = reinterpret_cast<float4*>(vec);
-          if (has) zv[lane] = make_float4(u, across == 0.f ? 0.f : __fdividef(ds, across), sumz, 0.f);
-          __syncwarp();
-          const float* tab = t.table_of(c);
-          if (r == 32) {                           // a lane takes two columns of every other row: 4-byte stores
-            const int half = lane >> 4, b = 2 * (lane & 15);
-            const float x0 = __shfl_sync(kFull, x, b), x1 = __shfl_sync(kFull, x, b + 1);
-            const float e0 = __shfl_sync(kFull, e, b), e1 = __shfl_sync(kFull, e, b + 1);
-            float a0 = 0.f, a1 = 0.f;
+        // dL/dT_c[z][b] = T_c[z][b] (u[z] x[b] + y[z] e[b] - (pd + dS)[z]), x = dD / below, y = dS / across; dprod[b] = e[b] sum_z T y
+        const float x = tiny_b ? 0.f : __fdividef(dDc, below), y = tiny_z ? 0.f : __fdividef(ds, across);
+        float4* zv = reinterpret_cast<float4*>(vec);
+        if (has) zv[lane] = make_float4(u, y, sumz, 0.f);
+        __syncwarp();
+        const float* tab = t.table_of(c);
+        if (r == 32) {                           // a lane takes two columns of every other row: 4-byte stores
+          const int half = lane >> 4, b = 2 * (lane & 15);
+          const float x0 = __shfl_sync(kFull, x, b), x1 = __shfl_sync(kFull, x, b + 1);
+          const float e0 = __shfl_sync(kFull, e, b), e1 = __shfl_sync(kFull, e, b + 1);
+          float a0 = 0.f, a1 = 0.f;
 #pragma unroll 8
-            for (int q = 0; q < 16; ++q) {
-              const int z = 2 * q + half;
-              const float2 p = *reinterpret_cast<const float2*>(tab + z * 32 + b);
-              const float4 f = zv[z];
-              a0 = fmaf(p.x, f.y, a0);
-              a1 = fmaf(p.y, f.y, a1);
-              const float g0 = p.x * fmaf(f.y, e0, fmaf(f.x, x0, -f.z)), g1 = p.y * fmaf(f.y, e1, fmaf(f.x, x1, -f.z));
-              *reinterpret_cast<__nv_bfloat162*>(dst + z * 32 + b) = __floats2bfloat162_rn(g0, g1);
-            }
-            a0 += __shfl_xor_sync(kFull, a0, 16);
-            a1 += __shfl_xor_sync(kFull, a1, 16);
-            if (half == 0) *reinterpret_cast<float2*>(dP + c * vr + b) = make_float2(a0 * e0, a1 * e1);
-          } else if (has) {
-            float a0 = 0.f;
-            for (int z = 0; z < r; ++z) {
-              const float p = tab[z * r + lane];
-              const float4 f = zv[z];
-              a0 = fmaf(p, f.y, a0);
-              dst[z * r + lane] = __float2bfloat16_rn(p * fmaf(f.y, e, fmaf(f.x, x, -f.z)));
-            }
-            dP[c * vr + lane] = a0 * e;
+          for (int q = 0; q < 16; ++q) {
+            const int z = 2 * q + half;
+            const float2 p = *reinterpret_cast<const float2*>(tab + z * 32 + b);
+            const float4 f = zv[z];
+            a0 = fmaf(p.x, f.y, a0);
+            a1 = fmaf(p.y, f.y, a1);
+            const float g0 = p.x * fmaf(f.y, e0, fmaf(f.x, x0, -f.z)), g1 = p.y * fmaf(f.y, e1, fmaf(f.x, x1, -f.z));
+            *reinterpret_cast<__nv_bfloat162*>(dst + z * 32 + b) = __floats2bfloat162_rn(g0, g1);
           }
-        } else {                                   // terms may have been lost: with logarithms
-          float *inv = vec, *sv = vec + vr, *dsv = vec + 2 * vr, *sumv = vec + 3 * vr;
-          if (has) {
-            inv[lane] = in_z;
-            sv[lane] = Sz;
-            dsv[lane] = ds;
-            sumv[lane] = sumz;
+          a0 += __shfl_xor_sync(kFull, a0, 16);
+          a1 += __shfl_xor_sync(kFull, a1, 16);
+          if (half == 0) *reinterpret_cast<float2*>(dP + c * vr + b) = make_float2(a0 * e0, a1 * e1);
+        } else if (has) {
+          float a0 = 0.f;
+          for (int z = 0; z < r; ++z) {
+            const float p = tab[z * r + lane];
+            const float4 f = zv[z];
+            a0 = fmaf(p, f.y, a0);
+            dst[z * r + lane] = __float2bfloat16_rn(p * fmaf(f.y, e, fmaf(f.x, x, -f.z)));
+          }
+          dP[c * vr + lane] = a0 * e;
+        }
+        if ((lost_b | lost_z) != 0) {              // columns and rows left out above: with logarithms, over what was stored
+          const float* logt = t.log_table(c);
+          __syncwarp();
+          for (; lost_b != 0; lost_b &= lost_b - 1) {                    // lane = z
+            const int b = __ffs(lost_b) - 1;
+            const float D_b = __shfl_sync(kFull, Dc, b), dD_b = __shfl_sync(kFull, dDc, b), e_b = __shfl_sync(kFull, e, b);
+            if (has)
+              dst[lane * r + b] = __float2bfloat16_rn(fmaf(dD_b, __expf(in_z + logt[lane * r + b] - D_b), tab[lane * r + b] * fmaf(y, e_b, -sumz)));
           }
           __syncwarp();
-          if (has) {
-            const float* col = t.log_table(c) + lane;
-            float acc = 0.f;
-            for (int z = 0; z < r; ++z) {
-              const float l = col[z * r];
-              float xi = dDc * __expf(inv[z] + l - Dc);
-              if (!edge) {
-                const float e2 = dsv[z] * __expf(l + prod - sv[z]);
-                acc += e2;
-                xi += e2;
-              }
-              dst[z * r + lane] = __float2bfloat16_rn(fmaf(-__expf(l), sumv[z], xi));
+          float more = 0.f;
+          for (; lost_z != 0; lost_z &= lost_z - 1) {                    // lane = b
+            const int z = __ffs(lost_z) - 1;
+            const float S_z = __shfl_sync(kFull, Sz, z), ds_z = __shfl_sync(kFull, ds, z), in = __shfl_sync(kFull, in_z, z);
+            if (has) {
+              const float l = logt[z * r + lane], own = ds_z * __expf(l + prod - S_z);
+              const float4 f = zv[z];
+              const float up = tiny_b && dDc != 0.f ? dDc * __expf(in + l - Dc) : 0.f;
+              dst[z * r + lane] = __float2bfloat16_rn(fmaf(tab[z * r + lane], fmaf(f.x, x, -f.z), own + up));
+              more += own;
             }
-            dP[c * vr + lane] = acc;
           }
+          if (has) dP[c * vr + lane] += more;
         }
         __syncwarp();
       }

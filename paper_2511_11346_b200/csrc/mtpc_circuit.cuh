@@ -293,14 +293,12 @@ __global__ void circuit_btree_kernel(const float* __restrict__ G, const float* _
   }
 }
 
-// LSE_q(vec[q] + tab[q * step]) by one lane, for steps that are rarely taken: a row of a log table (step 1) or a column (step r).
-__device__ __noinline__ float layer_lse(const float* tab, int step, const float* vec, int r) {
-  float m = -CUDART_INF_F;
-  for (int q = 0; q < r; ++q) m = fmaxf(m, vec[q] + tab[q * step]);
-  if (m == -CUDART_INF_F) m = 0.f;
-  float s = 0.f;
-  for (int q = 0; q < r; ++q) s += __expf(vec[q] + tab[q * step] - m);
-  return m + __logf(s);                            // NaN evidence survives through the sum
+// Whether a sum of products of probabilities, each scaled by its maximum, is no divisor for the gradient that came to it. The build keeps
+// subnormal numbers, so 32 products of factors rounded at 2^-149 are off by 2^-144 at most: from 2^-118 on nothing of a sum is lost.
+// And a quotient above 2^112 (a state that its evidence alone makes likely) could overflow where quotients are added over many windows.
+constexpr float kSumFloor = 0x1p-118f;
+__device__ __forceinline__ bool sum_lost(float sum, float gradient) {
+  return sum < fmaxf(kSumFloor, fabsf(gradient) * 0x1p-112f);           // (NaN is not lost: it goes on through the quotient)
 }
 // sum_b tab[lane][b] vec[b] and sum_z vec[z] tab[z][lane] over a table [r, r] and a vector [r] in shared memory (16-byte aligned for r >= 4);
 // lanes past r return 0. Rows are read as float4 rotated by the lane (see sum_layer_staged_vec).
@@ -361,6 +359,20 @@ __device__ __forceinline__ float warp_lse_nan(float x) {
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
   return m + __logf(s);
 }
+// For every lane in `lost` LSE_q(vec_q + tab[lane * own + q * step]), vec_q in lane q < r and tab in global memory; the others keep `x`.
+__device__ __noinline__ float warp_relog(unsigned lost, float x, float vec, const float* __restrict__ tab, int own, int step, int lane, int r) {
+  auto entry = [&](unsigned left) { return lane < r && left != 0 ? tab[(__ffs(left) - 1) * own + lane * step] : -CUDART_INF_F; };
+  float next = entry(lost);
+  do {
+    const int z = __ffs(lost) - 1;
+    lost &= lost - 1;
+    const float y = lane < r ? vec + next : -CUDART_INF_F;
+    next = entry(lost);
+    const float l = warp_lse_nan(y);
+    if (lane == z) x = l;
+  } while (lost != 0);
+  return x;
+}
 
 // Binary tree: every prefix marginal and slot message from one upward and one downward sweep. With
 //   S[c][z] = LSE_b(logOmega_c[z][b] + prod[c][b])  the subtree of node c under its parent's value z (all its tokens seen), and
@@ -376,11 +388,10 @@ __device__ __forceinline__ float warp_lse_nan(float x) {
 // position stays the same. Measured against one warp per window and a path per prefix: 4096 windows at n = 16, r = 32:
 // 256 -> 148 us; 108 windows at n = 8: 36 -> 6 us.
 // In shared memory the tables are probabilities, exponentiated once on their way there, so that a step of either sweep is one warp
-// maximum, r multiply-adds per lane and one logarithm (r exponentials of sums, a maximum over them and their sum before). Where a
-// step's sum falls below kTreeFloor against its maximum, so that terms may have been lost, the warp takes the step once more with
-// logarithms from the log tables in global memory. (4096 windows at n = 16, r = 32, inside a draft: 102 -> 96 us, latency of a window's
-// levels; 27 positions of 4 windows at n = 8: 8.7 -> 5.8.) Shared memory: btree_prefix_smem_floats.
-constexpr float kTreeFloor = 0x1p-100f;
+// maximum, r multiply-adds per lane and one logarithm (r exponentials of sums, a maximum over them and their sum before). A value whose
+// sum falls below kSumFloor takes the step once more with logarithms, the warp working on its row or column of the log tables in global
+// memory. (4096 windows at n = 16, r = 32, inside a draft: 102 -> 96 us, latency of a window's levels; 27 positions of 4 windows at n = 8:
+// 8.7 -> 5.8.) Shared memory: btree_prefix_smem_floats.
 // One window of a tree sweep, shared by a CTA. vr: pitch of the [r] vectors (r rounded up to 4 floats).
 template <int R>                                   // r, where the kernel is built for it (0: any)
 struct TreeSweep {
@@ -468,12 +479,8 @@ struct TreeSweep {
         __syncwarp();
         const float q = row_dot(table_of(c), vec, lane, r);
         float sc = m + __logf(q);
-        if (__any_sync(kFull, lane < r && q < kTreeFloor)) {
-          __syncwarp();
-          if (lane < r) vec[lane] = prod;
-          __syncwarp();
-          if (lane < r) sc = layer_lse(log_table(c) + lane * r, 1, vec, r);
-        }
+        const unsigned lost = __ballot_sync(kFull, lane < r && q < kSumFloor);
+        if (lost != 0) sc = warp_relog(lost, sc, prod, log_table(c), r, 1, lane, r);
         if (lane < r) S[c * vr + lane] = sc;
         __syncwarp();
       }
@@ -490,12 +497,8 @@ struct TreeSweep {
         __syncwarp();
         const float q = col_dot(table_of(c), vec, lane, r);
         float dc = m + __logf(q);
-        if (__any_sync(kFull, lane < r && q < kTreeFloor)) {
-          __syncwarp();
-          if (lane < r) vec[lane] = in;
-          __syncwarp();
-          if (lane < r) dc = layer_lse(log_table(c) + lane, r, vec, r);
-        }
+        const unsigned lost = __ballot_sync(kFull, lane < r && q < kSumFloor);
+        if (lost != 0) dc = warp_relog(lost, dc, in, log_table(c), 1, r, lane, r);
         if (lane < r) D[c * vr + lane] = dc;
         __syncwarp();
       }
@@ -564,13 +567,6 @@ __device__ __forceinline__ HmmLanes hmm_lanes(int r, int lane) {
   l.part = lane / r;
   l.active = lane < r * l.parts;
   return l;
-}
-// Whether a sum of products of probabilities, each scaled by its maximum, is no divisor for the gradient that came to it. The build keeps
-// subnormal numbers, so 32 products of factors rounded at 2^-149 are off by 2^-144 at most: from 2^-118 on nothing of a sum is lost.
-// And a quotient above 2^112 (a state that its evidence alone makes likely) could overflow where quotients are added over many windows.
-constexpr float kSumFloor = 0x1p-118f;
-__device__ __forceinline__ bool sum_lost(float sum, float gradient) {
-  return sum < fmaxf(kSumFloor, fabsf(gradient) * 0x1p-112f);           // (NaN is not lost: it goes on through the quotient)
 }
 // One step of the forward recursion: LSE_a(alpha[a] + logA[a][k]) = m + log sum_a exp(alpha[a] - m) A[a][k] for lane's state k
 // (every part returns it). alpha: per active lane, -inf elsewhere; NaN in any of them reaches every state. A [r, r] in shared

@@ -2141,7 +2141,7 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   head->launches++;
   pt.end();
   if ((rc = check_launch()) != MTPC_OK) return rc;
-  // 2. circuit: every prefix and the whole gradient of the loss, then the loss itself. The sum units' logit gradients (bf16)
+  // 2. circuit: every prefix and the whole gradient of the loss. The sum units' logit gradients (bf16)
   // go to the right of dlogit, or of [s | y] on a factored head.
   pt.begin();
   CircuitBackwardArgs a;
@@ -2155,16 +2155,20 @@ static int window_loss_backward_impl(mtpc_head* head, const void* hidden, const 
   a.dsum_pitch = static_cast<int>(factored ? R.pitch : B.Kd);
   a.W = T;
   if ((rc = launch_circuit_backward(head, a, dT_static, st)) != MTPC_OK) return rc;
+  const bool beside = overlapped(head);
+  auto launch_loss = [&] {
+    launch_kernel(loss_partial_kernel, num_sequences, kLossThreads, 0, st, beside, prefix, targets, partial, sequence_length, c.n,
+                  beside ? 1 : 0);
+    launch_kernel(loss_final_kernel, 1, kLossThreads, 0, st, beside, partial, out_slot_loss, out_loss, num_sequences, c.n, gamma);
+    head->launches += 2;
+  };
+  if (!beside) launch_loss();                                  // between events: in the phase of the circuit
   pt.end();
+  if ((rc = check_launch()) != MTPC_OK) return rc;
   rc = factored ? lowrank_backward_tail(head, R, bw, hb, targets, T, d_hidden, dW_base, dA, dB, dW_sum, pt, st)
                 : backward_tail(head, B, bw, hb, targets, T, d_hidden, dW_emit, dW_sum, pt, st);
   if (rc != MTPC_OK) return rc;
-  // 5. the loss, from the prefixes: beside the last GEMM
-  launch_kernel(loss_partial_kernel, num_sequences, kLossThreads, 0, st, overlapped(head), prefix, targets, partial,
-                sequence_length, c.n, overlapped(head) ? 1 : 0);
-  launch_kernel(loss_final_kernel, 1, kLossThreads, 0, st, overlapped(head), partial, out_slot_loss, out_loss, num_sequences,
-                c.n, gamma);
-  head->launches += 2;
+  if (beside) launch_loss();                                   // from the prefixes, beside the last GEMM
   return check_launch();
 }
 

@@ -384,3 +384,20 @@ def test_gradient_descent_on_the_device_gradients_lowers_the_loss(family):
     _, ref = O.composite_loss(pre, wl.targets, N, gamma)
     assert abs(losses[-1] - ref) <= 2e-3 * n, (losses[-1], ref)
     dh.close()
+
+
+def test_the_training_calls_circuit_phase_holds_the_loss():
+    """The kernel that sums a sequence's loss is one CTA per sequence: for the same windows in one long sequence instead of sixty-four it takes
+    many times as long, and the phase that holds it shows that (nothing else in it depends on the sequences)."""
+    T = 32768
+    wl = I.make_workload("phase", I.HeadShape(I.CP, 16, 1, 16, 64), T, seed=15, weight_std=0.3)
+    dh = DeviceHead(wl)
+    h, t = dh.hidden_device(), torch.from_numpy(wl.targets).cuda()
+    dh.head.mtpc_set_timing(8)
+    circuit = {}
+    for N in (64, 1):
+        for _ in range(8):
+            dh.window_loss_backward(N, T // N, 0.9, hidden=h, targets=t)
+        circuit[N] = min(dh.head.mtpc_get_timing(i)[1] for i in range(6))
+    assert circuit[1] > circuit[64] + 0.02, circuit           # ms
+    dh.close()

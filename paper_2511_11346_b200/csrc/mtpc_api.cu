@@ -340,9 +340,16 @@ int check_launch() { return cudaGetLastError() == cudaSuccess ? MTPC_OK : MTPC_E
 // Launch `kernel`, optionally allowed to start before the kernel ahead of it in the stream has finished (programmatic
 // dependent launch): such a kernel calls grid_dependency_wait() before it touches global memory, so what overlaps is its launch and
 // set-up (about 2 us a kernel). cluster > 1: in clusters of that many CTAs.
-// Three kernels copy a static head's transition tables before they wait (draft_slot_kernel, circuit_hmm_kernel and the static HMM's Eq. 6
-// kernel). The tables are written by a plain launch (bind_parameters), and the first kernel of every call that runs one of them lets its dependents in only after
-// its own wait (the fp32 conversion, the projection, the weight pass), so the tables are complete before any of them starts.
+// Five kernels do more before they wait. A kernel that lets its dependents in after its own wait (a gate) has nothing unfinished ahead of
+// it, so whatever was launched before it has ended when anything behind it starts; each of the five relies on one:
+//   draft_slot_kernel, circuit_hmm_kernel and the static HMM's Eq. 6 kernel copy the head's static tables. The tables are written by a plain
+//     launch (bind_parameters), and the first kernel of every call that runs one of the three is a gate (the fp32 conversion, the projection,
+//     the weight pass; an acceptance call, whose first kernel may be circuit_hmm_kernel, needs a draft since the last update).
+//   loss_coeff_kernel reads the targets and writes the coefficients. The projection it is launched behind is a gate (on a factored head the
+//     merge), so the caller's writes and the readers of the last call's coefficients are done.
+//   loss_partial_kernel, beside the last GEMM, reads the prefixes and writes its partial sums. The GEMMs are NOT gates, they let their
+//     dependents in before they wait. What lies between them and the circuit is: logit_gradient_kernel, by its plain launch, or on a factored
+//     head lowrank_pad_kernel. Whoever makes the one a dependent or lets the other's dependents in early breaks the loss.
 template <typename... Params, typename... Args>
 void launch_clusters(void (*kernel)(Params...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent,
                      Args&&... args) {
@@ -1357,7 +1364,7 @@ int backward_tail(mtpc_head* head, const BackwardLayout& B, uint8_t* bw, const v
     if (row_blocks > T) row_blocks = T;
     if (row_blocks > 65535) row_blocks = 65535;
     // not as a dependent: CTAs scheduled beside the circuit kernel's last ones would share a few SMs (517 us became 690 at 4096
-    // positions of a 16 x 32 x 256 head)
+    // positions of a 16 x 32 x 256 head); and loss_partial_kernel, which works before it waits, relies on it (launch_clusters)
     launch_kernel(logit_gradient_kernel, dim3(col_blocks, row_blocks), 256, 0, st, /*dependent=*/false, la);
   }
   head->launches++;

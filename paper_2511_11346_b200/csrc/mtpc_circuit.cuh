@@ -832,8 +832,9 @@ __device__ __forceinline__ void loss_add_rows(T* x, int step, int n) {
   __syncthreads();
 }
 
-// `beside`: the prefixes are older than the kernel ahead of this one, which it then runs beside; it ends behind that kernel all the same,
-// so that what follows finds both complete. (In a training call the loss is formed beside the last GEMM, not between circuit and gradients.)
+// `beside`: runs beside the kernel ahead of it, the last GEMM of a training call, and ends behind it, so that what follows finds both
+// complete. The prefixes have to be complete when this kernel starts, for which some kernel between the circuit and that GEMM lets its
+// dependents in only after its own wait or is launched plainly (the list at launch_clusters).
 // grid = N. partial[i, j] = (1/V_ij) sum_{t valid} (prefix[t, j] - prefix[t, j-1]), 0 if V_ij = 0.
 __global__ void __launch_bounds__(kLossThreads) loss_partial_kernel(const float* __restrict__ prefix,
                                                                     const int* __restrict__ targets,

@@ -700,7 +700,7 @@ __global__ void lowrank_pad_kernel(const uint4* __restrict__ A, uint4* __restric
   const int b = static_cast<int>(rest % v64);
   const size_t u = rest / v64;
   out[idx] = b < v ? A[(u * v + b) * kv + q] : make_uint4(0u, 0u, 0u, 0u);
-  grid_launch_dependents();
+  grid_launch_dependents();   // (after the wait: loss_partial_kernel, which works before it waits, relies on it)
 }
 
 // Byte draws of a long draft on a factored head (Algorithm 1, input-unit step): one warp per (window, slot) forms the v

@@ -72,7 +72,8 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
 // ---------------------------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-stream-serialization attribute may start while the kernel before it in the
 // stream is still running; it must not touch that kernel's results before grid_dependency_wait() returns (which is
-// when the earlier grid has completed and its writes are visible). Without the attribute the wait returns at once.
+// when the earlier grid has completed and its writes are visible). Without the attribute the wait returns at once. (The few kernels
+// that touch older results before it are listed at launch_clusters, with what makes each sound.)
 // grid_launch_dependents(): this CTA no longer objects to the next kernel's CTAs being scheduled. The GEMMs call it once their
 // tensor memory is allocated (a waiting CTA of the next GEMM must not take it first), short kernels at their start, kernels that
 // stream much memory at their end: a GEMM's CTAs that wait on the same SM claim its shared memory, and with it the L1 that keeps

@@ -108,3 +108,55 @@ def test_parameters_updated_between_calls(n, r, v, d, T, P, wpp, dtype):
     per = len(want) // 6
     assert not torch.equal(want[per], want[2 * per])       # the tables matter
     dh.close()
+
+
+@pytest.mark.parametrize("family,n,r,v,d,N,L,dtype,rank", [
+    (I.HMM, 6, 32, 64, 128, 4, 500, "bf16", 0), (I.HMM, 4, 8, 48, 1600, 3, 100, "f32", 0), (I.BTREE, 8, 16, 64, 128, 2, 400, "bf16", 0),
+    (I.CP, 3, 8, 320, 64, 5, 60, "f32", 0), (I.HMM, 6, 32, 64, 128, 4, 500, "bf16", 16), (I.CP, 2, 64, 80, 64, 2, 90, "bf16", 32),
+])
+def test_training_calls_follow_one_another(family, n, r, v, d, N, L, dtype, rank):
+    """Training calls of the loss over overlapping windows. Three of their kernels work before they wait: the static HMM's sweep copies its
+    tables, the coefficients are formed from the targets, the loss from the prefixes. What they read and write so early must be the work of
+    kernels that have ended, and nobody's any more. On inputs that alternate, and static tables updated right before, each call must give what it
+    gives on an idle device, bit for bit (the gradient of a static table, added up by atomics: 1e-5 of its largest entry)."""
+    T = N * L
+    wl = I.make_workload("train_chain", I.HeadShape(family, n, r, v, d, io_dtype=I.F32 if dtype == "f32" else I.BF16), T, seed=67 + rank, weight_std=0.25)
+    lowrank = I.lowrank_parameters(n, r, v, d, rank, seed=68, weight_std=0.2, adaptor_std=0.1) if rank else None
+    dh = DeviceHead(wl, lowrank=lowrank) if rank else DeviceHead(wl)
+    torch.manual_seed(11)
+    hidden = [dh.hidden_device()]
+    hidden.append(torch.randn_like(hidden[0]))
+    targets = [torch.from_numpy(wl.targets).cuda(), torch.randint(v, (T, n), dtype=torch.int32, device="cuda")]
+    targets[1][::3, n - 1] = -1
+    static = family == I.HMM
+    tables = [dh.T_static, 3.0 * torch.flip(dh.T_static, dims=(2,)).contiguous()] if static else None
+    shapes = dict(W_base=(n, v, d), A=(n, r, v, rank), B=(n, r, rank, d)) if rank else dict(W_emit=(n, r, v, d))
+
+    def run(alone):
+        got = []
+        for i in range(6):
+            out = {k: torch.full(s, 7.0, device="cuda") for k, s in
+                   dict(slot=(n,), loss=(1,), dh=(T, d), **shapes, W_sum=tuple(dh.W_sum.shape)).items()}
+            if static:
+                out["T_static"] = torch.full((n - 1, r, r), 7.0, device="cuda")
+                if not rank:
+                    dh.head.mtpc_update_parameters(dh.W_emit, dh.W_sum, tables[(i // 2) % 2])
+            if alone:
+                torch.cuda.synchronize()
+            call = dh.head.mtpc_lowrank_window_loss_backward if rank else dh.head.mtpc_window_loss_backward
+            call(hidden[i % 2], targets[(i // 3) % 2], N, L, 0.9, *[out[k] for k in ("slot", "loss", "dh", *shapes, "W_sum")], out.get("T_static"))
+            got.append(out)
+        torch.cuda.synchronize()
+        return got
+
+    want, got = run(alone=True), run(alone=False)
+    assert dh.head.mtpc_get_status() == 0
+    for a, b in zip(want, got):
+        for k in a:
+            assert torch.isfinite(a[k]).all(), k
+            if k == "T_static":
+                assert (a[k] - b[k]).abs().max() <= 1e-5 * a[k].abs().max()
+            else:
+                assert torch.equal(a[k], b[k]), k
+    assert not torch.equal(want[0]["slot"], want[1]["slot"]) and not torch.equal(want[2]["slot"], want[3]["slot"])
+    dh.close()

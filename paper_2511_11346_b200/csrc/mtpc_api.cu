@@ -668,6 +668,7 @@ void choose_decode_tiling(long long rows, int sum_rows, int kblocks, int ctas, c
   }
 }
 
+constexpr int kDecodeShortRing = 205000;         // bytes of the weight pass's ring on long runs (see launch_decode_gemm)
 // Few-position draft path: one pass over all weight rows with the positions on the N axis.
 int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_t st) {
   const mtpc_config& c = h->cfg;
@@ -705,13 +706,21 @@ int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_
   if (p.pass_tiles > kDecodeMaxTiles) p.pass_tiles = kDecodeMaxTiles;
   const int tiles = p.emit_tiles + p.emit2_tiles + p.sum_tiles;
   const int per_cta = (tiles + h->num_sms - 1) / h->num_sms;         // no wider stages than a CTA has tiles
-  // A long run of tiles and few positions: passes of two tiles and a ring 28 KB short of the limit. Three tiles a step spread the same bytes
-  // in flight over half as many rows again, 128 bytes from each. 16 x 32 x 320 (9 tiles a CTA), d = 4096, draft alone, as elsewhere / so:
-  // 1 position 225.2 / 213.2 us, 8 229.1 / 217.9, 32 237.5 / 231.2, but 64 253.2 / 251.4 and 128 283.9 / 305.7 (the hidden states, once per
-  // pass, are then a third of what it fetches); 16 x 32 x 256, d = 1024, 8 positions (6 or 7 tiles) 64.5 / 64.0; with 5 tiles a CTA
-  // (16 x 16 x 320) 109.4 / 110.9, with 3 61.6 / 68.8.
-  const bool narrow = per_cta >= 7 && p.Ppad <= 32;
-  if (narrow && p.pass_tiles > 2) p.pass_tiles = 2;
+  // A long run of tiles and few positions (what a stage holds is then nearly all weights). (1) Passes of two tiles where they come out even and
+  // passes of three would end with a pass of one, whose stages are two thirds empty; not with a short K, where more passes cost their starts.
+  // (2) A ring of at most 205 KB: with more bytes in flight the same pass is slower. (Why was not found; it is not the room left to the next
+  // kernel, the pass alone shows it. 154 KB are as slow as 230.) Drafts + acceptance of 1 / 8 / 16 / 32 positions, three tiles and
+  // a full ring / so, in us:
+  //   HMM 16 x 32 x 320 (10 tiles of 112 rows a CTA), d = 4096: 236 242 248 254 / 222 231 238 250; d = 2048: 134 138 145 149.5 / 129 133 142 149.7
+  //   mixture 16 x 64 x 320 (31 of 72), d = 2048: 232 243 253 / 222 230 242, but 32 positions 253 / 256: left as it was from 17 on
+  //   tree 16 x 32 x 256 (9 of 112), d = 3072: 158 163 165 / 156 160 162; contextual HMM 16 x 32 x 256: 170 174 184 / 169 172 180
+  //   16 x 32 x 272 (8 of 120, 11 of 96), 16 x 32 x 256 (7 of 128): the same ring, the same times
+  // Two tiles a pass regardless of what is left over: tree 16 x 32 x 272 125 -> 129, HMM 16 x 32 x 272 115 -> 117; with 10 tiles but d = 1024
+  // 100 -> 101.5 at 32 positions.
+  const bool long_run = per_cta >= 7 && p.Ppad <= 32;
+  const bool by_twos = long_run && p.pass_tiles > 2 && per_cta % 6 == 4 && p.kblocks >= 32;
+  const bool short_ring = by_twos || (long_run && p.Ppad <= 16);
+  if (by_twos) p.pass_tiles = 2;
   const int passes = (per_cta + p.pass_tiles - 1) / p.pass_tiles;
   p.pass_tiles = (per_cta + passes - 1) / passes;                     // passes of one length keep as many bytes in flight throughout
   p.ksplit = h->decode_ksplit;
@@ -722,7 +731,7 @@ int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_
   if (stage < reach) stage = reach;
   p.stage_bytes = (stage + 1023) / 1024 * 1024;
   const int ctl = 1024 + static_cast<int>(sizeof(GemmControl)) + static_cast<int>(decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad));
-  p.stages = (kSmemLimit - ctl - (narrow ? 28000 : 0)) / p.stage_bytes;
+  p.stages = (short_ring ? min(kSmemLimit - ctl, kDecodeShortRing) : kSmemLimit - ctl) / p.stage_bytes;
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   p.logw = at<float>(h, L.off_logw);
   p.sum_bias = sum_bias(h);

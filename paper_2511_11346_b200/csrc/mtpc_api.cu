@@ -1272,7 +1272,10 @@ BackwardShape circuit_backward_shape(const mtpc_head* h, bool loss) {
 }
 
 // Warps (windows at a time) of a CTA of the static HMM's Eq. 6 kernel: the running sums of all n - 1 tables lie in shared memory beside the
-// tables themselves, so few fit for long windows (n = 17 at r = 32 is the last with four); 0: the streaming kernel.
+// tables themselves, so few fit for long windows (at r = 32 sixteen up to n = 16, eight up to n = 21, four up to n = 24); 0: the streaming
+// kernel. Four warps still win, and so do few windows, which sixteen warps a CTA leave on few SMs. Whole training calls of small heads (d = 64),
+// streaming / so, in us: n = 24, r = 32 at 50 windows 202 / 105, 500 271 / 168, 2000 664 / 541; n = 20 at 100 180 / 94; n = 8 at 30 88 / 56,
+// 200 109 / 64, 1500 181 / 129, 8192 677 / 514; n = 8, r = 16 at 200 76 / 51; n = 4, r = 8 at 40 45 / 38.
 size_t hmm_static_loss_smem(const mtpc_config& c, int warps) {
   const size_t tables = (static_cast<size_t>(c.n - 1) * c.r * c.r + 3) / 4 * 4;
   return (2 * tables + warps * hmm_static_loss_warp_floats(c.n, c.r)) * sizeof(float);
@@ -1325,7 +1328,9 @@ int launch_circuit_backward(mtpc_head* h, CircuitBackwardArgs a, float* dT, cuda
     const bool fits = btree_loss_smem_floats(c.n, c.r, tw, true) * sizeof(float) <= static_cast<size_t>(kSmemLimit);
     const size_t tsmem = btree_loss_smem_floats(c.n, c.r, tw, fits) * sizeof(float);
     const int grid = a.W < sms_times_resident(h, tsmem) ? a.W : sms_times_resident(h, tsmem);
-    // (as a dependent, its CTAs crowded beside the projection's last ones: 350 -> 395 us at 4096 positions of a 16 x 32 head)
+    // (Plainly since its sweep on log tables, whose CTAs crowded beside the projection's last ones: 350 -> 395 us at 4096 windows of a 16 x 32
+    // head. For the present sweep it makes no difference there, whole calls plainly / as a dependent 9.66 / 9.71 ms, nor at 1000 windows, 2.56 /
+    // 2.57; small calls would be shorter as dependents: 8 x 16 x 64, d = 512, 2000 windows 202 / 177 us, 4 x 8 x 256, d = 256, 200 windows 59 / 53.)
     auto* kernel = c.r == 32 ? circuit_btree_loss_backward_kernel<32> : c.r == 16 ? circuit_btree_loss_backward_kernel<16>
                    : c.r == 8 ? circuit_btree_loss_backward_kernel<8> : circuit_btree_loss_backward_kernel<0>;
     launch_kernel(kernel, grid, tw * 32, tsmem, st, /*dependent=*/false, a, fits ? 1 : 0);

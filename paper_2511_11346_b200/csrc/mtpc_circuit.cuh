@@ -390,7 +390,10 @@ __device__ __noinline__ float warp_relog(unsigned lost, float x, float vec, cons
 // In shared memory the tables are probabilities, exponentiated once on their way there, so that a step of either sweep is one warp
 // maximum, r multiply-adds per lane and one logarithm (r exponentials of sums, a maximum over them and their sum before). A value whose
 // sum falls below kSumFloor takes the step once more with logarithms, the warp working on its row or column of the log tables in global
-// memory. (4096 windows at n = 16, r = 32, inside a draft: 102 -> 96 us, latency of a window's levels; 27 positions of 4 windows at n = 8:
+// memory. The logarithm is the full-precision one: the fast one's error is relative away from 1, and these sums of products of
+// probabilities lie well below it where a log-sum-exp's lies above, so that log-marginals were off by up to 1.4 times as much as from log tables (rms at
+// 300 windows of n = 16, r = 32: 1.65e-6 from log tables, 2.28e-6 with the fast logarithm, 1.58e-6 so; 0.5 % of the prefix call).
+// (4096 windows at n = 16, r = 32, inside a draft: 102 -> 96 us, latency of a window's levels; 27 positions of 4 windows at n = 8:
 // 8.7 -> 5.8.) Shared memory: btree_prefix_smem_floats.
 // One window of a tree sweep, shared by a CTA. vr: pitch of the [r] vectors (r rounded up to 4 floats).
 template <int R>                                   // r, where the kernel is built for it (0: any)
@@ -478,7 +481,7 @@ struct TreeSweep {
         if (lane < r) vec[lane] = e;
         __syncwarp();
         const float q = row_dot(table_of(c), vec, lane, r);
-        float sc = m + __logf(q);
+        float sc = m + logf(q);
         const unsigned lost = __ballot_sync(kFull, lane < r && q < kSumFloor);
         if (lost != 0) sc = warp_relog(lost, sc, prod, log_table(c), r, 1, lane, r);
         if (lane < r) S[c * vr + lane] = sc;
@@ -496,7 +499,7 @@ struct TreeSweep {
         if (lane < r) vec[lane] = u;
         __syncwarp();
         const float q = col_dot(table_of(c), vec, lane, r);
-        float dc = m + __logf(q);
+        float dc = m + logf(q);
         const unsigned lost = __ballot_sync(kFull, lane < r && q < kSumFloor);
         if (lost != 0) dc = warp_relog(lost, dc, in, log_table(c), 1, r, lane, r);
         if (lane < r) D[c * vr + lane] = dc;

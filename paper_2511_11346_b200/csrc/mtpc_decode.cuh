@@ -70,6 +70,10 @@ __device__ __forceinline__ DecodeTile decode_tile(const DecodeParams& p, int t) 
   return d;
 }
 
+// The warps that issue copies and MMAs run as wholes (elect_one): four MMAs of N = 16 and their copies, issued from a branch of lane 0's own,
+// took 650 cycles a K step and tile, more than the step's bytes where a CTA has one tile (draft + acceptance of 8 positions of a factored
+// head, d = 4096: 32.7 -> 27.0 us; 4 x 8 x 256, d = 1024, 16 positions: 20.0 -> 17.4) and nearly as much where it has three (mixture
+// 8 x 16 x 320, 1 position 65.7 -> 63.6, HMM 16 x 32 x 320, 8 positions 225.7 -> 221.5; 128 positions of the mixture 96.7 -> 89.3).
 // A CTA walks its run of tiles in passes of up to pass_tiles tiles (of either matrix). Shared-memory stage:
 // pass_tiles weight tiles at a pitch of tile_bytes (the MMA reads 128 rows from each tile's base: what lies beyond
 // the tile's own rows is other data, and the TMEM lanes it produces are never read), then the hidden tile
@@ -92,10 +96,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
   uint8_t* exchange = tiles + static_cast<size_t>(p.stages) * p.stage_bytes;
   GemmControl* ctl = reinterpret_cast<GemmControl*>(exchange + decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad));
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = static_cast<int>(warp_uniform(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   const int total_tiles = p.emit_tiles + p.emit2_tiles + p.sum_tiles;
-  const int rank = p.ksplit > 1 ? static_cast<int>(cluster_cta_rank()) : 0;
+  const int rank = p.ksplit > 1 ? static_cast<int>(warp_uniform(cluster_cta_rank())) : 0;
   const int group = static_cast<int>(blockIdx.x) / p.ksplit, groups = static_cast<int>(gridDim.x) / p.ksplit;
   const int tile_begin = static_cast<int>(static_cast<long long>(group) * total_tiles / groups);
   const int tile_end = static_cast<int>(static_cast<long long>(group + 1) * total_tiles / groups);
@@ -129,7 +133,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
   __syncthreads();
   if (p.ksplit > 1) cluster_sync_all();   // every CTA of the cluster runs before one writes into another's shared memory
   tc_fence_after();
-  const uint32_t tmem_base = ctl->tmem_base;
+  const uint32_t tmem_base = warp_uniform(ctl->tmem_base);
   grid_dependency_wait();     // a draft that follows another call closely sets up its barriers while that one finishes
   grid_launch_dependents();   // (after the wait: the per-slot kernel reads static tables early) it waits for this grid's results
 
@@ -194,83 +198,78 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued = 0;
-      bool ok = true;
-      const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-      for (int cur = tile_begin; cur < tile_end && ok;) {
-        const int ntiles = min(p.pass_tiles, tile_end - cur);
-        uint32_t bytes = p.Ppad * (kBlockK * 2);                   // out-of-range rows are zero-filled and counted
-        const CUtensorMap* map[kDecodeMaxTiles];
-        int row[kDecodeMaxTiles];
+    const uint32_t lead = elect_one();
+    uint32_t stage = 0, phase = 0, issued = 0;
+    bool ok = true;
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+    for (int cur = tile_begin; cur < tile_end && ok;) {
+      const int ntiles = min(p.pass_tiles, tile_end - cur);
+      uint32_t bytes = p.Ppad * (kBlockK * 2);                   // out-of-range rows are zero-filled and counted
+      const CUtensorMap* map[kDecodeMaxTiles];
+      int row[kDecodeMaxTiles];
 #pragma unroll
-        for (int q = 0; q < kDecodeMaxTiles; ++q) {
-          const DecodeTile t = decode_tile(p, min(cur + q, tile_end - 1));
-          map[q] = t.is_sum ? &p.tm_sum : (t.second ? &p.tm_emit2 : &p.tm_emit);
-          row[q] = t.index * t.rows;
-          if (q < ntiles) bytes += t.rows * (kBlockK * 2);
-        }
-        for (int k = kb0 * kBlockK; k < kb1 * kBlockK; k += kBlockK) {
-          if (!bounded_wait(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
-          const uint32_t full = full0 + 8 * stage, dst = tiles_addr + stage * p.stage_bytes;
-          mbar_arrive_expect_tx(full, bytes);
+      for (int q = 0; q < kDecodeMaxTiles; ++q) {
+        const DecodeTile t = decode_tile(p, min(cur + q, tile_end - 1));
+        map[q] = t.is_sum ? &p.tm_sum : (t.second ? &p.tm_emit2 : &p.tm_emit);
+        row[q] = t.index * t.rows;
+        if (q < ntiles) bytes += t.rows * (kBlockK * 2);
+      }
+      for (int k = kb0 * kBlockK; k < kb1 * kBlockK; k += kBlockK) {
+        if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
+        const uint32_t full = full0 + 8 * stage, dst = tiles_addr + stage * p.stage_bytes;
+        mbar_arrive_expect_tx(lead, full, bytes);
 #pragma unroll
-          for (int q = 0; q < kDecodeMaxTiles; ++q)
-            if (q < ntiles) tma_load_2d(dst + q * p.tile_bytes, map[q], full, k, row[q]);
-          tma_load_2d(dst + hidden_off, &p.tm_h, full, k, 0);
-          ++issued;
-          if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
-        }
-        cur += ntiles;
+        for (int q = 0; q < kDecodeMaxTiles; ++q)
+          if (q < ntiles) tma_load_2d(lead, dst + q * p.tile_bytes, map[q], full, k, row[q]);
+        tma_load_2d(lead, dst + hidden_off, &p.tm_h, full, k, 0);
+        ++issued;
+        if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
       }
-      // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
-      for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s) {
-        const uint32_t par = ((issued - 1 - s) / p.stages) & 1u;
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(full0 + 8 * s, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
-      }
+      cur += ntiles;
     }
+    // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
+    for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s)
+      drain_wait(full0 + 8 * s, ((issued - 1 - s) / p.stages) & 1u);
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer: D[row, p] = W[row, :] . h[p, :]
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, use = 0;
-      bool ok = true;
-      const uint32_t idesc = umma_idesc_bf16(kBlockM, p.Ppad);
-      const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-      const uint32_t stage_step = p.stage_bytes >> 4, tile_step = p.tile_bytes >> 4;          // descriptors step in 16-byte units
-      const uint64_t a_desc0 = umma_smem_desc_sw128(tiles_addr), b_desc0 = umma_smem_desc_sw128(tiles_addr + hidden_off);
-      for (int cur = tile_begin; cur < tile_end && ok; ++use) {
-        const int ntiles = min(p.pass_tiles, tile_end - cur);
-        cur += ntiles;
-        const uint32_t slot = use & 1u;
-        if (!bounded_wait(smem_u32(&ctl->tempty[slot]), ((use >> 1) & 1u) ^ 1u, ctl, p.status)) {
-          ok = false;
-          break;
-        }
+    const uint32_t lead = elect_one();
+    uint32_t stage = 0, phase = 0, use = 0;
+    bool ok = true;
+    const uint32_t idesc = umma_idesc_bf16(kBlockM, p.Ppad);
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+    const uint32_t stage_step = p.stage_bytes >> 4, tile_step = p.tile_bytes >> 4;          // descriptors step in 16-byte units
+    const uint64_t a_desc0 = umma_smem_desc_sw128(tiles_addr), b_desc0 = umma_smem_desc_sw128(tiles_addr + hidden_off);
+    for (int cur = tile_begin; cur < tile_end && ok; ++use) {
+      const int ntiles = min(p.pass_tiles, tile_end - cur);
+      cur += ntiles;
+      const uint32_t slot = use & 1u;
+      if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use >> 1) & 1u) ^ 1u, ctl, p.status)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + slot * slot_cols;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + slot * slot_cols;
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!bounded_wait(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
-          tc_fence_after();
-          const uint64_t b_desc = b_desc0 + stage * stage_step;
-          for (int q = 0; q < ntiles; ++q) {
-            const uint64_t a_desc = a_desc0 + stage * stage_step + q * tile_step;
+        const uint64_t a_desc = a_desc0 + stage * stage_step, b_desc = b_desc0 + stage * stage_step;
+#pragma unroll
+        for (int q = 0; q < kDecodeMaxTiles; ++q)
+          if (q < ntiles) {
 #pragma unroll
             for (int kk = 0; kk < kBlockK / 16; ++kk)
-              umma_bf16(d_tmem + q * p.tile_stride, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
+              umma_bf16(lead, d_tmem + q * p.tile_stride, a_desc + q * tile_step + 2 * kk, b_desc + 2 * kk, idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
           }
-          umma_commit(empty0 + 8 * stage);
-          if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
-        }
-        if (!ok) break;
-        umma_commit(smem_u32(&ctl->tfull[slot]));
+        umma_commit(lead, empty0 + 8 * stage);
+        if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) {
-        umma_commit(smem_u32(&ctl->drain));
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(smem_u32(&ctl->drain), 0) && global_timer_ns() - t0 < kWaitLimitNs) {}
-      }
+      if (!ok) break;
+      umma_commit(lead, smem_u32(&ctl->tfull[slot]));
+    }
+    if (!ok) {
+      umma_commit(lead, smem_u32(&ctl->drain));
+      drain_wait(smem_u32(&ctl->drain), 0);
     }
     __syncwarp();
   } else {

@@ -105,7 +105,7 @@ __device__ __forceinline__ bool bounded_wait(uint32_t bar, uint32_t parity, Gemm
   uint32_t it = 0;
   while (true) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((++it & 63u) == 0) {
+    if ((++it & 15u) == 0) {
       if (ctl->abort) return false;
       if (global_timer_ns() - t0 > ctl->wait_limit_ns) {
         ctl->abort = 1;
@@ -121,6 +121,29 @@ __device__ __forceinline__ bool bounded_wait_warp(uint32_t bar, uint32_t parity,
   int ok = 1;
   if (lane == 0) ok = bounded_wait(bar, parity, ctl, status) ? 1 : 0;
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+// The whole warp waits and learns the outcome, known to be the same in every lane. A warp that waits as a whole sleeps in try_wait until
+// the barrier's phase is over or the hardware's own limit is, which is longer than any wait of a healthy call: limits of microseconds are
+// noticed by the epilogue's warps, whose lane 0 polls.
+__device__ __forceinline__ bool bounded_wait_all(uint32_t bar, uint32_t parity, GemmControl* ctl, unsigned* status) {
+  constexpr unsigned all = 0xffffffffu;
+  if (__all_sync(all, mbar_try_wait(bar, parity))) return true;
+  const uint64_t t0 = global_timer_ns();
+  while (true) {
+    if (__all_sync(all, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(all, ctl->abort)) return false;
+    if (__any_sync(all, global_timer_ns() - t0 > ctl->wait_limit_ns)) {
+      ctl->abort = 1;
+      if (elect_one()) atomicOr(status, kStatusTimeout);
+      return false;
+    }
+  }
+}
+// A wait that decides nothing: for what may still be in flight when a CTA goes away.
+__device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity) {
+  const uint64_t t0 = global_timer_ns();
+  while (!mbar_try_wait(bar, parity) && global_timer_ns() - t0 < kWaitLimitNs) {}
 }
 
 struct TileCoord {

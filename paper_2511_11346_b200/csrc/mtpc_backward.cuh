@@ -1159,11 +1159,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
   const uint32_t tiles_addr = (raw_addr + 1023u) & ~1023u;
   uint8_t* tiles = smem_raw + (tiles_addr - raw_addr);
   GemmControl* ctl = reinterpret_cast<GemmControl*>(tiles + static_cast<size_t>(p.stages) * p.stage_bytes);
-  const int warp = threadIdx.x >> 5;
+  const int warp = static_cast<int>(warp_uniform(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   const int kblocks = p.seg_kblocks[0] + p.seg_kblocks[1] + p.seg_kblocks[2];
   const int num_items = p.m_tiles * p.n_tiles * p.batches + p.tail_tiles * (p.split - 1);
-  const uint32_t cta_rank = CTAS == 2 ? cluster_cta_rank() : 0u;      // 0 = the pair's leader
+  const uint32_t cta_rank = CTAS == 2 ? warp_uniform(cluster_cta_rank()) : 0u;      // 0 = the pair's leader
   const int first_item = CTAS == 2 ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
   const int item_step = CTAS == 2 ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
   constexpr uint32_t kSlots = 2;
@@ -1202,64 +1202,61 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
   __syncthreads();
   if (CTAS == 2) cluster_sync_all();   // the peer's barriers are initialised before anything arrives on them
   tc_fence_after();
-  const uint32_t tmem_base = ctl->tmem_base;
+  const uint32_t tmem_base = warp_uniform(ctl->tmem_base);
   grid_launch_dependents();            // the next kernel's CTAs may be scheduled as SMs free up
   grid_dependency_wait();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // One K block must be asked for in less time than its MMAs take (256 cycles), so that little is computed per block.
-      uint32_t stage = 0, phase = 0, issued = 0;
-      bool ok = true;
-      auto load = [&](uint32_t dst, const CUtensorMap* tm, uint32_t full, int x, int y) {
-        if (CTAS == 2) tma_load_2d_pair(dst, tm, full, x, y);
-        else tma_load_2d(dst, tm, full, x, y);
-      };
-      const uint32_t own_full = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-      const uint32_t full0 = CTAS == 2 ? cluster_map_shared(own_full, 0) : own_full;             // the leader's barriers
-      for (int item = first_item; item < num_items && ok; item += item_step) {
-        const PlainItem w = plain_item(p, item, kblocks);
-        const int am = (w.mt * CTAS + static_cast<int>(cta_rank)) * kBlockM + w.bt * p.a_m_step;   // this CTA's rows of A,
-        const int bn = w.nt * TN + static_cast<int>(cta_rank) * kBCols + w.bt * p.b_n_step;        // its columns of B
-        int kb = w.kb0, seg_begin = 0;
-        for (int seg = 0; seg < 3 && ok; ++seg) {
-          const int seg_end = seg_begin + p.seg_kblocks[seg], stop = min(seg_end, w.kb1);
-          const CUtensorMap* tm_b = &p.tm_b[seg];
-          int ak = p.a_k0[seg] + (kb - seg_begin) * kBlockK + w.bt * p.a_k_step, bk = (kb - seg_begin) * kBlockK + w.bt * p.b_k_step;
-          for (; kb < stop; ++kb, ak += kBlockK, bk += kBlockK) {
-            if (!bounded_wait(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
-            const uint32_t full = full0 + 8 * stage, a_dst = tiles_addr + stage * p.stage_bytes;
-            if (cta_rank == 0) mbar_arrive_expect_tx(own_full + 8 * stage, CTAS * (kABytes + kBBytes));   // of both CTAs' copies when paired
-            if (A_MN) {
+    // One K block must be asked for in less time than its MMAs take (256 cycles), so that little is computed per block.
+    const uint32_t lead = elect_one(), expects = cta_rank == 0 ? lead : 0u;
+    uint32_t stage = 0, phase = 0, issued = 0;
+    bool ok = true;
+    auto load = [&](uint32_t dst, const CUtensorMap* tm, uint32_t full, int x, int y) {
+      if (CTAS == 2) tma_load_2d_pair(lead, dst, tm, full, x, y);
+      else tma_load_2d(lead, dst, tm, full, x, y);
+    };
+    const uint32_t own_full = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+    const uint32_t full0 = CTAS == 2 ? warp_uniform(cluster_map_shared(own_full, 0)) : own_full;   // the leader's barriers
+    for (int item = first_item; item < num_items && ok; item += item_step) {
+      const PlainItem w = plain_item(p, item, kblocks);
+      const int am = (w.mt * CTAS + static_cast<int>(cta_rank)) * kBlockM + w.bt * p.a_m_step;   // this CTA's rows of A,
+      const int bn = w.nt * TN + static_cast<int>(cta_rank) * kBCols + w.bt * p.b_n_step;        // its columns of B
+      int kb = w.kb0, seg_begin = 0;
+      for (int seg = 0; seg < 3 && ok; ++seg) {
+        const int seg_end = seg_begin + p.seg_kblocks[seg], stop = min(seg_end, w.kb1);
+        const CUtensorMap* tm_b = &p.tm_b[seg];
+        int ak = p.a_k0[seg] + (kb - seg_begin) * kBlockK + w.bt * p.a_k_step, bk = (kb - seg_begin) * kBlockK + w.bt * p.b_k_step;
+        for (; kb < stop; ++kb, ak += kBlockK, bk += kBlockK) {
+          if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
+          const uint32_t full = full0 + 8 * stage, a_dst = tiles_addr + stage * p.stage_bytes;
+          mbar_arrive_expect_tx(expects, own_full + 8 * stage, CTAS * (kABytes + kBBytes));      // of both CTAs' copies when paired
+          if (A_MN) {
 #pragma unroll
-              for (int q = 0; q < kBlockM / 64; ++q) load(a_dst + q * kMnBoxBytes, &p.tm_a, full, am + q * 64, ak);
-            } else {
-              load(a_dst, &p.tm_a, full, ak, am);
-            }
-            if (B_MN) {
-#pragma unroll
-              for (int q = 0; q < kBCols / 64; ++q) load(a_dst + kABytes + q * kMnBoxBytes, tm_b, full, bn + q * 64, bk);
-            } else {
-              load(a_dst + kABytes, tm_b, full, bk, bn);
-            }
-            ++issued;
-            if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
+            for (int q = 0; q < kBlockM / 64; ++q) load(a_dst + q * kMnBoxBytes, &p.tm_a, full, am + q * 64, ak);
+          } else {
+            load(a_dst, &p.tm_a, full, ak, am);
           }
-          seg_begin = seg_end;
+          if (B_MN) {
+#pragma unroll
+            for (int q = 0; q < kBCols / 64; ++q) load(a_dst + kABytes + q * kMnBoxBytes, tm_b, full, bn + q * 64, bk);
+          } else {
+            load(a_dst + kABytes, tm_b, full, bk, bn);
+          }
+          ++issued;
+          if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
         }
+        seg_begin = seg_end;
       }
-      // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
-      if (CTAS == 1 || cta_rank == 0) {
-        for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s) {
-          const uint32_t par = ((issued - 1 - s) / p.stages) & 1u;
-          const uint64_t t0 = global_timer_ns();
-          while (!mbar_try_wait(own_full + 8 * s, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
-        }
-      }
+    }
+    // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
+    if (CTAS == 1 || cta_rank == 0) {
+      for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s)
+        drain_wait(own_full + 8 * s, ((issued - 1 - s) / p.stages) & 1u);
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && cta_rank == 0) {
+    if (cta_rank == 0) {
+      const uint32_t lead = elect_one();
       uint32_t stage = 0, phase = 0, use = 0;
       bool ok = true;
       const uint32_t idesc = umma_idesc_bf16(kBlockM * CTAS, TN, A_MN, B_MN);
@@ -1270,35 +1267,35 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
       const uint64_t b_desc0 = B_MN ? umma_smem_desc_mn_sw128(tiles_addr + kABytes, kMnBoxBytes)
                                     : umma_smem_desc_sw128(tiles_addr + kABytes);
       const uint32_t stage_step = p.stage_bytes >> 4, full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+      auto commit = [&](uint32_t bar) {                        // pairs: in both CTAs
+        if (CTAS == 2) umma_commit_pair(lead, bar);
+        else umma_commit(lead, bar);
+      };
       for (int item = first_item; item < num_items && ok; item += item_step, ++use) {
         const PlainItem w = plain_item(p, item, kblocks);
         const uint32_t slot = use % kSlots;
-        if (!bounded_wait(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+        if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + slot * TN;
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (!bounded_wait(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
+          if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
           tc_fence_after();
           const uint64_t a_desc = a_desc0 + stage * stage_step, b_desc = b_desc0 + stage * stage_step;
 #pragma unroll
           for (int kk = 0; kk < kBlockK / 16; ++kk) {
             const uint32_t acc = (kb != w.kb0 || kk != 0) ? 1u : 0u;
-            if (CTAS == 2) umma_bf16_pair(d_tmem, a_desc + kStepA * kk, b_desc + kStepB * kk, idesc, acc);
-            else umma_bf16(d_tmem, a_desc + kStepA * kk, b_desc + kStepB * kk, idesc, acc);
+            if (CTAS == 2) umma_bf16_pair(lead, d_tmem, a_desc + kStepA * kk, b_desc + kStepB * kk, idesc, acc);
+            else umma_bf16(lead, d_tmem, a_desc + kStepA * kk, b_desc + kStepB * kk, idesc, acc);
           }
-          if (CTAS == 2) umma_commit_pair(empty0 + 8 * stage);
-          else umma_commit(empty0 + 8 * stage);
+          commit(empty0 + 8 * stage);
           if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        if (CTAS == 2) umma_commit_pair(smem_u32(&ctl->tfull[slot]));
-        else umma_commit(smem_u32(&ctl->tfull[slot]));
+        commit(smem_u32(&ctl->tfull[slot]));
       }
       if (!ok) {
-        if (CTAS == 2) umma_commit_pair(smem_u32(&ctl->drain));
-        else umma_commit(smem_u32(&ctl->drain));
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(smem_u32(&ctl->drain), 0) && global_timer_ns() - t0 < kWaitLimitNs) {}
+        commit(smem_u32(&ctl->drain));
+        drain_wait(smem_u32(&ctl->drain), 0);
       }
     }
     __syncwarp();

@@ -6,7 +6,9 @@
 // One persistent CTA per SM, 6 warps:
 //   warp 0      TMA producer: per 64-wide K block, one 128-row tile of h and the v rows of one emission unit
 //               (or one tile of sum-unit rows) into a ring of shared-memory stages (128-byte swizzle).
-//   warp 1      allocates the 512 TMEM columns, issues tcgen05.mma (M=128, N=chunk, K=16) from one thread.
+//   warp 1      allocates the 512 TMEM columns, issues tcgen05.mma (M=128, N=chunk, K=16) from one thread. Warps 0 and 1 run as wholes
+//               and predicate what they issue (elect_one): short calls 1 to 6 % shorter than from branches of lane 0's own (300 factored
+//               positions of 4 x 8 x 256, d = 1024: 45.6 -> 42.8 us, 500 of 8 x 16 x 320, d = 2048: 69.0 -> 67.7).
 //   warps 2..5  epilogue; warp w reads TMEM lanes 32*(w%4)..+31, one thread per position (row), so every
 //               row-wise reduction over the vocabulary is a plain in-thread loop.
 // The N axis of the GEMM is the flattened (slot i, unit k, byte b) row index of W_emit. A work item is 128
@@ -277,13 +279,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   uint8_t* tiles = smem_raw + (tiles_addr - raw_addr);
   GemmControl* ctl = reinterpret_cast<GemmControl*>(tiles + static_cast<size_t>(p.stages) * p.stage_bytes);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = static_cast<int>(warp_uniform(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   constexpr bool kGrouped = MODE == kModeLogitsGrouped;
   if (kGrouped) grid_dependency_wait();   // the tiles are read below
   static_assert(!kGrouped || CTAS == 1, "grouped tiles are ragged: no pairing");
-  const int emit_items = kGrouped ? *p.group_num_tiles * p.num_groups : p.num_groups * p.m_units;
-  const uint32_t cta_rank = CTAS == 2 ? cluster_cta_rank() : 0u;      // 0 = the pair's leader
+  const int emit_items = kGrouped ? static_cast<int>(warp_uniform(*p.group_num_tiles)) * p.num_groups : p.num_groups * p.m_units;
+  const uint32_t cta_rank = CTAS == 2 ? warp_uniform(cluster_cta_rank()) : 0u;      // 0 = the pair's leader
   auto coord = [&](int item) {
     if (kGrouped) return group_coord(p, item);
     TileCoord c = tile_coord(p, item);
@@ -325,94 +327,92 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   __syncthreads();
   if (CTAS == 2) cluster_sync_all();   // the peer's barriers are initialised before anything arrives on them
   tc_fence_after();
-  const uint32_t tmem_base = ctl->tmem_base;
+  const uint32_t tmem_base = warp_uniform(ctl->tmem_base);
   grid_dependency_wait();     // barriers and tensor memory were set up while the kernel before this one finished
   grid_launch_dependents();   // (after the wait: kernels behind this one read a head's static tables early) they wait for this grid's results
   if (p.work_counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *p.work_counter = 0;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued = 0;
-      bool ok = true;
-      const uint32_t own_full = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-      const uint32_t full0 = CTAS == 2 ? cluster_map_shared(own_full, 0) : own_full;             // the leader's barriers
-      for (int item = walk.first(); item < walk.end && ok; item = walk.next(item)) {
-        const TileCoord tc = coord(item);
-        const CUtensorMap* tmb = tc.is_sum ? &p.tm_sum : &p.tm_emit;
-        const int brows = tc.cols / CTAS;                                 // weight rows this CTA stages per tile
-        const uint32_t bytes = CTAS * (kABytes + brows * (kBlockK * 2));   // of both CTAs' copies when paired
-        const int arow = tc.arow;
-        for (int t = 0; t < tc.ntiles && ok; ++t) {
-          const int brow = tc.brow0 + t * tc.cols + static_cast<int>(cta_rank) * brows;
-          for (int k = 0; k < p.kblocks * kBlockK; k += kBlockK) {
-            if (!bounded_wait(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
-            const uint32_t full = full0 + 8 * stage, a_dst = tiles_addr + stage * p.stage_bytes;
-            if (cta_rank == 0) mbar_arrive_expect_tx(own_full + 8 * stage, bytes);
-            if (CTAS == 2) {
-              tma_load_2d_pair(a_dst, &p.tm_a, full, k, arow);
-              tma_load_2d_pair(a_dst + kABytes, tmb, full, k, brow);
-            } else {
-              tma_load_2d(a_dst, &p.tm_a, full, k, arow);
-              tma_load_2d(a_dst + kABytes, tmb, full, k, brow);
-            }
-            ++issued;
-            if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
+    const uint32_t lead = elect_one(), expects = cta_rank == 0 ? lead : 0u;
+    uint32_t stage = 0, phase = 0, issued = 0;
+    bool ok = true;
+    const uint32_t own_full = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+    const uint32_t full0 = CTAS == 2 ? warp_uniform(cluster_map_shared(own_full, 0)) : own_full;   // the leader's barriers
+    for (int item = walk.first(); item < walk.end && ok; item = walk.next(item)) {
+      const TileCoord tc = coord(item);
+      const CUtensorMap* tmb = tc.is_sum ? &p.tm_sum : &p.tm_emit;
+      const int brows = tc.cols / CTAS;                                 // weight rows this CTA stages per tile
+      const uint32_t bytes = CTAS * (kABytes + brows * (kBlockK * 2));   // of both CTAs' copies when paired
+      const int arow = kGrouped ? static_cast<int>(warp_uniform(tc.arow)) : tc.arow;
+      const int brow0 = kGrouped ? static_cast<int>(warp_uniform(tc.brow0)) : tc.brow0;
+      for (int t = 0; t < tc.ntiles && ok; ++t) {
+        const int brow = brow0 + t * tc.cols + static_cast<int>(cta_rank) * brows;
+        for (int k = 0; k < p.kblocks * kBlockK; k += kBlockK) {
+          if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
+          const uint32_t full = full0 + 8 * stage, a_dst = tiles_addr + stage * p.stage_bytes;
+          mbar_arrive_expect_tx(expects, own_full + 8 * stage, bytes);
+          if (CTAS == 2) {
+            tma_load_2d_pair(lead, a_dst, &p.tm_a, full, k, arow);
+            tma_load_2d_pair(lead, a_dst + kABytes, tmb, full, k, brow);
+          } else {
+            tma_load_2d(lead, a_dst, &p.tm_a, full, k, arow);
+            tma_load_2d(lead, a_dst + kABytes, tmb, full, k, brow);
           }
+          ++issued;
+          if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
         }
       }
-      // The CTA must not go away with copies in flight. After a full run they have all landed already (the MMA warp
-      // consumed them); after an abort, by this warp or by another one, give them a bounded chance to land.
-      if (CTAS == 1 || cta_rank == 0) {
-        for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s) {
-          const uint32_t par = ((issued - 1 - s) / p.stages) & 1u;
-          const uint64_t t0 = global_timer_ns();
-          while (!mbar_try_wait(own_full + 8 * s, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
-        }
-      }
+    }
+    // The CTA must not go away with copies in flight. After a full run they have all landed already (the MMA warp
+    // consumed them); after an abort, by this warp or by another one, give them a bounded chance to land.
+    if (CTAS == 1 || cta_rank == 0) {
+      for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s)
+        drain_wait(own_full + 8 * s, ((issued - 1 - s) / p.stages) & 1u);
     }
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0 && cta_rank == 0) {
+    if (cta_rank == 0) {
+      const uint32_t lead = elect_one();
       uint32_t stage = 0, phase = 0, use = 0;
       bool ok = true;
       const uint64_t a_desc0 = umma_smem_desc_sw128(tiles_addr), b_desc0 = umma_smem_desc_sw128(tiles_addr + kABytes);
       const uint32_t stage_step = p.stage_bytes >> 4, full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+      auto commit = [&](uint32_t bar) {                        // pairs: in both CTAs
+        if (CTAS == 2) umma_commit_pair(lead, bar);
+        else umma_commit(lead, bar);
+      };
       for (int item = walk.first(); item < walk.end && ok; item = walk.next(item)) {
         const TileCoord tc = coord(item);
         const uint32_t idesc = umma_idesc_bf16(kBlockM * CTAS, tc.cols);
         for (int t = 0; t < tc.ntiles && ok; ++t, ++use) {
           const uint32_t slot = use % p.num_slots;
-          if (!bounded_wait(smem_u32(&ctl->tempty[slot]), ((use / p.num_slots) & 1u) ^ 1u, ctl, p.status)) {
+          if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use / p.num_slots) & 1u) ^ 1u, ctl, p.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + slot * p.slot_stride;
           for (int kb = 0; kb < p.kblocks; ++kb) {
-            if (!bounded_wait(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
+            if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
             tc_fence_after();
             const uint64_t a_desc = a_desc0 + stage * stage_step, b_desc = b_desc0 + stage * stage_step;
 #pragma unroll
             for (int kk = 0; kk < kBlockK / 16; ++kk) {   // +32 bytes per K=16 step inside the swizzled row
-              if (CTAS == 2) umma_bf16_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
-              else umma_bf16(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+              if (CTAS == 2) umma_bf16_pair(lead, d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+              else umma_bf16(lead, d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
             }
-            if (CTAS == 2) umma_commit_pair(empty0 + 8 * stage);   // frees the stage in both CTAs
-            else umma_commit(empty0 + 8 * stage);
+            commit(empty0 + 8 * stage);                   // frees the stage
             if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
           }
           if (!ok) break;
-          if (CTAS == 2) umma_commit_pair(smem_u32(&ctl->tfull[slot]));      // the accumulators of both CTAs are ready
-          else umma_commit(smem_u32(&ctl->tfull[slot]));
+          commit(smem_u32(&ctl->tfull[slot]));            // the accumulators are ready
         }
       }
       if (!ok) {   // wait (bounded) for the MMAs already issued before TMEM is freed
-        if (CTAS == 2) umma_commit_pair(smem_u32(&ctl->drain));
-        else umma_commit(smem_u32(&ctl->drain));
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(smem_u32(&ctl->drain), 0) && global_timer_ns() - t0 < kWaitLimitNs) {}
+        commit(smem_u32(&ctl->drain));
+        drain_wait(smem_u32(&ctl->drain), 0);
       }
     }
     __syncwarp();

@@ -25,6 +25,7 @@
 // busy for 73 / 43 % of the cycles (61 / 38); the gradient's rest is instructions (two thirds of an issue slot a logit) and its warps' latency.
 // The fused projection that kept logits took 801 us and the passes that made g and its sum from them 921.
 // Roles: warp 0 TMA producer, warp 1 MMA issuer, then the epilogue warps (TMEM quarter warp % 4).
+// Both issue from a converged warp (elect_one): forward 240 -> 222 us, gradient 403 -> 398.
 // Operand ring: one entry holds 32 / k components, all as 128-byte rows with the 128-byte swizzle: z as one box of 128
 // positions x 64 values ([hi | lo] of the components), and A as one box of the item's vocabulary rows x 64 values (the components' k
 // adaptor columns first) of a copy laid out [n, v, r, k] (lowrank_repack_kernel, made on every call: A is small and may have changed).
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) low
   float* patches = reinterpret_cast<float*>(smem_raw + (ring - raw_addr) + kLrStages * kLrStageBytes);
   GemmControl* ctl = reinterpret_cast<GemmControl*>(patches + lowrank_patch_floats(MODE));
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = static_cast<int>(warp_uniform(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   const int num_items = p.m_tiles * p.n * p.blocks;
   const int npairs = (p.r + 1) / 2;                       // components go through in pairs (r = 1: one and its copy)
@@ -150,89 +151,85 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) low
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = ctl->tmem_base;
+  const uint32_t tmem_base = warp_uniform(ctl->tmem_base);
   grid_launch_dependents();
   grid_dependency_wait();
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      uint32_t st = 0, phase = 0, issued_mask = 0, phase_mask = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-        const LowRankItem w = lowrank_item(p, item);
-        for (int e = 0; e < nent; ++e) {
-          if (!bounded_wait(smem_u32(&ctl->empty[st]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
-          const uint32_t full = smem_u32(&ctl->full[st]);
-          const uint32_t dst = ring + st * kLrStageBytes;
-          const int j = e * per_entry;                       // first component of the entry
-          mbar_arrive_expect_tx(full, kLrStageBytes);
-          // the boxes may cover components past the slot's last (the next slot's, or zeros past the end), adaptor columns past the
-          // entry's and rows past the unit: none of that is multiplied
-          tma_load_2d(dst, &p.tm_z, full, (w.slot * p.r + j) * 2 * p.k, w.mt * kBlockM);
-          tma_load_2d(dst + kLrZBox, &p.tm_a, full, j * p.k, w.slot * p.v + w.block * kLrCols);
-          issued_mask |= 1u << st;
-          phase_mask = (phase_mask & ~(1u << st)) | (phase << st);
-          if (++st == kLrStages) { st = 0; phase ^= 1u; }
-        }
+    const uint32_t lead = elect_one();
+    uint32_t st = 0, phase = 0, issued = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
+      const LowRankItem w = lowrank_item(p, item);
+      for (int e = 0; e < nent; ++e) {
+        if (!bounded_wait_all(smem_u32(&ctl->empty[st]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
+        const uint32_t full = smem_u32(&ctl->full[st]);
+        const uint32_t dst = ring + st * kLrStageBytes;
+        const int j = e * per_entry;                       // first component of the entry
+        mbar_arrive_expect_tx(lead, full, kLrStageBytes);
+        // the boxes may cover components past the slot's last (the next slot's, or zeros past the end), adaptor columns past the
+        // entry's and rows past the unit: none of that is multiplied
+        tma_load_2d(lead, dst, &p.tm_z, full, (w.slot * p.r + j) * 2 * p.k, w.mt * kBlockM);
+        tma_load_2d(lead, dst + kLrZBox, &p.tm_a, full, j * p.k, w.slot * p.v + w.block * kLrCols);
+        ++issued;
+        if (++st == kLrStages) { st = 0; phase ^= 1u; }
       }
-      // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
-      for (int s = 0; s < kLrStages; ++s)
-        if (issued_mask & (1u << s)) {
-          const uint32_t bar = smem_u32(&ctl->full[s]);
-          const uint32_t par = (phase_mask >> s) & 1u;
-          const uint64_t t0 = global_timer_ns();
-          while (!mbar_try_wait(bar, par) && global_timer_ns() - t0 < kWaitLimitNs) {}
-        }
     }
+    // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
+    for (uint32_t s = 0; s < kLrStages && s < issued; ++s) drain_wait(smem_u32(&ctl->full[s]), ((issued - 1 - s) / kLrStages) & 1u);
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer: pair u overall into slot u % kSlots
-    if (lane == 0) {
-      uint32_t st = 0, phase = 0, use = 0;
-      bool ok = true;
-      const uint64_t z_desc0 = umma_smem_desc_sw128(ring), a_desc0 = umma_smem_desc_sw128(ring + kLrZBox);
-      constexpr uint32_t kStageStep = kLrStageBytes >> 4;      // descriptors step in 16-byte units
-      auto next_stage = [&] {
-        umma_commit(smem_u32(&ctl->empty[st]));
-        if (++st == kLrStages) { st = 0; phase ^= 1u; }
-      };
-      for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
-        const LowRankItem w = lowrank_item(p, item);
-        const uint32_t idesc = umma_idesc_bf16(kBlockM, w.width);
-        for (int pr = 0; pr < npairs && ok; ++pr, ++use) {
-          const uint32_t slot = use % kSlots;
-          if (!bounded_wait(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+    const uint32_t lead = elect_one();
+    uint32_t st = 0, phase = 0, use = 0;
+    bool ok = true;
+    const uint64_t z_desc0 = umma_smem_desc_sw128(ring), a_desc0 = umma_smem_desc_sw128(ring + kLrZBox);
+    constexpr uint32_t kStageStep = kLrStageBytes >> 4;      // descriptors step in 16-byte units
+    auto next_stage = [&] {
+      umma_commit(lead, smem_u32(&ctl->empty[st]));
+      if (++st == kLrStages) { st = 0; phase ^= 1u; }
+    };
+    for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
+      const LowRankItem w = lowrank_item(p, item);
+      const uint32_t idesc = umma_idesc_bf16(kBlockM, w.width);
+      for (int pr = 0; pr < npairs && ok; ++pr, ++use) {
+        const uint32_t slot = use % kSlots;
+        if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + slot * 2 * kLrCols;
+        const int count = min(2, p.r - 2 * pr);
+        if (p.k == 16) {                                     // one entry: [hi | lo] of two components, 16 adaptor columns each
+          if (!bounded_wait_all(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t d_tmem = tmem_base + slot * 2 * kLrCols;
-          const int count = min(2, p.r - 2 * pr);
-          if (p.k == 16) {                                     // one entry: [hi | lo] of two components, 16 adaptor columns each
-            if (!bounded_wait(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
+          const uint64_t z = z_desc0 + st * kStageStep, a = a_desc0 + st * kStageStep;
+          const uint32_t z1 = count == 2 ? 4u : 0u, a1 = count == 2 ? 2u : 0u;
+#pragma unroll
+          for (int part = 0; part < 2; ++part) {             // (the two alternate: an MMA does not follow the one whose result it adds to)
+            umma_bf16(lead, d_tmem, z + 2 * part, a, idesc, part);
+            umma_bf16(lead, d_tmem + kLrCols, z + z1 + 2 * part, a + a1, idesc, part);
+          }
+          next_stage();
+        } else {                                             // an entry per component: hi at 0, lo at 32 of its 64 values
+          for (int q = 0; q < count && ok; ++q) {
+            if (!bounded_wait_all(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
             tc_fence_after();
             const uint64_t z = z_desc0 + st * kStageStep, a = a_desc0 + st * kStageStep;
-            for (int part = 0; part < 2; ++part)               // (the two alternate: an MMA does not follow the one whose result it adds to)
-              for (int q = 0; q < 2; ++q)
-                umma_bf16(d_tmem + q * kLrCols, z + (q < count ? 4 * q : 0) + 2 * part, a + (q < count ? 2 * q : 0), idesc, part);
-            next_stage();
-          } else {                                             // an entry per component: hi at 0, lo at 32 of its 64 values
-            for (int q = 0; q < count && ok; ++q) {
-              if (!bounded_wait(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
-              tc_fence_after();
-              const uint64_t z = z_desc0 + st * kStageStep, a = a_desc0 + st * kStageStep;
-              for (int kk = 0; kk < 4; ++kk) umma_bf16(d_tmem + q * kLrCols, z + 2 * kk, a + 2 * (kk & 1), idesc, kk != 0 ? 1u : 0u);
-              for (int kk = 0; kk < 4 && count == 1; ++kk)
-                umma_bf16(d_tmem + kLrCols, z + 2 * kk, a + 2 * (kk & 1), idesc, kk != 0 ? 1u : 0u);
-              next_stage();
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) umma_bf16(lead, d_tmem + q * kLrCols, z + 2 * kk, a + 2 * (kk & 1), idesc, kk != 0 ? 1u : 0u);
+            if (count == 1) {
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk) umma_bf16(lead, d_tmem + kLrCols, z + 2 * kk, a + 2 * (kk & 1), idesc, kk != 0 ? 1u : 0u);
             }
+            next_stage();
           }
-          if (!ok) break;
-          umma_commit(smem_u32(&ctl->tfull[slot]));
         }
+        if (!ok) break;
+        umma_commit(lead, smem_u32(&ctl->tfull[slot]));
       }
-      if (!ok || ctl->abort) {   // wait (bounded) for the MMAs already issued before tensor memory is freed
-        umma_commit(smem_u32(&ctl->drain));
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(smem_u32(&ctl->drain), 0) && global_timer_ns() - t0 < kWaitLimitNs) {}
-      }
+    }
+    if (!ok || __any_sync(kFull, ctl->abort)) {   // wait (bounded) for the MMAs already issued before tensor memory is freed
+      umma_commit(lead, smem_u32(&ctl->drain));
+      drain_wait(smem_u32(&ctl->drain), 0);
     }
     __syncwarp();
   } else {
@@ -833,7 +830,7 @@ __global__ void __launch_bounds__(32 * kDrawWarps) lowrank_slot_logits_kernel(
 // y's accumulators (two, of k columns) leave at the end of each 128 positions, dA's (two sets of up to four tiles of 128 symbols) at
 // the end of the unit. z: the bf16 high half the forward pass left, k of the 64 columns that a box brings in. Bound by the bytes
 // of g: 2 T n r v. Two batched GEMMs, each reading g, took 505 us at 8192 positions of 8 x 32 units of 320 symbols,
-// k = 16; this takes 281, for 205 us of bytes (the second round of units leaves a quarter of the SMs idle; equal runs of tiles over
+// k = 16; this takes 237 (280 while a branch of lane 0's own issued the sixteen small MMAs of a stage), for 205 us of bytes (the second round of units leaves a quarter of the SMs idle; equal runs of tiles over
 // all units, which do not, took 353: CTAs at the same positions of neighbouring units read whole rows of g between them). Units of
 // more than 512 symbols, or too few units to occupy the device, keep those products.
 struct AdaptorGradParams {
@@ -860,7 +857,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) adaptor_grad_kernel(const __g
   const uint32_t tiles_addr = (raw_addr + 1023u) & ~1023u;
   const uint32_t z_addr = tiles_addr + p.stages * kAdaptorStage, a_addr = z_addr + 2 * kAdaptorBox;
   GemmControl* ctl = reinterpret_cast<GemmControl*>(smem_raw + (a_addr - raw_addr) + static_cast<size_t>(p.v64) * 128);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = static_cast<int>(warp_uniform(threadIdx.x >> 5)), lane = threadIdx.x & 31;
   const int t_tiles = (p.T + kBlockM - 1) / kBlockM, pairs = (p.v64 + 127) / 128;
 
   if (threadIdx.x == 0) {
@@ -887,101 +884,100 @@ __global__ void __launch_bounds__(kGemmThreads, 1) adaptor_grad_kernel(const __g
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = ctl->tmem_base;
+  const uint32_t tmem_base = warp_uniform(ctl->tmem_base);
   grid_dependency_wait();
   grid_launch_dependents();
   // tensor memory: y at columns 0 and 32, dA's tiles at 64 and 192, 32 columns each
   auto da_col = [&](uint32_t set, int tile) { return 64 + set * 128 + tile * 32; };
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0, tc = 0, uc = 0;
-      bool ok = true;
-      auto issued = [&](uint32_t bar, uint32_t par) {
-        issued_mask |= 1u << bar;
-        phase_mask = (phase_mask & ~(1u << bar)) | (par << bar);
-      };
-      for (int unit = blockIdx.x; unit < p.units && ok; unit += gridDim.x, ++uc) {
-        bool a_loaded = false;
-        for (int t = 0; t < t_tiles && ok; ++t, ++tc) {
-          const uint32_t zbuf = tc & 1u;
-          for (int q = 0; q < pairs; ++q) {
-            if (!bounded_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
-            if (q == 0 && !bounded_wait(smem_u32(&ctl->empty[kAdaptorBarZ + zbuf]), ((tc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
-            const int boxes = q * 128 + 64 < p.v64 ? 2 : 1;
-            const uint32_t full = smem_u32(&ctl->full[stage]), dst = tiles_addr + stage * kAdaptorStage;
-            mbar_arrive_expect_tx(full, (boxes + (q == 0 ? 1 : 0)) * kAdaptorBox);
-            for (int b = 0; b < boxes; ++b) tma_load_2d(dst + b * kAdaptorBox, &p.tm_g, full, unit * p.v + q * 128 + b * 64, t * kBlockM);
-            if (q == 0) tma_load_2d(z_addr + zbuf * kAdaptorBox, &p.tm_z, full, unit * 2 * p.k, t * kBlockM);
-            issued(stage, phase);
-            if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
-            // A_u goes into the buffer that the unit before it has finished with: asked for behind the unit's first stage, so that
-            // the wait does not keep g from being fetched
-            if (!a_loaded) {
-              a_loaded = true;
-              if (!bounded_wait(smem_u32(&ctl->empty[kAdaptorBarA]), (uc & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
-              const uint32_t afull = smem_u32(&ctl->full[kAdaptorBarA]);
-              mbar_arrive_expect_tx(afull, p.v64 * 128);
-              for (int b = 0; b < p.v64; b += 64) tma_load_2d(a_addr + b * 128, &p.tm_a, afull, 0, unit * p.v64 + b);
-              issued(kAdaptorBarA, uc & 1u);
-            }
+    const uint32_t lead = elect_one();
+    uint32_t stage = 0, phase = 0, issued_mask = 0, phase_mask = 0, tc = 0, uc = 0;
+    bool ok = true;
+    auto issued = [&](uint32_t bar, uint32_t par) {
+      issued_mask |= 1u << bar;
+      phase_mask = (phase_mask & ~(1u << bar)) | (par << bar);
+    };
+    for (int unit = blockIdx.x; unit < p.units && ok; unit += gridDim.x, ++uc) {
+      bool a_loaded = false;
+      for (int t = 0; t < t_tiles && ok; ++t, ++tc) {
+        const uint32_t zbuf = tc & 1u;
+        for (int q = 0; q < pairs; ++q) {
+          if (!bounded_wait_all(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
+          if (q == 0 && !bounded_wait_all(smem_u32(&ctl->empty[kAdaptorBarZ + zbuf]), ((tc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+          const bool two = q * 128 + 64 < p.v64;
+          const uint32_t full = smem_u32(&ctl->full[stage]), dst = tiles_addr + stage * kAdaptorStage;
+          mbar_arrive_expect_tx(lead, full, ((two ? 2 : 1) + (q == 0 ? 1 : 0)) * kAdaptorBox);
+          tma_load_2d(lead, dst, &p.tm_g, full, unit * p.v + q * 128, t * kBlockM);
+          if (two) tma_load_2d(lead, dst + kAdaptorBox, &p.tm_g, full, unit * p.v + q * 128 + 64, t * kBlockM);
+          if (q == 0) tma_load_2d(lead, z_addr + zbuf * kAdaptorBox, &p.tm_z, full, unit * 2 * p.k, t * kBlockM);
+          issued(stage, phase);
+          if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
+          // A_u goes into the buffer that the unit before it has finished with: asked for behind the unit's first stage, so that
+          // the wait does not keep g from being fetched
+          if (!a_loaded) {
+            a_loaded = true;
+            if (!bounded_wait_all(smem_u32(&ctl->empty[kAdaptorBarA]), (uc & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+            const uint32_t afull = smem_u32(&ctl->full[kAdaptorBarA]);
+            mbar_arrive_expect_tx(lead, afull, p.v64 * 128);
+            for (int b = 0; b < p.v64; b += 64) tma_load_2d(lead, a_addr + b * 128, &p.tm_a, afull, 0, unit * p.v64 + b);
+            issued(kAdaptorBarA, uc & 1u);
           }
         }
       }
-      // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
-      for (int s = 0; s < kMaxStages; ++s)
-        if (issued_mask & (1u << s)) {
-          const uint64_t t0 = global_timer_ns();
-          while (!mbar_try_wait(smem_u32(&ctl->full[s]), (phase_mask >> s) & 1u) && global_timer_ns() - t0 < kWaitLimitNs) {}
-        }
     }
+    // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
+    for (int s = 0; s < kMaxStages; ++s)
+      if (issued_mask & (1u << s)) drain_wait(smem_u32(&ctl->full[s]), (phase_mask >> s) & 1u);
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, tc = 0, uc = 0;
-      bool ok = true;
-      const uint32_t idesc_y = umma_idesc_bf16(kBlockM, p.k, false, true), idesc_da = umma_idesc_bf16(kBlockM, p.k, true, true);
-      for (int unit = blockIdx.x; unit < p.units && ok; unit += gridDim.x, ++uc) {
-        const uint32_t set = uc & 1u;
-        if (!bounded_wait(smem_u32(&ctl->tempty[2 + set]), ((uc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
-        if (!bounded_wait(smem_u32(&ctl->full[kAdaptorBarA]), uc & 1u, ctl, p.status)) { ok = false; break; }
-        for (int t = 0; t < t_tiles && ok; ++t, ++tc) {
-          const uint32_t yslot = tc & 1u;
-          if (!bounded_wait(smem_u32(&ctl->tempty[yslot]), ((tc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
-          const uint64_t z_desc = umma_smem_desc_mn_sw128(z_addr + yslot * kAdaptorBox, kAdaptorBox);
-          for (int q = 0; q < pairs; ++q) {
-            if (!bounded_wait(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t g_addr = tiles_addr + stage * kAdaptorStage;
-            const int boxes = q * 128 + 64 < p.v64 ? 2 : 1;
-            for (int b = 0; b < boxes; ++b) {
-              const uint64_t g_desc = umma_smem_desc_sw128(g_addr + b * kAdaptorBox);
-              const uint64_t a_desc = umma_smem_desc_mn_sw128(a_addr + (2 * q + b) * kMnBoxBytes, kMnBoxBytes);
+    const uint32_t lead = elect_one();
+    uint32_t stage = 0, phase = 0, tc = 0, uc = 0;
+    bool ok = true;
+    const uint32_t idesc_y = umma_idesc_bf16(kBlockM, p.k, false, true), idesc_da = umma_idesc_bf16(kBlockM, p.k, true, true);
+    const uint64_t g_desc0 = umma_smem_desc_sw128(tiles_addr), gt_desc0 = umma_smem_desc_mn_sw128(tiles_addr, kAdaptorBox);
+    const uint64_t z_desc0 = umma_smem_desc_mn_sw128(z_addr, kAdaptorBox), a_desc0 = umma_smem_desc_mn_sw128(a_addr, kMnBoxBytes);
+    for (int unit = blockIdx.x; unit < p.units && ok; unit += gridDim.x, ++uc) {
+      const uint32_t set = uc & 1u;
+      if (!bounded_wait_all(smem_u32(&ctl->tempty[2 + set]), ((uc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+      if (!bounded_wait_all(smem_u32(&ctl->full[kAdaptorBarA]), uc & 1u, ctl, p.status)) { ok = false; break; }
+      for (int t = 0; t < t_tiles && ok; ++t, ++tc) {
+        const uint32_t yslot = tc & 1u;
+        if (!bounded_wait_all(smem_u32(&ctl->tempty[yslot]), ((tc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+        const uint64_t z_desc = z_desc0 + yslot * (kAdaptorBox >> 4);
+        const uint32_t y_tmem = tmem_base + yslot * 32;
+        for (int q = 0; q < pairs; ++q) {
+          if (!bounded_wait_all(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t at = stage * (kAdaptorStage >> 4);
+          const bool two = q * 128 + 64 < p.v64;
+          const uint64_t g_desc = g_desc0 + at, gt_desc = gt_desc0 + at, a_desc = a_desc0 + q * (2 * kMnBoxBytes >> 4);
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)                 // 16 symbols: 32 bytes along g's rows, 16 rows down A_u's box
-                umma_bf16(tmem_base + yslot * 32, g_desc + 2 * kk, a_desc + 128 * kk, idesc_y, (q | b | kk) != 0 ? 1u : 0u);
-            }
-            // the second box of an odd number is whatever the stage held before: rows past the unit's symbols, never read
-            const uint64_t gt_desc = umma_smem_desc_mn_sw128(g_addr, kAdaptorBox);
+          for (int kk = 0; kk < 4; ++kk)                     // 16 symbols: 32 bytes along g's rows, 16 rows down A_u's box
+            umma_bf16(lead, y_tmem, g_desc + 2 * kk, a_desc + 128 * kk, idesc_y, (q | kk) != 0 ? 1u : 0u);
+          if (two) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk)                   // 16 positions: 16 rows down both
-              umma_bf16(tmem_base + da_col(set, q), gt_desc + 128 * kk, z_desc + 128 * kk, idesc_da, (t | kk) != 0 ? 1u : 0u);
-            umma_commit(smem_u32(&ctl->empty[stage]));
-            if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
+            for (int kk = 0; kk < 4; ++kk)
+              umma_bf16(lead, y_tmem, g_desc + (kAdaptorBox >> 4) + 2 * kk, a_desc + (kMnBoxBytes >> 4) + 128 * kk, idesc_y, 1u);
           }
-          if (!ok) break;
-          umma_commit(smem_u32(&ctl->tfull[yslot]));
-          umma_commit(smem_u32(&ctl->empty[kAdaptorBarZ + yslot]));
+          // the second box of an odd number is whatever the stage held before: rows past the unit's symbols, never read
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk)                     // 16 positions: 16 rows down both
+            umma_bf16(lead, tmem_base + da_col(set, q), gt_desc + 128 * kk, z_desc + 128 * kk, idesc_da, (t | kk) != 0 ? 1u : 0u);
+          umma_commit(lead, smem_u32(&ctl->empty[stage]));
+          if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        umma_commit(smem_u32(&ctl->tfull[2 + set]));
-        umma_commit(smem_u32(&ctl->empty[kAdaptorBarA]));
+        umma_commit(lead, smem_u32(&ctl->tfull[yslot]));
+        umma_commit(lead, smem_u32(&ctl->empty[kAdaptorBarZ + yslot]));
       }
-      if (!ok) {
-        umma_commit(smem_u32(&ctl->drain));
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(smem_u32(&ctl->drain), 0) && global_timer_ns() - t0 < kWaitLimitNs) {}
-      }
+      if (!ok) break;
+      umma_commit(lead, smem_u32(&ctl->tfull[2 + set]));
+      umma_commit(lead, smem_u32(&ctl->empty[kAdaptorBarA]));
+    }
+    if (!ok) {
+      umma_commit(lead, smem_u32(&ctl->drain));
+      drain_wait(smem_u32(&ctl->drain), 0);
     }
     __syncwarp();
   } else {

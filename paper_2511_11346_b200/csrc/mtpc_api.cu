@@ -632,19 +632,19 @@ int resident_clusters(K kernel, int size, int which, int dev) {
 }
 
 // Rows per tile of the few-position draft path: the height in [64, 128] (multiple of 8) with which the longest of `ctas` persistent
-// CTAs has the fewest rows, emission and sum-unit tiles dealt evenly together, a pass of up to kDecodeMaxTiles tiles counted as 8 rows
-// more (its copy of the hidden states); ties go to the taller tile. (By the emission rows alone, a tree head of n = 8, r = 32,
-// v = 256 got 5 tiles of 112 rows on its longest CTA where the mean is 485 rows, 4 of 128 now: a decode step of 27 positions
-// 103.7 -> 100.4 us; a contextual head of n = 16, r = 32, v = 320, d = 2048, 115 positions: 283.6 -> 268.3.)
+// CTAs has the fewest rows, emission and sum-unit tiles dealt evenly together, a tile counted as 3 rows more and as one for every six
+// positions the head may draft at once (its copies of their hidden states); ties go to the taller tile. (By the emission rows alone, a tree
+// head of n = 8, r = 32, v = 256 got 5 tiles of 112 rows on its longest CTA where the mean is 485 rows, 4 of 128 now. 3 or 24 rows a tile whatever
+// the positions, us: tree 16 x 32 x 256, 8 positions 154.1 / 155.8, 128 positions 209.9 / 206.6; tree 16 x 32 x 272, 8 positions 118.4 / 119.8.)
 long long decode_tiles(long long rows, int sum_rows, int tr) {
   return (rows + tr - 1) / tr + (sum_rows + tr / 32 * 32 - 1) / (tr / 32 * 32);
 }
-int decode_tile_rows(long long rows, int sum_rows, int ctas) {
+int decode_tile_rows(long long rows, int sum_rows, int positions, int ctas) {
   int best = 128;
   long long best_cost = -1;
   for (int tr = 128; tr >= 64; tr -= 8) {
     const long long per_cta = (decode_tiles(rows, sum_rows, tr) + ctas - 1) / ctas;
-    const long long cost = per_cta * tr + 8 * ((per_cta + kDecodeMaxTiles - 1) / kDecodeMaxTiles);
+    const long long cost = per_cta * (tr + 3 + positions / 6);
     if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = tr; }
   }
   return best;
@@ -653,8 +653,8 @@ int decode_tile_rows(long long rows, int sum_rows, int ctas) {
 // resident at once (max_clusters: a size does not pack the SMs of every GPC, so fours cover less of the chip than twos) and
 // every CTA keeps at least four K blocks. A CTA's time goes as its K steps x (rows it fetches per step + a fixed part worth
 // about 32 rows) and the exchange of a cluster costs about 40 steps' worth of a row.
-void choose_decode_tiling(long long rows, int sum_rows, int kblocks, int ctas, const int (&max_clusters)[3], int* tile_rows, int* ksplit) {
-  *tile_rows = decode_tile_rows(rows, sum_rows, ctas);
+void choose_decode_tiling(long long rows, int sum_rows, int positions, int kblocks, int ctas, const int (&max_clusters)[3], int* tile_rows, int* ksplit) {
+  *tile_rows = decode_tile_rows(rows, sum_rows, positions, ctas);
   *ksplit = 1;
   const long long per_cta = (decode_tiles(rows, sum_rows, *tile_rows) + ctas - 1) / ctas;
   long long best = kblocks * (per_cta * *tile_rows + 48);
@@ -668,7 +668,6 @@ void choose_decode_tiling(long long rows, int sum_rows, int kblocks, int ctas, c
   }
 }
 
-constexpr int kDecodeShortRing = 205000;         // bytes of the weight pass's ring on long runs (see launch_decode_gemm)
 // Few-position draft path: one pass over all weight rows with the positions on the N axis.
 int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_t st) {
   const mtpc_config& c = h->cfg;
@@ -702,37 +701,20 @@ int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_
   p.emit2_tiles = (p.emit2_rows + p.tile_rows - 1) / p.tile_rows;
   p.sum_tiles = (p.sum_rows + p.sum_tile_rows - 1) / p.sum_tile_rows;
   p.tile_stride = (p.Ppad + 31) / 32 * 32;
-  p.pass_tiles = kTmemCols / (2 * p.tile_stride);                     // two slots of pass_tiles accumulators
-  if (p.pass_tiles > kDecodeMaxTiles) p.pass_tiles = kDecodeMaxTiles;
   const int tiles = p.emit_tiles + p.emit2_tiles + p.sum_tiles;
-  const int per_cta = (tiles + h->num_sms - 1) / h->num_sms;         // no wider stages than a CTA has tiles
-  // A long run of tiles and few positions (what a stage holds is then nearly all weights). (1) Passes of two tiles where they come out even and
-  // passes of three would end with a pass of one, whose stages are two thirds empty; not with a short K, where more passes cost their starts.
-  // (2) A ring of at most 205 KB: with more bytes in flight the same pass is slower. (Why was not found; it is not the room left to the next
-  // kernel, the pass alone shows it. 154 KB are as slow as 230.) Drafts + acceptance of 1 / 8 / 16 / 32 positions, three tiles and
-  // a full ring / so, in us:
-  //   HMM 16 x 32 x 320 (10 tiles of 112 rows a CTA), d = 4096: 236 242 248 254 / 222 231 238 250; d = 2048: 134 138 145 149.5 / 129 133 142 149.7
-  //   mixture 16 x 64 x 320 (31 of 72), d = 2048: 232 243 253 / 222 230 242, but 32 positions 253 / 256: left as it was from 17 on
-  //   tree 16 x 32 x 256 (9 of 112), d = 3072: 158 163 165 / 156 160 162; contextual HMM 16 x 32 x 256: 170 174 184 / 169 172 180
-  //   16 x 32 x 272 (8 of 120, 11 of 96), 16 x 32 x 256 (7 of 128): the same ring, the same times
-  // Two tiles a pass regardless of what is left over: tree 16 x 32 x 272 125 -> 129, HMM 16 x 32 x 272 115 -> 117; with 10 tiles but d = 1024
-  // 100 -> 101.5 at 32 positions.
-  const bool long_run = per_cta >= 7 && p.Ppad <= 32;
-  const bool by_twos = long_run && p.pass_tiles > 2 && per_cta % 6 == 4 && p.kblocks >= 32;
-  const bool short_ring = by_twos || (long_run && p.Ppad <= 16);
-  if (by_twos) p.pass_tiles = 2;
-  const int passes = (per_cta + p.pass_tiles - 1) / p.pass_tiles;
-  p.pass_tiles = (per_cta + passes - 1) / passes;                     // passes of one length keep as many bytes in flight throughout
   p.ksplit = h->decode_ksplit;
-  while (p.ksplit > 1 && decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad) > 64 * 1024) p.ksplit /= 2;
-  // stage = weight tiles + hidden tile, padded so that a 128-row operand read from the last tile's base stays inside
-  int stage = p.pass_tiles * p.tile_bytes + p.Ppad * kBlockK * 2;
-  const int reach = (p.pass_tiles - 1) * p.tile_bytes + kABytes;
-  if (stage < reach) stage = reach;
+  while (p.ksplit > 1 && decode_exchange_bytes(p.ksplit, p.Ppad) > 64 * 1024) p.ksplit /= 2;
+  // stage = weight tile + hidden tile, padded so that a 128-row operand read from the tile's base stays inside
+  int stage = p.tile_bytes + p.Ppad * kBlockK * 2;
+  if (stage < static_cast<int>(kABytes)) stage = kABytes;
   p.stage_bytes = (stage + 1023) / 1024 * 1024;
-  const int ctl = 1024 + static_cast<int>(sizeof(GemmControl)) + static_cast<int>(decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad));
-  p.stages = (short_ring ? min(kSmemLimit - ctl, kDecodeShortRing) : kSmemLimit - ctl) / p.stage_bytes;
-  if (p.stages > kMaxStages) p.stages = kMaxStages;
+  const int ctl = 1024 + static_cast<int>(sizeof(GemmControl)) + static_cast<int>(decode_exchange_bytes(p.ksplit, p.Ppad));
+  p.stages = (kSmemLimit - ctl) / p.stage_bytes;
+  // At most nine stages, 144 KB up to 16 positions: with more of them, or fewer, the same pass is slower (why was not found). Drafts +
+  // acceptance with 7 / 8 / 9 / 10 stages, us: HMM 16 x 32 x 320, d = 4096, 1 position 215.0 213.4 211.4 213.3, 8 227.2 225.5 223.4 225.6;
+  // mixture 8 x 16 x 320, 1 position 64.4 64.4 62.6 63.5; 16 x 16 x 320, 64 positions 139.3 138.8 138.3 139.2; tree 8 x 32 x 256, 27 positions
+  // 89.7 90.0 88.2 89.4; with 12 and 13 stages the HMM's 8 positions take 230.2 and 231.3.
+  if (p.stages > kDecodeMaxStages) p.stages = kDecodeMaxStages;
   p.logw = at<float>(h, L.off_logw);
   p.sum_bias = sum_bias(h);
   p.status = at<unsigned>(h, L.off_status);
@@ -1602,7 +1584,7 @@ static int bind_parameters(mtpc_head* h, const void* W_emit, const void* W_sum, 
   if (rc == MTPC_OK && dense) rc = make_tmap(&h->tm_emit_lp2, h->W_emit_bf16, emit_rows, cfg->d, L.lp.tile_cols / 2);
   if (rc == MTPC_OK) rc = make_tmap(&h->tm_sum2, h->W_sum_bf16, L.sum_rows, cfg->d, L.sum_cols / 2);
   const uint64_t base_rows = static_cast<uint64_t>(cfg->n) * cfg->v, adapt_rows = static_cast<uint64_t>(cfg->n) * cfg->r * h->lr_k;
-  choose_decode_tiling(static_cast<long long>(dense ? emit_rows : base_rows + adapt_rows), L.sum_rows, cfg->d / kBlockK, h->num_sms,
+  choose_decode_tiling(static_cast<long long>(dense ? emit_rows : base_rows + adapt_rows), L.sum_rows, L.decode_max_p, cfg->d / kBlockK, h->num_sms,
                        h->max_decode_clusters, &h->decode_tile_rows, &h->decode_ksplit);
   if (rc == MTPC_OK && dense) rc = make_tmap(&h->tm_emit_dec, h->W_emit_bf16, emit_rows, cfg->d, h->decode_tile_rows);
   if (rc == MTPC_OK && !dense) rc = make_tmap(&h->tm_emit_dec, h->lr_W_base, base_rows, cfg->d, h->decode_tile_rows);

@@ -12,9 +12,7 @@
 //                             are, and the kernels that follow normalise them where they need to.
 //                             Weight rows are cut into tiles of `tile_rows` <= 128 rows, chosen by the host so that
 //                             the tiles divide evenly over the persistent CTAs; each CTA takes a contiguous run
-//                             of tiles and walks K once per pass of up to three tiles, which share one copy of
-//                             the hidden-state block, so the bytes in flight per SM stay high and the hidden
-//                             states cross L2 once per pass instead of once per tile.
+//                             of tiles and walks K once per tile.
 //   draft_slot_kernel         one CTA per (position, window slot i): log-sum-exp of the r input units of the
 //                             slot, then per window (one warp each): latent draws down to the unit that owns
 //                             slot i, the byte by inverse CDF of that unit's categorical, and the evidence
@@ -26,10 +24,7 @@
 namespace mtpc {
 
 constexpr int kDecodeMaxP = 128;                   // positions per call on this path
-#ifndef MTPC_DECODE_MAX_TILES
-#define MTPC_DECODE_MAX_TILES 3
-#endif
-constexpr int kDecodeMaxTiles = MTPC_DECODE_MAX_TILES;   // weight tiles that share one copy of the hidden states
+constexpr int kDecodeMaxStages = 9;                // of the weight pass's ring (see launch_decode_gemm)
 constexpr int kSlotThreads = 512;
 
 struct DecodeParams {
@@ -45,7 +40,6 @@ struct DecodeParams {
   int sum_tile_rows;             // rows of a sum tile (a multiple of 32, <= tile_rows rounded up to 32)
   int tile_bytes;                // shared-memory pitch of a weight tile
   int emit_tiles, sum_tiles;
-  int pass_tiles;                // tiles per pass (<= kDecodeMaxTiles)
   int tile_stride;               // TMEM columns per tile
   int stages, stage_bytes;
   int ksplit;                    // CTAs of a cluster that share a run of tiles, each with its part of K (1: no cluster)
@@ -74,19 +68,17 @@ __device__ __forceinline__ DecodeTile decode_tile(const DecodeParams& p, int t) 
 // took 650 cycles a K step and tile, more than the step's bytes where a CTA has one tile (draft + acceptance of 8 positions of a factored
 // head, d = 4096: 32.7 -> 27.0 us; 4 x 8 x 256, d = 1024, 16 positions: 20.0 -> 17.4) and nearly as much where it has three (mixture
 // 8 x 16 x 320, 1 position 65.7 -> 63.6, HMM 16 x 32 x 320, 8 positions 225.7 -> 221.5; 128 positions of the mixture 96.7 -> 89.3).
-// A CTA walks its run of tiles in passes of up to pass_tiles tiles (of either matrix). Shared-memory stage:
-// pass_tiles weight tiles at a pitch of tile_bytes (the MMA reads 128 rows from each tile's base: what lies beyond
-// the tile's own rows is other data, and the TMEM lanes it produces are never read), then the hidden tile
-// (Ppad rows x 128 bytes) followed by slack so that the last tile's 128-row read stays inside the stage.
-// Tensor memory: two slots of pass_tiles * tile_stride columns.
+// A CTA walks its run of tiles one after the other. Shared-memory stage: the weight tile (the MMA reads 128 rows from its base: what
+// lies beyond the tile's own rows is other data, and the TMEM lanes it produces are never read), then the hidden tile
+// (Ppad rows x 128 bytes) followed by slack so that the 128-row read stays inside the stage. Tensor memory: two slots of tile_stride columns.
 // ksplit > 1: where the tiles leave most SMs idle (a factored head's 4600 rows are 72 tiles) a cluster of ksplit CTAs takes a
 // tile, each walking its part of K; the others hand their fp32 accumulators to the first one through its shared memory (behind
-// the ring: [rank - 1][tile][position quad][128 rows] of float4), which adds them in rank order and runs the epilogue.
-// Every CTA then has one pass. The pass over 39 MB of weights (n = 8, r = 16, v = 320, d = 4096, rank 16) took 30 us as 72 CTAs
+// the ring: [rank - 1][position quad][128 rows] of float4), which adds them in rank order and runs the epilogue.
+// Every CTA then has one tile. The pass over 39 MB of weights (n = 8, r = 16, v = 320, d = 4096, rank 16) took 30 us as 72 CTAs
 // of 64 K steps and half the SMs idle; draft + acceptance of 8 positions: 51 -> 38 us with clusters
 // of two.
-__host__ __device__ inline size_t decode_exchange_bytes(int ksplit, int pass_tiles, int Ppad) {
-  return static_cast<size_t>(ksplit - 1) * pass_tiles * kBlockM * Ppad * sizeof(float);
+__host__ __device__ inline size_t decode_exchange_bytes(int ksplit, int Ppad) {
+  return static_cast<size_t>(ksplit - 1) * kBlockM * Ppad * sizeof(float);
 }
 __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -94,7 +86,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
   const uint32_t tiles_addr = (raw_addr + 1023u) & ~1023u;
   uint8_t* tiles = smem_raw + (tiles_addr - raw_addr);
   uint8_t* exchange = tiles + static_cast<size_t>(p.stages) * p.stage_bytes;
-  GemmControl* ctl = reinterpret_cast<GemmControl*>(exchange + decode_exchange_bytes(p.ksplit, p.pass_tiles, p.Ppad));
+  GemmControl* ctl = reinterpret_cast<GemmControl*>(exchange + decode_exchange_bytes(p.ksplit, p.Ppad));
 
   const int warp = static_cast<int>(warp_uniform(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
@@ -104,8 +96,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
   const int tile_begin = static_cast<int>(static_cast<long long>(group) * total_tiles / groups);
   const int tile_end = static_cast<int>(static_cast<long long>(group + 1) * total_tiles / groups);
   const int kb0 = rank * p.kblocks / p.ksplit, kb1 = (rank + 1) * p.kblocks / p.ksplit;
-  const uint32_t hidden_off = p.pass_tiles * p.tile_bytes;
-  const uint32_t slot_cols = p.pass_tiles * p.tile_stride;
+  const uint32_t hidden_off = p.tile_bytes;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -157,7 +148,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
         for (int part = 0; part + 1 < p.ksplit; ++part) {
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            const float4 y = others[(part * p.pass_tiles * (p.Ppad / 4) + b * 4 + c) * kBlockM + local];
+            const float4 y = others[(part * (p.Ppad / 4) + b * 4 + c) * kBlockM + local];
             x[4 * c] += y.x;
             x[4 * c + 1] += y.y;
             x[4 * c + 2] += y.z;
@@ -202,30 +193,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
     uint32_t stage = 0, phase = 0, issued = 0;
     bool ok = true;
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-    for (int cur = tile_begin; cur < tile_end && ok;) {
-      const int ntiles = min(p.pass_tiles, tile_end - cur);
-      uint32_t bytes = p.Ppad * (kBlockK * 2);                   // out-of-range rows are zero-filled and counted
-      const CUtensorMap* map[kDecodeMaxTiles];
-      int row[kDecodeMaxTiles];
-#pragma unroll
-      for (int q = 0; q < kDecodeMaxTiles; ++q) {
-        const DecodeTile t = decode_tile(p, min(cur + q, tile_end - 1));
-        map[q] = t.is_sum ? &p.tm_sum : (t.second ? &p.tm_emit2 : &p.tm_emit);
-        row[q] = t.index * t.rows;
-        if (q < ntiles) bytes += t.rows * (kBlockK * 2);
-      }
+    for (int tile = tile_begin; tile < tile_end && ok; ++tile) {
+      const DecodeTile t = decode_tile(p, tile);
+      const CUtensorMap* map = t.is_sum ? &p.tm_sum : (t.second ? &p.tm_emit2 : &p.tm_emit);
+      const int row = t.index * t.rows;
+      const uint32_t bytes = (t.rows + p.Ppad) * (kBlockK * 2);    // out-of-range rows are zero-filled and counted
       for (int k = kb0 * kBlockK; k < kb1 * kBlockK; k += kBlockK) {
         if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
         const uint32_t full = full0 + 8 * stage, dst = tiles_addr + stage * p.stage_bytes;
         mbar_arrive_expect_tx(lead, full, bytes);
-#pragma unroll
-        for (int q = 0; q < kDecodeMaxTiles; ++q)
-          if (q < ntiles) tma_load_2d(lead, dst + q * p.tile_bytes, map[q], full, k, row[q]);
+        tma_load_2d(lead, dst, map, full, k, row);
         tma_load_2d(lead, dst + hidden_off, &p.tm_h, full, k, 0);
         ++issued;
         if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
       }
-      cur += ntiles;
     }
     // no copy may still be in flight when the CTA goes away (they have all landed unless some warp gave up)
     for (uint32_t s = 0; s < static_cast<uint32_t>(p.stages) && s < issued; ++s)
@@ -238,29 +219,23 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
     bool ok = true;
     const uint32_t idesc = umma_idesc_bf16(kBlockM, p.Ppad);
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-    const uint32_t stage_step = p.stage_bytes >> 4, tile_step = p.tile_bytes >> 4;          // descriptors step in 16-byte units
+    const uint32_t stage_step = p.stage_bytes >> 4;             // descriptors step in 16-byte units
     const uint64_t a_desc0 = umma_smem_desc_sw128(tiles_addr), b_desc0 = umma_smem_desc_sw128(tiles_addr + hidden_off);
-    for (int cur = tile_begin; cur < tile_end && ok; ++use) {
-      const int ntiles = min(p.pass_tiles, tile_end - cur);
-      cur += ntiles;
+    for (int tile = tile_begin; tile < tile_end && ok; ++tile, ++use) {
       const uint32_t slot = use & 1u;
       if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use >> 1) & 1u) ^ 1u, ctl, p.status)) {
         ok = false;
         break;
       }
       tc_fence_after();
-      const uint32_t d_tmem = tmem_base + slot * slot_cols;
+      const uint32_t d_tmem = tmem_base + slot * p.tile_stride;
       for (int kb = kb0; kb < kb1; ++kb) {
         if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
         tc_fence_after();
         const uint64_t a_desc = a_desc0 + stage * stage_step, b_desc = b_desc0 + stage * stage_step;
 #pragma unroll
-        for (int q = 0; q < kDecodeMaxTiles; ++q)
-          if (q < ntiles) {
-#pragma unroll
-            for (int kk = 0; kk < kBlockK / 16; ++kk)
-              umma_bf16(lead, d_tmem + q * p.tile_stride, a_desc + q * tile_step + 2 * kk, b_desc + 2 * kk, idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
-          }
+        for (int kk = 0; kk < kBlockK / 16; ++kk)
+          umma_bf16(lead, d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
         umma_commit(lead, empty0 + 8 * stage);
         if (++stage == static_cast<uint32_t>(p.stages)) { stage = 0; phase ^= 1u; }
       }
@@ -276,8 +251,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
     // ------------------------------------------------------------------ epilogue: warp q owns lanes 32q .. 32q+31
     uint32_t use = 0;
     bool ok = true;
-    for (int cur = tile_begin; cur < tile_end && ok; ++use) {
-      const int ntiles = min(p.pass_tiles, tile_end - cur);
+    for (int tile = tile_begin; tile < tile_end && ok; ++tile, ++use) {
       const uint32_t slot = use & 1u;
       if (!bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use >> 1) & 1u, ctl, p.status, lane)) {
         ok = false;
@@ -285,20 +259,18 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
       }
       tc_fence_after();
       if (p.ksplit == 1) {
-        for (int q = 0; q < ntiles; ++q) finish_tile(cur + q, slot * slot_cols + q * p.tile_stride, nullptr);
+        finish_tile(tile, slot * p.tile_stride, nullptr);
       } else if (rank > 0) {
-        // one pass: the accumulators go to the cluster's first CTA
+        // the cluster's one tile: the accumulators go to its first CTA
         const uint32_t dst0 = cluster_map_shared(smem_u32(exchange), 0) + (quarter * 32 + lane) * 16;
-        for (int q = 0; q < ntiles; ++q)
-          for (int b = 0; b < (p.P + 15) / 16; ++b) {
-            float x[16];
-            tmem_ld16(lane_base + q * p.tile_stride + b * 16, x);
-            const uint32_t dst = dst0 + (((rank - 1) * p.pass_tiles + q) * (p.Ppad / 4) + b * 4) * (kBlockM * 16);
+        for (int b = 0; b < (p.P + 15) / 16; ++b) {
+          float x[16];
+          tmem_ld16(lane_base + b * 16, x);
+          const uint32_t dst = dst0 + ((rank - 1) * (p.Ppad / 4) + b * 4) * (kBlockM * 16);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) st_cluster_v4(dst + c * (kBlockM * 16), x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
-          }
+          for (int c = 0; c < 4; ++c) st_cluster_v4(dst + c * (kBlockM * 16), x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+        }
       }
-      cur += ntiles;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&ctl->tempty[slot]));
@@ -311,8 +283,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
     cluster_sync_all();       // the other CTAs' accumulators have arrived
     if (rank == 0 && warp >= 2) {
       tc_fence_after();
-      for (int q = 0; q < tile_end - tile_begin; ++q)
-        finish_tile(tile_begin + q, q * p.tile_stride, reinterpret_cast<const float4*>(exchange) + q * (p.Ppad / 4) * kBlockM);
+      if (tile_begin < tile_end) finish_tile(tile_begin, 0, reinterpret_cast<const float4*>(exchange));
       tc_fence_before();
     }
     __syncthreads();

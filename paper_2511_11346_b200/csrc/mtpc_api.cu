@@ -541,12 +541,19 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
     launch_kernel(circuit_cp_kernel, blocks, threads, 0, st, overlapped(h), G, logw, out, W, wpp, c.n, c.r, L.sum_rows,
                   raw_mixture ? 1 : 0);
   } else if (c.family == MTPC_HMM) {
+    const int stride = hmm_table_stride(h);
+    const bool probabilities = stride == 0 && L.off_probA != 0;          // (a call without a head has log-probabilities alone)
+    // Windows (a warp each) of a CTA: eight; of few windows with static tables as few as spread them over the SMs, two at least: a step is 40 reads of shared
+    // memory a warp, which eight warps wait for in turn. Whole calls of a small head with eight / two, us: n = 16, r = 16, 120 positions
+    // 33.6 / 23.7, 250 44.5 / 35.2; n = 8, r = 32, 120 positions 26.3 / 20.7; drafts + acceptance of n = 16, r = 32, v = 272, 16 positions of 16
+    // windows 201.7 / 196.6. One a CTA: the same; two, and six warps that only help to copy tables, take longer. With r = 8 a step is too short to gain (n = 16, 250 positions 31.3 / 31.8).
+    int warps = kHmmWarps;
+    while (probabilities && c.r >= 16 && warps > 2 && (W + warps / 2 - 1) / (warps / 2) <= h->num_sms) warps /= 2;
     // as many tables as fit beside the warps' vectors (all of them but for very long windows)
     int chunk = c.n > 1 ? c.n - 1 : 1;
-    while (chunk > 1 && hmm_circuit_smem_floats(c.n, c.r, prefix != nullptr, chunk) * sizeof(float) > static_cast<size_t>(kSmemLimit)) --chunk;
-    const size_t smem = hmm_circuit_smem_floats(c.n, c.r, prefix != nullptr, chunk) * sizeof(float);
-    const int stride = hmm_table_stride(h);
-    const int items = stride == 0 ? (W + kHmmWarps - 1) / kHmmWarps : W / wpp * ((wpp + kHmmWarps - 1) / kHmmWarps);
+    while (chunk > 1 && hmm_circuit_smem_floats(c.n, c.r, prefix != nullptr, chunk, warps) * sizeof(float) > static_cast<size_t>(kSmemLimit)) --chunk;
+    const size_t smem = hmm_circuit_smem_floats(c.n, c.r, prefix != nullptr, chunk, warps) * sizeof(float);
+    const int items = stride == 0 ? (W + warps - 1) / warps : W / wpp * ((wpp + warps - 1) / warps);
     const int resident = sms_times_resident(h, smem);
     // contextual tables: a CTA per position while about one round of CTAs holds all positions, else a warp per window (both
     // measured at circuit_hmm_stream_kernel; the two cross between 1.0 and 1.6 rounds over n = 4 to 64, r = 8 to 32)
@@ -557,8 +564,7 @@ int launch_circuit(mtpc_head* h, int W, int wpp, float* out, float* prefix, cuda
       launch_kernel(circuit_hmm_stream_kernel, ctas < held ? ctas : held, kHmmStreamWarps * 32, stream_smem, st, overlapped(h), G, logw,
                     hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r, L.sum_rows);
     } else {
-      const bool probabilities = stride == 0 && L.off_probA != 0;        // (a call without a head has log-probabilities alone)
-      launch_kernel(circuit_hmm_kernel, items < resident ? items : resident, kHmmWarps * 32, smem, st, overlapped(h), G, logw,
+      launch_kernel(circuit_hmm_kernel, items < resident ? items : resident, warps * 32, smem, st, overlapped(h), G, logw,
                     probabilities ? at<float>(h, L.off_probA) : hmm_tables(h), stride, out, prefix, msg, W, wpp, c.n, c.r,
                     L.sum_rows, chunk, probabilities ? 1 : 0);
     }

@@ -625,13 +625,13 @@ __device__ __forceinline__ float hmm_forward_step(float alpha, float* ev, const 
 // memory round trip in it. Tables that do not fit (n = 64 at r = 32) go through in chunks of chunk_tables. The prefix log-sum-exps are taken at the
 // end, lane = slot. Measured against one warp per window streaming log tables: 8192 windows at n = 8, r = 32: 42 -> 22 us;
 // 128 windows at n = 16: 27 -> 13 us. Shared memory: hmm_circuit_smem_floats.
-constexpr int kHmmWarps = 8;
+constexpr int kHmmWarps = 8;                                         // at most: launch_circuit gives a CTA fewer where windows are few
 __host__ __device__ inline int hmm_circuit_warp_floats(int n, int r, bool with_prefix) {
   return 64 + (with_prefix ? (n * (r + 1) + 3) / 4 * 4 : 0);          // two vectors of 32, alphas [n][r + 1]
 }
-__host__ __device__ inline size_t hmm_circuit_smem_floats(int n, int r, bool with_prefix, int chunk_tables) {
+__host__ __device__ inline size_t hmm_circuit_smem_floats(int n, int r, bool with_prefix, int chunk_tables, int warps) {
   return (static_cast<size_t>(chunk_tables) * r * r + 3) / 4 * 4 +
-         static_cast<size_t>(kHmmWarps) * hmm_circuit_warp_floats(n, r, with_prefix);
+         static_cast<size_t>(warps) * hmm_circuit_warp_floats(n, r, with_prefix);
 }
 __global__ void __launch_bounds__(32 * kHmmWarps, 5) circuit_hmm_kernel(
     const float* __restrict__ G, const float* __restrict__ logw, const float* __restrict__ tables, int table_stride,
@@ -639,9 +639,10 @@ __global__ void __launch_bounds__(32 * kHmmWarps, 5) circuit_hmm_kernel(
     int chunk_tables, int probabilities) {
   extern __shared__ __align__(16) float sm[];
   grid_launch_dependents();
+  const int warps = blockDim.x >> 5;
   const bool early = probabilities && chunk_tables >= n - 1;           // a static set, complete before the call's first kernel lets this in
   if (early) {
-    fetch_floats(sm, tables, (n - 1) * r * r, 32 * kHmmWarps);
+    fetch_floats(sm, tables, (n - 1) * r * r, 32 * warps);
     cp_async_commit();
   }
   grid_dependency_wait();   // G and log omega come from the kernel before this one
@@ -658,19 +659,19 @@ __global__ void __launch_bounds__(32 * kHmmWarps, 5) circuit_hmm_kernel(
   const HmmLanes l = hmm_lanes(r, lane);
   const int k = l.k, part = l.part;
   const bool active = l.active;
-  // work items: kHmmWarps windows each; contextual tables: of one position
-  const int per_pos = table_stride == 0 ? 0 : (wpp + kHmmWarps - 1) / kHmmWarps;
-  const int items = table_stride == 0 ? (W + kHmmWarps - 1) / kHmmWarps : (W / wpp) * per_pos;
+  // work items: a window a warp; contextual tables: of one position
+  const int per_pos = table_stride == 0 ? 0 : (wpp + warps - 1) / warps;
+  const int items = table_stride == 0 ? (W + warps - 1) / warps : (W / wpp) * per_pos;
   int loaded_pos = early ? 0 : -1, loaded_first = loaded_pos;          // which tables E holds
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
     int pos_tab = 0, w;
     bool valid;
     if (table_stride == 0) {
-      w = item * kHmmWarps + wib;
+      w = item * warps + wib;
       valid = w < W;
     } else {
       pos_tab = item / per_pos;
-      const int j = (item - pos_tab * per_pos) * kHmmWarps + wib;
+      const int j = (item - pos_tab * per_pos) * warps + wib;
       w = pos_tab * wpp + j;
       valid = j < wpp;
     }
@@ -701,16 +702,16 @@ __global__ void __launch_bounds__(32 * kHmmWarps, 5) circuit_hmm_kernel(
         const float* src = tb + static_cast<size_t>(t0) * rr;
         const int count = nt * rr;
         if (probabilities) {
-          fetch_floats(E, src, count, 32 * kHmmWarps);
+          fetch_floats(E, src, count, 32 * warps);
           cp_async_commit();
           cp_async_wait<0>();
         } else if ((count & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
-          for (int e = threadIdx.x * 4; e < count; e += 32 * kHmmWarps * 4) {
+          for (int e = threadIdx.x * 4; e < count; e += 32 * warps * 4) {
             const float4 x = *reinterpret_cast<const float4*>(src + e);
             *reinterpret_cast<float4*>(E + e) = make_float4(__expf(x.x), __expf(x.y), __expf(x.z), __expf(x.w));
           }
         } else {
-          for (int e = threadIdx.x; e < count; e += 32 * kHmmWarps) E[e] = __expf(src[e]);
+          for (int e = threadIdx.x; e < count; e += 32 * warps) E[e] = __expf(src[e]);
         }
         __syncthreads();
         loaded_pos = pos_tab;

@@ -923,13 +923,17 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
       const size_t smem = (in_smem ? with_tables : base) + weights;
       const int weights_in_smem = c.v <= kMaxDraftVocab && 2 * wpp >= c.r &&
                                   (smem <= kSlotSmemPair || (smem <= kSlotSmemLimit && c.n * P <= h->num_sms));
-      // builds of the narrow kernel that unroll 4, 8, 10 or 16 batches of 32 symbols: the smallest that covers v
-      auto* slot_kernel = c.v > kMaxDraftVocab ? draft_slot_kernel<true, 16>
-                          : c.v <= 128 ? draft_slot_kernel<false, 4>
-                          : c.v <= 256 ? draft_slot_kernel<false, 8>
-                          : c.v <= 320 ? draft_slot_kernel<false, 10> : draft_slot_kernel<false, 16>;
-      launch_kernel(slot_kernel, dim3(c.n, P), kSlotThreads,
-                    weights_in_smem ? smem : smem - weights, st, overlapped(h), c.family,
+      // builds of the narrow kernel that unroll 4, 8, 10 or 16 batches of 32 symbols: the smallest that covers v; where a device full of
+      // CTAs is not all of them, and a third fits an SM's shared memory, the builds whose registers let it (see draft_slot_kernel; not of
+      // contextual tables, which come by L2 for every position: n = 16, r = 32, d = 2048, 115 positions 210.6 us with two, 212.4 with three)
+      const size_t slot_smem = weights_in_smem ? smem : smem - weights;
+      const bool crowd = !is_ctx(h) && c.n * P > 2 * h->num_sms && 3 * (slot_smem + 1024) <= static_cast<size_t>(kSmemLimit);
+      auto* slot_kernel = c.v > kMaxDraftVocab ? draft_slot_kernel<true, 16, 2>
+                          : c.v <= 128 ? (crowd ? draft_slot_kernel<false, 4, 3> : draft_slot_kernel<false, 4, 2>)
+                          : c.v <= 256 ? (crowd ? draft_slot_kernel<false, 8, 3> : draft_slot_kernel<false, 8, 2>)
+                          : c.v <= 320 ? (crowd ? draft_slot_kernel<false, 10, 3> : draft_slot_kernel<false, 10, 2>)
+                                       : draft_slot_kernel<false, 16, 2>;
+      launch_kernel(slot_kernel, dim3(c.n, P), kSlotThreads, slot_smem, st, overlapped(h), c.family,
                     at<float>(h, L.off_logits), at<float>(h, L.off_logw), is_ctx(h) ? hmm_tables(h) : at<float>(h, L.off_cdfA), uniforms, out_bytes,
                     at<float>(h, L.off_G), at<float>(h, L.off_unit_lse), at<unsigned>(h, L.off_status),
                     at<unsigned>(h, L.off_status) + kWorkCounterWord, wpp, c.n, c.r, c.v, valid_symbols(c), L.sum_rows,
@@ -1719,11 +1723,9 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
           cudaSuccess;
   for (int e = 0; e < 3; ++e) h->max_decode_clusters[e] = fail ? 0 : resident_clusters(mtpc_decode_gemm_kernel, 2 << e, 1 + e, dev);
   const int slot_smem = static_cast<int>(kSlotSmemLimit);
-  fail |= cudaFuncSetAttribute(draft_slot_kernel<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
-  fail |= cudaFuncSetAttribute(draft_slot_kernel<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
-  fail |= cudaFuncSetAttribute(draft_slot_kernel<false, 10>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
-  fail |= cudaFuncSetAttribute(draft_slot_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
-  fail |= cudaFuncSetAttribute(draft_slot_kernel<true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
+  for (auto* kernel : {draft_slot_kernel<false, 4, 2>, draft_slot_kernel<false, 8, 2>, draft_slot_kernel<false, 10, 2>, draft_slot_kernel<false, 16, 2>,
+                       draft_slot_kernel<false, 4, 3>, draft_slot_kernel<false, 8, 3>, draft_slot_kernel<false, 10, 3>, draft_slot_kernel<true, 16, 2>})
+    fail |= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
   fail |= !set_circuit_attributes();
   fail |= !allow_full_smem(spec_accept_kernel<true>) || !allow_full_smem(spec_accept_kernel<false>);
   fail |= cudaMemsetAsync(h->ws + L.off_status, 0, 256, st) != cudaSuccess;

@@ -493,8 +493,12 @@ __device__ __forceinline__ int warp_inv_cdf_chunk(const float* __restrict__ x, i
 // these durations fetching instructions counts. Time after the weight pass, per slot stage: mixture n = 16, r = 16, v = 320, 64
 // positions of 16 windows 22 -> 15.5 us; HMM n = 16, r = 32, 8 positions 16.2 -> 9.8; tree n = 8, r = 32, 27 positions 10.4 -> 8.
 // WIDE: vocabularies of more than 512 symbols (a separate build: the narrow one keeps a unit's logits in registers).
-template <bool WIDE, int NQ>   // NQ: batches of 32 symbols of a unit that are unrolled (v <= 32 NQ; WIDE: 16)
-__global__ void __launch_bounds__(kSlotThreads, 2) draft_slot_kernel(
+// CTAS: of them that an SM's registers hold. Two leave a warp everything in flight that it asks for; of more CTAs than the device then holds
+// three an SM take less time, a few values spilled (draft + acceptance, two / three, us: mixture 16 x 16 x 320, 64 positions of 16 windows
+// 137.1 / 134.4, 128 positions of one window, d = 1024, 71.9 / 67.4; tree 16 x 32 x 256, 128 positions 207.4 / 200.6), fewer CTAs more
+// (HMM 16 x 16 x 256, d = 512, 1 position of 16 windows 32.2 / 33.7, tree 8 x 32 x 256, 27 positions 88.4 / 89.6).
+template <bool WIDE, int NQ, int CTAS>   // NQ: batches of 32 symbols of a unit that are unrolled (v <= 32 NQ; WIDE: 16)
+__global__ void __launch_bounds__(kSlotThreads, CTAS) draft_slot_kernel(
     int family, const float* __restrict__ logits, const float* __restrict__ logw, const float* __restrict__ hmm_tables,
     const float* __restrict__ uniforms, int* __restrict__ out_bytes, float* __restrict__ G,
     float* __restrict__ unit_lse_out, unsigned* status, unsigned* work_counter, int wpp, int n, int r, int v, int vv,

@@ -1,5 +1,6 @@
-"""Launch shapes that depend on how many windows a call has: the HMM's circuit gives a CTA eight windows, or four or two where they are few.
-A window's arithmetic does not depend on it, so its results are bit for bit those that it has in a call of another size."""
+"""Launch shapes that depend on how many windows a call has: the HMM's circuit gives a CTA eight windows, or four or two where they are few, and
+the per-slot draws of many (position, slot) pairs take a build of which three CTAs share an SM. A window's arithmetic does not depend on
+either, so its results are bit for bit those that it has in a call of another size."""
 import pytest
 import torch
 
@@ -41,3 +42,23 @@ def test_windows_per_cta(n, r):
         joint, prefix = run(t)
         assert torch.equal(joint, want[0][:t]) and torch.equal(prefix, want[1][:t])
     assert head.mtpc_get_status() == 0
+
+
+@pytest.mark.parametrize("family,n,r,v,v_valid,wpp", [
+    (B.MTPC_CP, 16, 16, 320, 0, 16), (B.MTPC_CP, 8, 64, 112, 0, 1), (B.MTPC_BTREE, 8, 32, 256, 0, 3), (B.MTPC_HMM, 16, 32, 272, 268, 2),
+    (B.MTPC_CP, 16, 8, 400, 0, 4)])
+def test_draws_of_many_slots(family, n, r, v, v_valid, wpp):
+    P = 100                                          # n P > 2 x 148
+    few = 148 // n
+    head, hidden, g = _head(family, n, r, v, 64, P, wpp, v_valid)
+    uniforms = torch.rand(P * wpp, 2 * n, device="cuda", generator=g)
+    uniforms[5, n] = 1.0                             # one refused draw
+
+    def draft(p):
+        out, prefix = torch.empty(p * wpp, n, dtype=torch.int32, device="cuda"), torch.empty(p * wpp, n, device="cuda")
+        head.mtpc_draft_sample_prefix(hidden[:p].contiguous(), wpp, uniforms[:p * wpp].contiguous(), out, prefix)
+        return out, prefix
+
+    many, some = draft(P), draft(few)
+    assert torch.equal(some[0], many[0][:few * wpp]) and torch.equal(some[1].nan_to_num(1.0), many[1][:few * wpp].nan_to_num(1.0))
+    assert (many[0] < 0).sum() == 1 and many[0][5, 0] == -1 and (many[0] < (v_valid or v)).all()

@@ -82,7 +82,7 @@ bool fit_tiling(Tiling* t, int sum_cols) {
   t->num_slots = kTmemCols / t->slot_stride;
   if (t->num_slots > kMaxSlots) t->num_slots = kMaxSlots;
   t->stage_bytes = (kABytes + widest * kBlockK * 2 + 1023) / 1024 * 1024;   // A tile + one B tile
-  const int ctl = 1024 + static_cast<int>(sizeof(GemmControl));
+  const int ctl = 1024 + static_cast<int>(sizeof(GemmControl)) + kExchangeBytes;
   int stages = (kSmemLimit - ctl) / t->stage_bytes;
   if (stages > kMaxStages) stages = kMaxStages;
   t->stages = stages;
@@ -445,9 +445,9 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
   p.m_tiles = (rows + kBlockM - 1) / kBlockM;
   // Every CTA alone, or two CTAs per MMA (when there are two m-tiles to pair up and the device can hold a cluster at all): whichever
   // plan takes less time. A pair moves less operand data per MMA, which counts when K is long; with few K steps the epilogue bounds
-  // a tile, and a lone CTA need not wait for its partner's. Time per tile in pairs / alone over 256 to 4096 positions of 8 x 16 x 320,
-  // 4 x 8 x 256 and 8 x 8 x 272 heads: d = 1024 1.00 to 1.17, d = 1088 1.00 to 1.14, d = 1280 0.95 to 1.08, d = 1536 0.90 to 1.08,
-  // d = 1792 0.92 to 1.08, d = 2048 0.85 to 1.08, d = 4096 0.85 to 1.10 (above 1 only where a CTA has one or two tiles). A ragged
+  // a tile, and a lone CTA need not wait for its partner's. Whole calls in pairs / alone over 256 to 4000 positions of 8 x 16 x 320,
+  // 4 x 8 x 256 and 8 x 8 x 272 heads: d = 256 1.09 to 1.19, d = 512 1.08 to 1.32, d = 1024 0.96 to 1.11, d = 1280 0.94 to 1.15, d = 1536
+  // 0.97 to 1.17, d = 2048 0.97 to 1.08, d = 4096 0.93 to 1.08 (above 1 there where a CTA has one or two tiles). A ragged
   // number of m-tiles costs the pairs more tiles (384 positions, d = 4096, 8 x 16 x 320: 5 a pair against 4, 150 us / 138).
   const int emit_units = with_emit ? c.n * c.r : 0, launch_sums = with_sum ? L.sum_tiles : 0;
   bool pair = grp == nullptr && h->projection_variant == 2;
@@ -502,9 +502,9 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
   const int grid = ctas * static_cast<int>(items < workers ? items : workers);
   const size_t smem = pair ? tl.pair_smem : tl.smem;
   p.work_counter = with_sum ? p.status + kWorkCounterWord : nullptr;    // (the first launch of every call that needs it zeroed)
-  if (grp) launch_kernel(mtpc_gemm_kernel<kModeLogitsGrouped, 1>, grid, kGemmThreads, smem, st, overlapped(h), p);
-  else if (!pair) launch_kernel(mtpc_gemm_kernel<kModeLogprob, 1>, grid, kGemmThreads, smem, st, overlapped(h), p);
-  else launch_clusters(mtpc_gemm_kernel<kModeLogprob, 2>, 2, grid, kGemmThreads, smem, st, overlapped(h), p);
+  if (grp) launch_kernel(mtpc_gemm_kernel<kModeLogitsGrouped, 1, 16>, grid, gemm_threads(kModeLogitsGrouped), smem, st, overlapped(h), p);
+  else if (!pair) launch_kernel(c.v % 32 == 0 ? mtpc_gemm_kernel<kModeLogprob, 1, 32> : mtpc_gemm_kernel<kModeLogprob, 1, 16>, grid, gemm_threads(kModeLogprob), smem, st, overlapped(h), p);
+  else launch_clusters(c.v % 32 == 0 ? mtpc_gemm_kernel<kModeLogprob, 2, 32> : mtpc_gemm_kernel<kModeLogprob, 2, 16>, 2, grid, gemm_threads(kModeLogprob), smem, st, overlapped(h), p);
   h->launches++;
   return check_launch();
 }
@@ -611,7 +611,7 @@ bool set_circuit_attributes() {
 // How many clusters of `size` CTAs of a kernel, each with all the shared memory a CTA can have, device `dev` holds at once (0:
 // none). Asked of the driver once per device and `which` (about 30 us each, a property of the device): heads are made often.
 template <typename K>
-int resident_clusters(K kernel, int size, int which, int dev) {
+int resident_clusters(K kernel, int size, int threads, int which, int dev) {
   constexpr int kDevices = 64;
   static std::atomic<int> known[4][kDevices];                            // count + 1
   std::atomic<int>* entry = dev >= 0 && dev < kDevices ? &known[which][dev] : nullptr;
@@ -619,7 +619,7 @@ int resident_clusters(K kernel, int size, int which, int dev) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(size);
-  cfg.blockDim = dim3(kGemmThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = kSmemLimit;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1705,11 +1705,10 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   bool fail = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess;
   // the attribute is per function, not per head: always ask for the full 227 KB so that heads do not undo each other
-  fail |= cudaFuncSetAttribute(mtpc_gemm_kernel<kModeLogprob, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kSmemLimit) != cudaSuccess;
-  fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogitsGrouped, 1>);
-  fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 2>);
-  h->max_pairs = fail ? 0 : resident_clusters(mtpc_gemm_kernel<kModeLogprob, 2>, 2, 0, dev);
+  fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 1, 16>) || !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 1, 32>);
+  fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogitsGrouped, 1, 16>);
+  fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 2, 16>) || !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 2, 32>);
+  h->max_pairs = fail ? 0 : resident_clusters(mtpc_gemm_kernel<kModeLogprob, 2, 16>, 2, gemm_threads(kModeLogprob), 0, dev);
   fail |= !allow_full_smem(plain_gemm_kernel<false, false>);
   fail |= !allow_full_smem(plain_gemm_kernel<false, true>);
   fail |= !allow_full_smem(plain_gemm_kernel<true, true>);
@@ -1721,7 +1720,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   fail |= !allow_full_smem(adaptor_grad_kernel);
   fail |= cudaFuncSetAttribute(mtpc_decode_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) !=
           cudaSuccess;
-  for (int e = 0; e < 3; ++e) h->max_decode_clusters[e] = fail ? 0 : resident_clusters(mtpc_decode_gemm_kernel, 2 << e, 1 + e, dev);
+  for (int e = 0; e < 3; ++e) h->max_decode_clusters[e] = fail ? 0 : resident_clusters(mtpc_decode_gemm_kernel, 2 << e, kGemmThreads, 1 + e, dev);
   const int slot_smem = static_cast<int>(kSlotSmemLimit);
   for (auto* kernel : {draft_slot_kernel<false, 4, 2>, draft_slot_kernel<false, 8, 2>, draft_slot_kernel<false, 10, 2>, draft_slot_kernel<false, 16, 2>,
                        draft_slot_kernel<false, 4, 3>, draft_slot_kernel<false, 8, 3>, draft_slot_kernel<false, 10, 3>, draft_slot_kernel<true, 16, 2>})
@@ -2552,8 +2551,7 @@ extern "C" int mtpc_window_logprob_static(const mtpc_config* cfg, const void* W_
   h.wait_limit_ns = kWaitLimitNs;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   bool fail = cudaDeviceGetAttribute(&h.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess;
-  fail |= cudaFuncSetAttribute(mtpc_gemm_kernel<kModeLogprob, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kSmemLimit) != cudaSuccess;
+  fail |= !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 1, 16>) || !allow_full_smem(mtpc_gemm_kernel<kModeLogprob, 1, 32>);
   fail |= !set_circuit_attributes();
   // The array keeps whatever the previous call left in it. Only the status word has to start at zero; G, log omega
   // and logA are fully rewritten for the rows this call reads.

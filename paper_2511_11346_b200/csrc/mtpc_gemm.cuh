@@ -3,14 +3,14 @@
 // in the epilogue straight out of tensor memory. The [positions, n, r, v] logit tensor never exists in HBM, except when a
 // training call or a draft of many positions asks the epilogue to keep it (logit_out).
 //
-// One persistent CTA per SM, 6 warps:
+// One persistent CTA per SM, 10 warps:
 //   warp 0      TMA producer: per 64-wide K block, one 128-row tile of h and the v rows of one emission unit
 //               (or one tile of sum-unit rows) into a ring of shared-memory stages (128-byte swizzle).
 //   warp 1      allocates the 512 TMEM columns, issues tcgen05.mma (M=128, N=chunk, K=16) from one thread. Warps 0 and 1 run as wholes
 //               and predicate what they issue (elect_one): short calls 1 to 6 % shorter than from branches of lane 0's own (300 factored
 //               positions of 4 x 8 x 256, d = 1024: 45.6 -> 42.8 us, 500 of 8 x 16 x 320, d = 2048: 69.0 -> 67.7).
-//   warps 2..5  epilogue; warp w reads TMEM lanes 32*(w%4)..+31, one thread per position (row), so every
-//               row-wise reduction over the vocabulary is a plain in-thread loop.
+//   warps 2..9  epilogue (2..5 on sorted rows); warp w reads TMEM lanes 32*(w%4)..+31, one thread per position (row), so every
+//               row-wise reduction over the vocabulary is an in-thread loop, shared by the two warps of the same lanes.
 // The N axis of the GEMM is the flattened (slot i, unit k, byte b) row index of W_emit. A work item is 128
 // positions x one "group": `group_units` consecutive emission units = a run of rows that starts at a unit
 // boundary, covered by accumulator tiles of `tile_cols` columns. The log-likelihood mode uses 256-column tiles
@@ -32,7 +32,7 @@ namespace mtpc {
 constexpr int kBlockM = 128;         // positions per tile (= TMEM lanes)
 constexpr int kBlockK = 64;          // bf16 elements per 128-byte swizzled row
 constexpr int kMaxStages = 16;
-constexpr int kMaxSlots = 16;
+constexpr int kMaxSlots = 8;
 constexpr int kTmemCols = 512;
 constexpr int kGemmThreads = 192;
 constexpr uint64_t kWaitLimitNs = 1000ull * 1000ull * 1000ull;   // 1 s per barrier wait (the default, and always the limit of the drain waits)
@@ -237,13 +237,32 @@ __device__ __forceinline__ ItemWalk item_walk(const GemmParams& p, int emit_item
 }
 
 // Padding columns of a unit (vocabulary not a multiple of 16) count as logit = -inf: never the maximum, no mass.
-__device__ __forceinline__ void mask_padding(float (&x)[16], int col_in_unit, int vv) {
-  if (col_in_unit + 16 > vv) {
+template <int N>
+__device__ __forceinline__ void mask_padding(float (&x)[N], int col_in_unit, int vv) {
+  if (col_in_unit + N > vv) {
 #pragma unroll
-    for (int q = 0; q < 16; ++q)
+    for (int q = 0; q < N; ++q)
       if (col_in_unit + q >= vv) x[q] = -CUDART_INF_F;
   }
 }
+// x[i] for an i < N that differs from lane to lane.
+template <int N>
+__device__ __forceinline__ float select_column(const float (&x)[N], int i) {
+  float a[N / 2];
+#pragma unroll
+  for (int q = 0; q < N / 2; ++q) a[q] = i & (N / 2) ? x[q + N / 2] : x[q];
+#pragma unroll
+  for (int step = N / 4; step >= 1; step /= 2)
+#pragma unroll
+    for (int q = 0; q < step; ++q) a[q] = i & step ? a[q + step] : a[q];
+  return a[0];
+}
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void issue_batch(uint32_t taddr, uint32_t (&r)[16]) { tmem_ld16_issue(taddr, r); }
+__device__ __forceinline__ void issue_batch(uint32_t taddr, uint32_t (&r)[32]) { tmem_ld32_issue(taddr, r); }
+__device__ __forceinline__ void wait_batch(uint32_t (&r)[16]) { tmem_ld_wait16(r); }
+__device__ __forceinline__ void wait_batch(uint32_t (&r)[32]) { tmem_ld_wait32(r); }
 
 // log-softmax over groups of R adjacent columns inside one 16-column batch (R in {1,2,4,8,16}).
 template <int R>
@@ -271,8 +290,19 @@ __device__ __forceinline__ void sum_groups_in_batch(const float (&x)[16], float*
 // 128 accumulator rows. Barriers: full[s] lives in the leader and counts the bytes of both CTAs' copies; empty[s] and
 // tfull[slot] exist in both CTAs and are signalled together by the leader's commits; tempty[slot] lives in the leader
 // and collects the arrivals of both CTAs' epilogue warps.
-template <int MODE, int CTAS>
-__global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid_constant__ GemmParams p) {
+//
+// Epilogue of the log-likelihood mode: eight warps, two on each quarter of the accumulator rows, which take its batches of COLS columns in turn
+// (32, or 16 where v is no multiple of 32). Each keeps a maximum, a sum and the target's logit of a unit's columns that it has seen; at the end of
+// the unit the second hands its three to the first (in shared memory behind the control block, by a pair of named barriers), which adds
+// them up. One warp alone issued on a fifth of the cycles: batches of 16 columns took it 600 cycles where their exponentials take
+// 128, so that short K was bound by it and every call ended with 5 us of it. (8 x 16 x 320, d = 256, 4000 positions 188 us; with 32 columns,
+// a maximum by halves and no branch around the target 118;
+// with two warps 102. 4 x 8 x 256, d = 256, 256 positions 10.9 -> 9.0 us; 8 x 16 x 256, d = 1024, 3000 positions 161 -> 149.)
+__host__ __device__ constexpr int gemm_subs(int mode) { return mode == kModeLogprob ? 2 : 1; }
+__host__ __device__ constexpr int gemm_threads(int mode) { return 64 + 128 * gemm_subs(mode); }
+constexpr int kExchangeBytes = 4 * 3 * 32 * 4;
+template <int MODE, int CTAS, int COLS>
+__global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const __grid_constant__ GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t tiles_addr = (raw_addr + 1023u) & ~1023u;
@@ -282,6 +312,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
   const int warp = static_cast<int>(warp_uniform(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   constexpr bool kGrouped = MODE == kModeLogitsGrouped;
+  constexpr int kSubs = gemm_subs(MODE);
   if (kGrouped) grid_dependency_wait();   // the tiles are read below
   static_assert(!kGrouped || CTAS == 1, "grouped tiles are ragged: no pairing");
   const int emit_items = kGrouped ? static_cast<int>(warp_uniform(*p.group_num_tiles)) * p.num_groups : p.num_groups * p.m_units;
@@ -304,7 +335,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
     }
     for (int s = 0; s < p.num_slots; ++s) {
       mbar_init(smem_u32(&ctl->tfull[s]), 1);
-      mbar_init(smem_u32(&ctl->tempty[s]), 4 * CTAS);
+      mbar_init(smem_u32(&ctl->tempty[s]), 4 * CTAS * kSubs);
     }
     mbar_init(smem_u32(&ctl->drain), 1);
     ctl->abort = 0;
@@ -418,7 +449,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue
-    const int quarter = warp & 3;
+    const int quarter = warp & 3, sub = (warp - 2) >> 2;
     const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
     uint32_t use = 0;
     bool ok = true;
@@ -427,7 +458,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
       if (CTAS == 2) mbar_arrive_cluster(cluster_map_shared(smem_u32(&ctl->tempty[slot]), 0));
       else mbar_arrive(smem_u32(&ctl->tempty[slot]));
     };
-    for (int item = walk.first(); item < walk.end && ok; item = walk.next(item)) {
+    bool handed = false;                                       // (of two warps, the second: the first has a unit's share to read)
+    float* share = reinterpret_cast<float*>(ctl + 1) + quarter * 96 + lane;
+    // (two warps that meet at barriers both go on after a wait that gave up, without waiting)
+    for (int item = walk.first(); item < walk.end && (ok || kSubs == 2); item = walk.next(item)) {
       const TileCoord tc = coord(item);
       const int row = tc.arow + quarter * 32 + lane;
       const bool valid = quarter * 32 + lane < tc.count;
@@ -436,16 +470,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
       if (tc.is_sum) {
         // ---- sum-unit logits -> log omega (Sec. 3.3): log-softmax over groups of r adjacent columns
         const uint32_t slot = use % p.num_slots;
-        if (!bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use / p.num_slots) & 1u, ctl, p.status, lane)) {
-          ok = false;
-          break;
-        }
+        ok = ok && bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use / p.num_slots) & 1u, ctl, p.status, lane);
+        if (!ok && kSubs == 1) break;
         tc_fence_after();
         const uint32_t tcol = lane_base + slot * p.slot_stride;
         const int col_base = tc.unit0 * p.sum_cols;
         float* dst = p.logw + static_cast<size_t>(valid ? row : 0) * p.sum_rows;
         if (p.r <= 16) {
-          for (int b = 0; b < nbatch; ++b) {
+          for (int b = sub; b < nbatch; b += kSubs) {
             float x[16];
             tmem_ld16(tcol + b * 16, x);
             if (valid) {
@@ -466,7 +498,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
           }
         } else {
           const int bpg = p.r / 16;   // batches per group
-          for (int g = 0; g < tc.cols / p.r; ++g) {
+          for (int g = sub; g < tc.cols / p.r; g += kSubs) {
             float m = -CUDART_INF_F, s = 0.f;
             const int gcol = col_base + g * p.r;
             const bool biased = p.sum_bias != nullptr && gcol < p.sum_rows;
@@ -558,100 +590,132 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_gemm_kernel(const __grid
       } else {
         // ---- log phi at the target byte: online log-sum-exp over the v columns of each unit + gather. The
         // running (m, s) and the gathered logit live across tile boundaries; a unit is closed when its v-th
-        // column has been consumed.
+        // column has been passed.
         const int* tgts = (valid && p.targets != nullptr) ? p.targets + static_cast<size_t>(row) * p.n : nullptr;
         const int units_end = tc.unit0 + tc.nunits;
         int unit = tc.unit0, col_in_unit = 0;
         int slot_i = unit / p.r, k = unit - slot_i * p.r;
         float m = -CUDART_INF_F, s = 0.f, tval = 0.f;
         int tgt = tgts != nullptr ? tgts[slot_i] : -1;
-        for (int t = 0; t < tc.ntiles && ok; ++t, ++use) {
-          const uint32_t slot = use % p.num_slots;
-          if (!bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use / p.num_slots) & 1u, ctl, p.status, lane)) {
-            ok = false;
-            break;
+        // ---- unit (slot_i, k) complete
+        auto close_unit = [&] {
+          if (kSubs == 2 && sub == 1) {
+            if (handed) pair_sync(5 + quarter);                          // the share before this one has been read
+            share[0] = m;
+            share[32] = s;
+            share[64] = tval;
+            pair_arrive(1 + quarter);
+            handed = true;
+          } else {
+            if (kSubs == 2) {
+              pair_sync(1 + quarter);
+              const float m2 = share[0], s2 = share[32];
+              tval += share[64];                                         // (one of the two has seen the target's column)
+              pair_arrive(5 + quarter);
+              // the same bits whichever warp had the unit's first batch, which depends on where in an item the unit lies
+              const float mn = fmaxf(m, m2);
+              s = __fadd_rn(__fmul_rn(s, fast_ex2((m - mn) * kLog2e)), __fmul_rn(s2, fast_ex2((m2 - mn) * kLog2e)));
+              m = mn;
+            }
+            const float lse = m + fast_lg2(s) * kLn2;
+            if (valid) {
+              const size_t at = (static_cast<size_t>(row) * p.n + slot_i) * p.r + k;
+              if (p.lse_out != nullptr) p.lse_out[at] = lse;
+              if (tgts != nullptr) {
+                p.G[at] = tgt < 0 ? 0.f : tgt >= p.vv ? CUDART_NAN_F : tval - lse;      // < 0: a marginalised byte, the input unit sums to 1
+                if (tgt >= p.vv) atomicOr(p.status, kStatusBadTarget);
+              }
+            }
           }
+          col_in_unit = 0;
+          m = -CUDART_INF_F; s = 0.f; tval = 0.f;
+          if (++unit < units_end && ++k == p.r) {
+            k = 0;
+            ++slot_i;
+            if (tgts != nullptr) tgt = tgts[slot_i];
+          }
+        };
+        // past one batch of columns, whoever's it was; false once the item's last unit has been closed
+        auto pass_batch = [&]() -> bool {
+          col_in_unit += COLS;
+          if (col_in_unit != p.v) return true;
+          close_unit();
+          return unit < units_end;
+        };
+        for (int t = 0; t < tc.ntiles; ++t, ++use) {
+          const uint32_t slot = use % p.num_slots;
+          ok = ok && bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use / p.num_slots) & 1u, ctl, p.status, lane);
           tc_fence_after();
           const uint32_t tcol = lane_base + slot * p.slot_stride;
-          // one batch of 16 accumulator columns of this row; false once the item's last unit has been closed
-          auto consume = [&](const uint32_t (&raw)[16], int b) -> bool {
-            float x[16];
+          // one batch of accumulator columns of this row
+          auto consume = [&](const uint32_t (&raw)[COLS], int b) {
+            float x[COLS];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) x[q] = __uint_as_float(raw[q]);
+            for (int q = 0; q < COLS; ++q) x[q] = __uint_as_float(raw[q]);
             mask_padding(x, col_in_unit, p.vv);
-            if (p.logit_out != nullptr && valid) {                       // row of W_emit = column of the logit matrix
-              float* l = p.logit_out + static_cast<size_t>(row) * p.logit_pitch + tc.brow0 + t * tc.cols + b * 16;
-              st_global_v8(l, x);                                        // 64-byte aligned: v and the tile widths are multiples of 16
-              st_global_v8(l + 8, x + 8);
+            if (p.logit_out != nullptr) {                                // row of W_emit = column of the logit matrix
+              float* l = p.logit_out + static_cast<size_t>(row) * p.logit_pitch + tc.brow0 + t * tc.cols + b * COLS;
+              if (valid) {
+#pragma unroll
+                for (int q = 0; q < COLS; q += 8) st_global_v8(l + q, x + q);   // 64-byte aligned: v and the tile widths are multiples of 16
+              }
             }
-            float bm = x[0];
+            float bm[COLS / 2];
 #pragma unroll
-            for (int q = 1; q < 16; ++q) bm = fmaxf(bm, x[q]);
-            const float mn = fmaxf(m, bm);
-            const float mn2 = mn * kLog2e;
-            s *= fast_ex2((m - mn) * kLog2e);
+            for (int q = 0; q < COLS / 2; ++q) bm[q] = fmaxf(x[q], x[q + COLS / 2]);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) s += fast_ex2(fmaf(x[q], kLog2e, -mn2));
+            for (int step = COLS / 4; step >= 1; step /= 2)
+#pragma unroll
+              for (int q = 0; q < step; ++q) bm[q] = fmaxf(bm[q], bm[q + step]);
+            const float mn = fmaxf(m, bm[0]);
+            const float2 l2 = make_float2(kLog2e, kLog2e), nr = make_float2(-mn * kLog2e, -mn * kLog2e);
+            float2 sa = make_float2(s * fast_ex2((m - mn) * kLog2e), 0.f), sb = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < COLS; q += 2) {
+              const float2 y = __ffma2_rn(make_float2(x[q], x[q + 1]), l2, nr);
+              const float2 e = make_float2(fast_ex2(y.x), fast_ex2(y.y));
+              if (q & 2) sb = __fadd2_rn(sb, e);
+              else sa = __fadd2_rn(sa, e);
+            }
+            s = (sa.x + sa.y) + (sb.x + sb.y);
             m = mn;
             const int rel = tgt - col_in_unit;
-            if (static_cast<unsigned>(rel) < 16u) {
-#pragma unroll
-              for (int q = 0; q < 16; ++q)
-                if (rel == q) tval = x[q];
-            }
-            col_in_unit += 16;
-            if (col_in_unit == p.v) {
-              // ---- unit (slot_i, k) complete
-              const float lse = m + fast_lg2(s) * kLn2;
-              if (valid && p.lse_out != nullptr)
-                p.lse_out[(static_cast<size_t>(row) * p.n + slot_i) * p.r + k] = lse;
-              if (tgts != nullptr) {
-                float* g = p.G + (static_cast<size_t>(row) * p.n + slot_i) * p.r + k;
-                if (tgt < 0) {
-                  *g = 0.f;                              // marginalised byte: the input unit sums to 1
-                } else if (tgt >= p.vv) {
-                  *g = CUDART_NAN_F;
-                  atomicOr(p.status, kStatusBadTarget);
-                } else {
-                  *g = tval - lse;
-                }
-              }
-              ++unit;
-              col_in_unit = 0;
-              m = -CUDART_INF_F; s = 0.f; tval = 0.f;
-              if (unit < units_end) {
-                slot_i = unit / p.r;
-                k = unit - slot_i * p.r;
-                tgt = tgts != nullptr ? tgts[slot_i] : -1;
-              }
-            }
-            return unit < units_end;
+            const float at_rel = select_column(x, rel);                  // (a branch around it costs more than it saves)
+            tval = static_cast<unsigned>(rel) < COLS ? at_rel : tval;
+          };
+          // this warp's batch b and the ones that it passes on the way
+          auto take = [&](const uint32_t (&raw)[COLS], int b) -> bool {
+            if (sub == 1 && !pass_batch()) return false;
+            consume(raw, b);
+            if (!pass_batch()) return false;
+            return kSubs == 1 || sub == 1 || pass_batch();
           };
           // The load of the next batch is in flight while this one goes through the exponentials (two register buffers).
-          uint32_t ra[16], rb[16];
-          tmem_ld16_issue(tcol, ra);
-          tmem_ld_wait16(ra);
-          for (int b = 0;;) {
-            const bool more_b = b + 1 < nbatch;
-            if (more_b) tmem_ld16_issue(tcol + (b + 1) * 16, rb);
-            const bool go_a = consume(ra, b);
-            if (more_b) tmem_ld_wait16(rb);
+          const int batches = tc.cols / COLS;
+          uint32_t ra[COLS], rb[COLS];
+          issue_batch(tcol + sub * COLS, ra);
+          wait_batch(ra);
+          for (int b = sub;;) {
+            const bool more_b = b + kSubs < batches;
+            if (more_b) issue_batch(tcol + (b + kSubs) * COLS, rb);
+            const bool go_a = take(ra, b);
+            if (more_b) wait_batch(rb);
             if (!go_a || !more_b) break;
-            ++b;
-            const bool more_a = b + 1 < nbatch;
-            if (more_a) tmem_ld16_issue(tcol + (b + 1) * 16, ra);
-            const bool go_b = consume(rb, b);
-            if (more_a) tmem_ld_wait16(ra);
+            b += kSubs;
+            const bool more_a = b + kSubs < batches;
+            if (more_a) issue_batch(tcol + (b + kSubs) * COLS, ra);
+            const bool go_b = take(rb, b);
+            if (more_a) wait_batch(ra);
             if (!go_b || !more_a) break;
-            ++b;
+            b += kSubs;
           }
           tc_fence_before();
           __syncwarp();
           if (lane == 0) release_slot(slot);
         }
-        if (!ok) break;
       }
     }
+    if (kSubs == 2 && handed) pair_sync(5 + quarter);
   }
 
   tc_fence_before();

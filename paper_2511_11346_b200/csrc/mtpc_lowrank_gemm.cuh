@@ -25,7 +25,8 @@
 // busy for 73 / 43 % of the cycles (61 / 38); the gradient's rest is instructions (two thirds of an issue slot a logit) and its warps' latency.
 // The fused projection that kept logits took 801 us and the passes that made g and its sum from them 921.
 // Roles: warp 0 TMA producer, warp 1 MMA issuer, then the epilogue warps (TMEM quarter warp % 4).
-// Both issue from a converged warp (elect_one): forward 240 -> 222 us, gradient 403 -> 398.
+// Both issue from a converged warp (elect_one): forward 240 -> 222 us, gradient 403 -> 398. A quarter of the forward's exponentials are polynomials
+// (poly_ex2), since the exponential unit was busy for 73 % of the cycles and issue slots for 47: 222 -> 208.
 // Operand ring: one entry holds 32 / k components, all as 128-byte rows with the 128-byte swizzle: z as one box of 128
 // positions x 64 values ([hi | lo] of the components), and A as one box of the item's vocabulary rows x 64 values (the components' k
 // adaptor columns first) of a copy laid out [n, v, r, k] (lowrank_repack_kernel, made on every call: A is small and may have changed).
@@ -96,6 +97,27 @@ __device__ __forceinline__ void st_shared_bf16(uint32_t dst, __nv_bfloat16 x) {
   asm volatile("st.shared.b16 [%0], %1;" ::"r"(dst), "h"(__bfloat16_as_ushort(x)) : "memory");
 }
 
+// 2^y on the multiply-add pipe: y = n + f with |f| <= 1/2 by adding and taking away 1.5 * 2^23, a polynomial of degree 6 in f (its coefficients
+// by Remez' exchange for the least relative error, 1.9e-9), n added to the exponent (splitting exponentials between the two units is
+// FlashAttention-4's published idea). Against fp64 over [-120, 100] at most 8.0e-8 off (rms 2.7e-8), the exponential unit 1.5e-7 (5e-8). Below -126: 2^-126;
+// above 127 or no number: a number beyond 2^120 or no number, which the sums' check catches.
+__device__ __forceinline__ float2 poly_ex2(float2 y) {
+  asm("max.NaN.f32 %0, %0, %1;" : "+f"(y.x) : "f"(-126.f));
+  asm("max.NaN.f32 %0, %0, %1;" : "+f"(y.y) : "f"(-126.f));
+  asm("min.NaN.f32 %0, %0, %1;" : "+f"(y.x) : "f"(127.f));
+  asm("min.NaN.f32 %0, %0, %1;" : "+f"(y.y) : "f"(127.f));
+  auto both = [](float x) { return make_float2(x, x); };
+  const float2 t = __fadd2_rn(y, both(12582912.f));
+  const float2 f = __ffma2_rn(__fadd2_rn(t, both(-12582912.f)), both(-1.f), y);
+  float2 p = __ffma2_rn(both(1.53458124e-4f), f, both(1.33999309e-3f));
+  p = __ffma2_rn(p, f, both(9.61848907e-3f));
+  p = __ffma2_rn(p, f, both(5.55032864e-2f));
+  p = __ffma2_rn(p, f, both(2.40226462e-1f));
+  p = __ffma2_rn(p, f, both(6.93147182e-1f));
+  p = __ffma2_rn(p, f, both(1.f));
+  return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
+                     __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
+}
 struct LowRankItem {
   int mt, slot, block, width;     // width: columns of this block (a multiple of 16)
 };
@@ -349,7 +371,7 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) low
 #pragma unroll
               for (int e = 0; e < 8; ++e) {
                 const float2 y = __ffma2_rn(make_float2(__uint_as_float(c[2 * e]), __uint_as_float(c[2 * e + 1])), l2, base[8 * half + e]);
-                const float2 x = make_float2(fast_ex2(y.x), fast_ex2(y.y));
+                const float2 x = (e & 3) == 2 ? poly_ex2(y) : make_float2(fast_ex2(y.x), fast_ex2(y.y));   // a quarter of them
                 if (e & 1) sb = __fadd2_rn(sb, x);
                 else sa = __fadd2_rn(sa, x);
               }

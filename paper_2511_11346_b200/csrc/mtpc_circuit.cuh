@@ -932,8 +932,9 @@ __global__ void __launch_bounds__(kLossThreads) loss_coeff_kernel(const int* __r
 // (One value per thread took 16.6 us for 2005 x 3072 values, a sixth of the copy bandwidth.)
 __global__ void __launch_bounds__(256) f32_to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, size_t count,
                                                           int vec) {
-  grid_dependency_wait();
   const size_t first = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (vec && first < count / 8) prefetch_l2(src + 8 * first);    // (256 positions of 4 x 8 x 256, d = 256: a call of 10.8 us now 10.6)
+  grid_dependency_wait();
   const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
   if (!vec) {
     for (size_t i = first; i < count; i += stride) dst[i] = __float2bfloat16_rn(src[i]);

@@ -100,6 +100,9 @@ __device__ __forceinline__ float fast_lg2(float x) {
 }
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
+// The log-likelihood epilogue's exponentials never take a reference below this: its product with log2 e is rounded by 64 at most, so that what
+// lies below has no mass and never overflows, also where a run of -inf or of huge negative logits is all that a warp has seen.
+constexpr float kLowestRef = -0x1p30f;
 
 __device__ __forceinline__ bool bounded_wait(uint32_t bar, uint32_t parity, GemmControl* ctl, unsigned* status) {
   if (mbar_try_wait(bar, parity)) return true;
@@ -613,11 +616,12 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
               tval += share[64];                                         // (one of the two has seen the target's column)
               pair_arrive(5 + quarter);
               // the same bits whichever warp had the unit's first batch, which depends on where in an item the unit lies
-              const float mn = fmaxf(m, m2);
-              s = __fadd_rn(__fmul_rn(s, fast_ex2((m - mn) * kLog2e)), __fmul_rn(s2, fast_ex2((m2 - mn) * kLog2e)));
-              m = mn;
+              const float ref = fmaxf(m, kLowestRef), ref2 = fmaxf(m2, kLowestRef), rn = fmaxf(ref, ref2);
+              s = __fadd_rn(__fmul_rn(s, fast_ex2((ref - rn) * kLog2e)), __fmul_rn(s2, fast_ex2((ref2 - rn) * kLog2e)));
+              m = fmaxf(m, m2);
             }
-            const float lse = m + fast_lg2(s) * kLn2;
+            // a unit that lies below the lowest reference as a whole: less than half an ulp above its maximum (-inf, NaN: NaN)
+            const float lse = m >= kLowestRef ? fmaf(fast_lg2(s), kLn2, m) : fmaf(m - m, s, m);
             if (valid) {
               const size_t at = (static_cast<size_t>(row) * p.n + slot_i) * p.r + k;
               if (p.lse_out != nullptr) p.lse_out[at] = lse;
@@ -667,9 +671,11 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
             for (int step = COLS / 4; step >= 1; step /= 2)
 #pragma unroll
               for (int q = 0; q < step; ++q) bm[q] = fmaxf(bm[q], bm[q + step]);
-            const float mn = fmaxf(m, bm[0]);
-            const float2 l2 = make_float2(kLog2e, kLog2e), nr = make_float2(-mn * kLog2e, -mn * kLog2e);
-            float2 sa = make_float2(s * fast_ex2((m - mn) * kLog2e), 0.f), sb = make_float2(0.f, 0.f);
+            const float ref = fmaxf(m, kLowestRef);
+            m = fmaxf(m, bm[0]);
+            const float rn = fmaxf(m, kLowestRef);
+            const float2 l2 = make_float2(kLog2e, kLog2e), nr = make_float2(-rn * kLog2e, -rn * kLog2e);
+            float2 sa = make_float2(s * fast_ex2((ref - rn) * kLog2e), 0.f), sb = make_float2(0.f, 0.f);
 #pragma unroll
             for (int q = 0; q < COLS; q += 2) {
               const float2 y = __ffma2_rn(make_float2(x[q], x[q + 1]), l2, nr);
@@ -678,7 +684,6 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
               else sa = __fadd2_rn(sa, e);
             }
             s = (sa.x + sa.y) + (sb.x + sb.y);
-            m = mn;
             const int rel = tgt - col_in_unit;
             const float at_rel = select_column(x, rel);                  // (a branch around it costs more than it saves)
             tval = static_cast<unsigned>(rel) < COLS ? at_rel : tval;

@@ -1293,10 +1293,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
         if (!ok) break;
         commit(smem_u32(&ctl->tfull[slot]));
       }
-      if (!ok) {
-        commit(smem_u32(&ctl->drain));
-        drain_wait(smem_u32(&ctl->drain), 0);
-      }
     }
     __syncwarp();
   } else {
@@ -1338,12 +1334,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
 
   tc_fence_before();
   __syncthreads();
-  if (CTAS == 2) {
-    // a CTA of a pair may leave only when its partner no longer needs it; after an abort, first let what is in flight land
-    if (ctl->abort && threadIdx.x == 0) {
-      const uint64_t t0 = global_timer_ns();
-      while (global_timer_ns() - t0 < kAbortSettleNs) {}
-    }
+  if (warp == 1) drain_after_abort<CTAS>(ctl, cta_rank == 0);
+  if (CTAS == 2) {        // a CTA of a pair may leave only when its partner no longer needs it
     __syncthreads();
     cluster_sync_all();
   }

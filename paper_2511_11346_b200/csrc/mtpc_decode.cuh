@@ -251,10 +251,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
       if (!ok) break;
       umma_commit(lead, smem_u32(&ctl->tfull[slot]));
     }
-    if (!ok) {
-      umma_commit(lead, smem_u32(&ctl->drain));
-      drain_wait(smem_u32(&ctl->drain), 0);
-    }
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue: warp q owns lanes 32q .. 32q+31
@@ -288,6 +284,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
 
   tc_fence_before();
   __syncthreads();
+  if (warp == 1) drain_after_abort<1>(ctl, true);
   if (p.ksplit > 1) {
     cluster_sync_all();       // the other CTAs' accumulators have arrived
     if (rank == 0 && warp >= 2) {

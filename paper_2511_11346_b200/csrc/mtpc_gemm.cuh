@@ -151,6 +151,25 @@ __device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity) {
   while (!mbar_try_wait(bar, parity) && global_timer_ns() - t0 < kWaitLimitNs) {}
 }
 
+// Warp 1 of a CTA whose roles have all ended and met: if a wait gave up in any of them, its MMAs may still be in flight, also where it had issued
+// all it had to. They are waited for before tensor memory is freed and the CTA goes away. Pairs: the leader's (`issuer`), and then as long
+// as any copy of either CTA takes, since the peer's are counted on the leader's barriers and cannot be awaited.
+template <int CTAS>
+__device__ __forceinline__ void drain_after_abort(GemmControl* ctl, bool issuer) {
+  if (!__any_sync(0xffffffffu, ctl->abort)) return;
+  if (issuer) {
+    const uint32_t lead = elect_one();                          // the lane that issued them
+    if (CTAS == 2) umma_commit_pair(lead, smem_u32(&ctl->drain));
+    else umma_commit(lead, smem_u32(&ctl->drain));
+    drain_wait(smem_u32(&ctl->drain), 0);
+  }
+  if (CTAS == 2) {
+    const uint64_t t0 = global_timer_ns();
+    while (global_timer_ns() - t0 < kAbortSettleNs) {}
+  }
+  __syncwarp();
+}
+
 struct TileCoord {
   int mt, is_sum, ntiles, cols, brow0, unit0, nunits;
   int arow, count;   // first row of the A operand and the rows that count (set by the caller for ungrouped items)
@@ -444,10 +463,6 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
           commit(smem_u32(&ctl->tfull[slot]));            // the accumulators are ready
         }
       }
-      if (!ok) {   // wait (bounded) for the MMAs already issued before TMEM is freed
-        commit(smem_u32(&ctl->drain));
-        drain_wait(smem_u32(&ctl->drain), 0);
-      }
     }
     __syncwarp();
   } else {
@@ -725,14 +740,10 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
 
   tc_fence_before();
   __syncthreads();
+  if (warp == 1) drain_after_abort<CTAS>(ctl, cta_rank == 0);
   if (CTAS == 2) {
     // A CTA of a pair may leave only when its partner no longer needs it (MMAs read both CTAs' shared memory and write
-    // both CTAs' tensor memory; copies and arrivals cross over). After a run in which some wait gave up, first let
-    // whatever is still in flight land: the peer's copies are counted on the leader's barriers and cannot be awaited here.
-    if (ctl->abort && threadIdx.x == 0) {
-      const uint64_t t0 = global_timer_ns();
-      while (global_timer_ns() - t0 < kAbortSettleNs) {}
-    }
+    // both CTAs' tensor memory; copies and arrivals cross over).
     __syncthreads();      // every warp converged again before the cluster-wide barrier
     cluster_sync_all();
   }

@@ -249,10 +249,6 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) low
         umma_commit(lead, smem_u32(&ctl->tfull[slot]));
       }
     }
-    if (!ok || __any_sync(kFull, ctl->abort)) {   // wait (bounded) for the MMAs already issued before tensor memory is freed
-      umma_commit(lead, smem_u32(&ctl->drain));
-      drain_wait(smem_u32(&ctl->drain), 0);
-    }
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue
@@ -524,6 +520,7 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) low
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    drain_after_abort<1>(ctl, true);
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmem);
   }
@@ -1002,10 +999,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) adaptor_grad_kernel(const __g
       umma_commit(lead, smem_u32(&ctl->tfull[2 + set]));
       umma_commit(lead, smem_u32(&ctl->empty[kAdaptorBarA]));
     }
-    if (!ok) {
-      umma_commit(lead, smem_u32(&ctl->drain));
-      drain_wait(smem_u32(&ctl->drain), 0);
-    }
     __syncwarp();
   } else {
     const int quarter = warp & 3;
@@ -1059,6 +1052,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) adaptor_grad_kernel(const __g
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    drain_after_abort<1>(ctl, true);
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }

@@ -258,3 +258,57 @@ def test_draft_and_acceptance_calls_can_be_captured_into_a_cuda_graph(family, n,
     assert np.abs(replayed[5].cpu().numpy()[:, -1] - oracle_logprob(wl)).max() <= LOGPROB_TOL
     del graph
     dh.close()
+
+
+@pytest.mark.parametrize("path", ["logprob", "logprob_single_ctas", "draft_few", "backward", "factored"])
+def test_a_call_right_behind_one_that_gave_up(path):
+    """A kernel that gave up leaves nothing in flight: the call that follows it in the stream, of another head and with nothing between them,
+    has the bits that it has by itself. (An MMA that outlived its CTA would write into tensor memory that the next CTA there has.)"""
+    T = 8 if path.startswith("draft") else 700
+    n, r, v, d = 4, 8, 256, 2048
+    g = torch.Generator(device="cuda")
+    g.manual_seed(31)
+
+    def normal(*shape, std):
+        return torch.empty(shape, dtype=torch.bfloat16, device="cuda").normal_(0.0, std, generator=g)
+
+    lowrank = (normal(n, v, d, std=0.05), normal(n, r, v, 16, std=0.1), normal(n, r, 16, d, std=0.05)) if path == "factored" else None
+    W_emit, W_sum = None if lowrank else normal(n, r, v, d, std=0.05), normal(r, d, std=0.05)
+    heads = [B.MtpcHead(B.MTPC_CP, n, r, v, d, B.MTPC_BF16, T, 2, W_emit, W_sum, lowrank=lowrank) for _ in range(2)]
+    hidden, weight = normal(T, d, std=1.0), torch.full((T,), -1.0 / T, device="cuda")
+    targets = torch.randint(0, v, (T, n), device="cuda", generator=g, dtype=torch.int32)
+    u = torch.rand(2 * T, 2 * n, device="cuda", generator=g)
+
+    def empty(*shape):
+        return torch.empty(shape, device="cuda")
+
+    def call(head):
+        if path == "logprob_single_ctas":
+            head.mtpc_debug_set_projection_variant(1)
+        out = [empty(T)]
+        if path.startswith("draft"):
+            out = [torch.empty(2 * T, n, dtype=torch.int32, device="cuda"), empty(2 * T)]
+            head.mtpc_draft_sample(hidden, 2, u, *out)
+        elif path == "backward":
+            out += [empty(T, d), empty(n, r, v, d), empty(r, d)]
+            head.mtpc_window_logprob_backward(hidden, targets, weight, *out)
+        elif path == "factored":
+            out += [empty(T, d), empty(n, v, d), empty(n, r, v, 16), empty(n, r, 16, d), empty(r, d)]
+            head.mtpc_lowrank_window_logprob_backward(hidden, targets, weight, *out)
+        else:
+            head.mtpc_window_logprob(hidden, targets, *out)
+        return out
+
+    want = call(heads[1])
+    torch.cuda.synchronize()
+    for _ in range(5):
+        heads[0].mtpc_debug_set_wait_limit_ns(50)
+        call(heads[0])                                    # gives up; outputs unspecified
+        got = call(heads[1])
+        code, bits = heads[0].mtpc_get_status(with_code=True)
+        assert code == B.ERR_TIMEOUT and bits & B.STATUS_TIMEOUT
+        assert heads[1].mtpc_get_status(with_code=True) == (B.MTPC_OK, 0)
+        for a, b in zip(want, got):
+            assert torch.equal(a, b)
+    for head in heads:
+        head.mtpc_destroy()

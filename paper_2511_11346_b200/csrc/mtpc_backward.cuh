@@ -1227,7 +1227,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
         const CUtensorMap* tm_b = &p.tm_b[seg];
         int ak = p.a_k0[seg] + (kb - seg_begin) * kBlockK + w.bt * p.a_k_step, bk = (kb - seg_begin) * kBlockK + w.bt * p.b_k_step;
         for (; kb < stop; ++kb, ak += kBlockK, bk += kBlockK) {
-          if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
+          if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p)) { ok = false; break; }
           const uint32_t full = full0 + 8 * stage, a_dst = tiles_addr + stage * p.stage_bytes;
           mbar_arrive_expect_tx(expects, own_full + 8 * stage, CTAS * (kABytes + kBBytes));      // of both CTAs' copies when paired
           if (A_MN) {
@@ -1258,7 +1258,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
     if (cta_rank == 0) {
       const uint32_t lead = elect_one();
       uint32_t stage = 0, phase = 0, use = 0;
-      bool ok = true;
+      bool ok = first_item >= num_items || first_wait(smem_u32(&ctl->full[0]), ctl, p);
       const uint32_t idesc = umma_idesc_bf16(kBlockM * CTAS, TN, A_MN, B_MN);
       // descriptor advance per K=16 step, in 16-byte units: 32 bytes along a swizzled K-major row, two 8-row groups
       // (2048 bytes) down an MN-major box
@@ -1274,11 +1274,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
       for (int item = first_item; item < num_items && ok; item += item_step, ++use) {
         const PlainItem w = plain_item(p, item, kblocks);
         const uint32_t slot = use % kSlots;
-        if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+        if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + slot * TN;
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
+          if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p)) { ok = false; break; }
           tc_fence_after();
           const uint64_t a_desc = a_desc0 + stage * stage_step, b_desc = b_desc0 + stage * stage_step;
 #pragma unroll

@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
       const int row = t.index * t.rows;
       const uint32_t bytes = (t.rows + p.Ppad) * (kBlockK * 2);    // out-of-range rows are zero-filled and counted
       for (int k = kb0 * kBlockK; k < kb1 * kBlockK; k += kBlockK) {
-        if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
+        if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p)) { ok = false; break; }
         const uint32_t full = full0 + 8 * stage, dst = tiles_addr + stage * p.stage_bytes;
         mbar_arrive_expect_tx(lead, full, bytes);
         tma_load_2d(lead, dst, map, full, k, row);
@@ -225,21 +225,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mtpc_decode_gemm_kernel(const
     // ------------------------------------------------------------------ MMA issuer: D[row, p] = W[row, :] . h[p, :]
     const uint32_t lead = elect_one();
     uint32_t stage = 0, phase = 0, use = 0;
-    bool ok = true;
+    bool ok = tile_begin >= tile_end || first_wait(smem_u32(&ctl->full[0]), ctl, p);
     const uint32_t idesc = umma_idesc_bf16(kBlockM, p.Ppad);
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
     const uint32_t stage_step = p.stage_bytes >> 4;             // descriptors step in 16-byte units
     const uint64_t a_desc0 = umma_smem_desc_sw128(tiles_addr), b_desc0 = umma_smem_desc_sw128(tiles_addr + hidden_off);
     for (int tile = tile_begin; tile < tile_end && ok; ++tile, ++use) {
       const uint32_t slot = use & 1u;
-      if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use >> 1) & 1u) ^ 1u, ctl, p.status)) {
+      if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use >> 1) & 1u) ^ 1u, ctl, p)) {
         ok = false;
         break;
       }
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + slot * p.tile_stride;
       for (int kb = kb0; kb < kb1; ++kb) {
-        if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
+        if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p)) { ok = false; break; }
         tc_fence_after();
         const uint64_t a_desc = a_desc0 + stage * stage_step, b_desc = b_desc0 + stage * stage_step;
 #pragma unroll

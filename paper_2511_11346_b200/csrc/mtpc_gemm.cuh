@@ -36,6 +36,7 @@ constexpr int kMaxSlots = 8;
 constexpr int kTmemCols = 512;
 constexpr int kGemmThreads = 192;
 constexpr uint64_t kWaitLimitNs = 1000ull * 1000ull * 1000ull;   // 1 s per barrier wait (the default, and always the limit of the drain waits)
+constexpr uint64_t kAwakeNs = 100ull * 1000ull;                  // limits below this: see first_wait
 constexpr uint64_t kAbortSettleNs = 200ull * 1000ull;            // 0.2 ms: far longer than any copy or MMA in flight takes
 constexpr int kABytes = kBlockM * kBlockK * 2;                   // 16 KB
 constexpr uint32_t kStatusBadTarget = 1u, kStatusBadUniform = 2u, kStatusTimeout = 4u;
@@ -128,22 +129,40 @@ __device__ __forceinline__ bool bounded_wait_warp(uint32_t bar, uint32_t parity,
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-// The whole warp waits and learns the outcome, known to be the same in every lane. A warp that waits as a whole sleeps in try_wait until
-// the barrier's phase is over or the hardware's own limit is, which is longer than any wait of a healthy call: limits of microseconds are
-// noticed by the epilogue's warps, whose lane 0 polls.
-__device__ __forceinline__ bool bounded_wait_all(uint32_t bar, uint32_t parity, GemmControl* ctl, unsigned* status) {
+// The whole warp waits and learns the outcome, known to be the same in every lane. It sleeps in try_wait until the barrier's phase is over or for
+// as long as the hardware lets it (a suspend-time hint of 50 ns does not shorten that), and then looks whether another role has given up. P: the
+// kernel's parameters.
+template <typename P>
+__device__ __forceinline__ bool bounded_wait_all(uint32_t bar, uint32_t parity, GemmControl* ctl, const P& p) {
   constexpr unsigned all = 0xffffffffu;
   if (__all_sync(all, mbar_try_wait(bar, parity))) return true;
   const uint64_t t0 = global_timer_ns();
   while (true) {
-    if (__all_sync(all, mbar_try_wait(bar, parity))) return true;
     if (__any_sync(all, ctl->abort)) return false;
-    if (__any_sync(all, global_timer_ns() - t0 > ctl->wait_limit_ns)) {
+    if (__all_sync(all, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(all, global_timer_ns() - t0 > p.wait_limit_ns)) {
       ctl->abort = 1;
-      if (elect_one()) atomicOr(status, kStatusTimeout);
+      if (elect_one()) atomicOr(p.status, kStatusTimeout);
       return false;
     }
   }
+}
+// A sleep outlasts limits of microseconds, and a choice between sleeping and not at every wait costs GEMMs 1.5 % (5 x 401 positions of a training call
+// 990 -> 1005 us). So with a limit that short the MMA issuer keeps awake for its first copies, and what it decides reaches the other roles by the
+// abort flag.
+template <typename P>
+__device__ __forceinline__ bool first_wait(uint32_t bar, GemmControl* ctl, const P& p) {
+  constexpr unsigned all = 0xffffffffu;
+  if (p.wait_limit_ns >= kAwakeNs) return true;
+  const uint64_t t0 = global_timer_ns();
+  while (!__all_sync(all, mbar_test_wait(bar, 0))) {
+    if (__any_sync(all, global_timer_ns() - t0 > p.wait_limit_ns)) {
+      ctl->abort = 1;
+      if (elect_one()) atomicOr(p.status, kStatusTimeout);
+      return false;
+    }
+  }
+  return true;
 }
 // A wait that decides nothing: for what may still be in flight when a CTA goes away.
 __device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity) {
@@ -402,7 +421,7 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
       for (int t = 0; t < tc.ntiles && ok; ++t) {
         const int brow = brow0 + t * tc.cols + static_cast<int>(cta_rank) * brows;
         for (int k = 0; k < p.kblocks * kBlockK; k += kBlockK) {
-          if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p.status)) { ok = false; break; }
+          if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p)) { ok = false; break; }
           const uint32_t full = full0 + 8 * stage, a_dst = tiles_addr + stage * p.stage_bytes;
           mbar_arrive_expect_tx(expects, own_full + 8 * stage, bytes);
           if (CTAS == 2) {
@@ -429,7 +448,7 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
     if (cta_rank == 0) {
       const uint32_t lead = elect_one();
       uint32_t stage = 0, phase = 0, use = 0;
-      bool ok = true;
+      bool ok = walk.first() >= walk.end || first_wait(smem_u32(&ctl->full[0]), ctl, p);
       const uint64_t a_desc0 = umma_smem_desc_sw128(tiles_addr), b_desc0 = umma_smem_desc_sw128(tiles_addr + kABytes);
       const uint32_t stage_step = p.stage_bytes >> 4, full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
       auto commit = [&](uint32_t bar) {                        // pairs: in both CTAs
@@ -441,14 +460,14 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
         const uint32_t idesc = umma_idesc_bf16(kBlockM * CTAS, tc.cols);
         for (int t = 0; t < tc.ntiles && ok; ++t, ++use) {
           const uint32_t slot = use % p.num_slots;
-          if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use / p.num_slots) & 1u) ^ 1u, ctl, p.status)) {
+          if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use / p.num_slots) & 1u) ^ 1u, ctl, p)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + slot * p.slot_stride;
           for (int kb = 0; kb < p.kblocks; ++kb) {
-            if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p.status)) { ok = false; break; }
+            if (!bounded_wait_all(full0 + 8 * stage, phase, ctl, p)) { ok = false; break; }
             tc_fence_after();
             const uint64_t a_desc = a_desc0 + stage * stage_step, b_desc = b_desc0 + stage * stage_step;
 #pragma unroll
@@ -478,7 +497,19 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
     };
     bool handed = false;                                       // (of two warps, the second: the first has a unit's share to read)
     float* share = reinterpret_cast<float*>(ctl + 1) + quarter * 96 + lane;
-    // (two warps that meet at barriers both go on after a wait that gave up, without waiting)
+    // After a wait that gave up a warp reads, stores and releases nothing more; it only meets its partner at the barriers of the units left.
+    auto meet = [&](int units) {
+      for (; units > 0; --units) {
+        if (sub == 1) {
+          if (handed) pair_sync(5 + quarter);
+          pair_arrive(1 + quarter);
+          handed = true;
+        } else {
+          pair_sync(1 + quarter);
+          pair_arrive(5 + quarter);
+        }
+      }
+    };
     for (int item = walk.first(); item < walk.end && (ok || kSubs == 2); item = walk.next(item)) {
       const TileCoord tc = coord(item);
       const int row = tc.arow + quarter * 32 + lane;
@@ -489,7 +520,7 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
         // ---- sum-unit logits -> log omega (Sec. 3.3): log-softmax over groups of r adjacent columns
         const uint32_t slot = use % p.num_slots;
         ok = ok && bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use / p.num_slots) & 1u, ctl, p.status, lane);
-        if (!ok && kSubs == 1) break;
+        if (!ok) continue;
         tc_fence_after();
         const uint32_t tcol = lane_base + slot * p.slot_stride;
         const int col_base = tc.unit0 * p.sum_cols;
@@ -664,6 +695,10 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
         for (int t = 0; t < tc.ntiles; ++t, ++use) {
           const uint32_t slot = use % p.num_slots;
           ok = ok && bounded_wait_warp(smem_u32(&ctl->tfull[slot]), (use / p.num_slots) & 1u, ctl, p.status, lane);
+          if (!ok) {
+            meet(units_end - unit);
+            break;
+          }
           tc_fence_after();
           const uint32_t tcol = lane_base + slot * p.slot_stride;
           // one batch of accumulator columns of this row

@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) low
     for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
       const LowRankItem w = lowrank_item(p, item);
       for (int e = 0; e < nent; ++e) {
-        if (!bounded_wait_all(smem_u32(&ctl->empty[st]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
+        if (!bounded_wait_all(smem_u32(&ctl->empty[st]), phase ^ 1u, ctl, p)) { ok = false; break; }
         const uint32_t full = smem_u32(&ctl->full[st]);
         const uint32_t dst = ring + st * kLrStageBytes;
         const int j = e * per_entry;                       // first component of the entry
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) low
     // ------------------------------------------------------------------ MMA issuer: pair u overall into slot u % kSlots
     const uint32_t lead = elect_one();
     uint32_t st = 0, phase = 0, use = 0;
-    bool ok = true;
+    bool ok = blockIdx.x >= num_items || first_wait(smem_u32(&ctl->full[0]), ctl, p);
     const uint64_t z_desc0 = umma_smem_desc_sw128(ring), a_desc0 = umma_smem_desc_sw128(ring + kLrZBox);
     constexpr uint32_t kStageStep = kLrStageBytes >> 4;      // descriptors step in 16-byte units
     auto next_stage = [&] {
@@ -216,12 +216,12 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) low
       const uint32_t idesc = umma_idesc_bf16(kBlockM, w.width);
       for (int pr = 0; pr < npairs && ok; ++pr, ++use) {
         const uint32_t slot = use % kSlots;
-        if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+        if (!bounded_wait_all(smem_u32(&ctl->tempty[slot]), ((use / kSlots) & 1u) ^ 1u, ctl, p)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + slot * 2 * kLrCols;
         const int count = min(2, p.r - 2 * pr);
         if (p.k == 16) {                                     // one entry: [hi | lo] of two components, 16 adaptor columns each
-          if (!bounded_wait_all(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
+          if (!bounded_wait_all(smem_u32(&ctl->full[st]), phase, ctl, p)) { ok = false; break; }
           tc_fence_after();
           const uint64_t z = z_desc0 + st * kStageStep, a = a_desc0 + st * kStageStep;
           const uint32_t z1 = count == 2 ? 4u : 0u, a1 = count == 2 ? 2u : 0u;
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(lowrank_threads(MODE), lowrank_ctas(MODE)) low
           next_stage();
         } else {                                             // an entry per component: hi at 0, lo at 32 of its 64 values
           for (int q = 0; q < count && ok; ++q) {
-            if (!bounded_wait_all(smem_u32(&ctl->full[st]), phase, ctl, p.status)) { ok = false; break; }
+            if (!bounded_wait_all(smem_u32(&ctl->full[st]), phase, ctl, p)) { ok = false; break; }
             tc_fence_after();
             const uint64_t z = z_desc0 + st * kStageStep, a = a_desc0 + st * kStageStep;
 #pragma unroll
@@ -927,8 +927,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) adaptor_grad_kernel(const __g
       for (int t = 0; t < t_tiles && ok; ++t, ++tc) {
         const uint32_t zbuf = tc & 1u;
         for (int q = 0; q < pairs; ++q) {
-          if (!bounded_wait_all(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p.status)) { ok = false; break; }
-          if (q == 0 && !bounded_wait_all(smem_u32(&ctl->empty[kAdaptorBarZ + zbuf]), ((tc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+          if (!bounded_wait_all(smem_u32(&ctl->empty[stage]), phase ^ 1u, ctl, p)) { ok = false; break; }
+          if (q == 0 && !bounded_wait_all(smem_u32(&ctl->empty[kAdaptorBarZ + zbuf]), ((tc >> 1) & 1u) ^ 1u, ctl, p)) { ok = false; break; }
           const bool two = q * 128 + 64 < p.v64;
           const uint32_t full = smem_u32(&ctl->full[stage]), dst = tiles_addr + stage * kAdaptorStage;
           mbar_arrive_expect_tx(lead, full, ((two ? 2 : 1) + (q == 0 ? 1 : 0)) * kAdaptorBox);
@@ -941,7 +941,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) adaptor_grad_kernel(const __g
           // the wait does not keep g from being fetched
           if (!a_loaded) {
             a_loaded = true;
-            if (!bounded_wait_all(smem_u32(&ctl->empty[kAdaptorBarA]), (uc & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+            if (!bounded_wait_all(smem_u32(&ctl->empty[kAdaptorBarA]), (uc & 1u) ^ 1u, ctl, p)) { ok = false; break; }
             const uint32_t afull = smem_u32(&ctl->full[kAdaptorBarA]);
             mbar_arrive_expect_tx(lead, afull, p.v64 * 128);
             for (int b = 0; b < p.v64; b += 64) tma_load_2d(lead, a_addr + b * 128, &p.tm_a, afull, 0, unit * p.v64 + b);
@@ -957,21 +957,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1) adaptor_grad_kernel(const __g
   } else if (warp == 1) {
     const uint32_t lead = elect_one();
     uint32_t stage = 0, phase = 0, tc = 0, uc = 0;
-    bool ok = true;
+    bool ok = blockIdx.x >= p.units || first_wait(smem_u32(&ctl->full[0]), ctl, p);
     const uint32_t idesc_y = umma_idesc_bf16(kBlockM, p.k, false, true), idesc_da = umma_idesc_bf16(kBlockM, p.k, true, true);
     const uint64_t g_desc0 = umma_smem_desc_sw128(tiles_addr), gt_desc0 = umma_smem_desc_mn_sw128(tiles_addr, kAdaptorBox);
     const uint64_t z_desc0 = umma_smem_desc_mn_sw128(z_addr, kAdaptorBox), a_desc0 = umma_smem_desc_mn_sw128(a_addr, kMnBoxBytes);
     for (int unit = blockIdx.x; unit < p.units && ok; unit += gridDim.x, ++uc) {
       const uint32_t set = uc & 1u;
-      if (!bounded_wait_all(smem_u32(&ctl->tempty[2 + set]), ((uc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
-      if (!bounded_wait_all(smem_u32(&ctl->full[kAdaptorBarA]), uc & 1u, ctl, p.status)) { ok = false; break; }
+      if (!bounded_wait_all(smem_u32(&ctl->tempty[2 + set]), ((uc >> 1) & 1u) ^ 1u, ctl, p)) { ok = false; break; }
+      if (!bounded_wait_all(smem_u32(&ctl->full[kAdaptorBarA]), uc & 1u, ctl, p)) { ok = false; break; }
       for (int t = 0; t < t_tiles && ok; ++t, ++tc) {
         const uint32_t yslot = tc & 1u;
-        if (!bounded_wait_all(smem_u32(&ctl->tempty[yslot]), ((tc >> 1) & 1u) ^ 1u, ctl, p.status)) { ok = false; break; }
+        if (!bounded_wait_all(smem_u32(&ctl->tempty[yslot]), ((tc >> 1) & 1u) ^ 1u, ctl, p)) { ok = false; break; }
         const uint64_t z_desc = z_desc0 + yslot * (kAdaptorBox >> 4);
         const uint32_t y_tmem = tmem_base + yslot * 32;
         for (int q = 0; q < pairs; ++q) {
-          if (!bounded_wait_all(smem_u32(&ctl->full[stage]), phase, ctl, p.status)) { ok = false; break; }
+          if (!bounded_wait_all(smem_u32(&ctl->full[stage]), phase, ctl, p)) { ok = false; break; }
           tc_fence_after();
           const uint32_t at = stage * (kAdaptorStage >> 4);
           const bool two = q * 128 + 64 < p.v64;

@@ -260,12 +260,14 @@ def test_draft_and_acceptance_calls_can_be_captured_into_a_cuda_graph(family, n,
     dh.close()
 
 
-@pytest.mark.parametrize("path", ["logprob", "logprob_single_ctas", "draft_few", "backward", "factored"])
+@pytest.mark.parametrize("path", ["logprob", "logprob_single_ctas", "draft_few", "draft_few_clusters", "backward", "factored"])
 def test_a_call_right_behind_one_that_gave_up(path):
     """A kernel that gave up leaves nothing in flight: the call that follows it in the stream, of another head and with nothing between them,
     has the bits that it has by itself. (An MMA that outlived its CTA would write into tensor memory that the next CTA there has.)"""
     T = 8 if path.startswith("draft") else 700
     n, r, v, d = 4, 8, 256, 2048
+    if path == "draft_few_clusters":
+        n, v = 2, 64                                      # few tiles: clusters share their K
     g = torch.Generator(device="cuda")
     g.manual_seed(31)
 

@@ -456,9 +456,9 @@ int launch_gemm(mtpc_head* h, const void* hidden_bf16, int rows, bool with_emit,
     plan = choose_group_units(c.v, emit_units, p.m_tiles, h->num_sms, launch_sums);
     if (h->projection_variant != 1 && h->max_pairs > 0) {
       const ItemPlan two = choose_group_units(c.v, emit_units, (p.m_tiles + 1) / 2, h->max_pairs, launch_sums);
-      if (h->projection_variant == 0 && p.m_tiles >= 2)
-        pair = c.d < 1536 ? two.tiles * 34 <= plan.tiles * 33 : two.tiles * 12 <= plan.tiles * 13;
-      if (!with_emit && L.sum_cols <= 64) pair = false;       // few columns: an MMA of a pair takes twice as long as a lone CTA's (see below)
+      if (h->projection_variant == 0 && p.m_tiles >= 2)       // (sum tiles of few columns: an MMA of a pair takes twice as long as a lone CTA's, see below)
+        pair = !with_emit && L.sum_cols <= 64 ? false
+               : c.d < 1536 ? two.tiles * 34 <= plan.tiles * 33 : two.tiles * 12 <= plan.tiles * 13;
       if (pair) plan = two;
     }
   }

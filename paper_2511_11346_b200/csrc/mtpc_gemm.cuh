@@ -639,7 +639,8 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
       } else {
         // ---- log phi at the target byte: online log-sum-exp over the v columns of each unit + gather. The
         // running (m, s) and the gathered logit live across tile boundaries; a unit is closed when its v-th
-        // column has been passed.
+        // column has been passed. Two warps share a row (one on sorted rows, which never come here).
+        static_assert(kGrouped || kSubs == 2, "a unit's columns are dealt to two warps");
         const int* tgts = (valid && p.targets != nullptr) ? p.targets + static_cast<size_t>(row) * p.n : nullptr;
         const int units_end = tc.unit0 + tc.nunits;
         int unit = tc.unit0, col_in_unit = 0;
@@ -648,7 +649,7 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
         int tgt = tgts != nullptr ? tgts[slot_i] : -1;
         // ---- unit (slot_i, k) complete
         auto close_unit = [&] {
-          if (kSubs == 2 && sub == 1) {
+          if (sub == 1) {
             if (handed) pair_sync(5 + quarter);                          // the share before this one has been read
             share[0] = m;
             share[32] = s;
@@ -656,16 +657,14 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
             pair_arrive(1 + quarter);
             handed = true;
           } else {
-            if (kSubs == 2) {
-              pair_sync(1 + quarter);
-              const float m2 = share[0], s2 = share[32];
-              tval += share[64];                                         // (one of the two has seen the target's column)
-              pair_arrive(5 + quarter);
-              // the same bits whichever warp had the unit's first batch, which depends on where in an item the unit lies
-              const float ref = fmaxf(m, kLowestRef), ref2 = fmaxf(m2, kLowestRef), rn = fmaxf(ref, ref2);
-              s = __fadd_rn(__fmul_rn(s, fast_ex2((ref - rn) * kLog2e)), __fmul_rn(s2, fast_ex2((ref2 - rn) * kLog2e)));
-              m = fmaxf(m, m2);
-            }
+            pair_sync(1 + quarter);
+            const float m2 = share[0], s2 = share[32];
+            tval += share[64];                                           // (one of the two has seen the target's column)
+            pair_arrive(5 + quarter);
+            // the same bits whichever warp had the unit's first batch, which depends on where in an item the unit lies
+            const float ref = fmaxf(m, kLowestRef), ref2 = fmaxf(m2, kLowestRef), rn = fmaxf(ref, ref2);
+            s = __fadd_rn(__fmul_rn(s, fast_ex2((ref - rn) * kLog2e)), __fmul_rn(s2, fast_ex2((ref2 - rn) * kLog2e)));
+            m = fmaxf(m, m2);
             // a unit that lies below the lowest reference as a whole: less than half an ulp above its maximum (-inf, NaN: NaN)
             const float lse = m >= kLowestRef ? fmaf(fast_lg2(s), kLn2, m) : fmaf(m - m, s, m);
             if (valid) {
@@ -743,7 +742,7 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
             if (sub == 1 && !pass_batch()) return false;
             consume(raw, b);
             if (!pass_batch()) return false;
-            return kSubs == 1 || sub == 1 || pass_batch();
+            return sub == 1 || pass_batch();
           };
           // The load of the next batch is in flight while this one goes through the exponentials (two register buffers).
           const int batches = tc.cols / COLS;
@@ -770,7 +769,7 @@ __global__ void __launch_bounds__(gemm_threads(MODE), 1) mtpc_gemm_kernel(const 
         }
       }
     }
-    if (kSubs == 2 && handed) pair_sync(5 + quarter);
+    if (handed) pair_sync(5 + quarter);
   }
 
   tc_fence_before();

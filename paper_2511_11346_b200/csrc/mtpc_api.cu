@@ -827,6 +827,16 @@ unsigned long long capture_id(cudaStream_t st) {
   if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) { cudaGetLastError(); return 0; }
   return status == cudaStreamCaptureStatusActive ? id + 1 : 0;
 }
+// Dynamic shared memory that leaves an SM room for its even share of `ctas` CTAs and no more. The CTAs of a programmatic dependent that do not fit
+// beside the projection's (ten warps of 168 registers; with six of 120 they did) pile up on the SMs that fall free first, up to sixteen on one while
+// others stay empty. Latent draws behind a projection, six warps ahead / ten / ten and so, us: tree 16 x 8, 595 positions 10.4 / 16.7 / 10.4, 16 x 32,
+// 400 positions 10.2 / 18.0 / 10.4, 3000 positions 21 / 21 / 15; HMM 16 x 16, 568 positions 10.7 / 16.4 / 10.5, 1000 positions 17.2 / 17.7 / 11.4. (A plain
+// launch 13, since its start is then in the chain; one window a CTA 11 to 13; 144 registers a thread in the projection: only the HMM's 568 10.2.)
+size_t even_share_smem(const mtpc_head* h, long long ctas) {
+  const size_t share = static_cast<size_t>((ctas + h->num_sms - 1) / h->num_sms);
+  if (share == 0 || share > 16) return 0;                               // (sixteen CTAs are all that an SM's threads let in)
+  return ((kSmemLimit + 1024) / share - 1024) / 1024 * 1024;            // (1 KB of an SM's 228 goes with every CTA)
+}
 
 // out_logprob [W] (joint) and / or out_prefix [W, n] (prefix log-marginals of the draft); either may be NULL, not both.
 int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, const float* uniforms,
@@ -979,7 +989,8 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
     if (rc != MTPC_OK) return rc;
     int* sel = at<int>(h, L.off_sel) + w0 * c.n;
     pt.begin();
-    launch_kernel(latent_sample_kernel, (wc + kLatentWarps - 1) / kLatentWarps, 32 * kLatentWarps, 0, st, overlapped(h),
+    const int latent_ctas = (wc + kLatentWarps - 1) / kLatentWarps;
+    launch_kernel(latent_sample_kernel, latent_ctas, 32 * kLatentWarps, even_share_smem(h, latent_ctas), st, overlapped(h),
                   c.family, at<float>(h, L.off_logw) + static_cast<size_t>(p0) * L.sum_rows,
                   hmm_tables(h) + static_cast<size_t>(p0) * hmm_table_stride(h), u, sel, out_bytes + w0 * c.n,
                   at<unsigned>(h, L.off_status), wc, wpp, c.n, c.r, L.sum_rows, hmm_table_stride(h));
@@ -1738,7 +1749,7 @@ static int create_head_impl(const mtpc_config* cfg, const void* W_emit, const Lo
   for (auto* kernel : {draft_slot_kernel<false, 4, 2>, draft_slot_kernel<false, 8, 2>, draft_slot_kernel<false, 10, 2>, draft_slot_kernel<false, 16, 2>,
                        draft_slot_kernel<false, 4, 3>, draft_slot_kernel<false, 8, 3>, draft_slot_kernel<false, 10, 3>, draft_slot_kernel<true, 16, 2>})
     fail |= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, slot_smem) != cudaSuccess;
-  fail |= !set_circuit_attributes();
+  fail |= !set_circuit_attributes() || !allow_full_smem(latent_sample_kernel);
   fail |= !allow_full_smem(spec_accept_kernel<true>) || !allow_full_smem(spec_accept_kernel<false>);
   fail |= cudaMemsetAsync(h->ws + L.off_status, 0, 256, st) != cudaSuccess;
   if (fail) { delete h; return MTPC_ERR_CUDA; }

@@ -1208,6 +1208,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
 
   if (warp == 0) {
     // One K block must be asked for in less time than its MMAs take (256 cycles), so that little is computed per block.
+    // Weight gradients of few positions in pairs are bound by their fp32 stores, and this warp waits most of the time: then one lane does. As a whole warp /
+    // so / issued from lane 0's own branch, us: dW_emit of 8 x 16 x 320, d = 4096 from 60 positions 192 / 166 / 168, 250 208 / 186 / 195, 500 232 / 213 / 224, 1000
+    // (16 K blocks) 293 / 281 / 294; but 1100 319 / 317 / 311, 1500 371 / 381 / 372, 4096 906 / 935 / 935. Lone CTAs, 8 x 8 x 256, d = 2048, 900 positions
+    // 58 / 61 / 62; K-major operands (long K) 250 positions 75 / 78 / 79.
+    const bool few_blocks = A_MN && CTAS == 2 && kblocks <= 16;
     const uint32_t lead = elect_one(), expects = cta_rank == 0 ? lead : 0u;
     uint32_t stage = 0, phase = 0, issued = 0;
     bool ok = true;
@@ -1227,7 +1232,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) plain_gemm_kernel(const __gri
         const CUtensorMap* tm_b = &p.tm_b[seg];
         int ak = p.a_k0[seg] + (kb - seg_begin) * kBlockK + w.bt * p.a_k_step, bk = (kb - seg_begin) * kBlockK + w.bt * p.b_k_step;
         for (; kb < stop; ++kb, ak += kBlockK, bk += kBlockK) {
-          if (!bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p)) { ok = false; break; }
+          ok = few_blocks ? bounded_wait_warp(empty0 + 8 * stage, phase ^ 1u, ctl, p.status, lane) : bounded_wait_all(empty0 + 8 * stage, phase ^ 1u, ctl, p);
+          if (!ok) break;
           const uint32_t full = full0 + 8 * stage, a_dst = tiles_addr + stage * p.stage_bytes;
           mbar_arrive_expect_tx(expects, own_full + 8 * stage, CTAS * (kABytes + kBBytes));      // of both CTAs' copies when paired
           if (A_MN) {

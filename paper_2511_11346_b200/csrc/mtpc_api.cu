@@ -651,7 +651,9 @@ int resident_clusters(K kernel, int size, int threads, int which, int dev) {
 // CTAs has the fewest rows, emission and sum-unit tiles dealt evenly together, a tile counted as 3 rows more and as one for every six
 // positions the head may draft at once (its copies of their hidden states); ties go to the taller tile. (By the emission rows alone, a tree
 // head of n = 8, r = 32, v = 256 got 5 tiles of 112 rows on its longest CTA where the mean is 485 rows, 4 of 128 now. 3 or 24 rows a tile whatever
-// the positions, us: tree 16 x 32 x 256, 8 positions 154.1 / 155.8, 128 positions 209.9 / 206.6; tree 16 x 32 x 272, 8 positions 118.4 / 119.8.)
+// the positions, us: tree 16 x 32 x 256, 8 positions 154.1 / 155.8, 128 positions 209.9 / 206.6; tree 16 x 32 x 272, 8 positions 118.4 / 119.8. A head
+// has one height, and one made for 128 positions loses nothing on fewer: made for the call's / for 128, tree 16 x 32 x 256, 8 positions 149.7 / 149.0, HMM
+// 16 x 32 x 320, 1 position 208.3 / 208.2, mixture 8 x 16 x 320, 4 positions 63.1 / 62.8, tree 16 x 32 x 272, d = 2048, 8 positions 114.4 / 113.5.)
 long long decode_tiles(long long rows, int sum_rows, int tr) {
   return (rows + tr - 1) / tr + (sum_rows + tr / 32 * 32 - 1) / (tr / 32 * 32);
 }
@@ -726,10 +728,13 @@ int launch_decode_gemm(mtpc_head* h, const void* hidden_bf16, int P, cudaStream_
   p.stage_bytes = (stage + 1023) / 1024 * 1024;
   const int ctl = 1024 + static_cast<int>(sizeof(GemmControl)) + static_cast<int>(decode_exchange_bytes(p.ksplit, p.Ppad));
   p.stages = (kSmemLimit - ctl) / p.stage_bytes;
-  // At most nine stages, 144 KB up to 16 positions: with more of them, or fewer, the same pass is slower (why was not found). Drafts +
-  // acceptance with 7 / 8 / 9 / 10 stages, us: HMM 16 x 32 x 320, d = 4096, 1 position 215.0 213.4 211.4 213.3, 8 227.2 225.5 223.4 225.6;
-  // mixture 8 x 16 x 320, 1 position 64.4 64.4 62.6 63.5; 16 x 16 x 320, 64 positions 139.3 138.8 138.3 139.2; tree 8 x 32 x 256, 27 positions
-  // 89.7 90.0 88.2 89.4; with 12 and 13 stages the HMM's 8 positions take 230.2 and 231.3.
+  // At most nine stages (up to 16 positions 144 to 162 KB, by the tile's height): with more of them, or fewer, the same pass is up to 3 % slower. Why was
+  // not found, but it is the number that counts, not the bytes, and it does on every head tried, whatever d, r, v and the circuit. Drafts +
+  // acceptance with 7 / 8 / 9 / 10 / 12 stages, us: HMM 16 x 32 x 320, d = 4096, 8 positions 219.3 219.6 218.0 219.1 223.1; 16 x 16 x 272, d = 4096,
+  // 12 positions 106.9 106.5 105.5 106.4 107.4; 8 x 32 x 272, d = 3072, 16 positions 84.6 84.1 83.7 84.2 84.4; mixture 4 x 32 x 256, d = 4096, 2
+  // positions 55.1 55.3 53.6 54.2 54.1; 16 x 32 x 320, d = 2048, 6 positions 117.0 117.4 115.2 117.0 117.6; 8 x 8 x 256, d = 2048, 4 positions 22.4 22.6
+  // 22.3 22.7 22.7; tree 8 x 16 x 256, d = 4096, 24 positions 60.9 60.4 59.7 59.9 60.1; 16 x 16 x 320, d = 2048, 40 positions 79.6 79.6 79.2 79.5 79.5;
+  // the one exception mixture 8 x 16 x 320, d = 4096, 1 position 63.8 63.4 62.0 62.1 61.7. Six stages are 2 to 50 % slower.
   if (p.stages > kDecodeMaxStages) p.stages = kDecodeMaxStages;
   p.logw = at<float>(h, L.off_logw);
   p.sum_bias = sum_bias(h);
@@ -945,7 +950,9 @@ int draft_sample_impl(mtpc_head* h, const void* hidden, int32_t P, int32_t wpp, 
                                   (smem <= kSlotSmemPair || (smem <= kSlotSmemLimit && c.n * P <= h->num_sms));
       // builds of the narrow kernel that unroll 4, 8, 10 or 16 batches of 32 symbols: the smallest that covers v; where a device full of
       // CTAs is not all of them, and a third fits an SM's shared memory, the builds whose registers let it (see draft_slot_kernel; not of
-      // contextual tables, which come by L2 for every position: n = 16, r = 32, d = 2048, 115 positions 210.6 us with two, 212.4 with three)
+      // contextual tables, which come by L2 for every position. Two / three there, us: one window a position, n = 16, r = 16, 100 positions 116.2 /
+      // 116.9, r = 32, 115 positions 204.8 / 204.9, r = 8, 120 positions 75.8 / 75.7; but four windows, n = 8, r = 16, 64 positions 44.1 / 42.9, n = 16, r = 32,
+      // 128 positions 162.0 / 161.1, and sixteen, n = 8, r = 32, 100 positions 129.8 / 126.5: with many draws to a table three would gain)
       const size_t slot_smem = weights_in_smem ? smem : smem - weights;
       const bool crowd = !is_ctx(h) && c.n * P > 2 * h->num_sms && 3 * (slot_smem + 1024) <= static_cast<size_t>(kSmemLimit);
       auto* slot_kernel = c.v > kMaxDraftVocab ? draft_slot_kernel<true, 16, 2>

@@ -21,12 +21,12 @@
 // r = 32, v = 320), in the gradient also the 1.3 GB of g.
 // 64 columns divide more vocabularies evenly than 128 (of the third item of v = 320 half the warps had nothing), one wait and one
 // release serve two components, and log-sums leave as 128 contiguous bytes (position fastest; transposed through shared memory
-// before). Measured, forward / merge / gradient, same sizes: 292 / 62 / 450 us before, 247 / 67 / 387 now, the exponential unit
-// busy for 73 / 43 % of the cycles (61 / 38); the gradient's rest is instructions (two thirds of an issue slot a logit) and its warps' latency.
+// before). Measured, forward / merge / gradient, same sizes: 292 / 62 / 450 us before, 240 / 67 / 403 so, 208 / 64 / 398 now.
 // The fused projection that kept logits took 801 us and the passes that made g and its sum from them 921.
 // Roles: warp 0 TMA producer, warp 1 MMA issuer, then the epilogue warps (TMEM quarter warp % 4).
 // Both issue from a converged warp (elect_one): forward 240 -> 222 us, gradient 403 -> 398. A quarter of the forward's exponentials are polynomials
-// (poly_ex2), since the exponential unit was busy for 73 % of the cycles and issue slots for 47: 222 -> 208.
+// (poly_ex2), since the exponential unit was busy for 73 % of the cycles and issue slots for 47: 222 -> 208, the unit busy for 65 % now and
+// issue slots for 60. The gradient is at neither bound (45 % and 49 %): nine instructions a logit, and its warps' latency.
 // Operand ring: one entry holds 32 / k components, all as 128-byte rows with the 128-byte swizzle: z as one box of 128
 // positions x 64 values ([hi | lo] of the components), and A as one box of the item's vocabulary rows x 64 values (the components' k
 // adaptor columns first) of a copy laid out [n, v, r, k] (lowrank_repack_kernel, made on every call: A is small and may have changed).

@@ -242,7 +242,7 @@ def test_a_wait_that_runs_out_in_the_factored_kernel_is_reported_and_the_head_re
     """Both pipelines of the factored projection (base and corrections, each with its own producer and MMA issuer) give up
     at their first wait under a 50 ns limit: the status must say so, the context must stay usable, and the next call
     with the default limit must be right again."""
-    family, n, r, v, d, k, T = I.CP, 3, 8, 320, 4096, 16, 400      # (d = 4096: 64 K blocks in the base product)
+    family, n, r, v, d, k, T = I.CP, 3, 8, 320, 4096, 16, 400      # d = 4096: the first copies take longer than 64 polls
     wl, W, A, Bm = _factored_case(family, n, r, v, 0, d, k, T, seed=4500)
     head = B.MtpcHead(family, n, r, v, d, B.MTPC_BF16, T, 1, None, to_device_bf16(wl.W_sum_q), None,
                       lowrank=(_device(W), _device(A), _device(Bm)))
